@@ -15,6 +15,8 @@
 
 #include "../../include/xfp_quant.h"
 #include "xfp_internal.h"   // sm_count()
+#include "xfp_quant_common.cuh"
+#include "xfp_quant_internal.h"
 
 namespace xq {
 
@@ -23,122 +25,65 @@ constexpr int kRedThreads = 256;
 constexpr int kTieChunk = 4096;    // elements per block in the ordered tie pass (256 threads x 16)
 constexpr int kTiePer = 16;
 
-__device__ __forceinline__ double h2d(uint16_t h) { return (double)__half2float(__ushort_as_half(h)); }
-__device__ __forceinline__ uint16_t d2h(double d) { return __half_as_ushort(__double2half(d)); }
-
-// D16 of a V2a weight: one fp32 rounding of scale*lib + mid (the product of two fp16 is exact in fp32),
-// then one fp16 rounding ("V2a: Shared Codebook Library").
-__device__ __forceinline__ uint16_t v2a_value16(uint16_t scale, uint16_t lib, uint16_t mid) {
-    const float r = __fmaf_rn(__half2float(__ushort_as_half(scale)), __half2float(__ushort_as_half(lib)),
-                              __half2float(__ushort_as_half(mid)));
-    return __half_as_ushort(__float2half_rn(r));
-}
-
-// Index of the entry nearest to x among e[0..E), ties to the lower index: the answer of a linear scan that keeps an
-// entry only when it is strictly nearer.  When the entries ascend (codebooks and decoded library entries do) x is
-// bracketed by bisection and only its two neighbours are measured; the scan's answer is the nearer of the two
-// (the lower on an exact tie: fp64 rounding is monotone and distinct fp16 values are too far apart to round to
-// the same distance), moved down over duplicates of its value.
-__device__ __forceinline__ int nearest_entry(const double* e, int E, double x, bool ascending) {
-    if (!ascending) {
-        int best = 0;
-        double bd = fabs(__dsub_rn(x, e[0]));
-        for (int j = 1; j < E; ++j) {
-            const double d = fabs(__dsub_rn(x, e[j]));
-            if (d < bd) { bd = d; best = j; }
-        }
-        return best;
-    }
-    int lo = 0, hi = E;   // first index whose entry is >= x
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (e[mid] < x) lo = mid + 1; else hi = mid;
-    }
-    int best;
-    if (lo == 0) best = 0;
-    else if (lo == E) best = E - 1;
-    else best = fabs(__dsub_rn(x, e[lo - 1])) <= fabs(__dsub_rn(x, e[lo])) ? lo - 1 : lo;
-    while (best > 0 && e[best - 1] == e[best]) --best;
-    return best;
-}
-
-// Sum over the block in a fixed tree order; every thread gets the result.
-__device__ double block_sum(double v, double* sh) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x >> 1; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] = __dadd_rn(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
-    }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
-}
-
-// Exclusive scan of one int per thread over the block (blockDim.x <= 1024, a multiple of 32); returns
-// the thread's offset and leaves the block total in *total.
-__device__ int block_excl_scan(int v, int* sh_warp, int* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += t;
-    }
-    if (lane == 31) sh_warp[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        int x = lane < nw ? sh_warp[lane] : 0;
-        int xi = x;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, xi, d);
-            if (lane >= d) xi += t;
-        }
-        if (lane < nw) sh_warp[lane] = xi - x;
-        if (lane == 31) *total = xi;
-    }
-    __syncthreads();
-    const int r = sh_warp[w] + inc - v;
-    __syncthreads();
-    return r;
-}
-
 // ------------------------------------------------------------------ statistics
 
-// PASS 0: sum of w.  PASS 1: sum of (w - mu)^2.
-template <int PASS>
-__global__ void __launch_bounds__(kRedThreads) stats_partial(const float* __restrict__ W, int64_t n,
-                                                              const double* __restrict__ ms, double* part) {
+// One pass for both moments: a block sums d and d^2 of its chunk, d = w - p with p the mean of the chunk's first values,
+// and leaves (sum of w, sum of squared deviations from the chunk's own mean); stats_final combines the chunks around the
+// matrix mean.  The shift keeps the cancellation of sum d^2 - (sum d)^2 / n at a factor near one, so sigma is as good as
+// that of a second pass over the matrix (which took another 37 us of 12288 x 4096 weights).
+__global__ void __launch_bounds__(kRedThreads) stats_partial(const float* __restrict__ W, int64_t n, double2* part) {
     __shared__ double sh[kRedThreads];
-    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t b0 = (int64_t)blockIdx.x * per;
-    const int64_t b1 = b0 + per < n ? b0 + per : n;
-    const double mu = PASS ? ms[0] : 0.0;
-    double acc = 0.0;
-    for (int64_t t = b0 + threadIdx.x; t < b1; t += kRedThreads) {
-        const double w = (double)W[t];
-        if (PASS) {
-            const double d = __dsub_rn(w, mu);
-            acc = __dadd_rn(acc, __dmul_rn(d, d));
-        } else {
-            acc = __dadd_rn(acc, w);
+    const int64_t n4 = n >> 2, per = (n4 + gridDim.x - 1) / gridDim.x;
+    const int64_t b0 = (int64_t)blockIdx.x * per, b1 = b0 + per < n4 ? b0 + per : n4;
+    const float4* W4 = (const float4*)W;
+    const int tail = blockIdx.x == 0 ? (int)(n & 3) : 0;      // the last n mod 4 weights belong to block 0
+    int64_t cnt = (b1 > b0 ? b1 - b0 : 0) * 4 + tail;
+    double s = 0.0;
+    int64_t t = b0 + threadIdx.x;
+    int have = 0;
+    if (t < b1) { const float4 w = __ldg(W4 + t); s = ((double)w.x + (double)w.y) + ((double)w.z + (double)w.w); have = 4; }
+    else if ((int)threadIdx.x < tail && b1 <= b0) { s = (double)W[(n & ~(int64_t)3) + threadIdx.x]; have = 1; }
+    const double ps = block_sum(s, sh), pn = block_sum((double)have, sh);
+    const double p = pn > 0.0 ? ps / pn : 0.0;
+    double a[4] = {0.0, 0.0, 0.0, 0.0}, q[4] = {0.0, 0.0, 0.0, 0.0};
+    for (; t < b1; t += 4 * kRedThreads) {
+        float4 w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (t + u * kRedThreads < b1) w[u] = __ldg(W4 + t + u * kRedThreads);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (t + u * kRedThreads < b1) {
+                const float f[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { const double d = (double)f[i] - p; a[i] += d; q[i] = fma(d, d, q[i]); }
+            }
         }
     }
-    const double r = block_sum(acc, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = r;
+    if ((int)threadIdx.x < tail) { const double d = (double)W[(n & ~(int64_t)3) + threadIdx.x] - p; a[0] += d; q[0] = fma(d, d, q[0]); }
+    const double sa = block_sum((a[0] + a[1]) + (a[2] + a[3]), sh), sq = block_sum((q[0] + q[1]) + (q[2] + q[3]), sh);
+    if (threadIdx.x == 0)
+        part[blockIdx.x] = cnt ? make_double2(p * (double)cnt + sa, sq - sa * (sa / (double)cnt)) : make_double2(0.0, 0.0);
 }
 
-template <int PASS>
-__global__ void __launch_bounds__(kRedThreads) stats_final(const double* part, int64_t n, double* ms) {
+__global__ void __launch_bounds__(kRedThreads) stats_final(const double2* part, int64_t n, double* ms) {
     __shared__ double sh[kRedThreads];
+    const int64_t n4 = n >> 2, per = (n4 + kRedBlocks - 1) / kRedBlocks;
+    double2 v[kRedBlocks / kRedThreads];
     double acc = 0.0;
-    for (int t = threadIdx.x; t < kRedBlocks; t += kRedThreads) acc = __dadd_rn(acc, part[t]);
-    const double r = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-        if (PASS == 0) ms[0] = __ddiv_rn(r, (double)n);
-        else ms[1] = __dsqrt_rn(__ddiv_rn(r, (double)n));
+#pragma unroll
+    for (int i = 0; i < kRedBlocks / kRedThreads; ++i) { v[i] = part[threadIdx.x + i * kRedThreads]; acc += v[i].x; }
+    const double mu = block_sum(acc, sh) / (double)n;
+    acc = 0.0;
+#pragma unroll
+    for (int i = 0; i < kRedBlocks / kRedThreads; ++i) {
+        const int b = threadIdx.x + i * kRedThreads;
+        const int64_t b0 = (int64_t)b * per, b1 = b0 + per < n4 ? b0 + per : n4;
+        const int64_t cnt = (b1 > b0 ? b1 - b0 : 0) * 4 + (b == 0 ? (n & 3) : 0);
+        if (cnt) { const double d = v[i].x / (double)cnt - mu; acc += v[i].y + (double)cnt * d * d; }
     }
+    const double ss = block_sum(acc, sh);
+    if (threadIdx.x == 0) { ms[0] = mu; ms[1] = sqrt(fmax(ss, 0.0) / (double)n); }
 }
 
 // ------------------------------------------------------------------ exact selection by radix descent
@@ -254,41 +199,97 @@ __global__ void median_finish(const SelState* st, int64_t n, double scale, doubl
     *out = scale == 1.0 ? m : __dmul_rn(scale, m);
 }
 
-// The same descent for a short array of doubles (the per-channel cosines), one block, one launch.
+// Median of a short array (the per-channel cosines), one block, one launch: the keys' range is cut into 2048 equal steps
+// and counted, and the members of the one or two steps that hold the middle values are ranked against each other.  Where
+// those steps hold more than a block's worth of keys (many equal values) their range is cut again.
 __global__ void __launch_bounds__(1024) median_small_kernel(const double* __restrict__ v, int n, double* out) {
-    __shared__ unsigned int hist[256];
-    __shared__ unsigned long long s_prefix;
-    __shared__ long long s_k;
-    __shared__ double val[2];
+    constexpr int kBins = 2048, kCand = 1024;
+    __shared__ unsigned int hist[kBins];
+    __shared__ unsigned long long cand[kCand], s_lo, s_hi, s_val[2];
+    __shared__ int sh[32];
+    __shared__ int total, s_n, s_bin[2], s_before;
     const SrcDouble src{v};
-    for (int slot = 0; slot < 2; ++slot) {
-        if (threadIdx.x == 0) { s_prefix = 0; s_k = slot == 0 ? (n - 1) / 2 : n / 2; }
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            if (threadIdx.x < 256) hist[threadIdx.x] = 0;
-            __syncthreads();
-            const unsigned long long prefix = s_prefix;
-            for (int t = threadIdx.x; t < n; t += 1024) {
-                const unsigned long long key = src.key(t, 0.0);
-                if (shift == 56 || ((key ^ prefix) >> (shift + 8)) == 0) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                long long k = s_k;
-                int d;
-                for (d = 0; d < 255; ++d) {
-                    const long long c = hist[d];
-                    if (k < c) break;
-                    k -= c;
-                }
-                s_k = k;
-                s_prefix = prefix | ((unsigned long long)d << shift);
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) val[slot] = unflip(s_prefix);
-        __syncthreads();
+    const int tid = threadIdx.x;
+    unsigned long long lo = ~0ull, hi = 0ull;
+    for (int t = tid; t < n; t += 1024) { const unsigned long long k = src.key(t, 0.0); lo = k < lo ? k : lo; hi = k > hi ? k : hi; }
+    if (tid == 0) { s_lo = ~0ull; s_hi = 0ull; }
+    __syncthreads();
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, d), b = __shfl_xor_sync(0xffffffffu, hi, d);
+        lo = a < lo ? a : lo; hi = b > hi ? b : hi;
     }
-    if (threadIdx.x == 0) *out = (n & 1) ? val[1] : __dmul_rn(0.5, __dadd_rn(val[0], val[1]));
+    if ((tid & 31) == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
+    __syncthreads();
+    lo = s_lo; hi = s_hi;
+    int k0 = (n - 1) / 2, k1 = n / 2;        // ranks of the middle values among the keys of [lo, hi]
+    for (;;) {
+        if (lo == hi) { if (tid == 0) s_val[0] = s_val[1] = lo; break; }
+        const unsigned long long span = hi - lo;
+        const int sft = 64 - __clzll((long long)span) > 11 ? 64 - __clzll((long long)span) - 11 : 0;   // span >> sft < 2048
+        for (int i = tid; i < kBins; i += 1024) hist[i] = 0;
+        if (tid == 0) s_n = 0;
+        __syncthreads();
+        for (int t = tid; t < n; t += 1024) {
+            const unsigned long long k = src.key(t, 0.0);
+            if (k >= lo && k <= hi) atomicAdd(&hist[(k - lo) >> sft], 1u);
+        }
+        __syncthreads();
+        const int h0 = (int)hist[2 * tid], h1 = (int)hist[2 * tid + 1];
+        const int off = block_excl_scan(h0 + h1, sh, &total);
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const int k = w ? k1 : k0;
+            if (k >= off && k < off + h0) { s_bin[w] = 2 * tid; if (w == 0) s_before = off; }
+            else if (k >= off + h0 && k < off + h0 + h1) { s_bin[w] = 2 * tid + 1; if (w == 0) s_before = off + h0; }
+        }
+        __syncthreads();
+        const unsigned long long a = lo + ((unsigned long long)s_bin[0] << sft);
+        const unsigned long long bb = lo + (((unsigned long long)s_bin[1] + 1ull) << sft) - 1ull, b = bb < hi ? bb : hi;
+        k0 -= s_before; k1 -= s_before;
+        for (int t = tid; t < n; t += 1024) {
+            const unsigned long long k = src.key(t, 0.0);
+            if (k >= a && k <= b) { const int at = atomicAdd(&s_n, 1); if (at < kCand) cand[at] = k; }
+        }
+        __syncthreads();
+        const int c = s_n;
+        if (c <= kCand) {
+            if (tid < c) {
+                const unsigned long long mine = cand[tid];
+                int rank = 0;
+                for (int j = 0; j < c; ++j) rank += cand[j] < mine || (cand[j] == mine && j < tid);
+                if (rank == k0) s_val[0] = mine;
+                if (rank == k1) s_val[1] = mine;
+            }
+            break;
+        }
+        if (s_bin[0] != s_bin[1]) {
+            // the middle falls between two crowded steps: the largest key of the first and the smallest of the next
+            const unsigned long long edge = lo + ((unsigned long long)(s_bin[0] + 1) << sft);
+            unsigned long long l = 0ull, h = ~0ull;
+            for (int t = tid; t < n; t += 1024) {
+                const unsigned long long k = src.key(t, 0.0);
+                if (k < edge) l = k > l ? k : l; else h = k < h ? k : h;
+            }
+            if (tid == 0) { s_val[0] = 0ull; s_val[1] = ~0ull; }
+            __syncthreads();
+            atomicMax(&s_val[0], l); atomicMin(&s_val[1], h);
+            break;
+        }
+        // the common step, narrowed to the keys it holds
+        unsigned long long l = ~0ull, h = 0ull;
+        for (int t = tid; t < n; t += 1024) {
+            const unsigned long long k = src.key(t, 0.0);
+            if (k >= a && k <= b) { l = k < l ? k : l; h = k > h ? k : h; }
+        }
+        if (tid == 0) { s_lo = ~0ull; s_hi = 0ull; }
+        __syncthreads();
+        atomicMin(&s_lo, l); atomicMax(&s_hi, h);
+        __syncthreads();
+        lo = s_lo; hi = s_hi;
+    }
+    __syncthreads();
+    if (tid == 0) *out = (n & 1) ? unflip(s_val[1]) : __dmul_rn(0.5, __dadd_rn(unflip(s_val[0]), unflip(s_val[1])));
 }
 
 template <class Src>
@@ -323,6 +324,7 @@ static cudaError_t run_median(Src src, int64_t n, double scale, bool absdev, dou
 
 // ------------------------------------------------------------------ outlier mask
 
+// Sixteen weights per thread and step: four 16-byte loads in flight, one 16-byte store of mask bytes.
 __global__ void __launch_bounds__(256) mask_threshold(const float* __restrict__ W, int64_t n,
                                                        const double* __restrict__ ms, double k, uint8_t* mask,
                                                        SelState* st) {
@@ -330,7 +332,22 @@ __global__ void __launch_bounds__(256) mask_threshold(const float* __restrict__ 
     const double mu = ms[0];
     const double thresh = __dmul_rn(k, ms[1]);
     int c = 0;
-    for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 256) {
+    const int64_t n16 = n >> 4;
+    for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < n16; t += (int64_t)gridDim.x * 256) {
+        const float4* p = (const float4*)W + 4 * t;
+        const float4 w[4] = {__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3)};
+        uint32_t o[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t a = fabs(__dsub_rn((double)w[u].x, mu)) > thresh, b = fabs(__dsub_rn((double)w[u].y, mu)) > thresh,
+                           d = fabs(__dsub_rn((double)w[u].z, mu)) > thresh, e = fabs(__dsub_rn((double)w[u].w, mu)) > thresh;
+            o[u] = a | (b << 8) | (d << 16) | (e << 24);
+            c += (int)(a + b + d + e);
+        }
+        ((uint4*)mask)[t] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    if (blockIdx.x == 0 && (int64_t)threadIdx.x < (n & 15)) {
+        const int64_t t = (n & ~(int64_t)15) + threadIdx.x;
         const int m = fabs(__dsub_rn((double)W[t], mu)) > thresh;
         mask[t] = (uint8_t)m;
         c += m;
@@ -348,14 +365,15 @@ __global__ void __launch_bounds__(256) mask_threshold(const float* __restrict__ 
 __global__ void outlier_zero(SelState* st) { st->count = 0; }
 
 // Decide what the selection has to do.  mode 0: keep = floor(cap*n), select only when more qualified.
-// mode 1: keep = floor(rate*n) of all weights.
-__global__ void outlier_plan(SelState* st, int64_t n, int mode, double frac, int64_t* count_out) {
+// mode 1: keep = floor(rate*n) of all weights.  skip_out (may be null): a copy of the decision for the host.
+__global__ void outlier_plan(SelState* st, int64_t n, int mode, double frac, int64_t* count_out, int64_t* skip_out) {
     const long long keep = (long long)floor(__dmul_rn(frac, (double)n));
+    if (threadIdx.x < 256) st->hist[threadIdx.x] = 0;
+    if (threadIdx.x) return;
     st->keep = keep;
     st->prefix = 0;
     st->shift = 56;
     st->descending = 1;
-    for (int j = 0; j < 256; ++j) st->hist[j] = 0;
     if (mode == 0) {
         st->skip = st->count <= keep;
         st->k = keep - 1;
@@ -366,6 +384,7 @@ __global__ void outlier_plan(SelState* st, int64_t n, int mode, double frac, int
         st->k = keep - 1;
         *count_out = keep > 0 ? keep : 0;
     }
+    if (skip_out) *skip_out = st->skip;
 }
 
 __global__ void __launch_bounds__(256) mask_clear(uint8_t* mask, int64_t n) {
@@ -439,276 +458,6 @@ __global__ void __launch_bounds__(256) tie_apply(Src src, int64_t n, const SelSt
     }
 }
 
-// ------------------------------------------------------------------ Lloyd, one channel per block
-
-constexpr int kLloydThreads = 256;
-
-#ifdef XFP_TRACE
-// phase boundaries of block 0 (clock64), read back by xfp_debug_lloyd_phases: a timing probe
-__device__ long long g_lloyd_phase[8];
-#define LLOYD_STAMP(i) do { if (blockIdx.x == 0 && threadIdx.x == 0) g_lloyd_phase[i] = clock64(); } while (0)
-#else
-#define LLOYD_STAMP(i) do { } while (0)
-#endif
-
-__device__ __forceinline__ double bulk_value(const float* __restrict__ W, const uint8_t* __restrict__ mask,
-                                             int64_t t, double mu) {
-    return (mask != nullptr && mask[t]) ? mu : (double)W[t];
-}
-
-// Compare-exchange of the bitonic network: after it a <= b when `asc`, a >= b otherwise; equal keys stay put.
-__device__ __forceinline__ void cswap(float& a, float& b, bool asc) {
-    const bool sw = (a > b) == asc;
-    const float x = sw ? b : a, y = sw ? a : b;
-    a = x;
-    b = y;
-}
-// the stages with partner distance 4, 2, 1 on eight consecutive elements
-__device__ __forceinline__ void last3(float (&v)[8], bool asc) {
-    cswap(v[0], v[4], asc); cswap(v[1], v[5], asc); cswap(v[2], v[6], asc); cswap(v[3], v[7], asc);
-    cswap(v[0], v[2], asc); cswap(v[1], v[3], asc); cswap(v[4], v[6], asc); cswap(v[5], v[7], asc);
-    cswap(v[0], v[1], asc); cswap(v[2], v[3], asc); cswap(v[4], v[5], asc); cswap(v[6], v[7], asc);
-}
-__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
-    const float4 a = *(const float4*)p, b = *(const float4*)(p + 4);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-__device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
-    *(float4*)p = make_float4(v[0], v[1], v[2], v[3]);
-    *(float4*)(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
-}
-
-// The channel's bulk values in ascending order without storing them as doubles: the weights that were not
-// extracted, sorted as floats, with the m copies of mu (one per extracted position) inserted at p0.
-struct SortedBulk {
-    const float* r;
-    int p0, m;
-    double mu;
-    __device__ __forceinline__ double at(int t) const {   // one load, then a select: no branch
-        const int u = t < p0 ? t : (t - m > 0 ? t - m : 0);
-        const double v = (double)r[u];
-        return (t >= p0 && t < p0 + m) ? mu : v;
-    }
-};
-
-// LONG = false: one channel per CTA, its two arrays in shared memory (channels of up to 16384 weights).
-// LONG = true: the arrays live in a slice of global scratch owned by the CTA (L1/L2 resident; the CTA's own
-// writes are ordered by its barriers) and the resident CTAs walk the channels; any length the format allows.
-template <bool LONG>
-__global__ void __launch_bounds__(kLloydThreads, 4) lloyd_kernel(const float* __restrict__ W,
-                                                               const uint8_t* __restrict__ mask,
-                                                               const double* __restrict__ ms, int rows, int K, int Kp2,
-                                                               int bits, int iters, uint16_t* __restrict__ cb16,
-                                                               uint8_t* __restrict__ idx, double* scratch,
-                                                               size_t slice_doubles) {
-    extern __shared__ __align__(16) double sm[];
-    double* base = LONG ? scratch + (size_t)blockIdx.x * slice_doubles : sm;
-    double* pre = base;                      // [K + 1] serial prefix sums of the sorted bulk values
-    float* r = (float*)(base + ((K + 2) & ~1));   // [Kp2] kept weights, ascending (extracted slots and padding = +inf); 16-byte aligned
-    __shared__ double c[64];
-    __shared__ double e16[64];
-    __shared__ int cut[65];
-    __shared__ int s_m, s_p0;
-    const int tid = threadIdx.x;
-    const int E = 1 << bits;
-    const double mu = ms[0];
-
-#pragma unroll 1
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-    const int64_t row0 = (int64_t)row * K;
-    LLOYD_STAMP(0);
-    if (tid == 0) s_m = 0;
-    __syncthreads();
-    int extracted = 0;
-    for (int kb = tid; kb < Kp2; kb += 8 * kLloydThreads) {   // eight loads in flight per thread
-        float v[8];
-        uint8_t x[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = kb + e * kLloydThreads;
-            v[e] = k < K ? W[row0 + k] : INFINITY;
-            x[e] = (k < K && mask != nullptr) ? mask[row0 + k] : (uint8_t)0;
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = kb + e * kLloydThreads;
-            if (k < Kp2) r[k] = x[e] ? INFINITY : v[e];
-            extracted += x[e] != 0;
-        }
-    }
-    if (extracted) atomicAdd(&s_m, extracted);
-    __syncthreads();
-    LLOYD_STAMP(1);
-    // bitonic sort, ascending.  The stages with partner distance 4, 2, 1 stay inside blocks of 8 consecutive
-    // elements and run in registers (one pass per step instead of three trips through the array); the wider
-    // stages go through the array, a thread's eight pairs loaded before any is written back.
-    const int half = Kp2 >> 1, nblk8 = Kp2 >> 3;
-    for (int b8 = tid; b8 < nblk8; b8 += kLloydThreads) {   // steps 2, 4 and 8 entirely in registers
-        float v[8];
-        load8(r + 8 * b8, v);
-        cswap(v[0], v[1], true); cswap(v[2], v[3], false); cswap(v[4], v[5], true); cswap(v[6], v[7], false);
-        cswap(v[0], v[2], true); cswap(v[1], v[3], true); cswap(v[4], v[6], false); cswap(v[5], v[7], false);
-        cswap(v[0], v[1], true); cswap(v[2], v[3], true); cswap(v[4], v[5], false); cswap(v[6], v[7], false);
-        last3(v, ((8 * b8) & 8) == 0);
-        store8(r + 8 * b8, v);
-    }
-    __syncthreads();
-    for (int size = 16; size <= Kp2; size <<= 1) {
-        for (int j = size >> 1; j >= 8; j >>= 1) {
-            for (int pb = tid; pb < half; pb += 8 * kLloydThreads) {
-                int ia[8];
-                float a[8], b[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int p = pb + e * kLloydThreads;
-                    ia[e] = p < half ? (((p & ~(j - 1)) << 1) | (p & (j - 1))) : -1;
-                    if (ia[e] >= 0) { a[e] = r[ia[e]]; b[e] = r[ia[e] + j]; }
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (ia[e] >= 0 && (a[e] > b[e]) == ((ia[e] & size) == 0)) { r[ia[e]] = b[e]; r[ia[e] + j] = a[e]; }
-            }
-            __syncthreads();
-        }
-        for (int b8 = tid; b8 < nblk8; b8 += kLloydThreads) {
-            float v[8];
-            load8(r + 8 * b8, v);
-            last3(v, ((8 * b8) & size) == 0);
-            store8(r + 8 * b8, v);
-        }
-        __syncthreads();
-    }
-    LLOYD_STAMP(2);
-    if (tid == 0) {   // where mu sits among the kept weights
-        int lo = 0, hi = K - s_m;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if ((double)r[mid] <= mu) lo = mid + 1; else hi = mid;
-        }
-        s_p0 = lo;
-    }
-    __syncthreads();
-    SortedBulk s{r, s_p0, s_m, mu};
-    // serial prefix sums: cell sums below are differences of these, as in a one-pass CPU evaluation.
-    // All threads first lay the sorted values out as doubles in pre[1..K]; one thread then scans in place,
-    // fetching the next eight values before it starts the current chain of eight dependent adds.
-    for (int t = tid; t < K; t += kLloydThreads) pre[t + 1] = s.at(t);
-    __syncthreads();
-    if (tid == 0) {
-        double run = 0.0;
-        double f[8], g[8];
-        pre[0] = 0.0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] = pre[1 + e];
-        for (int t = 0; t < K; t += 8) {   // K is a multiple of 128
-            if (t + 8 < K) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) g[e] = pre[t + 9 + e];
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                run = __dadd_rn(run, f[e]);
-                f[e] = run;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) pre[t + 1 + e] = f[e];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) f[e] = g[e];
-        }
-    }
-    if (tid >= 32 && tid < 32 + E) {   // a warp other than the one that runs the prefix
-        const int j = tid - 32;
-        long long q = (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)j, 0.5), (double)K), (double)E));
-        if (q >= K) q = K - 1;
-        c[j] = s.at((int)q);
-    }
-    if (tid == 32) { cut[0] = 0; cut[E] = K; }
-    __syncthreads();
-    LLOYD_STAMP(3);
-
-    // P lanes share one boundary search (P = 256 / 2^N, at most a warp): each round probes P positions of
-    // the remaining range at once, so 4096 values take three rounds at N = 4 instead of twelve steps.
-    const int P = (kLloydThreads >> bits) > 32 ? 32 : (kLloydThreads >> bits);
-    const int jb = tid / P, sub = tid % P;
-    const unsigned gmask = (P == 32 ? 0xffffffffu : ((1u << P) - 1u)) << ((tid & 31) & ~(P - 1));
-    for (int it = 0; it < iters; ++it) {
-        // cell j = (b_{j-1}, b_j], b_j the midpoint of entries j and j+1: cut[j+1] = #{t : s[t] <= b_j}
-        {
-            const bool mine = jb < E - 1;
-            const double b = mine ? __dmul_rn(0.5, __dadd_rn(c[jb], c[jb + 1])) : 0.0;
-            int lo = 0, hi = mine ? K : 0;   // every t < lo has s[t] <= b, every t >= hi has s[t] > b
-            while (__any_sync(0xffffffffu, lo < hi)) {
-                const int step = (hi - lo + P - 1) / P;
-                const int pos = lo + (sub + 1) * step - 1;
-                const bool below = lo < hi && pos < hi && s.at(pos) <= b;
-                const int cnt = __popc(__ballot_sync(0xffffffffu, below) & gmask);   // the probes are ordered
-                if (lo < hi) {
-                    const int nlo = lo + cnt * step;
-                    const int nhi = cnt < P ? lo + (cnt + 1) * step - 1 : hi;
-                    lo = nlo < hi ? nlo : hi;
-                    hi = nhi < hi ? nhi : hi;
-                    if (hi < lo) hi = lo;
-                }
-            }
-            if (mine && sub == 0) cut[jb + 1] = lo;
-        }
-        __syncthreads();
-        int changed = 0;
-        if (tid < E) {
-            const int n = cut[tid + 1] - cut[tid];
-            if (n > 0) {
-                const double mean = __ddiv_rn(__dsub_rn(pre[cut[tid + 1]], pre[cut[tid]]), (double)n);
-                if (mean != c[tid]) { c[tid] = mean; changed = 1; }
-            }
-        }
-        if (!__syncthreads_or(changed)) break;
-    }
-    LLOYD_STAMP(4);
-    if (tid < E) {
-        const uint16_t h = d2h(c[tid]);
-        cb16[(int64_t)row * E + tid] = h;
-        e16[tid] = h2d(h);
-    }
-    __syncthreads();
-    // every weight goes to the nearest STORED entry (ties: lower index), four weights per thread at a time.  Up to
-    // 16 entries the plain scan with four chains of compares in flight is the faster form; above, bisection.
-    bool e_asc = E > 16;
-    for (int j = 1; j < E && e_asc; ++j) e_asc = e16[j] >= e16[j - 1];
-    for (int kb = tid; kb < K; kb += 4 * kLloydThreads) {
-        double v[4], bd[4];
-        int best[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int k = kb + e * kLloydThreads;
-            v[e] = k < K ? bulk_value(W, mask, row0 + k, mu) : 0.0;
-        }
-        if (e_asc) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) best[e] = nearest_entry(e16, E, v[e], true);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { bd[e] = fabs(__dsub_rn(v[e], e16[0])); best[e] = 0; }
-            for (int j = 1; j < E; ++j) {
-                const double ej = e16[j];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const double d = fabs(__dsub_rn(v[e], ej));
-                    if (d < bd[e]) { bd[e] = d; best[e] = j; }
-                }
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int k = kb + e * kLloydThreads;
-            if (k < K) idx[row0 + k] = (uint8_t)best[e];
-        }
-    }
-    LLOYD_STAMP(5);
-    if (!LONG) break;  // one channel per CTA
-    __syncthreads();   // the arrays and the small tables are reused by the CTA's next channel
-    }
-}
-
 // ------------------------------------------------------------------ decoded value of a stored index
 
 struct Unpacked {
@@ -728,77 +477,116 @@ __device__ __forceinline__ uint16_t decode16(const Unpacked& u, int row, int k) 
 
 // ------------------------------------------------------------------ residual (CSR)
 
-__global__ void __launch_bounds__(256) row_count_kernel(const uint8_t* __restrict__ mask, int K, int* cnt) {
-    __shared__ int sh[8];
-    __shared__ int total;
-    const uint8_t* m = mask + (int64_t)blockIdx.x * K;
+__global__ void __launch_bounds__(256) row_count_kernel(const uint8_t* __restrict__ mask, int rows, int K, int* cnt) {
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const uint32_t* m = (const uint32_t*)(mask + (int64_t)row * K);
     int c = 0;
-    for (int k = threadIdx.x; k < K; k += 256) c += m[k] != 0;
-    block_excl_scan(c, sh, &total);
-    if (threadIdx.x == 0) cnt[blockIdx.x] = total;
+#pragma unroll 8
+    for (int k = lane; k < K / 4; k += 32) c += __popc(__vcmpne4(__ldg(m + k), 0u)) >> 3;
+    for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
+    if (lane == 0) cnt[row] = c;
 }
 
-__global__ void __launch_bounds__(1024) rowptr_scan(const int* cnt, int rows, int32_t* rowptr) {
+// One block; every thread owns a run of consecutive rows.
+__global__ void __launch_bounds__(1024) rowptr_scan(const int* __restrict__ cnt, int rows, int32_t* rowptr) {
     __shared__ int sh[32];
     __shared__ int total;
-    int carry = 0;
-    for (int b0 = 0; b0 < rows; b0 += 1024) {
-        const int b = b0 + threadIdx.x;
-        const int v = b < rows ? cnt[b] : 0;
-        const int off = block_excl_scan(v, sh, &total);
-        if (b < rows) rowptr[b] = carry + off;
-        carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) rowptr[rows] = carry;
+    const int per = (rows + 1023) / 1024, b0 = threadIdx.x * per, b1 = b0 + per < rows ? b0 + per : rows;
+    int v = 0;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) v += cnt[b];
+    int run = block_excl_scan(v, sh, &total);
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) { const int x = cnt[b]; rowptr[b] = run; run += x; }
+    if (threadIdx.x == 0) rowptr[rows] = total;
 }
 
+// A warp per channel: the mask is read 128 weights at a time (a word per lane, the next four in flight); where a word is set
+// the places of its entries follow from four ballots, one per byte, without a barrier.
 __global__ void __launch_bounds__(256) residual_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask,
-                                                        Unpacked u, const int32_t* __restrict__ rowptr,
+                                                        Unpacked u, int rows, const int32_t* __restrict__ rowptr,
                                                         int32_t* ocol, uint16_t* oval, int64_t capacity) {
-    __shared__ int sh[8];
-    __shared__ int total;
-    const int row = blockIdx.x;
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
     int64_t p = rowptr[row];
     if (rowptr[row + 1] == p) return;
-    for (int k0 = 0; k0 < u.K; k0 += 256) {
-        const int k = k0 + threadIdx.x;
-        const int64_t t = (int64_t)row * u.K + k;
-        const int f = k < u.K && mask[t] != 0;
-        const int off = block_excl_scan(f, sh, &total);
-        if (f && p + off < capacity) {
-            ocol[p + off] = k;
-            oval[p + off] = d2h(__dsub_rn((double)W[t], h2d(decode16(u, row, k))));
+    const uint32_t* m4 = (const uint32_t*)(mask + (int64_t)row * u.K);
+    const uint32_t below = (1u << lane) - 1u;
+    const int words = u.K / 4;          // a multiple of 32
+    for (int w0 = 0; w0 < words; w0 += 128) {
+        uint32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = w0 + 32 * i < words ? __ldg(m4 + w0 + 32 * i + lane) : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (!__any_sync(0xffffffffu, x[i])) continue;
+            int before = 0, tot = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint32_t v = __ballot_sync(0xffffffffu, (x[i] >> (8 * b)) & 0xffu);
+                before += __popc(v & below); tot += __popc(v);
+            }
+            int64_t at = p + before;
+            for (int b = 0; b < 4; ++b) {
+                if (!((x[i] >> (8 * b)) & 0xffu)) continue;
+                if (at < capacity) {
+                    const int k = (w0 + 32 * i + lane) * 4 + b;
+                    ocol[at] = k;
+                    oval[at] = d2h(__dsub_rn((double)W[(int64_t)row * u.K + k], h2d(decode16(u, row, k))));
+                }
+                ++at;
+            }
+            p += tot;
         }
-        p += total;
-        __syncthreads();
     }
 }
 
 // ------------------------------------------------------------------ per-channel cosine
 
+// A warp per channel, four weights per lane and step; fp64 sums.
 __global__ void __launch_bounds__(256) cosine_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask,
-                                                      Unpacked u, double* cosv) {
-    __shared__ double sh[256];
-    const int row = blockIdx.x;
+                                                      Unpacked u, int rows, double* cosv) {
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const float4* w4 = (const float4*)(W + (int64_t)row * u.K);
+    const uint32_t* i4 = (const uint32_t*)(u.idx + (int64_t)row * u.K);
+    const uint8_t* mrow = mask ? mask + (int64_t)row * u.K : nullptr;
+    const bool words = ((uintptr_t)mask & 3u) == 0;      // the public call takes a mask at any address
     double ab = 0.0, aa = 0.0, bb = 0.0;
-    for (int k = threadIdx.x; k < u.K; k += 256) {
-        const int64_t t = (int64_t)row * u.K + k;
-        const double a = (double)W[t];
-        const uint16_t d16 = decode16(u, row, k);
-        double b = h2d(d16);
-        if (mask != nullptr && mask[t]) {
-            const uint16_t s16 = d2h(__dsub_rn(a, b));           // the stored residual
-            b = h2d(d2h(__dadd_rn(b, h2d(s16))));                // W^ = fp16(D16 + S), one rounding
+#pragma unroll 4
+    for (int q = lane; q < u.K / 4; q += 32) {
+        const float4 w = __ldg(w4 + q);
+        const uint32_t ix = __ldg(i4 + q);
+        uint32_t x = 0;
+        if (mrow) {
+            if (words) x = __ldg((const uint32_t*)mrow + q);
+            else for (int i = 0; i < 4; ++i) x |= (uint32_t)mrow[4 * q + i] << (8 * i);
         }
-        ab = __dadd_rn(ab, __dmul_rn(a, b));
-        aa = __dadd_rn(aa, __dmul_rn(a, a));
-        bb = __dadd_rn(bb, __dmul_rn(b, b));
+        const float f[4] = {w.x, w.y, w.z, w.w};
+        const uint16_t* book = u.cb + (int64_t)row * u.E;
+        uint16_t sc = 0, mid = 0;
+        if (u.mode) {
+            const int64_t g = (int64_t)row * u.G + q * 4 / u.group;      // four weights never straddle two groups
+            book = u.cb + (int)u.gid[g] * u.E; sc = u.gscale[g]; mid = u.gmid[g];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint16_t e = __ldg(book + ((ix >> (8 * i)) & 0xffu));
+            const double a = (double)f[i];
+            double b = h2d(u.mode ? v2a_value16(sc, e, mid) : e);
+            if ((x >> (8 * i)) & 0xffu) {
+                const uint16_t s16 = d2h(__dsub_rn(a, b));           // the stored residual
+                b = h2d(d2h(__dadd_rn(b, h2d(s16))));                // W^ = fp16(D16 + S), one rounding
+            }
+            ab = fma(a, b, ab); aa = fma(a, a, aa); bb = fma(b, b, bb);
+        }
     }
-    ab = block_sum(ab, sh);
-    aa = block_sum(aa, sh);
-    bb = block_sum(bb, sh);
-    if (threadIdx.x == 0)
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        ab += __shfl_xor_sync(0xffffffffu, ab, d); aa += __shfl_xor_sync(0xffffffffu, aa, d); bb += __shfl_xor_sync(0xffffffffu, bb, d);
+    }
+    if (lane == 0)
         cosv[row] = (aa == 0.0 || bb == 0.0) ? 1.0 : __ddiv_rn(ab, __dmul_rn(__dsqrt_rn(aa), __dsqrt_rn(bb)));
 }
 
@@ -1051,7 +839,7 @@ __global__ void __launch_bounds__(GS) libfit_group_kernel(const float* __restric
 // ------------------------------------------------------------------ host side
 
 struct Workspace {
-    double* part;      // [kRedBlocks]
+    double2* part;     // [kRedBlocks]
     SelState* sel;
     int* flags;        // [2] LibFit changed / done
     int* tie;          // [ceil(n / kTieChunk)]
@@ -1072,7 +860,7 @@ static Workspace carve(void* base, int64_t rows, int64_t cols) {
     size_t o = 0;
     auto take = [&](size_t bytes) { char* r = p + o; o += align256(bytes); return r; };
     const int64_t n = rows * cols;
-    w.part = (double*)take(sizeof(double) * kRedBlocks);
+    w.part = (double2*)take(sizeof(double2) * kRedBlocks);
     w.sel = (SelState*)take(sizeof(SelState));
     w.flags = (int*)take(sizeof(int) * 2);
     w.tie = (int*)take(sizeof(int) * (size_t)((n + kTieChunk - 1) / kTieChunk + 1));
@@ -1082,13 +870,8 @@ static Workspace carve(void* base, int64_t rows, int64_t cols) {
     w.order = (int*)take(sizeof(int) * (size_t)rows);
     w.asg = (int*)take(sizeof(int) * (size_t)rows);
     w.cen = (double*)take(sizeof(double) * 256 * 64);
-    if (cols > 16384) {   // channels too long for shared memory: the Lloyd kernel's arrays (it uses the scratch from its start)
-        size_t kp2 = 1;
-        while ((int64_t)kp2 < cols) kp2 <<= 1;
-        const size_t slice = (((size_t)cols + 2) & ~(size_t)1) + kp2 / 2;
-        const size_t need = slice * sizeof(double) * (size_t)(rows < 2 * xfp::kSizingSMs ? rows : 2 * xfp::kSizingSMs);
-        if (o < need) o = align256(need);
-    }
+    const size_t lloyd = lloyd_scratch_bytes((int)rows, (int)cols);   // the Lloyd kernel uses the scratch from its start
+    if (o < lloyd) o = align256(lloyd);
     w.bytes = o;
     return w;
 }
@@ -1099,13 +882,6 @@ static int shape_status(int64_t rows, int64_t cols) {
     if (rows < 1 || cols < 128 || cols % 128 != 0) return XFP_ERR_SHAPE;
     if (cols > 65536 || rows > (1 << 24)) return XFP_ERR_UNSUPPORTED;
     return XFP_OK;
-}
-
-static int lloyd_smem(int cols, int* kp2_out) {
-    int kp2 = 1;
-    while (kp2 < cols) kp2 <<= 1;
-    *kp2_out = kp2;
-    return (int)(sizeof(double) * (((size_t)cols + 2) & ~(size_t)1) + sizeof(float) * (size_t)kp2);
 }
 
 static Unpacked unpacked_of(const xfp_desc* d, const uint8_t* idx, const uint16_t* cb, const uint8_t* gid,
@@ -1125,6 +901,33 @@ static int desc_status(const xfp_desc* d) {
     if (d->cols > 0 && d->cols % d->group_size) return XFP_ERR_SHAPE;
     if (d->mode == 1 && (d->lib_size < 1 || d->lib_size > 256)) return XFP_ERR_SHAPE;
     return shape_status(d->rows, d->cols);
+}
+
+// Extraction, first half: the candidates in `mask` (mode 0: above the threshold) and the plan of the selection.
+static void outliers_candidates(const float* W, int64_t n, const double* ms, int mode, double k_or_rate, double cap_frac,
+                                uint8_t* mask, int64_t* count, int64_t* skip_out, const Workspace& w, cudaStream_t s) {
+    const int64_t nblk = (n + kTieChunk - 1) / kTieChunk, cap = (int64_t)xfp::sm_count() * 8;
+    const int sweep = (int)(nblk < cap ? (nblk < 1 ? 1 : nblk) : cap);
+    if (mode == 0) {
+        outlier_zero<<<1, 1, 0, s>>>(w.sel);
+        mask_threshold<<<sweep, 256, 0, s>>>(W, n, ms, k_or_rate, mask, w.sel);
+        outlier_plan<<<1, 256, 0, s>>>(w.sel, n, 0, cap_frac, count, skip_out);
+    } else {
+        mask_clear<<<sweep, 256, 0, s>>>(mask, n);
+        outlier_plan<<<1, 256, 0, s>>>(w.sel, n, 1, k_or_rate, count, skip_out);
+    }
+}
+// Second half: the largest |w - mu| of the candidates, ties by position.  A no-op on the device where the plan says skip.
+static cudaError_t outliers_select(const float* W, int64_t n, const double* ms, int mode, uint8_t* mask, const Workspace& w,
+                                   cudaStream_t s) {
+    const unsigned nblk = (unsigned)((n + kTieChunk - 1) / kTieChunk);
+    const SrcAbsDev src{W, ms, mode == 0 ? mask : nullptr};
+    const cudaError_t e = run_select(src, n, w.sel, s);
+    if (e != cudaSuccess) return e;
+    tie_count<SrcAbsDev><<<nblk, 256, 0, s>>>(src, n, w.sel, w.tie);
+    tie_scan<<<1, 1024, 0, s>>>(w.tie, (int)nblk, w.sel);
+    tie_apply<SrcAbsDev><<<nblk, 256, 0, s>>>(src, n, w.sel, w.tie, mask);
+    return cudaGetLastError();
 }
 
 }  // namespace xq
@@ -1149,12 +952,9 @@ int xfp_quant_stats(const float* W, int64_t n, int32_t sigma_mode, double* mu_si
     if (workspace_bytes < carve(nullptr, 1, 128).bytes) return XFP_ERR_BUFFER_TOO_SMALL;
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(workspace, 1, 128);
-    stats_partial<0><<<kRedBlocks, kRedThreads, 0, s>>>(W, n, mu_sigma, w.part);
-    stats_final<0><<<1, kRedThreads, 0, s>>>(w.part, n, mu_sigma);
-    if (sigma_mode == 0) {
-        stats_partial<1><<<kRedBlocks, kRedThreads, 0, s>>>(W, n, mu_sigma, w.part);
-        stats_final<1><<<1, kRedThreads, 0, s>>>(w.part, n, mu_sigma);
-    } else {
+    stats_partial<<<kRedBlocks, kRedThreads, 0, s>>>(W, n, w.part);
+    stats_final<<<1, kRedThreads, 0, s>>>(w.part, n, mu_sigma);
+    if (sigma_mode == 1) {
         SrcAbsDev src{W, mu_sigma, nullptr};
         if (run_median(src, n, 1.4826, true, mu_sigma + 1, w.sel, s) != cudaSuccess) return XFP_ERR_CUDA;
     }
@@ -1176,32 +976,10 @@ int xfp_quant_outliers(const float* W, int64_t n, const double* mu_sigma, int32_
     if (workspace_bytes < tie_offset + (size_t)nblk * sizeof(int)) return XFP_ERR_BUFFER_TOO_SMALL;
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(workspace, 1, 128);   // part, sel, flags, then the tie counters
-    const int64_t sweep_cap = (int64_t)xfp::sm_count() * 8;
-    const int sweep = (int)(nblk < sweep_cap ? (nblk < 1 ? 1 : nblk) : sweep_cap);
-    if (outlier_mode == 0) {
-        outlier_zero<<<1, 1, 0, s>>>(w.sel);
-        mask_threshold<<<sweep, 256, 0, s>>>(W, n, mu_sigma, k_or_rate, mask, w.sel);
-        outlier_plan<<<1, 1, 0, s>>>(w.sel, n, 0, cap_frac, count);
-        SrcAbsDev src{W, mu_sigma, mask};
-        if (run_select(src, n, w.sel, s) != cudaSuccess) return XFP_ERR_CUDA;
-        tie_count<SrcAbsDev><<<(unsigned)nblk, 256, 0, s>>>(src, n, w.sel, w.tie);
-        tie_scan<<<1, 1024, 0, s>>>(w.tie, (int)nblk, w.sel);
-        tie_apply<SrcAbsDev><<<(unsigned)nblk, 256, 0, s>>>(src, n, w.sel, w.tie, mask);
-    } else {
-        mask_clear<<<sweep, 256, 0, s>>>(mask, n);
-        outlier_plan<<<1, 1, 0, s>>>(w.sel, n, 1, k_or_rate, count);
-        SrcAbsDev src{W, mu_sigma, nullptr};
-        if (run_select(src, n, w.sel, s) != cudaSuccess) return XFP_ERR_CUDA;
-        tie_count<SrcAbsDev><<<(unsigned)nblk, 256, 0, s>>>(src, n, w.sel, w.tie);
-        tie_scan<<<1, 1024, 0, s>>>(w.tie, (int)nblk, w.sel);
-        tie_apply<SrcAbsDev><<<(unsigned)nblk, 256, 0, s>>>(src, n, w.sel, w.tie, mask);
-    }
+    outliers_candidates(W, n, mu_sigma, outlier_mode, k_or_rate, cap_frac, mask, count, nullptr, w, s);
+    if (outliers_select(W, n, mu_sigma, outlier_mode, mask, w, s) != cudaSuccess) return XFP_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
-
-// long channels: resident CTAs, each with a slice of scratch for its two arrays
-// (the scratch is sized for two CTAs on each of kSizingSMs SMs; a launch never uses more)
-static size_t lloyd_slice_doubles(int cols, int kp2) { return (((size_t)cols + 2) & ~(size_t)1) + (size_t)kp2 / 2; }
 
 int xfp_quant_lloyd(const float* W, const uint8_t* mask, const double* mu_sigma, int32_t rows, int32_t cols,
                     int32_t bits, int32_t iters, uint16_t* codebook, uint8_t* idx, void* workspace,
@@ -1211,25 +989,14 @@ int xfp_quant_lloyd(const float* W, const uint8_t* mask, const double* mu_sigma,
     const int st = shape_status(rows, cols);
     if (st) return st;
     if (bits < 2 || bits > 6 || iters < 0) return XFP_ERR_SHAPE;
-    int kp2;
-    const int smem = lloyd_smem(cols, &kp2);
-    if (smem <= 227 * 1024 - 2048) {
-        if (cudaFuncSetAttribute(lloyd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-            cudaFuncSetAttribute(lloyd_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
-            return XFP_ERR_CUDA;
-        lloyd_kernel<false><<<rows, kLloydThreads, smem, (cudaStream_t)stream>>>(W, mask, mu_sigma, rows, cols, kp2, bits,
-                                                                                 iters, codebook, idx, nullptr, 0);
-    } else {
+    const size_t scratch = lloyd_scratch_bytes(rows, cols);
+    if (scratch) {
         if (!workspace) return XFP_ERR_NULL;
         if (!aligned16(workspace)) return XFP_ERR_ALIGN;
-        const size_t slice = lloyd_slice_doubles(cols, kp2);
-        const int want = 2 * xfp::sched_sms();   // two resident CTAs per SM
-        const int ctas = rows < want ? rows : want;
-        if (workspace_bytes < slice * sizeof(double) * (size_t)ctas) return XFP_ERR_BUFFER_TOO_SMALL;
-        lloyd_kernel<true><<<ctas, kLloydThreads, 0, (cudaStream_t)stream>>>(W, mask, mu_sigma, rows, cols, kp2, bits, iters,
-                                                                             codebook, idx, (double*)workspace, slice);
+        if (workspace_bytes < scratch) return XFP_ERR_BUFFER_TOO_SMALL;
     }
-    return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    return launch_lloyd(W, mask, mu_sigma, rows, cols, bits, iters, codebook, idx, nullptr, nullptr, workspace,
+                        (cudaStream_t)stream) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
 
 int xfp_quant_libfit_library(const uint16_t* codebook, int32_t rows, int32_t bits, int32_t L, int32_t iters,
@@ -1304,10 +1071,11 @@ int xfp_quant_residual(const xfp_desc* desc, const float* W, const uint8_t* mask
     if (workspace_bytes < carve(nullptr, desc->rows, desc->cols).bytes) return XFP_ERR_BUFFER_TOO_SMALL;
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(workspace, desc->rows, desc->cols);
-    row_count_kernel<<<desc->rows, 256, 0, s>>>(mask, desc->cols, w.rowcnt);
+    const unsigned grid = (unsigned)((desc->rows + 7) / 8);
+    row_count_kernel<<<grid, 256, 0, s>>>(mask, desc->rows, desc->cols, w.rowcnt);
     rowptr_scan<<<1, 1024, 0, s>>>(w.rowcnt, desc->rows, out_rowptr);
-    residual_kernel<<<desc->rows, 256, 0, s>>>(W, mask, unpacked_of(desc, idx, codebook, gid, gscale, gmid), out_rowptr,
-                                               out_col, out_val, capacity);
+    residual_kernel<<<grid, 256, 0, s>>>(W, mask, unpacked_of(desc, idx, codebook, gid, gscale, gmid), desc->rows, out_rowptr,
+                                         out_col, out_val, capacity);
     return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
 
@@ -1318,8 +1086,8 @@ int xfp_quant_cosine(const xfp_desc* desc, const float* W, const uint8_t* mask, 
     if (st) return st;
     if (!cos) return XFP_ERR_NULL;
     if (!aligned16(cos) || (mask && !aligned16(mask))) return XFP_ERR_ALIGN;
-    cosine_kernel<<<desc->rows, 256, 0, (cudaStream_t)stream>>>(W, mask, unpacked_of(desc, idx, codebook, gid, gscale, gmid),
-                                                                cos);
+    cosine_kernel<<<(unsigned)((desc->rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(
+        W, mask, unpacked_of(desc, idx, codebook, gid, gscale, gmid), desc->rows, cos);
     return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
 
@@ -1356,25 +1124,31 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
     if (st) return st;
     size_t need;
     xfp_quant_workspace_size(rows, cols, &need);
-    // two doubles (mu, sigma), the median and the count live behind the carved scratch
+    // mu, sigma, the median, the count and the extraction's plan live behind the carved scratch
     if (workspace_bytes < need + 256) return XFP_ERR_BUFFER_TOO_SMALL;
+    if (!aligned16(W) || !aligned16(mask) || !aligned16(workspace) || !aligned16(codebook) || !aligned16(idx)) return XFP_ERR_ALIGN;
+    if (p->lloyd_iters < 0 || (p->outlier_mode != 0 && p->outlier_mode != 1) || (p->outlier_mode == 0 ? !(p->k_sigma >= 0.0) || !(p->cap_frac >= 0.0 && p->cap_frac <= 1.0)
+                                                                              : !(p->rate >= 0.0 && p->rate <= 1.0)))
+        return XFP_ERR_SHAPE;
     cudaStream_t s = (cudaStream_t)stream;
-    double* ms = (double*)((char*)workspace + need);
-    double* med_dev = ms + 2;
-    int64_t* cnt_dev = (int64_t*)(ms + 4);
+    struct Head { double mu, sigma, med, pad; int64_t count, skip; } host;
+    Head* dev = (Head*)((char*)workspace + need);
+    double* ms = &dev->mu;
+    double* med_dev = &dev->med;
     const int64_t n = (int64_t)rows * cols;
 
     st = xfp_quant_stats(W, n, p->sigma_mode, ms, workspace, need, stream);
     if (st) return st;
-    st = xfp_quant_outliers(W, n, ms, p->outlier_mode, p->outlier_mode ? p->rate : p->k_sigma, p->cap_frac, mask,
-                            cnt_dev, workspace, need, stream);
-    if (st) return st;
-    double host_ms[2];
-    int64_t host_cnt = 0;
-    if (cudaMemcpyAsync(host_ms, ms, sizeof(host_ms), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(&host_cnt, cnt_dev, sizeof(host_cnt), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    // One read-back tells the host the count and whether the cap (or a fixed rate) calls for a selection at all: the
+    // selection is twenty small launches, 2 - 3 us each even where every one of them returns at once.
+    const Workspace small = carve(workspace, 1, 128);
+    outliers_candidates(W, n, ms, p->outlier_mode, p->outlier_mode ? p->rate : p->k_sigma, p->cap_frac, mask, &dev->count,
+                        &dev->skip, small, s);
+    if (cudaMemcpyAsync(&host, dev, sizeof(host), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return XFP_ERR_CUDA;
+    if (!host.skip && outliers_select(W, n, ms, p->outlier_mode, mask, small, s) != cudaSuccess) return XFP_ERR_CUDA;
+    const int64_t host_cnt = host.count;
     if (host_cnt > capacity) return XFP_ERR_BUFFER_TOO_SMALL;
 
     xfp_desc d;
@@ -1383,23 +1157,35 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
     if (d.group_size != 64 && d.group_size != 128 && d.group_size != 256) return d.group_size > 0 ? XFP_ERR_UNSUPPORTED : XFP_ERR_SHAPE;
     if (cols % d.group_size) return XFP_ERR_SHAPE;
     d.col_bits = 32; d.nnz = host_cnt;
-    result->mu = host_ms[0]; result->sigma = host_ms[1]; result->nnz = host_cnt;
+    result->mu = host.mu; result->sigma = host.sigma; result->nnz = host_cnt;
     result->fallback = 1; result->tried = 0; result->reserved = 0;
+    if (mode == 1 && (lib_size < 1 || lib_size > 256)) return XFP_ERR_SHAPE;
+    // What a channel's Lloyd block has at hand it also delivers: the count of its extracted weights and (V2) its cosine.
+    // For V2a its indices are not wanted, LibFit assigns its own.
+    const bool fused = lloyd_fuses_cosine(cols);
+    int* rowcnt = carve(workspace, rows, cols).rowcnt;
+    const unsigned rgrid = (unsigned)((rows + 7) / 8);
+    if (!fused) {
+        row_count_kernel<<<rgrid, 256, 0, s>>>(mask, rows, cols, rowcnt);
+        rowptr_scan<<<1, 1024, 0, s>>>(rowcnt, rows, out_rowptr);
+    }
     for (int c = 0; c < n_candidates; ++c) {
         d.bits = candidates[c];
-        st = xfp_quant_lloyd(W, mask, ms, rows, cols, d.bits, p->lloyd_iters, codebook, idx, workspace, need, stream);
-        if (st) return st;
-        const uint16_t* table = codebook;
+        if (launch_lloyd(W, mask, ms, rows, cols, d.bits, p->lloyd_iters, codebook, mode ? nullptr : idx,
+                         mode == 0 && fused ? cos : nullptr, c == 0 && fused ? rowcnt : nullptr, workspace, s) != cudaSuccess)
+            return XFP_ERR_CUDA;
+        if (c == 0 && fused) rowptr_scan<<<1, 1024, 0, s>>>(rowcnt, rows, out_rowptr);
         if (mode == 1) {
             st = xfp_quant_libfit_library(codebook, rows, d.bits, lib_size, p->lloyd_iters, lib, workspace, need, stream);
             if (st) return st;
             st = xfp_quant_libfit_assign(W, mask, ms, rows, cols, d.bits, lib_size, d.group_size, lib, idx, gid, gscale, gmid,
                                          stream);
             if (st) return st;
-            table = lib;
         }
-        st = xfp_quant_cosine(&d, W, mask, idx, table, gid, gscale, gmid, cos, stream);
-        if (st) return st;
+        if (mode == 1 || !fused) {
+            st = xfp_quant_cosine(&d, W, mask, idx, mode ? lib : codebook, gid, gscale, gmid, cos, stream);
+            if (st) return st;
+        }
         st = xfp_quant_median(cos, rows, med_dev, workspace, need, stream);
         if (st) return st;
         double med = 0.0;
@@ -1411,15 +1197,10 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
         result->tried = c + 1;
         if (med >= tau) { result->fallback = 0; break; }
     }
-    return xfp_quant_residual(&d, W, mask, idx, mode ? lib : codebook, gid, gscale, gmid, out_rowptr, out_col, out_val,
-                              capacity, workspace, need, stream);
+    if (capacity > 0 && (!out_col || !out_val)) return XFP_ERR_NULL;
+    residual_kernel<<<rgrid, 256, 0, s>>>(W, mask, unpacked_of(&d, idx, mode ? lib : codebook, gid, gscale, gmid), rows,
+                                          out_rowptr, out_col, out_val, capacity);
+    return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
-
-#ifdef XFP_TRACE
-/* timing probe: clock64 at the six phase boundaries of block 0 of the last xfp_quant_lloyd launch (host array) */
-int xfp_debug_lloyd_phases(long long* out) {
-    return cudaMemcpyFromSymbol(out, g_lloyd_phase, sizeof(long long) * 8) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
-}
-#endif
 
 }  // extern "C"
