@@ -502,18 +502,23 @@ __global__ void __launch_bounds__(1024) rowptr_scan(const int* __restrict__ cnt,
     if (threadIdx.x == 0) rowptr[rows] = total;
 }
 
-// A warp per channel: the mask is read 128 weights at a time (a word per lane, the next four in flight); where a word is set
-// the places of its entries follow from four ballots, one per byte, without a barrier.
+// A warp per channel.  The mask is read 512 weights at a time (four words per lane in flight); the places of the set bytes
+// follow from four ballots per word, and their columns are collected in shared memory so that the gathers (weight, index,
+// codebook entry: three dependent trips) run with every lane busy instead of with the few lanes that found something.
 __global__ void __launch_bounds__(256) residual_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask,
                                                         Unpacked u, int rows, const int32_t* __restrict__ rowptr,
                                                         int32_t* ocol, uint16_t* oval, int64_t capacity) {
+    constexpr int kList = 1024;         // a step adds at most 512 columns, the list is emptied when 512 are waiting
+    __shared__ uint16_t s_list[8][kList];
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (row >= rows) return;
+    uint16_t* list = s_list[threadIdx.x >> 5];
     int64_t p = rowptr[row];
     if (rowptr[row + 1] == p) return;
     const uint32_t* m4 = (const uint32_t*)(mask + (int64_t)row * u.K);
     const uint32_t below = (1u << lane) - 1u;
     const int words = u.K / 4;          // a multiple of 32
+    int n = 0;
     for (int w0 = 0; w0 < words; w0 += 128) {
         uint32_t x[4];
 #pragma unroll
@@ -527,18 +532,22 @@ __global__ void __launch_bounds__(256) residual_kernel(const float* __restrict__
                 const uint32_t v = __ballot_sync(0xffffffffu, (x[i] >> (8 * b)) & 0xffu);
                 before += __popc(v & below); tot += __popc(v);
             }
-            int64_t at = p + before;
-            for (int b = 0; b < 4; ++b) {
-                if (!((x[i] >> (8 * b)) & 0xffu)) continue;
-                if (at < capacity) {
-                    const int k = (w0 + 32 * i + lane) * 4 + b;
-                    ocol[at] = k;
-                    oval[at] = d2h(__dsub_rn((double)W[(int64_t)row * u.K + k], h2d(decode16(u, row, k))));
-                }
-                ++at;
-            }
-            p += tot;
+            int at = n + before;
+            for (int b = 0; b < 4; ++b)
+                if ((x[i] >> (8 * b)) & 0xffu) list[at++] = (uint16_t)((w0 + 32 * i + lane) * 4 + b);
+            n += tot;
         }
+        if (n < 512 && w0 + 128 < words) continue;
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) {
+            if (p + i >= capacity) break;
+            const int k = list[i];
+            ocol[p + i] = k;
+            oval[p + i] = d2h(__dsub_rn((double)W[(int64_t)row * u.K + k], h2d(decode16(u, row, k))));
+        }
+        p += n;
+        n = 0;
+        __syncwarp();
     }
 }
 
@@ -590,258 +599,12 @@ __global__ void __launch_bounds__(256) cosine_kernel(const float* __restrict__ W
         cosv[row] = (aa == 0.0 || bb == 0.0) ? 1.0 : __ddiv_rn(ab, __dmul_rn(__dsqrt_rn(aa), __dsqrt_rn(bb)));
 }
 
-// ------------------------------------------------------------------ LibFit: the library
-
-// u[i][j] = (c_ij - m_i) / s_i and nn[i] = |u_i|^2, one thread per channel
-__global__ void libfit_normalise(const uint16_t* __restrict__ cb, int rows, int E, double* u, double* nn) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    double lo = INFINITY, hi = -INFINITY;
-    for (int j = 0; j < E; ++j) {
-        const double c = h2d(cb[(int64_t)i * E + j]);
-        if (c < lo) lo = c;
-        if (c > hi) hi = c;
-    }
-    const double m = __dmul_rn(0.5, __dadd_rn(hi, lo));
-    double s = __dmul_rn(0.5, __dsub_rn(hi, lo));
-    if (s == 0.0) s = 1.0;
-    double acc = 0.0;
-    for (int j = 0; j < E; ++j) {
-        const double v = __ddiv_rn(__dsub_rn(h2d(cb[(int64_t)i * E + j]), m), s);
-        u[(int64_t)i * E + j] = v;
-        acc = __dadd_rn(acc, __dmul_rn(v, v));
-    }
-    nn[i] = acc;
-}
-
-// order[r] = the channel of rank r by (nn, channel): rank by counting, exact and order independent
-__global__ void __launch_bounds__(256) libfit_rank(const double* __restrict__ nn, int rows, int* order) {
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    __shared__ double tile[256];
-    const double mine = i < rows ? nn[i] : 0.0;
-    int r = 0;
-    for (int j0 = 0; j0 < rows; j0 += 256) {
-        __syncthreads();
-        tile[threadIdx.x] = j0 + threadIdx.x < rows ? nn[j0 + threadIdx.x] : INFINITY;
-        __syncthreads();
-        const int lim = rows - j0 < 256 ? rows - j0 : 256;
-        for (int j = 0; j < lim; ++j) {
-            const double o = tile[j];
-            r += (o < mine) || (o == mine && j0 + j < i);
-        }
-    }
-    if (i < rows) order[r] = i;
-}
-
-__global__ void libfit_seed(const double* __restrict__ u, const int* __restrict__ order, int rows, int E, int L,
-                            double* cen) {
-    const int l = blockIdx.x, j = threadIdx.x;
-    if (j >= E) return;
-    long long t = rows >= L ? (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)l, 0.5), (double)rows), (double)L))
-                            : (long long)(l % rows);
-    if (t >= rows) t = rows - 1;
-    cen[l * E + j] = u[(int64_t)order[t] * E + j];
-}
-
-// asg[i] = nearest centroid (squared distance summed entry by entry; ties: lower centroid).  One warp per channel,
-// lane = centroid (32 at a time): every lane sums its distance in entry order, the warp keeps the smallest
-// (distance, centroid) pair -- the answer of a scan over the centroids with a strict "less than".
-__global__ void __launch_bounds__(256) libfit_assign_rows(const double* __restrict__ u, const double* __restrict__ cen,
-                                                           int rows, int E, int L, int* asg, const int* done) {
-    if (*done) return;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= rows) return;
-    int best = 0;
-    double bd = INFINITY;
-    for (int l0 = 0; l0 < L; l0 += 32) {
-        const int l = l0 + lane;
-        double d = INFINITY;
-        if (l < L) {
-            d = 0.0;
-            for (int j = 0; j < E; ++j) {
-                const double t = __dsub_rn(u[(int64_t)i * E + j], cen[l * E + j]);
-                d = __dadd_rn(d, __dmul_rn(t, t));
-            }
-        }
-        int bl = l;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {   // smallest distance, lower centroid on a tie
-            const double od = __shfl_xor_sync(0xffffffffu, d, o);
-            const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
-            if (od < d || (od == d && ol < bl)) { d = od; bl = ol; }
-        }
-        if (d < bd) { bd = d; best = bl; }   // a later group of 32 wins only when strictly nearer
-    }
-    if (lane == 0) asg[i] = best;
-}
-
-// centroid l <- mean of its members, every entry summed in channel order.  One block per centroid: the
-// members of each tile of 1024 channels are compacted in order, then thread j adds them to entry j.
-__global__ void __launch_bounds__(1024) libfit_update(const double* __restrict__ u, const int* __restrict__ asg,
-                                                       int rows, int E, int L, double* cen, int* changed,
-                                                       const int* done) {
-    __shared__ int sh[32];
-    __shared__ int total;
-    __shared__ int member[1024];
-    if (*done) return;
-    const int l = blockIdx.x, j = threadIdx.x;
-    double acc = 0.0;
-    long long cnt = 0;
-    for (int i0 = 0; i0 < rows; i0 += 1024) {
-        const int i = i0 + threadIdx.x;
-        const int f = i < rows && asg[i] == l;
-        const int off = block_excl_scan(f, sh, &total);
-        if (f) member[off] = i;
-        __syncthreads();
-        const int n = total;
-        if (j < E)
-            for (int m = 0; m < n; ++m) acc = __dadd_rn(acc, u[(int64_t)member[m] * E + j]);
-        cnt += n;
-        __syncthreads();
-    }
-    if (j < E && cnt > 0) {
-        const double m = __ddiv_rn(acc, (double)cnt);
-        if (m != cen[l * E + j]) { cen[l * E + j] = m; *changed = 1; }
-    }
-}
-
-// done |= !changed; changed = 0
-__global__ void libfit_round_end(int* changed, int* done) {
-    if (!*done && !*changed) *done = 1;
-    *changed = 0;
-}
-__global__ void libfit_flags_init(int* changed, int* done) { *changed = 0; *done = 0; }
-
-// lib[l] = the centroid's entries in ascending order, fp16
-__global__ void libfit_store(const double* __restrict__ cen, int E, uint16_t* lib) {
-    const int l = blockIdx.x;
-    if (threadIdx.x != 0) return;
-    double tmp[64];
-    for (int j = 0; j < E; ++j) tmp[j] = cen[l * E + j];
-    for (int a = 1; a < E; ++a) {   // insertion sort
-        const double v = tmp[a];
-        int b = a - 1;
-        while (b >= 0 && tmp[b] > v) { tmp[b + 1] = tmp[b]; --b; }
-        tmp[b + 1] = v;
-    }
-    for (int j = 0; j < E; ++j) lib[l * E + j] = d2h(tmp[j]);
-}
-
-// ------------------------------------------------------------------ LibFit: per-group assignment
-
-// A block of GS threads takes `gpb` consecutive groups of GS weights (4 when L <= 32; GS = 64, 128 or 256, the
-// group size of the format).  Thread (s, l) scores library entry l on group s serially over the GS values; one
-// thread per group picks the winner; then the GS threads index each group against its winner.
-template <int GS>
-__global__ void __launch_bounds__(GS) libfit_group_kernel(const float* __restrict__ W,
-                                                            const uint8_t* __restrict__ mask,
-                                                            const double* __restrict__ ms, int64_t groups, int bits,
-                                                            int L, int gpb, const uint16_t* __restrict__ lib,
-                                                            uint8_t* idx, uint8_t* gid, uint16_t* gscale,
-                                                            uint16_t* gmid) {
-    constexpr int NW = GS / 32;
-    __shared__ double gv[4][GS];
-    __shared__ double red_lo[4][NW], red_hi[4][NW];
-    __shared__ double sse[256];
-    __shared__ double dec[4][64];
-    __shared__ uint16_t s_mid[4], s_sc[4];
-    __shared__ int s_best[4], s_const[4];
-    const int E = 1 << bits;
-    const int tid = threadIdx.x;
-    const int lw = GS / gpb;                   // threads per group while scoring
-    const double mu = ms[0];
-    const int64_t g0 = (int64_t)blockIdx.x * gpb;
-    for (int s = 0; s < gpb; ++s) {
-        const int64_t grp = g0 + s;
-        if (grp >= groups) break;
-        const double v = bulk_value(W, mask, grp * GS + tid, mu);
-        gv[s][tid] = v;
-        double lo = v, hi = v;
-        for (int d = 16; d > 0; d >>= 1) {
-            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-        }
-        if ((tid & 31) == 0) { red_lo[s][tid >> 5] = lo; red_hi[s][tid >> 5] = hi; }
-    }
-    __syncthreads();
-    if (tid < gpb && g0 + tid < groups) {
-        double lo = red_lo[tid][0], hi = red_hi[tid][0];
-#pragma unroll
-        for (int w = 1; w < NW; ++w) { lo = fmin(lo, red_lo[tid][w]); hi = fmax(hi, red_hi[tid][w]); }
-        s_mid[tid] = d2h(__dmul_rn(0.5, __dadd_rn(hi, lo)));
-        s_sc[tid] = d2h(__dmul_rn(0.5, __dsub_rn(hi, lo)));
-        s_const[tid] = hi == lo;
-    }
-    __syncthreads();
-    {
-        const int s = tid / lw;
-        const int64_t grp = g0 + s;
-        if (grp < groups && !s_const[s]) {
-            const uint16_t mid16 = s_mid[s], sc16 = s_sc[s];
-            for (int l = tid % lw; l < L; l += lw) {
-                double d16[64];
-                bool asc = true;
-                for (int j = 0; j < E; ++j) {
-                    d16[j] = h2d(v2a_value16(sc16, lib[l * E + j], mid16));
-                    if (j && d16[j] < d16[j - 1]) asc = false;
-                }
-                double acc = 0.0;
-                for (int t = 0; t < GS; t += 4) {   // four searches in flight, the sum stays in value order
-                    double d[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const double x = gv[s][t + e];
-                        d[e] = __dsub_rn(x, d16[nearest_entry(d16, E, x, asc)]);
-                    }
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc = __dadd_rn(acc, __dmul_rn(d[e], d[e]));
-                }
-                sse[s * L + l] = acc;   // gpb * L <= 256
-            }
-        }
-    }
-    __syncthreads();
-    if (tid < gpb && g0 + tid < groups) {
-        const int64_t grp = g0 + tid;
-        int best = 0;
-        if (!s_const[tid]) {
-            double b = INFINITY;
-            for (int l = 0; l < L; ++l) {
-                const double e = sse[tid * L + l];
-                if (e < b) { b = e; best = l; }
-            }
-        }
-        s_best[tid] = best;
-        gid[grp] = (uint8_t)best;
-        gscale[grp] = s_const[tid] ? (uint16_t)0 : s_sc[tid];   // a constant group: scale 0, entry 0, indices 0
-        gmid[grp] = s_mid[tid];
-    }
-    __syncthreads();
-    for (int e = tid; e < gpb * E; e += GS) {
-        const int s = e / E, j = e % E;
-        if (g0 + s < groups) dec[s][j] = h2d(v2a_value16(s_sc[s], lib[s_best[s] * E + j], s_mid[s]));
-    }
-    __syncthreads();
-    for (int s = 0; s < gpb; ++s) {
-        const int64_t grp = g0 + s;
-        if (grp >= groups) break;
-        int bj = 0;
-        if (!s_const[s]) {
-            bool asc = true;
-            for (int j = 1; j < E; ++j) asc = asc && dec[s][j] >= dec[s][j - 1];
-            bj = nearest_entry(dec[s], E, gv[s][tid], asc);
-        }
-        idx[grp * GS + tid] = (uint8_t)bj;
-    }
-}
-
 // ------------------------------------------------------------------ host side
 
 struct Workspace {
     double2* part;     // [kRedBlocks]
     SelState* sel;
-    int* flags;        // [2] LibFit changed / done
+    int* flags;        // [3] LibFit: did round i change a centroid
     int* tie;          // [ceil(n / kTieChunk)]
     int* rowcnt;       // [rows]
     double* u;         // [rows][64]
@@ -862,7 +625,7 @@ static Workspace carve(void* base, int64_t rows, int64_t cols) {
     const int64_t n = rows * cols;
     w.part = (double2*)take(sizeof(double2) * kRedBlocks);
     w.sel = (SelState*)take(sizeof(SelState));
-    w.flags = (int*)take(sizeof(int) * 2);
+    w.flags = (int*)take(sizeof(int) * 3);
     w.tie = (int*)take(sizeof(int) * (size_t)((n + kTieChunk - 1) / kTieChunk + 1));
     w.rowcnt = (int*)take(sizeof(int) * (size_t)rows);
     w.u = (double*)take(sizeof(double) * (size_t)rows * 64);
@@ -1009,18 +772,8 @@ int xfp_quant_libfit_library(const uint16_t* codebook, int32_t rows, int32_t bit
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(workspace, rows, 128);
     const int E = 1 << bits;
-    const int rb = (rows + 255) / 256;
-    libfit_normalise<<<rb, 256, 0, s>>>(codebook, rows, E, w.u, w.nn);
-    libfit_rank<<<rb, 256, 0, s>>>(w.nn, rows, w.order);
-    libfit_seed<<<L, 64, 0, s>>>(w.u, w.order, rows, E, L, w.cen);
-    libfit_flags_init<<<1, 1, 0, s>>>(w.flags, w.flags + 1);
-    for (int it = 0; it < iters; ++it) {
-        libfit_assign_rows<<<(rows + 7) / 8, 256, 0, s>>>(w.u, w.cen, rows, E, L, w.asg, w.flags + 1);
-        libfit_update<<<L, 1024, 0, s>>>(w.u, w.asg, rows, E, L, w.cen, w.flags, w.flags + 1);
-        libfit_round_end<<<1, 1, 0, s>>>(w.flags, w.flags + 1);
-    }
-    libfit_store<<<L, 32, 0, s>>>(w.cen, E, lib);
-    return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    return launch_libfit_library(codebook, rows, E, L, iters, w.u, w.nn, w.order, w.asg, w.cen, w.flags, lib, s) == cudaSuccess
+               ? XFP_OK : XFP_ERR_CUDA;
 }
 
 int xfp_quant_libfit_assign(const float* W, const uint8_t* mask, const double* mu_sigma, int32_t rows, int32_t cols,
@@ -1037,16 +790,8 @@ int xfp_quant_libfit_assign(const float* W, const uint8_t* mask, const double* m
     if (cols % group_size) return XFP_ERR_SHAPE;
     const int64_t groups = (int64_t)rows * (cols / group_size);
     if (groups > 0x7fffffff) return XFP_ERR_UNSUPPORTED;
-    const int gpb = L <= 32 ? 4 : (L <= 64 ? 2 : 1);
-    const unsigned grid = (unsigned)((groups + gpb - 1) / gpb);
-    cudaStream_t s = (cudaStream_t)stream;
-    if (group_size == 64)
-        libfit_group_kernel<64><<<grid, 64, 0, s>>>(W, mask, mu_sigma, groups, bits, L, gpb, lib, idx, gid, gscale, gmid);
-    else if (group_size == 128)
-        libfit_group_kernel<128><<<grid, 128, 0, s>>>(W, mask, mu_sigma, groups, bits, L, gpb, lib, idx, gid, gscale, gmid);
-    else
-        libfit_group_kernel<256><<<grid, 256, 0, s>>>(W, mask, mu_sigma, groups, bits, L, gpb, lib, idx, gid, gscale, gmid);
-    return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    return launch_libfit_assign(W, mask, mu_sigma, rows, cols, bits, L, group_size, lib, idx, gid, gscale, gmid, nullptr,
+                                (cudaStream_t)stream) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
 
 static int unpacked_args_status(const xfp_desc* desc, const float* W, const uint8_t* idx, const uint16_t* codebook,
@@ -1178,12 +923,11 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
         if (mode == 1) {
             st = xfp_quant_libfit_library(codebook, rows, d.bits, lib_size, p->lloyd_iters, lib, workspace, need, stream);
             if (st) return st;
-            st = xfp_quant_libfit_assign(W, mask, ms, rows, cols, d.bits, lib_size, d.group_size, lib, idx, gid, gscale, gmid,
-                                         stream);
-            if (st) return st;
-        }
-        if (mode == 1 || !fused) {
-            st = xfp_quant_cosine(&d, W, mask, idx, mode ? lib : codebook, gid, gscale, gmid, cos, stream);
+            if (launch_libfit_assign(W, mask, ms, rows, cols, d.bits, lib_size, d.group_size, lib, idx, gid, gscale, gmid, cos,
+                                     s) != cudaSuccess)
+                return XFP_ERR_CUDA;
+        } else if (!fused) {
+            st = xfp_quant_cosine(&d, W, mask, idx, codebook, nullptr, nullptr, nullptr, cos, stream);
             if (st) return st;
         }
         st = xfp_quant_median(cos, rows, med_dev, workspace, need, stream);

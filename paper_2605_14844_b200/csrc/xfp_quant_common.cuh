@@ -95,4 +95,38 @@ __device__ __forceinline__ double bulk_value(const float* __restrict__ W, const 
     return (mask != nullptr && mask[t]) ? mu : (double)W[t];
 }
 
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// floats in the order of their values as integers
+__device__ __forceinline__ int ordered(float f) { const int i = __float_as_int(f); return i < 0 ? (int)(0x80000000u - (uint32_t)i) : i; }
+__device__ __forceinline__ float unordered(int o) { return __int_as_float(o < 0 ? (int)(0x80000000u - (uint32_t)o) : o); }
+
+// Largest float x in [a, b) that the nearest-entry rule gives to entry a: |x - a| <= |x - b| in fp64.  The rule is
+// monotone in x; the float below the midpoint keeps it, and the next one nearly always breaks it.
+__device__ __forceinline__ float last_of_lower(double a, double b) {
+    const double mid = __dmul_rn(0.5, __dadd_rn(a, b));       // exact: a and b are fp16 values
+    const float c = __double2float_rd(mid);
+    int lo = ordered(c), hi = ordered(__double2float_rn(b));   // the rule holds at lo, breaks at hi
+    if (lo + 1 < hi) {
+        const double x = (double)unordered(lo + 1);
+        if (fabs(__dsub_rn(x, a)) <= fabs(__dsub_rn(x, b))) {
+            while (lo + 1 < hi) {
+                const int m = lo + ((hi - lo) >> 1);
+                const double y = (double)unordered(m);
+                if (fabs(__dsub_rn(y, a)) <= fabs(__dsub_rn(y, b))) lo = m; else hi = m;
+            }
+        }
+    }
+    return unordered(lo);
+}
+
 }  // namespace xq

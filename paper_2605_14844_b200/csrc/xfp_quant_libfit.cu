@@ -1,0 +1,472 @@
+// LibFit ("V2a: Shared Codebook Library"): the library (a k-means pass over normalised per-channel codebooks) and the
+// assignment of every group of weights to a library entry.  Integers and fp16 values are those of the serial fp64
+// evaluation, bit for bit.
+#include <cooperative_groups.h>
+
+#include "xfp_quant_common.cuh"
+#include "xfp_quant_internal.h"
+#include "xfp_internal.h"
+#include "../../include/xfp_quant.h"
+
+namespace xq {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+// ------------------------------------------------------------------ the library
+
+constexpr int kLibThreads = 256;
+constexpr int kLibTile = 2048;      // channels whose members are compacted at a time
+constexpr int kLibVals = 2048;      // member values staged at a time
+
+// The whole k-means in one cooperative launch: normalise, order by norm, seed, `iters` rounds of assignment and update,
+// store.  As separate launches (three per round) the rounds were bound by launches and by the update's chain of dependent
+// loads: 3072 channels, N = 2, 20 rounds 515 us; here a round costs two grid barriers and the update's serial sums.
+//   assignment  a warp per channel, a lane per centroid (32 at a time); every lane sums its squared distance in entry
+//               order and the smallest (distance, centroid) pair wins: the answer of a scan with a strict "less than"
+//   update      a block per centroid compacts its members in channel order, stages their entries in shared memory, and
+//               thread j adds them to entry j one by one: the order of the serial evaluation
+__global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint16_t* __restrict__ cb, int rows, int E, int L,
+                                                                     int iters, double* u, double* nn, int* order, int* asg,
+                                                                     double* cen, int* flag, uint16_t* lib) {
+    __shared__ int sh[32];
+    __shared__ int total;
+    __shared__ int member[kLibTile];
+    __shared__ double vals[kLibVals];
+    cg::grid_group grid = cg::this_grid();
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int gt = blockIdx.x * kLibThreads + tid, nt = gridDim.x * kLibThreads;
+    const int gw = gt >> 5, nw = nt >> 5;
+    // u[i][j] = (c_ij - m_i) / s_i, m and s the middle and half-width of the codebook's range; nn[i] = |u_i|^2
+    for (int i = gt; i < rows; i += nt) {
+        double lo = INFINITY, hi = -INFINITY;
+        for (int j = 0; j < E; ++j) {
+            const double c = h2d(cb[(int64_t)i * E + j]);
+            if (c < lo) lo = c;
+            if (c > hi) hi = c;
+        }
+        const double m = __dmul_rn(0.5, __dadd_rn(hi, lo));
+        double s = __dmul_rn(0.5, __dsub_rn(hi, lo));
+        if (s == 0.0) s = 1.0;
+        double acc = 0.0;
+        for (int j = 0; j < E; ++j) {
+            const double v = __ddiv_rn(__dsub_rn(h2d(cb[(int64_t)i * E + j]), m), s);
+            u[(int64_t)i * E + j] = v;
+            acc = __dadd_rn(acc, __dmul_rn(v, v));
+        }
+        nn[i] = acc;
+    }
+    if (gt < 3) flag[gt] = 0;
+    grid.sync();
+    // order[r] = the channel of rank r by (nn, channel): rank by counting
+    for (int i = gw; i < rows; i += nw) {
+        const double mine = __ldcg(nn + i);
+        int r = 0;
+#pragma unroll 4
+        for (int j = lane; j < rows; j += 32) {
+            const double o = __ldcg(nn + j);
+            r += (o < mine) || (o == mine && j < i);
+        }
+        r = __reduce_add_sync(0xffffffffu, r);
+        if (lane == 0) order[r] = i;
+    }
+    grid.sync();
+    for (int i = gt; i < L * E; i += nt) {      // L evenly spaced channels of that order
+        const int l = i / E, j = i % E;
+        long long t = rows >= L ? (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)l, 0.5), (double)rows), (double)L))
+                                : (long long)(l % rows);
+        if (t >= rows) t = rows - 1;
+        cen[i] = __ldcg(u + (int64_t)__ldcg(order + t) * E + j);
+    }
+    grid.sync();
+    for (int it = 0; it < iters; ++it) {
+        const bool staged = L * E <= kLibVals;
+        if (staged) {
+            for (int i = tid; i < L * E; i += kLibThreads) vals[(i % E) * L + i / E] = __ldcg(cen + i);   // [entry][centroid]
+            __syncthreads();
+        }
+        for (int i = gw; i < rows; i += nw) {
+            int best = 0;
+            double bd = INFINITY;
+            for (int l0 = 0; l0 < L; l0 += 32) {
+                const int l = l0 + lane;
+                double d = INFINITY;
+                if (l < L) {
+                    d = 0.0;
+#pragma unroll 4
+                    for (int j = 0; j < E; ++j) {
+                        const double t = __dsub_rn(__ldcg(u + (int64_t)i * E + j), staged ? vals[j * L + l] : __ldcg(cen + l * E + j));
+                        d = __dadd_rn(d, __dmul_rn(t, t));
+                    }
+                }
+                int bl = l;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) {   // smallest distance, lower centroid on a tie
+                    const double od = __shfl_xor_sync(0xffffffffu, d, o);
+                    const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
+                    if (od < d || (od == d && ol < bl)) { d = od; bl = ol; }
+                }
+                if (d < bd) { bd = d; best = bl; }   // a later group of 32 wins only when strictly nearer
+            }
+            if (lane == 0) asg[i] = best;
+        }
+        grid.sync();
+        if (gt == 0) flag[(it + 1) % 3] = 0;         // last read two barriers ago
+        for (int l = blockIdx.x; l < L; l += gridDim.x) {
+            double acc = 0.0;
+            long long cnt = 0;
+            for (int i0 = 0; i0 < rows; i0 += kLibTile) {
+                constexpr int per = kLibTile / kLibThreads;
+                int hit = 0;
+#pragma unroll
+                for (int e = 0; e < per; ++e) {
+                    const int i = i0 + tid * per + e;
+                    if (i < rows && __ldcg(asg + i) == l) hit |= 1 << e;
+                }
+                int at = block_excl_scan(__popc(hit), sh, &total);
+                for (int e = 0; e < per; ++e)
+                    if ((hit >> e) & 1) member[at++] = i0 + tid * per + e;
+                __syncthreads();
+                const int n = total, chunk = kLibVals / E;
+                for (int m0 = 0; m0 < n; m0 += chunk) {
+                    const int c = n - m0 < chunk ? n - m0 : chunk;
+                    for (int i = tid; i < c * E; i += kLibThreads) vals[i] = __ldcg(u + (int64_t)member[m0 + i / E] * E + i % E);
+                    __syncthreads();
+                    if (tid < E) {
+#pragma unroll 8
+                        for (int m = 0; m < c; ++m) acc = __dadd_rn(acc, vals[m * E + tid]);
+                    }
+                    __syncthreads();
+                }
+                cnt += n;
+                __syncthreads();
+            }
+            if (tid < E && cnt > 0) {
+                const double m = __ddiv_rn(acc, (double)cnt);
+                if (m != __ldcg(cen + l * E + tid)) { cen[l * E + tid] = m; flag[it % 3] = 1; }
+            }
+        }
+        grid.sync();
+        if (!__ldcg(flag + it % 3)) break;
+    }
+    // lib[l] = the centroid's entries in ascending order, fp16
+    for (int l = blockIdx.x; l < L; l += gridDim.x) {
+        __syncthreads();
+        if (tid < E) vals[tid] = __ldcg(cen + l * E + tid);
+        __syncthreads();
+        if (tid < E) {
+            const double x = vals[tid];
+            int r = 0;
+            for (int j = 0; j < E; ++j) r += vals[j] < x || (vals[j] == x && j < tid);
+            lib[l * E + r] = d2h(x);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ the assignment of a group
+
+constexpr int kLibSmem = 2048;      // library entries (L * 2^N) staged in shared memory
+
+template <int GS>
+struct GroupGeo {
+    static constexpr int VPL = GS / 32;                 // consecutive weights of a lane
+    static constexpr int WARPS = GS == 256 ? 4 : 8;     // groups of a channel at a time
+};
+
+// Ascending over the warp: element lane * VPL + e.
+template <int VPL>
+__device__ __forceinline__ void warp_sort(float (&a)[VPL], int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32 * VPL; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j; j >>= 1) {
+            if (j >= VPL) {
+                const bool low = ((lane * VPL) & j) == 0, up = ((lane * VPL) & k) == 0;
+#pragma unroll
+                for (int e = 0; e < VPL; ++e) {
+                    const float o = __shfl_xor_sync(0xffffffffu, a[e], j / VPL);
+                    a[e] = low == up ? fminf(a[e], o) : fmaxf(a[e], o);
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < VPL; ++e) {
+                    if (e & j) continue;
+                    const bool up = k < VPL ? (e & k) == 0 : ((lane * VPL + e) & k) == 0;
+                    const float x = fminf(a[e], a[e | j]), y = fmaxf(a[e], a[e | j]);
+                    a[e] = up ? x : y; a[e | j] = up ? y : x;
+                }
+            }
+        }
+    }
+}
+
+// One block per channel, one warp per group of GS weights.  The squared error of a group against a library entry is, in
+// exact arithmetic, a sum over the 2^N cells of (sum v^2 - 2 d sum v + n d^2): with the group sorted once and its prefix
+// sums of v and v^2 at hand a lane scores an entry by 2^N - 1 searches instead of GS nearest-entry decisions (3072 x 4096
+// weights, N = 2, L = 32: 1065 us with every decision and every square taken in fp64).  Those scores carry a rounding
+// error far below the differences between entries: an entry is ruled out when its score less its error bound lies above
+// another's score plus bound, and only where more than one entry is left are their errors summed value by value in the
+// order the method states.
+template <int GS>
+__global__ void __launch_bounds__(32 * GroupGeo<GS>::WARPS) libfit_group_kernel(
+    const float* __restrict__ W, const uint8_t* __restrict__ mask, const double* __restrict__ ms, int K, int bits, int L,
+    const uint16_t* __restrict__ lib, uint8_t* __restrict__ idx, uint8_t* __restrict__ gid, uint16_t* __restrict__ gscale,
+    uint16_t* __restrict__ gmid, double* __restrict__ cosv) {
+    constexpr int VPL = GroupGeo<GS>::VPL, WARPS = GroupGeo<GS>::WARPS;
+    __shared__ uint16_t slib[kLibSmem];                 // [entry of a codebook][codebook]
+    __shared__ __align__(16) float s_v[WARPS][GS];
+    __shared__ double2 s_p[WARPS][GS + 1];              // sums of v - mid and (v - mid)^2 in front of sorted position i
+    __shared__ double s_dec[WARPS][64];
+    __shared__ float s_thr[WARPS][64];
+    __shared__ double s_red[3][WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int E = 1 << bits;
+    const double mu = ms[0];
+    const float fmu = (float)mu;
+    const int64_t row = blockIdx.x;
+    const int G = K / GS;
+    const bool staged = L * E <= kLibSmem;
+    if (staged)
+        for (int i = tid; i < L * E; i += blockDim.x) slib[(i % E) * L + i / E] = lib[i];
+    __syncthreads();
+    float* sv = s_v[warp];
+    double2* sp = s_p[warp];
+    double* dec = s_dec[warp];
+    float* thr = s_thr[warp];
+    double sab = 0.0, saa = 0.0, sbb = 0.0;
+    for (int g = warp; g < G; g += nwarps) {
+        const int64_t grp = row * G + g, base = grp * GS + lane * VPL;
+        float w[VPL];
+        uint32_t ext = 0;                               // bit e: weight e of this lane was extracted
+#pragma unroll
+        for (int e = 0; e < VPL; e += 2) { const float2 t = __ldg((const float2*)(W + base + e)); w[e] = t.x; w[e + 1] = t.y; }
+        if (mask) {
+#pragma unroll
+            for (int e = 0; e < VPL; e += 2) {
+                const uint16_t t = __ldg((const uint16_t*)(mask + base + e));
+                ext |= ((t & 0xffu) ? 1u << e : 0u) | ((t & 0xff00u) ? 2u << e : 0u);
+            }
+        }
+        float a[VPL];
+        float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < VPL; ++e) {
+            const bool x = (ext >> e) & 1u;
+            a[e] = x ? fmu : w[e];
+            lo = fminf(lo, x ? INFINITY : w[e]); hi = fmaxf(hi, x ? -INFINITY : w[e]);
+        }
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+        }
+        const int nx = __reduce_add_sync(0xffffffffu, __popc(ext));
+        double dlo = (double)lo, dhi = (double)hi;
+        if (nx) { dlo = fmin(dlo, mu); dhi = fmax(dhi, mu); }
+        const uint16_t mid16 = d2h(__dmul_rn(0.5, __dadd_rn(dhi, dlo))), sc16 = d2h(__dmul_rn(0.5, __dsub_rn(dhi, dlo)));
+        const bool flat = dhi == dlo;                   // a constant group: scale 0, entry 0, indices 0
+        int best = 0;
+        if (!flat) {
+            const double mid = h2d(mid16);
+            warp_sort<VPL>(a, lane);
+            double p1 = 0.0, p2 = 0.0;
+            double2 own[VPL];
+#pragma unroll
+            for (int e = 0; e < VPL; ++e) {
+                const double t = (double)a[e] - mid;
+                p1 += t; p2 = fma(t, t, p2);
+                own[e] = make_double2(p1, p2);
+            }
+            double i1 = p1, i2 = p2;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const double t1 = __shfl_up_sync(0xffffffffu, i1, d), t2 = __shfl_up_sync(0xffffffffu, i2, d);
+                if (lane >= d) { i1 += t1; i2 += t2; }
+            }
+            __syncwarp();                               // the previous group's readers are done
+#pragma unroll
+            for (int e = 0; e < VPL; ++e) {
+                sv[lane * VPL + e] = a[e];
+                sp[lane * VPL + e + 1] = make_double2(i1 - p1 + own[e].x, i2 - p2 + own[e].y);
+            }
+            if (lane == 0) sp[0] = make_double2(0.0, 0.0);
+            __syncwarp();
+            const double2 all = sp[GS];
+            // values sorted as floats: mu's copies by at most half a float ulp
+            const double slack = 1e-9 * all.y + (double)nx * (dhi - dlo) * fabs(mu) * 2.4e-7;
+            double score[8], bound[8];
+            double least = INFINITY;
+#pragma unroll 1
+            for (int l0 = 0; l0 < L; l0 += 32) {
+                const int l = l0 + lane;
+                double sc = INFINITY, bd = 0.0;
+                if (l < L) {
+                    bool asc = true;
+                    double far = 0.0, prev = 0.0;
+                    double2 at = make_double2(0.0, 0.0);
+                    int cut = 0;
+                    sc = 0.0;
+                    for (int j = 0; j <= E; ++j) {
+                        double d = 0.0, x = INFINITY;
+                        if (j < E) {
+                            d = h2d(v2a_value16(sc16, staged ? slib[j * L + l] : __ldg(lib + l * E + j), mid16));
+                            far = fmax(far, fabs(d - mid));
+                            if (j == 0) { prev = d; continue; }
+                            if (d < prev) asc = false;
+                            x = 0.5 * (prev + d);
+                        }
+                        int c = GS;
+                        if (j < E) {
+                            const float xf = __double2float_rd(x);
+                            c = 0;
+#pragma unroll
+                            for (int step = GS / 2; step; step >>= 1) c += sv[c + step - 1] <= xf ? step : 0;
+                            c += sv[c] <= xf;
+                            c = c > cut ? c : cut;
+                        }
+                        const double2 to = sp[c];
+                        const double q = prev - mid;
+                        sc += (to.y - at.y) - 2.0 * q * (to.x - at.x) + (double)(c - cut) * q * q;
+                        at = to; cut = c; prev = d;
+                    }
+                    bd = asc ? slack + 1e-12 * GS * far * far : INFINITY;    // a codebook out of order is always summed exactly
+                    least = fmin(least, sc + bd);
+                }
+                score[l0 >> 5] = sc; bound[l0 >> 5] = bd;
+            }
+#pragma unroll
+            for (int d = 16; d; d >>= 1) least = fmin(least, __shfl_xor_sync(0xffffffffu, least, d));
+            int count = 0;
+            best = L;
+#pragma unroll 1
+            for (int l0 = 0; l0 < L; l0 += 32) {
+                const bool in = l0 + lane < L && !(score[l0 >> 5] - bound[l0 >> 5] > least);
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                count += __popc(b);
+                if (b && best == L) best = l0 + __ffs(b) - 1;
+            }
+            if (count > 1) {                            // too close to call: value by value
+                double bs = INFINITY;
+                int bl = L;
+#pragma unroll 1
+                for (int l0 = 0; l0 < L; l0 += 32) {
+                    const int l = l0 + lane;
+                    if (l >= L || score[l0 >> 5] - bound[l0 >> 5] > least) continue;
+                    double d16[64];
+                    bool asc = true;
+                    for (int j = 0; j < E; ++j) {
+                        d16[j] = h2d(v2a_value16(sc16, __ldg(lib + l * E + j), mid16));
+                        if (j && d16[j] < d16[j - 1]) asc = false;
+                    }
+                    double acc = 0.0;
+                    for (int t = 0; t < GS; ++t) {
+                        const double x = bulk_value(W, mask, grp * GS + t, mu), d = __dsub_rn(x, d16[nearest_entry(d16, E, x, asc)]);
+                        acc = __dadd_rn(acc, __dmul_rn(d, d));
+                    }
+                    if (acc < bs) { bs = acc; bl = l; }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int o = 16; o; o >>= 1) {
+                    const double os = __shfl_xor_sync(0xffffffffu, bs, o);
+                    const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
+                    if (os < bs || (os == bs && ol < bl)) { bs = os; bl = ol; }
+                }
+                best = bl < L ? bl : 0;
+            }
+        }
+        if (lane == 0) {
+            gid[grp] = (uint8_t)best;
+            gscale[grp] = flat ? (uint16_t)0 : sc16;
+            gmid[grp] = mid16;
+        }
+        // indices against the winner
+        __syncwarp();
+        for (int j = lane; j < E; j += 32) dec[j] = h2d(v2a_value16(flat ? (uint16_t)0 : sc16, __ldg(lib + best * E + j), mid16));
+        __syncwarp();
+        bool rise = true;
+        for (int j = lane; j < E; j += 32) {
+            thr[j] = INFINITY;
+            if (j < E - 1) {
+                if (dec[j] < dec[j + 1]) thr[j] = last_of_lower(dec[j], dec[j + 1]);
+                else rise = false;
+            }
+        }
+        rise = __all_sync(0xffffffffu, rise);
+        __syncwarp();
+        int at[VPL];
+#pragma unroll
+        for (int e = 0; e < VPL; ++e) at[e] = 0;
+        if (!flat) {
+            bool asc = true;
+            if (!rise)
+                for (int j = 1; j < E; ++j) asc = asc && dec[j] >= dec[j - 1];
+            if (rise) {
+                for (int step = E >> 1; step; step >>= 1) {
+#pragma unroll
+                    for (int e = 0; e < VPL; ++e) at[e] += w[e] > thr[at[e] + step - 1] ? step : 0;
+                }
+            } else {
+#pragma unroll 1
+                for (int e = 0; e < VPL; ++e) at[e] = nearest_entry(dec, E, (double)w[e], asc);
+            }
+            if (nx) {
+                const int xi = nearest_entry(dec, E, mu, asc);
+#pragma unroll
+                for (int e = 0; e < VPL; ++e)
+                    if ((ext >> e) & 1u) at[e] = xi;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < VPL; e += 2) *(uint16_t*)(idx + base + e) = (uint16_t)(at[e] | (at[e + 1] << 8));
+        if (cosv) {
+#pragma unroll
+            for (int e = 0; e < VPL; ++e) {
+                const double x = (double)w[e];
+                double b = dec[at[e]];
+                if ((ext >> e) & 1u) b = h2d(d2h(__dadd_rn(b, h2d(d2h(__dsub_rn(x, b))))));   // W^ = fp16(D16 + S)
+                sab = fma(x, b, sab); saa = fma(x, x, saa); sbb = fma(b, b, sbb);
+            }
+        }
+    }
+    if (cosv) {
+        sab = warp_sum(sab); saa = warp_sum(saa); sbb = warp_sum(sbb);
+        if (lane == 0) { s_red[0][warp] = sab; s_red[1][warp] = saa; s_red[2][warp] = sbb; }
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < nwarps; ++w) { sab += s_red[0][w]; saa += s_red[1][w]; sbb += s_red[2][w]; }
+            cosv[row] = (saa == 0.0 || sbb == 0.0) ? 1.0 : __ddiv_rn(sab, __dmul_rn(__dsqrt_rn(saa), __dsqrt_rn(sbb)));
+        }
+    }
+}
+
+template <int GS>
+cudaError_t launch_groups(const float* W, const uint8_t* mask, const double* ms, int rows, int cols, int bits, int L,
+                          const uint16_t* lib, uint8_t* idx, uint8_t* gid, uint16_t* gscale, uint16_t* gmid, double* cosv,
+                          cudaStream_t s) {
+    const int groups = cols / GS, warps = groups < GroupGeo<GS>::WARPS ? groups : GroupGeo<GS>::WARPS;
+    libfit_group_kernel<GS><<<rows, warps * 32, 0, s>>>(W, mask, ms, cols, bits, L, lib, idx, gid, gscale, gmid, cosv);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_libfit_assign(const float* W, const uint8_t* mask, const double* ms, int rows, int cols, int bits, int L,
+                                 int group_size, const uint16_t* lib, uint8_t* idx, uint8_t* gid, uint16_t* gscale,
+                                 uint16_t* gmid, double* cosv, cudaStream_t s) {
+    if (group_size == 64) return launch_groups<64>(W, mask, ms, rows, cols, bits, L, lib, idx, gid, gscale, gmid, cosv, s);
+    if (group_size == 128) return launch_groups<128>(W, mask, ms, rows, cols, bits, L, lib, idx, gid, gscale, gmid, cosv, s);
+    return launch_groups<256>(W, mask, ms, rows, cols, bits, L, lib, idx, gid, gscale, gmid, cosv, s);
+}
+
+cudaError_t launch_libfit_library(const uint16_t* codebook, int rows, int E, int L, int iters, double* u, double* nn,
+                                  int* order, int* asg, double* cen, int* flags, uint16_t* lib, cudaStream_t s) {
+    // a warp per channel, within one block per SM (the blocks wait for one another)
+    const int want = (rows + kLibThreads / 32 - 1) / (kLibThreads / 32), sms = xfp::sm_count();
+    int blocks = want > L ? want : L;
+    if (blocks > sms) blocks = sms;
+    void* args[] = {&codebook, &rows, &E, &L, &iters, &u, &nn, &order, &asg, &cen, &flags, &lib};
+    return cudaLaunchCooperativeKernel((const void*)libfit_library_kernel, dim3((unsigned)blocks), dim3(kLibThreads), args, 0, s);
+}
+
+}  // namespace xq

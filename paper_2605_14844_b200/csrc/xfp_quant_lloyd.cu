@@ -1,23 +1,23 @@
 // "Learned Codebook via Lloyd Iteration": one channel per block, the answer of the serial fp64 evaluation bit for bit.
 //
-// A channel's bulk values (extracted positions hold mu) are sorted, prefix sums are taken in ascending order in fp64, and
-// every round turns 2^N - 1 boundaries into cell means by differences of prefix sums.  lloyd_kernel (channels of up to
-// 16384 weights) spends a few instructions per weight on that:
+// A channel's bulk values (extracted positions hold mu) are put in ascending order, prefix sums are taken in fp64, and every
+// round turns 2^N - 1 boundaries into cell means by differences of prefix sums.  lloyd_kernel (channels of up to 16384
+// weights) spends a few instructions per weight on that:
 //
-//   sort      the kept weights are dealt to about as many equal-width buckets as there are weights (bounds from the
-//             channel's mean and deviation), counted and placed with shared-memory atomics on packed 16-bit counters, and
-//             every weight then counts the smaller members of its own bucket (two or three of them).  A channel whose
-//             fullest bucket holds more than kMaxBucket weights (few distinct values) takes a bitonic network instead.
+//   order     the kept weights are dealt to half as many equal-width buckets as there are weights (bounds from the
+//             channel's mean and deviation), counted and placed with shared-memory atomics on packed 16-bit counters.
+//             Nothing below needs the order inside a bucket except around zero and mu.  A channel whose fullest bucket
+//             holds more than kMaxBucket weights (few distinct values) is sorted by a bitonic network instead.
 //   prefix    a serial chain of K fp64 additions would be the longest phase.  Where no addition of the chain rounds, any
 //             order gives its bits, and that is provable here: with A >= sum |v|, every float of magnitude >= T =
 //             2^(ceil(log2 A) - 30) is a multiple of r = 2^(ceil(log2 A) - 53), and a sum of such values stays below
-//             2^53 r.  So the values below -T are summed in parallel, the few values around zero and mu (and the run of
-//             copies of mu itself) serially, and the values above T in parallel again if the sum S2 that the serial part
-//             left behind is a multiple of 2^-53 times a power of two above every later partial sum (checked; else the
-//             chain goes on serially).  Kept: the prefix at every fourth position ("anchors"); a prefix in between
-//             continues its anchor serially, which is the serial chain itself.
-//   rounds    one warp, a lane per boundary: the boundary's bucket gives its place among the sorted weights to within
-//             a few positions.
+//             2^53 r.  So the values below -T are summed in parallel; the few values around zero and mu (and the run of
+//             copies of mu itself) are sorted and added serially; the values above T are summed in parallel again if the
+//             sum that the serial part left behind is a multiple of 2^-53 times a power of two above every later partial
+//             sum (checked; else the channel is sorted and the chain goes on serially).  Kept: the sum in front of every
+//             fourth position ("anchors"); a sum in between continues its anchor.
+//   rounds    one warp, a lane per boundary: the sum in front of the boundary's bucket, and the bucket's members (two to
+//             five) that are not above it.
 //   indices   the nearest-entry rule is monotone in the weight, so every boundary between two stored entries is one
 //             float threshold, found by evaluating the rule itself; a weight is placed by N comparisons.
 //
@@ -32,7 +32,8 @@ namespace xq {
 namespace {
 
 constexpr int kEpt = 32;            // weights per thread: a block of TH threads takes channels of up to 32 * TH weights
-constexpr int kMaxBucket = 96;      // weights in one bucket beyond which the bitonic network is the cheaper sort
+constexpr int kMaxBucket = 128;     // weights in one bucket beyond which the bitonic network is cheaper than looking through it
+constexpr int kMid = 4;             // weights around zero and mu that are sorted for the serial part, per thread
 constexpr int kShortCols = 16384;   // longest channel that is sorted in shared memory
 
 // Monotone map of a weight to a bucket: one rounding of v * inv + off, clamped; the addition of 2^23 rounds to an integer.
@@ -43,17 +44,6 @@ struct Buckets {
         return __float_as_int(f + 8388608.f) & 0x7fffff;
     }
 };
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    return v;
-}
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    return v;
-}
 
 // r[0..K) ascending: a bitonic network in its all-ascending form (the first step of a merge compares mirrored
 // positions), which tolerates any K: positions beyond it would hold +inf and never move.
@@ -86,36 +76,13 @@ __device__ __forceinline__ int upper_bound(const float* r, int lo, int hi, float
     return lo;
 }
 
-// floats in the order of their values as integers
-__device__ __forceinline__ int ordered(float f) { const int i = __float_as_int(f); return i < 0 ? (int)(0x80000000u - (uint32_t)i) : i; }
-__device__ __forceinline__ float unordered(int o) { return __int_as_float(o < 0 ? (int)(0x80000000u - (uint32_t)o) : o); }
-
-// Largest float x in [a, b) that the nearest-entry rule gives to entry a: |x - a| <= |x - b| in fp64.  The rule is
-// monotone in x; the float below the midpoint keeps it, and the next one nearly always breaks it.
-__device__ float last_of_lower(double a, double b) {
-    const double mid = __dmul_rn(0.5, __dadd_rn(a, b));       // exact: a and b are fp16 values
-    const float c = __double2float_rd(mid);
-    int lo = ordered(c), hi = ordered(__double2float_rn(b));   // the rule holds at lo, breaks at hi
-    if (lo + 1 < hi) {
-        const double x = (double)unordered(lo + 1);
-        if (fabs(__dsub_rn(x, a)) <= fabs(__dsub_rn(x, b))) {
-            while (lo + 1 < hi) {
-                const int m = lo + ((hi - lo) >> 1);
-                const double y = (double)unordered(m);
-                if (fabs(__dsub_rn(y, a)) <= fabs(__dsub_rn(y, b))) lo = m; else hi = m;
-            }
-        }
-    }
-    return unordered(lo);
-}
-
-// What the rounds need of the sorted channel: `r` the kept weights, ascending; m copies of mu behind the first p0 of them.
+// The ordered channel: `r` the kept weights, m copies of mu behind the first p0 of them.
 struct Channel {
     const float* r;
-    const double* anchor;   // prefix sum in front of position 4 i (mu's copies included once 4 i > p0)
-    double p1;              // prefix sum behind mu's copies
+    const double* anchor;   // sum in front of position 4 i (mu's copies included once 4 i > p0)
+    double p1;              // sum behind mu's copies
     int p0;
-    // prefix sum behind the first cu kept weights, and behind mu's copies when `incl` (then cu >= p0)
+    // sum of the first cu kept weights, and of mu's copies when `incl` (then cu >= p0)
     __device__ __forceinline__ double prefix(int cu, bool incl) const {
         int u = cu & ~3;
         double run;
@@ -136,13 +103,13 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
     double* anchor = (double*)(smem + (size_t)K * 4);           // [K / 4 + 1], padded to K / 4 + 2
     uint32_t* cnt2 = (uint32_t*)(anchor + K / 4 + 2);           // [nb / 2] two 16-bit bucket counters a word
     __shared__ double s_red[3][NW];
-    __shared__ float s_f[5][NW];
+    __shared__ float s_f[4][NW];
     __shared__ int s_i[NW];
     __shared__ double c[64], e16[64], val[65];
     __shared__ float thr[64];
     __shared__ int cut[65];
     __shared__ double s_p1, s_p2, s_s1, s_total;
-    __shared__ int s_pos[3], s_shift, s_direct, s_mu_idx;
+    __shared__ int s_pos[3], s_shift, s_direct, s_mu_idx, s_n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = 1 << bits;
     const double mu = ms[0];
@@ -152,44 +119,39 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
 
     // ---- load; moments that bound the buckets and the sums (their own rounding decides nothing) ----
     float v[kEpt];
-    float sum = 0.f, sq = 0.f, ab = 0.f, mn = INFINITY, mx = -INFINITY;
+    float sum = 0.f, sq = 0.f, ab = 0.f, some = 0.f;
     int kept = 0;
 #pragma unroll
     for (int e = 0; e < kEpt / 4; ++e) {
         const int q = e * TH + tid;
         float4 w = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-        uint32_t x = 0;
-        if (q * 4 < K) { w = __ldg(w4 + q); if (m4) x = __ldg(m4 + q); }
+        uint32_t x = 0x01010101u;
+        if (q * 4 < K) { w = __ldg(w4 + q); x = m4 ? __ldg(m4 + q) : 0u; }
         v[4 * e] = (x & 0xffu) ? INFINITY : w.x; v[4 * e + 1] = (x & 0xff00u) ? INFINITY : w.y;
         v[4 * e + 2] = (x & 0xff0000u) ? INFINITY : w.z; v[4 * e + 3] = (x & 0xff000000u) ? INFINITY : w.w;
     }
     for (int i = tid; i < nb / 2; i += TH) cnt2[i] = 0u;
+    // every weight for sum |v| and the count, every fourth for the mean and the deviation
 #pragma unroll
     for (int e = 0; e < kEpt; ++e) {
-        const float x = v[e];
-        if (x < INFINITY) {
-            ++kept; sum += x; sq = fmaf(x, x, sq); ab += fabsf(x); mn = fminf(mn, x); mx = fmaxf(mx, x);
-        }
+        const bool ok = v[e] < INFINITY;
+        const float x = ok ? v[e] : 0.f;
+        kept += ok; ab += fabsf(x);
+        if ((e & 3) == 0) { some += ok ? 1.f : 0.f; sum += x; sq = fmaf(x, x, sq); }
     }
-    sum = warp_sum(sum); sq = warp_sum(sq); ab = warp_sum(ab);
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, d)); mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-        kept += __shfl_xor_sync(0xffffffffu, kept, d);
-    }
-    if (lane == 0) { s_f[0][warp] = sum; s_f[1][warp] = sq; s_f[2][warp] = ab; s_f[3][warp] = mn; s_f[4][warp] = mx; s_i[warp] = kept; }
+    sum = warp_sum(sum); sq = warp_sum(sq); ab = warp_sum(ab); some = warp_sum(some);
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane == 0) { s_f[0][warp] = sum; s_f[1][warp] = sq; s_f[2][warp] = ab; s_f[3][warp] = some; s_i[warp] = kept; }
     __syncthreads();
-    sum = sq = ab = 0.f; mn = INFINITY; mx = -INFINITY; kept = 0;
+    sum = sq = ab = some = 0.f; kept = 0;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        sum += s_f[0][w]; sq += s_f[1][w]; ab += s_f[2][w]; mn = fminf(mn, s_f[3][w]); mx = fmaxf(mx, s_f[4][w]); kept += s_i[w];
-    }
+    for (int w = 0; w < NW; ++w) { sum += s_f[0][w]; sq += s_f[1][w]; ab += s_f[2][w]; some += s_f[3][w]; kept += s_i[w]; }
     const int n = kept, m = K - n;
     Buckets bk{0.f, 0.f, (float)(nb - 1)};
     {
         // 3.3 deviations either side of the mean: a bell-shaped channel then puts at most three or four weights in a bucket
-        const float mean = sum / (float)n, half = 3.3f * sqrtf(fmaxf(sq / (float)n - mean * mean, 0.f));
-        const float lo = fmaxf(mn, mean - half), hi = fminf(mx, mean + half), inv = (float)(nb - 1) / (hi - lo);
+        const float mean = sum / some, half = 3.3f * sqrtf(fmaxf(sq / some - mean * mean, 0.f));
+        const float lo = mean - half, hi = mean + half, inv = (float)(nb - 1) / (hi - lo);
         if (hi > lo && inv < 1e30f && fabsf(lo * inv) < 1e30f) { bk.inv = inv; bk.off = -lo * inv; }
     }
 
@@ -237,7 +199,13 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
     }
     __syncthreads();
     const uint16_t* ends = (const uint16_t*)cnt2;   // after the placement: bucket b holds positions [ends[b - 1], ends[b])
-    if (!full) {
+    const double A = (double)ab * 1.01 + (double)m * fabs(mu);
+    const int eA = A > 0.0 ? ilogb(A) + 1 : -1000;
+    // the values that are added serially lie in [low, high]: zero within T, and mu
+    const double T = ldexp(1.0, eA - 30), low = fmin(-T, mu), high = fmax(T, mu);
+    int q0 = 0, q1 = nb - 1;         // buckets whose members are in ascending order (all of them when `sorted`)
+    bool sorted = full != 0;
+    if (!sorted) {
 #pragma unroll
         for (int e = 0; e < kEpt; ++e)
             if (v[e] < INFINITY) {
@@ -245,44 +213,48 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
                 const uint32_t old = atomicAdd(&cnt2[b >> 1], 1u << sh);
                 r[(old >> sh) & 0xffffu] = v[e];
             }
+        q0 = bk.of(__double2float_rd(low)); q1 = bk.of(__double2float_ru(high));
         __syncthreads();
-        uint32_t to[kEpt / 2];
+        // sort the buckets around zero and mu: a weight counts the smaller members of its own bucket
+        const int t0 = q0 ? ends[q0 - 1] : 0, t1 = ends[q1];
+        sorted = t1 - t0 > kMid * TH;
+        if (!sorted) {
+            float x[kMid];
+            int to[kMid];
 #pragma unroll
-        for (int e = 0; e < kEpt; ++e) {
-            const int t = e * TH + tid;
-            int p = 0;
-            if (t < n) {
-                const float x = r[t];
-                const int b = bk.of(x);
-                const int b0 = b ? ends[b - 1] : 0, b1 = ends[b];
-                p = b0;
-                for (int u = b0; u < b1; ++u) { const float y = r[u]; p += (y < x) || (y == x && u < t); }
-                v[e] = x;
+            for (int e = 0; e < kMid; ++e) {
+                const int t = t0 + e * TH + tid;
+                to[e] = -1;
+                if (t < t1) {
+                    x[e] = r[t];
+                    const int b = bk.of(x[e]), b0 = b ? ends[b - 1] : 0, b1 = ends[b];
+                    to[e] = b0;
+                    for (int u = b0; u < b1; ++u) { const float y = r[u]; to[e] += (y < x[e]) || (y == x[e] && u < t); }
+                }
             }
-            if (e & 1) to[e >> 1] |= (uint32_t)p << 16; else to[e >> 1] = (uint32_t)p;
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < kMid; ++e)
+                if (to[e] >= 0) r[to[e]] = x[e];
+        } else {
+            sort_bitonic(r, n, tid, TH);
         }
+    } else {
+        if (tid == 0) s_n = 0;
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < kEpt; ++e)
-            if (e * TH + tid < n) r[(to[e >> 1] >> ((e & 1) * 16)) & 0xffffu] = v[e];
+            if (v[e] < INFINITY) r[atomicAdd(&s_n, 1)] = v[e];
         __syncthreads();
-    } else {
-#pragma unroll
-        for (int e = 0; e < kEpt; ++e) {
-            const int k = ((e >> 2) * TH + tid) * 4 + (e & 3);
-            if (k < K) r[k] = v[e];               // +inf at the extracted positions: they end up behind the kept weights
-        }
-        __syncthreads();
-        sort_bitonic(r, K, tid, TH);
+        sort_bitonic(r, n, tid, TH);
     }
+    __syncthreads();
 
     // ---- prefix sums (see the head of this file) ----
-    const double A = (double)ab * 1.01 + (double)m * fabs(mu);
-    const int eA = A > 0.0 ? ilogb(A) + 1 : -1000;
     if (warp == 0 && lane < 3) {
-        const double T = ldexp(1.0, eA - 30);
-        const double x = lane == 0 ? fmin(-T, mu) : lane == 1 ? fmax(T, mu) : mu;
+        const double x = lane == 0 ? low : lane == 1 ? high : mu;
         int lo = 0, hi = n;
+        if (!sorted) { lo = q0 ? ends[q0 - 1] : 0; hi = ends[q1]; }
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
             const double y = (double)r[mid];
@@ -333,21 +305,22 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
         }
         if (tid == 0 && n == K && K == kEpt * TH) anchor[K / 4] = total;   // the one anchor no lane owns
         __syncthreads();
-        if (tid == 0) {
-            double run = anchor[pa >> 2];
-            for (int u = pa & ~3; u < pa; ++u) run += (double)r[u];
-            const double s1 = run;
-            double p1 = 0.0;
-            int u = pa;
-            for (;; ++u) {      // the values around zero and mu, in ascending order
+        // the chain over positions [u, end) in ascending order, mu's copies behind position p0
+        auto chain = [&](int u, int end, double run) {
+            for (;; ++u) {
                 if ((u & 3) == 0) anchor[u >> 2] = run;
                 if (u == p0) {
                     for (int i = 0; i < m; ++i) run = __dadd_rn(run, mu);
-                    p1 = run;
+                    s_p1 = run;
                 }
-                if (u >= pb) break;
+                if (u >= end) return run;
                 run = __dadd_rn(run, (double)r[u]);
             }
+        };
+        if (tid == 0) {
+            double s1 = anchor[pa >> 2];
+            for (int u = pa & ~3; u < pa; ++u) s1 += (double)r[u];
+            const double run = chain(pa, pb, s1);
             const double end = run + (total - s1), big = fmax(fabs(run), fabs(end));
             bool direct = true;
             if (big > 0.0) {
@@ -355,19 +328,41 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
                 const double x = ldexp(run, 53 - k);
                 direct = k <= eA && x == rint(x);
             }
-            double fin = end;
-            if (!direct) {      // an addition behind mu may round: the chain itself
-                for (; u < n; ) {
-                    run = __dadd_rn(run, (double)r[u]);
-                    ++u;
-                    if ((u & 3) == 0) anchor[u >> 2] = run;
+            s_s1 = s1; s_p2 = run; s_total = end; s_direct = direct;
+        }
+        // meanwhile the other warps find the start of the rounds, the (j + 1/2) / 2^N quantiles: P threads to a quantile,
+        // each ranks its share of the quantile's bucket
+        {
+            int P = 1;
+            while (2 * P * E <= TH - 32) P *= 2;
+            for (int i = tid - 32; i >= 0 && i < E * P; i += TH - 32) {
+                const int j = i / P, sub = i % P;
+                long long q = (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)j, 0.5), (double)K), (double)E));
+                if (q >= K) q = K - 1;
+                int t = (int)q;
+                if (t >= p0 && t < p0 + m) { c[j] = mu; continue; }
+                if (t >= p0 + m) t -= m;
+                if (sorted) { c[j] = (double)r[t]; continue; }
+                int lo = 0, hi = nb - 1;          // the bucket of position t
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (ends[mid] > t) hi = mid; else lo = mid + 1;
                 }
-                fin = run;
+                const int b0 = lo ? ends[lo - 1] : 0, b1 = ends[lo];
+                for (int a = b0 + sub; a < b1; a += P) {
+                    const float y = r[a];
+                    int less = 0, same = 0;
+                    for (int u = b0; u < b1; ++u) { less += r[u] < y; same += r[u] == y; }
+                    if (t - b0 >= less && t - b0 < less + same) c[j] = (double)y;
+                }
             }
-            s_s1 = s1; s_p1 = p1; s_p2 = run; s_total = fin; s_direct = direct;
         }
         __syncthreads();
-        if (s_direct) {
+        if (!s_direct) {          // an addition behind mu may round: sort everything and run the whole chain
+            if (!sorted) sort_bitonic(r, n, tid, TH);
+            sorted = true;
+            if (tid == 0) s_total = chain(0, n, 0.0);
+        } else {
             const double s1 = s_s1, p2 = s_p2;
 #pragma unroll
             for (int e = 0; e < kEpt / 4; ++e) {
@@ -382,40 +377,84 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
     // ---- rounds: one warp, a lane per boundary and entry ----
     if (warp == 0) {
         const Channel ch{r, anchor, s_p1, p0};
-        for (int j = lane; j < E; j += 32) {
-            long long q = (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)j, 0.5), (double)K), (double)E));
-            if (q >= K) q = K - 1;
-            const int t = (int)q;
-            c[j] = t < p0 ? (double)r[t] : t < p0 + m ? mu : (double)r[t - m];
-        }
-        if (lane == 0) { cut[0] = 0; val[0] = 0.0; cut[E] = K; val[E] = s_total; }
-        __syncwarp();
-        for (int it = 0; it < iters; ++it) {
-            // cell j = (b_{j-1}, b_j], b_j the midpoint of entries j and j+1: cut[j+1] = #{values <= b_j}
-            for (int j = lane; j < E - 1; j += 32) {
-                const double b = __dmul_rn(0.5, __dadd_rn(c[j], c[j + 1]));
-                const float bf = __double2float_rd(b);       // a float is <= b when it is <= bf
-                const bool incl = mu <= b;
-                int lo = 0, hi = n;
-                if (!full) {
-                    const int q = bk.of(bf);
-                    lo = q ? ends[q - 1] : 0; hi = ends[q];
-                }
+        const double total = s_total;
+        constexpr int kWin = 16;        // weights from the boundary's anchor on that are looked at without a loop
+        // count of the values <= b and their sum in the chain's order
+        auto below = [&](double b, int& cu, double& sum_b) {
+            const float bf = __double2float_rd(b);       // a float is <= b when it is <= bf
+            const bool incl = mu <= b;
+            int lo = 0, hi = n;
+            bool look = sorted;
+            if (!sorted) {
+                const int q = bk.of(bf);
+                lo = q ? ends[q - 1] : 0; hi = ends[q];
+                look = q >= q0 && q <= q1;
+            }
+            const int u0 = lo & ~3;
+            if (look) {
                 lo = upper_bound(r, lo, hi, bf);
-                cut[j + 1] = lo + (incl ? m : 0);
-                val[j + 1] = ch.prefix(lo, incl);
-            }
-            __syncwarp();
-            bool changed = false;
-            for (int j = lane; j < E; j += 32) {
-                const int cells = cut[j + 1] - cut[j];
-                if (cells > 0) {
-                    const double mean = __ddiv_rn(__dsub_rn(val[j + 1], val[j]), (double)cells);
-                    if (mean != c[j]) { c[j] = mean; changed = true; }
+                sum_b = ch.prefix(lo, incl);
+            } else if (hi <= u0 + kWin && (!incl || (u0 >= pb && u0 > p0))) {     // no addition rounds here, whatever the order
+                double part[4] = {anchor[u0 >> 2], 0.0, 0.0, 0.0};
+                int in = 0;
+#pragma unroll
+                for (int i = 0; i < kWin / 4; ++i) {
+                    // the window may reach past the channel (into the anchors behind it): masked by `hi`
+                    const float4 f4 = *(const float4*)(r + u0 + 4 * i);
+                    const float f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int u = u0 + 4 * i + k;
+                        const bool take = u < lo || (u < hi && f[k] <= bf);
+                        in += take;
+                        part[k] += (double)(take ? f[k] : 0.f);
+                    }
                 }
+                sum_b = (part[0] + part[1]) + (part[2] + part[3]);
+                lo = u0 + in;
+            } else {
+                sum_b = ch.prefix(lo, incl);
+                const int b0 = lo;
+                for (int u = b0; u < hi; ++u) { const float y = r[u]; if (y <= bf) { sum_b += (double)y; ++lo; } }
             }
-            if (!__any_sync(0xffffffffu, changed)) break;
-            __syncwarp();
+            cu = lo + (incl ? m : 0);
+        };
+        // cell j = (b_{j-1}, b_j], b_j the midpoint of entries j and j+1: a lane's cell ends where its boundary lies
+        if (E <= 32) {
+            double cj = c[lane < E ? lane : E - 1];
+            for (int it = 0; it < iters; ++it) {
+                const double cn = __shfl_down_sync(0xffffffffu, cj, 1);
+                int cu = K;
+                double sum_b = total;
+                if (lane < E - 1) below(__dmul_rn(0.5, __dadd_rn(cj, cn)), cu, sum_b);
+                __syncwarp();
+                int c0 = __shfl_up_sync(0xffffffffu, cu, 1);
+                double v0 = __shfl_up_sync(0xffffffffu, sum_b, 1);
+                if (lane == 0) { c0 = 0; v0 = 0.0; }
+                bool changed = false;
+                if (lane < E && cu > c0) {
+                    const double mean = __ddiv_rn(__dsub_rn(sum_b, v0), (double)(cu - c0));
+                    changed = mean != cj;
+                    cj = mean;
+                }
+                if (!__any_sync(0xffffffffu, changed)) break;
+            }
+            if (lane < E) c[lane] = cj;
+        } else {
+            if (lane == 0) { cut[0] = 0; val[0] = 0.0; cut[E] = K; val[E] = total; }
+            for (int it = 0; it < iters; ++it) {
+                for (int j = lane; j < E - 1; j += 32) below(__dmul_rn(0.5, __dadd_rn(c[j], c[j + 1])), cut[j + 1], val[j + 1]);
+                __syncwarp();
+                bool changed = false;
+                for (int j = lane; j < E; j += 32) {
+                    if (cut[j + 1] > cut[j]) {
+                        const double mean = __ddiv_rn(__dsub_rn(val[j + 1], val[j]), (double)(cut[j + 1] - cut[j]));
+                        if (mean != c[j]) { c[j] = mean; changed = true; }
+                    }
+                }
+                if (!__any_sync(0xffffffffu, changed)) break;
+                __syncwarp();
+            }
         }
         __syncwarp();
         for (int j = lane; j < E; j += 32) {
@@ -748,8 +787,8 @@ size_t long_slice_doubles(int cols, int* kp2_out) {
 template <int TH>
 cudaError_t launch_short(const float* W, const uint8_t* mask, const double* ms, int rows, int cols, int bits, int iters,
                          uint16_t* codebook, uint8_t* idx, double* cosv, int* rowcnt, cudaStream_t s) {
-    int nb = 8 * TH;                                   // a counter per weight, within 8 TH (the scan's vectors) .. 8192
-    while (nb < cols && nb < 8192) nb <<= 1;
+    int nb = 8 * TH;                                   // a counter per two weights, at least the scan's vectors
+    while (nb < cols / 2) nb <<= 1;
     const size_t smem = (size_t)cols * 4 + ((size_t)cols / 4 + 2) * 8 + (size_t)nb * 2;
     static xfp::DeviceOnce done;
     const int dev = xfp::DeviceOnce::current();
