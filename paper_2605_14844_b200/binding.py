@@ -1,8 +1,10 @@
 """Python binding of the XFP C ABI (include/xfp.h): argument marshalling only.
 
 Every function takes torch tensors (device memory, streams) and hands raw pointers to
-libxfp.so; all arithmetic runs in the library's CUDA kernels.  There is no CPU fallback: if the
-library has not been built the import of a function fails with XfpError.
+libxfp.so; all arithmetic runs in the library's CUDA kernels.  The calls that queue device work go
+through a native module (csrc/xfp_native.cpp), because a decode step's kernels take a few
+microseconds each; the rest uses ctypes.  There is no CPU fallback: if the library has not been
+built the first call of a function fails with XfpError.
 """
 from __future__ import annotations
 
@@ -14,6 +16,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB = None
+_NATIVE = None     # the marshalling module (csrc/xfp_native.cpp), bound to the loaded library
 
 EXPORTS = ("xfp_packed_size", "xfp_pack", "xfp_gemv_v2", "xfp_gemv_v2a", "xfp_gemv_grouped", "xfp_gemv_host",
            "xfp_dequant", "xfp_status_str", "xfp_gemv_v2_noalloc", "xfp_gemv_grouped_epilogue", "xfp_gemv_typed",
@@ -77,6 +80,22 @@ def load_library() -> C.CDLL:
     return lib
 
 
+def _native():
+    """_xfp_native, its entry points taken from the loaded library."""
+    global _NATIVE
+    if _NATIVE is None:
+        lib = load_library()
+        try:
+            from . import _xfp_native as native
+        except ImportError as e:
+            raise XfpError(f"_xfp_native.so: {e}: run `python -m paper_2605_14844_b200.build`") from e
+        native.bind(*[C.cast(getattr(lib, n), C.c_void_p).value for n in
+                      ("xfp_pack", "xfp_gemv_v2", "xfp_gemv_v2a", "xfp_gemv_typed", "xfp_gemv_grouped_typed",
+                       "xfp_gemv_host", "xfp_gemv_v2_noalloc", "xfp_gemm_typed", "xfp_dequant")])
+        _NATIVE = native
+    return _NATIVE
+
+
 def xfp_status_str(status: int) -> str:
     return load_library().xfp_status_str(int(status)).decode()
 
@@ -105,23 +124,22 @@ def xfp_packed_size(desc: XfpDesc):
 
 def xfp_pack(desc: XfpDesc, idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, out_val,
              packed: torch.Tensor, err_word: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(load_library().xfp_pack(C.byref(desc), _ptr(idx), _ptr(codebook), _ptr(group_id), _ptr(group_scale),
-                                   _ptr(group_mid), _ptr(out_rowptr), _ptr(out_col), _ptr(out_val), _ptr(packed),
-                                   packed.numel() * packed.element_size(), _ptr(err_word), _stream(stream)),
-           "xfp_pack")
-
-
-def _gemv(fn, desc, packed, x, batch, y, y_is_fp16, workspace, stream):
-    _check(fn(C.byref(desc), _ptr(packed), _ptr(x), int(batch), _ptr(y), int(bool(y_is_fp16)), _ptr(workspace),
-              workspace.numel() * workspace.element_size(), _stream(stream)), fn.__name__)
+    status = (_NATIVE or _native()).pack(desc, idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, out_val,
+                                         packed, err_word, stream)
+    if status:
+        _check(status, "xfp_pack")
 
 
 def xfp_gemv_v2(desc, packed, x, batch, y, y_is_fp16, workspace, stream=None) -> None:
-    _gemv(load_library().xfp_gemv_v2, desc, packed, x, batch, y, y_is_fp16, workspace, stream)
+    status = (_NATIVE or _native()).gemv(0, desc, packed, x, batch, y, y_is_fp16, workspace, stream)
+    if status:
+        _check(status, "xfp_gemv_v2")
 
 
 def xfp_gemv_v2a(desc, packed, x, batch, y, y_is_fp16, workspace, stream=None) -> None:
-    _gemv(load_library().xfp_gemv_v2a, desc, packed, x, batch, y, y_is_fp16, workspace, stream)
+    status = (_NATIVE or _native()).gemv(1, desc, packed, x, batch, y, y_is_fp16, workspace, stream)
+    if status:
+        _check(status, "xfp_gemv_v2a")
 
 
 _TORCH_TYPE = {torch.float32: XFP_T_F32, torch.float16: XFP_T_F16, torch.bfloat16: XFP_T_BF16}
@@ -129,9 +147,9 @@ _TORCH_TYPE = {torch.float32: XFP_T_F32, torch.float16: XFP_T_F16, torch.bfloat1
 
 def xfp_gemv_typed(desc, packed, x: torch.Tensor, batch, y: torch.Tensor, workspace, stream=None) -> None:
     """The fused GEMV of desc.mode with x in fp16 or bf16 and y in fp32, fp16 or bf16 (taken from the tensors' dtypes)."""
-    _check(load_library().xfp_gemv_typed(C.byref(desc), _ptr(packed), _ptr(x), _TORCH_TYPE[x.dtype], int(batch), _ptr(y),
-                                         _TORCH_TYPE[y.dtype], _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream)), "xfp_gemv_typed")
+    status = (_NATIVE or _native()).gemv_typed(desc, packed, x, batch, y, workspace, stream)
+    if status:
+        _check(status, "xfp_gemv_typed")
 
 
 def xfp_gemm_workspace_size(desc, m: int) -> int:
@@ -158,18 +176,23 @@ def xfp_gemm_typed_workspace_size(desc, m: int, x_dtype=torch.bfloat16) -> int:
 def xfp_gemm_typed(desc, packed, x: torch.Tensor, y: torch.Tensor, workspace: torch.Tensor, stream=None) -> None:
     """xfp_gemm with x in fp16 or bf16 (taken from the tensor's dtype); workspace sized by
     xfp_gemm_typed_workspace_size(desc, m, x.dtype)."""
-    _check(load_library().xfp_gemm_typed(C.byref(desc), _ptr(packed), _ptr(x), _TORCH_TYPE[x.dtype], int(x.shape[0]),
-                                         _ptr(y), _TORCH_TYPE[y.dtype], _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream)), "xfp_gemm_typed")
+    status = (_NATIVE or _native()).gemm(desc, packed, x, y, workspace, stream)
+    if status:
+        _check(status, "xfp_gemm_typed")
+
+
+def _grouped(what: str, desc, n, packed_ptrs, x_ptrs, x_type, y_ptrs, y_type, epilogue, weights, workspace, stream) -> None:
+    status = (_NATIVE or _native()).grouped(desc, n, packed_ptrs, x_ptrs, x_type, y_ptrs, y_type, epilogue, weights, workspace,
+                                            stream)
+    if status:
+        _check(status, what)
 
 
 def xfp_gemv_grouped(desc, n: int, packed_ptrs: torch.Tensor, x_ptrs: torch.Tensor, y_ptrs: torch.Tensor,
                      y_is_fp16, workspace: torch.Tensor, stream=None) -> None:
     """packed_ptrs / x_ptrs / y_ptrs: int64 device tensors holding n device addresses each."""
-    _check(load_library().xfp_gemv_grouped(C.byref(desc), int(n), _ptr(packed_ptrs), _ptr(x_ptrs), _ptr(y_ptrs),
-                                           int(bool(y_is_fp16)), _ptr(workspace),
-                                           workspace.numel() * workspace.element_size(), _stream(stream)),
-           "xfp_gemv_grouped")
+    _grouped("xfp_gemv_grouped", desc, n, packed_ptrs, x_ptrs, XFP_T_F16, y_ptrs, XFP_T_F16 if y_is_fp16 else XFP_T_F32,
+             XFP_EPI_NONE, None, workspace, stream)
 
 
 def xfp_gemv_grouped_epilogue(desc, n: int, packed_ptrs: torch.Tensor, x_ptrs: torch.Tensor, y_ptrs: torch.Tensor,
@@ -177,10 +200,8 @@ def xfp_gemv_grouped_epilogue(desc, n: int, packed_ptrs: torch.Tensor, x_ptrs: t
                               stream=None) -> None:
     """xfp_gemv_grouped with a fused store: XFP_EPI_SWIGLU (y[j] gets rows/2 values SiLU(gate)*up) or
     XFP_EPI_COMBINE (y[0] = sum_j weights[j] * W_j x[j]; weights: float32 device tensor of n values)."""
-    _check(load_library().xfp_gemv_grouped_epilogue(C.byref(desc), int(n), _ptr(packed_ptrs), _ptr(x_ptrs),
-                                                    _ptr(y_ptrs), int(bool(y_is_fp16)), int(epilogue), _ptr(weights),
-                                                    _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                                    _stream(stream)), "xfp_gemv_grouped_epilogue")
+    _grouped("xfp_gemv_grouped_epilogue", desc, n, packed_ptrs, x_ptrs, XFP_T_F16, y_ptrs,
+             XFP_T_F16 if y_is_fp16 else XFP_T_F32, epilogue, weights, workspace, stream)
 
 
 def xfp_gemv_grouped_typed(desc, n: int, packed_ptrs: torch.Tensor, x_ptrs: torch.Tensor, x_dtype, y_ptrs: torch.Tensor,
@@ -188,30 +209,29 @@ def xfp_gemv_grouped_typed(desc, n: int, packed_ptrs: torch.Tensor, x_ptrs: torc
                            stream=None) -> None:
     """The grouped launch with fp16 / bf16 activations and fp32 / fp16 / bf16 outputs (torch dtypes) and an optional
     fused store (XFP_EPI_*)."""
-    _check(load_library().xfp_gemv_grouped_typed(C.byref(desc), int(n), _ptr(packed_ptrs), _ptr(x_ptrs),
-                                                 _TORCH_TYPE[x_dtype], _ptr(y_ptrs), _TORCH_TYPE[y_dtype], int(epilogue),
-                                                 _ptr(weights), _ptr(workspace),
-                                                 workspace.numel() * workspace.element_size(), _stream(stream)),
-           "xfp_gemv_grouped_typed")
+    _grouped("xfp_gemv_grouped_typed", desc, n, packed_ptrs, x_ptrs, _TORCH_TYPE[x_dtype], y_ptrs, _TORCH_TYPE[y_dtype],
+             epilogue, weights, workspace, stream)
 
 
 def xfp_gemv_host(desc, packed, x_host: torch.Tensor, x_dev, batch, y_host: torch.Tensor, y_dev, y_is_fp16,
                   workspace, stream=None) -> None:
-    _check(load_library().xfp_gemv_host(C.byref(desc), _ptr(packed), _ptr(x_host), _ptr(x_dev), int(batch),
-                                        _ptr(y_host), _ptr(y_dev), int(bool(y_is_fp16)), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _stream(stream)),
-           "xfp_gemv_host")
+    status = (_NATIVE or _native()).gemv_host(desc, packed, x_host, x_dev, batch, y_host, y_dev, y_is_fp16, workspace, stream)
+    if status:
+        _check(status, "xfp_gemv_host")
 
 
 def xfp_gemv_v2_noalloc(desc, packed, x, batch, y, y_is_fp16, stream=None) -> None:
     """V2 GEMV that uses the library's built-in 8 MiB scratch instead of a caller workspace: for callers
     that are not allowed to allocate device memory.  Calls must not overlap on the GPU (shared scratch)."""
-    _check(load_library().xfp_gemv_v2_noalloc(C.byref(desc), _ptr(packed), _ptr(x), int(batch), _ptr(y),
-                                              int(bool(y_is_fp16)), _stream(stream)), "xfp_gemv_v2_noalloc")
+    status = (_NATIVE or _native()).noalloc(desc, packed, x, batch, y, y_is_fp16, stream)
+    if status:
+        _check(status, "xfp_gemv_v2_noalloc")
 
 
 def xfp_dequant(desc, packed, W: torch.Tensor, stream=None) -> None:
-    _check(load_library().xfp_dequant(C.byref(desc), _ptr(packed), _ptr(W), _stream(stream)), "xfp_dequant")
+    status = (_NATIVE or _native()).dequant(desc, packed, W, stream)
+    if status:
+        _check(status, "xfp_dequant")
 
 
 # ------------------------------------------------------------------ conveniences (still marshalling only)
@@ -245,11 +265,12 @@ class PackedMatrix:
 
     def gemv(self, x: torch.Tensor, y: Optional[torch.Tensor] = None, y_fp16: bool = False, stream=None):
         """x: fp16 [batch, cols] on the device -> y [batch, rows] fp32 (or fp16)."""
-        batch = x.shape[0] if x.dim() == 2 else 1
         if y is None:
-            y = torch.empty((batch, self.desc.rows), dtype=torch.float16 if y_fp16 else torch.float32, device=x.device)
-        fn = xfp_gemv_v2a if self.desc.mode else xfp_gemv_v2
-        fn(self.desc, self.packed, x, batch, y, y_fp16, self.workspace, stream)
+            y = torch.empty((x.shape[0] if x.dim() == 2 else 1, self.desc.rows),
+                            dtype=torch.float16 if y_fp16 else torch.float32, device=x.device)
+        status = (_NATIVE or _native()).gemv(-1, self.desc, self.packed, x, -1, y, y_fp16, self.workspace, stream)
+        if status:
+            _check(status, "xfp_gemv_v2a" if self.desc.mode else "xfp_gemv_v2")
         return y
 
     def dequant(self, stream=None) -> torch.Tensor:
