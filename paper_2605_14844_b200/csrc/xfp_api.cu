@@ -248,12 +248,13 @@ int xfp_gemm_workspace_size(const xfp_desc* desc, int32_t m, size_t* workspace_b
     if (m < 1) return XFP_ERR_SHAPE;
     const Layout l = layout_of(desc);
     if (!gemm_tc_supported(l, m)) return XFP_ERR_UNSUPPORTED;
-    *workspace_bytes = gemm_workspace_bytes(l, m);
+    *workspace_bytes = prefill_workspace_bytes(l, m);
     return XFP_OK;
 }
 
-int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
-             void* workspace, size_t workspace_bytes, void* stream) {
+// x_type as for xfp_gemm_typed; the sizes and pointers of the call are checked here
+static int gemm_common(const xfp_desc* desc, const void* packed, const void* x, int32_t x_type, int32_t m, void* y,
+                       int32_t y_type, void* workspace, size_t workspace_bytes, cudaStream_t s) {
     int st = check_desc(desc);
     if (st) return st;
     if (m < 1 || y_type < 0 || y_type > 2) return XFP_ERR_SHAPE;
@@ -261,9 +262,23 @@ int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_
     if (!aligned16(packed) || !aligned16(x) || !aligned16(y) || !aligned16(workspace)) return XFP_ERR_ALIGN;
     const Layout l = layout_of(desc);
     if (!gemm_tc_supported(l, m)) return XFP_ERR_UNSUPPORTED;
-    if (workspace_bytes < gemm_workspace_bytes(l, m)) return XFP_ERR_BUFFER_TOO_SMALL;
-    GemmCall c{packed, x, y, m, y_type, workspace, workspace_bytes};
-    return launch_gemm_tc(l, c, (cudaStream_t)stream) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    const bool dense = dense_preferred(l, m);
+    const size_t own = dense ? dense_workspace_bytes(l, m) : gemm_workspace_bytes(l, m);
+    const size_t need = x_type == XFP_T_BF16 ? align256(own) + gemm_x_scratch_bytes(l, m) : own;
+    if (workspace_bytes < need) return XFP_ERR_BUFFER_TOO_SMALL;
+    uint16_t* x16 = x_type == XFP_T_BF16 ? (uint16_t*)((char*)workspace + align256(own)) : nullptr;
+    GemmCall c{packed, (const uint16_t*)x, y, m, y_type, workspace, own};
+    if (dense) return launch_gemm_dense(l, c, x16, s) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    if (x16) {
+        if (launch_x_to_f16(x, x16, (size_t)m * l.cols, s) != cudaSuccess) return XFP_ERR_CUDA;
+        c.x = x16;
+    }
+    return launch_gemm_tc(l, c, s) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+}
+
+int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
+             void* workspace, size_t workspace_bytes, void* stream) {
+    return gemm_common(desc, packed, x, XFP_T_F16, m, y, y_type, workspace, workspace_bytes, (cudaStream_t)stream);
 }
 
 int xfp_gemm_typed_workspace_size(const xfp_desc* desc, int32_t m, int32_t x_type, size_t* workspace_bytes) {
@@ -279,19 +294,8 @@ int xfp_gemm_typed_workspace_size(const xfp_desc* desc, int32_t m, int32_t x_typ
 
 int xfp_gemm_typed(const xfp_desc* desc, const void* packed, const void* x, int32_t x_type, int32_t m, void* y,
                    int32_t y_type, void* workspace, size_t workspace_bytes, void* stream) {
-    if (x_type == XFP_T_F16) return xfp_gemm(desc, packed, (const uint16_t*)x, m, y, y_type, workspace, workspace_bytes, stream);
-    if (x_type != XFP_T_BF16) return XFP_ERR_SHAPE;
-    size_t need = 0;
-    int st = xfp_gemm_typed_workspace_size(desc, m, x_type, &need);
-    if (st) return st;
-    if (!packed || !x || !y || !workspace) return XFP_ERR_NULL;
-    if (!aligned16(x) || !aligned16(workspace)) return XFP_ERR_ALIGN;
-    if (workspace_bytes < need) return XFP_ERR_BUFFER_TOO_SMALL;
-    const Layout l = layout_of(desc);
-    const size_t own = align256(gemm_workspace_bytes(l, m));
-    uint16_t* x16 = (uint16_t*)((char*)workspace + own);
-    if (launch_x_to_f16(x, x16, (size_t)m * l.cols, (cudaStream_t)stream) != cudaSuccess) return XFP_ERR_CUDA;
-    return xfp_gemm(desc, packed, x16, m, y, y_type, workspace, own, stream);
+    if (x_type != XFP_T_F16 && x_type != XFP_T_BF16) return XFP_ERR_SHAPE;
+    return gemm_common(desc, packed, x, x_type, m, y, y_type, workspace, workspace_bytes, (cudaStream_t)stream);
 }
 
 int xfp_dequant(const xfp_desc* desc, const void* packed, uint16_t* W, void* stream) {
