@@ -262,13 +262,13 @@ static int gemm_common(const xfp_desc* desc, const void* packed, const void* x, 
     if (!aligned16(packed) || !aligned16(x) || !aligned16(y) || !aligned16(workspace)) return XFP_ERR_ALIGN;
     const Layout l = layout_of(desc);
     if (!gemm_tc_supported(l, m)) return XFP_ERR_UNSUPPORTED;
-    const bool dense = dense_preferred(l, m);
-    const size_t own = dense ? dense_workspace_bytes(l, m) : gemm_workspace_bytes(l, m);
+    const bool fused = fused_preferred(l, m);
+    const size_t own = prefill_workspace_bytes(l, m);
     const size_t need = x_type == XFP_T_BF16 ? align256(own) + gemm_x_scratch_bytes(l, m) : own;
     if (workspace_bytes < need) return XFP_ERR_BUFFER_TOO_SMALL;
     uint16_t* x16 = x_type == XFP_T_BF16 ? (uint16_t*)((char*)workspace + align256(own)) : nullptr;
     GemmCall c{packed, (const uint16_t*)x, y, m, y_type, workspace, own};
-    if (dense) return launch_gemm_dense(l, c, x16, s) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    if (fused) return launch_gemm_fused(l, c, x16, s) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
     if (x16) {
         if (launch_x_to_f16(x, x16, (size_t)m * l.cols, s) != cudaSuccess) return XFP_ERR_CUDA;
         c.x = x16;

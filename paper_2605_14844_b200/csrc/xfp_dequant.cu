@@ -1,5 +1,4 @@
-// xfp_dequant: device layout -> W^ = fp16(D16 + S), bit-exact ("Reconstruct" in Algorithm 1), as the caller's fp16 matrix
-// or as the A-operand tiles of the prefill GEMM (xfp_gemm_dense.cu).
+// xfp_dequant: device layout -> fp16 matrix W^ = fp16(D16 + S), bit-exact ("Reconstruct" in Algorithm 1).
 //
 // A block of eight warps takes one row-block (32 channels, a lane each) and a range of super-chunks; a warp decodes one
 // super-chunk at a time from index vectors fetched one super-chunk ahead.
@@ -8,9 +7,7 @@
 //   V2a  a lane decodes the 2^N entries its channel's group can take once -- D16 = fp16(fp32(scale * lib[id] + mid)) --
 //        into a column of a table of its warp, and the weights of the group are look-ups as in V2: 2^N conversions per
 //        group instead of one per weight (N = 2: pairs; at N = 6 64 entries serve 128 weights).
-//   out  matrix: a tile of shared memory turns a lane's 64 weights into whole 128-byte lines of the channels' rows.
-//        GEMM tiles: 128 channels x 64 k in core-matrix order, [k / 8][channel][8], so that a lane's 16 bytes lie beside its
-//        neighbours' and a warp stores 512 consecutive bytes straight from registers.
+//   out  a tile of shared memory turns a lane's 64 weights into whole 128-byte lines of the channels' rows.
 //   S    when the block has stored its range, its outliers are added in place, one correctly rounded fp16 addition each:
 //        the slots of the transposed slab are dealt to the warps eight at a time, so that the loads of a batch overlap.
 #include "xfp_internal.h"
@@ -56,37 +53,24 @@ struct DqArgs {
     Blob b;
     uint16_t* out;
     int rows, cols, RB, SC, GH, L, ell_slots;
-    int rb0;                  // first row-block of this launch
     int range;                // super-chunks of a block
-    int blocks;               // decode blocks; the blocks behind them convert x
-    const uint4* x_bf16;      // bf16 activations to convert to fp16 (null: none), 8 values each
-    uint4* x_f16;
-    unsigned x8;
-    int wait;                 // the launch runs under the previous GEMM: its last block waits for that one's end
 };
 
-template <int N, int MODE, bool TILES>
-__global__ void __launch_bounds__(kDqWarps * 32) decode_kernel(const DqArgs a) {
+template <int N, int MODE>
+__global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) {
     using T = DqTab<N, MODE>;
     constexpr int E = T::E;
     extern __shared__ unsigned char dq_smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    asm volatile("griddepcontrol.launch_dependents;");
-    if ((int)blockIdx.x >= a.blocks) {
-        const unsigned step = (gridDim.x - (unsigned)a.blocks) * (kDqWarps * 32);
-        for (unsigned i = ((unsigned)blockIdx.x - (unsigned)a.blocks) * (kDqWarps * 32) + tid; i < a.x8; i += step)
-            a.x_f16[i] = x8_as_f16(__ldg(a.x_bf16 + i), 1);
-        return;
-    }
     const int parts = (a.SC + a.range - 1) / a.range;
-    const int rb = a.rb0 + (int)blockIdx.x / parts, part = (int)blockIdx.x % parts;
+    const int rb = (int)blockIdx.x / parts, part = (int)blockIdx.x % parts;
     const int s0 = part * a.range, s1 = min(a.SC, s0 + a.range);
     // tables aligned to their size in the shared window (at least 1 KB), so that an entry's offset is merged, not added
     constexpr uint32_t kAlign = T::kBytes < 1024 ? 1024 : T::kBytes;
     const uint32_t raw = smem_addr(dq_smem), tab0 = (raw + kAlign - 1) & ~(kAlign - 1);
     unsigned char* base = dq_smem + (tab0 - raw);
-    unsigned char* tiles = base + T::kTables * kAlign;                        // [warps][32 * kTileRow], matrix output only
-    uint16_t* slib = (uint16_t*)(tiles + (TILES ? 0 : kDqWarps * 32 * kTileRow));   // [L][lib_stride]
+    unsigned char* tiles = base + T::kTables * kAlign;                        // [warps][32 * kTileRow]
+    uint16_t* slib = (uint16_t*)(tiles + kDqWarps * 32 * kTileRow);   // [L][lib_stride]
     constexpr int kLibStride = E + 8;                                        // 16 bytes of padding spread the ids over the banks
     const bool staged = MODE == 1 && a.L * E <= kLibEntries;
     if (MODE == 0) {
@@ -176,26 +160,17 @@ __global__ void __launch_bounds__(kDqWarps * 32) decode_kernel(const DqArgs a) {
                     }
                 }
                 const uint4 v = make_uint4(d[0], d[1], d[2], d[3]);
-                if (TILES) {
-                    const int rl = row - a.rb0 * kRowsPerBlock;            // channel inside the launch's tiles
-                    unsigned char* dst = (unsigned char*)a.out + ((size_t)(rl >> 7) * (2 * a.SC) + 2 * sc + h) * 16384 +
-                                         (size_t)c * 2048 + (size_t)(rl & 127) * 16;
-                    *(uint4*)dst = v;
-                } else {
-                    *(uint4*)(tile + lane * kTileRow + c * 16) = v;
-                }
+                *(uint4*)(tile + lane * kTileRow + c * 16) = v;
             }
-            if (!TILES) {
-                __syncwarp();
+            __syncwarp();
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {             // four channels' 128 bytes per step
-                    const int r = 4 * i + (lane >> 3), orow = rb * kRowsPerBlock + r;
-                    if (orow < a.rows)
-                        *(uint4*)(a.out + (size_t)orow * a.cols + (size_t)sc * kSuper + h * 64 + (lane & 7) * 8) =
-                            *(const uint4*)(tile + r * kTileRow + (lane & 7) * 16);
-                }
-                __syncwarp();
+            for (int i = 0; i < 8; ++i) {                 // four channels' 128 bytes per step
+                const int r = 4 * i + (lane >> 3), orow = rb * kRowsPerBlock + r;
+                if (orow < a.rows)
+                    *(uint4*)(a.out + (size_t)orow * a.cols + (size_t)sc * kSuper + h * 64 + (lane & 7) * 8) =
+                        *(const uint4*)(tile + r * kTileRow + (lane & 7) * 16);
             }
+            __syncwarp();
         }
     }
     // ---- W^ += S on the values this block has just stored ----
@@ -204,12 +179,7 @@ __global__ void __launch_bounds__(kDqWarps * 32) decode_kernel(const DqArgs a) {
         const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
         const int len = row < a.rows ? (int)__ldg(slab) : 0, in_slab = min(len, a.ell_slots);
         const uint32_t k0 = (uint32_t)s0 * kSuper, k1 = (uint32_t)s1 * kSuper;
-        auto place = [&](uint32_t col) -> uint16_t* {
-            if (!TILES) return a.out + (size_t)row * a.cols + col;
-            const int rl = row - a.rb0 * kRowsPerBlock;
-            return (uint16_t*)((unsigned char*)a.out + ((size_t)(rl >> 7) * (2 * a.SC) + (col >> 6)) * 16384 +
-                               (size_t)((col >> 3) & 7u) * 2048 + (size_t)(rl & 127) * 16) + (col & 7u);
-        };
+        uint16_t* out = a.out + (size_t)row * a.cols;
         constexpr int kBatch = 8;
         auto batch = [&](const uint32_t* src, int stride, int first, int end) {       // entries first, first + kDqWarps, ...
             uint32_t e[kBatch];
@@ -221,11 +191,11 @@ __global__ void __launch_bounds__(kDqWarps * 32) decode_kernel(const DqArgs a) {
             for (int i = 0; i < kBatch; ++i) {
                 const uint32_t col = e[i] & 0xffffu;
                 ok[i] = first + i * kDqWarps < end && col >= k0 && col < k1;
-                if (ok[i]) old[i] = *place(col);
+                if (ok[i]) old[i] = out[col];
             }
 #pragma unroll
             for (int i = 0; i < kBatch; ++i)
-                if (ok[i]) *place(e[i] & 0xffffu) = __half_as_ushort(__hadd(__ushort_as_half(old[i]), __ushort_as_half((uint16_t)(e[i] >> 16))));
+                if (ok[i]) out[e[i] & 0xffffu] = __half_as_ushort(__hadd(__ushort_as_half(old[i]), __ushort_as_half((uint16_t)(e[i] >> 16))));
         };
         const int most = __reduce_max_sync(0xffffffffu, in_slab);
         for (int j = warp; j < most; j += kBatch * kDqWarps) batch(slab + 32, 32, j, in_slab);
@@ -234,87 +204,52 @@ __global__ void __launch_bounds__(kDqWarps * 32) decode_kernel(const DqArgs a) {
             for (int j = a.ell_slots + warp; j < n; j += kBatch * kDqWarps) batch(a.b.oent + p0, 1, j, n);
         }
     }
-    if (a.wait && (int)blockIdx.x == a.blocks - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <int N, int MODE, bool TILES>
-cudaError_t launch_decode(DqArgs a, int n_rb, int x_blocks, bool pdl, cudaStream_t s) {
+template <int N, int MODE>
+cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s) {
     using T = DqTab<N, MODE>;
     constexpr size_t kAlign = T::kBytes < 1024 ? 1024 : T::kBytes;
+    DqArgs a = {};
+    a.b = blob_at(packed, offsets_of(l));
+    a.out = W;
+    a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.GH = l.GH; a.L = l.L; a.ell_slots = l.ell_slots;
     const size_t lib = MODE == 1 && a.L * T::E <= kLibEntries ? (size_t)a.L * (T::E + 8) * 2 : 0;
-    const size_t smem = kAlign + T::kTables * kAlign + (TILES ? 0 : kDqWarps * 32 * kTileRow) + lib;
+    const size_t smem = kAlign + T::kTables * kAlign + kDqWarps * 32 * kTileRow + lib;
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        const cudaError_t e = cudaFuncSetAttribute(decode_kernel<N, MODE, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        const cudaError_t e = cudaFuncSetAttribute(dequant_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
     // few row-blocks: shorter ranges, at least one super-chunk per warp, until the blocks fill the GPU twice
     int range = a.SC < kDqRange ? a.SC : kDqRange;
-    while (range > kDqWarps && (long long)n_rb * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
+    while (range > kDqWarps && (long long)l.RB * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
     a.range = range;
-    a.blocks = n_rb * ((a.SC + range - 1) / range);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.blocks + x_blocks), 1, 1);
-    cfg.blockDim = dim3(kDqWarps * 32, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, decode_kernel<N, MODE, TILES>, a);
-}
-
-template <bool TILES>
-cudaError_t dispatch(const Layout& l, const DqArgs& a, int n_rb, int x_blocks, bool pdl, cudaStream_t s) {
-    if (l.mode == 0) {
-        switch (l.bits) {
-            case 2: return launch_decode<2, 0, TILES>(a, n_rb, x_blocks, pdl, s);
-            case 3: return launch_decode<3, 0, TILES>(a, n_rb, x_blocks, pdl, s);
-            case 4: return launch_decode<4, 0, TILES>(a, n_rb, x_blocks, pdl, s);
-            case 5: return launch_decode<5, 0, TILES>(a, n_rb, x_blocks, pdl, s);
-            default: return launch_decode<6, 0, TILES>(a, n_rb, x_blocks, pdl, s);
-        }
-    }
-    switch (l.bits) {
-        case 2: return launch_decode<2, 1, TILES>(a, n_rb, x_blocks, pdl, s);
-        case 3: return launch_decode<3, 1, TILES>(a, n_rb, x_blocks, pdl, s);
-        case 4: return launch_decode<4, 1, TILES>(a, n_rb, x_blocks, pdl, s);
-        case 5: return launch_decode<5, 1, TILES>(a, n_rb, x_blocks, pdl, s);
-        default: return launch_decode<6, 1, TILES>(a, n_rb, x_blocks, pdl, s);
-    }
-}
-
-DqArgs args_of(const Layout& l, const void* packed, uint16_t* out) {
-    DqArgs a = {};
-    a.b = blob_at(packed, offsets_of(l));
-    a.out = out;
-    a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.GH = l.GH; a.L = l.L; a.ell_slots = l.ell_slots;
-    return a;
+    dequant_kernel<N, MODE><<<(unsigned)(l.RB * ((a.SC + range - 1) / range)), kDqWarps * 32, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_dequant(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s) {
-    return dispatch<false>(l, args_of(l, packed, W), l.RB, 0, false, s);
-}
-
-// Row-blocks [rb0, rb0 + n_rb) as GEMM tiles; x_bf16 (may be null): x8 vectors of eight bf16 activations to convert.
-cudaError_t launch_decode_tiles(const Layout& l, const void* packed, int rb0, int n_rb, uint16_t* tiles, const void* x_bf16,
-                                void* x_f16, size_t x8, bool overlap, cudaStream_t s) {
-    DqArgs a = args_of(l, packed, tiles);
-    a.rb0 = rb0;
-    a.wait = overlap ? 1 : 0;
-    int x_blocks = 0;
-    if (x_bf16) {
-        a.x_bf16 = (const uint4*)x_bf16; a.x_f16 = (uint4*)x_f16; a.x8 = (unsigned)x8;
-        const size_t want = (x8 + kDqWarps * 32 - 1) / (kDqWarps * 32), cap = (size_t)sm_count() * 4;
-        x_blocks = (int)(want < cap ? want : cap);
+    if (l.mode == 0) {
+        switch (l.bits) {
+            case 2: return launch_decode<2, 0>(l, packed, W, s);
+            case 3: return launch_decode<3, 0>(l, packed, W, s);
+            case 4: return launch_decode<4, 0>(l, packed, W, s);
+            case 5: return launch_decode<5, 0>(l, packed, W, s);
+            default: return launch_decode<6, 0>(l, packed, W, s);
+        }
     }
-    return dispatch<true>(l, a, n_rb, x_blocks, overlap, s);
+    switch (l.bits) {
+        case 2: return launch_decode<2, 1>(l, packed, W, s);
+        case 3: return launch_decode<3, 1>(l, packed, W, s);
+        case 4: return launch_decode<4, 1>(l, packed, W, s);
+        case 5: return launch_decode<5, 1>(l, packed, W, s);
+        default: return launch_decode<6, 1>(l, packed, W, s);
+    }
 }
 
 }  // namespace xfp

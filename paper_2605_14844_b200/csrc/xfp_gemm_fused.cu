@@ -1,0 +1,843 @@
+// Prefill form of the fused decode kernel, Y = X (D + S)^T for many rows of x ("Fused Decode Kernel", steps (1)-(4): depack,
+// codebook gather, outlier scatter-add into the dequantised tile, GEMM on the tensor cores), on pairs of SMs.
+//
+//   pair     two CTAs (tcgen05 cta_group::2) share a tile of 256 channels x T rows of x, T up to 512: each decodes its own
+//            128 channels and stages half of the rows of x, the first CTA issues the products of both.  What bounds a GEMM
+//            on this layout is the path from L2 (about 9 TB/s, 32 bytes per clock and SM): decoded in place the weights cost
+//            N / 16 of an fp16 operand there, and sharing x in a pair halves the rest.  (Decoding into global tiles first
+//            and multiplying from there ran at those 9 TB/s: 4096 x 4096, 100 rows 26 us, 28672 x 8192, 1024 rows 640 us.)
+//   stage    64 k: A = W^ [128 channels][64 k] fp16 in core-matrix order (k / 8, channel, 8), 16 KB; B = the CTA's half of
+//            the rows of x in the 128-byte swizzle, by tensor copies.  2 .. 12 stages in a ring: a stage is in decode for
+//            about 1900 clocks (four of them at once), then 300 for its outliers, then in the products.
+//   warps    16 decode: a stage is decoded by four warps, one per row-block; 64 look-ups per lane, stored as eight 16-byte
+//            vectors.  4 outliers: for eight stages at a time the channels' lists are dealt to a list per stage; once a stage
+//            is decoded its list is added to the stored values, an entry per thread, one correctly rounded fp16 addition
+//            each (a lane walking its channel's list took 1500 clocks per 128 k at 0.9 %, and in the decode warps, where
+//            the addition has to find its register by nested tests, it cost as much as the decode).  1 copies, 1 products
+//            (in the second CTA: passes on that x has landed).  Roles meet at mbarriers only.
+//   K cut    few tiles: a cluster of 2, 3 or 4 pairs cuts the tile along K; the partial sums meet through distributed shared
+//            memory and are added in slice order.  Many tiles: resident pairs walk them.
+//   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
+//            table (D16 = fp16(fp32(scale * lib + mid))); the look-ups are then those of V2.
+// Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace, stops
+// issuing and leaves through the exit that frees its tensor memory.
+#include <cuda.h>
+
+#include "xfp_internal.h"
+#include "xfp_pair_common.cuh"
+
+namespace xfp {
+
+namespace {
+
+constexpr int kCh = 128;                       // channels of a CTA
+constexpr int kStageK = 64;
+constexpr int kABytes = kCh * kStageK * 2;     // A of one stage
+constexpr int kMaxSlots = 12;
+constexpr int kWindow = 8;                     // stages whose outliers are dealt to lists at a time
+constexpr int kListCap = 256;                  // entries of a stage's list (mean 8192 x rate); beyond it the channels' own lists are walked
+constexpr size_t kListBytes = (size_t)2 * kWindow * kListCap * 4;
+constexpr int kDecodeWarps = 16, kOutWarps = 4;
+constexpr int kCopyWarp = kDecodeWarps + kOutWarps, kMmaWarp = kCopyWarp + 1;
+constexpr int kThreads = (kMmaWarp + 1) * 32;
+constexpr uint32_t kSpins = 1u << 20, kPollHint = 1000;
+constexpr size_t kSmemMax = 226 * 1024;
+constexpr int kLibEntries = 8192;              // V2a library entries staged in shared memory
+constexpr int kMaxCut = 4;                     // pairs of a cluster
+
+struct FusedArgs {
+    Blob b;
+    void* y;
+    int* ctrl;                  // [0] error word
+    int rows, RB, SC, M, ell_slots, GH, L, y_kind;
+    int pairs, tok_tiles;       // tiles: 256 channels, T rows of x
+    int T, Tp, parts;           // T = parts * Tp, Tp <= 256: one product instruction covers Tp rows
+    int slots, x_bytes;         // stages in the ring; bytes of x per stage and CTA
+    int tab_bytes;
+    int ks, sc_slice;           // pairs along K, super-chunks of each
+    int tmem_cols;
+};
+
+__device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity) {
+    for (uint32_t i = 0; i < kSpins; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "r"(parity), "r"(kPollHint) : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+// One lane of a converged warp.  Instructions that take uniform registers are then issued by one thread as the compiler
+// sees it; behind a plain lane == 0 it serialises over the lanes it cannot rule out (a copy or a product took 70 - 250 clocks).
+__device__ __forceinline__ bool elected() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// the same address in the shared memory of CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t peer(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void arrive_local(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory"); }
+__device__ __forceinline__ void arrive_cluster(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(bar) : "memory"); }
+__device__ __forceinline__ void init_bar(const uint64_t* bar, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(sa(bar)), "r"(n)); }
+__device__ __forceinline__ uint32_t lds32(uint32_t a) { uint32_t v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; }
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+// lo | hi << 16 for words whose upper halves are zero, on the FMA pipe (the decode leans on the ALU pipe)
+__device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
+    return d;
+}
+// K-major operand descriptors (version 1).  A: core matrices of 8 rows x 16 bytes, the next 8 k 2048 bytes on, the next 8
+// rows 128 bytes on, no swizzle.  B: rows of 128 bytes in the 128-byte swizzle, 8 rows 1024 bytes.
+__device__ __forceinline__ uint64_t desc_a(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)(2048 >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+__device__ __forceinline__ uint64_t desc_b(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
+}
+// the products issued so far arrive on the barrier of both CTAs of the pair
+__device__ __forceinline__ void commit_pair(uint32_t bar, uint32_t mask) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(bar), "h"((uint16_t)mask) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void decode_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kDecodeWarps * 32) : "memory"); }
+__device__ __forceinline__ void outlier_sync() { asm volatile("bar.sync 2, %0;" :: "n"(kOutWarps * 32) : "memory"); }
+
+// Position in the ring after a number of stages: slot and the parity of its current use.
+struct Ring {
+    int slot;
+    uint32_t phase;
+    __device__ __forceinline__ void step(int n, int slots) {
+        slot += n;
+        while (slot >= slots) { slot -= slots; phase ^= 1u; }
+    }
+};
+
+// Decode tables.  kPair: entry t = first index | second index << N holds two fp16 values; else entry q one.  N = 4 entries lie
+// 256 bytes apart (two tables interleaved): an index isolated in its own byte becomes the second byte of the address.
+// V2: a table per row-block.  V2a: a table per warp.
+template <int N, int MODE>
+struct Tab {
+    static constexpr int E = 1 << N;
+    static constexpr bool kPair = MODE == 0 ? N <= 3 : N == 2;
+    static constexpr int kEntries = kPair ? E * E : E;
+    static constexpr int kStride = N == 4 ? 256 : 128;
+    static constexpr int kOne = N == 4 ? 4096 : (kEntries * 128 < 1024 ? 1024 : kEntries * 128);   // of one (N = 4: two) tables
+    static constexpr int kUnits = MODE == 0 ? 4 : kDecodeWarps;
+    static constexpr int kBytes = N == 4 ? kOne * kUnits / 2 : kOne * kUnits;
+    // address of table u's entry 0 for this lane
+    __device__ static __forceinline__ uint32_t at(uint32_t base, int u, int lane) {
+        return N == 4 ? base + (uint32_t)(u >> 1) * kOne + (uint32_t)(u & 1) * 128u + (uint32_t)lane * 4u
+                      : base + (uint32_t)u * kOne + (uint32_t)lane * 4u;
+    }
+};
+
+// The 16-byte vectors that hold words [PART * 2N, PART * 2N + 2N) of a lane's 128 * N-bit stream.
+template <int N, int PART>
+struct Half {
+    static constexpr int V0 = PART * 2 * N / 4, V1 = (PART * 2 * N + 2 * N + 3) / 4, NV = V1 - V0;
+};
+
+// V2: the codebooks of the CTA's four row-blocks into their tables (all decode warps).
+template <int N>
+__device__ __forceinline__ void fill_tables(const FusedArgs& a, uint32_t tab0, int rb0, int warp, int lane) {
+    using T = Tab<N, 0>;
+    constexpr int E = T::E;
+    const int q = warp & 3, sub = warp >> 2, rb = rb0 + q;
+    if (rb >= a.RB) return;
+    const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * E;      // padding rows exist in the blob
+    const uint32_t t = T::at(tab0, q, lane);
+    if (T::kPair) {
+        uint32_t v[E];
+#pragma unroll
+        for (int e = 0; e < E; e += 4) {
+            const uint2 p = __ldg((const uint2*)(cb + e));
+            v[e] = p.x & 0xffffu; v[e + 1] = p.x >> 16; v[e + 2] = p.y & 0xffffu; v[e + 3] = p.y >> 16;
+        }
+#pragma unroll
+        for (int hi = 0; hi < E; ++hi)
+            if ((hi & 3) == sub) {
+#pragma unroll
+                for (int lo = 0; lo < E; ++lo) sts32(t + (uint32_t)((lo | (hi << N)) * 128), __byte_perm(v[lo], v[hi], 0x5410));
+            }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E / 4; e += 4) {
+            const int e0 = sub * (E / 4) + e;
+            const uint2 p = __ldg((const uint2*)(cb + e0));
+            sts32(t + (uint32_t)(e0 * T::kStride), p.x & 0xffffu); sts32(t + (uint32_t)((e0 + 1) * T::kStride), p.x >> 16);
+            sts32(t + (uint32_t)((e0 + 2) * T::kStride), p.y & 0xffffu); sts32(t + (uint32_t)((e0 + 3) * T::kStride), p.y >> 16);
+        }
+    }
+}
+
+struct Bars {
+    uint32_t decoded, ready, landed, freed;       // address of slot 0's; slot s is 8 s further
+};
+
+// The decode warps' share of one tile: half PART of super-chunks grp, grp + 2, ... of [sc0, sc1): every fourth stage.
+template <int N, int MODE, int PART>
+__device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_ok, int q, int grp, int lane, int sc0, int sc1,
+                                            uint32_t tab, const uint16_t* slib, uint32_t sA, const Bars& bars, Ring ring) {
+    using T = Tab<N, MODE>;
+    using H = Half<N, PART>;
+    constexpr int E = T::E;
+    const uint32_t nib = ((tab >> 12) & 0xfu) * 0x10101010u;
+    const uint4* idx = a.b.idx + ((size_t)rb * a.SC + sc0 + grp) * N * 32 + lane;
+    const size_t meta0 = (((size_t)rb * a.SC + sc0 + grp) * a.GH + (a.GH - 1) * PART) * 32 + lane;
+    uint4 nx[H::NV];
+    uint32_t id_n = 0, sm_n = 0;
+    auto fetch = [&](int it) {                    // the vectors of this warp's super-chunk `it` steps of two ahead
+#pragma unroll
+        for (int v = 0; v < H::NV; ++v) nx[v] = ld_stream(idx + (size_t)it * 2 * N * 32 + (size_t)(H::V0 + v) * 32);
+        if (MODE == 1) {
+            const size_t m = meta0 + (size_t)it * 2 * a.GH * 32;
+            id_n = __ldg(a.b.gid + m); sm_n = __ldg(a.b.gsm + m);
+        }
+    };
+    if (rb_ok && sc0 + grp < sc1) fetch(0);
+    ring.step(2 * grp + PART, a.slots);
+    int it = 0;
+    for (int sc = sc0 + grp; sc < sc1; sc += 2, ++it) {
+        uint32_t w[4 * N + 1];
+        if (rb_ok) {
+#pragma unroll
+            for (int i = 0; i <= 4 * N; ++i) w[i] = 0u;
+#pragma unroll
+            for (int v = 0; v < H::NV; ++v) {
+                w[4 * (H::V0 + v)] = nx[v].x; w[4 * (H::V0 + v) + 1] = nx[v].y;
+                w[4 * (H::V0 + v) + 2] = nx[v].z; w[4 * (H::V0 + v) + 3] = nx[v].w;
+            }
+            const uint32_t id = id_n, sm = sm_n;
+            if (sc + 2 < sc1) fetch(it + 1);
+            if (MODE == 1) {
+                const float scale = h2f((uint16_t)(sm & 0xffffu)), mid = h2f((uint16_t)(sm >> 16));
+                auto decoded = [&](uint32_t l) { return (uint32_t)f2h(__fmaf_rn(scale, h2f((uint16_t)l), mid)); };
+                if (N == 2) {
+                    const uint2 l4 = slib ? *(const uint2*)(slib + id * (E + 8)) : __ldg((const uint2*)(a.b.cb + (size_t)id * E));
+                    const uint32_t d[4] = {decoded(l4.x & 0xffffu), decoded(l4.x >> 16), decoded(l4.y & 0xffffu), decoded(l4.y >> 16)};
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) sts32(tab + t * 128, join16(d[t & 3], d[t >> 2]));
+                } else {
+#pragma unroll
+                    for (int e = 0; e < E; e += 8) {
+                        const uint4 l8 = slib ? *(const uint4*)(slib + id * (E + 8) + e) : __ldg((const uint4*)(a.b.cb + (size_t)id * E + e));
+                        const uint32_t lw[4] = {l8.x, l8.y, l8.z, l8.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            sts32(tab + (e + 2 * i) * T::kStride, decoded(lw[i] & 0xffffu));
+                            sts32(tab + (e + 2 * i + 1) * T::kStride, decoded(lw[i] >> 16));
+                        }
+                    }
+                }
+            }
+        }
+        // the slot's previous use: its products are done
+        if (!wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u)) return false;
+        if (rb_ok) {
+            const uint32_t dst = sA + (uint32_t)ring.slot * kABytes + (uint32_t)(q * 32 + lane) * 16u;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                uint32_t d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int p = PART * 32 + c * 4 + i;
+                    if (T::kPair) {
+                        d[i] = lds32(pair_addr<N, 1>(w, p, tab));
+                    } else if (N == 4) {
+                        const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
+                        const uint32_t sel = 0x7604u | ((uint32_t)(p & 3) << 4);   // [tab.b3, tab.b2, index byte, tab.b0]
+                        d[i] = join16(lds32(__byte_perm(wlo, tab, sel)), lds32(__byte_perm(whi, tab, sel)));
+                    } else {
+                        d[i] = join16(lds32(single_addr<N, 1>(w, 2 * p, tab)), lds32(single_addr<N, 1>(w, 2 * p + 1, tab)));
+                    }
+                }
+                sts128(dst + (uint32_t)c * 2048u, d[0], d[1], d[2], d[3]);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the products read through the async proxy
+        __syncwarp();
+        if (elected()) arrive_local(bars.decoded + 8u * ring.slot);
+        ring.step(4, a.slots);
+    }
+    return true;
+}
+
+// A channel's outliers in ascending column order: transposed slab first, the CSR arrays behind it.
+struct Outliers {
+    const uint32_t* slab;
+    const uint32_t* spill;
+    int nslab, total;
+    __device__ __forceinline__ uint32_t at(int j) const { return __ldg(j < nslab ? slab + (size_t)(1 + j) * 32 : spill + j); }
+    __device__ __forceinline__ void open(const FusedArgs& a, int rb, int row, int lane) {
+        slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
+        spill = a.b.oent;
+        nslab = total = 0;
+        if (rb < a.RB && row < a.rows) {
+            const int len = (int)__ldg(slab);
+            nslab = total = min(len, a.ell_slots);
+            if (len >= a.ell_slots) {
+                const int p0 = __ldg(a.b.rowptr + row);
+                total = __ldg(a.b.rowptr + row + 1) - p0;
+                spill = a.b.oent + p0;
+            }
+        }
+    }
+    // first entry at or behind column k0: sixteen independent loads at a time (every 16th entry, then the 15 in front of the hit)
+    __device__ __forceinline__ int find(uint32_t k0) const {
+        if (!k0 || !total) return 0;
+        int coarse = 0, fine = 0;
+        for (int j = 15; j < total; j += 16) coarse += (at(j) & 0xffffu) < k0;
+#pragma unroll
+        for (int j = 0; j < 15; ++j) fine += coarse * 16 + j < total && (at(min(coarse * 16 + j, total - 1)) & 0xffffu) < k0;
+        return coarse * 16 + fine;
+    }
+};
+
+// W^ = fp16(D16 + S) at weight k (0 .. 63) of channel ch of a stage
+__device__ __forceinline__ void add_outlier(unsigned char* stage, uint32_t k, uint32_t ch, uint16_t val) {
+    uint16_t* w = (uint16_t*)(stage + (k >> 3) * 2048u + ch * 16u + (k & 7u) * 2u);
+    *w = __half_as_ushort(__hadd(__ushort_as_half(*w), __ushort_as_half(val)));
+}
+
+// The outlier warps' share of one tile.  list[2][kWindow][kListCap]: k | channel << 6 | value << 16; cnt[2][kWindow].
+// `ready0`: the first CTA's "ready" barrier of slot 0.
+__device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int lane, int q, int st0, int st1, unsigned char* pA,
+                                             uint32_t* list, int* cnt, const Bars& bars, uint32_t ready0, Ring ring, bool ok) {
+    constexpr int kBatch = 8;
+    const int ch = q * 32 + lane;
+    const bool any = a.ell_slots != 0;
+    Outliers o;
+    int cur = 0, start = 0;                     // next entry to deal; first entry of the window being added
+    uint32_t e[kBatch];
+    auto load = [&]() {
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) e[i] = cur + i < o.total ? o.at(cur + i) : 0u;
+    };
+    // deal the entries of window [w0, w0 + kWindow) to its lists
+    auto deal = [&](int w0, int buf) {
+        const uint32_t end = (uint32_t)min(w0 + kWindow, st1) * kStageK;
+        for (;;) {
+            int n = 0;
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                const uint32_t col = e[i] & 0xffffu;
+                if (cur + i < o.total && col < end) {
+                    const int st = (int)(col >> 6) - w0, at = atomicAdd(&cnt[buf * kWindow + st], 1);
+                    if (at < kListCap) list[(buf * kWindow + st) * kListCap + at] = (col & 63u) | (uint32_t)ch << 6 | (e[i] & 0xffff0000u);
+                    ++n;
+                }
+            }
+            cur += n;
+            if (n) load();
+            if (n < kBatch) break;
+        }
+    };
+    if (any) {
+        o.open(a, rb, rb * kRowsPerBlock + lane, lane);
+        cur = start = o.find((uint32_t)st0 * kStageK);
+        load();
+        outlier_sync();                         // the lists' last use, in the previous tile, is over
+        if (ch < 2 * kWindow) cnt[ch] = 0;
+        outlier_sync();
+        deal(st0, 0);
+    }
+    for (int w0 = st0, buf = 0; w0 < st1; w0 += kWindow, buf ^= 1) {
+        const int next = cur;
+        if (any) {
+            outlier_sync();                     // the window's lists are complete, the other buffer is idle
+            if (ch < kWindow) cnt[(buf ^ 1) * kWindow + ch] = 0;
+            outlier_sync();
+        }
+        for (int st = w0; st < w0 + kWindow; ++st) {
+            if (any && st == w0 + kWindow / 2) deal(w0 + kWindow, buf ^ 1);
+            if (st >= st1) continue;
+            ok = ok && wait_bar(bars.decoded + 8u * ring.slot, ring.phase);
+            if (!ok) { ring.step(1, a.slots); continue; }         // this warp still meets the others at their barrier
+            if (any) {
+                unsigned char* stage = pA + (size_t)ring.slot * kABytes;
+                const int n = cnt[buf * kWindow + st - w0];
+                if (n <= kListCap) {
+                    const uint32_t* l = list + (buf * kWindow + st - w0) * kListCap;
+                    for (int i = ch; i < n; i += kOutWarps * 32) add_outlier(stage, l[i] & 63u, (l[i] >> 6) & 127u, (uint16_t)(l[i] >> 16));
+                } else {                        // more than the list holds: the channel's own entries
+                    for (int j = start; j < next; ++j) {
+                        const uint32_t v = o.at(j);
+                        if ((int)((v & 0xffffu) >> 6) == st) add_outlier(stage, v & 63u, (uint32_t)ch, (uint16_t)(v >> 16));
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            __syncwarp();
+            if (elected()) arrive_cluster(ready0 + 8u * ring.slot);
+            ring.step(1, a.slots);
+        }
+        start = next;
+    }
+    return ok;
+}
+
+// SPLIT: a cluster of a.ks pairs per tile, one tile per cluster; else resident pairs walk the tiles.
+template <int N, int MODE, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
+    using T = Tab<N, MODE>;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    // tables aligned to 8 KB of the shared window, so that an entry's offset is merged with the address, not added
+    unsigned char* smem = smem_raw + ((8192u - (sa(smem_raw) & 8191u)) & 8191u);      // the same offset in every CTA
+    __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_landed[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail, s_cnt[2 * kWindow];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t crank = cluster_rank(), h = crank & 1u, lead = crank & ~1u;        // half of the pair, its first CTA
+    const int slice = (int)(crank >> 1);
+    const int first = SPLIT ? (int)blockIdx.x / (2 * a.ks) : (int)blockIdx.x >> 1, step = SPLIT ? 1 << 28 : (int)gridDim.x >> 1;
+    const int tiles = a.pairs * a.tok_tiles;
+    const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), st0 = 2 * sc0, st1 = 2 * sc1, nst = st1 - st0;
+    unsigned char* pA = smem + a.tab_bytes;
+    unsigned char* pB = pA + (size_t)a.slots * kABytes;
+    uint32_t* list = (uint32_t*)(pB + (size_t)a.slots * a.x_bytes);                  // the outlier warps' lists (with outliers)
+    uint16_t* lib = (uint16_t*)((unsigned char*)list + (a.ell_slots ? kListBytes : 0));
+    const Bars bars{sa(b_decoded), sa(b_ready), sa(b_landed), sa(b_freed)};
+    asm volatile("griddepcontrol.launch_dependents;");
+
+    if (tid == 0) {
+        for (int i = 0; i < a.slots; ++i) {
+            init_bar(&b_decoded[i], 4);                       // a warp per row-block
+            init_bar(&b_ready[i], 2 * kOutWarps + 1);         // outlier warps of both CTAs, x of the second (in the first CTA)
+            init_bar(&b_landed[i], 1);
+            init_bar(&b_freed[i], 1);
+        }
+        init_bar(&acc_full, 1);
+        init_bar(&acc_empty, 2 * kDecodeWarps);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const bool staged = MODE == 1 && a.L * T::E <= kLibEntries;
+    if (staged)
+        for (int i = tid; i < a.L * T::E; i += kThreads) lib[(i / T::E) * (T::E + 8) + i % T::E] = __ldg(a.b.cb + i);
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(sa(&s_tmem)), "r"(a.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    // Nothing remote happens before the wait that belongs to this arrival: the decode warps begin at once and wait in front of
+    // their first epilogue, the others before they start.
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    auto cluster_wait = [] {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+
+    bool ok = true;
+    Ring ring{0, 0u};
+    uint32_t acc_ph = 0;
+    if (warp < kDecodeWarps) {
+        const int q = warp & 3, part = (warp >> 2) & 1, grp = warp >> 3;
+        const uint32_t tab = T::at(sa(smem), MODE == 0 ? q : warp, lane);
+        int have = -1;                                        // tile of channels whose tables are in place
+        for (int t = first; t < tiles; t += step) {           // a warp whose wait ran out still meets the others at their barrier
+            const int tx = t / a.tok_tiles, ty = t % a.tok_tiles, t0 = ty * a.T;
+            const int rb = (2 * tx + (int)h) * 4 + q;
+            if (MODE == 0 && tx != have) {
+                decode_sync();                                // every warp is done with the previous tables
+                fill_tables<N>(a, sa(smem), rb - q, warp, lane);
+                decode_sync();
+                have = tx;
+            }
+            const uint16_t* slib = staged ? lib : nullptr;
+            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, sc0, sc1, tab, slib, sa(pA), bars, ring)
+                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, sc0, sc1, tab, slib, sa(pA), bars, ring));
+            ring.step(nst, a.slots);
+            if (t == first) cluster_wait();
+            ok = ok && wait_bar(sa(&acc_full), acc_ph);
+            acc_ph ^= 1u;
+            if (!ok) continue;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t tmem = s_tmem;
+            const int r = q * 32 + lane, row = (2 * tx + (int)h) * kCh + r;
+            const int tend = min(a.T, a.M - t0);
+            for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
+                uint32_t v[16];
+                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), v);
+                if (SPLIT) {
+                    // every product of the pair is complete, its slots are idle: the partial sums go there, [t][channel]
+                    float* p = (float*)pA + (size_t)c * 16 * kCh + r;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) p[(size_t)j * kCh] = __uint_as_float(v[j]);
+                } else if (row < a.rows) {
+                    const int n = min(16, tend - c * 16);
+                    const size_t o = (size_t)(t0 + c * 16) * a.rows + row;
+                    if (a.y_kind == 1) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = f2h(__uint_as_float(v[j]));
+                    } else if (a.y_kind == 2) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[j])));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < n) ((float*)a.y)[o + (size_t)j * a.rows] = __uint_as_float(v[j]);
+                    }
+                }
+            }
+            if (!SPLIT) {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (elected()) arrive_cluster(peer(sa(&acc_empty), lead));
+            }
+        }
+    } else if (warp < kCopyWarp) {
+        const int q = warp - kDecodeWarps;
+        const uint32_t ready0 = peer(bars.ready, lead);
+        cluster_wait();
+        for (int t = first; t < tiles; t += step) {
+            const int tx = t / a.tok_tiles, rb = (2 * tx + (int)h) * 4 + q;
+            ok = outlier_tile(a, rb, lane, q, st0, st1, pA, list, s_cnt, bars, ready0, ring, ok);
+            ring.step(nst, a.slots);
+        }
+    } else if (warp == kCopyWarp) {
+        cluster_wait();
+        asm volatile("griddepcontrol.wait;" ::: "memory");    // x may come from the previous kernel of the stream
+        for (int t = first; t < tiles && ok; t += step) {
+            const int t0 = (t % a.tok_tiles) * a.T;
+            for (int st = st0; st < st1; ++st) {
+                if (!(ok = wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u))) break;
+                if (elected()) {
+                    const uint32_t bar = bars.landed + 8u * ring.slot;
+                    uint32_t dst = sa(pB) + (uint32_t)(ring.slot * a.x_bytes);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"((uint32_t)a.x_bytes) : "memory");
+                    for (int p = 0; p < a.parts; ++p, dst += (uint32_t)a.Tp * 64u) {
+                        // this CTA's half of the part's rows (of those that exist, rounded up to 16; more may be copied along)
+                        const int p0 = t0 + p * a.Tp, n = min(a.Tp, max((a.M - p0 + 15) & ~15, 16)), xrow = p0 + (int)h * (n >> 1);
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                     :: "r"(dst), "l"(&tmap), "r"(st * kStageK), "r"(xrow), "r"(bar) : "memory");
+                    }
+                }
+                __syncwarp();
+                ring.step(1, a.slots);
+            }
+        }
+    } else if (h == 1) {                                      // the second CTA: tell the first that x has landed here
+        const uint32_t ready0 = peer(bars.ready, lead);
+        cluster_wait();
+        for (int t = first; t < tiles && ok; t += step) {
+            for (int st = st0; st < st1; ++st) {
+                if (!(ok = wait_bar(bars.landed + 8u * ring.slot, ring.phase))) break;
+                if (elected()) arrive_cluster(ready0 + 8u * ring.slot);
+                __syncwarp();
+                ring.step(1, a.slots);
+            }
+        }
+    } else {
+        const uint64_t da0 = desc_a(sa(pA)), db0 = desc_b(sa(pB));
+        const uint32_t mask = 3u << lead;
+        cluster_wait();
+        const uint32_t tmem = s_tmem;
+        for (int t = first; t < tiles && ok; t += step) {
+            const int t0 = (t % a.tok_tiles) * a.T;
+            if (t != first) {
+                ok = wait_bar(sa(&acc_empty), acc_ph);        // the previous tile's sums have been read
+                acc_ph ^= 1u;
+                if (!ok) break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int st = st0; st < st1; ++st) {
+                if (!(ok = wait_bar(bars.landed + 8u * ring.slot, ring.phase) && wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (elected()) {
+                    const uint64_t da = da0 + (uint64_t)((uint32_t)ring.slot * (kABytes >> 4));
+                    uint64_t db = db0 + (uint64_t)((uint32_t)(ring.slot * a.x_bytes) >> 4);
+                    for (int p = 0; p < a.parts; ++p, db += (uint64_t)(a.Tp * 4)) {
+                        const int p0 = t0 + p * a.Tp;
+                        if (p0 >= a.M) break;
+                        const int n = min(a.Tp, (a.M - p0 + 15) & ~15);
+                        const uint32_t idesc = (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * kCh >> 4) << 24);
+#pragma unroll
+                        for (int i = 0; i < kStageK / 16; ++i)
+                            mma_pair(tmem + (uint32_t)(p * a.Tp), da + i * 256, db + i * 2, idesc, (st > st0 || i > 0) ? 1u : 0u);
+                    }
+                    commit_pair(bars.freed + 8u * ring.slot, mask);
+                    if (st + 1 == st1) commit_pair(sa(&acc_full), mask);
+                }
+                __syncwarp();
+                ring.step(1, a.slots);
+            }
+        }
+    }
+    if (!ok) { s_fail = 1; atomicExch(a.ctrl, 1); }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (s_fail && tid == 0)      // copies in flight land before the CTA goes
+        for (int i = 0; i < a.slots; ++i) wait_bar(bars.landed + 8u * i, 0);
+    __syncwarp();
+    cluster_sync();
+    if (SPLIT) {
+        // this CTA's share of the rows of x of its 128 channels: the slices' sums added in slice order
+        if (first < tiles) {
+            const int tx = first / a.tok_tiles, t0 = (first % a.tok_tiles) * a.T, Tn = min(a.T, a.M - t0);
+            const int share = (Tn + a.ks - 1) / a.ks, b0 = slice * share, b1 = min(Tn, b0 + share);
+            const uint32_t own = sa(pA);
+            const bool wide = (a.rows & 3) == 0;               // four channels in one store
+            for (int i0 = b0 * (kCh / 4) + tid; i0 < b1 * (kCh / 4); i0 += 2 * kThreads) {
+                float4 v[2][kMaxCut];                         // two places, every slice's share in flight
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int z = 0; z < kMaxCut; ++z) {
+                        const int i = i0 + u * kThreads;
+                        v[u][z] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (z < a.ks && i < b1 * (kCh / 4))
+                            asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[u][z].x), "=f"(v[u][z].y), "=f"(v[u][z].z), "=f"(v[u][z].w)
+                                         : "r"(peer(own + (uint32_t)i * 16u, 2u * (uint32_t)z + h)));
+                    }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + u * kThreads;
+                    if (i >= b1 * (kCh / 4)) break;
+                    float4 sum = v[u][0];
+#pragma unroll
+                    for (int z = 1; z < kMaxCut; ++z)
+                        if (z < a.ks) { sum.x += v[u][z].x; sum.y += v[u][z].y; sum.z += v[u][z].z; sum.w += v[u][z].w; }
+                    const int tt = t0 + i / (kCh / 4), row = (2 * tx + (int)h) * kCh + (i % (kCh / 4)) * 4;
+                    const size_t o = (size_t)tt * a.rows + row;
+                    if (wide && row < a.rows) {
+                        if (a.y_kind == 0) *(float4*)((float*)a.y + o) = sum;
+                        else if (a.y_kind == 1) {
+                            const __half2 lo = __floats2half2_rn(sum.x, sum.y), hi = __floats2half2_rn(sum.z, sum.w);
+                            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
+                        } else {
+                            const __nv_bfloat162 lo = __floats2bfloat162_rn(sum.x, sum.y), hi = __floats2bfloat162_rn(sum.z, sum.w);
+                            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
+                        }
+                    } else {
+                        if (row < a.rows) put_y(a.y, o, sum.x, a.y_kind);
+                        if (row + 1 < a.rows) put_y(a.y, o + 1, sum.y, a.y_kind);
+                        if (row + 2 < a.rows) put_y(a.y, o + 2, sum.z, a.y_kind);
+                        if (row + 3 < a.rows) put_y(a.y, o + 3, sum.w, a.y_kind);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        cluster_sync();          // no CTA leaves while another reads its shared memory
+    }
+    if (warp == kMmaWarp)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(s_tmem), "r"(a.tmem_cols) : "memory");
+}
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_fn() {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+        return nullptr;
+    return (EncodeTiledFn)fn;
+}
+
+// Clusters of 2 * ks CTAs of this kernel that the current device runs at once (a cluster stays inside a GPC, so the larger
+// ones leave SMs idle), asked once per device.
+int clusters_at_once(int ks) {
+    static std::atomic<int> cache[256][kMaxCut + 1] = {};
+    std::atomic<int>& slot = cache[DeviceOnce::current()][ks];
+    int n = slot.load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(2 * ks), 1, 1);
+        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.dynamicSmemBytes = kSmemMax;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)(2 * ks); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(gemm_fused_kernel<4, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, gemm_fused_kernel<4, 0, true>, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            n = sm_count() / (2 * ks) > 0 ? sm_count() / (2 * ks) : 1;
+        }
+        slot.store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+// ------------------------------------------------------------------ plan
+
+struct FusedPlan {
+    int T, Tp, parts, tok_tiles, pairs, ks, sc_slice, slots;
+    size_t tab, lib, smem;
+    double clocks;             // what the model expects
+};
+
+// Clocks of a tile's super-chunk: the products (4 T), the decode of 128 x 128 weights, or the operands' way from L2 (the
+// index stream and the CTA's half of x at about 40 bytes per clock).
+double slot_clocks(const Layout& l, int T) {
+    const double products = 4.0 * T, decode = l.mode ? (l.bits >= 5 ? 1700.0 : 1250.0) : (l.bits >= 5 ? 1200.0 : 1000.0);
+    const double feed = (l.bits * 2048.0 + 128.0 * T) / 40.0;
+    const double m = products > decode ? products : decode;
+    return m > feed ? m : feed;
+}
+
+size_t table_bytes(const Layout& l) {
+    const size_t one = l.mode == 0 ? (l.bits <= 3 ? l.E * l.E : l.E) : (l.bits == 2 ? 16 : l.E);
+    const size_t units = l.mode == 0 ? 4 : kDecodeWarps;
+    if (l.bits == 4) return 4096 * units / 2;
+    return (one * 128 < 1024 ? 1024 : one * 128) * units;
+}
+
+FusedPlan plan_fused(const Layout& l, int M) {
+    FusedPlan best = {};
+    const size_t tab = (table_bytes(l) + 1023) & ~size_t(1023);
+    const size_t lib = l.mode && (size_t)l.L * l.E <= kLibEntries ? ((size_t)l.L * (l.E + 8) * 2 + 15) & ~size_t(15) : 0;
+    const size_t lists = l.ell_slots ? kListBytes : 0;
+    const int pairs = (l.RB + 7) / 8;
+    int last_T = 0;
+    for (int n = (M + 511) / 512; n <= (M + 15) / 16; ++n) {          // tiles along the rows of x
+        const int t = (M + n - 1) / n, parts = t > 256 ? 2 : 1, Tp = ((t + parts - 1) / parts + 15) & ~15, T = parts * Tp;
+        if (T == last_T || T > 512) continue;
+        last_T = T;
+        if (T < 64 && best.clocks > 0.0) break;
+        const int tok = (M + T - 1) / T;
+        int slots = (int)((kSmemMax - 8192 - tab - lib - lists) / (kABytes + (size_t)T * 64));
+        if (slots > kMaxSlots) slots = kMaxSlots;
+        if (slots < 2) continue;
+        for (int ks = 1; ks <= kMaxCut; ++ks) {
+            const int spp = (l.SC + ks - 1) / ks;
+            if (ks > 1 && ((ks - 1) * spp >= l.SC || spp < 2 || (size_t)T * kCh * 4 > slots * (kABytes + (size_t)T * 64))) break;
+            const int at_once = clusters_at_once(ks);
+            const int tiles = pairs * tok, waves = (tiles + at_once - 1) / at_once;
+            // a stage's way through decode, outliers and products takes about 2900 clocks and its share of the products
+            const double chain = (2900.0 + 2.0 * T) / slots * 2.0, busy = slot_clocks(l, T);
+            const double clocks = waves * (spp * (busy > chain ? busy : chain) + 1500.0 + 10.0 * T + (ks > 1 ? 1500.0 + 8.0 * T : 0.0));
+            if (best.clocks == 0.0 || clocks < best.clocks) {
+                best.T = T; best.Tp = Tp; best.parts = parts; best.tok_tiles = tok; best.pairs = pairs; best.ks = ks;
+                best.sc_slice = spp; best.slots = slots; best.clocks = clocks;
+            }
+        }
+    }
+    best.tab = tab; best.lib = lib;
+    best.smem = 8192 + tab + lib + lists + (size_t)best.slots * (kABytes + (size_t)best.T * 64);
+    return best;
+}
+
+template <int N, int MODE>
+cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
+    const FusedPlan p = plan_fused(l, c.M);
+    static const EncodeTiledFn encode = encode_fn();
+    if (!encode || !p.slots) return cudaErrorNotSupported;
+    CUtensorMap tmap;
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)l.cols, (cuuint64_t)c.M};
+        const cuuint64_t strides[1] = {(cuuint64_t)l.cols * 2};
+        const cuuint32_t box[2] = {64, (cuuint32_t)(p.Tp / 2)};
+        const cuuint32_t estr[2] = {1, 1};
+        if (encode(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<uint16_t*>(c.x), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    static DeviceOnce attr_done;
+    const int dev = DeviceOnce::current();
+    if (!attr_done.is_set(dev)) {
+        cudaError_t e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        if (e != cudaSuccess) return e;
+        attr_done.set(dev);
+    }
+    FusedArgs a = {};
+    a.b = blob_at(c.packed, offsets_of(l));
+    a.y = c.y; a.ctrl = (int*)c.workspace;
+    a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L; a.y_kind = c.y_kind;
+    a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
+    a.slots = p.slots; a.x_bytes = p.T * 64; a.tab_bytes = (int)p.tab;
+    a.ks = p.ks; a.sc_slice = p.sc_slice;
+    a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
+    const int tiles = p.pairs * p.tok_tiles, pair_slots = clusters_at_once(1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.ks > 1 ? tiles * 2 * p.ks : 2 * (tiles < pair_slots ? tiles : pair_slots)), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)(2 * p.ks); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return p.ks > 1 ? cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, true>, a, tmap)
+                    : cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, false>, a, tmap);
+}
+
+}  // namespace
+
+bool fused_preferred(const Layout& l, int M) {
+#ifdef LANE_TUNE
+    if (const char* e = getenv("XFP_FUSED")) return M >= atoi(e) && gemm_tc_supported(l, M);
+#endif
+    return M > 64 && gemm_tc_supported(l, M);
+}
+size_t fused_workspace_bytes(const Layout& l, int M) { return gemm_ctrl_bytes(l, M); }
+
+// c.x: the activations as fp16; or bf16, converted first into x_f16
+cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& call, void* x_f16, cudaStream_t s) {
+    GemmCall c = call;
+    if (x_f16) {
+        const cudaError_t e = launch_x_to_f16(c.x, x_f16, (size_t)c.M * l.cols, s);
+        if (e != cudaSuccess) return e;
+        c.x = (const uint16_t*)x_f16;
+    }
+    if (l.mode == 1) {
+        switch (l.bits) {
+            case 2: return launch_n<2, 1>(l, c, s);
+            case 3: return launch_n<3, 1>(l, c, s);
+            case 4: return launch_n<4, 1>(l, c, s);
+            case 5: return launch_n<5, 1>(l, c, s);
+            default: return launch_n<6, 1>(l, c, s);
+        }
+    }
+    switch (l.bits) {
+        case 2: return launch_n<2, 0>(l, c, s);
+        case 3: return launch_n<3, 0>(l, c, s);
+        case 4: return launch_n<4, 0>(l, c, s);
+        case 5: return launch_n<5, 0>(l, c, s);
+        default: return launch_n<6, 0>(l, c, s);
+    }
+}
+
+}  // namespace xfp

@@ -891,6 +891,8 @@ size_t gemm_workspace_bytes(const Layout& l, int M) {
 namespace {
 // bf16 rows of x -> fp16 (round to nearest even, clamped to the finite fp16 range), eight values per thread and step
 __global__ void x_to_f16_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n8) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x)
         dst[i] = x8_as_f16(__ldg(src + i), 1);
 }
@@ -902,8 +904,16 @@ cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaS
     const size_t n8 = elems / 8;     // cols is a multiple of 128
     const size_t cap = (size_t)sm_count() * 8;
     const unsigned grid = (unsigned)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap);
-    x_to_f16_kernel<<<grid ? grid : 1, 256, 0, s>>>((const uint4*)x_bf16, (uint4*)x_f16, n8);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid ? grid : 1, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, x_to_f16_kernel, (const uint4*)x_bf16, (uint4*)x_f16, n8);
 }
 
 cudaError_t launch_gemm_tc(const Layout& l, const GemmCall& c, cudaStream_t s) {

@@ -116,15 +116,12 @@ cudaError_t launch_gemm_tc(const Layout& l, const GemmCall& c, cudaStream_t s);
 size_t gemm_x_scratch_bytes(const Layout& l, int M);
 cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaStream_t s);
 
-// The prefill form in two steps: the weights decoded once into GEMM tiles in the workspace (xfp_dequant.cu), then a dense
-// tcgen05 GEMM (xfp_gemm_dense.cu).
-cudaError_t launch_decode_tiles(const Layout& l, const void* packed, int rb0, int n_rb, uint16_t* tiles, const void* x_bf16,
-                                void* x_f16, size_t x8, bool overlap, cudaStream_t s);
-bool dense_preferred(const Layout& l, int M);          // which of the two forms xfp_gemm takes
-size_t dense_workspace_bytes(const Layout& l, int M);
-cudaError_t launch_gemm_dense(const Layout& l, const GemmCall& c, void* x_f16, cudaStream_t s);
+// The prefill form for many rows of x on pairs of SMs; see xfp_gemm_fused.cu.
+bool fused_preferred(const Layout& l, int M);          // which of the two kernels xfp_gemm takes
+size_t fused_workspace_bytes(const Layout& l, int M);
+cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& c, void* x_f16, cudaStream_t s);
 inline size_t prefill_workspace_bytes(const Layout& l, int M) {
-    return dense_preferred(l, M) ? dense_workspace_bytes(l, M) : gemm_workspace_bytes(l, M);
+    return fused_preferred(l, M) ? fused_workspace_bytes(l, M) : gemm_workspace_bytes(l, M);
 }
 
 // Batches of 9..16 rows of x run on the tensor-core kernel (xfp_gemm_tc.cu) when the matrix is large and the blob
