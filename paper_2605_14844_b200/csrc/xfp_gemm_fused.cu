@@ -8,13 +8,13 @@
 //            and multiplying from there ran at those 9 TB/s: 4096 x 4096, 100 rows 26 us, 28672 x 8192, 1024 rows 640 us.)
 //   stage    64 k: A = W^ [128 channels][64 k] fp16 in core-matrix order (k / 8, channel, 8), 16 KB; B = the CTA's half of
 //            the rows of x in the 128-byte swizzle, by tensor copies.  2 .. 12 stages in a ring: a stage is in decode for
-//            about 1900 clocks (four of them at once), then 300 for its outliers, then in the products.
+//            about 1900 clocks (four of them at once), then 200 for its outliers, then in the products.
 //   warps    16 decode: a stage is decoded by four warps, one per row-block; 64 look-ups per lane, stored as eight 16-byte
-//            vectors.  4 outliers: for eight stages at a time the channels' lists are dealt to a list per stage; once a stage
-//            is decoded its list is added to the stored values, an entry per thread, one correctly rounded fp16 addition
-//            each (a lane walking its channel's list took 1500 clocks per 128 k at 0.9 %, and in the decode warps, where
-//            the addition has to find its register by nested tests, it cost as much as the decode).  1 copies, 1 products
-//            (in the second CTA: passes on that x has landed).  Roles meet at mbarriers only.
+//            vectors.  4 outliers: a lane per channel with the next four entries of its list in registers adds those that
+//            fall into the stage to the stored values, one correctly rounded fp16 addition each, by address (in the decode
+//            warps, where the addition has to find its register by nested tests, it cost as much as the decode).  1 copies,
+//            1 products.  Roles meet at mbarriers only: a stage is "ready" on the first CTA's barrier when the last of both
+//            CTAs' row-blocks are stored and both CTAs' x has landed (the copies of both count their bytes there).
 //   K cut    few tiles: a cluster of 2, 3 or 4 pairs cuts the tile along K; the partial sums meet through distributed shared
 //            memory and are added in slice order.  Many tiles: resident pairs walk them.
 //   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
@@ -34,9 +34,6 @@ constexpr int kCh = 128;                       // channels of a CTA
 constexpr int kStageK = 64;
 constexpr int kABytes = kCh * kStageK * 2;     // A of one stage
 constexpr int kMaxSlots = 12;
-constexpr int kWindow = 8;                     // stages whose outliers are dealt to lists at a time
-constexpr int kListCap = 256;                  // entries of a stage's list (mean 8192 x rate); beyond it the channels' own lists are walked
-constexpr size_t kListBytes = (size_t)2 * kWindow * kListCap * 4;
 constexpr int kDecodeWarps = 16, kOutWarps = 4;
 constexpr int kCopyWarp = kDecodeWarps + kOutWarps, kMmaWarp = kCopyWarp + 1;
 constexpr int kThreads = (kMmaWarp + 1) * 32;
@@ -59,6 +56,15 @@ struct FusedArgs {
 };
 
 __device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool test_bar(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity) {
     for (uint32_t i = 0; i < kSpins; ++i) {
         uint32_t ok;
@@ -131,7 +137,6 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void decode_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kDecodeWarps * 32) : "memory"); }
-__device__ __forceinline__ void outlier_sync() { asm volatile("bar.sync 2, %0;" :: "n"(kOutWarps * 32) : "memory"); }
 
 // Position in the ring after a number of stages: slot and the parity of its current use.
 struct Ring {
@@ -202,7 +207,8 @@ __device__ __forceinline__ void fill_tables(const FusedArgs& a, uint32_t tab0, i
 }
 
 struct Bars {
-    uint32_t decoded, ready, landed, freed;       // address of slot 0's; slot s is 8 s further
+    uint32_t decoded, freed;      // address of slot 0's; slot s is 8 s further
+    uint32_t ready;               // of the first CTA of the pair
 };
 
 // The decode warps' share of one tile: half PART of super-chunks grp, grp + 2, ... of [sc0, sc1): every fourth stage.
@@ -287,7 +293,10 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the products read through the async proxy
         __syncwarp();
-        if (elected()) arrive_local(bars.decoded + 8u * ring.slot);
+        if (elected()) {
+            if (a.ell_slots) arrive_local(bars.decoded + 8u * ring.slot);      // the outlier warps come next
+            else arrive_cluster(bars.ready + 8u * ring.slot);
+        }
         ring.step(4, a.slots);
     }
     return true;
@@ -330,81 +339,59 @@ __device__ __forceinline__ void add_outlier(unsigned char* stage, uint32_t k, ui
     *w = __half_as_ushort(__hadd(__ushort_as_half(*w), __ushort_as_half(val)));
 }
 
-// The outlier warps' share of one tile.  list[2][kWindow][kListCap]: k | channel << 6 | value << 16; cnt[2][kWindow].
-// `ready0`: the first CTA's "ready" barrier of slot 0.
-__device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int lane, int q, int st0, int st1, unsigned char* pA,
-                                             uint32_t* list, int* cnt, const Bars& bars, uint32_t ready0, Ring ring, bool ok) {
-    constexpr int kBatch = 8;
-    const int ch = q * 32 + lane;
-    const bool any = a.ell_slots != 0;
+// The outlier warps' share of one tile (matrices with outliers): warp q adds those of row-block q.
+__device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int q, int lane, int st0, int st1, unsigned char* pA,
+                                             const Bars& bars, Ring ring) {
+    constexpr int kAhead = 4;
     Outliers o;
-    int cur = 0, start = 0;                     // next entry to deal; first entry of the window being added
-    uint32_t e[kBatch];
+    o.open(a, rb, rb * kRowsPerBlock + lane, lane);
+    int cur = o.find((uint32_t)st0 * kStageK);
+    const bool spills = __any_sync(0xffffffffu, o.total > o.nslab);
+    uint32_t e[kAhead];
     auto load = [&]() {
+        if (!spills) {
+            const uint32_t* p = o.slab + (size_t)(1 + cur) * 32;
 #pragma unroll
-        for (int i = 0; i < kBatch; ++i) e[i] = cur + i < o.total ? o.at(cur + i) : 0u;
+            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? __ldg(p + i * 32) : 0u;
+        } else {
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? o.at(cur + i) : 0u;
+        }
     };
-    // deal the entries of window [w0, w0 + kWindow) to its lists
-    auto deal = [&](int w0, int buf) {
-        const uint32_t end = (uint32_t)min(w0 + kWindow, st1) * kStageK;
+    load();
+    for (int st = st0; st < st1; ++st) {
+        const uint32_t end = (uint32_t)(st + 1) * kStageK;
+        unsigned char* mine = pA + (size_t)ring.slot * kABytes + (size_t)(q * 32 + lane) * 16;
+        if (!wait_bar(bars.decoded + 8u * ring.slot, ring.phase)) return false;
         for (;;) {
             int n = 0;
+            uint16_t* w[kAhead];
+            uint16_t v[kAhead];
+            bool in[kAhead];
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-                const uint32_t col = e[i] & 0xffffu;
-                if (cur + i < o.total && col < end) {
-                    const int st = (int)(col >> 6) - w0, at = atomicAdd(&cnt[buf * kWindow + st], 1);
-                    if (at < kListCap) list[(buf * kWindow + st) * kListCap + at] = (col & 63u) | (uint32_t)ch << 6 | (e[i] & 0xffff0000u);
-                    ++n;
-                }
+            for (int i = 0; i < kAhead; ++i) {
+                const uint32_t col = e[i] & 0xffffu, k = col & 63u;
+                in[i] = cur + i < o.total && col < end;
+                n += in[i];
+                w[i] = (uint16_t*)(mine + (k >> 3) * 2048u + (k & 7u) * 2u);
+                if (in[i]) v[i] = *w[i];
             }
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i)
+                if (in[i]) *w[i] = __half_as_ushort(__hadd(__ushort_as_half(v[i]), __ushort_as_half((uint16_t)(e[i] >> 16))));
             cur += n;
-            if (n) load();
-            if (n < kBatch) break;
-        }
-    };
-    if (any) {
-        o.open(a, rb, rb * kRowsPerBlock + lane, lane);
-        cur = start = o.find((uint32_t)st0 * kStageK);
-        load();
-        outlier_sync();                         // the lists' last use, in the previous tile, is over
-        if (ch < 2 * kWindow) cnt[ch] = 0;
-        outlier_sync();
-        deal(st0, 0);
-    }
-    for (int w0 = st0, buf = 0; w0 < st1; w0 += kWindow, buf ^= 1) {
-        const int next = cur;
-        if (any) {
-            outlier_sync();                     // the window's lists are complete, the other buffer is idle
-            if (ch < kWindow) cnt[(buf ^ 1) * kWindow + ch] = 0;
-            outlier_sync();
-        }
-        for (int st = w0; st < w0 + kWindow; ++st) {
-            if (any && st == w0 + kWindow / 2) deal(w0 + kWindow, buf ^ 1);
-            if (st >= st1) continue;
-            ok = ok && wait_bar(bars.decoded + 8u * ring.slot, ring.phase);
-            if (!ok) { ring.step(1, a.slots); continue; }         // this warp still meets the others at their barrier
-            if (any) {
-                unsigned char* stage = pA + (size_t)ring.slot * kABytes;
-                const int n = cnt[buf * kWindow + st - w0];
-                if (n <= kListCap) {
-                    const uint32_t* l = list + (buf * kWindow + st - w0) * kListCap;
-                    for (int i = ch; i < n; i += kOutWarps * 32) add_outlier(stage, l[i] & 63u, (l[i] >> 6) & 127u, (uint16_t)(l[i] >> 16));
-                } else {                        // more than the list holds: the channel's own entries
-                    for (int j = start; j < next; ++j) {
-                        const uint32_t v = o.at(j);
-                        if ((int)((v & 0xffffu) >> 6) == st) add_outlier(stage, v & 63u, (uint32_t)ch, (uint16_t)(v >> 16));
-                    }
-                }
+            if (!__any_sync(0xffffffffu, n == kAhead)) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (elected()) arrive_cluster(bars.ready + 8u * ring.slot);
+                if (n) load();                  // they travel while the next stage is decoded
+                break;
             }
-            __syncwarp();
-            if (elected()) arrive_cluster(ready0 + 8u * ring.slot);
-            ring.step(1, a.slots);
+            if (n) load();
         }
-        start = next;
+        ring.step(1, a.slots);
     }
-    return ok;
+    return true;
 }
 
 // SPLIT: a cluster of a.ks pairs per tile, one tile per cluster; else resident pairs walk the tiles.
@@ -414,10 +401,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // tables aligned to 8 KB of the shared window, so that an entry's offset is merged with the address, not added
     unsigned char* smem = smem_raw + ((8192u - (sa(smem_raw) & 8191u)) & 8191u);      // the same offset in every CTA
-    __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_landed[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
+    __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail, s_cnt[2 * kWindow];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int s_fail;
+    // the warp index through a shuffle: uniform as the compiler sees it, so that the roles run on uniform registers
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const uint32_t crank = cluster_rank(), h = crank & 1u, lead = crank & ~1u;        // half of the pair, its first CTA
     const int slice = (int)(crank >> 1);
     const int first = SPLIT ? (int)blockIdx.x / (2 * a.ks) : (int)blockIdx.x >> 1, step = SPLIT ? 1 << 28 : (int)gridDim.x >> 1;
@@ -425,16 +413,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), st0 = 2 * sc0, st1 = 2 * sc1, nst = st1 - st0;
     unsigned char* pA = smem + a.tab_bytes;
     unsigned char* pB = pA + (size_t)a.slots * kABytes;
-    uint32_t* list = (uint32_t*)(pB + (size_t)a.slots * a.x_bytes);                  // the outlier warps' lists (with outliers)
-    uint16_t* lib = (uint16_t*)((unsigned char*)list + (a.ell_slots ? kListBytes : 0));
-    const Bars bars{sa(b_decoded), sa(b_ready), sa(b_landed), sa(b_freed)};
+    uint16_t* lib = (uint16_t*)(pB + (size_t)a.slots * a.x_bytes);
+    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), lead)};
     asm volatile("griddepcontrol.launch_dependents;");
 
     if (tid == 0) {
         for (int i = 0; i < a.slots; ++i) {
             init_bar(&b_decoded[i], 4);                       // a warp per row-block
-            init_bar(&b_ready[i], 2 * kOutWarps + 1);         // outlier warps of both CTAs, x of the second (in the first CTA)
-            init_bar(&b_landed[i], 1);
+            init_bar(&b_ready[i], 2 * kOutWarps + 1);         // four row-blocks of both CTAs, and the bytes of x
             init_bar(&b_freed[i], 1);
         }
         init_bar(&acc_full, 1);
@@ -521,13 +507,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
         }
     } else if (warp < kCopyWarp) {
         const int q = warp - kDecodeWarps;
-        const uint32_t ready0 = peer(bars.ready, lead);
         cluster_wait();
-        for (int t = first; t < tiles; t += step) {
-            const int tx = t / a.tok_tiles, rb = (2 * tx + (int)h) * 4 + q;
-            ok = outlier_tile(a, rb, lane, q, st0, st1, pA, list, s_cnt, bars, ready0, ring, ok);
-            ring.step(nst, a.slots);
-        }
+        if (a.ell_slots)
+            for (int t = first; t < tiles && ok; t += step) {
+                ok = outlier_tile(a, (2 * (t / a.tok_tiles) + (int)h) * 4 + q, q, lane, st0, st1, pA, bars, ring);
+                ring.step(nst, a.slots);
+            }
     } else if (warp == kCopyWarp) {
         cluster_wait();
         asm volatile("griddepcontrol.wait;" ::: "memory");    // x may come from the previous kernel of the stream
@@ -536,13 +521,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             for (int st = st0; st < st1; ++st) {
                 if (!(ok = wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u))) break;
                 if (elected()) {
-                    const uint32_t bar = bars.landed + 8u * ring.slot;
+                    const uint32_t bar = bars.ready + 8u * ring.slot;
                     uint32_t dst = sa(pB) + (uint32_t)(ring.slot * a.x_bytes);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"((uint32_t)a.x_bytes) : "memory");
+                    if (h == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(sa(b_ready) + 8u * ring.slot), "r"((uint32_t)(2 * a.x_bytes)) : "memory");
                     for (int p = 0; p < a.parts; ++p, dst += (uint32_t)a.Tp * 64u) {
                         // this CTA's half of the part's rows (of those that exist, rounded up to 16; more may be copied along)
                         const int p0 = t0 + p * a.Tp, n = min(a.Tp, max((a.M - p0 + 15) & ~15, 16)), xrow = p0 + (int)h * (n >> 1);
-                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                        asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                                      :: "r"(dst), "l"(&tmap), "r"(st * kStageK), "r"(xrow), "r"(bar) : "memory");
                     }
                 }
@@ -550,17 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 ring.step(1, a.slots);
             }
         }
-    } else if (h == 1) {                                      // the second CTA: tell the first that x has landed here
-        const uint32_t ready0 = peer(bars.ready, lead);
-        cluster_wait();
-        for (int t = first; t < tiles && ok; t += step) {
-            for (int st = st0; st < st1; ++st) {
-                if (!(ok = wait_bar(bars.landed + 8u * ring.slot, ring.phase))) break;
-                if (elected()) arrive_cluster(ready0 + 8u * ring.slot);
-                __syncwarp();
-                ring.step(1, a.slots);
-            }
-        }
+    } else if (h == 1) {
+        cluster_wait();                                       // the first CTA issues the pair's products
     } else {
         const uint64_t da0 = desc_a(sa(pA)), db0 = desc_b(sa(pB));
         const uint32_t mask = 3u << lead;
@@ -574,9 +550,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 if (!ok) break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            bool there = test_bar(bars.ready + 8u * ring.slot, ring.phase);
             for (int st = st0; st < st1; ++st) {
-                if (!(ok = wait_bar(bars.landed + 8u * ring.slot, ring.phase) && wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
+                if (!there && !(ok = wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                Ring on = ring;
+                on.step(1, a.slots);
+                there = st + 1 < st1 && test_bar(bars.ready + 8u * on.slot, on.phase);     // the answer comes under the products
                 if (elected()) {
                     const uint64_t da = da0 + (uint64_t)((uint32_t)ring.slot * (kABytes >> 4));
                     uint64_t db = db0 + (uint64_t)((uint32_t)(ring.slot * a.x_bytes) >> 4);
@@ -593,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                     if (st + 1 == st1) commit_pair(sa(&acc_full), mask);
                 }
                 __syncwarp();
-                ring.step(1, a.slots);
+                ring = on;
             }
         }
     }
@@ -601,8 +581,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (s_fail && tid == 0)      // copies in flight land before the CTA goes
-        for (int i = 0; i < a.slots; ++i) wait_bar(bars.landed + 8u * i, 0);
+    if (s_fail)                  // copies in flight land before the CTA goes (a millisecond is a thousand times their way)
+        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     __syncwarp();
     cluster_sync();
     if (SPLIT) {
@@ -724,7 +704,6 @@ FusedPlan plan_fused(const Layout& l, int M) {
     FusedPlan best = {};
     const size_t tab = (table_bytes(l) + 1023) & ~size_t(1023);
     const size_t lib = l.mode && (size_t)l.L * l.E <= kLibEntries ? ((size_t)l.L * (l.E + 8) * 2 + 15) & ~size_t(15) : 0;
-    const size_t lists = l.ell_slots ? kListBytes : 0;
     const int pairs = (l.RB + 7) / 8;
     int last_T = 0;
     for (int n = (M + 511) / 512; n <= (M + 15) / 16; ++n) {          // tiles along the rows of x
@@ -733,7 +712,7 @@ FusedPlan plan_fused(const Layout& l, int M) {
         last_T = T;
         if (T < 64 && best.clocks > 0.0) break;
         const int tok = (M + T - 1) / T;
-        int slots = (int)((kSmemMax - 8192 - tab - lib - lists) / (kABytes + (size_t)T * 64));
+        int slots = (int)((kSmemMax - 8192 - tab - lib) / (kABytes + (size_t)T * 64));
         if (slots > kMaxSlots) slots = kMaxSlots;
         if (slots < 2) continue;
         for (int ks = 1; ks <= kMaxCut; ++ks) {
@@ -751,7 +730,7 @@ FusedPlan plan_fused(const Layout& l, int M) {
         }
     }
     best.tab = tab; best.lib = lib;
-    best.smem = 8192 + tab + lib + lists + (size_t)best.slots * (kABytes + (size_t)best.T * 64);
+    best.smem = 8192 + tab + lib + (size_t)best.slots * (kABytes + (size_t)best.T * 64);
     return best;
 }
 
