@@ -15,8 +15,10 @@
 //            warps, where the addition has to find its register by nested tests, it cost as much as the decode).  1 copies,
 //            1 products.  Roles meet at mbarriers only: a stage is "ready" on the first CTA's barrier when the last of both
 //            CTAs' row-blocks are stored and both CTAs' x has landed (the copies of both count their bytes there).
-//   K cut    few tiles: a cluster of 2, 3 or 4 pairs cuts the tile along K; the partial sums meet through distributed shared
-//            memory and are added in slice order.  Many tiles: resident pairs walk them.
+//   schedule resident pairs.  Whole rounds of tiles run whole tiles; what remains is one stream of super-chunks that is dealt
+//            evenly over the pairs, so a pair ends one tile and begins the next (28672 x 8192, 1024 rows: 4.5 rounds instead of
+//            5; 10007 x 4992, 301 rows: 40 tiles on 74 pairs).  A CTA that had part of a tile leaves fp32 sums in the
+//            workspace; the last to come of a tile adds the parts in order of K.  Nobody waits for another pair.
 //   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
 //            table (D16 = fp16(fp32(scale * lib + mid))); the look-ups are then those of V2.
 // Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace, stops
@@ -35,23 +37,25 @@ constexpr int kStageK = 64;
 constexpr int kABytes = kCh * kStageK * 2;     // A of one stage
 constexpr int kMaxSlots = 12;
 constexpr int kDecodeWarps = 16, kOutWarps = 4;
-constexpr int kCopyWarp = kDecodeWarps + kOutWarps, kMmaWarp = kCopyWarp + 1;
+constexpr int kCopyWarps = 2, kCopyWarp = kDecodeWarps + kOutWarps, kMmaWarp = kCopyWarp + kCopyWarps;
 constexpr int kThreads = (kMmaWarp + 1) * 32;
 constexpr uint32_t kSpins = 1u << 20, kPollHint = 1000;
 constexpr size_t kSmemMax = 226 * 1024;
 constexpr int kLibEntries = 8192;              // V2a library entries staged in shared memory
-constexpr int kMaxCut = 4;                     // pairs of a cluster
+constexpr int kPairs = kSizingSMs / 2;         // pairs that the schedule deals to; a device with fewer runs them in turn
 
 struct FusedArgs {
     Blob b;
     void* y;
-    int* ctrl;                  // [0] error word
+    int* ctrl;                  // [0] error word, [1 + 2 * tile + half] arrivals of the parts of a cut tile
+    float* part;                // [2 * pair + which][half][T][128] sums of a part
     int rows, RB, SC, M, ell_slots, GH, L, y_kind;
     int pairs, tok_tiles;       // tiles: 256 channels, T rows of x
-    int T, Tp, parts;           // T = parts * Tp, Tp <= 256: one product instruction covers Tp rows
+    int T, Tp, parts;           // one product instruction covers Tp <= 256 rows, the second T - Tp; both multiples of 32
     int slots, x_bytes;         // stages in the ring; bytes of x per stage and CTA
     int tab_bytes;
-    int ks, sc_slice;           // pairs along K, super-chunks of each
+    int whole;                  // whole tiles per pair; the rest (`stream` super-chunks from tile whole * kPairs on) is dealt
+    int stream, dealt;          // evenly to pairs 0 .. dealt - 1
     int tmem_cols;
 };
 
@@ -120,9 +124,9 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t da, uint64_t 
         :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
 }
 // the products issued so far arrive on the barrier of both CTAs of the pair
-__device__ __forceinline__ void commit_pair(uint32_t bar, uint32_t mask) {
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 :: "r"(bar), "h"((uint16_t)mask) : "memory");
+                 :: "r"(bar), "h"((uint16_t)3) : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
@@ -136,6 +140,11 @@ __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("m
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// the other half of the kernel's first arrival at the cluster barrier: the other CTA's barriers exist
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
 __device__ __forceinline__ void decode_sync() { asm volatile("bar.sync 1, %0;" :: "n"(kDecodeWarps * 32) : "memory"); }
 
 // Position in the ring after a number of stages: slot and the parity of its current use.
@@ -146,7 +155,32 @@ struct Ring {
         slot += n;
         while (slot >= slots) { slot -= slots; phase ^= 1u; }
     }
+    __device__ __forceinline__ void jump(int n, int slots) {
+        const int q = (slot + n) / slots;
+        slot += n - q * slots;
+        phase ^= (uint32_t)q & 1u;
+    }
 };
+
+// The i-th piece of work of pair g: super-chunks [sc0, sc1) of a tile.  Pair g has [g S / D, (g + 1) S / D) of the S dealt
+// super-chunks, at most a tile's worth, so at most two pieces.
+struct Piece { int tile, sc0, sc1; };
+__device__ __forceinline__ bool piece_of(const FusedArgs& a, int g, int i, Piece& p) {
+    if (i < a.whole) { p.tile = g + i * kPairs; p.sc0 = 0; p.sc1 = a.SC; return true; }
+    i -= a.whole;
+    if (g >= a.dealt || i > 1) return false;
+    const int u0 = (int)((long long)g * a.stream / a.dealt), u1 = (int)((long long)(g + 1) * a.stream / a.dealt);
+    const int t = u0 / a.SC + i, b = t * a.SC;
+    if (u1 <= b) return false;
+    p.tile = a.whole * kPairs + t; p.sc0 = u0 > b ? u0 - b : 0; p.sc1 = min(a.SC, u1 - b);
+    return true;
+}
+// rows of x of the p-th product of a stage, which begins at row p0: those that exist, rounded up to 32
+__device__ __forceinline__ int product_rows(const FusedArgs& a, int p0, int p) {
+    return min(p ? a.T - a.Tp : a.Tp, max((a.M - p0 + 31) & ~31, 32));
+}
+// the pair that has dealt super-chunk u: the largest g with g S / D <= u
+__device__ __forceinline__ int dealt_to(const FusedArgs& a, int u) { return (int)(((long long)(u + 1) * a.dealt - 1) / a.stream); }
 
 // Decode tables.  kPair: entry t = first index | second index << N holds two fp16 values; else entry q one.  N = 4 entries lie
 // 256 bytes apart (two tables interleaved): an index isolated in its own byte becomes the second byte of the address.
@@ -214,7 +248,7 @@ struct Bars {
 // The decode warps' share of one tile: half PART of super-chunks grp, grp + 2, ... of [sc0, sc1): every fourth stage.
 template <int N, int MODE, int PART>
 __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_ok, int q, int grp, int lane, int sc0, int sc1,
-                                            uint32_t tab, const uint16_t* slib, uint32_t sA, const Bars& bars, Ring ring) {
+                                            uint32_t tab, const uint16_t* slib, uint32_t sA, const Bars& bars, Ring ring, bool& met) {
     using T = Tab<N, MODE>;
     using H = Half<N, PART>;
     constexpr int E = T::E;
@@ -293,6 +327,7 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the products read through the async proxy
         __syncwarp();
+        if (!a.ell_slots && !met) { cluster_wait(); met = true; }             // the first arrival at the other CTA
         if (elected()) {
             if (a.ell_slots) arrive_local(bars.decoded + 8u * ring.slot);      // the outlier warps come next
             else arrive_cluster(bars.ready + 8u * ring.slot);
@@ -394,8 +429,25 @@ __device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int q, 
     return true;
 }
 
-// SPLIT: a cluster of a.ks pairs per tile, one tile per cluster; else resident pairs walk the tiles.
-template <int N, int MODE, bool SPLIT>
+// 16 sums of one channel, rows of x t0 .. t0 + n - 1
+__device__ __forceinline__ void store_rows(const FusedArgs& a, int t0, int n, int row, const uint32_t (&v)[16]) {
+    const size_t o = (size_t)t0 * a.rows + row;
+    if (a.y_kind == 1) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = f2h(__uint_as_float(v[j]));
+    } else if (a.y_kind == 2) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[j])));
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < n) ((float*)a.y)[o + (size_t)j * a.rows] = __uint_as_float(v[j]);
+    }
+}
+
+template <int N, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
     using T = Tab<N, MODE>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -403,31 +455,28 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     unsigned char* smem = smem_raw + ((8192u - (sa(smem_raw) & 8191u)) & 8191u);      // the same offset in every CTA
     __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail;
+    __shared__ int s_fail, s_last;
     // the warp index through a shuffle: uniform as the compiler sees it, so that the roles run on uniform registers
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const uint32_t crank = cluster_rank(), h = crank & 1u, lead = crank & ~1u;        // half of the pair, its first CTA
-    const int slice = (int)(crank >> 1);
-    const int first = SPLIT ? (int)blockIdx.x / (2 * a.ks) : (int)blockIdx.x >> 1, step = SPLIT ? 1 << 28 : (int)gridDim.x >> 1;
-    const int tiles = a.pairs * a.tok_tiles;
-    const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), st0 = 2 * sc0, st1 = 2 * sc1, nst = st1 - st0;
+    const uint32_t h = cluster_rank();                        // half of the pair; CTA 0 issues the products
+    const int g = (int)blockIdx.x >> 1;
     unsigned char* pA = smem + a.tab_bytes;
     unsigned char* pB = pA + (size_t)a.slots * kABytes;
     uint16_t* lib = (uint16_t*)(pB + (size_t)a.slots * a.x_bytes);
-    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), lead)};
+    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), 0)};
     asm volatile("griddepcontrol.launch_dependents;");
 
-    if (tid == 0) {
-        for (int i = 0; i < a.slots; ++i) {
-            init_bar(&b_decoded[i], 4);                       // a warp per row-block
-            init_bar(&b_ready[i], 2 * kOutWarps + 1);         // four row-blocks of both CTAs, and the bytes of x
-            init_bar(&b_freed[i], 1);
-        }
+    if (tid < a.slots) {
+        init_bar(&b_decoded[tid], 4);                         // a warp per row-block
+        init_bar(&b_ready[tid], 2 * 4 + 1);                   // four row-blocks of both CTAs, and the bytes of x
+        init_bar(&b_freed[tid], 1);
+    }
+    if (tid == 32) {
         init_bar(&acc_full, 1);
         init_bar(&acc_empty, 2 * kDecodeWarps);
         s_fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     const bool staged = MODE == 1 && a.L * T::E <= kLibEntries;
     if (staged)
         for (int i = tid; i < a.L * T::E; i += kThreads) lib[(i / T::E) * (T::E + 8) + i % T::E] = __ldg(a.b.cb + i);
@@ -438,22 +487,20 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     // Nothing remote happens before the wait that belongs to this arrival: the decode warps begin at once and wait in front of
-    // their first epilogue, the others before they start.
+    // their first arrival at the other CTA, the others before they start.
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    auto cluster_wait = [] {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    };
 
     bool ok = true;
     Ring ring{0, 0u};
     uint32_t acc_ph = 0;
+    Piece pc;
     if (warp < kDecodeWarps) {
         const int q = warp & 3, part = (warp >> 2) & 1, grp = warp >> 3;
         const uint32_t tab = T::at(sa(smem), MODE == 0 ? q : warp, lane);
+        bool met = false;                                     // has waited for the other CTA's barriers
         int have = -1;                                        // tile of channels whose tables are in place
-        for (int t = first; t < tiles; t += step) {           // a warp whose wait ran out still meets the others at their barrier
-            const int tx = t / a.tok_tiles, ty = t % a.tok_tiles, t0 = ty * a.T;
+        for (int i = 0; piece_of(a, g, i, pc); ++i) {         // a warp whose wait ran out still meets the others at their barrier
+            const int tx = pc.tile / a.tok_tiles, ty = pc.tile % a.tok_tiles, t0 = ty * a.T;
             const int rb = (2 * tx + (int)h) * 4 + q;
             if (MODE == 0 && tx != have) {
                 decode_sync();                                // every warp is done with the previous tables
@@ -462,96 +509,119 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 have = tx;
             }
             const uint16_t* slib = staged ? lib : nullptr;
-            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, sc0, sc1, tab, slib, sa(pA), bars, ring)
-                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, sc0, sc1, tab, slib, sa(pA), bars, ring));
-            ring.step(nst, a.slots);
-            if (t == first) cluster_wait();
+            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met)
+                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met));
+            ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
             ok = ok && wait_bar(sa(&acc_full), acc_ph);
             acc_ph ^= 1u;
-            if (!ok) continue;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t tmem = s_tmem;
+            const uint32_t acc = s_tmem + ((uint32_t)(q * 32) << 16);
             const int r = q * 32 + lane, row = (2 * tx + (int)h) * kCh + r;
             const int tend = min(a.T, a.M - t0);
-            for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), v);
-                if (SPLIT) {
-                    // every product of the pair is complete, its slots are idle: the partial sums go there, [t][channel]
-                    float* p = (float*)pA + (size_t)c * 16 * kCh + r;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) p[(size_t)j * kCh] = __uint_as_float(v[j]);
-                } else if (row < a.rows) {
-                    const int n = min(16, tend - c * 16);
-                    const size_t o = (size_t)(t0 + c * 16) * a.rows + row;
-                    if (a.y_kind == 1) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = f2h(__uint_as_float(v[j]));
-                    } else if (a.y_kind == 2) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (j < n) ((uint16_t*)a.y)[o + (size_t)j * a.rows] = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[j])));
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (j < n) ((float*)a.y)[o + (size_t)j * a.rows] = __uint_as_float(v[j]);
+            const bool whole = pc.sc0 == 0 && pc.sc1 == a.SC;
+            const size_t psize = (size_t)a.T * kCh;
+            if (whole) {
+                if (ok)
+                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
+                        uint32_t v[16];
+                        tmem_ld16(acc + (uint32_t)(c * 16), v);             // the whole warp
+                        if (row < a.rows) store_rows(a, t0 + c * 16, min(16, tend - c * 16), row, v);
                     }
+            } else {
+                const int u0 = (pc.tile - a.whole * kPairs) * a.SC, g0 = dealt_to(a, u0), g1 = dealt_to(a, u0 + a.SC - 1);
+                // part of pair z: its second piece unless its first begins in this tile
+                auto part_at = [&](int z) {
+                    const int first = (int)((long long)z * a.stream / a.dealt) / a.SC;
+                    return a.part + ((size_t)(2 * z + (first == pc.tile - a.whole * kPairs ? 0 : 1)) * 2 + h) * psize + r;
+                };
+                float* mine = part_at(g);
+                if (ok)
+                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
+                        uint32_t v[16];
+                        tmem_ld16(acc + (uint32_t)(c * 16), v);
+                        float* p = mine + (size_t)c * 16 * kCh;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) __stcg(p + (size_t)j * kCh, __uint_as_float(v[j]));
+                    }
+                __threadfence();
+                decode_sync();
+                if (tid == 0) {
+                    int* count = a.ctrl + 1 + 2 * (pc.tile - a.whole * kPairs) + h;
+                    const int last = atomicAdd(count, 1) == g1 - g0;
+                    if (last) *count = 0;
+                    s_last = last;
+                    __threadfence();
                 }
+                decode_sync();
+                if (s_last && ok && row < a.rows)
+                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
+                        uint32_t sum[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[j] = 0u;
+                        for (int z = g0; z <= g1; ++z) {
+                            const float* p = part_at(z) + (size_t)c * 16 * kCh;
+                            float v[16];
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) v[j] = __ldcg(p + (size_t)j * kCh);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) sum[j] = __float_as_uint(z == g0 ? v[j] : __uint_as_float(sum[j]) + v[j]);
+                        }
+                        store_rows(a, t0 + c * 16, min(16, tend - c * 16), row, sum);
+                    }
             }
-            if (!SPLIT) {
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (elected()) arrive_cluster(peer(sa(&acc_empty), lead));
-            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            if (!met) { cluster_wait(); met = true; }
+            __syncwarp();
+            if (elected()) arrive_cluster(peer(sa(&acc_empty), 0));
         }
     } else if (warp < kCopyWarp) {
         const int q = warp - kDecodeWarps;
         cluster_wait();
         if (a.ell_slots)
-            for (int t = first; t < tiles && ok; t += step) {
-                ok = outlier_tile(a, (2 * (t / a.tok_tiles) + (int)h) * 4 + q, q, lane, st0, st1, pA, bars, ring);
-                ring.step(nst, a.slots);
+            for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
+                ok = outlier_tile(a, (2 * (pc.tile / a.tok_tiles) + (int)h) * 4 + q, q, lane, 2 * pc.sc0, 2 * pc.sc1, pA, bars, ring);
+                ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
             }
-    } else if (warp == kCopyWarp) {
+    } else if (warp < kMmaWarp) {
         cluster_wait();
         asm volatile("griddepcontrol.wait;" ::: "memory");    // x may come from the previous kernel of the stream
-        for (int t = first; t < tiles && ok; t += step) {
-            const int t0 = (t % a.tok_tiles) * a.T;
-            for (int st = st0; st < st1; ++st) {
+        int n = warp - kCopyWarp;                             // the two warps take the stages in turn
+        for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
+            const int t0 = (pc.tile % a.tok_tiles) * a.T;
+            for (int st = 2 * pc.sc0; st < 2 * pc.sc1; ++st, ring.step(1, a.slots)) {
+                if (n++ & 1) continue;
                 if (!(ok = wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u))) break;
                 if (elected()) {
                     const uint32_t bar = bars.ready + 8u * ring.slot;
                     uint32_t dst = sa(pB) + (uint32_t)(ring.slot * a.x_bytes);
                     if (h == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(sa(b_ready) + 8u * ring.slot), "r"((uint32_t)(2 * a.x_bytes)) : "memory");
                     for (int p = 0; p < a.parts; ++p, dst += (uint32_t)a.Tp * 64u) {
-                        // this CTA's half of the part's rows (of those that exist, rounded up to 16; more may be copied along)
-                        const int p0 = t0 + p * a.Tp, n = min(a.Tp, max((a.M - p0 + 15) & ~15, 16)), xrow = p0 + (int)h * (n >> 1);
+                        // this CTA's half of the rows that the product takes (more may be copied along)
+                        const int p0 = t0 + p * a.Tp, xrow = p0 + (int)h * (product_rows(a, p0, p) >> 1);
                         asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                                      :: "r"(dst), "l"(&tmap), "r"(st * kStageK), "r"(xrow), "r"(bar) : "memory");
                     }
                 }
                 __syncwarp();
-                ring.step(1, a.slots);
             }
         }
     } else if (h == 1) {
         cluster_wait();                                       // the first CTA issues the pair's products
     } else {
         const uint64_t da0 = desc_a(sa(pA)), db0 = desc_b(sa(pB));
-        const uint32_t mask = 3u << lead;
         cluster_wait();
         const uint32_t tmem = s_tmem;
-        for (int t = first; t < tiles && ok; t += step) {
-            const int t0 = (t % a.tok_tiles) * a.T;
-            if (t != first) {
-                ok = wait_bar(sa(&acc_empty), acc_ph);        // the previous tile's sums have been read
+        for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
+            const int t0 = (pc.tile % a.tok_tiles) * a.T, st1 = 2 * pc.sc1;
+            if (i) {
+                ok = wait_bar(sa(&acc_empty), acc_ph);        // the previous piece's sums have been read
                 acc_ph ^= 1u;
                 if (!ok) break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t acc = 0;
             bool there = test_bar(bars.ready + 8u * ring.slot, ring.phase);
-            for (int st = st0; st < st1; ++st) {
+            for (int st = 2 * pc.sc0; st < st1; ++st) {
                 if (!there && !(ok = wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 Ring on = ring;
@@ -563,15 +633,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                     for (int p = 0; p < a.parts; ++p, db += (uint64_t)(a.Tp * 4)) {
                         const int p0 = t0 + p * a.Tp;
                         if (p0 >= a.M) break;
-                        const int n = min(a.Tp, (a.M - p0 + 15) & ~15);
+                        const int n = product_rows(a, p0, p);
                         const uint32_t idesc = (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * kCh >> 4) << 24);
 #pragma unroll
-                        for (int i = 0; i < kStageK / 16; ++i)
-                            mma_pair(tmem + (uint32_t)(p * a.Tp), da + i * 256, db + i * 2, idesc, (st > st0 || i > 0) ? 1u : 0u);
+                        for (int k = 0; k < kStageK / 16; ++k)
+                            mma_pair(tmem + (uint32_t)(p * a.Tp), da + k * 256, db + k * 2, idesc, k ? 1u : acc);
                     }
-                    commit_pair(bars.freed + 8u * ring.slot, mask);
-                    if (st + 1 == st1) commit_pair(sa(&acc_full), mask);
+                    commit_pair(bars.freed + 8u * ring.slot);
+                    if (st + 1 == st1) commit_pair(sa(&acc_full));
                 }
+                acc = 1;
                 __syncwarp();
                 ring = on;
             }
@@ -585,56 +656,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     __syncwarp();
     cluster_sync();
-    if (SPLIT) {
-        // this CTA's share of the rows of x of its 128 channels: the slices' sums added in slice order
-        if (first < tiles) {
-            const int tx = first / a.tok_tiles, t0 = (first % a.tok_tiles) * a.T, Tn = min(a.T, a.M - t0);
-            const int share = (Tn + a.ks - 1) / a.ks, b0 = slice * share, b1 = min(Tn, b0 + share);
-            const uint32_t own = sa(pA);
-            const bool wide = (a.rows & 3) == 0;               // four channels in one store
-            for (int i0 = b0 * (kCh / 4) + tid; i0 < b1 * (kCh / 4); i0 += 2 * kThreads) {
-                float4 v[2][kMaxCut];                         // two places, every slice's share in flight
-#pragma unroll
-                for (int u = 0; u < 2; ++u)
-#pragma unroll
-                    for (int z = 0; z < kMaxCut; ++z) {
-                        const int i = i0 + u * kThreads;
-                        v[u][z] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (z < a.ks && i < b1 * (kCh / 4))
-                            asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[u][z].x), "=f"(v[u][z].y), "=f"(v[u][z].z), "=f"(v[u][z].w)
-                                         : "r"(peer(own + (uint32_t)i * 16u, 2u * (uint32_t)z + h)));
-                    }
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int i = i0 + u * kThreads;
-                    if (i >= b1 * (kCh / 4)) break;
-                    float4 sum = v[u][0];
-#pragma unroll
-                    for (int z = 1; z < kMaxCut; ++z)
-                        if (z < a.ks) { sum.x += v[u][z].x; sum.y += v[u][z].y; sum.z += v[u][z].z; sum.w += v[u][z].w; }
-                    const int tt = t0 + i / (kCh / 4), row = (2 * tx + (int)h) * kCh + (i % (kCh / 4)) * 4;
-                    const size_t o = (size_t)tt * a.rows + row;
-                    if (wide && row < a.rows) {
-                        if (a.y_kind == 0) *(float4*)((float*)a.y + o) = sum;
-                        else if (a.y_kind == 1) {
-                            const __half2 lo = __floats2half2_rn(sum.x, sum.y), hi = __floats2half2_rn(sum.z, sum.w);
-                            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
-                        } else {
-                            const __nv_bfloat162 lo = __floats2bfloat162_rn(sum.x, sum.y), hi = __floats2bfloat162_rn(sum.z, sum.w);
-                            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
-                        }
-                    } else {
-                        if (row < a.rows) put_y(a.y, o, sum.x, a.y_kind);
-                        if (row + 1 < a.rows) put_y(a.y, o + 1, sum.y, a.y_kind);
-                        if (row + 2 < a.rows) put_y(a.y, o + 2, sum.z, a.y_kind);
-                        if (row + 3 < a.rows) put_y(a.y, o + 3, sum.w, a.y_kind);
-                    }
-                }
-            }
-        }
-        __syncwarp();
-        cluster_sync();          // no CTA leaves while another reads its shared memory
-    }
     if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(s_tmem), "r"(a.tmem_cols) : "memory");
 }
@@ -650,36 +671,10 @@ EncodeTiledFn encode_fn() {
     return (EncodeTiledFn)fn;
 }
 
-// Clusters of 2 * ks CTAs of this kernel that the current device runs at once (a cluster stays inside a GPC, so the larger
-// ones leave SMs idle), asked once per device.
-int clusters_at_once(int ks) {
-    static std::atomic<int> cache[256][kMaxCut + 1] = {};
-    std::atomic<int>& slot = cache[DeviceOnce::current()][ks];
-    int n = slot.load(std::memory_order_relaxed);
-    if (n == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(2 * ks), 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
-        cfg.dynamicSmemBytes = kSmemMax;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)(2 * ks); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(gemm_fused_kernel<4, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, gemm_fused_kernel<4, 0, true>, &cfg) != cudaSuccess || n < 1) {
-            cudaGetLastError();
-            n = sm_count() / (2 * ks) > 0 ? sm_count() / (2 * ks) : 1;
-        }
-        slot.store(n, std::memory_order_relaxed);
-    }
-    return n;
-}
-
 // ------------------------------------------------------------------ plan
 
 struct FusedPlan {
-    int T, Tp, parts, tok_tiles, pairs, ks, sc_slice, slots;
+    int T, Tp, parts, tok_tiles, pairs, slots, whole, stream, dealt;
     size_t tab, lib, smem;
     double clocks;             // what the model expects
 };
@@ -707,32 +702,38 @@ FusedPlan plan_fused(const Layout& l, int M) {
     const int pairs = (l.RB + 7) / 8;
     int last_T = 0;
     for (int n = (M + 511) / 512; n <= (M + 15) / 16; ++n) {          // tiles along the rows of x
-        const int t = (M + n - 1) / n, parts = t > 256 ? 2 : 1, Tp = ((t + parts - 1) / parts + 15) & ~15, T = parts * Tp;
-        if (T == last_T || T > 512) continue;
+        const int t = (M + n - 1) / n, parts = t > 256 ? 2 : 1, T = (t + 31) & ~31, Tp = parts == 1 ? T : (T / 2 + 31) & ~31;
+        if (T == last_T) continue;
         last_T = T;
         if (T < 64 && best.clocks > 0.0) break;
         const int tok = (M + T - 1) / T;
-        int slots = (int)((kSmemMax - 8192 - tab - lib) / (kABytes + (size_t)T * 64));
+        int slots = (int)((kSmemMax - 8192 - tab - lib) / (kABytes + (size_t)parts * Tp * 64));
         if (slots > kMaxSlots) slots = kMaxSlots;
         if (slots < 2) continue;
-        for (int ks = 1; ks <= kMaxCut; ++ks) {
-            const int spp = (l.SC + ks - 1) / ks;
-            if (ks > 1 && ((ks - 1) * spp >= l.SC || spp < 2 || (size_t)T * kCh * 4 > slots * (kABytes + (size_t)T * 64))) break;
-            const int at_once = clusters_at_once(ks);
-            const int tiles = pairs * tok, waves = (tiles + at_once - 1) / at_once;
-            // a stage's way through decode, outliers and products takes about 2900 clocks and its share of the products
-            const double chain = (2900.0 + 2.0 * T) / slots * 2.0, busy = slot_clocks(l, T);
-            const double clocks = waves * (spp * (busy > chain ? busy : chain) + 1500.0 + 10.0 * T + (ks > 1 ? 1500.0 + 8.0 * T : 0.0));
+        // a stage's way through decode, outliers and products takes about 2900 clocks and its share of the products
+        const double chain = (2900.0 + 2.0 * T) / slots * 2.0, busy = slot_clocks(l, T), step = busy > chain ? busy : chain;
+        const double move = T * 512.0 / 40.0;                  // a CTA's sums to or from the workspace
+        const int tiles = pairs * tok, whole = tiles / kPairs, rest = tiles - whole * kPairs;
+        const double rounds = whole * (l.SC * step + 1500.0 + 10.0 * T);
+        for (int k = 1; k <= 9 && rest * (k > 8 ? 1 : k) <= kPairs; ++k) {     // every remaining tile in k parts; or an even deal
+            const int dealt = rest == 0 ? 0 : k > 8 ? kPairs : rest * k, stream = rest * l.SC;
+            if (rest && (dealt > stream / 2 && k > 1)) continue;  // a part has at least two super-chunks
+            const int most = rest ? (stream + dealt - 1) / dealt : 0, cuts = k == 1 ? 1 : k > 8 ? (l.SC - 1) / most + 2 : k;
+            const double clocks = rounds + (rest ? most * step + 1500.0 + 10.0 * T + (k > 8 ? 2000.0 : 0.0) : 0.0) + (cuts > 1 ? 3000.0 + cuts * move : 0.0);
             if (best.clocks == 0.0 || clocks < best.clocks) {
-                best.T = T; best.Tp = Tp; best.parts = parts; best.tok_tiles = tok; best.pairs = pairs; best.ks = ks;
-                best.sc_slice = spp; best.slots = slots; best.clocks = clocks;
+                best.T = T; best.Tp = Tp; best.parts = parts; best.tok_tiles = tok; best.pairs = pairs; best.slots = slots;
+                best.whole = whole; best.stream = stream; best.dealt = dealt; best.clocks = clocks;
             }
+            if (!rest) break;
         }
     }
     best.tab = tab; best.lib = lib;
-    best.smem = 8192 + tab + lib + (size_t)best.slots * (kABytes + (size_t)best.T * 64);
+    best.smem = 8192 + tab + lib + (size_t)best.slots * (kABytes + (size_t)best.parts * best.Tp * 64);
     return best;
 }
+
+// counters behind the error word: two per tile, and at least one for every 128 channels and 256 rows of x
+size_t fused_ctrl_bytes(const Layout& l, int M) { return align256(4 * (size_t)(1 + 2 * ((l.RB + 7) / 8) * ((M + 63) / 64))); }
 
 template <int N, int MODE>
 cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
@@ -753,34 +754,31 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        const cudaError_t e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
     FusedArgs a = {};
     a.b = blob_at(c.packed, offsets_of(l));
-    a.y = c.y; a.ctrl = (int*)c.workspace;
+    a.y = c.y; a.ctrl = (int*)c.workspace; a.part = (float*)((char*)c.workspace + fused_ctrl_bytes(l, c.M));
     a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L; a.y_kind = c.y_kind;
     a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
-    a.slots = p.slots; a.x_bytes = p.T * 64; a.tab_bytes = (int)p.tab;
-    a.ks = p.ks; a.sc_slice = p.sc_slice;
+    a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
+    a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
     a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
-    const int tiles = p.pairs * p.tok_tiles, pair_slots = clusters_at_once(1);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.ks > 1 ? tiles * 2 * p.ks : 2 * (tiles < pair_slots ? tiles : pair_slots)), 1, 1);
+    cfg.gridDim = dim3((unsigned)(2 * (p.whole ? kPairs : p.dealt)), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)(2 * p.ks); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return p.ks > 1 ? cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, true>, a, tmap)
-                    : cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, false>, a, tmap);
+    return cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE>, a, tmap);
 }
 
 }  // namespace
@@ -791,7 +789,11 @@ bool fused_preferred(const Layout& l, int M) {
 #endif
     return M > 64 && gemm_tc_supported(l, M);
 }
-size_t fused_workspace_bytes(const Layout& l, int M) { return gemm_ctrl_bytes(l, M); }
+size_t fused_workspace_bytes(const Layout& l, int M) {
+    const FusedPlan p = plan_fused(l, M);
+    const bool cut = p.dealt && p.dealt * l.SC != p.stream;
+    return fused_ctrl_bytes(l, M) + (cut ? (size_t)p.dealt * 4 * p.T * kCh * 4 : 0);
+}
 
 // c.x: the activations as fp16; or bf16, converted first into x_f16
 cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& call, void* x_f16, cudaStream_t s) {
