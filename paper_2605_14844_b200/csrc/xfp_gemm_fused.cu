@@ -8,17 +8,22 @@
 //            and multiplying from there ran at those 9 TB/s: 4096 x 4096, 100 rows 26 us, 28672 x 8192, 1024 rows 640 us.)
 //   stage    64 k: A = W^ [128 channels][64 k] fp16 in core-matrix order (k / 8, channel, 8), 16 KB; B = the CTA's half of
 //            the rows of x in the 128-byte swizzle, by tensor copies.  2 .. 12 stages in a ring: a stage is in decode for
-//            about 1900 clocks (four of them at once), then 200 for its outliers, then in the products.
-//   warps    16 decode: a stage is decoded by four warps, one per row-block; 64 look-ups per lane, stored as eight 16-byte
-//            vectors.  4 outliers: a lane per channel with the next four entries of its list in registers adds those that
-//            fall into the stage to the stored values, one correctly rounded fp16 addition each, by address (in the decode
-//            warps, where the addition has to find its register by nested tests, it cost as much as the decode).  1 copies,
-//            1 products.  Roles meet at mbarriers only: a stage is "ready" on the first CTA's barrier when the last of both
-//            CTAs' row-blocks are stored and both CTAs' x has landed (the copies of both count their bytes there).
+//            about 1900 clocks (four of them at once), then 300 for its outliers, then in the products.
+//   warps    1 products, 2 copies, 4 outliers, 16 decode.  A stage is decoded by four warps, one per row-block: 64 look-ups per
+//            lane, stored as eight 16-byte vectors.  Outliers: a lane per channel with the next entries of its list in
+//            registers adds those that fall into two stages to the stored values, one correctly rounded fp16 addition each, by
+//            address.  (In the decode warps, in registers, where the register has to be found by nested tests, the same
+//            addition cost as much as the decode; in the decode warps by address it lengthened a stage's decode from 1900 to
+//            3000 clocks, the SM's issue slots being full.)  Roles meet at mbarriers only: a stage is "ready" on the first
+//            CTA's barrier when all row-blocks of both CTAs are stored and the x of both has landed (the copies of both count
+//            their bytes there).
 //   schedule resident pairs.  Whole rounds of tiles run whole tiles; what remains is one stream of super-chunks that is dealt
 //            evenly over the pairs, so a pair ends one tile and begins the next (28672 x 8192, 1024 rows: 4.5 rounds instead of
 //            5; 10007 x 4992, 301 rows: 40 tiles on 74 pairs).  A CTA that had part of a tile leaves fp32 sums in the
 //            workspace; the last to come of a tile adds the parts in order of K.  Nobody waits for another pair.
+//            Where clusters of 2 or 3 pairs on one tile each fit the GPU at once (few tiles), they cut K instead and the sums
+//            meet through distributed shared memory: writing and reading them through L2 takes 9 us at 4096 x 4096, 100 rows
+//            in four parts, the exchange in a cluster of three pairs 3 us.
 //   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
 //            table (D16 = fp16(fp32(scale * lib + mid))); the look-ups are then those of V2.
 // Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace, stops
@@ -36,12 +41,16 @@ constexpr int kCh = 128;                       // channels of a CTA
 constexpr int kStageK = 64;
 constexpr int kABytes = kCh * kStageK * 2;     // A of one stage
 constexpr int kMaxSlots = 12;
-constexpr int kDecodeWarps = 16, kOutWarps = 4;
-constexpr int kCopyWarps = 2, kCopyWarp = kDecodeWarps + kOutWarps, kMmaWarp = kCopyWarp + kCopyWarps;
-constexpr int kThreads = (kMmaWarp + 1) * 32;
+// Warp roles, the short ones first: the scheduler serves older warps first, and behind the decode warps, which can issue in
+// every clock, the others' few instructions waited.
+constexpr int kMmaWarp = 0, kCopyWarp = 1, kCopyWarps = 2, kOutWarp = 4, kOutWarps = 4, kDecodeWarp = 8, kDecodeWarps = 16;
+constexpr int kThreads = (kDecodeWarp + kDecodeWarps) * 32;
 constexpr uint32_t kSpins = 1u << 20, kPollHint = 1000;
 constexpr size_t kSmemMax = 226 * 1024;
 constexpr int kLibEntries = 8192;              // V2a library entries staged in shared memory
+constexpr int kMaxCut = 4;                     // pairs of a cluster
+constexpr int kClusters[kMaxCut + 1] = {0, 74, 33, 22, 15};   // clusters of k pairs that a B200 runs at once (cudaOccupancyMaxActiveClusters:
+                                                              // a cluster stays inside a GPC); more of them run in turn
 constexpr int kPairs = kSizingSMs / 2;         // pairs that the schedule deals to; a device with fewer runs them in turn
 
 struct FusedArgs {
@@ -54,6 +63,7 @@ struct FusedArgs {
     int T, Tp, parts;           // one product instruction covers Tp <= 256 rows, the second T - Tp; both multiples of 32
     int slots, x_bytes;         // stages in the ring; bytes of x per stage and CTA
     int tab_bytes;
+    int ks, sc_slice;           // ks > 1: pairs of a cluster and the super-chunks of each; the schedule below is not used
     int whole;                  // whole tiles per pair; the rest (`stream` super-chunks from tile whole * kPairs on) is dealt
     int stream, dealt;          // evenly to pairs 0 .. dealt - 1
     int tmem_cols;
@@ -124,9 +134,9 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t da, uint64_t 
         :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
 }
 // the products issued so far arrive on the barrier of both CTAs of the pair
-__device__ __forceinline__ void commit_pair(uint32_t bar) {
+__device__ __forceinline__ void commit_pair(uint32_t bar, uint32_t mask) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 :: "r"(bar), "h"((uint16_t)3) : "memory");
+                 :: "r"(bar), "h"((uint16_t)mask) : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
@@ -165,11 +175,17 @@ struct Ring {
 // The i-th piece of work of pair g: super-chunks [sc0, sc1) of a tile.  Pair g has [g S / D, (g + 1) S / D) of the S dealt
 // super-chunks, at most a tile's worth, so at most two pieces.
 struct Piece { int tile, sc0, sc1; };
+template <bool SPLIT>
 __device__ __forceinline__ bool piece_of(const FusedArgs& a, int g, int i, Piece& p) {
+    if (SPLIT) {
+        const int s = g % a.ks;
+        p.tile = g / a.ks; p.sc0 = s * a.sc_slice; p.sc1 = min(a.SC, p.sc0 + a.sc_slice);
+        return i == 0;
+    }
     if (i < a.whole) { p.tile = g + i * kPairs; p.sc0 = 0; p.sc1 = a.SC; return true; }
     i -= a.whole;
     if (g >= a.dealt || i > 1) return false;
-    const int u0 = (int)((long long)g * a.stream / a.dealt), u1 = (int)((long long)(g + 1) * a.stream / a.dealt);
+    const int u0 = g * a.stream / a.dealt, u1 = (g + 1) * a.stream / a.dealt;      // below 74 * 74 * 512
     const int t = u0 / a.SC + i, b = t * a.SC;
     if (u1 <= b) return false;
     p.tile = a.whole * kPairs + t; p.sc0 = u0 > b ? u0 - b : 0; p.sc1 = min(a.SC, u1 - b);
@@ -180,7 +196,7 @@ __device__ __forceinline__ int product_rows(const FusedArgs& a, int p0, int p) {
     return min(p ? a.T - a.Tp : a.Tp, max((a.M - p0 + 31) & ~31, 32));
 }
 // the pair that has dealt super-chunk u: the largest g with g S / D <= u
-__device__ __forceinline__ int dealt_to(const FusedArgs& a, int u) { return (int)(((long long)(u + 1) * a.dealt - 1) / a.stream); }
+__device__ __forceinline__ int dealt_to(const FusedArgs& a, int u) { return ((u + 1) * a.dealt - 1) / a.stream; }
 
 // Decode tables.  kPair: entry t = first index | second index << N holds two fp16 values; else entry q one.  N = 4 entries lie
 // 256 bytes apart (two tables interleaved): an index isolated in its own byte becomes the second byte of the address.
@@ -200,6 +216,14 @@ struct Tab {
                       : base + (uint32_t)u * kOne + (uint32_t)lane * 4u;
     }
 };
+
+// W^ = fp16(D16 + S) in place
+__device__ __forceinline__ void add_outlier(uint32_t addr, uint16_t val) {
+    uint16_t w;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(w) : "r"(addr));
+    w = __half_as_ushort(__hadd(__ushort_as_half(w), __ushort_as_half(val)));
+    asm volatile("st.shared.u16 [%0], %1;" :: "r"(addr), "h"(w) : "memory");
+}
 
 // The 16-byte vectors that hold words [PART * 2N, PART * 2N + 2N) of a lane's 128 * N-bit stream.
 template <int N, int PART>
@@ -239,6 +263,38 @@ __device__ __forceinline__ void fill_tables(const FusedArgs& a, uint32_t tab0, i
         }
     }
 }
+
+// A channel's outliers in ascending column order: transposed slab first, the CSR arrays behind it.
+struct Outliers {
+    const uint32_t* slab;
+    const uint32_t* spill;
+    int nslab, total;
+    __device__ __forceinline__ const uint32_t* addr(int j) const { return j < nslab ? slab + (size_t)(1 + j) * 32 : spill + j; }
+    __device__ __forceinline__ uint32_t at(int j) const { return __ldg(addr(j)); }
+    __device__ __forceinline__ void open(const FusedArgs& a, int rb, int row, int lane) {
+        slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
+        spill = a.b.oent;
+        nslab = total = 0;
+        if (rb < a.RB && row < a.rows) {
+            const int len = (int)__ldg(slab);
+            nslab = total = min(len, a.ell_slots);
+            if (len >= a.ell_slots) {
+                const int p0 = __ldg(a.b.rowptr + row);
+                total = __ldg(a.b.rowptr + row + 1) - p0;
+                spill = a.b.oent + p0;
+            }
+        }
+    }
+    // first entry at or behind column k0: sixteen independent loads at a time (every 16th entry, then the 15 in front of the hit)
+    __device__ __forceinline__ int find(uint32_t k0) const {
+        if (!k0 || !total) return 0;
+        int coarse = 0, fine = 0;
+        for (int j = 15; j < total; j += 16) coarse += (at(j) & 0xffffu) < k0;
+#pragma unroll
+        for (int j = 0; j < 15; ++j) fine += coarse * 16 + j < total && (at(min(coarse * 16 + j, total - 1)) & 0xffffu) < k0;
+        return coarse * 16 + fine;
+    }
+};
 
 struct Bars {
     uint32_t decoded, freed;      // address of slot 0's; slot s is 8 s further
@@ -337,93 +393,56 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
     return true;
 }
 
-// A channel's outliers in ascending column order: transposed slab first, the CSR arrays behind it.
-struct Outliers {
-    const uint32_t* slab;
-    const uint32_t* spill;
-    int nslab, total;
-    __device__ __forceinline__ uint32_t at(int j) const { return __ldg(j < nslab ? slab + (size_t)(1 + j) * 32 : spill + j); }
-    __device__ __forceinline__ void open(const FusedArgs& a, int rb, int row, int lane) {
-        slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
-        spill = a.b.oent;
-        nslab = total = 0;
-        if (rb < a.RB && row < a.rows) {
-            const int len = (int)__ldg(slab);
-            nslab = total = min(len, a.ell_slots);
-            if (len >= a.ell_slots) {
-                const int p0 = __ldg(a.b.rowptr + row);
-                total = __ldg(a.b.rowptr + row + 1) - p0;
-                spill = a.b.oent + p0;
-            }
-        }
-    }
-    // first entry at or behind column k0: sixteen independent loads at a time (every 16th entry, then the 15 in front of the hit)
-    __device__ __forceinline__ int find(uint32_t k0) const {
-        if (!k0 || !total) return 0;
-        int coarse = 0, fine = 0;
-        for (int j = 15; j < total; j += 16) coarse += (at(j) & 0xffffu) < k0;
-#pragma unroll
-        for (int j = 0; j < 15; ++j) fine += coarse * 16 + j < total && (at(min(coarse * 16 + j, total - 1)) & 0xffffu) < k0;
-        return coarse * 16 + fine;
-    }
-};
-
-// W^ = fp16(D16 + S) at weight k (0 .. 63) of channel ch of a stage
-__device__ __forceinline__ void add_outlier(unsigned char* stage, uint32_t k, uint32_t ch, uint16_t val) {
-    uint16_t* w = (uint16_t*)(stage + (k >> 3) * 2048u + ch * 16u + (k & 7u) * 2u);
-    *w = __half_as_ushort(__hadd(__ushort_as_half(*w), __ushort_as_half(val)));
-}
-
-// The outlier warps' share of one tile (matrices with outliers): warp q adds those of row-block q.
-__device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int q, int lane, int st0, int st1, unsigned char* pA,
+// The outlier warps' share of one tile (matrices with outliers): warp q adds those of row-block q, two stages at a time.
+__device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int q, int lane, int sc0, int sc1, uint32_t sA,
                                              const Bars& bars, Ring ring) {
-    constexpr int kAhead = 4;
+    constexpr int kAhead = 6;
     Outliers o;
     o.open(a, rb, rb * kRowsPerBlock + lane, lane);
-    int cur = o.find((uint32_t)st0 * kStageK);
+    int cur = o.find((uint32_t)sc0 * kSuper);
     const bool spills = __any_sync(0xffffffffu, o.total > o.nslab);
+    const uint32_t mine = sA + (uint32_t)(q * 32 + lane) * 16u;
     uint32_t e[kAhead];
-    auto load = [&]() {
+    auto look = [&]() {                     // behind the list's end: an entry that adds +0 to the last weight a row can have
         if (!spills) {
             const uint32_t* p = o.slab + (size_t)(1 + cur) * 32;
 #pragma unroll
-            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? __ldg(p + i * 32) : 0u;
+            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? __ldg(p + i * 32) : 0xffffu;
         } else {
 #pragma unroll
-            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? o.at(cur + i) : 0u;
+            for (int i = 0; i < kAhead; ++i) e[i] = cur + i < o.total ? o.at(cur + i) : 0xffffu;
         }
     };
-    load();
-    for (int st = st0; st < st1; ++st) {
-        const uint32_t end = (uint32_t)(st + 1) * kStageK;
-        unsigned char* mine = pA + (size_t)ring.slot * kABytes + (size_t)(q * 32 + lane) * 16;
-        if (!wait_bar(bars.decoded + 8u * ring.slot, ring.phase)) return false;
+    look();
+    for (int sc = sc0; sc < sc1; ++sc) {
+        Ring on = ring;
+        on.step(1, a.slots);
+        const uint32_t k0 = (uint32_t)sc * kSuper, first = mine + (uint32_t)ring.slot * kABytes, second = mine + (uint32_t)on.slot * kABytes;
+        if (!wait_bar(bars.decoded + 8u * ring.slot, ring.phase) || !wait_bar(bars.decoded + 8u * on.slot, on.phase)) return false;
         for (;;) {
             int n = 0;
-            uint16_t* w[kAhead];
-            uint16_t v[kAhead];
-            bool in[kAhead];
 #pragma unroll
             for (int i = 0; i < kAhead; ++i) {
-                const uint32_t col = e[i] & 0xffffu, k = col & 63u;
-                in[i] = cur + i < o.total && col < end;
-                n += in[i];
-                w[i] = (uint16_t*)(mine + (k >> 3) * 2048u + (k & 7u) * 2u);
-                if (in[i]) v[i] = *w[i];
+                const uint32_t k = (e[i] & 0xffffu) - k0;           // ascending: never below
+                if (k < (uint32_t)kSuper) {
+                    ++n;
+                    add_outlier((k < (uint32_t)kStageK ? first : second) + ((k >> 3) & 7u) * 2048u + (k & 7u) * 2u, (uint16_t)(e[i] >> 16));
+                }
             }
-#pragma unroll
-            for (int i = 0; i < kAhead; ++i)
-                if (in[i]) *w[i] = __half_as_ushort(__hadd(__ushort_as_half(v[i]), __ushort_as_half((uint16_t)(e[i] >> 16))));
             cur += n;
-            if (!__any_sync(0xffffffffu, n == kAhead)) {
+            const bool more = __any_sync(0xffffffffu, n == kAhead && cur < o.total);
+            if (!more) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (elected()) arrive_cluster(bars.ready + 8u * ring.slot);
-                if (n) load();                  // they travel while the next stage is decoded
-                break;
+                if (elected()) {
+                    arrive_cluster(bars.ready + 8u * ring.slot);
+                    arrive_cluster(bars.ready + 8u * on.slot);
+                }
             }
-            if (n) load();
+            if (n) look();                  // they travel while the next stages are decoded
+            if (!more) break;
         }
+        ring = on;
         ring.step(1, a.slots);
     }
     return true;
@@ -447,7 +466,28 @@ __device__ __forceinline__ void store_rows(const FusedArgs& a, int t0, int n, in
     }
 }
 
-template <int N, int MODE>
+// sums of four consecutive channels (from `row` on) of row t of x
+__device__ __forceinline__ void store_quad(const FusedArgs& a, int t, int row, const float4& v) {
+    const size_t o = (size_t)t * a.rows + row;
+    if ((a.rows & 3) == 0 && row < a.rows) {
+        if (a.y_kind == 0) *(float4*)((float*)a.y + o) = v;
+        else if (a.y_kind == 1) {
+            const __half2 lo = __floats2half2_rn(v.x, v.y), hi = __floats2half2_rn(v.z, v.w);
+            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
+        } else {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            *(uint2*)((uint16_t*)a.y + o) = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
+        }
+        return;
+    }
+    if (row < a.rows) put_y(a.y, o, v.x, a.y_kind);
+    if (row + 1 < a.rows) put_y(a.y, o + 1, v.y, a.y_kind);
+    if (row + 2 < a.rows) put_y(a.y, o + 2, v.z, a.y_kind);
+    if (row + 3 < a.rows) put_y(a.y, o + 3, v.w, a.y_kind);
+}
+
+// SPLIT: a cluster of a.ks pairs on one tile, cut along K.
+template <int N, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
     using T = Tab<N, MODE>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -456,14 +496,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail, s_last;
+    __shared__ const float* s_part[kPairs];
     // the warp index through a shuffle: uniform as the compiler sees it, so that the roles run on uniform registers
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const uint32_t h = cluster_rank();                        // half of the pair; CTA 0 issues the products
+    const uint32_t crank = cluster_rank(), h = crank & 1u, lead = crank & ~1u;        // half of the pair; CTA 0 of it issues the products
     const int g = (int)blockIdx.x >> 1;
     unsigned char* pA = smem + a.tab_bytes;
     unsigned char* pB = pA + (size_t)a.slots * kABytes;
     uint16_t* lib = (uint16_t*)(pB + (size_t)a.slots * a.x_bytes);
-    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), 0)};
+    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), lead)};
     asm volatile("griddepcontrol.launch_dependents;");
 
     if (tid < a.slots) {
@@ -494,17 +535,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     Ring ring{0, 0u};
     uint32_t acc_ph = 0;
     Piece pc;
-    if (warp < kDecodeWarps) {
-        const int q = warp & 3, part = (warp >> 2) & 1, grp = warp >> 3;
-        const uint32_t tab = T::at(sa(smem), MODE == 0 ? q : warp, lane);
+    if (warp >= kDecodeWarp) {
+        const int dw = warp - kDecodeWarp, q = dw & 3, part = (dw >> 2) & 1, grp = dw >> 3;
+        const uint32_t tab = T::at(sa(smem), MODE == 0 ? q : dw, lane);
         bool met = false;                                     // has waited for the other CTA's barriers
         int have = -1;                                        // tile of channels whose tables are in place
-        for (int i = 0; piece_of(a, g, i, pc); ++i) {         // a warp whose wait ran out still meets the others at their barrier
+        for (int i = 0; piece_of<SPLIT>(a, g, i, pc); ++i) {         // a warp whose wait ran out still meets the others at their barrier
             const int tx = pc.tile / a.tok_tiles, ty = pc.tile % a.tok_tiles, t0 = ty * a.T;
             const int rb = (2 * tx + (int)h) * 4 + q;
             if (MODE == 0 && tx != have) {
                 decode_sync();                                // every warp is done with the previous tables
-                fill_tables<N>(a, sa(smem), rb - q, warp, lane);
+                fill_tables<N>(a, sa(smem), rb - q, dw, lane);
                 decode_sync();
                 have = tx;
             }
@@ -518,34 +559,39 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             const uint32_t acc = s_tmem + ((uint32_t)(q * 32) << 16);
             const int r = q * 32 + lane, row = (2 * tx + (int)h) * kCh + r;
             const int tend = min(a.T, a.M - t0);
-            const bool whole = pc.sc0 == 0 && pc.sc1 == a.SC;
+            const bool whole = !SPLIT && pc.sc0 == 0 && pc.sc1 == a.SC;
+            // a CTA that has part of a tile: its sums as [t][channel] -- into its idle stages, every product being complete, or
+            // into the workspace
+            float* sums = (float*)pA + r;
+            int g0 = 0, g1 = 0;
             const size_t psize = (size_t)a.T * kCh;
-            if (whole) {
-                if (ok)
-                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
-                        uint32_t v[16];
-                        tmem_ld16(acc + (uint32_t)(c * 16), v);             // the whole warp
+            // part of pair z: its second piece unless its first begins in this tile
+            auto part_at = [&](int z) {
+                const int first = z * a.stream / a.dealt / a.SC;
+                return a.part + ((size_t)(2 * z + (first == pc.tile - a.whole * kPairs ? 0 : 1)) * 2 + h) * psize;
+            };
+            if (!SPLIT && !whole) {
+                const int u0 = (pc.tile - a.whole * kPairs) * a.SC;
+                g0 = dealt_to(a, u0); g1 = dealt_to(a, u0 + a.SC - 1);
+                sums = part_at(g) + r;
+            }
+            if (ok)
+                for (int c = dw >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
+                    uint32_t v[16];
+                    tmem_ld16(acc + (uint32_t)(c * 16), v);             // the whole warp
+                    if (whole) {
                         if (row < a.rows) store_rows(a, t0 + c * 16, min(16, tend - c * 16), row, v);
-                    }
-            } else {
-                const int u0 = (pc.tile - a.whole * kPairs) * a.SC, g0 = dealt_to(a, u0), g1 = dealt_to(a, u0 + a.SC - 1);
-                // part of pair z: its second piece unless its first begins in this tile
-                auto part_at = [&](int z) {
-                    const int first = (int)((long long)z * a.stream / a.dealt) / a.SC;
-                    return a.part + ((size_t)(2 * z + (first == pc.tile - a.whole * kPairs ? 0 : 1)) * 2 + h) * psize + r;
-                };
-                float* mine = part_at(g);
-                if (ok)
-                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
-                        uint32_t v[16];
-                        tmem_ld16(acc + (uint32_t)(c * 16), v);
-                        float* p = mine + (size_t)c * 16 * kCh;
+                    } else {
+                        float* p = sums + (size_t)c * 16 * kCh;
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) __stcg(p + (size_t)j * kCh, __uint_as_float(v[j]));
+                        for (int j = 0; j < 16; ++j) p[(size_t)j * kCh] = __uint_as_float(v[j]);
                     }
+                }
+            if (!SPLIT && !whole) {
                 __threadfence();
+                if (dw < 4 && dw * 32 + lane <= g1 - g0) s_part[dw * 32 + lane] = part_at(g0 + dw * 32 + lane);
                 decode_sync();
-                if (tid == 0) {
+                if (dw == 0 && lane == 0) {
                     int* count = a.ctrl + 1 + 2 * (pc.tile - a.whole * kPairs) + h;
                     const int last = atomicAdd(count, 1) == g1 - g0;
                     if (last) *count = 0;
@@ -553,40 +599,48 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                     __threadfence();
                 }
                 decode_sync();
-                if (s_last && ok && row < a.rows)
-                    for (int c = warp >> 2; c * 16 < tend; c += kDecodeWarps / 4) {
-                        uint32_t sum[16];
+                if (s_last && ok) {
+                    // four channels of a row of x per thread and step, four rows and two parts in flight
+                    constexpr int kRowsIn = 4;
+                    const int ch = lane * 4, orow = (2 * tx + (int)h) * kCh + ch;
+                    for (int t = dw; t < tend; t += kDecodeWarps * kRowsIn) {
+                        float4 sum[kRowsIn];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) sum[j] = 0u;
-                        for (int z = g0; z <= g1; ++z) {
-                            const float* p = part_at(z) + (size_t)c * 16 * kCh;
-                            float v[16];
+                        for (int u = 0; u < kRowsIn; ++u) sum[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+                        for (int z = 0; z <= g1 - g0; ++z) {
+                            const float* p = s_part[z] + (size_t)t * kCh + ch;
+                            float4 v[kRowsIn];
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) v[j] = __ldcg(p + (size_t)j * kCh);
+                            for (int u = 0; u < kRowsIn; ++u)      // rows behind the last one exist in the part as well
+                                v[u] = __ldcg((const float4*)(p + (size_t)(t + u * kDecodeWarps < tend ? u * kDecodeWarps : 0) * kCh));
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) sum[j] = __float_as_uint(z == g0 ? v[j] : __uint_as_float(sum[j]) + v[j]);
+                            for (int u = 0; u < kRowsIn; ++u) { sum[u].x += v[u].x; sum[u].y += v[u].y; sum[u].z += v[u].z; sum[u].w += v[u].w; }
                         }
-                        store_rows(a, t0 + c * 16, min(16, tend - c * 16), row, sum);
+#pragma unroll
+                        for (int u = 0; u < kRowsIn; ++u)
+                            if (t + u * kDecodeWarps < tend) store_quad(a, t0 + t + u * kDecodeWarps, orow, sum[u]);
                     }
+                }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             if (!met) { cluster_wait(); met = true; }
             __syncwarp();
-            if (elected()) arrive_cluster(peer(sa(&acc_empty), 0));
+            if (elected()) arrive_cluster(peer(sa(&acc_empty), lead));
         }
-    } else if (warp < kCopyWarp) {
-        const int q = warp - kDecodeWarps;
+    } else if (warp >= kOutWarp) {
+        const int q = warp - kOutWarp;
         cluster_wait();
         if (a.ell_slots)
-            for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
-                ok = outlier_tile(a, (2 * (pc.tile / a.tok_tiles) + (int)h) * 4 + q, q, lane, 2 * pc.sc0, 2 * pc.sc1, pA, bars, ring);
+            for (int i = 0; ok && piece_of<SPLIT>(a, g, i, pc); ++i) {
+                ok = outlier_tile(a, (2 * (pc.tile / a.tok_tiles) + (int)h) * 4 + q, q, lane, pc.sc0, pc.sc1, sa(pA), bars, ring);
                 ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
             }
-    } else if (warp < kMmaWarp) {
+    } else if (warp >= kCopyWarp && warp < kCopyWarp + kCopyWarps) {
         cluster_wait();
         asm volatile("griddepcontrol.wait;" ::: "memory");    // x may come from the previous kernel of the stream
         int n = warp - kCopyWarp;                             // the two warps take the stages in turn
-        for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
+        for (int i = 0; ok && piece_of<SPLIT>(a, g, i, pc); ++i) {
             const int t0 = (pc.tile % a.tok_tiles) * a.T;
             for (int st = 2 * pc.sc0; st < 2 * pc.sc1; ++st, ring.step(1, a.slots)) {
                 if (n++ & 1) continue;
@@ -605,14 +659,18 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 __syncwarp();
             }
         }
-    } else if (h == 1) {
+    } else if (h == 1 || warp != kMmaWarp) {
         cluster_wait();                                       // the first CTA issues the pair's products
     } else {
         const uint64_t da0 = desc_a(sa(pA)), db0 = desc_b(sa(pB));
+        const uint32_t mask = 3u << lead;
         cluster_wait();
         const uint32_t tmem = s_tmem;
-        for (int i = 0; ok && piece_of(a, g, i, pc); ++i) {
+        for (int i = 0; ok && piece_of<SPLIT>(a, g, i, pc); ++i) {
             const int t0 = (pc.tile % a.tok_tiles) * a.T, st1 = 2 * pc.sc1;
+            const uint32_t id = (1u << 4) | ((uint32_t)(2 * kCh >> 4) << 24);
+            const uint32_t id0 = id | ((uint32_t)(product_rows(a, t0, 0) >> 3) << 17);
+            const uint32_t id1 = a.parts > 1 && t0 + a.Tp < a.M ? id | ((uint32_t)(product_rows(a, t0 + a.Tp, 1) >> 3) << 17) : 0u;
             if (i) {
                 ok = wait_bar(sa(&acc_empty), acc_ph);        // the previous piece's sums have been read
                 acc_ph ^= 1u;
@@ -625,22 +683,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 if (!there && !(ok = wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 Ring on = ring;
-                on.step(1, a.slots);
+                if (++on.slot == a.slots) { on.slot = 0; on.phase ^= 1u; }
                 there = st + 1 < st1 && test_bar(bars.ready + 8u * on.slot, on.phase);     // the answer comes under the products
                 if (elected()) {
-                    const uint64_t da = da0 + (uint64_t)((uint32_t)ring.slot * (kABytes >> 4));
-                    uint64_t db = db0 + (uint64_t)((uint32_t)(ring.slot * a.x_bytes) >> 4);
-                    for (int p = 0; p < a.parts; ++p, db += (uint64_t)(a.Tp * 4)) {
-                        const int p0 = t0 + p * a.Tp;
-                        if (p0 >= a.M) break;
-                        const int n = product_rows(a, p0, p);
-                        const uint32_t idesc = (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * kCh >> 4) << 24);
+                    const uint64_t da = da0 + (uint64_t)((uint32_t)ring.slot * (kABytes >> 4)), db = db0 + (uint64_t)((uint32_t)(ring.slot * a.x_bytes) >> 4);
 #pragma unroll
-                        for (int k = 0; k < kStageK / 16; ++k)
-                            mma_pair(tmem + (uint32_t)(p * a.Tp), da + k * 256, db + k * 2, idesc, k ? 1u : acc);
+                    for (int k = 0; k < kStageK / 16; ++k) mma_pair(tmem, da + k * 256, db + k * 2, id0, k ? 1u : acc);
+                    if (id1) {
+                        const uint64_t db1 = db + (uint64_t)(a.Tp * 4);
+#pragma unroll
+                        for (int k = 0; k < kStageK / 16; ++k) mma_pair(tmem + (uint32_t)a.Tp, da + k * 256, db1 + k * 2, id1, k ? 1u : acc);
                     }
-                    commit_pair(bars.freed + 8u * ring.slot);
-                    if (st + 1 == st1) commit_pair(sa(&acc_full));
+                    commit_pair(bars.freed + 8u * ring.slot, mask);
+                    if (st + 1 == st1) commit_pair(sa(&acc_full), mask);
                 }
                 acc = 1;
                 __syncwarp();
@@ -656,6 +711,34 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     __syncwarp();
     cluster_sync();
+    if (SPLIT) {
+        // this CTA's share of the rows of x of its 128 channels: the slices' sums added in slice order
+        const int tile = g / a.ks, slice = g % a.ks, t0 = (tile % a.tok_tiles) * a.T, Tn = min(a.T, a.M - t0);
+        const int share = (Tn + a.ks - 1) / a.ks, b0 = slice * share * (kCh / 4), b1 = min(Tn, (slice + 1) * share) * (kCh / 4);
+        const uint32_t own = sa(pA);
+        for (int i0 = b0 + tid; i0 < b1; i0 += 2 * kThreads) {
+            float4 v[2][kMaxCut];                             // two places, every slice's share in flight
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int z = 0; z < kMaxCut; ++z)
+                    if (z < a.ks && i0 + u * kThreads < b1)
+                        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[u][z].x), "=f"(v[u][z].y), "=f"(v[u][z].z), "=f"(v[u][z].w)
+                                     : "r"(peer(own + (uint32_t)(i0 + u * kThreads) * 16u, 2u * (uint32_t)z + h)));
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = i0 + u * kThreads;
+                if (i >= b1) break;
+                float4 sum = v[u][0];
+#pragma unroll
+                for (int z = 1; z < kMaxCut; ++z)
+                    if (z < a.ks) { sum.x += v[u][z].x; sum.y += v[u][z].y; sum.z += v[u][z].z; sum.w += v[u][z].w; }
+                store_quad(a, t0 + i / (kCh / 4), (2 * (tile / a.tok_tiles) + (int)h) * kCh + (i % (kCh / 4)) * 4, sum);
+            }
+        }
+        __syncwarp();
+        cluster_sync();          // no CTA leaves while another reads its shared memory
+    }
     if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(s_tmem), "r"(a.tmem_cols) : "memory");
 }
@@ -674,17 +757,20 @@ EncodeTiledFn encode_fn() {
 // ------------------------------------------------------------------ plan
 
 struct FusedPlan {
-    int T, Tp, parts, tok_tiles, pairs, slots, whole, stream, dealt;
+    int T, Tp, parts, tok_tiles, pairs, slots, whole, stream, dealt, ks, sc_slice;
     size_t tab, lib, smem;
     double clocks;             // what the model expects
 };
 
-// Clocks of a tile's super-chunk: the products (4 T), the decode of 128 x 128 weights, or the operands' way from L2 (the
-// index stream and the CTA's half of x at about 40 bytes per clock).
+// Clocks of a tile's super-chunk: the products (4 T), or shared memory, which every byte crosses at 128 per clock -- per 64 k
+// the look-ups of 4 warps (one wavefront each, half with pair tables), V2a's tables, 128 for storing A, 128 for the products'
+// reading it, T / 2 for x coming in and T / 2 for its being read --, or the operands' way from L2.
 double slot_clocks(const Layout& l, int T) {
-    const double products = 4.0 * T, decode = l.mode ? (l.bits >= 5 ? 1700.0 : 1250.0) : (l.bits >= 5 ? 1200.0 : 1000.0);
-    const double feed = (l.bits * 2048.0 + 128.0 * T) / 40.0;
-    const double m = products > decode ? products : decode;
+    const bool pair = l.mode ? l.bits == 2 : l.bits <= 3;
+    const double smem = 2.0 * ((pair ? 128 : 256) + (l.mode ? (l.bits == 2 ? 64 : 4 * l.E) : 0) + 256 + T) * 1.08;
+    const double products = 4.0 * T, feed = (l.bits * 2048.0 + 128.0 * T) / 40.0, issue = 1250.0;
+    double m = products > smem ? products : smem;
+    if (m < issue) m = issue;
     return m > feed ? m : feed;
 }
 
@@ -712,19 +798,31 @@ FusedPlan plan_fused(const Layout& l, int M) {
         if (slots < 2) continue;
         // a stage's way through decode, outliers and products takes about 2900 clocks and its share of the products
         const double chain = (2900.0 + 2.0 * T) / slots * 2.0, busy = slot_clocks(l, T), step = busy > chain ? busy : chain;
-        const double move = T * 512.0 / 40.0;                  // a CTA's sums to or from the workspace
+        // a CTA's sums to or from the workspace at 40 bytes a clock, and all of them through DRAM at 2 KB a clock (10007 x 4992,
+        // 301 rows, dealt over 74 pairs: 83 us, 23 MB of sums; 40 whole tiles 60 us)
+        const double move = T * 512.0 / 40.0, dram = T * 1024.0 / 2000.0;
         const int tiles = pairs * tok, whole = tiles / kPairs, rest = tiles - whole * kPairs;
         const double rounds = whole * (l.SC * step + 1500.0 + 10.0 * T);
-        for (int k = 1; k <= 9 && rest * (k > 8 ? 1 : k) <= kPairs; ++k) {     // every remaining tile in k parts; or an even deal
+        for (int k = 1; k <= 9; ++k) {     // every remaining tile in k parts; or an even deal
             const int dealt = rest == 0 ? 0 : k > 8 ? kPairs : rest * k, stream = rest * l.SC;
-            if (rest && (dealt > stream / 2 && k > 1)) continue;  // a part has at least two super-chunks
+            if (k > 1 && (dealt > kPairs || dealt > stream / 2)) continue;  // a part has at least two super-chunks
             const int most = rest ? (stream + dealt - 1) / dealt : 0, cuts = k == 1 ? 1 : k > 8 ? (l.SC - 1) / most + 2 : k;
-            const double clocks = rounds + (rest ? most * step + 1500.0 + 10.0 * T + (k > 8 ? 2000.0 : 0.0) : 0.0) + (cuts > 1 ? 3000.0 + cuts * move : 0.0);
+            const double clocks = rounds + (rest ? most * step + 1500.0 + 10.0 * T + (k > 8 ? 2000.0 : 0.0) : 0.0) + (cuts > 1 ? 6000.0 + cuts * move + 2.0 * dealt * dram : 0.0);
             if (best.clocks == 0.0 || clocks < best.clocks) {
                 best.T = T; best.Tp = Tp; best.parts = parts; best.tok_tiles = tok; best.pairs = pairs; best.slots = slots;
-                best.whole = whole; best.stream = stream; best.dealt = dealt; best.clocks = clocks;
+                best.whole = whole; best.stream = stream; best.dealt = dealt; best.ks = 1; best.sc_slice = 0; best.clocks = clocks;
             }
             if (!rest) break;
+        }
+        for (int ks = 2; ks <= kMaxCut; ++ks) {
+            const int spp = (l.SC + ks - 1) / ks;
+            if ((ks - 1) * spp >= l.SC || spp < 2 || (size_t)T * kCh * 4 > slots * (kABytes + (size_t)parts * Tp * 64) || tiles > kClusters[ks]) continue;
+            const double clocks = spp * step + 1500.0 + 4500.0 + 20.0 * T;
+            if (clocks < best.clocks) {
+                best = FusedPlan{};
+                best.T = T; best.Tp = Tp; best.parts = parts; best.tok_tiles = tok; best.pairs = pairs; best.slots = slots;
+                best.ks = ks; best.sc_slice = spp; best.clocks = clocks;
+            }
         }
     }
     best.tab = tab; best.lib = lib;
@@ -754,7 +852,8 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        const cudaError_t e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        cudaError_t e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_fused_kernel<N, MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
@@ -764,21 +863,22 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L; a.y_kind = c.y_kind;
     a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
     a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
-    a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
+    a.ks = p.ks; a.sc_slice = p.sc_slice; a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
     a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * (p.whole ? kPairs : p.dealt)), 1, 1);
+    cfg.gridDim = dim3((unsigned)(2 * (p.ks > 1 ? p.pairs * p.tok_tiles * p.ks : p.whole ? kPairs : p.dealt)), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = (unsigned)(2 * p.ks); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE>, a, tmap);
+    return p.ks > 1 ? cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, true>, a, tmap)
+                    : cudaLaunchKernelEx(&cfg, gemm_fused_kernel<N, MODE, false>, a, tmap);
 }
 
 }  // namespace

@@ -158,6 +158,29 @@ def test_gemm_more_tiles_than_sms(mode, bits, m):
         assert np.all(err <= TOL * absum[:, r0:r1] + 1e-30), (r0, float((err / (absum[:, r0:r1] + 1e-300)).max()))
 
 
+@pytest.mark.parametrize("mode,bits,rows,cols,m,placement", [
+    (0, 4, 255, 128, 65, "uniform"),        # one super-chunk, a pair whose second CTA lacks a channel
+    (0, 3, 257, 384, 96, "one_row"),        # a second pair of one channel; K too short to cut evenly
+    (1, 2, 129, 896, 288, "clustered"),     # two products of 160 and 128 rows
+    (0, 5, 512, 1664, 481, "uniform"),      # two products of 256 rows, the last rows of x missing
+    (1, 5, 300, 256, 513, "uniform"),       # two tiles along x, the second nearly empty
+    (0, 6, 20000, 256, 65, "clustered"),    # more tiles than pairs, two super-chunks each
+    (0, 2, 9500, 1152, 600, "uniform")])    # rounds of whole tiles and a dealt rest along x as well
+def test_gemm_on_pairs_of_sms(mode, bits, rows, cols, m, placement):
+    """The pair kernel (more than 64 rows of x) at the edges of its tiles, of its products and of its schedule; a second call
+    over the same workspace gives the same bits.  Tolerances as for every other shape (see _check)."""
+    q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=1400 + rows + m, placement=placement)
+    pm = xfp.pack_tensors(q, col_bits=16)
+    x16 = synth.activations(m, cols, seed=1410 + m)
+    y = _check(q, pm, x16)
+    xd = torch.from_numpy(x16.view(np.int16)).cuda().view(torch.float16)
+    _, ws, _ = _run(q, pm, x16)
+    y2 = torch.full_like(y, float("nan"))
+    xfp.xfp_gemm(pm.desc, pm.packed, xd, y2, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(y, y2) and int(ws[:4].view(torch.int32).item()) == 0
+
+
 def test_gemm_matches_gemv_rows_and_is_deterministic():
     q = synth.random_quantized(0, 512, 4096, 4, 0.01, seed=41)
     pm = xfp.pack_tensors(q)
