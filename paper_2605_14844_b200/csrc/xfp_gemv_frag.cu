@@ -1,0 +1,365 @@
+// Fused decode for 1..16 rows of x, V2 and V2a, in the tensor cores' own operand layout:  y[b] = (D + S) x[b].
+//
+// The lane kernels (xfp_gemv_lane.cuh, xfp_gemv_pair.cu, xfp_gemv_batch.cu) keep a channel's decoded weights in one lane, so x
+// has to sit on the diagonal lanes of the B operand and every row of x costs an mma and two shared-memory wavefronts per 8
+// weights of a lane.  Here lane (g, t) of a warp, g = lane / 4, t = lane mod 4, takes the t-th 32 of a super-chunk's 128
+// weights of the four channels g, g + 8, g + 16, g + 24 of a row-block.  That is the A operand of mma.m16n8k16 as it stands --
+// the order of k inside a super-chunk is free, and step s multiplies the k 32 t + 4 s .. + 3 of every t -- so one mma serves
+// eight rows of x, a lane's share of x is 16 consecutive bytes of one row (four wavefronts per super-chunk and row pair, none
+// wasted), and an accumulator holds four channels' sums: V2a's scale and mid-point are applied in place, without a shuffle.
+//
+//   look-ups  four lanes share a channel, so a table is kept in four copies, one per t: entry (..)*128 + lane*4 lies in the
+//             lane's own bank.  V2: pair tables up to N = 4 (128 KB of four channels' tables at N = 4), one entry per index
+//             above.  V2a: the library once per bank, two library ids to a word.
+//   x         staged once per CTA (fp16; bf16 is converted on the way) as 16-byte chunks, chunk c of row b at place
+//             c * NB + b with bits 1, 2 of the place exclusive-or'ed with c / 4 mod 4: the eight lanes of a quarter-warp and the
+//             staging threads meet eight different bank groups.  CTAs are resident and walk the row-blocks, so that x is staged
+//             once; a K too long for shared memory is cut into slices, a CTA staying in its slice.
+//   outliers  a lane per channel, slots of the transposed slab dealt to the warps; NB products per entry.
+//   sums      fragments -> shared memory -> fixed order over the warps; K slices meet in the workspace, the last to come adds
+//             them in order (a ticket, no waiting).
+#include "xfp_internal.h"
+#include "xfp_pair_common.cuh"
+
+namespace xfp {
+
+namespace {
+
+constexpr int kFW = 16;              // warps
+constexpr int kFThreads = kFW * 32;
+constexpr size_t kFSmem = 224 * 1024;
+
+struct FragArgs {
+    Blob b;
+    const uint16_t* x;
+    void* y;
+    float* partial;   // [row-block][slice][NB][32]
+    int* tickets;     // [row-block]
+    int rows, cols, RB, SC, ell_slots, L;
+    int nb, y_kind, x_bf16;
+    int S, sc_slice;  // K slices, super-chunks of each
+    int x_off, red_off;   // bytes behind the tables: staged x, per-warp sums
+};
+
+// Tables: V2 [4][entries][32 lanes] words (entry = pair of indices up to N = 4); V2a [ceil(L / 2)][2^N][32] words of two fp16.
+template <int N, int MODE>
+struct FTab {
+    static constexpr int E = 1 << N;
+    static constexpr bool kPair = MODE == 0 && N <= 4;
+    static constexpr int kEntries = kPair ? E * E : E;
+    static constexpr int kOne = kEntries * 128;        // bytes of one channel group's tables
+};
+
+// The lane's words [t N, (t + 1) N) of the index streams of its four channels of super-chunk sc.
+template <int N>
+__device__ __forceinline__ void load_words(uint32_t (&w)[4][N], const uint4* idx, int g, int t) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int ch = g + 8 * j;
+        if (N == 4) {
+            const uint4 v = ld_stream(idx + t * 32 + ch);
+            w[j][0] = v.x; w[j][1] = v.y; w[j][2 % N] = v.z; w[j][3 % N] = v.w;
+        } else if (N % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                const int wd = t * N + 2 * i;
+                const uint2 v = __ldg((const uint2*)(idx + (wd >> 2) * 32 + ch) + ((wd >> 1) & 1));
+                w[j][(2 * i) % N] = v.x; w[j][(2 * i + 1) % N] = v.y;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int wd = t * N + i;
+                w[j][i] = __ldg((const uint32_t*)(idx + (wd >> 2) * 32 + ch) + (wd & 3));
+            }
+        }
+    }
+}
+
+// byte offset of the 16-byte chunk c (8 k) of row b in the staged x
+template <int NB>
+__device__ __forceinline__ uint32_t x_chunk(int c, int b) {
+    return (uint32_t)((c * NB + b) ^ (((c >> 2) & 3) << 1)) << 4;
+}
+
+template <int N, int MODE, int NB>
+__global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs a) {
+    using T = FTab<N, MODE>;
+    constexpr int E = T::E;
+    constexpr int NT = NB > 8 ? 2 : 1;                 // tiles of eight rows of x
+    constexpr int kAhead = N <= 4 ? 2 : 1;             // super-chunks of indices in flight per warp
+    extern __shared__ __align__(1024) unsigned char smem[];
+    unsigned char* sX = smem + a.x_off;
+    float* red = (float*)(smem + a.red_off);           // [warp][NB][33]
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int slice = (int)blockIdx.x % a.S;
+    const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), nsc = sc1 - sc0;
+    float* sXg = (float*)(sX + (size_t)nsc * kSuper * NB * 2);      // V2a: sums of x over a group, [super-chunk][NB]
+    const int step = (int)gridDim.x / a.S;
+
+    auto fill = [&](int rb) {                          // the tables of row-block rb (V2)
+        const int ch = lane, j = ch >> 3;
+        const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + ch) * E;
+        unsigned char* dst = smem + (size_t)j * T::kOne + (ch & 7) * 16;
+        if (T::kPair) {
+            // a thread takes a channel and every sixteenth entry; one 16-byte store writes the four copies
+            uint32_t v[E];
+#pragma unroll
+            for (int e = 0; e < E; e += 4) {
+                const uint2 p = __ldg((const uint2*)(cb + e));
+                v[e] = p.x & 0xffffu; v[e + 1] = p.x >> 16; v[e + 2] = p.y & 0xffffu; v[e + 3] = p.y >> 16;
+            }
+#pragma unroll
+            for (int hi = 0; hi < E; ++hi) {
+                if (hi != warp % (E < kFW ? E : kFW)) continue;
+#pragma unroll
+                for (int lo = 0; lo < E; ++lo) {
+                    if (E < kFW && (lo % (kFW / E)) != warp / E) continue;
+                    const uint32_t p = v[lo] | (v[hi] << 16);
+                    *(uint4*)(dst + (size_t)(lo | (hi << N)) * 128) = make_uint4(p, p, p, p);
+                }
+            }
+        } else {
+            for (int e = warp; e < E; e += kFW) {
+                const uint32_t p = __ldg(cb + e);
+                *(uint4*)(dst + (size_t)e * 128) = make_uint4(p, p, p, p);
+            }
+        }
+    };
+    // indices (and V2a metadata) of the warp's next super-chunks
+    uint32_t nx[kAhead][4][N];
+    uint32_t id_n[kAhead][4], sm_n[kAhead][4];
+    auto fetch = [&](int rb, int sc, int slot) {
+        load_words<N>(nx[slot], a.b.idx + ((size_t)rb * a.SC + sc) * N * 32, g, t);
+        if (MODE == 1) {
+            const size_t m = ((size_t)rb * a.SC + sc) * 32 + g;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { id_n[slot][j] = __ldg(a.b.gid + m + 8 * j); sm_n[slot][j] = __ldg(a.b.gsm + m + 8 * j); }
+        }
+    };
+
+    // ---- what does not depend on the previous kernel: indices, tables ----
+    asm volatile("griddepcontrol.launch_dependents;");
+    int rb = (int)blockIdx.x / a.S;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+        if (rb < a.RB && sc0 + warp + i * kFW < sc1) fetch(rb, sc0 + warp + i * kFW, i);
+    if (MODE == 1) {
+        const int words = (a.L + 1) / 2 * E;
+        for (int i = warp; i < words; i += kFW) {
+            const int id = i / E * 2, q = i % E;
+            const uint32_t lo = __ldg(a.b.cb + id * E + q), hi = id + 1 < a.L ? (uint32_t)__ldg(a.b.cb + (id + 1) * E + q) : 0u;
+            ((uint32_t*)smem)[i * 32 + lane] = lo | (hi << 16);
+        }
+    } else if (rb < a.RB) {
+        fill(rb);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // ---- x: chunks of a row by consecutive threads ----
+    {
+        const int chunks = nsc * (kSuper / 8);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            for (int c = tid; c < chunks; c += kFThreads) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (b < a.nb) v = x8_as_f16(__ldg((const uint4*)(a.x + (size_t)b * a.cols + (size_t)sc0 * kSuper) + c), a.x_bf16);
+                *(uint4*)(sX + x_chunk<NB>(c, b)) = v;
+            }
+        }
+    }
+    __syncthreads();
+    if (MODE == 1) {
+        for (int i = tid; i < nsc * NB; i += kFThreads) {
+            const int sc = i / NB, b = i % NB;
+            float sum = 0.f;
+#pragma unroll 4
+            for (int c = 0; c < kSuper / 8; ++c) {
+                const uint4 v = *(const uint4*)(sX + x_chunk<NB>(sc * (kSuper / 8) + c, b));
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { const float2 f = __half22float2(*(const __half2*)&u[k]); sum += f.x + f.y; }
+            }
+            sXg[i] = sum;
+        }
+        __syncthreads();
+    }
+
+    const uint32_t lbase = (uint32_t)lane * 4u;
+    for (bool later = false; rb < a.RB; rb += step, later = true) {
+        if (later) {
+            __syncthreads();                           // tables and sums of the previous row-block are done with
+            if (MODE == 0) { fill(rb); __syncthreads(); }
+        }
+        float acc[NT][2][4];
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[n][i >> 2][i & 3] = 0.f;
+        for (int sc = sc0 + warp; sc < sc1; sc += kFW) {
+            uint32_t w[4][N + 1];
+            uint32_t base[4];
+            float scale[4], mid[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                for (int i = 0; i < N; ++i) w[j][i] = nx[0][j][i];
+                w[j][N] = 0u;
+                if (MODE == 1) {
+                    const __half2 sm = *(const __half2*)&sm_n[0][j];
+                    scale[j] = __low2float(sm); mid[j] = __high2float(sm);
+                    base[j] = (id_n[0][j] >> 1) * (uint32_t)(E * 128) + lbase + (id_n[0][j] & 1u) * 2u;
+                }
+#pragma unroll
+                for (int s = 0; s + 1 < kAhead; ++s) {
+#pragma unroll
+                    for (int i = 0; i < N; ++i) nx[s][j][i] = nx[s + 1][j][i];
+                    id_n[s][j] = id_n[s + 1][j]; sm_n[s][j] = sm_n[s + 1][j];
+                }
+            }
+            if (sc + kAhead * kFW < sc1) fetch(rb, sc + kAhead * kFW, kAhead - 1);
+            const int lsc = sc - sc0;
+            float c[NT][2][4];
+            if (MODE == 1) {
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) c[n][i >> 2][i & 3] = 0.f;
+            }
+            float(&d)[NT][2][4] = MODE == 1 ? c : acc;
+#pragma unroll
+            for (int s2 = 0; s2 < 4; ++s2) {           // two mma steps: 8 k of every t
+                uint4 xb[NT];
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    xb[n] = make_uint4(0u, 0u, 0u, 0u);
+                    if (NB >= 8 || g < NB) xb[n] = *(const uint4*)(sX + x_chunk<NB>(lsc * 16 + 4 * t + s2, g + 8 * n));
+                }
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const int p0 = 4 * s2 + 2 * s;     // pairs p0, p0 + 1 of the lane's 16
+                    uint32_t av[4][2];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            if (T::kPair) {
+                                av[j][u] = *(const uint32_t*)(smem + j * T::kOne + pair_addr<N, 1>(w[j], p0 + u, lbase));
+                            } else if (MODE == 0) {
+                                const uint32_t lo = *(const uint32_t*)(smem + j * T::kOne + single_addr<N, 1>(w[j], 2 * (p0 + u), lbase));
+                                const uint32_t hi = *(const uint32_t*)(smem + j * T::kOne + single_addr<N, 1>(w[j], 2 * (p0 + u) + 1, lbase));
+                                av[j][u] = lo | (hi << 16);
+                            } else {
+                                const uint32_t lo = *(const uint16_t*)(smem + (single_addr<N, 1>(w[j], 2 * (p0 + u), 0u) + base[j]));
+                                const uint32_t hi = *(const uint16_t*)(smem + (single_addr<N, 1>(w[j], 2 * (p0 + u) + 1, 0u) + base[j]));
+                                av[j][u] = lo | (hi << 16);
+                            }
+                        }
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) {
+                        const uint32_t b0 = s ? xb[n].z : xb[n].x, b1 = s ? xb[n].w : xb[n].y;
+                        mma16816(d[n][0], av[0][0], av[1][0], av[0][1], av[1][1], b0, b1);
+                        mma16816(d[n][1], av[2][0], av[3][0], av[2][1], av[3][1], b0, b1);
+                    }
+                }
+            }
+            if (MODE == 1) {
+                // accumulator element e of tile i: channel g + 8 (e / 2) + 16 i, row of x 2 t + e mod 2
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    const int b = 2 * t + 8 * n;
+                    float x0 = 0.f, x1 = 0.f;
+                    if (b < NB) x0 = sXg[lsc * NB + b];
+                    if (b + 1 < NB) x1 = sXg[lsc * NB + b + 1];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int j = 2 * i + (e >> 1);
+                            acc[n][i][e] = fmaf(scale[j], c[n][i][e], fmaf(mid[j], (e & 1) ? x1 : x0, acc[n][i][e]));
+                        }
+                }
+            }
+        }
+        // the first super-chunks of the next row-block travel while this one is finished
+        if (rb + step < a.RB) {
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i)
+                if (sc0 + warp + i * kFW < sc1) fetch(rb + step, sc0 + warp + i * kFW, i);
+        }
+        // ---- outliers: lane = channel ----
+        float ao[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) ao[b] = 0.f;
+        if (a.ell_slots) {
+            const int row = rb * kRowsPerBlock + lane;
+            const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
+            const int len = (int)__ldg(slab), nslab = min(len, a.ell_slots);
+            const uint32_t k0 = (uint32_t)sc0 * kSuper, kn = (uint32_t)nsc * kSuper;
+            auto add = [&](uint32_t e) {
+                const uint32_t k = (e & 0xffffu) - k0;
+                if (k < kn) {
+                    const float v = h2f((uint16_t)(e >> 16));
+                    const int c = (int)(k >> 3);
+                    const unsigned char* p = sX + (k & 7u) * 2u;
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) ao[b] = fmaf(v, h2f(*(const uint16_t*)(p + x_chunk<NB>(c, b))), ao[b]);
+                }
+            };
+            const int most = __reduce_max_sync(0xffffffffu, nslab);
+            for (int j0 = warp; j0 < most; j0 += 4 * kFW) {
+                uint32_t e[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) e[i] = j0 + i * kFW < nslab ? __ldg(slab + (size_t)(1 + j0 + i * kFW) * 32) : 0u;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) if (j0 + i * kFW < nslab) add(e[i]);
+            }
+            if (len >= a.ell_slots && row < a.rows) {  // the channel overflows its slab: the rest is in the CSR arrays
+                const int p1 = __ldg(a.b.rowptr + row + 1);
+                for (int p = __ldg(a.b.rowptr + row) + a.ell_slots + warp; p < p1; p += kFW) add(__ldg(a.b.oent + p));
+            }
+        }
+        // ---- sums over the warps ----
+        float* mine = red + (size_t)warp * NB * 33;
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int b = 2 * t + 8 * n + (e & 1);
+                    if (b < NB) mine[b * 33 + g + 8 * (2 * i + (e >> 1))] = acc[n][i][e];
+                }
+        __syncwarp();
+        if (a.ell_slots) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) mine[b * 33 + lane] += ao[b];
+        }
+        __syncthreads();
+        float sum = 0.f;
+        const int b = tid >> 5, row = rb * kRowsPerBlock + lane;
+        if (b < a.nb) {
+#pragma unroll
+            for (int w = 0; w < kFW; ++w) sum += red[(w * NB + b) * 33 + lane];
+        }
+        if (a.S == 1) {
+            if (b < a.nb && row < a.rows) put_y(a.y, (size_t)b * a.rows + row, sum, a.y_kind);
+        } else {
+            float* part = a.partial + ((size_t)rb * a.S * NB + b) * 32 + lane;
+            if (b < a.nb) __stcg(part + (size_t)slice * NB * 32, sum);
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                s_last = atomicAdd(a.tickets + rb, 1) == a.S - 1;
+                if (s_last) a.tickets[rb] = 0;
+                __threadfence();
+            }
+            __syncthreads();
+            if (s_last && b < a.nb && row < a.rows) {
+                sum = 0.f;
+                for (int s = 0; s < a.S; ++s) sum += __ldcg(part + (size_t)s * NB * 32);
+                put_y(a.y, (size_t)b * a.rows + row, sum, a.y_kind);
+            }
+        }
+    }
+}
