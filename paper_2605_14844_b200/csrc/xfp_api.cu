@@ -76,7 +76,9 @@ int gemv_common(const xfp_desc* desc, int want_mode, const GemvCall& c, void* st
         e = launch_gemv_v2a(l, cc, (cudaStream_t)stream);
         return e == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
     }
-    if (lane_supported(l, cc))
+    if (frag_supported(l, cc))
+        e = launch_gemv_frag(l, cc, (cudaStream_t)stream);
+    else if (lane_supported(l, cc))
         e = launch_gemv_lane(l, cc, (cudaStream_t)stream);
     else if (lane_batch_supported(l, cc))
         e = launch_gemv_lane_batch(l, cc, (cudaStream_t)stream);

@@ -363,3 +363,114 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
         }
     }
 }
+
+struct FragPlan { int S, sc_slice, grid; size_t x_off, red_off, smem; };
+
+size_t table_bytes(const Layout& l) {
+    if (l.mode) return (size_t)((l.L + 1) / 2) * l.E * 128;
+    return (size_t)4 * (l.bits <= 4 ? l.E * l.E : l.E) * 128;
+}
+
+int rows_of(int batch) { return batch <= 1 ? 1 : batch <= 2 ? 2 : batch <= 4 ? 4 : batch <= 8 ? 8 : 16; }
+
+bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
+    const int NB = rows_of(batch);
+    const size_t tab = table_bytes(l), red = (size_t)kFW * NB * 33 * 4 + 16;
+    const size_t per_sc = (size_t)kSuper * NB * 2 + (l.mode ? NB * 4 : 0);
+    if (tab + red + per_sc > kFSmem) return false;
+    const int fit = (int)((kFSmem - tab - red) / per_sc);             // super-chunks of x that fit
+    int S = (l.SC + fit - 1) / fit;
+    // few row-blocks: K slices until the SMs are busy, at least one super-chunk per warp
+    while (l.RB * (S + 1) <= sms && l.SC / (S + 1) >= kFW) ++S;
+    p.sc_slice = (l.SC + S - 1) / S;
+    p.S = (l.SC + p.sc_slice - 1) / p.sc_slice;
+    // partial sums behind the counters, inside the workspace that every GEMV kernel shares
+    if (p.S > 1 && align256((size_t)l.RB * 4) + (size_t)l.RB * p.S * NB * 32 * 4 > workspace_bytes_for(l)) return false;
+    const int ctas = sms / p.S * p.S;
+    if (ctas < 1) return false;
+    p.grid = l.RB * p.S < ctas ? l.RB * p.S : ctas;
+    p.x_off = tab;
+    p.red_off = (tab + (size_t)p.sc_slice * per_sc + 15) & ~size_t(15);
+    p.smem = p.red_off + red;
+    return true;
+}
+
+template <int N, int MODE, int NB>
+cudaError_t launch_one(const FragArgs& a, const FragPlan& p, cudaStream_t s) {
+    static DeviceOnce attr_done;
+    const int dev = DeviceOnce::current();
+    if (!attr_done.is_set(dev)) {
+        const cudaError_t e = cudaFuncSetAttribute(gemv_frag_kernel<N, MODE, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFSmem);
+        if (e != cudaSuccess) return e;
+        attr_done.set(dev);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.grid, 1, 1);
+    cfg.blockDim = dim3(kFThreads, 1, 1);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gemv_frag_kernel<N, MODE, NB>, a);
+}
+
+template <int N, int MODE>
+cudaError_t launch_rows(int NB, const FragArgs& a, const FragPlan& p, cudaStream_t s) {
+    switch (NB) {
+        case 1: return launch_one<N, MODE, 1>(a, p, s);
+        case 2: return launch_one<N, MODE, 2>(a, p, s);
+        case 4: return launch_one<N, MODE, 4>(a, p, s);
+        case 8: return launch_one<N, MODE, 8>(a, p, s);
+        default: return launch_one<N, MODE, 16>(a, p, s);
+    }
+}
+
+bool frag_preferred(const Layout& l, int batch) {
+#ifdef LANE_TUNE
+    if (const char* e = getenv("XFP_FRAG")) return batch >= atoi(e);
+#endif
+    return batch >= 2;
+}
+
+}  // namespace
+
+bool frag_supported(const Layout& l, const GemvCall& c) {
+    if (c.n != 1 || c.packed_list || c.epilogue != 0 || l.GH != 1) return false;
+    FragPlan p;
+    return frag_preferred(l, c.batch) && plan_frag(l, c.batch, sched_sms(), p);
+}
+
+cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s) {
+    FragPlan p;
+    if (!plan_frag(l, c.batch, sched_sms(), p)) return cudaErrorInvalidValue;
+    FragArgs a = {};
+    a.b = blob_at(c.packed, offsets_of(l));
+    a.x = c.x; a.y = c.y;
+    a.tickets = (int*)c.workspace;
+    a.partial = (float*)((char*)c.workspace + align256((size_t)l.RB * 4));
+    a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.ell_slots = l.ell_slots; a.L = l.L;
+    a.nb = c.batch; a.y_kind = c.y_is_fp16; a.x_bf16 = c.x_bf16;
+    a.S = p.S; a.sc_slice = p.sc_slice; a.x_off = (int)p.x_off; a.red_off = (int)p.red_off;
+    const int NB = rows_of(c.batch);
+    if (l.mode) {
+        switch (l.bits) {
+            case 2: return launch_rows<2, 1>(NB, a, p, s);
+            case 3: return launch_rows<3, 1>(NB, a, p, s);
+            case 4: return launch_rows<4, 1>(NB, a, p, s);
+            case 5: return launch_rows<5, 1>(NB, a, p, s);
+            default: return launch_rows<6, 1>(NB, a, p, s);
+        }
+    }
+    switch (l.bits) {
+        case 2: return launch_rows<2, 0>(NB, a, p, s);
+        case 3: return launch_rows<3, 0>(NB, a, p, s);
+        case 4: return launch_rows<4, 0>(NB, a, p, s);
+        case 5: return launch_rows<5, 0>(NB, a, p, s);
+        default: return launch_rows<6, 0>(NB, a, p, s);
+    }
+}
+
+}  // namespace xfp

@@ -86,6 +86,10 @@ cudaError_t launch_gemv_lane(const Layout& l, const GemvCall& c, cudaStream_t s)
 bool lane_batch_supported(const Layout& l, const GemvCall& c);
 cudaError_t launch_gemv_lane_batch(const Layout& l, const GemvCall& c, cudaStream_t s);
 
+// 1..16 rows of x, V2 and V2a, in the mma's own operand layout; see xfp_gemv_frag.cu.
+bool frag_supported(const Layout& l, const GemvCall& c);
+cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s);
+
 // Fast V2a path (per-bank library + mma.sync fragments, one or several blobs); see xfp_gemv_v2a.cu.
 bool v2a_supported(const Layout& l, int batch);
 size_t v2a_workspace_bytes(const Layout& l);
