@@ -10,7 +10,8 @@
 //
 //   look-ups  four lanes share a channel, so a table is kept in four copies, one per t: entry (..)*128 + lane*4 lies in the
 //             lane's own bank.  V2: pair tables up to N = 4 (128 KB of four channels' tables at N = 4), one entry per index
-//             above.  V2a: the library once per bank, two library ids to a word.
+//             above.  V2a: the library once per bank, two library ids to a word.  At N = 4 entries lie 256 bytes apart, two
+//             tables interleaved, so that one PRMT turns an index (V2: a byte of two) into the address.
 //   x         staged once per CTA (fp16; bf16 is converted on the way) as 16-byte chunks, chunk c of row b at place
 //             c * NB + b with bits 1, 2 of the place exclusive-or'ed with c / 4 mod 4: the eight lanes of a quarter-warp and the
 //             staging threads meet eight different bank groups.  CTAs are resident and walk the row-blocks, so that x is staged
@@ -41,13 +42,19 @@ struct FragArgs {
     int x_off, red_off;   // bytes behind the tables: staged x, per-warp sums
 };
 
-// Tables: V2 [4][entries][32 lanes] words (entry = pair of indices up to N = 4); V2a [ceil(L / 2)][2^N][32] words of two fp16.
+// Tables.  V2: one per channel group j, [entries][32 lanes] words (entry = pair of indices up to N = 4).  V2a: one per two
+// library ids, [2^N][32] words of two fp16.  kStride bytes from entry to entry: 128, at N = 4 256 with tables 2 i and 2 i + 1
+// interleaved.
 template <int N, int MODE>
 struct FTab {
     static constexpr int E = 1 << N;
     static constexpr bool kPair = MODE == 0 && N <= 4;
     static constexpr int kEntries = kPair ? E * E : E;
-    static constexpr int kOne = kEntries * 128;        // bytes of one channel group's tables
+    static constexpr int kStride = N == 4 ? 256 : 128;
+    // byte offset of table i
+    __host__ __device__ static constexpr uint32_t at(uint32_t i) {
+        return N == 4 ? (i >> 1) * (uint32_t)(kEntries * 256) + (i & 1u) * 128u : i * (uint32_t)(kEntries * 128);
+    }
 };
 
 // The lane's words [t N, (t + 1) N) of the index streams of its four channels of super-chunk sc.
@@ -98,32 +105,40 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     float* sXg = (float*)(sX + (size_t)nsc * kSuper * NB * 2);      // V2a: sums of x over a group, [super-chunk][NB]
     const int step = (int)gridDim.x / a.S;
 
-    auto fill = [&](int rb) {                          // the tables of row-block rb (V2)
+    // a thread's share of a row-block's codebooks (V2), on its way while the previous row-block is finished: the whole codebook
+    // of its channel where pairs are built, else the entries its warp stores
+    constexpr int kCb = MODE ? 1 : T::kPair ? E / 2 : (E + kFW - 1) / kFW;
+    uint32_t cbn[kCb];
+    auto book = [&](int rb) {
+        const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * E;
+        if (T::kPair) {
+#pragma unroll
+            for (int e = 0; e < E / 4; ++e) { const uint2 p = __ldg((const uint2*)cb + e); cbn[(2 * e) % kCb] = p.x; cbn[(2 * e + 1) % kCb] = p.y; }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kCb; ++i) cbn[i] = __ldg(cb + warp + i * kFW);
+        }
+    };
+    auto fill = [&]() {
         const int ch = lane, j = ch >> 3;
-        const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + ch) * E;
-        unsigned char* dst = smem + (size_t)j * T::kOne + (ch & 7) * 16;
+        unsigned char* dst = smem + T::at(j) + (ch & 7) * 16;
         if (T::kPair) {
             // a thread takes a channel and every sixteenth entry; one 16-byte store writes the four copies
-            uint32_t v[E];
-#pragma unroll
-            for (int e = 0; e < E; e += 4) {
-                const uint2 p = __ldg((const uint2*)(cb + e));
-                v[e] = p.x & 0xffffu; v[e + 1] = p.x >> 16; v[e + 2] = p.y & 0xffffu; v[e + 3] = p.y >> 16;
-            }
 #pragma unroll
             for (int hi = 0; hi < E; ++hi) {
                 if (hi != warp % (E < kFW ? E : kFW)) continue;
 #pragma unroll
                 for (int lo = 0; lo < E; ++lo) {
                     if (E < kFW && (lo % (kFW / E)) != warp / E) continue;
-                    const uint32_t p = v[lo] | (v[hi] << 16);
-                    *(uint4*)(dst + (size_t)(lo | (hi << N)) * 128) = make_uint4(p, p, p, p);
+                    const uint32_t p = __byte_perm(cbn[(lo / 2) % kCb], cbn[(hi / 2) % kCb], ((lo & 1) ? 0x32 : 0x10) | ((hi & 1) ? 0x7600 : 0x5400));
+                    *(uint4*)(dst + (size_t)(lo | (hi << N)) * T::kStride) = make_uint4(p, p, p, p);
                 }
             }
         } else {
-            for (int e = warp; e < E; e += kFW) {
-                const uint32_t p = __ldg(cb + e);
-                *(uint4*)(dst + (size_t)e * 128) = make_uint4(p, p, p, p);
+#pragma unroll
+            for (int i = 0; i < kCb; ++i) {
+                const uint32_t p = cbn[i];
+                *(uint4*)(dst + (size_t)(warp + i * kFW) * T::kStride) = make_uint4(p, p, p, p);
             }
         }
     };
@@ -147,13 +162,19 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
         if (rb < a.RB && sc0 + warp + i * kFW < sc1) fetch(rb, sc0 + warp + i * kFW, i);
     if (MODE == 1) {
         const int words = (a.L + 1) / 2 * E;
-        for (int i = warp; i < words; i += kFW) {
-            const int id = i / E * 2, q = i % E;
-            const uint32_t lo = __ldg(a.b.cb + id * E + q), hi = id + 1 < a.L ? (uint32_t)__ldg(a.b.cb + (id + 1) * E + q) : 0u;
-            ((uint32_t*)smem)[i * 32 + lane] = lo | (hi << 16);
+        for (int i0 = warp * 32; i0 < words; i0 += kFW * 32) {      // a lane fetches a word, the warp stores 32 of them
+            const int i = i0 + lane, id = i / E * 2, q = i % E;
+            uint32_t v = 0;
+            if (i < words) v = (uint32_t)__ldg(a.b.cb + id * E + q) | (id + 1 < a.L ? (uint32_t)__ldg(a.b.cb + (id + 1) * E + q) << 16 : 0u);
+#pragma unroll 8
+            for (int k = 0; k < 32; ++k) {
+                const uint32_t o = __shfl_sync(0xffffffffu, v, k);
+                if (i0 + k < words) *(uint32_t*)(smem + T::at((uint32_t)((i0 + k) / E)) + (size_t)((i0 + k) % E) * T::kStride + lane * 4) = o;
+            }
         }
     } else if (rb < a.RB) {
-        fill(rb);
+        book(rb);
+        fill();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // ---- x: chunks of a row by consecutive threads ----
@@ -189,35 +210,38 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     for (bool later = false; rb < a.RB; rb += step, later = true) {
         if (later) {
             __syncthreads();                           // tables and sums of the previous row-block are done with
-            if (MODE == 0) { fill(rb); __syncthreads(); }
+            if (MODE == 0) { fill(); __syncthreads(); }
         }
         float acc[NT][2][4];
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc[n][i >> 2][i & 3] = 0.f;
-        for (int sc = sc0 + warp; sc < sc1; sc += kFW) {
-            uint32_t w[4][N + 1];
+        // the row-block's first outliers travel under the loop
+        const int row = rb * kRowsPerBlock + lane;
+        const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
+        uint32_t len = 0, ent[2] = {0, 0};
+        if (a.ell_slots) {
+            len = __ldg(slab);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (warp + i * kFW < a.ell_slots) ent[i] = __ldg(slab + (size_t)(1 + warp + i * kFW) * 32);
+        }
+        for (int scu = sc0 + warp; scu < sc1; scu += kAhead * kFW) {
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u) {
+            const int sc = scu + u * kFW;
+            if (sc >= sc1) break;
             uint32_t base[4];
             float scale[4], mid[4];
+            if (MODE == 1) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) w[j][i] = nx[0][j][i];
-                w[j][N] = 0u;
-                if (MODE == 1) {
-                    const __half2 sm = *(const __half2*)&sm_n[0][j];
+                for (int j = 0; j < 4; ++j) {
+                    const __half2 sm = *(const __half2*)&sm_n[u][j];
                     scale[j] = __low2float(sm); mid[j] = __high2float(sm);
-                    base[j] = (id_n[0][j] >> 1) * (uint32_t)(E * 128) + lbase + (id_n[0][j] & 1u) * 2u;
-                }
-#pragma unroll
-                for (int s = 0; s + 1 < kAhead; ++s) {
-#pragma unroll
-                    for (int i = 0; i < N; ++i) nx[s][j][i] = nx[s + 1][j][i];
-                    id_n[s][j] = id_n[s + 1][j]; sm_n[s][j] = sm_n[s + 1][j];
+                    base[j] = T::at(id_n[u][j] >> 1) + lbase + (id_n[u][j] & 1u) * 2u;
                 }
             }
-            if (sc + kAhead * kFW < sc1) fetch(rb, sc + kAhead * kFW, kAhead - 1);
             const int lsc = sc - sc0;
             float c[NT][2][4];
             if (MODE == 1) {
@@ -242,17 +266,28 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
 #pragma unroll
-                        for (int u = 0; u < 2; ++u) {
+                        for (int v = 0; v < 2; ++v) {
+                            const uint32_t* w = nx[u][j];
+                            const int p = p0 + v;
                             if (T::kPair) {
-                                av[j][u] = *(const uint32_t*)(smem + j * T::kOne + pair_addr<N, 1>(w[j], p0 + u, lbase));
+                                // the second of two interleaved tables: its 128 bytes ride in the base
+                                const uint32_t off = N == 4 ? pair_addr<N, 2>(w, p, lbase | ((j & 1) * 128u)) : pair_addr<N, 1>(w, p, lbase);
+                                av[j][v] = *(const uint32_t*)(smem + (N == 4 ? T::at(j & ~1) : T::at(j)) + off);
                             } else if (MODE == 0) {
-                                const uint32_t lo = *(const uint32_t*)(smem + j * T::kOne + single_addr<N, 1>(w[j], 2 * (p0 + u), lbase));
-                                const uint32_t hi = *(const uint32_t*)(smem + j * T::kOne + single_addr<N, 1>(w[j], 2 * (p0 + u) + 1, lbase));
-                                av[j][u] = lo | (hi << 16);
+                                const uint32_t lo = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p, lbase));
+                                const uint32_t hi = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p + 1, lbase));
+                                av[j][v] = lo | (hi << 16);
+                            } else if (N == 4) {
+                                // byte 1 of the address: index and the low four bits of id / 4
+                                const uint32_t nib = ((base[j] >> 12) & 0xfu) * 0x10101010u, sel = 0x7604u | ((uint32_t)(p & 3) << 4);
+                                const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
+                                const uint32_t lo = *(const uint16_t*)(smem + __byte_perm(wlo, base[j], sel));
+                                const uint32_t hi = *(const uint16_t*)(smem + __byte_perm(whi, base[j], sel));
+                                av[j][v] = lo | (hi << 16);
                             } else {
-                                const uint32_t lo = *(const uint16_t*)(smem + (single_addr<N, 1>(w[j], 2 * (p0 + u), 0u) + base[j]));
-                                const uint32_t hi = *(const uint16_t*)(smem + (single_addr<N, 1>(w[j], 2 * (p0 + u) + 1, 0u) + base[j]));
-                                av[j][u] = lo | (hi << 16);
+                                const uint32_t lo = *(const uint16_t*)(smem + single_addr<N, 1>(w, 2 * p, base[j]));
+                                const uint32_t hi = *(const uint16_t*)(smem + single_addr<N, 1>(w, 2 * p + 1, base[j]));
+                                av[j][v] = lo | (hi << 16);
                             }
                         }
 #pragma unroll
@@ -280,21 +315,22 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                         }
                 }
             }
+            if (sc + kAhead * kFW < sc1) fetch(rb, sc + kAhead * kFW, u);
+          }
         }
         // the first super-chunks of the next row-block travel while this one is finished
         if (rb + step < a.RB) {
 #pragma unroll
             for (int i = 0; i < kAhead; ++i)
                 if (sc0 + warp + i * kFW < sc1) fetch(rb + step, sc0 + warp + i * kFW, i);
+            if (MODE == 0) book(rb + step);
         }
         // ---- outliers: lane = channel ----
         float ao[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) ao[b] = 0.f;
         if (a.ell_slots) {
-            const int row = rb * kRowsPerBlock + lane;
-            const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
-            const int len = (int)__ldg(slab), nslab = min(len, a.ell_slots);
+            const int nslab = min((int)len, a.ell_slots);
             const uint32_t k0 = (uint32_t)sc0 * kSuper, kn = (uint32_t)nsc * kSuper;
             auto add = [&](uint32_t e) {
                 const uint32_t k = (e & 0xffffu) - k0;
@@ -307,14 +343,17 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 }
             };
             const int most = __reduce_max_sync(0xffffffffu, nslab);
-            for (int j0 = warp; j0 < most; j0 += 4 * kFW) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (warp + i * kFW < nslab) add(ent[i]);
+            for (int j0 = warp + 2 * kFW; j0 < most; j0 += 4 * kFW) {
                 uint32_t e[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) e[i] = j0 + i * kFW < nslab ? __ldg(slab + (size_t)(1 + j0 + i * kFW) * 32) : 0u;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) if (j0 + i * kFW < nslab) add(e[i]);
             }
-            if (len >= a.ell_slots && row < a.rows) {  // the channel overflows its slab: the rest is in the CSR arrays
+            if ((int)len >= a.ell_slots && row < a.rows) {  // the channel overflows its slab: the rest is in the CSR arrays
                 const int p1 = __ldg(a.b.rowptr + row + 1);
                 for (int p = __ldg(a.b.rowptr + row) + a.ell_slots + warp; p < p1; p += kFW) add(__ldg(a.b.oent + p));
             }
@@ -337,7 +376,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
         }
         __syncthreads();
         float sum = 0.f;
-        const int b = tid >> 5, row = rb * kRowsPerBlock + lane;
+        const int b = tid >> 5;
         if (b < a.nb) {
 #pragma unroll
             for (int w = 0; w < kFW; ++w) sum += red[(w * NB + b) * 33 + lane];
@@ -367,7 +406,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
 struct FragPlan { int S, sc_slice, grid; size_t x_off, red_off, smem; };
 
 size_t table_bytes(const Layout& l) {
-    if (l.mode) return (size_t)((l.L + 1) / 2) * l.E * 128;
+    if (l.mode) { const int n = (l.L + 1) / 2; return (size_t)(l.bits == 4 ? (n + 1) & ~1 : n) * l.E * 128; }
     return (size_t)4 * (l.bits <= 4 ? l.E * l.E : l.E) * 128;
 }
 
