@@ -83,6 +83,29 @@ __device__ __forceinline__ void load_words(uint32_t (&w)[4][N], const uint4* idx
     }
 }
 
+// A load that stays where it is written: the compiler sank the plain form of these early loads to their uses, behind the K loop,
+// where a row-block then waited 2000 - 3800 clocks for them.
+__device__ __forceinline__ uint32_t ld_early(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_early2(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_early4(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_early16(const uint16_t* p) {
+    uint16_t v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 // byte offset of the 16-byte chunk c (8 k) of row b in the staged x
 template <int NB>
 __device__ __forceinline__ uint32_t x_chunk(int c, int b) {
@@ -112,11 +135,19 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     auto book = [&](int rb) {
         const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * E;
         if (T::kPair) {
+            if (E == 4) {
+                const uint2 p = ld_early2((const uint2*)cb);
+                cbn[0] = p.x; cbn[1 % kCb] = p.y;
+            } else {
 #pragma unroll
-            for (int e = 0; e < E / 4; ++e) { const uint2 p = __ldg((const uint2*)cb + e); cbn[(2 * e) % kCb] = p.x; cbn[(2 * e + 1) % kCb] = p.y; }
+                for (int e = 0; e < E / 8; ++e) {
+                    const uint4 p = ld_early4((const uint4*)cb + e);
+                    cbn[(4 * e) % kCb] = p.x; cbn[(4 * e + 1) % kCb] = p.y; cbn[(4 * e + 2) % kCb] = p.z; cbn[(4 * e + 3) % kCb] = p.w;
+                }
+            }
         } else {
 #pragma unroll
-            for (int i = 0; i < kCb; ++i) cbn[i] = __ldg(cb + warp + i * kFW);
+            for (int i = 0; i < kCb; ++i) cbn[i] = ld_early16(cb + warp + i * kFW);
         }
     };
     auto fill = [&]() {
@@ -179,13 +210,18 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // ---- x: chunks of a row by consecutive threads ----
     {
+        constexpr int kRows = NB > 8 ? 8 : NB;         // loads in flight per thread
         const int chunks = nsc * (kSuper / 8);
+        const uint4* xs = (const uint4*)(a.x + (size_t)sc0 * kSuper);
+        const int row16 = a.cols / 8;
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
+        for (int b0 = 0; b0 < NB; b0 += kRows) {
             for (int c = tid; c < chunks; c += kFThreads) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (b < a.nb) v = x8_as_f16(__ldg((const uint4*)(a.x + (size_t)b * a.cols + (size_t)sc0 * kSuper) + c), a.x_bf16);
-                *(uint4*)(sX + x_chunk<NB>(c, b)) = v;
+                uint4 v[kRows];
+#pragma unroll
+                for (int b = 0; b < kRows; ++b) v[b] = b0 + b < a.nb ? __ldg(xs + (size_t)(b0 + b) * row16 + c) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int b = 0; b < kRows; ++b) *(uint4*)(sX + x_chunk<NB>(c, b0 + b)) = x8_as_f16(v[b], a.x_bf16);
             }
         }
     }
@@ -220,12 +256,13 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
         // the row-block's first outliers travel under the loop
         const int row = rb * kRowsPerBlock + lane;
         const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
-        uint32_t len = 0, ent[2] = {0, 0};
+        constexpr int kEnt = 3;
+        uint32_t len = 0, ent[kEnt] = {};
         if (a.ell_slots) {
-            len = __ldg(slab);
+            len = ld_early(slab);
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-                if (warp + i * kFW < a.ell_slots) ent[i] = __ldg(slab + (size_t)(1 + warp + i * kFW) * 32);
+            for (int i = 0; i < kEnt; ++i)
+                if (warp + i * kFW < a.ell_slots) ent[i] = ld_early(slab + (size_t)(1 + warp + i * kFW) * 32);
         }
         for (int scu = sc0 + warp; scu < sc1; scu += kAhead * kFW) {
 #pragma unroll
@@ -315,16 +352,12 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                         }
                 }
             }
+            // the slot's next super-chunk, or the one that it holds first of the CTA's next row-block
             if (sc + kAhead * kFW < sc1) fetch(rb, sc + kAhead * kFW, u);
+            else if (rb + step < a.RB) fetch(rb + step, sc0 + warp + u * kFW, u);
           }
         }
-        // the first super-chunks of the next row-block travel while this one is finished
-        if (rb + step < a.RB) {
-#pragma unroll
-            for (int i = 0; i < kAhead; ++i)
-                if (sc0 + warp + i * kFW < sc1) fetch(rb + step, sc0 + warp + i * kFW, i);
-            if (MODE == 0) book(rb + step);
-        }
+        if (MODE == 0 && rb + step < a.RB) book(rb + step);
         // ---- outliers: lane = channel ----
         float ao[NB];
 #pragma unroll
@@ -344,9 +377,9 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
             };
             const int most = __reduce_max_sync(0xffffffffu, nslab);
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < kEnt; ++i)
                 if (warp + i * kFW < nslab) add(ent[i]);
-            for (int j0 = warp + 2 * kFW; j0 < most; j0 += 4 * kFW) {
+            for (int j0 = warp + kEnt * kFW; j0 < most; j0 += 4 * kFW) {
                 uint32_t e[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) e[i] = j0 + i * kFW < nslab ? __ldg(slab + (size_t)(1 + j0 + i * kFW) * 32) : 0u;
