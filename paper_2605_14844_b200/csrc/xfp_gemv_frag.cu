@@ -42,13 +42,13 @@ struct FragArgs {
     int x_off, red_off;   // bytes behind the tables: staged x, per-warp sums
 };
 
-// Tables.  V2: one per channel group j, [entries][32 lanes] words (entry = pair of indices up to N = 4).  V2a: one per two
+// Tables.  V2: one per channel group j, [entries][32 lanes] words (entry = pair of indices with PAIR, N <= 4).  V2a: one per two
 // library ids, [2^N][32] words of two fp16.  kStride bytes from entry to entry: 128, at N = 4 256 with tables 2 i and 2 i + 1
 // interleaved.
-template <int N, int MODE>
+template <int N, int MODE, bool PAIR>
 struct FTab {
     static constexpr int E = 1 << N;
-    static constexpr bool kPair = MODE == 0 && N <= 4;
+    static constexpr bool kPair = PAIR;
     static constexpr int kEntries = kPair ? E * E : E;
     static constexpr int kStride = N == 4 ? 256 : 128;
     // byte offset of table i
@@ -112,9 +112,9 @@ __device__ __forceinline__ uint32_t x_chunk(int c, int b) {
     return (uint32_t)((c * NB + b) ^ (((c >> 2) & 3) << 1)) << 4;
 }
 
-template <int N, int MODE, int NB>
+template <int N, int MODE, int NB, bool PAIR>
 __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs a) {
-    using T = FTab<N, MODE>;
+    using T = FTab<N, MODE, PAIR>;
     constexpr int E = T::E;
     constexpr int NT = NB > 8 ? 2 : 1;                 // tiles of eight rows of x
     constexpr int kAhead = N <= 4 ? 2 : 1;             // super-chunks of indices in flight per warp
@@ -310,6 +310,11 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                                 // the second of two interleaved tables: its 128 bytes ride in the base
                                 const uint32_t off = N == 4 ? pair_addr<N, 2>(w, p, lbase | ((j & 1) * 128u)) : pair_addr<N, 1>(w, p, lbase);
                                 av[j][v] = *(const uint32_t*)(smem + (N == 4 ? T::at(j & ~1) : T::at(j)) + off);
+                            } else if (MODE == 0 && N == 4) {
+                                const uint32_t lb = lbase | ((j & 1) * 128u), sel = 0x7604u | ((uint32_t)(p & 3) << 4);
+                                const uint32_t lo = *(const uint32_t*)(smem + T::at(j & ~1) + __byte_perm(w[p >> 2] & 0x0f0f0f0fu, lb, sel));
+                                const uint32_t hi = *(const uint32_t*)(smem + T::at(j & ~1) + __byte_perm((w[p >> 2] >> 4) & 0x0f0f0f0fu, lb, sel));
+                                av[j][v] = lo | (hi << 16);
                             } else if (MODE == 0) {
                                 const uint32_t lo = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p, lbase));
                                 const uint32_t hi = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p + 1, lbase));
@@ -436,22 +441,33 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     }
 }
 
-struct FragPlan { int S, sc_slice, grid; size_t x_off, red_off, smem; };
+struct FragPlan { int S, sc_slice, grid, pair; size_t x_off, red_off, smem; };
 
-size_t table_bytes(const Layout& l) {
+size_t table_bytes(const Layout& l, bool pair) {
     if (l.mode) { const int n = (l.L + 1) / 2; return (size_t)(l.bits == 4 ? (n + 1) & ~1 : n) * l.E * 128; }
-    return (size_t)4 * (l.bits <= 4 ? l.E * l.E : l.E) * 128;
+    return (size_t)4 * (pair ? l.E * l.E : l.E) * 128;
 }
 
 int rows_of(int batch) { return batch <= 1 ? 1 : batch <= 2 ? 2 : batch <= 4 ? 4 : batch <= 8 ? 8 : 16; }
 
 bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
     const int NB = rows_of(batch);
-    const size_t tab = table_bytes(l), red = (size_t)kFW * NB * 33 * 4 + 16;
+    const size_t red = (size_t)kFW * NB * 33 * 4 + 16;
     const size_t per_sc = (size_t)kSuper * NB * 2 + (l.mode ? NB * 4 : 0);
-    if (tab + red + per_sc > kFSmem) return false;
-    const int fit = (int)((kFSmem - tab - red) / per_sc);             // super-chunks of x that fit
-    int S = (l.SC + fit - 1) / fit;
+    auto slices = [&](bool pair) {                                    // K slices that x needs beside the tables
+        const size_t used = table_bytes(l, pair) + red;
+        const int fit = used + per_sc > kFSmem ? 0 : (int)((kFSmem - used) / per_sc);
+        return fit ? (l.SC + fit - 1) / fit : 0;
+    };
+    // N = 4: pair tables take 128 of 224 KB, and a slice more means that the tables are built once more and the outliers walked
+    // once more; where single entries (8 KB) need fewer slices they are the faster ones
+    p.pair = l.mode == 0 && l.bits <= 4;
+    int S = slices(p.pair);
+    if (p.pair && l.bits == 4) {
+        const int s1 = slices(false);
+        if (!S || s1 < S) { p.pair = 0; S = s1; }
+    }
+    if (!S) return false;
     // few row-blocks: K slices until the SMs are busy, at least one super-chunk per warp
     while (l.RB * (S + 1) <= sms && l.SC / (S + 1) >= kFW) ++S;
     p.sc_slice = (l.SC + S - 1) / S;
@@ -461,18 +477,18 @@ bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
     const int ctas = sms / p.S * p.S;
     if (ctas < 1) return false;
     p.grid = l.RB * p.S < ctas ? l.RB * p.S : ctas;
-    p.x_off = tab;
-    p.red_off = (tab + (size_t)p.sc_slice * per_sc + 15) & ~size_t(15);
+    p.x_off = table_bytes(l, p.pair);
+    p.red_off = (p.x_off + (size_t)p.sc_slice * per_sc + 15) & ~size_t(15);
     p.smem = p.red_off + red;
     return true;
 }
 
-template <int N, int MODE, int NB>
+template <int N, int MODE, int NB, bool PAIR>
 cudaError_t launch_one(const FragArgs& a, const FragPlan& p, cudaStream_t s) {
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        const cudaError_t e = cudaFuncSetAttribute(gemv_frag_kernel<N, MODE, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFSmem);
+        const cudaError_t e = cudaFuncSetAttribute(gemv_frag_kernel<N, MODE, NB, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFSmem);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
@@ -486,17 +502,17 @@ cudaError_t launch_one(const FragArgs& a, const FragPlan& p, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_frag_kernel<N, MODE, NB>, a);
+    return cudaLaunchKernelEx(&cfg, gemv_frag_kernel<N, MODE, NB, PAIR>, a);
 }
 
-template <int N, int MODE>
+template <int N, int MODE, bool PAIR = MODE == 0 && N <= 4>
 cudaError_t launch_rows(int NB, const FragArgs& a, const FragPlan& p, cudaStream_t s) {
     switch (NB) {
-        case 1: return launch_one<N, MODE, 1>(a, p, s);
-        case 2: return launch_one<N, MODE, 2>(a, p, s);
-        case 4: return launch_one<N, MODE, 4>(a, p, s);
-        case 8: return launch_one<N, MODE, 8>(a, p, s);
-        default: return launch_one<N, MODE, 16>(a, p, s);
+        case 1: return launch_one<N, MODE, 1, PAIR>(a, p, s);
+        case 2: return launch_one<N, MODE, 2, PAIR>(a, p, s);
+        case 4: return launch_one<N, MODE, 4, PAIR>(a, p, s);
+        case 8: return launch_one<N, MODE, 8, PAIR>(a, p, s);
+        default: return launch_one<N, MODE, 16, PAIR>(a, p, s);
     }
 }
 
@@ -539,7 +555,7 @@ cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s)
     switch (l.bits) {
         case 2: return launch_rows<2, 0>(NB, a, p, s);
         case 3: return launch_rows<3, 0>(NB, a, p, s);
-        case 4: return launch_rows<4, 0>(NB, a, p, s);
+        case 4: return p.pair ? launch_rows<4, 0>(NB, a, p, s) : launch_rows<4, 0, false>(NB, a, p, s);
         case 5: return launch_rows<5, 0>(NB, a, p, s);
         default: return launch_rows<6, 0>(NB, a, p, s);
     }
