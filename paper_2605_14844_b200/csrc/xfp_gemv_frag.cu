@@ -112,6 +112,24 @@ __device__ __forceinline__ uint32_t x_chunk(int c, int b) {
     return (uint32_t)((c * NB + b) ^ (((c >> 2) & 3) << 1)) << 4;
 }
 
+// Eight rows of x and more: [tile of eight rows][k][8 rows], 16 bytes per k, which ldmatrix.trans turns into B fragments and
+// which gives an outlier its eight values in one load.  The byte offset of k in a tile: the place of k among the eight of its
+// chunk is exclusive-or'ed so that the eight k of a fragment (32 t + 0, 1) and eight staging threads (consecutive chunks) each
+// meet eight bank groups.
+__device__ __forceinline__ uint32_t x_at(int k) {
+    const int c = k >> 3;
+    return (uint32_t)(k ^ (c & 7) ^ (((c >> 2) & 3) << 1)) << 4;
+}
+
+__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+__device__ __forceinline__ uint4 ldmatrix_x4_trans(uint32_t addr) {
+    uint4 v;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+
 template <int N, int MODE, int NB, bool PAIR>
 __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs a) {
     using T = FTab<N, MODE, PAIR>;
@@ -127,6 +145,10 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), nsc = sc1 - sc0;
     float* sXg = (float*)(sX + (size_t)nsc * kSuper * NB * 2);      // V2a: sums of x over a group, [super-chunk][NB]
     const int step = (int)gridDim.x / a.S;
+    constexpr bool kTiles = NB >= 8;
+    const uint32_t tile = (uint32_t)nsc * kSuper * 16;              // bytes of a tile of eight rows
+    // the lane's row of the four 8 x 8 matrices of two mma steps: k = 32 (r / 2) + 2 m + r mod 2, r = lane mod 8, m = lane / 8
+    const uint32_t xrow = (uint32_t)__cvta_generic_to_shared(sX) + x_at(32 * ((lane & 7) >> 1) + 2 * (lane >> 3) + (lane & 1));
 
     // a thread's share of a row-block's codebooks (V2), on its way while the previous row-block is finished: the whole codebook
     // of its channel where pairs are built, else the entries its warp stores
@@ -221,26 +243,50 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
 #pragma unroll
                 for (int b = 0; b < kRows; ++b) v[b] = b0 + b < a.nb ? __ldg(xs + (size_t)(b0 + b) * row16 + c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                for (int b = 0; b < kRows; ++b) *(uint4*)(sX + x_chunk<NB>(c, b0 + b)) = x8_as_f16(v[b], a.x_bf16);
+                for (int b = 0; b < kRows; ++b) v[b] = x8_as_f16(v[b], a.x_bf16);
+                if constexpr (kTiles) {
+                    unsigned char* dst = sX + (size_t)(b0 / 8) * tile;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {      // k = 8 c + i of the eight rows
+                        auto two = [&](int b) {
+                            const uint32_t lo = word(v[b % kRows], i >> 1), hi = word(v[(b + 1) % kRows], i >> 1);
+                            return __byte_perm(lo, hi, (i & 1) ? 0x7632 : 0x5410);
+                        };
+                        *(uint4*)(dst + x_at(8 * c + i)) = make_uint4(two(0), two(2 % kRows), two(4 % kRows), two(6 % kRows));
+                    }
+                } else {
+#pragma unroll
+                    for (int b = 0; b < kRows; ++b) *(uint4*)(sX + x_chunk<NB>(c, b)) = v[b];
+                }
+                if constexpr (MODE == 1) {
+                    // sums of a super-chunk: over the thread's eight k, then over the sixteen threads that hold its chunks
+                    float f[kRows];
+#pragma unroll
+                    for (int b = 0; b < kRows; ++b) {
+                        const float2 p0 = __half22float2(*(const __half2*)&v[b].x), p1 = __half22float2(*(const __half2*)&v[b].y),
+                                     p2 = __half22float2(*(const __half2*)&v[b].z), p3 = __half22float2(*(const __half2*)&v[b].w);
+                        f[b] = ((p0.x + p0.y) + (p1.x + p1.y)) + ((p2.x + p2.y) + (p3.x + p3.y));
+                    }
+                    const uint32_t half = 0xffffu << (lane & 16);
+                    int row = 0, d = 1;
+#pragma unroll
+                    for (int w = kRows / 2; w >= 1; w /= 2, d *= 2) {   // halve the rows a lane keeps
+                        const bool up = lane & d;
+#pragma unroll
+                        for (int b = 0; b < w; ++b) {
+                            const float give = up ? f[b] : f[b + w], keep = up ? f[b + w] : f[b];
+                            f[b] = keep + __shfl_xor_sync(half, give, d);
+                        }
+                        if (up) row += w;
+                    }
+#pragma unroll
+                    for (; d < 16; d *= 2) f[0] += __shfl_xor_sync(half, f[0], d);
+                    if ((lane & 15) < kRows) sXg[(c >> 4) * NB + b0 + row] = f[0];
+                }
             }
         }
     }
     __syncthreads();
-    if (MODE == 1) {
-        for (int i = tid; i < nsc * NB; i += kFThreads) {
-            const int sc = i / NB, b = i % NB;
-            float sum = 0.f;
-#pragma unroll 4
-            for (int c = 0; c < kSuper / 8; ++c) {
-                const uint4 v = *(const uint4*)(sX + x_chunk<NB>(sc * (kSuper / 8) + c, b));
-                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { const float2 f = __half22float2(*(const __half2*)&u[k]); sum += f.x + f.y; }
-            }
-            sXg[i] = sum;
-        }
-        __syncthreads();
-    }
 
     const uint32_t lbase = (uint32_t)lane * 4u;
     for (bool later = false; rb < a.RB; rb += step, later = true) {
@@ -293,8 +339,13 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 uint4 xb[NT];
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
-                    xb[n] = make_uint4(0u, 0u, 0u, 0u);
-                    if (NB >= 8 || g < NB) xb[n] = *(const uint4*)(sX + x_chunk<NB>(lsc * 16 + 4 * t + s2, g + 8 * n));
+                    if constexpr (kTiles) {
+                        // chunk s2 of each t: the exclusive-or of x_at has s2 as its two low bits
+                        xb[n] = ldmatrix_x4_trans((xrow ^ (uint32_t)(s2 << 4)) + (uint32_t)(lsc * kSuper * 16 + s2 * 128) + n * tile);
+                    } else {
+                        xb[n] = make_uint4(0u, 0u, 0u, 0u);
+                        if (g < NB) xb[n] = *(const uint4*)(sX + x_chunk<NB>(lsc * 16 + 4 * t + s2, g));
+                    }
                 }
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
@@ -374,10 +425,24 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 const uint32_t k = (e & 0xffffu) - k0;
                 if (k < kn) {
                     const float v = h2f((uint16_t)(e >> 16));
-                    const int c = (int)(k >> 3);
-                    const unsigned char* p = sX + (k & 7u) * 2u;
+                    if constexpr (kTiles) {
 #pragma unroll
-                    for (int b = 0; b < NB; ++b) ao[b] = fmaf(v, h2f(*(const uint16_t*)(p + x_chunk<NB>(c, b))), ao[b]);
+                        for (int n = 0; n < NT; ++n) {
+                            const uint4 x8 = *(const uint4*)(sX + n * tile + x_at((int)k));
+                            const uint32_t u[4] = {x8.x, x8.y, x8.z, x8.w};
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                const float2 f = __half22float2(*(const __half2*)&u[b]);
+                                ao[(8 * n + 2 * b) % NB] = fmaf(v, f.x, ao[(8 * n + 2 * b) % NB]);
+                                ao[(8 * n + 2 * b + 1) % NB] = fmaf(v, f.y, ao[(8 * n + 2 * b + 1) % NB]);
+                            }
+                        }
+                    } else {
+                        const int c = (int)(k >> 3);
+                        const unsigned char* p = sX + (k & 7u) * 2u;
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) ao[b] = fmaf(v, h2f(*(const uint16_t*)(p + x_chunk<NB>(c, b))), ao[b]);
+                    }
                 }
             };
             const int most = __reduce_max_sync(0xffffffffu, nslab);
