@@ -5,18 +5,19 @@
 // weights of a lane.  Here lane (g, t) of a warp, g = lane / 4, t = lane mod 4, takes the t-th 32 of a super-chunk's 128
 // weights of the four channels g, g + 8, g + 16, g + 24 of a row-block.  That is the A operand of mma.m16n8k16 as it stands --
 // the order of k inside a super-chunk is free, and step s multiplies the k 32 t + 4 s .. + 3 of every t -- so one mma serves
-// eight rows of x, a lane's share of x is 16 consecutive bytes of one row (four wavefronts per super-chunk and row pair, none
-// wasted), and an accumulator holds four channels' sums: V2a's scale and mid-point are applied in place, without a shuffle.
+// eight rows of x, none of the staged x that is read is wasted, and an accumulator holds four channels' sums: V2a's scale and
+// mid-point are applied in place, without a shuffle.
 //
 //   look-ups  four lanes share a channel, so a table is kept in four copies, one per t: entry (..)*128 + lane*4 lies in the
 //             lane's own bank.  V2: pair tables up to N = 4 (128 KB of four channels' tables at N = 4), one entry per index
 //             above.  V2a: the library once per bank, two library ids to a word.  At N = 4 entries lie 256 bytes apart, two
 //             tables interleaved, so that one PRMT turns an index (V2: a byte of two) into the address.
-//   x         staged once per CTA (fp16; bf16 is converted on the way) as 16-byte chunks, chunk c of row b at place
-//             c * NB + b with bits 1, 2 of the place exclusive-or'ed with c / 4 mod 4: the eight lanes of a quarter-warp and the
-//             staging threads meet eight different bank groups.  CTAs are resident and walk the row-blocks, so that x is staged
-//             once; a K too long for shared memory is cut into slices, a CTA staying in its slice.
-//   outliers  a lane per channel, slots of the transposed slab dealt to the warps; NB products per entry.
+//   x         staged once per CTA (fp16; bf16 is converted on the way), 16 bytes = eight rows per k, for ldmatrix.trans.  CTAs
+//             are resident and walk the row-blocks, so that x is staged once; a K too long for shared memory is cut into
+//             slices, a CTA staying in its slice.
+//   outliers  a lane per channel, slots of the transposed slab dealt to the warps; eight products per load of x.
+//             (The same walk over x as rows of k cost eight loads of two bytes per entry, 5 way conflicts each: 12288 x 4096, 8
+//             rows, 5 % outliers 32.1 -> 24.0 us.)
 //   sums      fragments -> shared memory -> fixed order over the warps; K slices meet in the workspace, the last to come adds
 //             them in order (a ticket, no waiting).
 #include "xfp_internal.h"
@@ -106,14 +107,7 @@ __device__ __forceinline__ uint32_t ld_early16(const uint16_t* p) {
     return v;
 }
 
-// byte offset of the 16-byte chunk c (8 k) of row b in the staged x
-template <int NB>
-__device__ __forceinline__ uint32_t x_chunk(int c, int b) {
-    return (uint32_t)((c * NB + b) ^ (((c >> 2) & 3) << 1)) << 4;
-}
-
-// Eight rows of x and more: [tile of eight rows][k][8 rows], 16 bytes per k, which ldmatrix.trans turns into B fragments and
-// which gives an outlier its eight values in one load.  The byte offset of k in a tile: the place of k among the eight of its
+// Staged x: [tile of eight rows][k][8 rows], 16 bytes per k, which ldmatrix.trans turns into B fragments and which gives an outlier its eight values in one load.  The byte offset of k in a tile: the place of k among the eight of its
 // chunk is exclusive-or'ed so that the eight k of a fragment (32 t + 0, 1) and eight staging threads (consecutive chunks) each
 // meet eight bank groups.
 __device__ __forceinline__ uint32_t x_at(int k) {
@@ -145,7 +139,6 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     const int sc0 = slice * a.sc_slice, sc1 = min(a.SC, sc0 + a.sc_slice), nsc = sc1 - sc0;
     float* sXg = (float*)(sX + (size_t)nsc * kSuper * NB * 2);      // V2a: sums of x over a group, [super-chunk][NB]
     const int step = (int)gridDim.x / a.S;
-    constexpr bool kTiles = NB >= 8;
     const uint32_t tile = (uint32_t)nsc * kSuper * 16;              // bytes of a tile of eight rows
     // the lane's row of the four 8 x 8 matrices of two mma steps: k = 32 (r / 2) + 2 m + r mod 2, r = lane mod 8, m = lane / 8
     const uint32_t xrow = (uint32_t)__cvta_generic_to_shared(sX) + x_at(32 * ((lane & 7) >> 1) + 2 * (lane >> 3) + (lane & 1));
@@ -232,7 +225,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // ---- x: chunks of a row by consecutive threads ----
     {
-        constexpr int kRows = NB > 8 ? 8 : NB;         // loads in flight per thread
+        constexpr int kRows = 8;                       // loads in flight per thread
         const int chunks = nsc * (kSuper / 8);
         const uint4* xs = (const uint4*)(a.x + (size_t)sc0 * kSuper);
         const int row16 = a.cols / 8;
@@ -244,19 +237,11 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 for (int b = 0; b < kRows; ++b) v[b] = b0 + b < a.nb ? __ldg(xs + (size_t)(b0 + b) * row16 + c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int b = 0; b < kRows; ++b) v[b] = x8_as_f16(v[b], a.x_bf16);
-                if constexpr (kTiles) {
-                    unsigned char* dst = sX + (size_t)(b0 / 8) * tile;
+                unsigned char* dst = sX + (size_t)(b0 / 8) * tile;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {      // k = 8 c + i of the eight rows
-                        auto two = [&](int b) {
-                            const uint32_t lo = word(v[b % kRows], i >> 1), hi = word(v[(b + 1) % kRows], i >> 1);
-                            return __byte_perm(lo, hi, (i & 1) ? 0x7632 : 0x5410);
-                        };
-                        *(uint4*)(dst + x_at(8 * c + i)) = make_uint4(two(0), two(2 % kRows), two(4 % kRows), two(6 % kRows));
-                    }
-                } else {
-#pragma unroll
-                    for (int b = 0; b < kRows; ++b) *(uint4*)(sX + x_chunk<NB>(c, b)) = v[b];
+                for (int i = 0; i < 8; ++i) {          // k = 8 c + i of the eight rows
+                    auto two = [&](int b) { return __byte_perm(word(v[b], i >> 1), word(v[b + 1], i >> 1), (i & 1) ? 0x7632 : 0x5410); };
+                    *(uint4*)(dst + x_at(8 * c + i)) = make_uint4(two(0), two(2), two(4), two(6));
                 }
                 if constexpr (MODE == 1) {
                     // sums of a super-chunk: over the thread's eight k, then over the sixteen threads that hold its chunks
@@ -268,9 +253,9 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                         f[b] = ((p0.x + p0.y) + (p1.x + p1.y)) + ((p2.x + p2.y) + (p3.x + p3.y));
                     }
                     const uint32_t half = 0xffffu << (lane & 16);
-                    int row = 0, d = 1;
+                    int row = 0;
 #pragma unroll
-                    for (int w = kRows / 2; w >= 1; w /= 2, d *= 2) {   // halve the rows a lane keeps
+                    for (int w = kRows / 2, d = 1; w >= 1; w /= 2, d *= 2) {   // halve the rows a lane keeps
                         const bool up = lane & d;
 #pragma unroll
                         for (int b = 0; b < w; ++b) {
@@ -279,8 +264,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                         }
                         if (up) row += w;
                     }
-#pragma unroll
-                    for (; d < 16; d *= 2) f[0] += __shfl_xor_sync(half, f[0], d);
+                    f[0] += __shfl_xor_sync(half, f[0], 8);
                     if ((lane & 15) < kRows) sXg[(c >> 4) * NB + b0 + row] = f[0];
                 }
             }
@@ -339,13 +323,8 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 uint4 xb[NT];
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
-                    if constexpr (kTiles) {
-                        // chunk s2 of each t: the exclusive-or of x_at has s2 as its two low bits
-                        xb[n] = ldmatrix_x4_trans((xrow ^ (uint32_t)(s2 << 4)) + (uint32_t)(lsc * kSuper * 16 + s2 * 128) + n * tile);
-                    } else {
-                        xb[n] = make_uint4(0u, 0u, 0u, 0u);
-                        if (g < NB) xb[n] = *(const uint4*)(sX + x_chunk<NB>(lsc * 16 + 4 * t + s2, g));
-                    }
+                    // chunk s2 of each t: the exclusive-or of x_at has s2 as its two low bits
+                    xb[n] = ldmatrix_x4_trans((xrow ^ (uint32_t)(s2 << 4)) + (uint32_t)(lsc * kSuper * 16 + s2 * 128) + n * tile);
                 }
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
@@ -396,9 +375,8 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
                     const int b = 2 * t + 8 * n;
-                    float x0 = 0.f, x1 = 0.f;
-                    if (b < NB) x0 = sXg[lsc * NB + b];
-                    if (b + 1 < NB) x1 = sXg[lsc * NB + b + 1];
+                    const float2 xs = *(const float2*)(sXg + lsc * NB + b);
+                    const float x0 = xs.x, x1 = xs.y;
 #pragma unroll
                     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -425,23 +403,16 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                 const uint32_t k = (e & 0xffffu) - k0;
                 if (k < kn) {
                     const float v = h2f((uint16_t)(e >> 16));
-                    if constexpr (kTiles) {
 #pragma unroll
-                        for (int n = 0; n < NT; ++n) {
-                            const uint4 x8 = *(const uint4*)(sX + n * tile + x_at((int)k));
-                            const uint32_t u[4] = {x8.x, x8.y, x8.z, x8.w};
+                    for (int n = 0; n < NT; ++n) {
+                        const uint4 x8 = *(const uint4*)(sX + n * tile + x_at((int)k));
+                        const uint32_t u[4] = {x8.x, x8.y, x8.z, x8.w};
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
-                                const float2 f = __half22float2(*(const __half2*)&u[b]);
-                                ao[(8 * n + 2 * b) % NB] = fmaf(v, f.x, ao[(8 * n + 2 * b) % NB]);
-                                ao[(8 * n + 2 * b + 1) % NB] = fmaf(v, f.y, ao[(8 * n + 2 * b + 1) % NB]);
-                            }
+                        for (int b = 0; b < 4; ++b) {
+                            const float2 f = __half22float2(*(const __half2*)&u[b]);
+                            ao[8 * n + 2 * b] = fmaf(v, f.x, ao[8 * n + 2 * b]);
+                            ao[8 * n + 2 * b + 1] = fmaf(v, f.y, ao[8 * n + 2 * b + 1]);
                         }
-                    } else {
-                        const int c = (int)(k >> 3);
-                        const unsigned char* p = sX + (k & 7u) * 2u;
-#pragma unroll
-                        for (int b = 0; b < NB; ++b) ao[b] = fmaf(v, h2f(*(const uint16_t*)(p + x_chunk<NB>(c, b))), ao[b]);
                     }
                 }
             };
@@ -470,7 +441,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int b = 2 * t + 8 * n + (e & 1);
-                    if (b < NB) mine[b * 33 + g + 8 * (2 * i + (e >> 1))] = acc[n][i][e];
+                    mine[b * 33 + g + 8 * (2 * i + (e >> 1))] = acc[n][i][e];
                 }
         __syncwarp();
         if (a.ell_slots) {
@@ -506,17 +477,15 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
     }
 }
 
-struct FragPlan { int S, sc_slice, grid, pair; size_t x_off, red_off, smem; };
+struct FragPlan { int S, sc_slice, grid, pair, room; size_t x_off, red_off, smem; };
 
 size_t table_bytes(const Layout& l, bool pair) {
     if (l.mode) { const int n = (l.L + 1) / 2; return (size_t)(l.bits == 4 ? (n + 1) & ~1 : n) * l.E * 128; }
     return (size_t)4 * (pair ? l.E * l.E : l.E) * 128;
 }
 
-int rows_of(int batch) { return batch <= 1 ? 1 : batch <= 2 ? 2 : batch <= 4 ? 4 : batch <= 8 ? 8 : 16; }
-
 bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
-    const int NB = rows_of(batch);
+    const int NB = batch <= 8 ? 8 : 16;
     const size_t red = (size_t)kFW * NB * 33 * 4 + 16;
     const size_t per_sc = (size_t)kSuper * NB * 2 + (l.mode ? NB * 4 : 0);
     auto slices = [&](bool pair) {                                    // K slices that x needs beside the tables
@@ -533,6 +502,7 @@ bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
         if (!S || s1 < S) { p.pair = 0; S = s1; }
     }
     if (!S) return false;
+    p.room = S;
     // few row-blocks: K slices until the SMs are busy, at least one super-chunk per warp
     while (l.RB * (S + 1) <= sms && l.SC / (S + 1) >= kFW) ++S;
     p.sc_slice = (l.SC + S - 1) / S;
@@ -572,20 +542,36 @@ cudaError_t launch_one(const FragArgs& a, const FragPlan& p, cudaStream_t s) {
 
 template <int N, int MODE, bool PAIR = MODE == 0 && N <= 4>
 cudaError_t launch_rows(int NB, const FragArgs& a, const FragPlan& p, cudaStream_t s) {
-    switch (NB) {
-        case 1: return launch_one<N, MODE, 1, PAIR>(a, p, s);
-        case 2: return launch_one<N, MODE, 2, PAIR>(a, p, s);
-        case 4: return launch_one<N, MODE, 4, PAIR>(a, p, s);
-        case 8: return launch_one<N, MODE, 8, PAIR>(a, p, s);
-        default: return launch_one<N, MODE, 16, PAIR>(a, p, s);
-    }
+    return NB == 8 ? launch_one<N, MODE, 8, PAIR>(a, p, s) : launch_one<N, MODE, 16, PAIR>(a, p, s);
 }
 
-bool frag_preferred(const Layout& l, int batch) {
+// Where this kernel is the faster one.  us per call on a B200, the kernel that otherwise takes the call -> this one, 0.3 %
+// outliers:
+//   * 5 rows and more: everywhere.  4096 x 4096 V2 N = 4, 8 rows 11.0 -> 6.5, 16 rows 21.4 -> 8.5; bf16 x 11.9 -> 7.3; V2a
+//     15.7 -> 8.2.  28672 x 8192, 8 rows: V2 N = 4 74.9 -> 68.7, V2a 103 -> 75.  Only 9 rows and more of fp16 x on a matrix
+//     that fills the chip with tiles of 128 channels stay on the tcgen05 kernel (16 rows, V2 N = 4: 77 against 107).
+//   * A tile has eight rows, whether they are used or not.  3 or 4 rows: V2 N <= 4 up to 2^24 weights (4096 x 4096 N = 4
+//     7.2 -> 6.4; 12288 x 4096 even, 28672 x 8192 53 -> 70) and N = 2 up to 2^26, V2 N >= 5 up to 2^23 (1536 x 4096 N = 5
+//     7.2 -> 6.5; 4096 x 4096 7.5 -> 8.2), V2a up to 2^26 where x needs no K slices (12288 x 4096 26 -> 19; 4096 x 12288 N = 3
+//     22 -> 23) or N = 6; with bf16 x also every V2a matrix (28672 x 8192 N = 4 91 -> 76) and those V2 ones that only the
+//     general kernel takes (12288 x 4096 N = 6 56 -> 24)
+//   * 2 rows: V2a up to 2^23 weights, with bf16 x up to 2^24 and every one of N = 6 (4096 x 4096 N = 4, bf16: 12.2 -> 9.0; fp16
+//     7.7 -> 8.1)
+//   * 1 row: up to 2^19 weights, where a call is launch and latency (256 x 1024 V2 N = 4 4.0 -> 3.1 us)
+bool frag_preferred(const Layout& l, const GemvCall& c, const FragPlan& p) {
+    const long long w = (long long)l.rows * l.cols;
 #ifdef LANE_TUNE
-    if (const char* e = getenv("XFP_FRAG")) return batch >= atoi(e);
+    if (const char* e = getenv("XFP_FRAG")) return c.batch >= atoi(e);
 #endif
-    return batch >= 2;
+    if (c.batch > 8) return c.x_bf16 || !batch_prefers_gemm(l, c.batch);
+    if (c.batch > 4) return true;
+    if (c.batch > 2) {
+        if (c.x_bf16 && (l.mode || !batch_supported(l, c.batch))) return true;
+        if (l.mode) return w <= 1 << 26 && (p.room == 1 || l.bits == 6);
+        return w <= 1 << (l.bits == 2 ? 26 : l.bits <= 4 ? 24 : 23);
+    }
+    if (c.batch == 2) return l.mode && (w <= 1 << (c.x_bf16 ? 24 : 23) || (c.x_bf16 && l.bits == 6));
+    return w <= 1 << 19;
 }
 
 }  // namespace
@@ -593,7 +579,7 @@ bool frag_preferred(const Layout& l, int batch) {
 bool frag_supported(const Layout& l, const GemvCall& c) {
     if (c.n != 1 || c.packed_list || c.epilogue != 0 || l.GH != 1) return false;
     FragPlan p;
-    return frag_preferred(l, c.batch) && plan_frag(l, c.batch, sched_sms(), p);
+    return plan_frag(l, c.batch, sched_sms(), p) && frag_preferred(l, c, p);
 }
 
 cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s) {
@@ -607,7 +593,7 @@ cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s)
     a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.ell_slots = l.ell_slots; a.L = l.L;
     a.nb = c.batch; a.y_kind = c.y_is_fp16; a.x_bf16 = c.x_bf16;
     a.S = p.S; a.sc_slice = p.sc_slice; a.x_off = (int)p.x_off; a.red_off = (int)p.red_off;
-    const int NB = rows_of(c.batch);
+    const int NB = c.batch <= 8 ? 8 : 16;
     if (l.mode) {
         switch (l.bits) {
             case 2: return launch_rows<2, 1>(NB, a, p, s);
