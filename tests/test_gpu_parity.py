@@ -172,6 +172,29 @@ def test_several_rows_of_x_on_matrices_of_one_round(mode, bits, group):
     assert int(tickets.abs().sum().item()) == 0
 
 
+@pytest.mark.parametrize("mode,bits,rows,cols,batch,placement", [
+    (0, 4, 33, 128, 9, "uniform"),          # one super-chunk, a row-block of one channel
+    (1, 5, 97, 1152, 5, "clustered"),       # fewer super-chunks than warps
+    (0, 3, 4767, 384, 16, "uniform"),       # more row-blocks than CTAs, two tiles of rows
+    (0, 4, 96, 16384, 16, "one_row"),       # K slices by the room for x, single-entry tables, a channel beyond its slab
+    (0, 4, 5000, 4224, 8, "uniform"),       # 33 super-chunks in one slice, pair tables built twice
+    (1, 6, 64, 8320, 12, "uniform"),        # K slices of unequal length
+    (1, 2, 31, 256, 2, "uniform"),          # two rows of a tile of eight
+    (0, 2, 40, 640, 3, "one_row"),
+    (0, 6, 70, 4224, 1, "clustered"),       # one row of x
+    (1, 3, 65, 2048, 1, "uniform")])
+def test_batches_in_the_operand_layout(mode, bits, rows, cols, batch, placement):
+    """The kernel of several rows of x at the edges of its tiles and slices; a second call over the same workspace gives the same
+    bits and leaves the counters at zero."""
+    q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=1700 + rows + batch, placement=placement)
+    pm = xfp.pack_tensors(q)
+    x16 = synth.activations(batch, cols, seed=1710 + batch)
+    _, y = _check_gemv(q, pm, x16)
+    y2 = pm.gemv(_x_dev(x16))
+    torch.cuda.synchronize()
+    assert torch.equal(y, y2) and int(pm.workspace[:4 * ((rows + 31) // 32)].view(torch.int32).abs().sum()) == 0
+
+
 @pytest.mark.parametrize("mode,bits,rows,cols", [(0, 6, 9600, 2048), (0, 5, 9700, 1024), (1, 4, 19200, 512), (1, 2, 9600, 2048),
                                                  (1, 6, 4800, 1024), (1, 3, 19000, 512)])
 def test_several_rows_of_x_with_resident_ctas_and_a_cut_tail(mode, bits, rows, cols):
