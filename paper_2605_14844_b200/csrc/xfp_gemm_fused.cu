@@ -112,12 +112,6 @@ __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st
 __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
-// lo | hi << 16 for words whose upper halves are zero, on the FMA pipe (the decode leans on the ALU pipe)
-__device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) {
-    uint32_t d;
-    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
-    return d;
-}
 // K-major operand descriptors (version 1).  A: core matrices of 8 rows x 16 bytes, the next 8 k 2048 bytes on, the next 8
 // rows 128 bytes on, no swizzle.  B: rows of 128 bytes in the 128-byte swizzle, 8 rows 1024 bytes.
 __device__ __forceinline__ uint64_t desc_a(uint32_t addr) {

@@ -344,22 +344,22 @@ __global__ void __launch_bounds__(kFThreads, 1) gemv_frag_kernel(const FragArgs 
                                 const uint32_t lb = lbase | ((j & 1) * 128u), sel = 0x7604u | ((uint32_t)(p & 3) << 4);
                                 const uint32_t lo = *(const uint32_t*)(smem + T::at(j & ~1) + __byte_perm(w[p >> 2] & 0x0f0f0f0fu, lb, sel));
                                 const uint32_t hi = *(const uint32_t*)(smem + T::at(j & ~1) + __byte_perm((w[p >> 2] >> 4) & 0x0f0f0f0fu, lb, sel));
-                                av[j][v] = lo | (hi << 16);
+                                av[j][v] = join16(lo, hi);
                             } else if (MODE == 0) {
                                 const uint32_t lo = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p, lbase));
                                 const uint32_t hi = *(const uint32_t*)(smem + T::at(j) + single_addr<N, 1>(w, 2 * p + 1, lbase));
-                                av[j][v] = lo | (hi << 16);
+                                av[j][v] = join16(lo, hi);
                             } else if (N == 4) {
                                 // byte 1 of the address: index and the low four bits of id / 4
                                 const uint32_t nib = ((base[j] >> 12) & 0xfu) * 0x10101010u, sel = 0x7604u | ((uint32_t)(p & 3) << 4);
                                 const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
                                 const uint32_t lo = *(const uint16_t*)(smem + __byte_perm(wlo, base[j], sel));
                                 const uint32_t hi = *(const uint16_t*)(smem + __byte_perm(whi, base[j], sel));
-                                av[j][v] = lo | (hi << 16);
+                                av[j][v] = join16(lo, hi);
                             } else {
                                 const uint32_t lo = *(const uint16_t*)(smem + single_addr<N, 1>(w, 2 * p, base[j]));
                                 const uint32_t hi = *(const uint16_t*)(smem + single_addr<N, 1>(w, 2 * p + 1, base[j]));
-                                av[j][v] = lo | (hi << 16);
+                                av[j][v] = join16(lo, hi);
                             }
                         }
 #pragma unroll

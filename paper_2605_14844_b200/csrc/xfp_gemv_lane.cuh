@@ -87,10 +87,10 @@ __device__ __forceinline__ void lookup8(uint32_t (&f)[4], const uint32_t* w, int
         uint32_t e[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = *(const uint16_t*)(tab + single_addr<N, 1>(w, 8 * j + i, base));
-        f[0] = __byte_perm(e[0], e[1], 0x5410);
-        f[2] = __byte_perm(e[2], e[3], 0x5410);
-        f[1] = __byte_perm(e[4], e[5], 0x5410);
-        f[3] = __byte_perm(e[6], e[7], 0x5410);
+        f[0] = join16(e[0], e[1]);
+        f[2] = join16(e[2], e[3]);
+        f[1] = join16(e[4], e[5]);
+        f[3] = join16(e[6], e[7]);
     } else if (QUAD) {
         // bytes 2j and 2j+1 of the stream; base = lane * 8
         const uint32_t a0 = __byte_perm(w[(2 * j) >> 2], base, 0x5504u | ((uint32_t)((2 * j) & 3) << 4));
@@ -102,10 +102,10 @@ __device__ __forceinline__ void lookup8(uint32_t (&f)[4], const uint32_t* w, int
         uint32_t e[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = *(const uint32_t*)(tab + single_addr<N, 1>(w, 8 * j + i, base));
-        f[0] = __byte_perm(e[0], e[1], 0x5410);
-        f[2] = __byte_perm(e[2], e[3], 0x5410);
-        f[1] = __byte_perm(e[4], e[5], 0x5410);
-        f[3] = __byte_perm(e[6], e[7], 0x5410);
+        f[0] = join16(e[0], e[1]);
+        f[2] = join16(e[2], e[3]);
+        f[1] = join16(e[4], e[5]);
+        f[3] = join16(e[6], e[7]);
     } else {
         constexpr int SL = N == 4 ? 2 : 1;   // N = 4: entries 256 bytes apart
         f[0] = *(const uint32_t*)(tab + pair_addr<N, SL>(w, 4 * j, base));

@@ -35,6 +35,7 @@
 #include <utility>
 
 #include "xfp_internal.h"
+#include "xfp_pair_common.cuh"
 
 namespace xfp {
 
@@ -339,10 +340,10 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
         const uint32_t l11 = *(const uint32_t*)(tab + entry_addr<N>(w1, 4 * m + 1, base1));
         const uint32_t l12 = *(const uint32_t*)(tab + entry_addr<N>(w1, 4 * m + 2, base1));
         const uint32_t l13 = *(const uint32_t*)(tab + entry_addr<N>(w1, 4 * m + 3, base1));
-        f[0] = __byte_perm(l00, l01, 0x5410);   // (k, k+1) of channel 0
-        f[1] = __byte_perm(l10, l11, 0x5410);   // (k, k+1) of channel 1
-        f[2] = __byte_perm(l02, l03, 0x5410);   // (k+2, k+3) of channel 0
-        f[3] = __byte_perm(l12, l13, 0x5410);   // (k+2, k+3) of channel 1
+        f[0] = join16(l00, l01);   // (k, k+1) of channel 0
+        f[1] = join16(l10, l11);   // (k, k+1) of channel 1
+        f[2] = join16(l02, l03);   // (k+2, k+3) of channel 0
+        f[3] = join16(l12, l13);   // (k+2, k+3) of channel 1
     };
 
 #pragma unroll 1

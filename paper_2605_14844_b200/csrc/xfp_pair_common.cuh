@@ -12,6 +12,13 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// lo | hi << 16 for words whose upper halves are zero, on the FMA pipe (the decode leans on the ALU pipe)
+__device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
+    return d;
+}
+
 // Byte offset of the table entry of pair p (compile time) of a 128-weight stream w[4N]:
 // t * 128 * RPL merged with `base` (= channel_half * 128 + lane * 4, below the t field).
 template <int N, int RPL>
