@@ -85,8 +85,17 @@ __device__ __forceinline__ void lookup8(uint32_t (&f)[4], const uint32_t* w, int
     if (HALF) {
         // V2a, one entry per index: a word holds the entry of TWO library ids, `base` selects the half
         uint32_t e[8];
+        if (N == 4) {
+            // step j's eight indices are word j: byte 1 of the address = index and the low four bits of the table's place
+            const uint32_t nib = ((base >> 12) & 0xfu) * 0x10101010u;
+            const uint32_t lo = (w[j] & 0x0f0f0f0fu) | nib, hi = ((w[j] >> 4) & 0x0f0f0f0fu) | nib;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = *(const uint16_t*)(tab + single_addr<N, 1>(w, 8 * j + i, base));
+            for (int i = 0; i < 8; ++i)
+                e[i] = *(const uint16_t*)(tab + __byte_perm((i & 1) ? hi : lo, base, 0x7604u | ((uint32_t)(i >> 1) << 4)));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = *(const uint16_t*)(tab + single_addr<N, 1>(w, 8 * j + i, base));
+        }
         f[0] = join16(e[0], e[1]);
         f[2] = join16(e[2], e[3]);
         f[1] = join16(e[4], e[5]);
@@ -229,6 +238,15 @@ __device__ __forceinline__ void fill_tables_v2(unsigned char* tab, uint32_t* cbs
     }
 }
 
+// V2a, a word per entry of two library ids: the byte offset of row e = m 2^N + q, the entry q of ids 2m and 2m + 1.  At N = 4 the
+// tables of two m are interleaved and entries lie 256 bytes apart, so that one PRMT builds an address from an index (a shift
+// and a mask per weight kept the ALU pipe busiest).
+template <int N>
+__device__ __forceinline__ uint32_t half_row(uint32_t e) {
+    if (N != 4) return e * 128u;
+    return (e >> 5) * 4096u + ((e >> 4) & 1u) * 128u + (e & 15u) * 256u;
+}
+
 // V2a tables: every row is one word repeated in the 32 banks -- HALF: row (id / 2) * 2^N + q holds lib[id][q] of ids
 // 2m (low half) and 2m + 1 (high half); else the pair table, row id * 4^N + (q1 << N | q0) holds (lib[id][q0],
 // lib[id][q1]).  A lane fetches the word of row e0 + lane, then the warp stores the 32 rows one after the other, each word
@@ -245,7 +263,7 @@ __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __
             const int m = e >> N, q = e & (E - 1);
             const uint32_t lo = __ldg(lib + (size_t)(2 * m) * E + q);
             const uint32_t hi = 2 * m + 1 < L ? (uint32_t)__ldg(lib + (size_t)(2 * m + 1) * E + q) : 0u;
-            *(uint32_t*)(tab + (size_t)e * 128 + lane * 4) = lo | (hi << 16);
+            *(uint32_t*)(tab + half_row<N>(e) + lane * 4) = lo | (hi << 16);
         }
         return;
     }
@@ -265,7 +283,7 @@ __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const uint32_t v = __shfl_sync(0xffffffffu, word, r);
-            if (e0 + r < trows) *(uint32_t*)(tab + (size_t)(e0 + r) * 128 + lane * 4) = v;
+            if (e0 + r < trows) *(uint32_t*)(tab + (HALF ? half_row<N>(e0 + r) : (e0 + r) * 128u) + lane * 4) = v;
         }
     }
 }
@@ -322,7 +340,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     const int src_a = (lane & ~3) | (t4 >> 1);
     // V2a: table offset of library id `id`
     auto id_offset = [](uint32_t id) -> uint32_t {
-        return kHalf ? (id >> 1) * (uint32_t)kIdBytes + (id & 1u) * 2u : id * (uint32_t)kIdBytes;
+        return kHalf ? half_row<N>((id >> 1) * (uint32_t)E) + (id & 1u) * 2u : id * (uint32_t)kIdBytes;
     };
 
 #pragma unroll 1
@@ -424,13 +442,13 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
                 }
 #pragma unroll
                 for (int i = 0; i < kRows; ++i)
-                    *(uint32_t*)(tab + (size_t)(warp + i * W) * 128 + lane * 4) = lo[i] | (hi[i] << 16);
+                    *(uint32_t*)(tab + half_row<N>(warp + i * W) + lane * 4) = lo[i] | (hi[i] << 16);
             } else {
                 for (int e = warp; e < ((a.L + 1) >> 1) * E; e += W) {
                     const int m = e >> N, q = e & (E - 1);
                     const uint32_t lo = __ldg(b.cb + (size_t)(2 * m) * E + q);
                     const uint32_t hi = 2 * m + 1 < a.L ? (uint32_t)__ldg(b.cb + (size_t)(2 * m + 1) * E + q) : 0u;
-                    *(uint32_t*)(tab + (size_t)e * 128 + lane * 4) = lo | (hi << 16);
+                    *(uint32_t*)(tab + half_row<N>(e) + lane * 4) = lo | (hi << 16);
                 }
             }
         }
@@ -696,7 +714,8 @@ inline size_t lane_tab_bytes(const Layout& l, bool sgl) {
     const size_t E = (size_t)1 << bits;
     if (l.mode) {   // the library, one copy per bank: a word per entry (per pair of entries), or half a word when that does not fit
         if (!sgl) return (size_t)l.L * E * E * 128;
-        return (size_t)((l.L + 1) / 2) * E * 128;   // a word holds one entry of two library ids
+        const size_t tables = (size_t)(l.L + 1) / 2;
+        return (bits == 4 ? (tables + 1) & ~size_t(1) : tables) * E * 128;   // (two interleaved at N = 4) a word holds one entry of two library ids
     }
     if (bits == 2) return 256 * 256;
     if (sgl) return E * 128;
