@@ -135,73 +135,109 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     const int per = epi == 2 ? a.comb_ng : 1;
     const int nrun = epi == 2 ? a.blocks * a.comb_G : a.items_x * a.n;
     float csum = 0.f;   // epi 2: this thread's channel, weighted sum over the blobs of the run
+    int run = blockIdx.x, jj = 0;
+    if (run >= nrun) return;
+    // where an item lies: blob, block, K slice
+    struct Item { int prob, bx, blk, ks, KS, sc0, nsc; };
+    auto locate = [&](int run_, int jj_) {
+        Item t;
+        if (epi == 2) {
+            t.bx = run_ / a.comb_G;
+            t.prob = (run_ - t.bx * a.comb_G) * a.comb_ng + jj_;
+        } else {
+            t.prob = run_ / a.items_x;
+            t.bx = run_ - t.prob * a.items_x;
+        }
+        int spp;
+        if (t.bx < a.n_full) {
+            t.blk = t.bx; t.ks = 0; t.KS = 1; spp = a.SC;
+        } else if (t.bx - a.n_full < a.n_a * a.kst) {
+            const int c = t.bx - a.n_full;
+            t.blk = a.n_full + c / a.kst; t.ks = c % a.kst; t.KS = a.kst; spp = a.sc_per_split;
+        } else {
+            const int c = t.bx - a.n_full - a.n_a * a.kst;
+            t.blk = a.n_full + a.n_a + c / a.kst_b; t.ks = c % a.kst_b; t.KS = a.kst_b; spp = a.sc_per_split_b;
+        }
+        t.sc0 = t.ks * spp;
+        t.nsc = max(0, min(a.SC, t.sc0 + spp) - t.sc0);
+        return t;
+    };
+    // a blob and the geometry of its outlier slabs (launches over several blobs read it from each: their counts differ)
+    const void* packed; const uint32_t* ell; int ell_slots;
+    auto open = [&](int prob, const void*& p, const uint32_t*& e, int& slots) {
+        if (a.packed_list) {
+            p = a.packed_list[prob];
+            const int* hdr = (const int*)((const char*)p + a.off.hdr);
+            slots = __ldg(hdr);
+            e = (const uint32_t*)((const char*)p + *(const long long*)(hdr + 2));
+        } else {
+            p = a.packed; slots = a.ell_slots; e = blob_at(p, a.off).ell;
+        }
+    };
+    // registers that an item's first loads arrive in: indices and group metadata of this warp's first super-chunk of both
+    // channels, slot counts and first slots of its outliers
+    uint32_t w0[4 * N + 1], w1[4 * N + 1];
+    w0[4 * N] = w1[4 * N] = 0u;
+    uint32_t id0 = 0, id1 = 0, sm0 = 0, sm1 = 0;              // current group: library ids and (scale, mid)
+    uint32_t nid0 = 0, nid1 = 0, nsm0 = 0, nsm1 = 0;          // next group
+    uint32_t olen[2], oe[2][kASlots];
+    auto issue = [&](const Item& t, const void* p, const uint32_t* e, int slots) {
+        const Blob b = blob_at(p, a.off);
+        const int r0 = 2 * t.blk, r1 = min(2 * t.blk + 1, a.RB - 1);
+        if (warp < t.nsc) {
+            const size_t g0 = (size_t)r0 * a.SC + t.sc0 + warp, g1 = (size_t)r1 * a.SC + t.sc0 + warp;
+#pragma unroll
+            for (int v = 0; v < N; ++v) {
+                const uint4 t0 = ld_stream(b.idx + (g0 * N + v) * 32 + lane);
+                const uint4 t1 = ld_stream(b.idx + (g1 * N + v) * 32 + lane);
+                w0[4 * v] = t0.x; w0[4 * v + 1] = t0.y; w0[4 * v + 2] = t0.z; w0[4 * v + 3] = t0.w;
+                w1[4 * v] = t1.x; w1[4 * v + 1] = t1.y; w1[4 * v + 2] = t1.z; w1[4 * v + 3] = t1.w;
+            }
+            id0 = b.gid[g0 * 32 + lane]; id1 = b.gid[g1 * 32 + lane];
+            sm0 = b.gsm[g0 * 32 + lane]; sm1 = b.gsm[g1 * 32 + lane];
+        }
+        const int first = t.ks * kAWarps + warp, stride = t.KS * kAWarps;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t* sl = e + (size_t)(h ? r1 : r0) * (slots + 1) * 32 + lane;
+            olen[h] = slots ? __ldg(sl) : 0u;
+#pragma unroll
+            for (int q = 0; q < kASlots; ++q) {
+                const int j = first + q * stride;
+                oe[h][q] = j < slots ? __ldg(sl + (size_t)(1 + j) * 32) : 0u;
+            }
+        }
+    };
+    Item item = locate(run, 0);
+    open(item.prob, packed, ell, ell_slots);
+    issue(item, packed, ell, ell_slots);
 #pragma unroll 1
-    for (int run = blockIdx.x; run < nrun; run += gridDim.x) {
-#pragma unroll 1
-    for (int jj = 0; jj < per; ++jj) {
-    int prob, bx;
-    if (epi == 2) {
-        bx = run / a.comb_G;
-        prob = (run - bx * a.comb_G) * a.comb_ng + jj;
-        if (prob >= a.n) break;
-        if (jj == 0) csum = 0.f;
-    } else {
-        prob = run / a.items_x;
-        bx = run - prob * a.items_x;
-    }
-    int blk, ks, KS, spp;
-    if (bx < a.n_full) {
-        blk = bx; ks = 0; KS = 1; spp = a.SC;
-    } else if (bx - a.n_full < a.n_a * a.kst) {
-        const int t = bx - a.n_full;
-        blk = a.n_full + t / a.kst; ks = t % a.kst; KS = a.kst; spp = a.sc_per_split;
-    } else {
-        const int t = bx - a.n_full - a.n_a * a.kst;
-        blk = a.n_full + a.n_a + t / a.kst_b; ks = t % a.kst_b; KS = a.kst_b; spp = a.sc_per_split_b;
-    }
+    for (;;) {
+    const int prob = item.prob, bx = item.bx, blk = item.blk, ks = item.ks, KS = item.KS, sc0 = item.sc0, nsc = item.nsc;
+    if (jj == 0) csum = 0.f;
     const float epi_wj = epi == 2 ? __ldg(a.epi_w + prob) : 0.f;   // fetched now, used in the store
-    const void* packed = a.packed_list ? a.packed_list[prob] : a.packed;
     const uint16_t* x = a.x_list ? a.x_list[prob] : a.x;
     void* y = a.y_list ? a.y_list[prob] : a.y;
     const Blob b = blob_at(packed, a.off);
-    const int sc0 = ks * spp;
-    const int nsc = max(0, min(a.SC, sc0 + spp) - sc0);
-
+    // the CTA's next item: its pointers travel under this one's K loop, its first loads under this one's reduction (an item is
+    // two groups per warp on the routed experts' shapes, and the chain pointer - header - slab cost as much as one of them)
+    const bool same_run = epi == 2 && jj + 1 < per && prob + 1 < a.n;
+    const int run_n = same_run ? run : run + (int)gridDim.x, jj_n = same_run ? jj + 1 : 0;
+    const bool more = (PAIR || a.persist) && run_n < nrun;
+    Item item_n = item;
+    const void* packed_n = packed; const uint32_t* ell_n = ell; int slots_n = ell_slots;
+    if (more) {
+        item_n = locate(run_n, jj_n);
+        open(item_n.prob, packed_n, ell_n, slots_n);
+    }
     const int blk0 = 2 * blk;
     const int blk1 = min(2 * blk + 1, a.RB - 1);              // clamped when RB is odd; its results are dropped
-
-    // ---- (0) start streaming: first super-chunk of this warp (indices and group metadata of both channels)
-    uint32_t w0[4 * N + 1], w1[4 * N + 1];
-    w0[4 * N] = w1[4 * N] = 0u;
     const uint4* i0 = b.idx + ((size_t)(blk0 * a.SC + sc0) * N) * 32 + lane;
     const uint4* i1 = b.idx + ((size_t)(blk1 * a.SC + sc0) * N) * 32 + lane;
     const size_t m0 = (size_t)(blk0 * a.SC + sc0) * 32 + lane, m1 = (size_t)(blk1 * a.SC + sc0) * 32 + lane;
-    uint32_t id0 = 0, id1 = 0, sm0 = 0, sm1 = 0;              // current group: library ids and (scale, mid)
-    uint32_t nid0 = 0, nid1 = 0, nsm0 = 0, nsm1 = 0;          // next group
-    if (warp < nsc) {
-#pragma unroll
-        for (int v = 0; v < N; ++v) {
-            const uint4 t0 = ld_stream(i0 + ((size_t)warp * N + v) * 32);
-            const uint4 t1 = ld_stream(i1 + ((size_t)warp * N + v) * 32);
-            w0[4 * v] = t0.x; w0[4 * v + 1] = t0.y; w0[4 * v + 2] = t0.z; w0[4 * v + 3] = t0.w;
-            w1[4 * v] = t1.x; w1[4 * v + 1] = t1.y; w1[4 * v + 2] = t1.z; w1[4 * v + 3] = t1.w;
-        }
-        id0 = b.gid[m0 + (size_t)warp * 32]; id1 = b.gid[m1 + (size_t)warp * 32];
-        sm0 = b.gsm[m0 + (size_t)warp * 32]; sm1 = b.gsm[m1 + (size_t)warp * 32];
-    }
-    // outlier slabs of this CTA's two row-blocks: slots gw, gw + stride, ... belong to this warp.  Launches
-    // over several blobs read the slab geometry from each blob (their outlier counts differ).
-    int ell_slots = a.ell_slots;
-    const uint32_t* ell = b.ell;
-    if (a.packed_list) {
-        const int* hdr = (const int*)((const char*)packed + a.off.hdr);
-        ell_slots = __ldg(hdr);
-        ell = (const uint32_t*)((const char*)packed + *(const long long*)(hdr + 2));
-    }
+    // outlier slabs of this CTA's two row-blocks: slots gw, gw + stride, ... belong to this warp
     const int gw = ks * kAWarps + warp, ostride = KS * kAWarps;
     const uint32_t* slab[2];
-    uint32_t olen[2];
-    uint32_t oe[2][kASlots];
     int width[2];
     float acc[NB][2];
     int oround = 0, nrounds = 0;
@@ -209,7 +245,6 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     for (int h = 0; h < 2; ++h) {
         slab[h] = ell + (size_t)(h ? blk1 : blk0) * (ell_slots + 1) * 32 + lane;
         width[h] = ell_slots;
-        olen[h] = ell_slots ? __ldg(slab[h]) : 0u;
 #pragma unroll
         for (int bb = 0; bb < NB; ++bb) acc[bb][h] = 0.f;
     }
@@ -233,10 +268,10 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
                 for (int bb = 0; bb < NB; ++bb) acc[bb][h] = fmaf(v, h2f(xs[(size_t)bb * K + col]), acc[bb][h]);
             }
     };
-    if (ell_slots) fetch_slots(0);
 
     // ---- (1) library tables (after the item's first loads are on their way).  The blobs of a launch normally share one library (one per layer), so the tables are
     //      built once per CTA; a blob whose library differs from the one they were built from rebuilds them.
+    bool fresh = false;
     {
         const uint4* cb4 = (const uint4*)b.cb;
         const int nvec = a.L * E / 8;   // the library in 16-byte vectors (L * E is a multiple of 8)
@@ -246,7 +281,9 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
                 const uint4 u = __ldg(cb4 + i), v = libcopy[i];
                 differs |= (u.x != v.x) | (u.y != v.y) | (u.z != v.z) | (u.w != v.w);
             }
+        // (also the barrier behind which the previous item's sums and flag may be overwritten)
         if (__syncthreads_or(differs)) {
+            fresh = true;
             for (int i = threadIdx.x; i < nvec; i += kAThreads) libcopy[i] = __ldg(cb4 + i);
             if (PAIR) {
                 // pair tables, 16 copies: words (id * E*E + pair) * 16 .. + 15 hold the same half2.  Four threads per
@@ -301,8 +338,9 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
             if (lane == 0) xg[u] = t;
         }
         x_staged = x;
+        fresh = true;
     }
-    __syncthreads();   // tables, x and X_g visible
+    if (fresh) __syncthreads();   // tables, x and X_g visible
 #pragma unroll
     for (int h = 0; h < 2; ++h) {   // the rows' slot counts have arrived: this warp's number of outlier rounds
         int wmax = (int)olen[h];
@@ -433,6 +471,8 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
         }
     }
 
+    if (more) issue(item_n, packed_n, ell_n, slots_n);
+
     // ---- (4) fixed-order reduction over the warps, store or split-K finish
 #pragma unroll
     for (int bb = 0; bb < NB; ++bb) {
@@ -518,10 +558,8 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
             }
         }
     }
-    if (!PAIR && !a.persist) break;   // the per-bank library is launched with one CTA per item
-    __syncthreads();   // red, x and the ticket flag are reused by the CTA's next item
-    }
-    if (!PAIR && !a.persist) break;
+    if (!more) break;   // (the per-bank library may be launched with one CTA per item)
+    item = item_n; packed = packed_n; ell = ell_n; ell_slots = slots_n; run = run_n; jj = jj_n;
     }
 }
 
