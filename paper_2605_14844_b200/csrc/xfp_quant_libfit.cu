@@ -16,20 +16,26 @@ namespace cg = cooperative_groups;
 
 // ------------------------------------------------------------------ the library
 
-constexpr int kLibThreads = 256;
-constexpr int kLibTile = 2048;      // channels whose members are compacted at a time
+constexpr int kLibThreads = 512;
+constexpr int kLibTile = 4096;      // channels whose members are compacted at a time
 constexpr int kLibVals = 2048;      // member values staged at a time
+constexpr size_t kLibSmemU = 160 * 1024;   // normalised codebooks of this size stay in every block's shared memory
 
 // The whole k-means in one cooperative launch: normalise, order by norm, seed, `iters` rounds of assignment and update,
 // store.  As separate launches (three per round) the rounds were bound by launches and by the update's chain of dependent
 // loads: 3072 channels, N = 2, 20 rounds 515 us; here a round costs two grid barriers and the update's serial sums.
 //   assignment  a warp per channel, a lane per centroid (32 at a time); every lane sums its squared distance in entry
 //               order and the smallest (distance, centroid) pair wins: the answer of a scan with a strict "less than"
-//   update      a block per centroid compacts its members in channel order, stages their entries in shared memory, and
-//               thread j adds them to entry j one by one: the order of the serial evaluation
+//   update      a block per centroid compacts its members in channel order, and thread j adds their entries j one by one:
+//               the order of the serial evaluation
+// A round is a chain of latencies (the two barriers, L2 round trips, the serial sums).  Where the normalised codebooks fit
+// (resident: 3072 channels of N = 2 are 96 KB) every block keeps them in shared memory, which takes the L2 round trip out of
+// each channel's assignment and the staging of the members out of the update (quantising 3072 x 4096 at N = 2 in all: 723 -> 677 us); larger ones are read from
+// L2.
 __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint16_t* __restrict__ cb, int rows, int E, int L,
                                                                      int iters, double* u, double* nn, int* order, int* asg,
-                                                                     double* cen, int* flag, uint16_t* lib) {
+                                                                     double* cen, int* flag, uint16_t* lib, int resident) {
+    extern __shared__ double su[];      // resident: u
     __shared__ int sh[32];
     __shared__ int total;
     __shared__ int member[kLibTile];
@@ -59,6 +65,11 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
     }
     if (gt < 3) flag[gt] = 0;
     grid.sync();
+    if (resident) {                     // (used behind the next barriers)
+        const int n2 = rows * E / 2;    // E is even
+#pragma unroll 4
+        for (int i = tid; i < n2; i += kLibThreads) ((double2*)su)[i] = __ldcg((const double2*)u + i);
+    }
     // order[r] = the channel of rank r by (nn, channel): rank by counting
     for (int i = gw; i < rows; i += nw) {
         const double mine = __ldcg(nn + i);
@@ -96,7 +107,8 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
                     d = 0.0;
 #pragma unroll 4
                     for (int j = 0; j < E; ++j) {
-                        const double t = __dsub_rn(__ldcg(u + (int64_t)i * E + j), staged ? vals[j * L + l] : __ldcg(cen + l * E + j));
+                        const double x = resident ? su[i * E + j] : __ldcg(u + (int64_t)i * E + j);
+                        const double t = __dsub_rn(x, staged ? vals[j * L + l] : __ldcg(cen + l * E + j));
                         d = __dadd_rn(d, __dmul_rn(t, t));
                     }
                 }
@@ -119,16 +131,25 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
             for (int i0 = 0; i0 < rows; i0 += kLibTile) {
                 constexpr int per = kLibTile / kLibThreads;
                 int hit = 0;
+                static_assert(per % 4 == 0, "whole vectors of assignments");
 #pragma unroll
-                for (int e = 0; e < per; ++e) {
+                for (int e = 0; e < per; e += 4) {
                     const int i = i0 + tid * per + e;
-                    if (i < rows && __ldcg(asg + i) == l) hit |= 1 << e;
+                    int4 t = make_int4(-1, -1, -1, -1);
+                    if (i + 3 < rows) t = __ldcg((const int4*)(asg + i));
+                    else if (i < rows) { t.x = __ldcg(asg + i); if (i + 1 < rows) t.y = __ldcg(asg + i + 1); if (i + 2 < rows) t.z = __ldcg(asg + i + 2); }
+                    hit |= ((t.x == l) | (t.y == l) << 1 | (t.z == l) << 2 | (t.w == l) << 3) << e;
                 }
                 int at = block_excl_scan(__popc(hit), sh, &total);
                 for (int e = 0; e < per; ++e)
                     if ((hit >> e) & 1) member[at++] = i0 + tid * per + e;
                 __syncthreads();
                 const int n = total, chunk = kLibVals / E;
+                if (resident && tid < E) {
+#pragma unroll 8
+                    for (int m = 0; m < n; ++m) acc = __dadd_rn(acc, su[member[m] * E + tid]);
+                }
+                if (!resident)
                 for (int m0 = 0; m0 < n; m0 += chunk) {
                     const int c = n - m0 < chunk ? n - m0 : chunk;
                     for (int i = tid; i < c * E; i += kLibThreads) vals[i] = __ldcg(u + (int64_t)member[m0 + i / E] * E + i % E);
@@ -465,8 +486,18 @@ cudaError_t launch_libfit_library(const uint16_t* codebook, int rows, int E, int
     const int want = (rows + kLibThreads / 32 - 1) / (kLibThreads / 32), sms = xfp::sm_count();
     int blocks = want > L ? want : L;
     if (blocks > sms) blocks = sms;
-    void* args[] = {&codebook, &rows, &E, &L, &iters, &u, &nn, &order, &asg, &cen, &flags, &lib};
-    return cudaLaunchCooperativeKernel((const void*)libfit_library_kernel, dim3((unsigned)blocks), dim3(kLibThreads), args, 0, s);
+    size_t smem = (size_t)rows * E * sizeof(double);
+    int resident = smem <= kLibSmemU;
+    if (!resident) smem = 0;
+    static xfp::DeviceOnce attr_done;
+    const int dev = xfp::DeviceOnce::current();
+    if (!attr_done.is_set(dev)) {
+        const cudaError_t e = cudaFuncSetAttribute(libfit_library_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLibSmemU);
+        if (e != cudaSuccess) return e;
+        attr_done.set(dev);
+    }
+    void* args[] = {&codebook, &rows, &E, &L, &iters, &u, &nn, &order, &asg, &cen, &flags, &lib, &resident};
+    return cudaLaunchCooperativeKernel((const void*)libfit_library_kernel, dim3((unsigned)blocks), dim3(kLibThreads), args, smem, s);
 }
 
 }  // namespace xq

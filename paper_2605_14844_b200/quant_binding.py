@@ -169,15 +169,15 @@ def quantize_and_pack(W: torch.Tensor, mode: int, candidates: Sequence[int], tau
     group = params.group_size or 128
     buf = QuantBuffers(rows, cols, mode, max(candidates), lib_size, int(frac * rows * cols), device=W.device,
                        group_size=group)
-    res = xfp_quantize(mode, W, params, candidates, tau, buf, stream)
+    err = torch.zeros(1, dtype=torch.int32, device=W.device)
+    res = xfp_quantize(mode, W, params, candidates, tau, buf, stream)   # waits for the width and the count it chose
     E = 1 << res.bits
     desc = XfpDesc(mode, rows, cols, res.bits, group, lib_size if mode else 0, 32, int(res.nnz))
     pb, wb = xfp_packed_size(desc)
     packed = torch.empty(pb, dtype=torch.uint8, device=W.device)
-    workspace = torch.zeros(max(wb, 16), dtype=torch.uint8, device=W.device)
-    err = torch.zeros(1, dtype=torch.int32, device=W.device)
     table = (buf.lib.view(-1)[:lib_size * E] if mode else buf.codebook.view(-1)[:rows * E]).contiguous()
     xfp_pack(desc, buf.idx, table, buf.gid, buf.gscale, buf.gmid, buf.rowptr, buf.ocol, buf.oval, packed, err, stream)
+    workspace = torch.zeros(max(wb, 16), dtype=torch.uint8, device=W.device)   # under the pack kernel
     return PackedMatrix(desc, packed, workspace, err), res
 
 
