@@ -105,7 +105,7 @@ __device__ __forceinline__ uint32_t pair_entry_addr(const uint32_t* w, int p, ui
 
 // FEAT instantiations carry typed IO (bf16 x, bf16 y) and the fused stores; the plain ones compile them out.
 template <int N, int NB, int W, bool PAIR, bool FEAT>
-__global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const V2aArgs a) {
+__global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_kernel(const V2aArgs a) {
     const int epi = FEAT ? a.epi : 0;
     constexpr int E = 1 << N;
     constexpr int kAWarps = W;
@@ -575,7 +575,7 @@ static size_t v2a_smem_bytes(const Layout& l, int nb, bool pair, int warps) {
            (size_t)l.L * l.E * 2 + 16;   // + the copy of the library the tables were built from, 16-byte aligned
 }
 
-static V2aConfig v2a_config(const Layout& l, int nb, int n = 1) {
+static V2aConfig v2a_config(const Layout& l, int nb, int n = 1, int epilogue = 0) {
     // Pair tables cost 128 KB of fills per resident CTA and run one CTA of 12 or 16 warps per SM: they pay off
     // when every SM has a few hundred thousand weights to decode and K is long enough to keep those warps busy
     // (measured: 28672 x 8192 53 vs 61 us, 8192 x 8192 18.6 vs 22.9, 12288 x 4096 18.7 vs 20.0 in their favour;
@@ -588,6 +588,13 @@ static V2aConfig v2a_config(const Layout& l, int nb, int n = 1) {
         const size_t sm = v2a_smem_bytes(l, nb, true, warps);
         if (sm <= 224u * 1024u) return V2aConfig{true, warps, sms, sm};
     }
+    // The weighted sum over the blobs (K is the routed experts' short hidden size) with more items than two CTAs per SM: four
+    // CTAs of four warps leave fewer warps without a group (12 groups are 3 each, against 2 or 1 of 8 warps) and wait for one
+    // another at four barriers instead of two.  Routed block of 8 experts, N = 3: 4096 x 1536 49.9 -> 47.1 us, 7168 x 2048
+    // 101.9 -> 95.8; with fewer items the SMs run out of warps (6144 x 2560, 2 experts: 39.5 -> 50.6).
+    const size_t sm4 = v2a_smem_bytes(l, nb, false, 4);
+    if (epilogue == 2 && l.bits <= 3 && (long long)((l.RB + 1) / 2) * n > 2 * sms && sm4 <= 55u * 1024u)
+        return V2aConfig{false, 4, 4 * sms, sm4};
     const size_t sm8 = v2a_smem_bytes(l, nb, false, 8);
     if (sm8 <= 110u * 1024u) return V2aConfig{false, 8, 2 * sms, sm8};
     return V2aConfig{false, 16, sms, v2a_smem_bytes(l, nb, false, 16)};   // large library (N = 5): one CTA per SM
@@ -612,7 +619,7 @@ static cudaError_t launch_v2a_feat(const V2aArgs& a, dim3 grid, size_t smem, cud
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
         cudaError_t e = cudaFuncSetAttribute(gemv_v2a_kernel<N, NB, W, PAIR, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             W == 8 ? 112 * 1024 : 226 * 1024);
+                                             W == 4 ? 56 * 1024 : W == 8 ? 112 * 1024 : 226 * 1024);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
@@ -640,12 +647,13 @@ static cudaError_t launch_v2a_cfg(const V2aConfig& cfg, const V2aArgs& a, dim3 g
     if (N <= 3 && cfg.pair)
         return cfg.warps == 12 ? launch_v2a<(N <= 3 ? N : 3), NB, 12, true>(a, grid, cfg.smem, s)
                                : launch_v2a<(N <= 3 ? N : 3), NB, 16, true>(a, grid, cfg.smem, s);
+    if (N <= 3 && NB == 1 && cfg.warps == 4) return launch_v2a<(N <= 3 ? N : 3), 1, 4, false>(a, grid, cfg.smem, s);
     if (cfg.warps == 16) return launch_v2a<N, NB, 16, false>(a, grid, cfg.smem, s);
     return launch_v2a<N, NB, 8, false>(a, grid, cfg.smem, s);
 }
 
 cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s) {
-    const V2aConfig cfg = v2a_config(l, c.batch, c.n);
+    const V2aConfig cfg = v2a_config(l, c.batch, c.n, c.epilogue);
     V2aArgs a{};
     a.off = offsets_of(l);
     a.packed = c.packed; a.x = c.x; a.y = c.y;

@@ -30,8 +30,8 @@ constexpr size_t kLibSmemU = 160 * 1024;   // normalised codebooks of this size 
 //               the order of the serial evaluation
 // A round is a chain of latencies (the two barriers, L2 round trips, the serial sums).  Where the normalised codebooks fit
 // (resident: 3072 channels of N = 2 are 96 KB) every block keeps them in shared memory, which takes the L2 round trip out of
-// each channel's assignment and the staging of the members out of the update (quantising 3072 x 4096 at N = 2 in all: 723 -> 677 us); larger ones are read from
-// L2.
+// each channel's assignment and the staging of the members out of the update (quantising 3072 x 4096 at N = 2 in all:
+// 723 -> 677 us); larger ones are read from L2.
 __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint16_t* __restrict__ cb, int rows, int E, int L,
                                                                      int iters, double* u, double* nn, int* order, int* asg,
                                                                      double* cen, int* flag, uint16_t* lib, int resident) {
