@@ -1,28 +1,24 @@
-// Prefill form of the fused decode kernel, Y = X (D + S)^T for M >= 1 rows of x ("Fused Decode Kernel", steps
-// (1)-(4): depack, codebook gather, outlier scatter-add into the dequantised tile, GEMM on the tensor cores), on
-// the fifth-generation tensor cores.  The decoded fp16 tile never touches shared memory: the lane-per-channel
+// Prefill form of the fused decode kernel, Y = X (D + S)^T for up to 64 rows of x ("Fused Decode Kernel", steps (1)-(4):
+// depack, codebook gather, GEMM on the tensor cores, outliers), on the fifth-generation tensor cores; more rows run on pairs of
+// SMs (xfp_gemm_fused.cu).  The decoded fp16 tile never touches shared memory: the lane-per-channel
 // decode of the GEMV kernels produces exactly the register image of a tensor-memory tile (lane = row, 32-bit
 // column = two consecutive k), so it is stored with tcgen05.st and used as the A operand of tcgen05.mma from
 // tensor memory; the x tile is the B operand in shared memory, brought there by one bulk tensor copy (TMA) per
 // stage; the fp32 accumulator is a second tensor-memory region.
 //
-//   CTA      128 output channels (four row-blocks) x up to 128 rows of x x one K slice; eight decode warps and a
-//            ninth that issues the tensor copies and the products; two CTAs per SM (256 of the 512 tensor-memory
-//            columns each: 128 accumulator columns, two A stages of 64).  For many rows of x (see plan_of) the tile
-//            is 256 rows: 256 accumulator columns and FOUR A stages, all 512 columns, one CTA per SM (a group of decode
-//            warps then stores its next stage while the products of its previous one still run: 28672 x 8192 with
-//            0.3 % outliers, 256 rows of x 209 -> 164 us, 512 rows 381 -> 314 us).
+//   CTA      128 output channels (four row-blocks) x the rows of x x one K slice; eight decode warps and a ninth that issues
+//            the tensor copies and the products; two CTAs per SM (256 of the 512 tensor-memory columns each: 128
+//            accumulator columns, two A stages of 64).  Where the tables leave no room for two CTAs, one CTA per SM with two
+//            groups of decode warps, FOUR A stages and all 512 columns.
 //   stage    one super-chunk (128 k): A = W^[128][128] fp16 in tensor memory, B = x[T][128] fp16 in shared memory as
 //            two K-major halves of 64 k in the 128-byte swizzle, each written by one tensor copy with the box
 //            {64 k, T rows} (128 contiguous bytes per row of x; rows beyond M arrive as zeros).
 //   decode   warp (row-block, half of the super-chunk): index vectors prefetched two super-chunks ahead, 64
 //            look-ups in one straight block into 32 registers.  V2: per-lane shared-memory tables (pair tables up
 //            to N = 3, one entry per index above).  V2a: the library replicated once per bank, then
-//            D16 = fp16(fp32(scale * lib[id][q] + mid)) with the group's scale and mid-point.  The outliers of the
-//            lane's channel that fall into its half are added to the register that holds them with one correctly
-//            rounded fp16 addition each, so the tile is the matrix xfp_dequant writes.  Up to 64 rows of x the
-//            outliers stay out of the tile (the walk through a lane's list cost 37 - 50 us of 141 at 28672 x 8192
-//            with 0.3 % outliers): the epilogue adds S x^T to the accumulator instead, see below.
+//            D16 = fp16(fp32(scale * lib[id][q] + mid)) with the group's scale and mid-point.  The outliers stay out of the
+//            tile (a walk through a lane's list cost 37 - 50 us of 141 at 28672 x 8192 with 0.3 % outliers): the epilogue
+//            adds S x^T to the accumulator instead, see below.
 //   mma      one thread waits for "A stage stored" (eight arrivals) and "x tile landed" (transaction bytes), issues
 //            eight m128 nT k16 instructions and commits them to a "products done" mbarrier; the decode of
 //            iteration i waits for the products of iteration i - 2 (i - 4 with four stages), whose A stage it
@@ -30,7 +26,7 @@
 //            barrier inside the loop.
 //   epilogue tcgen05.ld (lane = channel, registers = rows of x), direct store, or fp32 partials through the
 //            workspace when K is cut (few row tiles): the last CTA of a tile adds the slices in slice order.
-//            With the sparse outlier product, a thread first walks its channel's outliers inside the K slice and adds
+//            Before that a thread walks its channel's outliers inside the K slice and adds
 //            value * x[t][column] for its 16 rows of x in fp32, entries in ascending column order; the 16 activations
 //            are 32 contiguous bytes of a transposed copy of x that a small kernel writes before the launch.
 // Every wait on an mbarrier has an iteration limit; when one runs out the CTA stops issuing work, records it in
@@ -49,10 +45,10 @@ namespace xfp {
 namespace {
 
 constexpr int kTileRows = 128;   // output channels per CTA (the M of the instruction)
-constexpr int kSmallT = 128;     // rows of x per CTA (the N of the instruction): 128 with two CTAs per SM, or
-constexpr int kBigT = 256;       // 256 with one (more than 128 rows of x: the weights are decoded once per 256 rows)
+constexpr int kSmallT = 128;     // accumulator columns of a CTA that shares its SM,
+constexpr int kBigT = 256;       // and of one that has it to itself
 constexpr int kWarps = 8;        // decode warps of one group (row-block x half); the warp behind the last group issues
-                                 // the tensor copies and the products.  256-row tiles (one CTA per SM) run two groups:
+                                 // the tensor copies and the products.  The CTA that has its SM to itself runs two groups:
                                  // group g decodes the iterations with it % 2 == g, i.e. owns A stage g
 constexpr int threads_of(bool big) { return ((big ? 2 : 1) * kWarps + 1) * 32; }
 constexpr uint32_t kSpinLimit = 1u << 20;   // polls of a bounded wait, each of at most kPollNs: about a second
@@ -61,13 +57,10 @@ constexpr uint32_t kPollNs = 1000;
 constexpr int kAStageCols = 64;  // 128 k as fp16 pairs
 constexpr int kXStages = 3;      // x tiles in flight: the copy of iteration i + 1 is issued at the top of iteration i
 constexpr size_t kV2aTabMax = 128 * 1024;   // V2a: the per-bank library (L * 2^N * 128 bytes) must fit beside the x stages
-// Up to this many rows of x the outliers are a sparse product in the epilogue.  The product reads 32 bytes of the
-// transposed x per outlier and 16 rows, scattered through L2 at about 2.4 TB/s (28672 x 8192, 0.3 %: 13 us at 16 rows,
-// 19 at 32, 39 at 64, 78 at 128); the walk through the lists costs about as much per outlier as 64 rows of the product
-// whatever the rows (0.3 %: 45 - 50 us, 1 %: 114 us).
-constexpr int kSparseRows = 64;
-constexpr size_t kMinSmem = 80 * 1024;   // at most two CTAs per SM: each holds half of the tensor memory (a CTA with
-                                         // 256-row tiles holds all of it and asks for more than half of the shared memory)
+// The outliers are a sparse product in the epilogue.  It reads 32 bytes of the transposed x per outlier and 16 rows, scattered
+// through L2 at about 2.4 TB/s (28672 x 8192, 0.3 %: 13 us at 16 rows, 19 at 32, 39 at 64).
+constexpr size_t kMinSmem = 80 * 1024;   // at most two CTAs per SM: each holds half of the tensor memory (the CTA that
+                                         // has its SM to itself holds all of it and asks for more than half of the shared memory)
 
 struct GemmArgs {
     Blob b;
@@ -88,8 +81,8 @@ struct GemmArgs {
     int ns_log;       // log2 of the A stages: 1 (two; two CTAs per SM) or 2 (four; the CTA that has the SM to itself)
     int x_stages;     // x tiles in shared memory: kXStages, or 2 when three large ones do not fit
     int b_half;       // bytes of one 64-k half of an x tile: rows of x per tile * 128 (a multiple of 1024)
-    // outliers as a sparse product in the epilogue (few rows of x): x transposed, [K][Mp] fp16 with Mp a multiple of 32
-    // and zeros behind row M; null: the decode warps add the outliers to the tile instead
+    // the sparse product of the outliers in the epilogue: x transposed, [K][Mp] fp16 with Mp a multiple of 32
+    // and zeros behind row M; null: no outliers
     const uint16_t* xT;
     int Mp;
 };
@@ -180,39 +173,13 @@ struct Half {
     static constexpr int V0 = W0 / 4, V1 = (W1 + 3) / 4, NV = V1 - V0;
 };
 
-// A lane's outlier list (transposed slab first, the CSR arrays behind it) with the next four entries in registers:
-// an entry is consumed long after its load was issued, so a channel with several outliers close together does not
-// stall its warp (and, through the barrier, its CTA) on a chain of dependent loads.
+// A lane's outlier list: the transposed slab first, the CSR arrays behind it.
 struct Outliers {
     const uint32_t* slab;
     const uint32_t* spill;
-    const uint32_t* nextp;      // address of entry cur + 4, the next one to load
-    int step;                   // words between consecutive entries at nextp: 32 in the slab, 1 in the CSR arrays
-    int nslab, total, cur;
-    uint32_t col;               // column of entry cur, 0xffffffff behind the last one
-    uint32_t ent, e1, e2, e3;   // entries cur .. cur + 3 (column | fp16 value << 16)
-    __device__ __forceinline__ const uint32_t* addr(int j) const {
-        return j < nslab ? slab + (size_t)(1 + j) * 32 : spill + j;
-    }
-    __device__ __forceinline__ uint32_t fetch(int j) const { return __ldg(addr(j)); }
-    __device__ __forceinline__ void start(int first) {
-        cur = first;
-        if (cur < total) { ent = fetch(cur); }
-        if (cur + 1 < total) e1 = fetch(cur + 1);
-        if (cur + 2 < total) e2 = fetch(cur + 2);
-        if (cur + 3 < total) e3 = fetch(cur + 3);
-        col = cur < total ? (ent & 0xffffu) : 0xffffffffu;
-        nextp = addr(cur + 4);
-        step = cur + 4 < nslab ? 32 : 1;
-    }
-    __device__ __forceinline__ void advance() {
-        ++cur;
-        ent = e1; e1 = e2; e2 = e3;
-        col = cur < total ? (ent & 0xffffu) : 0xffffffffu;
-        if (cur + 3 < total) {
-            e3 = __ldg(nextp);
-            if (cur + 4 == nslab) { nextp = spill + nslab; step = 1; } else nextp += step;
-        }
+    int nslab, total, cur;      // entries in the slab, in all; the first one of this K slice
+    __device__ __forceinline__ uint32_t fetch(int j) const {   // column | fp16 value << 16
+        return __ldg(j < nslab ? slab + (size_t)(1 + j) * 32 : spill + j);
     }
 };
 
@@ -258,7 +225,7 @@ __device__ __forceinline__ void sparse_rows(const GemmArgs& a, const Outliers& o
 template <int N, int MODE, int PART>
 __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok, int q, int lane, int tid, int Tn,
                                           int t0, int sc0, int sc1, const unsigned char* tab, unsigned char* sB,
-                                          uint64_t* bars, uint32_t tmem, Outliers& o, const CUtensorMap* tmap,
+                                          uint64_t* bars, uint32_t tmem, const CUtensorMap* tmap,
                                           int grp, int G) {
     using H = Half<N, PART>;
     const int NS = 1 << a.ns_log;
@@ -300,7 +267,6 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         if (!ok) break;
-        const uint32_t k0 = (uint32_t)sc * kSuper;
         uint32_t d[32];
         if (rb_ok) {
             uint32_t w[4 * N + 1];
@@ -356,37 +322,6 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
                     const uint32_t hi = lds32(single_addr<N, 1>(w, 2 * p + 1, tabs));
                     d[i] = join16(lo, hi);
                 }
-            }
-            // W^ = fp16(D16 + S) at the outliers of this channel inside this half; the entries of the other half
-            // (the other warp's) are passed over.  One loop, one copy of the code that advances the list.
-            const uint32_t lo_k = k0 + PART * 64;
-            // warp-uniform loop (as many trips as the busiest lane needs, the lanes converged at the top of each)
-            while (__any_sync(0xffffffffu, o.col < k0 + kSuper)) {
-                const bool mine_now = o.col < k0 + kSuper;
-                const uint32_t kk = o.col - lo_k;              // wraps around for entries below this half
-                if (mine_now && kk < 64u) {
-                    const uint32_t v2 = (o.ent >> 16) << ((kk & 1u) * 16u);
-                    // the register that holds weight kk: found by nested tests, not a switch -- the indirect
-                    // branch of a jump table inside this divergent loop stalled the warps (176 vs 149 us on
-                    // 28672 x 8192 with 0.3 % outliers, same instruction count)
-                    const uint32_t r = kk >> 1;
-#define XFP_OUT_GROUP(g)                                                                                          \
-    if ((r >> 2) == g##u)                                                                                         \
-        asm("{\n\t.reg .pred p0, p1, p2, p3;\n\t"                                                                 \
-            "setp.eq.u32 p0, %4, 0;\n\tsetp.eq.u32 p1, %4, 1;\n\t"                                                 \
-            "setp.eq.u32 p2, %4, 2;\n\tsetp.eq.u32 p3, %4, 3;\n\t"                                                 \
-            "@p0 add.rn.f16x2 %0, %0, %5;\n\t@p1 add.rn.f16x2 %1, %1, %5;\n\t"                                     \
-            "@p2 add.rn.f16x2 %2, %2, %5;\n\t@p3 add.rn.f16x2 %3, %3, %5;\n\t}"                                    \
-            : "+r"(d[4 * g]), "+r"(d[4 * g + 1]), "+r"(d[4 * g + 2]), "+r"(d[4 * g + 3])                          \
-            : "r"(r & 3u), "r"(v2));
-                    if (r < 16u) {
-                        if (r < 8u) { XFP_OUT_GROUP(0) XFP_OUT_GROUP(1) } else { XFP_OUT_GROUP(2) XFP_OUT_GROUP(3) }
-                    } else {
-                        if (r < 24u) { XFP_OUT_GROUP(4) XFP_OUT_GROUP(5) } else { XFP_OUT_GROUP(6) XFP_OUT_GROUP(7) }
-                    }
-#undef XFP_OUT_GROUP
-                }
-                if (mine_now) o.advance();
             }
         } else {
 #pragma unroll
@@ -536,7 +471,7 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     const uint32_t tmem = s_tmem;
 
     // ---- the lane's outlier list: transposed slab first, the CSR arrays behind it ----
-    Outliers o{nullptr, nullptr, nullptr, 1, 0, 0, 0, 0xffffffffu, 0u, 0u, 0u, 0u};
+    Outliers o{nullptr, nullptr, 0, 0, 0};
     if (rb_ok && a.ell_slots) {
         o.slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
         const int olen = (int)__ldg(o.slab);
@@ -560,8 +495,7 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
             for (int j = 0; j < 15; ++j) fine += (first + j < o.total) && (o.fetch(min(first + j, o.total - 1)) & 0xffffu) < kb;
             first += fine;
         }
-        if (a.xT) { o.cur = first; o.col = 0xffffffffu; }   // the epilogue walks the list from `first`
-        else o.start(first);
+        o.cur = first;
     }
 
     const unsigned char* tab = MODE == 1 ? sTab : N == 4 ? sTab + (size_t)(q >> 1) * TW * 256 : sTab + (size_t)q * TW * 128;
@@ -571,8 +505,8 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
         __syncwarp();
     } else {
         done = part == 0
-            ? main_loop<N, MODE, 0>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, o, &tmap, grp, G)
-            : main_loop<N, MODE, 1>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, o, &tmap, grp, G);
+            ? main_loop<N, MODE, 0>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, &tmap, grp, G)
+            : main_loop<N, MODE, 1>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, &tmap, grp, G);
     }
     // what the finish needs of the schedule is worked out again from a fresh read of the CTA index, so that it does
     // not occupy registers through the main loop
@@ -739,22 +673,16 @@ Plan plan_of(const Layout& l, int M, int sms) {
     p.tab_bytes = l.mode == 1 ? (size_t)l.L * l.E * 128 : (size_t)4 * (l.bits <= 3 ? l.E * l.E : l.E) * 128;
     if (l.mode == 0) p.tab_bytes += 8192;                    // room to align the tables to 8 KB in the shared window
     p.tab_bytes = (p.tab_bytes + 1023) & ~size_t(1023);      // the x stages behind the tables are 1024-byte aligned
-    // More than 128 rows of x: tiles of 256 rows (one CTA per SM with two groups of decode warps, all 512 tensor-memory
-    // columns), which decode the weights once per 256 rows -- 28672 x 8192, M = 512: 555 -> 450 us; 4096 x 4096,
-    // M = 512: 80 -> 72 us -- when their x stages fit beside the tables.
     p.maxT = kSmallT; p.x_stages = kXStages; p.lone = false;
-    // the same CTA shape (16 decode warps, alone on its SM) also serves fewer rows of x when the tables leave no room
-    // for two CTAs of 128-row tiles on an SM (V2a from N = 4: a 64 KB library; 28672 x 8192, M = 128: 274 us with one
-    // CTA of 8 decode warps per SM)
+    // a CTA of 16 decode warps, alone on its SM, when the tables leave no room for two CTAs on an SM (V2a from N = 4: a 64 KB
+    // library)
     const int tsmall = M >= kSmallT ? kSmallT : (M + 15) & ~15;
-    const bool lone_anyway = p.tab_bytes + (size_t)2 * tsmall * 256 > 113 * 1024;
-    if (M > kSmallT || lone_anyway) {
+    const bool lone = p.tab_bytes + (size_t)2 * tsmall * 256 > 113 * 1024;
+    if (lone) {
         for (int xs = kXStages; xs >= 2; --xs) {
             const int tbig = M >= kBigT ? kBigT : (M + 15) & ~15;    // rows of x its largest tile would hold
             if (p.tab_bytes + (size_t)xs * tbig * 256 <= kSmemLimit) { p.maxT = kBigT; p.x_stages = xs; p.lone = true; break; }
         }
-        // tables too large for 256-row x stages (V2a, N = 5: 128 KB): the lone CTA with 128-row tiles
-        if (!p.lone && lone_anyway) { p.lone = true; p.x_stages = 2; }
     }
     const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;    // rows of x in the largest tile of this launch
     // 128-row tiles: two x stages instead of three where that keeps two CTAs on an SM (N = 3 pair tables and N = 6
@@ -871,9 +799,9 @@ size_t gemm_core_bytes(const Layout& l, int M) {
     return p.slots ? partial_offset(l, M) + partial_bytes(p, M) : gemm_ctrl_bytes(l, M);
 }
 
-// the transposed copy of x for the sparse outlier product: up to kSparseRows rows of x on a matrix with outliers
+// the transposed copy of x for the sparse outlier product, on a matrix with outliers
 size_t gemm_xt_bytes(const Layout& l, int M) {
-    if (l.nnz == 0 || M > kSparseRows) return 0;
+    if (l.nnz == 0) return 0;
     return align256((size_t)l.cols * ((M + 31) & ~31) * 2);
 }
 

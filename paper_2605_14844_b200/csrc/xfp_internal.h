@@ -99,7 +99,7 @@ cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s);
 bool batch_supported(const Layout& l, int batch);
 cudaError_t launch_gemv_batch(const Layout& l, const GemvCall& c, cudaStream_t s);
 
-// Prefill form on the tcgen05 tensor cores (V2, any number of rows of x); see xfp_gemm_tc.cu.
+// Prefill form on the tcgen05 tensor cores (V2 and V2a, up to 64 rows of x); see xfp_gemm_tc.cu.
 struct GemmCall {
     const void* packed;
     const uint16_t* x;   // [M][cols] fp16
@@ -128,9 +128,8 @@ inline size_t prefill_workspace_bytes(const Layout& l, int M) {
     return fused_preferred(l, M) ? fused_workspace_bytes(l, M) : gemm_workspace_bytes(l, M);
 }
 
-// Batches of 9..16 rows of x run on the tensor-core kernel (xfp_gemm_tc.cu) when the matrix is large and the blob
-// sparse in outliers: the batched GEMV kernels decode once per 8 rows of x, the tcgen05 kernel decodes once for up to
-// 128 rows (measurements at batch_prefers_gemm).
+// Batches of 9..16 rows of fp16 x run on the tensor-core kernel (xfp_gemm_tc.cu) when the matrix is large and the blob
+// sparse in outliers: the tcgen05 kernel decodes once for all rows (measurements at batch_prefers_gemm).
 // Layout of a GEMV workspace, shared by every kernel that may be given it: counters (split-K tickets, one int per
 // row-block and blob at most) in [0, align256(4 * RB * n)), zero-filled before first use and left zero-filled by every
 // call; partial sums behind it, written before they are read.
@@ -150,8 +149,8 @@ inline bool batch_prefers_gemm(const Layout& l, int batch) {
     // 28672 x 8192, us per call, tensor-core kernel against the batched kernels (0.3 % outliers unless noted):
     //   9..16 rows: V2 N = 4 74 against 124..148 (2 %: 107 against 146..174), V2a 102 against 210..246, N = 2 73
     //               against 110..133, N = 6 99 against 494..792
-    //   5..8 rows:  V2a 102 against 123, V2 N = 6 98 against 115; V2 N = 4 73 against 74 (1 %: 87 against 80) and
-    //               N = 2 72 against 67 stay on the batched lane kernel
+    //   5..8 rows:  where xfp_gemv_frag.cu (68..77) does not take the blob (V2a in groups of 64 weights): V2a 102 against 123,
+    //               V2 N = 6 98 against 115
     int least = ((l.mode || l.bits >= 5) && l.nnz * 100 <= (long long)l.rows * l.cols) ? 5 : 9;
 #ifdef LANE_TUNE
     if (const char* e = getenv("XFP_GEMM_MIN")) least = atoi(e);
