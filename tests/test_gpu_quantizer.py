@@ -144,6 +144,27 @@ def test_lloyd_degenerate_channels():
             assert np.array_equal(idx, m.idx), (bits, iters)
 
 
+@pytest.mark.parametrize("cols,bits", [(128, 6), (4096, 4), (4224, 3), (8192, 2), (8320, 5), (16384, 6)])
+def test_lloyd_channels_that_fall_out_of_the_fast_order(cols, bits):
+    """Block sizes at their limits, and channels that need the network sort (few distinct values), the serial chain (values over
+    many binades, a mean far from zero) or sort a long middle (most weights around zero), with and without extracted weights."""
+    rng = np.random.default_rng(cols + bits)
+    W = np.stack([rng.standard_normal(cols),
+                  rng.choice([-1.0, -0.25, 0.0, 0.5], cols),
+                  np.where(rng.random(cols) < 0.9, 1e-9, 1.0) * rng.standard_normal(cols),
+                  rng.standard_normal(cols) * 2.0 ** rng.integers(-40, 40, cols),
+                  1000.0 + rng.standard_normal(cols),
+                  np.sign(rng.standard_normal(cols)) * np.exp(rng.standard_normal(cols) * 3)]).astype(np.float32)
+    mask = (rng.random(W.shape) < 0.01).astype(np.uint8)
+    mask[0] = 0
+    mask[1, : cols // 2] = 1
+    mu = float(W.mean(dtype=np.float64))
+    m = xo.quantize_v2(W, bits, mask, mu, 20)
+    cb, idx = _gpu_lloyd(W, mask, mu, bits, 20)
+    assert np.array_equal(cb, m.codebook)
+    assert np.array_equal(idx, m.idx)
+
+
 # ------------------------------------------------------------------ LibFit (V2a)
 
 @pytest.mark.parametrize("bits,L,rows", [(2, 32, 96), (3, 32, 200), (4, 32, 64), (4, 7, 40), (3, 32, 20), (6, 16, 48)])
@@ -156,6 +177,22 @@ def test_libfit_library_is_bit_exact(bits, L, rows):
     xo._lib.xo_libfit_library(v2.codebook.reshape(-1), rows, bits, L, 20, want.reshape(-1))
     lib = torch.zeros((L, 1 << bits), dtype=torch.int16, device="cuda")
     qb.xfp_quant_libfit_library(_dev(v2.codebook), rows, bits, L, 20, lib, _ws(rows, cols))
+    torch.cuda.synchronize()
+    assert np.array_equal(_u16(lib), want)
+
+
+@pytest.mark.parametrize("bits,rows", [(6, 321), (2, 4099), (3, 2560), (4, 1281)])
+def test_libfit_library_in_shared_memory_and_beyond(bits, rows):
+    """Codebooks at and above the 160 KB that stay in shared memory, more channels than are compacted at a time, equal channels."""
+    rng = np.random.default_rng(rows)
+    cb = np.sort(rng.standard_normal((rows, 1 << bits)), axis=1).astype(np.float16)
+    cb[rows // 2:rows // 2 + 40] = cb[0]
+    cb = np.ascontiguousarray(cb).view(np.uint16)
+    L = 32
+    want = np.empty((L, 1 << bits), dtype=np.uint16)
+    xo._lib.xo_libfit_library(cb.reshape(-1), rows, bits, L, 20, want.reshape(-1))
+    lib = torch.zeros((L, 1 << bits), dtype=torch.int16, device="cuda")
+    qb.xfp_quant_libfit_library(_dev(cb), rows, bits, L, 20, lib, _ws(rows, 512))
     torch.cuda.synchronize()
     assert np.array_equal(_u16(lib), want)
 
