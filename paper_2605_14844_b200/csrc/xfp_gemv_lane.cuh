@@ -79,13 +79,13 @@ struct LaneCfg {
 };
 
 // The four A registers of mma step j (weights 8j .. 8j+7 of the lane's channel in this super-chunk).
-template <int N, bool SGL, bool HALF, bool QUAD>
+template <int N, bool SGL, bool HALF, bool QUAD, bool INTER>
 __device__ __forceinline__ void lookup8(uint32_t (&f)[4], const uint32_t* w, int j, const unsigned char* tab,
                                         uint32_t base) {
     if (HALF) {
         // V2a, one entry per index: a word holds the entry of TWO library ids, `base` selects the half
         uint32_t e[8];
-        if (N == 4) {
+        if (INTER) {
             // step j's eight indices are word j: byte 1 of the address = index and the low four bits of the table's place
             const uint32_t nib = ((base >> 12) & 0xfu) * 0x10101010u;
             const uint32_t lo = (w[j] & 0x0f0f0f0fu) | nib, hi = ((w[j] >> 4) & 0x0f0f0f0fu) | nib;
@@ -238,12 +238,12 @@ __device__ __forceinline__ void fill_tables_v2(unsigned char* tab, uint32_t* cbs
     }
 }
 
-// V2a, a word per entry of two library ids: the byte offset of row e = m 2^N + q, the entry q of ids 2m and 2m + 1.  At N = 4 the
-// tables of two m are interleaved and entries lie 256 bytes apart, so that one PRMT builds an address from an index (a shift
+// V2a, a word per entry of two library ids: the byte offset of row e = m 2^N + q, the entry q of ids 2m and 2m + 1.  INTER (N = 4):
+// the tables of two m are interleaved and entries lie 256 bytes apart, so that one PRMT builds an address from an index (a shift
 // and a mask per weight kept the ALU pipe busiest).
-template <int N>
+template <bool INTER>
 __device__ __forceinline__ uint32_t half_row(uint32_t e) {
-    if (N != 4) return e * 128u;
+    if (!INTER) return e * 128u;
     return (e >> 5) * 4096u + ((e >> 4) & 1u) * 128u + (e & 15u) * 256u;
 }
 
@@ -253,7 +253,7 @@ __device__ __forceinline__ uint32_t half_row(uint32_t e) {
 // handed round by a shuffle (a warp that fetched two halves per row with uniform loads paid their latency once per
 // row: 3.9 us for the 1024 rows of N = 6).  Not inlined: inside the kernel the unrolled stores changed the register
 // allocation of the K loop (N = 3, 4: 62.2 against 58.3 us at 28672 x 8192).
-template <int N, int W, bool HALF>
+template <int N, int W, bool HALF, bool INTER>
 __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __restrict__ lib, int L, int warp, int lane) {
     constexpr int E = 1 << N;
     const int trows = HALF ? ((L + 1) >> 1) * E : L * E * E;
@@ -263,7 +263,7 @@ __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __
             const int m = e >> N, q = e & (E - 1);
             const uint32_t lo = __ldg(lib + (size_t)(2 * m) * E + q);
             const uint32_t hi = 2 * m + 1 < L ? (uint32_t)__ldg(lib + (size_t)(2 * m + 1) * E + q) : 0u;
-            *(uint32_t*)(tab + half_row<N>(e) + lane * 4) = lo | (hi << 16);
+            *(uint32_t*)(tab + half_row<INTER>(e) + lane * 4) = lo | (hi << 16);
         }
         return;
     }
@@ -283,7 +283,7 @@ __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const uint32_t v = __shfl_sync(0xffffffffu, word, r);
-            if (e0 + r < trows) *(uint32_t*)(tab + (HALF ? half_row<N>(e0 + r) : (e0 + r) * 128u) + lane * 4) = v;
+            if (e0 + r < trows) *(uint32_t*)(tab + (HALF ? half_row<INTER>(e0 + r) : (e0 + r) * 128u) + lane * 4) = v;
         }
     }
 }
@@ -312,6 +312,9 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     // half, 2m + 1 in the high half): every lane still reads its own bank, whatever ids and indices the lanes hold,
     // and the tables are half as large (64 KB at N = 5, 128 KB at N = 6 with L = 32)
     constexpr bool kHalf = MODE == 1 && SGL;
+    // N = 4: interleaved tables except in the 8-warp CTAs of one row of x, which gained 2 % on their own and lost 2.4 us behind
+    // another launch (4096 x 4096 and 12288 x 4096 in turn: 23.2 us with plain tables, 25.6; the 16-warp CTAs 20.5 -> 19.5)
+    constexpr bool kInter = kHalf && N == 4 && !(W == 8 && NB == 1);
     constexpr int kIdBytes = (kLibPair ? E * E : E) * 128;   // V2a: bytes between the tables of two ids (kHalf: id pairs)
     constexpr int T = C::T;
     constexpr int kStride = C::kStride;
@@ -340,7 +343,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     const int src_a = (lane & ~3) | (t4 >> 1);
     // V2a: table offset of library id `id`
     auto id_offset = [](uint32_t id) -> uint32_t {
-        return kHalf ? half_row<N>((id >> 1) * (uint32_t)E) + (id & 1u) * 2u : id * (uint32_t)kIdBytes;
+        return kHalf ? half_row<kInter>((id >> 1) * (uint32_t)E) + (id & 1u) * 2u : id * (uint32_t)kIdBytes;
     };
 
 #pragma unroll 1
@@ -425,7 +428,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     if (MODE != 0) {
         if (!kMulti || it == 0) {   // one library per blob: a resident CTA fills it once
         if constexpr (N >= 5 || kLibPair || W == 8) {
-            fill_library<N, W, kHalf>(tab, b.cb, a.L, warp, lane);
+            fill_library<N, W, kHalf, kInter>(tab, b.cb, a.L, warp, lane);
         } else {
             // small tables in a CTA that has its SM to itself: inline, so that the index loads issued above stay in
             // flight (registers that are the target of a load are written back around a call, which waits for them:
@@ -442,13 +445,13 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
                 }
 #pragma unroll
                 for (int i = 0; i < kRows; ++i)
-                    *(uint32_t*)(tab + half_row<N>(warp + i * W) + lane * 4) = lo[i] | (hi[i] << 16);
+                    *(uint32_t*)(tab + half_row<kInter>(warp + i * W) + lane * 4) = lo[i] | (hi[i] << 16);
             } else {
                 for (int e = warp; e < ((a.L + 1) >> 1) * E; e += W) {
                     const int m = e >> N, q = e & (E - 1);
                     const uint32_t lo = __ldg(b.cb + (size_t)(2 * m) * E + q);
                     const uint32_t hi = 2 * m + 1 < a.L ? (uint32_t)__ldg(b.cb + (size_t)(2 * m + 1) * E + q) : 0u;
-                    *(uint32_t*)(tab + half_row<N>(e) + lane * 4) = lo | (hi << 16);
+                    *(uint32_t*)(tab + half_row<kInter>(e) + lane * 4) = lo | (hi << 16);
                 }
             }
         }
@@ -568,14 +571,14 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
                 c[r][0] = c[r][1] = c[r][2] = c[r][3] = 0.f;
             }
         };
-        lookup8<N, SGL, kHalf, C::kQuad>(fa, w, 0, tab, vbase);
+        lookup8<N, SGL, kHalf, C::kQuad, kInter>(fa, w, 0, tab, vbase);
 #pragma unroll
         for (int j = 0; j < kSuper / 8; j += 2) {
             if (NB <= RH) {
 #pragma unroll
                 for (int r = 0; r < NB; ++r) ld_x16_if(xr[r], xp + r * xrow + j * 16, dq);   // steps j and j + 1
             }
-            lookup8<N, SGL, kHalf, C::kQuad>(fb, w, j + 1, tab, vbase);
+            lookup8<N, SGL, kHalf, C::kQuad, kInter>(fb, w, j + 1, tab, vbase);
 #pragma unroll
             for (int v = 0; v < N; ++v)
                 if ((last_step_of_vector<N>(v) == j || last_step_of_vector<N>(v) == j + 1) && has_next) {
@@ -586,7 +589,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
 #pragma unroll
                 for (int r = 0; r < NB; ++r) mma16816(c[r], fa[0], fa[1], fa[2], fa[3], xr[r].x, xr[r].y);
                 if (MODE != 0 && j + 2 == kSuper / 16) vbase = base + id_offset(gid_c[1]);   // second half's library entry
-                if (j + 2 < kSuper / 8) lookup8<N, SGL, kHalf, C::kQuad>(fa, w, j + 2, tab, vbase);
+                if (j + 2 < kSuper / 8) lookup8<N, SGL, kHalf, C::kQuad, kInter>(fa, w, j + 2, tab, vbase);
 #pragma unroll
                 for (int r = 0; r < NB; ++r) mma16816(c[r], fb[0], fb[1], fb[2], fb[3], xr[r].z, xr[r].w);
             } else {
@@ -598,7 +601,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
                     for (int r = 0; r < RH; ++r) ld_x16_if(xr[r], xp + (h * RH + r) * xrow + j * 16, dq);
                     if (h == NB / RH - 1) {
                         if (MODE != 0 && j + 2 == kSuper / 16) vbase = base + id_offset(gid_c[1]);
-                        if (j + 2 < kSuper / 8) lookup8<N, SGL, kHalf, C::kQuad>(fn, w, j + 2, tab, vbase);
+                        if (j + 2 < kSuper / 8) lookup8<N, SGL, kHalf, C::kQuad, kInter>(fn, w, j + 2, tab, vbase);
                     }
 #pragma unroll
                     for (int r = 0; r < RH; ++r) mma16816(c[h * RH + r], fa[0], fa[1], fa[2], fa[3], xr[r].x, xr[r].y);
