@@ -41,6 +41,11 @@ constexpr int kCh = 128;                       // channels of a CTA
 constexpr int kStageK = 64;
 constexpr int kABytes = kCh * kStageK * 2;     // A of one stage
 constexpr int kMaxSlots = 12;
+// A decode warp takes every fourth stage.  At stage j it waits, by parity, for the products of stage j - slots; that is only
+// unambiguous once stage j - 2 slots is known to be done, and what the warp knows from its own stage j - 4 is that stage
+// j - 4 - slots is.  With three stages in the ring a warp ahead of the others could pass early and arrive in another stage's
+// phase (which faulted: V2a, N = 2, 7959 x 1920, 1991 rows, no outliers).
+constexpr int kMinSlots = 4;
 // Warp roles, the short ones first: the scheduler serves older warps first, and behind the decode warps, which can issue in
 // every clock, the others' few instructions waited.
 constexpr int kMmaWarp = 0, kCopyWarp = 1, kCopyWarps = 2, kOutWarp = 4, kOutWarps = 4, kDecodeWarp = 8, kDecodeWarps = 16;
@@ -789,7 +794,7 @@ FusedPlan plan_fused(const Layout& l, int M) {
         const int tok = (M + T - 1) / T;
         int slots = (int)((kSmemMax - 8192 - tab - lib) / (kABytes + (size_t)parts * Tp * 64));
         if (slots > kMaxSlots) slots = kMaxSlots;
-        if (slots < 2) continue;
+        if (slots < kMinSlots) continue;
         // a stage's way through decode, outliers and products takes about 2900 clocks and its share of the products
         const double chain = (2900.0 + 2.0 * T) / slots * 2.0, busy = slot_clocks(l, T), step = busy > chain ? busy : chain;
         // a CTA's sums to or from the workspace at 40 bytes a clock, and all of them through DRAM at 2 KB a clock (10007 x 4992,

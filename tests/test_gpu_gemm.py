@@ -181,6 +181,16 @@ def test_gemm_on_pairs_of_sms(mode, bits, rows, cols, m, placement):
     assert torch.equal(y, y2) and int(ws[:4].view(torch.int32).item()) == 0
 
 
+@pytest.mark.parametrize("mode,bits,rows,cols,m", [(1, 2, 2048, 1920, 512), (0, 3, 700, 1024, 512), (0, 6, 513, 640, 300),
+                                                   (1, 5, 520, 896, 257), (1, 2, 20000, 384, 500)])
+def test_gemm_on_pairs_without_outliers_and_with_large_tables(mode, bits, rows, cols, m):
+    """The ring of stages at its shortest (tables and x of 512 rows beside it), the decode warps signalling the products directly.
+    Tolerances as for every other shape (see _check)."""
+    q = synth.random_quantized(mode, rows, cols, bits, 0.0, seed=1500 + rows + m)
+    pm = xfp.pack_tensors(q, col_bits=16)
+    _check(q, pm, synth.activations(m, cols, seed=1510 + m))
+
+
 def test_gemm_matches_gemv_rows_and_is_deterministic():
     q = synth.random_quantized(0, 512, 4096, 4, 0.01, seed=41)
     pm = xfp.pack_tensors(q)
