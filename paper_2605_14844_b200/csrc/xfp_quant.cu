@@ -871,7 +871,12 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
     xfp_quant_workspace_size(rows, cols, &need);
     // mu, sigma, the median, the count and the extraction's plan live behind the carved scratch
     if (workspace_bytes < need + 256) return XFP_ERR_BUFFER_TOO_SMALL;
-    if (!aligned16(W) || !aligned16(mask) || !aligned16(workspace) || !aligned16(codebook) || !aligned16(idx)) return XFP_ERR_ALIGN;
+    // everything the stages below would refuse one by one: the kernels are launched past their entry points
+    if (!aligned16(W) || !aligned16(mask) || !aligned16(workspace) || !aligned16(codebook) || !aligned16(idx) ||
+        !aligned16(out_rowptr) || !aligned16(cos))
+        return XFP_ERR_ALIGN;
+    if (mode == 1 && (!aligned16(lib) || !aligned16(gid) || !aligned16(gscale) || !aligned16(gmid))) return XFP_ERR_ALIGN;
+    if ((reinterpret_cast<uintptr_t>(out_col) & 3u) || (reinterpret_cast<uintptr_t>(out_val) & 1u)) return XFP_ERR_ALIGN;
     if (p->lloyd_iters < 0 || (p->outlier_mode != 0 && p->outlier_mode != 1) || (p->outlier_mode == 0 ? !(p->k_sigma >= 0.0) || !(p->cap_frac >= 0.0 && p->cap_frac <= 1.0)
                                                                               : !(p->rate >= 0.0 && p->rate <= 1.0)))
         return XFP_ERR_SHAPE;
@@ -901,6 +906,7 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
     d.lib_size = mode ? lib_size : 0;
     if (d.group_size != 64 && d.group_size != 128 && d.group_size != 256) return d.group_size > 0 ? XFP_ERR_UNSUPPORTED : XFP_ERR_SHAPE;
     if (cols % d.group_size) return XFP_ERR_SHAPE;
+    if (mode == 1 && (int64_t)rows * (cols / d.group_size) > 0x7fffffff) return XFP_ERR_UNSUPPORTED;
     d.col_bits = 32; d.nnz = host_cnt;
     result->mu = host.mu; result->sigma = host.sigma; result->nnz = host_cnt;
     result->fallback = 1; result->tried = 0; result->reserved = 0;

@@ -88,6 +88,26 @@ def test_encoder_rejects_bad_arguments_on_the_host(lib):
                             C.byref(r), a, 128, n) == 5
 
 
+@pytest.mark.parametrize("mode,name", [(0, n) for n in ("W", "mask", "idx", "codebook", "rowptr", "cos", "workspace")]
+                         + [(1, n) for n in ("lib", "gid", "gscale", "gmid", "rowptr", "cos", "idx")])
+def test_quantize_rejects_misaligned_buffers_on_the_host(lib, mode, name):
+    """xfp_quantize launches its stages' kernels itself: what their entry points refuse has to be refused before the first
+    launch (a scale array at an odd address or a row-pointer array off by two would be misaligned stores on the device)."""
+    from paper_2605_14844_b200 import quant_binding as qb
+    qb._lib()
+    v = {n: 0x1000 for n in ("W", "mask", "idx", "codebook", "lib", "gid", "gscale", "gmid", "rowptr", "ocol", "oval", "cos",
+                             "workspace")}
+    for off in (1, 2, 8):
+        v[name] = 0x1000 + off
+        a = {n: C.c_void_p(x) for n, x in v.items()}
+        p = qb.XfpQuantParams(0, 0, 4.0, 0.02, 0.0, 20, 0)
+        r = qb.XfpQuantResult()
+        cand = (C.c_int32 * 1)(4)
+        assert lib.xfp_quantize(mode, a["W"], 64, 256, C.byref(p), cand, 1, 0.96, 32 if mode else 0, a["mask"], a["idx"],
+                                a["codebook"], a["lib"], a["gid"], a["gscale"], a["gmid"], a["rowptr"], a["ocol"], a["oval"],
+                                100, a["cos"], C.byref(r), a["workspace"], 1 << 30, None) == 2
+
+
 def _desc(**kw):
     d = dict(mode=0, rows=64, cols=256, bits=4, group_size=128, lib_size=0, col_bits=32, nnz=0)
     d.update(kw)
