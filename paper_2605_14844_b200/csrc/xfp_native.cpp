@@ -42,11 +42,24 @@ struct Args {
         }
         return &THPVariable_Unpack(a[i]);
     }
-    void* ptr(int i) { const at::Tensor* t = tensor(i); return t ? t->data_ptr() : nullptr; }
+    // what f throws (a sparse or a fake tensor has no data pointer, a symbolic size no value) as a Python exception: through a C
+    // function it would end the process
+    template <class F>
+    auto guarded(F&& f) -> decltype(f()) {
+        try { return f(); }
+        catch (const c10::Error& e) { PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace()); }
+        catch (const std::exception& e) { PyErr_SetString(PyExc_RuntimeError, e.what()); }
+        bad = true;
+        return {};
+    }
+    void* ptr(int i) {
+        const at::Tensor* t = tensor(i);
+        return t ? guarded([&] { return t->data_ptr(); }) : nullptr;
+    }
     void* buffer(int i, size_t* bytes) {
         const at::Tensor* t = tensor(i);
-        *bytes = t ? t->nbytes() : 0;
-        return t ? t->data_ptr() : nullptr;
+        *bytes = t ? guarded([&] { return t->nbytes(); }) : 0;
+        return ptr(i);
     }
     int32_t integer(int i) {
         if (bad) return 0;
@@ -74,10 +87,7 @@ struct Args {
     // None: the current stream of the current device; else a torch stream or the address of one
     void* stream(int i) {
         if (bad) return nullptr;
-        if (a[i] == Py_None) {
-            try { return c10::cuda::getCurrentCUDAStream().stream(); }
-            catch (const std::exception& e) { PyErr_SetString(PyExc_RuntimeError, e.what()); bad = true; return nullptr; }
-        }
+        if (a[i] == Py_None) return guarded([] { return (void*)c10::cuda::getCurrentCUDAStream().stream(); });
         PyObject* v = PyObject_GetAttrString(a[i], "cuda_stream");
         if (!v) { PyErr_Clear(); v = Py_NewRef(a[i]); }
         PyObject* n = PyNumber_Long(v);
@@ -125,8 +135,8 @@ PyObject* gemv(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void* ws = a.buffer(7, &bytes);
     void* s = a.stream(8);
     if (mode < 0) mode = d.mode;
-    if (batch == -1 && x) batch = x->dim() == 2 ? (int32_t)x->size(0) : 1;
-    const uint16_t* xp = x && !a.bad ? (const uint16_t*)x->data_ptr() : nullptr;
+    if (batch == -1 && x) batch = a.guarded([&] { return x->dim() == 2 ? (int32_t)x->size(0) : 1; });
+    const uint16_t* xp = (const uint16_t*)a.ptr(3);
     return call(a, [&] { return (mode ? g.gemv_v2a : g.gemv_v2)(&d, packed, xp, batch, y, half, ws, bytes, s); });
 }
 
@@ -174,8 +184,8 @@ PyObject* gemm(PyObject*, PyObject* const* args, Py_ssize_t n) {
     size_t bytes;
     void* ws = a.buffer(4, &bytes);
     void* s = a.stream(5);
-    const int32_t m = x && x->dim() ? (int32_t)x->size(0) : 0;
-    const void* xp = x && !a.bad ? x->data_ptr() : nullptr;
+    const int32_t m = x ? a.guarded([&] { return x->dim() ? (int32_t)x->size(0) : 0; }) : 0;
+    const void* xp = a.ptr(2);
     return call(a, [&] { return g.gemm_typed(&d, packed, xp, xt, m, y, yt, ws, bytes, s); });
 }
 

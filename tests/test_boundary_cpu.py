@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 import paper_2605_14844_b200 as xfp
 from paper_2605_14844_b200 import binding, build as xbuild
@@ -207,6 +208,39 @@ def test_null_alignment_and_size_checks_need_no_gpu(lib):
     assert lib.xfp_gemm_typed(C.byref(d), a, a, 2, 64, a, 0, a, 64, n) == 5
     assert lib.xfp_gemm_typed(C.byref(d), a, n, 2, 64, a, 0, a, 1 << 30, n) == 1
     assert xfp.xfp_status_str(0) == "ok" and "aligned" in xfp.xfp_status_str(2)
+
+
+def _without_storage(kind):
+    if kind == "sparse":
+        return torch.zeros(2, 256, dtype=torch.float16).to_sparse()
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        return torch.zeros(2, 256, dtype=torch.float16)
+
+
+@pytest.mark.parametrize("kind", ["sparse", "fake"])
+@pytest.mark.parametrize("arg", ["packed", "x", "y", "workspace"])
+def test_tensor_without_storage_is_an_exception(lib, kind, arg):
+    """Such a tensor has no data pointer and says so by a C++ exception, which must not pass through the binding's C functions."""
+    v = {n: torch.zeros(2, 256, dtype=torch.float16) for n in ("packed", "x", "y", "workspace")}
+    v[arg] = _without_storage(kind)
+    d, w, ptrs = _desc(), torch.zeros(4), torch.zeros(2, dtype=torch.int64)
+    pm = xfp.PackedMatrix(d, v["packed"], v["workspace"], None)
+    calls = [lambda: xfp.xfp_gemv_v2(d, v["packed"], v["x"], 2, v["y"], True, v["workspace"], 1),
+             lambda: xfp.xfp_gemv_typed(d, v["packed"], v["x"], 2, v["y"], v["workspace"], 1),
+             lambda: xfp.xfp_gemm_typed(d, v["packed"], v["x"], v["y"], v["workspace"], 1),
+             lambda: xfp.xfp_gemv_host(d, v["packed"], v["x"], v["x"], 2, v["y"], v["y"], True, v["workspace"], 1),
+             lambda: pm.gemv(v["x"], v["y"], True, 1)]
+    if arg != "workspace":
+        calls.append(lambda: xfp.xfp_gemv_v2_noalloc(d, v["packed"], v["x"], 2, v["y"], True, 1))
+    if arg in ("packed", "y"):
+        calls.append(lambda: xfp.xfp_dequant(d, v["packed"], v["y"], 1))
+        calls.append(lambda: xfp.xfp_gemv_grouped(d, 2, v[arg], ptrs, ptrs, True, w, 1))
+        calls.append(lambda: xfp.xfp_pack(d, v[arg], w, None, None, None, None, None, None, w, None, 1))
+    for call in calls:
+        with pytest.raises(RuntimeError) as e:
+            call()
+        assert not isinstance(e.value, xfp.XfpError)          # raised by the tensor, not by a status of the library
 
 
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
