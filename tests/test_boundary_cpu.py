@@ -210,20 +210,25 @@ def test_null_alignment_and_size_checks_need_no_gpu(lib):
     assert xfp.xfp_status_str(0) == "ok" and "aligned" in xfp.xfp_status_str(2)
 
 
-def _without_storage(kind):
-    if kind == "sparse":
-        return torch.zeros(2, 256, dtype=torch.float16).to_sparse()
-    from torch._subclasses.fake_tensor import FakeTensorMode
-    with FakeTensorMode():
-        return torch.zeros(2, 256, dtype=torch.float16)
-
-
-@pytest.mark.parametrize("kind", ["sparse", "fake"])
+@pytest.mark.parametrize("kind", ["sparse", "batched"])
 @pytest.mark.parametrize("arg", ["packed", "x", "y", "workspace"])
 def test_tensor_without_storage_is_an_exception(lib, kind, arg):
     """Such a tensor has no data pointer and says so by a C++ exception, which must not pass through the binding's C functions."""
     v = {n: torch.zeros(2, 256, dtype=torch.float16) for n in ("packed", "x", "y", "workspace")}
-    v[arg] = _without_storage(kind)
+    if kind == "batched":                     # as inside a torch.vmap of the caller's function
+
+        def inner(t):
+            v[arg] = t
+            _expect_exceptions(v, arg)
+            return t
+
+        torch.vmap(inner)(torch.zeros(3, 2, 256, dtype=torch.float16))
+    else:
+        v[arg] = v[arg].to_sparse()
+        _expect_exceptions(v, arg)
+
+
+def _expect_exceptions(v, arg):
     d, w, ptrs = _desc(), torch.zeros(4), torch.zeros(2, dtype=torch.int64)
     pm = xfp.PackedMatrix(d, v["packed"], v["workspace"], None)
     calls = [lambda: xfp.xfp_gemv_v2(d, v["packed"], v["x"], 2, v["y"], True, v["workspace"], 1),
