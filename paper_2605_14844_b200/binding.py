@@ -268,7 +268,7 @@ class PackedMatrix:
         if y is None:
             y = torch.empty((x.shape[0] if x.dim() == 2 else 1, self.desc.rows),
                             dtype=torch.float16 if y_fp16 else torch.float32, device=x.device)
-        status = (_NATIVE or _native()).gemv(-1, self.desc, self.packed, x, -1, y, y_fp16, self.workspace, stream)
+        status = (_NATIVE or _native()).gemv(-1, self.desc, self.packed, x, None, y, y_fp16, self.workspace, stream)
         if status:
             _check(status, "xfp_gemv_v2a" if self.desc.mode else "xfp_gemv_v2")
         return y

@@ -121,21 +121,22 @@ PyObject* call(const Args& x, F&& f) {
     return PyLong_FromLong(st);
 }
 
-// (mode, desc, packed, x, batch, y, y_is_fp16, workspace, stream); mode -1: the descriptor's; batch -1: the rows of x
+// (mode, desc, packed, x, batch, y, y_is_fp16, workspace, stream); mode -1: the descriptor's; batch None: the rows of x (every
+// integer goes to the library as it is, which refuses those that are no batch)
 PyObject* gemv(PyObject*, PyObject* const* args, Py_ssize_t n) {
     Args a(args, n, 9);
     int32_t mode = a.integer(0);
     const xfp_desc d = a.desc(1);
     const void* packed = a.ptr(2);
     const at::Tensor* x = a.tensor(3);
-    int32_t batch = a.integer(4);
+    const bool rows = !a.bad && args[4] == Py_None;
+    const int32_t batch = !rows ? a.integer(4) : x ? a.guarded([&] { return x->dim() == 2 ? (int32_t)x->size(0) : 1; }) : 0;
     void* y = a.ptr(5);
     const int32_t half = a.truth(6);
     size_t bytes;
     void* ws = a.buffer(7, &bytes);
     void* s = a.stream(8);
     if (mode < 0) mode = d.mode;
-    if (batch == -1 && x) batch = a.guarded([&] { return x->dim() == 2 ? (int32_t)x->size(0) : 1; });
     const uint16_t* xp = (const uint16_t*)a.ptr(3);
     return call(a, [&] { return (mode ? g.gemv_v2a : g.gemv_v2)(&d, packed, xp, batch, y, half, ws, bytes, s); });
 }

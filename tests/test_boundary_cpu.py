@@ -210,6 +210,18 @@ def test_null_alignment_and_size_checks_need_no_gpu(lib):
     assert xfp.xfp_status_str(0) == "ok" and "aligned" in xfp.xfp_status_str(2)
 
 
+@pytest.mark.parametrize("batch", [-1, 0, 17, -2 ** 31])
+def test_binding_hands_the_batch_on_as_it_is(lib, batch):
+    """A batch outside 1..16 is a shape error, -1 like any other: the rows that x happens to have do not take its place."""
+    t = torch.zeros(4096, 64, dtype=torch.float32)
+    for mode, fn in ((0, xfp.xfp_gemv_v2), (1, xfp.xfp_gemv_v2a)):
+        d = _desc(mode=mode, lib_size=32 if mode else 0)
+        with pytest.raises(xfp.XfpError, match="status 3"):
+            fn(d, t, t[:2, :], batch, t, False, t, 1)
+        with pytest.raises(xfp.XfpError, match="status 3"):
+            xfp.xfp_gemv_typed(d, t, t.half(), batch, t, t, 1)
+
+
 @pytest.mark.parametrize("kind", ["sparse", "batched"])
 @pytest.mark.parametrize("arg", ["packed", "x", "y", "workspace"])
 def test_tensor_without_storage_is_an_exception(lib, kind, arg):
