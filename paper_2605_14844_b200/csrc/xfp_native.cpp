@@ -52,18 +52,38 @@ struct Args {
         bad = true;
         return {};
     }
+    // the integer that method `name` of argument i returns: objects that are no tensors but have a tensor's methods (a storage, a
+    // caller's own handle) are taken as the tensors are
+    size_t method(int i, const char* name) {
+        if (bad) return 0;
+        PyObject* r = PyObject_CallMethod(a[i], name, nullptr);
+        const size_t v = r ? PyLong_AsSize_t(r) : 0;
+        Py_XDECREF(r);
+        if (PyErr_Occurred()) bad = true;
+        return v;
+    }
+    bool duck(int i) const { return !bad && a[i] != Py_None && !THPVariable_Check(a[i]); }
     void* ptr(int i) {
+        if (duck(i)) return (void*)method(i, "data_ptr");
         const at::Tensor* t = tensor(i);
         return t ? guarded([&] { return t->data_ptr(); }) : nullptr;
     }
     void* buffer(int i, size_t* bytes) {
-        const at::Tensor* t = tensor(i);
-        *bytes = t ? guarded([&] { return t->nbytes(); }) : 0;
+        if (duck(i)) {
+            *bytes = method(i, "numel");
+            *bytes *= method(i, "element_size");
+        } else {
+            const at::Tensor* t = tensor(i);
+            *bytes = t ? guarded([&] { return t->nbytes(); }) : 0;
+        }
         return ptr(i);
     }
+    // as int() takes it: whole numbers of any kind, floats cut
     int32_t integer(int i) {
         if (bad) return 0;
-        const long v = PyLong_AsLong(a[i]);
+        long v = -1;
+        if (PyLong_Check(a[i])) v = PyLong_AsLong(a[i]);
+        else if (PyObject* n = PyNumber_Long(a[i])) { v = PyLong_AsLong(n); Py_DECREF(n); }
         if (v == -1 && PyErr_Occurred()) bad = true;
         return (int32_t)v;
     }
@@ -128,8 +148,8 @@ PyObject* gemv(PyObject*, PyObject* const* args, Py_ssize_t n) {
     int32_t mode = a.integer(0);
     const xfp_desc d = a.desc(1);
     const void* packed = a.ptr(2);
-    const at::Tensor* x = a.tensor(3);
     const bool rows = !a.bad && args[4] == Py_None;
+    const at::Tensor* x = rows ? a.tensor(3) : nullptr;
     const int32_t batch = !rows ? a.integer(4) : x ? a.guarded([&] { return x->dim() == 2 ? (int32_t)x->size(0) : 1; }) : 0;
     void* y = a.ptr(5);
     const int32_t half = a.truth(6);

@@ -222,6 +222,32 @@ def test_binding_hands_the_batch_on_as_it_is(lib, batch):
             xfp.xfp_gemv_typed(d, t, t.half(), batch, t, t, 1)
 
 
+def test_binding_takes_what_has_a_tensors_methods(lib):
+    """Arguments are read through data_ptr(), numel() and element_size(), a batch as int() reads it: a storage, a caller's own
+    handle, 1.0 or a 0-dim tensor reach the library (here its refusal of a workspace that is too small)."""
+    class Handle:
+        def __init__(self, t):
+            self.t = t
+
+        def data_ptr(self):
+            return self.t.data_ptr()
+
+        def numel(self):
+            return 4
+
+        def element_size(self):
+            return 2
+
+    d, t = _desc(), torch.zeros(4096, dtype=torch.float16)
+    assert t.data_ptr() % 16 == 0
+    for obj in (Handle(t), t.untyped_storage()):
+        for batch in (1, 1.0, torch.tensor(1)):
+            with pytest.raises(xfp.XfpError, match="status 5"):
+                xfp.xfp_gemv_v2(d, obj, obj, batch, obj, True, Handle(t), 1)
+    with pytest.raises(AttributeError):
+        xfp.xfp_gemv_v2(d, object(), t, 1, t, True, t, 1)
+
+
 @pytest.mark.parametrize("kind", ["sparse", "batched"])
 @pytest.mark.parametrize("arg", ["packed", "x", "y", "workspace"])
 def test_tensor_without_storage_is_an_exception(lib, kind, arg):
