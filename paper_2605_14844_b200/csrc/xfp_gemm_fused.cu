@@ -61,7 +61,7 @@ constexpr int kPairs = kSizingSMs / 2;         // pairs that the schedule deals 
 struct FusedArgs {
     Blob b;
     void* y;
-    int* ctrl;                  // [0] error word, [1 + 2 * tile + half] arrivals of the parts of a cut tile
+    int* ctrl;                  // [0] error word, [1 + 2 * tile + half] arrivals of the parts of a dealt tile (see prefill_ctrl_bytes)
     float* part;                // [2 * pair + which][half][T][128] sums of a part
     int rows, RB, SC, M, ell_slots, GH, L, y_kind;
     int pairs, tok_tiles;       // tiles: 256 channels, T rows of x
@@ -829,9 +829,6 @@ FusedPlan plan_fused(const Layout& l, int M) {
     return best;
 }
 
-// counters behind the error word: two per tile, and at least one for every 128 channels and 256 rows of x
-size_t fused_ctrl_bytes(const Layout& l, int M) { return align256(4 * (size_t)(1 + 2 * ((l.RB + 7) / 8) * ((M + 63) / 64))); }
-
 template <int N, int MODE>
 cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     const FusedPlan p = plan_fused(l, c.M);
@@ -858,7 +855,7 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     }
     FusedArgs a = {};
     a.b = blob_at(c.packed, offsets_of(l));
-    a.y = c.y; a.ctrl = (int*)c.workspace; a.part = (float*)((char*)c.workspace + fused_ctrl_bytes(l, c.M));
+    a.y = c.y; a.ctrl = (int*)c.workspace; a.part = (float*)((char*)c.workspace + prefill_ctrl_bytes(l));
     a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L; a.y_kind = c.y_kind;
     a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
     a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
@@ -883,6 +880,7 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
 }  // namespace
 
 bool fused_preferred(const Layout& l, int M) {
+    static_assert(2 * kPairs <= kSizingSMs, "two counters for each of fewer than kPairs dealt tiles (prefill_ctrl_bytes)");
 #ifdef LANE_TUNE
     if (const char* e = getenv("XFP_FUSED")) return M >= atoi(e) && gemm_tc_supported(l, M);
 #endif
@@ -891,7 +889,7 @@ bool fused_preferred(const Layout& l, int M) {
 size_t fused_workspace_bytes(const Layout& l, int M) {
     const FusedPlan p = plan_fused(l, M);
     const bool cut = p.dealt && p.dealt * l.SC != p.stream;
-    return fused_ctrl_bytes(l, M) + (cut ? (size_t)p.dealt * 4 * p.T * kCh * 4 : 0);
+    return prefill_ctrl_bytes(l) + (cut ? (size_t)p.dealt * 4 * p.T * kCh * 4 : 0);
 }
 
 // c.x: the activations as fp16; or bf16, converted first into x_f16

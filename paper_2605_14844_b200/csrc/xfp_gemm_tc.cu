@@ -699,7 +699,6 @@ Plan plan_of(const Layout& l, int M, int sms) {
     return p;
 }
 
-size_t partial_offset(const Layout& l, int M);
 size_t partial_bytes(const Plan& p, int M);
 
 template <int N, int MODE>
@@ -739,7 +738,7 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     a.b = blob_at(c.packed, offsets_of(l));
     a.y = c.y;
     a.ctrl = (int*)c.workspace;
-    a.partial = (float*)((char*)c.workspace + partial_offset(l, c.M));
+    a.partial = (float*)((char*)c.workspace + prefill_ctrl_bytes(l));
     a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots;
     a.GH = l.GH;
     a.y_kind = c.y_kind; a.b_half = b_half;
@@ -776,28 +775,14 @@ bool gemm_tc_supported(const Layout& l, int M) {
     return l.mode == 0 || (size_t)l.L * l.E * 128 <= kV2aTabMax;
 }
 
-size_t gemm_ctrl_bytes(const Layout& l, int M) {
-    const Plan p = plan_of(l, M, kSizingSMs);
-    return align256((size_t)(1 + p.row_tiles * p.tok_tiles) * 4);
-}
-
 namespace {
-// Partial sums start behind the counters, and behind the counter region that the GEMV kernels want left zero-filled (a
-// batch sent here by xfp_gemv brings the GEMV's workspace).
-size_t partial_offset(const Layout& l, int M) {
-    const size_t ctrl = gemm_ctrl_bytes(l, M), tickets = align256((size_t)l.RB * 4);
-    return ctrl > tickets ? ctrl : tickets;
-}
 size_t partial_bytes(const Plan& p, int M) {
     const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;      // rows of x in the largest tile: the rows of a slot
     return (size_t)p.slots * tmax * kTileRows * 4;
 }
 }  // namespace
 
-size_t gemm_core_bytes(const Layout& l, int M) {
-    const Plan p = plan_of(l, M, kSizingSMs);
-    return p.slots ? partial_offset(l, M) + partial_bytes(p, M) : gemm_ctrl_bytes(l, M);
-}
+size_t gemm_core_bytes(const Layout& l, int M) { return prefill_ctrl_bytes(l) + partial_bytes(plan_of(l, M, kSizingSMs), M); }
 
 // the transposed copy of x for the sparse outlier product, on a matrix with outliers
 size_t gemm_xt_bytes(const Layout& l, int M) {
@@ -805,11 +790,8 @@ size_t gemm_xt_bytes(const Layout& l, int M) {
     return align256((size_t)l.cols * ((M + 31) & ~31) * 2);
 }
 
-// where the transposed copy starts: behind the counters and partial sums, and behind the GEMV kernels' counter region
-size_t gemm_xt_offset(const Layout& l, int M) {
-    const size_t core = align256(gemm_core_bytes(l, M)), tickets = align256((size_t)l.RB * 4);
-    return core > tickets ? core : tickets;
-}
+// where the transposed copy starts: behind the counters and partial sums
+size_t gemm_xt_offset(const Layout& l, int M) { return align256(gemm_core_bytes(l, M)); }
 
 size_t gemm_workspace_bytes(const Layout& l, int M) {
     const size_t xt = gemm_xt_bytes(l, M);

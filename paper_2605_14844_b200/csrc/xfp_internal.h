@@ -110,7 +110,15 @@ struct GemmCall {
     size_t workspace_bytes;
 };
 bool gemm_tc_supported(const Layout& l, int M);
-size_t gemm_ctrl_bytes(const Layout& l, int M);
+// The counters of both prefill kernels: one region at the start of the workspace whose size does not depend on the rows of x, so
+// that calls of different rows may share a workspace (what one call keeps as a sum must not lie where another counts).  An error
+// word, then the larger of two words per dealt tile of the pair kernel (fewer tiles than pairs of SMs) and one per tile of 128
+// channels of the 64-row kernel; and the counters of the GEMV kernels, whose workspace a batch brings along.
+inline size_t prefill_ctrl_bytes(const Layout& l) {
+    const int tiles = (l.RB + 3) / 4;
+    const size_t own = align256(4 * (size_t)(1 + (tiles > kSizingSMs ? tiles : kSizingSMs))), tickets = align256((size_t)l.RB * 4);
+    return own > tickets ? own : tickets;
+}
 size_t gemm_core_bytes(const Layout& l, int M);        // counters and the partial sums of K slices
 size_t gemm_xt_bytes(const Layout& l, int M);          // the transposed copy of x of the sparse outlier product (0: not used)
 size_t gemm_xt_offset(const Layout& l, int M);         // where that copy starts in the workspace

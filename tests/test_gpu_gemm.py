@@ -191,6 +191,32 @@ def test_gemm_on_pairs_without_outliers_and_with_large_tables(mode, bits, rows, 
     _check(q, pm, synth.activations(m, cols, seed=1510 + m))
 
 
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("mode,rows,cols,bits,rate", [(0, 1792, 14336, 4, 0.003), (0, 1024, 4096, 3, 0.0), (1, 2500, 2048, 4, 0.01)])
+def test_gemm_calls_of_different_rows_share_a_workspace(mode, rows, cols, bits, rate, dtype):
+    """One workspace, zero-filled once, for prompts of many lengths in mixed order: sums of one call lie where no other call
+    counts, so every call gives the bits of a call with a workspace of its own (and stores every row: y starts as NaN)."""
+    q = synth.random_quantized_torch(mode, rows, cols, bits, rate, 1600 + rows, lib_size=32, group_size=128)
+    pm = xfp.pack_tensors(q)
+    ms = (80, 1792, 16, 300, 64, 1792, 100, 48, 1000, 80)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1610)
+    x = torch.randn((max(ms), cols), generator=g, device="cuda").to(dtype)
+    size = {m: xfp.xfp_gemm_typed_workspace_size(pm.desc, m, dtype) for m in ms}
+    shared = torch.zeros(max(size.values()), dtype=torch.uint8, device="cuda")
+    alone = {}
+    for m in ms:
+        if m not in alone:
+            ws = torch.zeros(size[m], dtype=torch.uint8, device="cuda")
+            alone[m] = torch.full((m, rows), float("nan"), dtype=torch.float32, device="cuda")
+            xfp.xfp_gemm_typed(pm.desc, pm.packed, x[:m], alone[m], ws)
+        y = torch.full((m, rows), float("nan"), dtype=torch.float32, device="cuda")
+        xfp.xfp_gemm_typed(pm.desc, pm.packed, x[:m], y, shared)
+        torch.cuda.synchronize()
+        assert int(shared[:4].view(torch.int32).item()) == 0
+        assert torch.isfinite(alone[m]).all() and torch.equal(y, alone[m]), m
+
+
 def test_gemm_matches_gemv_rows_and_is_deterministic():
     q = synth.random_quantized(0, 512, 4096, 4, 0.01, seed=41)
     pm = xfp.pack_tensors(q)
