@@ -183,7 +183,8 @@ int xfp_gemv_grouped_typed(const xfp_desc* desc, int32_t n, const void* const* p
  * shared-memory bank, fits 128 KB (lib_size * 2^bits <= 1024: L = 32 up to N = 5), else XFP_ERR_UNSUPPORTED.
  *   x  [m][cols] fp16;  y  [m][rows] of y_type (XFP_T_F32, XFP_T_F16 or XFP_T_BF16)
  *   workspace  xfp_gemm_workspace_size(desc, m) bytes, zero-filled once before first use; its counter part is left
- *              zero-filled by every call.  Its first 32-bit word is an error flag: the kernel sets it to 1 if one of
+ *              zero-filled by every call.  The size grows with m, and one workspace serves calls of any number of rows up
+ *              to m in any order (not calls that overlap in time).  Its first 32-bit word is an error flag: the kernel sets it to 1 if one of
  *              its bounded waits ran out (y is then not written); the caller may read it after synchronising.
  *              The library never clears the flag, and a call that set it may leave tile counters behind: a
  *              workspace whose flag reads 1 must be zero-filled again before it is reused.
@@ -195,7 +196,8 @@ int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_
 /* xfp_gemm with typed activations: x_type XFP_T_F16 (the call above) or XFP_T_BF16, the paper's native type.  bf16
  * rows of x are first converted to fp16 (round to nearest even, clamped to +-65504: exact for 2^-14 <= |x| <= 65504)
  * by a small kernel into a scratch area behind the GEMM's own workspace, then multiplied by the same kernel.
- *   workspace  xfp_gemm_typed_workspace_size(desc, m, x_type) bytes, zero-filled once before first use. */
+ *   workspace  xfp_gemm_typed_workspace_size(desc, m, x_type) bytes, zero-filled once before first use; serves calls of
+ *              up to m rows, and of both types where it was sized for XFP_T_BF16. */
 int xfp_gemm_typed_workspace_size(const xfp_desc* desc, int32_t m, int32_t x_type, size_t* workspace_bytes);
 int xfp_gemm_typed(const xfp_desc* desc, const void* packed, const void* x, int32_t x_type, int32_t m, void* y,
                    int32_t y_type, void* workspace, size_t workspace_bytes, void* stream);

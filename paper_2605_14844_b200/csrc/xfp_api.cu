@@ -250,7 +250,7 @@ int xfp_gemm_workspace_size(const xfp_desc* desc, int32_t m, size_t* workspace_b
     if (m < 1) return XFP_ERR_SHAPE;
     const Layout l = layout_of(desc);
     if (!gemm_tc_supported(l, m)) return XFP_ERR_UNSUPPORTED;
-    *workspace_bytes = prefill_workspace_bytes(l, m);
+    *workspace_bytes = prefill_workspace_for_up_to(l, m);
     return XFP_OK;
 }
 

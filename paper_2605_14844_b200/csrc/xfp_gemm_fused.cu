@@ -892,6 +892,31 @@ size_t fused_workspace_bytes(const Layout& l, int M) {
     return prefill_ctrl_bytes(l) + (cut ? (size_t)p.dealt * 4 * p.T * kCh * 4 : 0);
 }
 
+size_t prefill_workspace_for_up_to(const Layout& l, int M) {
+    size_t most = 0;
+    // the 64-row kernel: a function of the rows in sixteens; behind its range also with the transposed x that outliers take, so that
+    // the size of a longer prompt does not depend on their count
+    Layout any = l;
+    if (M > 64 && any.nnz == 0) any.nnz = 1;
+    for (int m = 16; m < M + 16 && m <= 64; m += 16) {
+        const size_t w = gemm_workspace_bytes(any, m < M ? m : M);
+        if (w > most) most = w;
+    }
+    // the pair kernel: its plan is a function of the rows in 32s.  Every plan up to 8192 rows (a few microseconds each); beyond, the
+    // most that any plan writes: a part of 512 rows at both ends of every pair's share.
+    constexpr int kExact = 8192;
+    for (int m = 96; m < M + 32 && m <= kExact; m += 32) {
+        if (!fused_preferred(l, m < M ? m : M)) continue;
+        const size_t w = fused_workspace_bytes(l, m < M ? m : M);
+        if (w > most) most = w;
+    }
+    if (M > kExact && fused_preferred(l, M)) {
+        const size_t w = prefill_ctrl_bytes(l) + (size_t)kPairs * 4 * 512 * kCh * 4;
+        if (w > most) most = w;
+    }
+    return most;
+}
+
 // c.x: the activations as fp16; or bf16, converted first into x_f16
 cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& call, void* x_f16, cudaStream_t s) {
     GemmCall c = call;

@@ -132,9 +132,12 @@ cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaS
 bool fused_preferred(const Layout& l, int M);          // which of the two kernels xfp_gemm takes
 size_t fused_workspace_bytes(const Layout& l, int M);
 cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& c, void* x_f16, cudaStream_t s);
+// what a call of M rows uses
 inline size_t prefill_workspace_bytes(const Layout& l, int M) {
     return fused_preferred(l, M) ? fused_workspace_bytes(l, M) : gemm_workspace_bytes(l, M);
 }
+// what the caller is asked for: enough for a call of any number of rows up to M (what a call uses neither grows nor falls with M)
+size_t prefill_workspace_for_up_to(const Layout& l, int M);
 
 // Batches of 9..16 rows of fp16 x run on the tensor-core kernel (xfp_gemm_tc.cu) when the matrix is large and the blob
 // sparse in outliers: the tcgen05 kernel decodes once for all rows (measurements at batch_prefers_gemm).

@@ -286,6 +286,29 @@ def _expect_exceptions(v, arg):
         assert not isinstance(e.value, xfp.XfpError)          # raised by the tensor, not by a status of the library
 
 
+@pytest.mark.parametrize("mode,rows,cols,bits,nnz", [(0, 4096, 4096, 4, 50000), (0, 28672, 8192, 4, 700000), (1, 10007, 4992, 4, 0),
+                                                     (0, 1792, 14336, 4, 77000), (1, 512, 1024, 6, 100), (0, 64, 65536, 2, 0)])
+def test_prefill_workspace_of_a_long_prompt_serves_shorter_ones(lib, mode, rows, cols, bits, nnz):
+    """The size grows with the rows of x, and a call of fewer rows never finds a workspace of more rows too small (status 5; on
+    a machine without a GPU a call that passes the checks ends with status 7)."""
+    d = _desc(mode=mode, rows=rows, cols=cols, bits=bits, lib_size=16 if mode else 0, nnz=nnz)
+    a, p = C.c_void_p(0x1000), C.byref(d)
+    sz = C.c_size_t()
+    ms = sorted({1, 8, 16, 17, 33, 48, 64, 65, 96, 97, 128, 160, 161, 257, 512, 513, 700, 1024, 1500, 1985, 2048, 5000, 8192, 9000,
+                 70000})
+    for x_type in (1, 2):
+        size = []
+        for m in ms:
+            assert lib.xfp_gemm_typed_workspace_size(p, m, x_type, C.byref(sz)) == 0
+            size.append(sz.value)
+        assert size == sorted(size)
+        if torch.cuda.is_available():
+            continue                                  # the pointers below are no memory
+        for i, m in enumerate(ms):
+            for s in size[i:]:
+                assert lib.xfp_gemm_typed(p, a, a, x_type, m, a, 0, a, s, None) == 7
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "_LIB", None)
     monkeypatch.setattr(binding, "_HERE", str(tmp_path))
