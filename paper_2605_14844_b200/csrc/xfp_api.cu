@@ -256,7 +256,7 @@ int xfp_gemm_workspace_size(const xfp_desc* desc, int32_t m, size_t* workspace_b
 
 // x_type as for xfp_gemm_typed; the sizes and pointers of the call are checked here
 static int gemm_common(const xfp_desc* desc, const void* packed, const void* x, int32_t x_type, int32_t m, void* y,
-                       int32_t y_type, void* workspace, size_t workspace_bytes, cudaStream_t s) {
+                       int32_t y_type, void* workspace, size_t workspace_bytes, cudaStream_t s, int short_cta = -1) {
     int st = check_desc(desc);
     if (st) return st;
     if (m < 1 || y_type < 0 || y_type > 2) return XFP_ERR_SHAPE;
@@ -269,7 +269,7 @@ static int gemm_common(const xfp_desc* desc, const void* packed, const void* x, 
     const size_t need = x_type == XFP_T_BF16 ? align256(own) + gemm_x_scratch_bytes(l, m) : own;
     if (workspace_bytes < need) return XFP_ERR_BUFFER_TOO_SMALL;
     uint16_t* x16 = x_type == XFP_T_BF16 ? (uint16_t*)((char*)workspace + align256(own)) : nullptr;
-    GemmCall c{packed, (const uint16_t*)x, y, m, y_type, workspace, own};
+    GemmCall c{packed, (const uint16_t*)x, y, m, y_type, workspace, own, short_cta};
     if (fused) return launch_gemm_fused(l, c, x16, s) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
     if (x16) {
         if (launch_x_to_f16(x, x16, (size_t)m * l.cols, s) != cudaSuccess) return XFP_ERR_CUDA;
@@ -281,6 +281,13 @@ static int gemm_common(const xfp_desc* desc, const void* packed, const void* x, 
 int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
              void* workspace, size_t workspace_bytes, void* stream) {
     return gemm_common(desc, packed, x, XFP_T_F16, m, y, y_type, workspace, workspace_bytes, (cudaStream_t)stream);
+}
+
+// For tests, not part of the API: xfp_gemm of more than 64 rows in which the bounded waits of one CTA give up at once.
+int xfp_debug_gemm_short_waits(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
+                               void* workspace, size_t workspace_bytes, int32_t cta, void* stream) {
+    if (m <= 64 || cta < 0) return XFP_ERR_SHAPE;
+    return gemm_common(desc, packed, x, XFP_T_F16, m, y, y_type, workspace, workspace_bytes, (cudaStream_t)stream, cta);
 }
 
 int xfp_gemm_typed_workspace_size(const xfp_desc* desc, int32_t m, int32_t x_type, size_t* workspace_bytes) {

@@ -26,8 +26,9 @@
 //            in four parts, the exchange in a cluster of three pairs 3 us.
 //   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
 //            table (D16 = fp16(fp32(scale * lib + mid))); the look-ups are then those of V2.
-// Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace, stops
-// issuing and leaves through the exit that frees its tensor memory.
+// Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace and stops
+// issuing; its cluster then stores no sums that lack a part, waits for what is in flight and leaves through the exit that frees
+// its tensor memory.
 #include <cuda.h>
 
 #include "xfp_internal.h"
@@ -72,6 +73,7 @@ struct FusedArgs {
     int whole;                  // whole tiles per pair; the rest (`stream` super-chunks from tile whole * kPairs on) is dealt
     int stream, dealt;          // evenly to pairs 0 .. dealt - 1
     int tmem_cols;
+    int short_cta;              // tests: the CTA whose waits give up at once (-1: none)
 };
 
 __device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -84,15 +86,16 @@ __device__ __forceinline__ bool test_bar(uint32_t bar, uint32_t parity) {
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kSpins; ++i) {
+// By a whole warp, which leaves it together (a lane that gave up alone would keep the others from the warp's next instruction).
+__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, uint32_t spins) {
+    for (uint32_t i = 0; i < spins; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok) : "r"(bar), "r"(parity), "r"(kPollHint) : "memory");
-        if (ok) return true;
+        if (__all_sync(0xffffffffu, ok)) return true;
     }
     return false;
 }
@@ -298,6 +301,7 @@ struct Outliers {
 struct Bars {
     uint32_t decoded, freed;      // address of slot 0's; slot s is 8 s further
     uint32_t ready;               // of the first CTA of the pair
+    uint32_t spins;               // polls of a wait
 };
 
 // The decode warps' share of one tile: half PART of super-chunks grp, grp + 2, ... of [sc0, sc1): every fourth stage.
@@ -358,7 +362,7 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
             }
         }
         // the slot's previous use: its products are done
-        if (!wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u)) return false;
+        if (!wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u, bars.spins)) return false;
         if (rb_ok) {
             const uint32_t dst = sA + (uint32_t)ring.slot * kABytes + (uint32_t)(q * 32 + lane) * 16u;
 #pragma unroll
@@ -417,7 +421,7 @@ __device__ __forceinline__ bool outlier_tile(const FusedArgs& a, int rb, int q, 
         Ring on = ring;
         on.step(1, a.slots);
         const uint32_t k0 = (uint32_t)sc * kSuper, first = mine + (uint32_t)ring.slot * kABytes, second = mine + (uint32_t)on.slot * kABytes;
-        if (!wait_bar(bars.decoded + 8u * ring.slot, ring.phase) || !wait_bar(bars.decoded + 8u * on.slot, on.phase)) return false;
+        if (!wait_bar(bars.decoded + 8u * ring.slot, ring.phase, bars.spins) || !wait_bar(bars.decoded + 8u * on.slot, on.phase, bars.spins)) return false;
         for (;;) {
             int n = 0;
 #pragma unroll
@@ -485,6 +489,38 @@ __device__ __forceinline__ void store_quad(const FusedArgs& a, int t, int row, c
     if (row + 3 < a.rows) put_y(a.y, o + 3, v.w, a.y_kind);
 }
 
+// After a wait has run out and every warp of the pair has stopped: returns when the copies into ring slot `slot` of both CTAs have
+// landed.  They count their bytes on the first CTA's "ready" barrier (`bar`), whose phase ends when its arrivals are complete and no
+// bytes are outstanding: what one CTA copied and the other did not any more is balanced, the missing arrivals are made up.
+__device__ __noinline__ void drain_copies(int slot, int slots, int x_bytes, const int* copied, uint32_t bar, uint32_t crank) {
+    int last[2];                 // the last stage that each CTA copied into the slot: warp w took the stages of parity w below `end`
+    for (int c = 0; c < 2; ++c) {
+        int end[kCopyWarps], top = 0;
+        for (int w = 0; w < kCopyWarps; ++w) {
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(end[w]) : "r"(peer(sa(copied + w), crank + c)));
+            top = max(top, end[w]);
+        }
+        int j = top - 1 - (top - 1 - slot + slots) % slots;     // the largest below `top` that falls into the slot
+        while (j >= 0 && j >= end[j & 1]) j -= slots;
+        last[c] = max(j, -1);
+    }
+    if (last[0] < 0 && last[1] < 0) return;
+    if (last[0] > last[1]) asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(x_bytes) : "memory");
+    if (last[1] > last[0]) asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(x_bytes) : "memory");
+    uint64_t state;
+    uint32_t pending, ok = 0;
+    do {
+        asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];" : "=l"(state) : "r"(bar) : "memory");
+        asm volatile("mbarrier.pending_count.b64 %0, %1;" : "=r"(pending) : "l"(state));
+    } while (pending > 1);
+    for (uint32_t i = 0; i < kSpins && !ok; ++i)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "l"(state) : "memory");
+}
+
 // SPLIT: a cluster of a.ks pairs on one tile, cut along K.
 template <int N, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
@@ -492,9 +528,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // tables aligned to 8 KB of the shared window, so that an entry's offset is merged with the address, not added
     unsigned char* smem = smem_raw + ((8192u - (sa(smem_raw) & 8191u)) & 8191u);      // the same offset in every CTA
-    __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty;
+    __shared__ __align__(8) uint64_t b_decoded[kMaxSlots], b_ready[kMaxSlots], b_freed[kMaxSlots], acc_full, acc_empty, b_drain;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail, s_last;
+    __shared__ int s_fail, s_last, s_copied[kCopyWarps];
     __shared__ const float* s_part[kPairs];
     // the warp index through a shuffle: uniform as the compiler sees it, so that the roles run on uniform registers
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -503,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     unsigned char* pA = smem + a.tab_bytes;
     unsigned char* pB = pA + (size_t)a.slots * kABytes;
     uint16_t* lib = (uint16_t*)(pB + (size_t)a.slots * a.x_bytes);
-    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), lead)};
+    const Bars bars{sa(b_decoded), sa(b_freed), peer(sa(b_ready), lead), (int)blockIdx.x == a.short_cta ? 0u : kSpins};
     asm volatile("griddepcontrol.launch_dependents;");
 
     if (tid < a.slots) {
@@ -514,6 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     if (tid == 32) {
         init_bar(&acc_full, 1);
         init_bar(&acc_empty, 2 * kDecodeWarps);
+        init_bar(&b_drain, 1);
         s_fail = 0;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -552,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met)
                                   : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met));
             ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
-            ok = ok && wait_bar(sa(&acc_full), acc_ph);
+            ok = ok && wait_bar(sa(&acc_full), acc_ph, bars.spins);
             acc_ph ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = s_tmem + ((uint32_t)(q * 32) << 16);
@@ -588,17 +625,18 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 }
             if (!SPLIT && !whole) {
                 __threadfence();
+                if (!ok) s_fail = 1;                          // a part that is not there is not counted: nobody adds up this tile
                 if (dw < 4 && dw * 32 + lane <= g1 - g0) s_part[dw * 32 + lane] = part_at(g0 + dw * 32 + lane);
                 decode_sync();
                 if (dw == 0 && lane == 0) {
                     int* count = a.ctrl + 1 + 2 * (pc.tile - a.whole * kPairs) + h;
-                    const int last = atomicAdd(count, 1) == g1 - g0;
+                    const int last = !s_fail && atomicAdd(count, 1) == g1 - g0;
                     if (last) *count = 0;
                     s_last = last;
                     __threadfence();
                 }
                 decode_sync();
-                if (s_last && ok) {
+                if (s_last) {
                     // four channels of a row of x per thread and step, four rows and two parts in flight
                     constexpr int kRowsIn = 4;
                     const int ch = lane * 4, orow = (2 * tx + (int)h) * kCh + ch;
@@ -638,12 +676,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     } else if (warp >= kCopyWarp && warp < kCopyWarp + kCopyWarps) {
         cluster_wait();
         asm volatile("griddepcontrol.wait;" ::: "memory");    // x may come from the previous kernel of the stream
-        int n = warp - kCopyWarp;                             // the two warps take the stages in turn
+        int n = warp - kCopyWarp, done = 0;                   // the two warps take the stages in turn; those copied so far end at `done`
         for (int i = 0; ok && piece_of<SPLIT>(a, g, i, pc); ++i) {
             const int t0 = (pc.tile % a.tok_tiles) * a.T;
             for (int st = 2 * pc.sc0; st < 2 * pc.sc1; ++st, ring.step(1, a.slots)) {
                 if (n++ & 1) continue;
-                if (!(ok = wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u))) break;
+                if (!(ok = wait_bar(bars.freed + 8u * ring.slot, ring.phase ^ 1u, bars.spins))) break;
                 if (elected()) {
                     const uint32_t bar = bars.ready + 8u * ring.slot;
                     uint32_t dst = sa(pB) + (uint32_t)(ring.slot * a.x_bytes);
@@ -656,8 +694,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                     }
                 }
                 __syncwarp();
+                done = n - (warp - kCopyWarp);
             }
         }
+        if (lane == 0) s_copied[warp - kCopyWarp] = done;
     } else if (h == 1 || warp != kMmaWarp) {
         cluster_wait();                                       // the first CTA issues the pair's products
     } else {
@@ -671,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             const uint32_t id0 = id | ((uint32_t)(product_rows(a, t0, 0) >> 3) << 17);
             const uint32_t id1 = a.parts > 1 && t0 + a.Tp < a.M ? id | ((uint32_t)(product_rows(a, t0 + a.Tp, 1) >> 3) << 17) : 0u;
             if (i) {
-                ok = wait_bar(sa(&acc_empty), acc_ph);        // the previous piece's sums have been read
+                ok = wait_bar(sa(&acc_empty), acc_ph, bars.spins);        // the previous piece's sums have been read
                 acc_ph ^= 1u;
                 if (!ok) break;
             }
@@ -679,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             uint32_t acc = 0;
             bool there = test_bar(bars.ready + 8u * ring.slot, ring.phase);
             for (int st = 2 * pc.sc0; st < st1; ++st) {
-                if (!there && !(ok = wait_bar(bars.ready + 8u * ring.slot, ring.phase))) break;
+                if (!__all_sync(0xffffffffu, there) && !(ok = wait_bar(bars.ready + 8u * ring.slot, ring.phase, bars.spins))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 Ring on = ring;
                 if (++on.slot == a.slots) { on.slot = 0; on.phase ^= 1u; }
@@ -702,15 +742,25 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
             }
         }
     }
-    if (!ok) { s_fail = 1; atomicExch(a.ctrl, 1); }
+    if (!ok) {                   // every CTA of the cluster learns of it behind the barrier below
+        atomicExch(a.ctrl, 1);
+        for (uint32_t r = 0; r < (SPLIT ? 2u * a.ks : 2u); ++r) asm volatile("st.shared::cluster.u32 [%0], 1;" :: "r"(peer(sa(&s_fail), r)) : "memory");
+    }
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (s_fail)                  // copies in flight land before the CTA goes (a millisecond is a thousand times their way)
-        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
-    __syncwarp();
     cluster_sync();
-    if (SPLIT) {
+    const bool failed = *(volatile int*)&s_fail != 0;             // the same answer in the whole cluster
+    if (failed) {                // nobody leaves before the pair's products and copies in flight are done
+        if (h == 0 && warp == kMmaWarp) {
+            if (elected()) commit_pair(sa(&b_drain), 3u << lead);
+            __syncwarp();
+            wait_bar(sa(&b_drain), 0u, kSpins);
+        }
+        if (h == 0 && tid >= 32 && tid < 32 + a.slots) drain_copies(tid - 32, a.slots, a.x_bytes, s_copied, sa(b_ready) + 8u * (uint32_t)(tid - 32), crank);
+        __syncwarp();
+        cluster_sync();
+    }
+    if (SPLIT && !failed) {
         // this CTA's share of the rows of x of its 128 channels: the slices' sums added in slice order
         const int tile = g / a.ks, slice = g % a.ks, t0 = (tile % a.tok_tiles) * a.T, Tn = min(a.T, a.M - t0);
         const int share = (Tn + a.ks - 1) / a.ks, b0 = slice * share * (kCh / 4), b1 = min(Tn, (slice + 1) * share) * (kCh / 4);
@@ -860,6 +910,7 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
     a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
     a.ks = p.ks; a.sc_slice = p.sc_slice; a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
+    a.short_cta = c.short_cta;
     a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * (p.ks > 1 ? p.pairs * p.tok_tiles * p.ks : p.whole ? kPairs : p.dealt)), 1, 1);

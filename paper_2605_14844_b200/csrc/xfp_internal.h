@@ -108,6 +108,7 @@ struct GemmCall {
     int y_kind;          // 0 fp32, 1 fp16, 2 bf16
     void* workspace;
     size_t workspace_bytes;
+    int short_cta = -1;  // tests of the pair kernel's failure path: the CTA whose bounded waits give up at once
 };
 bool gemm_tc_supported(const Layout& l, int M);
 // The counters of both prefill kernels: one region at the start of the workspace whose size does not depend on the rows of x, so

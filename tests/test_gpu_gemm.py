@@ -6,6 +6,7 @@ D16 + S itself where the outliers are a sparse product added to the accumulator 
 else the dequantised matrix W^ = fp16(D16 + S) (the outliers are added to the decoded tile); both are built from the
 oracle's dequantised matrices.
 """
+import ctypes as C
 import os
 
 import numpy as np
@@ -215,6 +216,35 @@ def test_gemm_calls_of_different_rows_share_a_workspace(mode, rows, cols, bits, 
         torch.cuda.synchronize()
         assert int(shared[:4].view(torch.int32).item()) == 0
         assert torch.isfinite(alone[m]).all() and torch.equal(y, alone[m]), m
+
+
+@pytest.mark.parametrize("mode,rows,cols,bits,m,rate,cta", [
+    (0, 4096, 4096, 4, 100, 0.009, 0),      # K cut over a cluster of three pairs: the CTA that issues a pair's products gives up
+    (0, 4096, 4096, 4, 100, 0.009, 5),      # one that only decodes and copies; the other pairs of its cluster are complete
+    (1, 4096, 4096, 3, 90, 0.0, 3),         # no outliers: the decode warps signal the other CTA themselves
+    (0, 1792, 14336, 4, 80, 0.003, 2),      # tiles in parts that meet in the workspace
+    (0, 20000, 1024, 3, 300, 0.002, 1)])    # whole tiles, several per pair
+def test_gemm_wait_that_runs_out(mode, rows, cols, bits, m, rate, cta):
+    """The bounded waits of one CTA give up at once, those of its peers after their limit of a second: the call ends, the error word
+    says so, and what y holds is either a complete sum or what it held before.  The context and, zero-filled, the workspace serve
+    the next call."""
+    q = synth.random_quantized_torch(mode, rows, cols, bits, rate, 1700 + cta, lib_size=32, group_size=128)
+    pm = xfp.pack_tensors(q)
+    x16 = synth.activations(m, cols, seed=1710)
+    good, ws, xd = _run(q, pm, x16)
+    fn = xfp.load_library().xfp_debug_gemm_short_waits
+    y = torch.full((m, rows), float("nan"), dtype=torch.float32, device="cuda")
+    p = lambda t: C.c_void_p(t.data_ptr())
+    assert fn(C.byref(pm.desc), p(pm.packed), p(xd), m, p(y), 0, p(ws), C.c_size_t(ws.numel()), cta, None) == 0
+    torch.cuda.synchronize()
+    assert int(ws[:4].view(torch.int32).item()) == 1
+    stored = ~torch.isnan(y)
+    assert not stored.all() and torch.equal(y[stored], good[stored])
+    again, _, _ = _run(q, pm, x16)
+    ws.zero_()
+    xfp.xfp_gemm(pm.desc, pm.packed, xd, y, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(again, good) and torch.equal(y, good) and int(ws[:4].view(torch.int32).item()) == 0
 
 
 def test_gemm_matches_gemv_rows_and_is_deterministic():
