@@ -37,6 +37,7 @@
  *    Blobs, pointer lists and routing weights must therefore be complete when the call is made: do not
  *    produce them with a kernel that itself releases its dependents early (a plain kernel, a copy or a memset
  *    on the same stream is fine).
+ *    xfp_gemm and xfp_gemm_typed start early as well but read nothing before the kernels in front are complete.
  */
 #ifndef XFP_H
 #define XFP_H

@@ -801,8 +801,9 @@ size_t gemm_workspace_bytes(const Layout& l, int M) {
 namespace {
 // bf16 rows of x -> fp16 (round to nearest even, clamped to the finite fp16 range), eight values per thread and step
 __global__ void x_to_f16_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n8) {
-    asm volatile("griddepcontrol.launch_dependents;");
+    // in this order: the pair kernel reads the blob without waiting for more than this kernel's release (xfp_gemm_fused.cu)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x)
         dst[i] = x8_as_f16(__ldg(src + i), 1);
 }

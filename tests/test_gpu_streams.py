@@ -99,3 +99,57 @@ def test_host_threads_call_concurrently():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+LATE = """
+#include <cuda_runtime.h>
+// releases its dependents at once, then waits and copies
+__global__ void late_copy_kernel(const uint4* src, uint4* dst, size_t n, long long clocks) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    const long long t0 = clock64();
+    while (clock64() - t0 < clocks) __nanosleep(1000);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = src[i];
+}
+extern "C" int late_copy(const void* src, void* dst, size_t bytes, long long clocks, void* stream) {
+    late_copy_kernel<<<8, 256, 0, (cudaStream_t)stream>>>((const uint4*)src, (uint4*)dst, bytes / 16, clocks);
+    return cudaGetLastError() != cudaSuccess;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def late_copy(tmp_path_factory):
+    import ctypes as C
+    import subprocess
+    from paper_2605_14844_b200 import build as xbuild
+    d = tmp_path_factory.mktemp("late")
+    (d / "late.cu").write_text(LATE)
+    subprocess.run([xbuild.NVCC, *xbuild.FLAGS[:2], "-Xcompiler", "-fPIC", "-shared", str(d / "late.cu"), "-o", str(d / "late.so")],
+                   check=True)
+    fn = C.CDLL(str(d / "late.so")).late_copy
+
+    def call(src, dst, clocks=400000):
+        assert fn(C.c_void_p(src.data_ptr()), C.c_void_p(dst.data_ptr()), C.c_size_t(src.numel()), C.c_longlong(clocks),
+                  C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    return call
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("mode,rows,cols,m", [(0, 4096, 4096, 100), (1, 2560, 2048, 300), (0, 1024, 1024, 40), (0, 1024, 256, 65)])
+def test_prefill_waits_for_a_blob_whose_producer_releases_early(late_copy, mode, rows, cols, m, dtype):
+    """The blob is completed by a kernel that lets its dependents start before it has written it.  The GEMV calls exclude that
+    (xfp.h); the prefill form reads the blob only when the kernel in front is complete.  Both blobs are without outliers and
+    valid, so that a call that read the earlier one would give the earlier matrix's y."""
+    old, new = (xfp.pack_tensors(synth.random_quantized_torch(mode, rows, cols, 4, 0.0, 9700 + i, lib_size=32, group_size=128))
+                for i in range(2))
+    x = torch.randn((m, cols), generator=torch.Generator().manual_seed(9710)).to(dtype).cuda()
+    ws = torch.zeros(xfp.xfp_gemm_typed_workspace_size(new.desc, m, dtype), dtype=torch.uint8, device="cuda")
+    ref, y = (torch.empty((m, rows), dtype=torch.float32, device="cuda") for _ in range(2))
+    xfp.xfp_gemm_typed(new.desc, new.packed, x, ref, ws)
+    for _ in range(3):
+        blob = old.packed.clone()
+        torch.cuda.synchronize()
+        late_copy(new.packed, blob)
+        xfp.xfp_gemm_typed(new.desc, blob, x, y, ws)
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref) and int(ws[:4].view(torch.int32).item()) == 0
