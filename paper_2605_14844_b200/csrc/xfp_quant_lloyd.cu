@@ -121,13 +121,13 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
     // ---- load; moments that bound the buckets and the sums (their own rounding decides nothing) ----
     float v[kEpt];
     float sum = 0.f, sq = 0.f, ab = 0.f, some = 0.f;
-    int kept = 0;
+    int kept = 0;                                // in its upper half the extracted weights (the mask of xfp_quantize holds 0 and 1)
 #pragma unroll
     for (int e = 0; e < kEpt / 4; ++e) {
         const int q = e * TH + tid;
         float4 w = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
         uint32_t x = 0x01010101u;
-        if (q * 4 < K) { w = __ldg(w4 + q); x = m4 ? __ldg(m4 + q) : 0u; }
+        if (q * 4 < K) { w = __ldg(w4 + q); x = m4 ? __ldg(m4 + q) : 0u; kept += __popc(x) << 16; }
         v[4 * e] = (x & 0xffu) ? INFINITY : w.x; v[4 * e + 1] = (x & 0xff00u) ? INFINITY : w.y;
         v[4 * e + 2] = (x & 0xff0000u) ? INFINITY : w.z; v[4 * e + 3] = (x & 0xff000000u) ? INFINITY : w.w;
     }
@@ -147,7 +147,8 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
     sum = sq = ab = some = 0.f; kept = 0;
 #pragma unroll
     for (int w = 0; w < NW; ++w) { sum += s_f[0][w]; sq += s_f[1][w]; ab += s_f[2][w]; some += s_f[3][w]; kept += s_i[w]; }
-    const int n = kept, m = K - n;
+    // weights that are no finite numbers are counted as copies of mu with the extracted ones, but only these have a residual
+    const int n = kept & 0xffff, m = K - n, extracted = kept >> 16;
     Buckets bk{0.f, 0.f, (float)(nb - 1)};
     {
         // 3.3 deviations either side of the mean: a bell-shaped channel then puts at most three or four weights in a bucket
@@ -479,7 +480,7 @@ lloyd_kernel(const float* __restrict__ W, const uint8_t* __restrict__ mask, cons
             for (int j = 1; j < E && bad; ++j) asc = asc && e16[j] >= e16[j - 1];
             s_shift = asc;
             s_mu_idx = m ? nearest_entry(e16, E, mu, asc) : 0;
-            if (rowcnt) rowcnt[row] = m;
+            if (rowcnt) rowcnt[row] = extracted;
         }
     }
     __syncthreads();

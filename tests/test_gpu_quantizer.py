@@ -383,6 +383,21 @@ def test_quantize_reports_a_small_outlier_buffer():
         qb.xfp_quantize(0, _dev(W), _params(), (4,), 0.9, buf)
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("cols", [512, 16512])
+def test_quantize_of_a_matrix_that_is_not_finite(value, cols):
+    """One weight that is no number makes mu one too and nothing is extracted: the row pointers say so as well."""
+    rows = 40
+    W = _weights(rows, cols, 95)
+    W[7, 130] = value
+    buf = qb.QuantBuffers(rows, cols, 0, 4, 0, 4096)
+    res = qb.xfp_quantize(0, _dev(W), _params(), (4,), 0.9, buf)
+    torch.cuda.synchronize()
+    assert res.nnz == 0 and int(buf.mask.max().item()) == 0
+    assert not buf.rowptr.any()
+    assert int(buf.idx.max().item()) < 16
+
+
 # ------------------------------------------------------------------ the paper's layer sizes
 
 @pytest.mark.parametrize("mode,rows,cols,bits", [(0, 4096, 4096, 4), (1, 3072, 4096, 3)])
