@@ -44,7 +44,8 @@ __global__ void __launch_bounds__(kRedThreads) stats_partial(const float* __rest
     if (t < b1) { const float4 w = __ldg(W4 + t); s = ((double)w.x + (double)w.y) + ((double)w.z + (double)w.w); have = 4; }
     else if ((int)threadIdx.x < tail && b1 <= b0) { s = (double)W[(n & ~(int64_t)3) + threadIdx.x]; have = 1; }
     const double ps = block_sum(s, sh), pn = block_sum((double)have, sh);
-    const double p = pn > 0.0 ? ps / pn : 0.0;
+    double p = pn > 0.0 ? ps / pn : 0.0;
+    if (!(fabs(p) < INFINITY)) p = 0.0;        // an infinite weight makes the mean infinite, not the differences from an infinite shift NaN
     double a[4] = {0.0, 0.0, 0.0, 0.0}, q[4] = {0.0, 0.0, 0.0, 0.0};
     for (; t < b1; t += 4 * kRedThreads) {
         float4 w[4];

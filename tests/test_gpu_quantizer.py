@@ -60,6 +60,32 @@ def test_stats_match_serial_fp64(rows, cols):
     assert abs(out.cpu().numpy()[1] - rs) <= 1e-10 * rs
 
 
+@pytest.mark.parametrize("value", [float("inf"), -float("inf")])
+@pytest.mark.parametrize("at", [0, 3, 5000, 383 * 1536 - 1])
+def test_stats_of_an_infinite_weight(value, at):
+    """The mean of a matrix with one infinite weight is that infinity wherever the weight stands, its deviation NaN."""
+    W = _weights(383, 1536, 6)
+    W.reshape(-1)[at] = value
+    out = torch.zeros(2, dtype=torch.float64, device="cuda")
+    qb.xfp_quant_stats(_dev(W), 0, out, _ws(383, 1536))
+    mu, sg = out.cpu().numpy()
+    assert mu == value and np.isnan(sg)
+
+
+def test_stats_where_a_part_does_not_start_like_the_rest():
+    """The one-pass moments are taken around the mean of each part's first values; weights far from them (a block of zeros in
+    front of a narrow band around 1000) cost no precision that the deviation itself does not dwarf."""
+    W = np.full((512, 4096), 1000.0, np.float32) + _weights(512, 4096, 7, rate=0.0)
+    W.reshape(1024, -1)[:, :1024] = 0.0
+    out = torch.zeros(2, dtype=torch.float64, device="cuda")
+    qb.xfp_quant_stats(_dev(W), 0, out, _ws(512, 4096))
+    d = W.astype(np.longdouble)
+    mu = d.mean()
+    sg = np.sqrt(((d - mu) ** 2).mean())
+    got = out.cpu().numpy()
+    assert abs(got[0] - mu) <= 1e-12 * abs(mu) and abs(got[1] - sg) <= 1e-12 * sg
+
+
 # ------------------------------------------------------------------ extraction mask
 
 def _gpu_mask(W, mu, sg, mode, k_or_rate, cap):
