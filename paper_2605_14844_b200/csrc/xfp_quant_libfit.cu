@@ -313,8 +313,11 @@ __global__ void __launch_bounds__(32 * GroupGeo<GS>::WARPS) libfit_group_kernel(
             if (lane == 0) sp[0] = make_double2(0.0, 0.0);
             __syncwarp();
             const double2 all = sp[GS];
-            // values sorted as floats: mu's copies by at most half a float ulp
-            const double slack = 1e-9 * all.y + (double)nx * (dhi - dlo) * fabs(mu) * 2.4e-7;
+            // Values are sorted as floats, which puts mu's copies off by `delta`: a copy's squared error is then off by at most
+            // delta (2 |mu - d| + delta), d the nearest entry, wherever the entries lie (a caller's library may reach far
+            // beyond the group, whose own library lies in [-1, 1] of it).
+            const double delta = fabs(mu - (double)fmu), off = (double)nx * delta;
+            const double slack = 1e-9 * all.y + off * (2.0 * fabs(mu - mid) + delta);
             double score[8], bound[8];
             double least = INFINITY;
 #pragma unroll 1
@@ -350,7 +353,7 @@ __global__ void __launch_bounds__(32 * GroupGeo<GS>::WARPS) libfit_group_kernel(
                         sc += (to.y - at.y) - 2.0 * q * (to.x - at.x) + (double)(c - cut) * q * q;
                         at = to; cut = c; prev = d;
                     }
-                    bd = asc ? slack + 1e-12 * GS * far * far : INFINITY;    // a codebook out of order is always summed exactly
+                    bd = asc ? slack + 2.0 * off * far + 1e-12 * GS * far * far : INFINITY;    // a codebook out of order is always summed exactly
                     least = fmin(least, sc + bd);
                 }
                 score[l0 >> 5] = sc; bound[l0 >> 5] = bd;

@@ -245,6 +245,31 @@ def test_libfit_assign_is_bit_exact(bits, group):
     assert np.array_equal(idx.cpu().numpy(), m.idx)
 
 
+def test_libfit_assign_with_a_library_beyond_the_group():
+    """A caller's library may hold entries far from the group's values (here at +-12 half-widths).  The scores that rule
+    entries out see mu's copies rounded to float; what that shifts grows with the entries' distance, and the two entries here are
+    closer than it: sixteen copies of mu = 1 + 5.5e-8 decide for the upper entry, rounded to 1 they would for the lower."""
+    W = np.ones((1, 128), np.float32)
+    w = W[0, :112]
+    steps = np.linspace(0.002, 0.125, 55).astype(np.float32)
+    w[0:55] = np.float32(1) + (np.round(steps * 2 ** 20) / 2 ** 20).astype(np.float32)
+    w[55:110] = np.float32(1) - (np.round(steps * 2 ** 20) / 2 ** 20).astype(np.float32)
+    w[110] = np.float32(1 - 10 * 2.0 ** -24)
+    mask = np.zeros((1, 128), np.uint8)
+    mask[0, 112:] = 1
+    mu = 1 + 5.5e-8
+    lib = np.array([[-12.0] * 4, [12.0] * 4], np.float16).view(np.uint16)
+    m = xo.quantize_v2a(W, 2, mask, mu, 2, 20, library=lib)
+    assert m.gid[0, 0] == 1
+    idx = torch.full((1, 128), 255, dtype=torch.uint8, device="cuda")
+    gid = torch.full((1, 1), 255, dtype=torch.uint8, device="cuda")
+    gs, gm = (torch.zeros((1, 1), dtype=torch.int16, device="cuda") for _ in range(2))
+    qb.xfp_quant_libfit_assign(_dev(W), _dev(mask), _ms(mu, 0.0), 2, 2, _dev(lib), idx, gid, gs, gm)
+    torch.cuda.synchronize()
+    assert np.array_equal(gid.cpu().numpy(), m.gid) and np.array_equal(idx.cpu().numpy(), m.idx)
+    assert np.array_equal(_u16(gs), m.gscale) and np.array_equal(_u16(gm), m.gmid)
+
+
 # ------------------------------------------------------------------ residual, cosine, median
 
 def _desc(m):
