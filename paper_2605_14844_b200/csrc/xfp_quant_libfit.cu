@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
             u[(int64_t)i * E + j] = v;
             acc = __dadd_rn(acc, __dmul_rn(v, v));
         }
-        nn[i] = acc;
+        nn[i] = acc == acc ? acc : INFINITY;     // a codebook with an infinity has no norm: last, so that `order` is a permutation
     }
     if (gt < 3) flag[gt] = 0;
     grid.sync();
@@ -179,7 +179,12 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
         if (tid < E) {
             const double x = vals[tid];
             int r = 0;
-            for (int j = 0; j < E; ++j) r += vals[j] < x || (vals[j] == x && j < tid);
+            // (entries that are no numbers behind the others, so that every place of the library is written)
+            for (int j = 0; j < E; ++j) {
+                const double v = vals[j];
+                const bool before = v < x || (x != x && v == v), after = x < v || (v != v && x == x);
+                r += before || (!before && !after && j < tid);
+            }
             lib[l * E + r] = d2h(x);
         }
     }

@@ -449,6 +449,26 @@ def test_quantize_of_a_matrix_that_is_not_finite(value, cols):
     assert int(buf.idx.max().item()) < 16
 
 
+def test_quantize_v2a_of_weights_beyond_fp16():
+    """Channels whose codebooks overflow fp16 have no normalised form.  Every output is still defined by the input: two runs over
+    workspaces and outputs of different contents agree, ids and indices stay in their ranges."""
+    rows, cols = 64, 512
+    W = _weights(rows, cols, 96)
+    W[8:16] = np.random.default_rng(97).choice(np.float32([-1e6, 1e6]), (8, cols))
+    got = []
+    for fill in (0, 255):
+        buf = qb.QuantBuffers(rows, cols, 1, 3, 8, 4096)
+        for t in vars(buf).values():
+            if isinstance(t, torch.Tensor):
+                t.view(torch.uint8).fill_(fill)
+        res = qb.xfp_quantize(1, _dev(W), _params(), (3,), 0.9, buf)
+        torch.cuda.synchronize()
+        assert int(buf.gid.max().item()) < 8 and int(buf.idx.max().item()) < 8
+        got.append([t.cpu() for t in (buf.lib.view(-1)[:8 * 8], buf.gid, buf.gscale, buf.gmid, buf.idx, buf.rowptr,
+                                      buf.ocol[:res.nnz], buf.oval[:res.nnz])])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
 # ------------------------------------------------------------------ the paper's layer sizes
 
 @pytest.mark.parametrize("mode,rows,cols,bits", [(0, 4096, 4096, 4), (1, 3072, 4096, 3)])
