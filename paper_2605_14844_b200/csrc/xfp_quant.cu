@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kRedThreads) stats_final(const double2* part, 
         if (cnt) { const double d = v[i].x / (double)cnt - mu; acc += v[i].y + (double)cnt * d * d; }
     }
     const double ss = block_sum(acc, sh);
-    if (threadIdx.x == 0) { ms[0] = mu; ms[1] = sqrt(fmax(ss, 0.0) / (double)n); }
+    if (threadIdx.x == 0) { ms[0] = mu; ms[1] = sqrt((ss < 0.0 ? 0.0 : ss) / (double)n); }   // NaN stays NaN
 }
 
 // ------------------------------------------------------------------ exact selection by radix descent
