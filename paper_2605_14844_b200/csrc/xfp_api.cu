@@ -51,6 +51,20 @@ Layout layout_of(const xfp_desc* d) {
     return make_layout(d->mode, d->rows, d->cols, d->bits, d->lib_size, d->nnz, d->group_size);
 }
 
+// The kernel that takes a GEMV call.
+enum Kernel { kNone, kFrag, kLane, kLaneBatch, kGemm, kPair, kBatch, kV2a, kGeneric };
+Kernel kernel_of(const Layout& l, const GemvCall& c) {
+    // fused epilogues exist in the V2a kernel only (batch 1)
+    if (c.epilogue != 0) return v2a_supported(l, c.batch) && c.batch == 1 ? kV2a : kNone;
+    if (frag_supported(l, c)) return kFrag;
+    if (lane_supported(l, c)) return kLane;
+    if (lane_batch_supported(l, c)) return kLaneBatch;
+    if (!c.packed_list && !c.x_bf16 && batch_prefers_gemm(l, c.batch)) return kGemm;
+    if (pair_supported(l, c.batch, c.n)) return kPair;
+    if (!c.packed_list && batch_supported(l, c.batch)) return kBatch;
+    return v2a_supported(l, c.batch) ? kV2a : kGeneric;
+}
+
 int gemv_common(const xfp_desc* desc, int want_mode, const GemvCall& c, void* stream) {
     int st = check_desc(desc);
     if (st) return st;
@@ -69,37 +83,24 @@ int gemv_common(const xfp_desc* desc, int want_mode, const GemvCall& c, void* st
     if (c.workspace_bytes < need) return XFP_ERR_BUFFER_TOO_SMALL;
     GemvCall cc = c;
     cc.workspace_bytes = need;
-    cudaError_t e;
-    if (c.epilogue != 0) {
-        // fused epilogues exist in the V2a kernel only (batch 1)
-        if (!v2a_supported(l, c.batch) || c.batch != 1) return XFP_ERR_UNSUPPORTED;
-        e = launch_gemv_v2a(l, cc, (cudaStream_t)stream);
-        return e == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (kernel_of(l, cc)) {
+        case kNone: return XFP_ERR_UNSUPPORTED;
+        case kFrag: e = launch_gemv_frag(l, cc, (cudaStream_t)stream); break;
+        case kLane: e = launch_gemv_lane(l, cc, (cudaStream_t)stream); break;
+        case kLaneBatch: e = launch_gemv_lane_batch(l, cc, (cudaStream_t)stream); break;
+        case kGemm: {
+            // many rows of x, few outliers: one decode for all rows on the tensor cores (y = x W^T with W the matrix
+            // xfp_dequant writes; inside the GEMV's bound)
+            GemmCall g{c.packed, c.x, c.y, c.batch, c.y_is_fp16, c.workspace, need};
+            e = launch_gemm_tc(l, g, (cudaStream_t)stream);
+            break;
+        }
+        case kPair: e = launch_gemv_pair(l, cc, (cudaStream_t)stream); break;
+        case kBatch: e = launch_gemv_batch(l, cc, (cudaStream_t)stream); break;
+        case kV2a: e = launch_gemv_v2a(l, cc, (cudaStream_t)stream); break;
+        case kGeneric: e = launch_gemv_generic(l, cc, (cudaStream_t)stream); break;
     }
-    if (frag_supported(l, cc))
-        e = launch_gemv_frag(l, cc, (cudaStream_t)stream);
-    else if (lane_supported(l, cc))
-        e = launch_gemv_lane(l, cc, (cudaStream_t)stream);
-    else if (lane_batch_supported(l, cc))
-        e = launch_gemv_lane_batch(l, cc, (cudaStream_t)stream);
-    else if (!c.packed_list && !c.x_bf16 && batch_prefers_gemm(l, c.batch)
-#ifdef LANE_TUNE
-             && !getenv("XFP_NO_GEMM")   // tuning build: keep batches off the tensor-core kernel
-#endif
-    ) {
-        // many rows of x, few outliers: one decode for all rows on the tensor cores (y = x W^T with W the matrix
-        // xfp_dequant writes; inside the GEMV's bound)
-        GemmCall g{c.packed, c.x, c.y, c.batch, c.y_is_fp16, c.workspace, need};
-        e = launch_gemm_tc(l, g, (cudaStream_t)stream);
-    }
-    else if (pair_supported(l, c.batch, c.n))
-        e = launch_gemv_pair(l, cc, (cudaStream_t)stream);
-    else if (!c.packed_list && batch_supported(l, c.batch))
-        e = launch_gemv_batch(l, cc, (cudaStream_t)stream);
-    else if (v2a_supported(l, c.batch))
-        e = launch_gemv_v2a(l, cc, (cudaStream_t)stream);
-    else
-        e = launch_gemv_generic(l, cc, (cudaStream_t)stream);
     return e == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
 }
 
@@ -283,7 +284,35 @@ int xfp_gemm(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_
     return gemm_common(desc, packed, x, XFP_T_F16, m, y, y_type, workspace, workspace_bytes, (cudaStream_t)stream);
 }
 
-// For tests, not part of the API: xfp_gemm of more than 64 rows in which the bounded waits of one CTA give up at once.
+// For tests, not part of the API: the kernel that takes a GEMV call (Kernel; host only) ...
+int xfp_debug_gemv_kernel(const xfp_desc* desc, int32_t batch, int32_t n, int32_t x_type, int32_t y_type, int32_t epilogue,
+                          int32_t* kernel) {
+    const int st = check_desc(desc);
+    if (st) return st;
+    const Layout l = layout_of(desc);
+    static const void* const list[1] = {};
+    GemvCall c{};
+    c.packed_list = n > 1 ? list : nullptr;
+    c.n = n; c.batch = batch; c.y_is_fp16 = y_type; c.x_bf16 = x_type == XFP_T_BF16; c.epilogue = epilogue;
+    c.workspace_bytes = workspace_bytes_for(l);
+    *kernel = kernel_of(l, c);
+    return XFP_OK;
+}
+
+// ... the plan of a prefill call of more than 64 rows, the i-th piece of work of its pair g (tile, first super-chunk, end; 0 when
+// there is none) ...
+int xfp_debug_prefill_plan(const xfp_desc* desc, int32_t m, int64_t* out) {
+    const int st = check_desc(desc);
+    if (st) return st;
+    if (!fused_preferred(layout_of(desc), m)) return XFP_ERR_UNSUPPORTED;
+    fused_plan_report(layout_of(desc), m, out);
+    return XFP_OK;
+}
+int xfp_debug_prefill_piece(const xfp_desc* desc, int32_t m, int32_t g, int32_t i, int32_t* out) {
+    return fused_piece_report(layout_of(desc), m, g, i, out);
+}
+
+// ... and xfp_gemm of more than 64 rows in which the bounded waits of one CTA give up at once.
 int xfp_debug_gemm_short_waits(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
                                void* workspace, size_t workspace_bytes, int32_t cta, void* stream) {
     if (m <= 64 || cta < 0) return XFP_ERR_SHAPE;

@@ -65,7 +65,7 @@ struct FusedArgs {
     int* ctrl;                  // [0] error word, [1 + 2 * tile + half] arrivals of the parts of a dealt tile (see prefill_ctrl_bytes)
     float* part;                // [2 * pair + which][half][T][128] sums of a part
     int rows, RB, SC, M, ell_slots, GH, L, y_kind;
-    int pairs, tok_tiles;       // tiles: 256 channels, T rows of x
+    int tok_tiles;              // tiles along x; a tile has 256 channels and T rows of x
     int T, Tp, parts;           // one product instruction covers Tp <= 256 rows, the second T - Tp; both multiples of 32
     int slots, x_bytes;         // stages in the ring; bytes of x per stage and CTA
     int tab_bytes;
@@ -179,10 +179,10 @@ struct Ring {
 // super-chunks, at most a tile's worth, so at most two pieces.
 struct Piece { int tile, sc0, sc1; };
 template <bool SPLIT>
-__device__ __forceinline__ bool piece_of(const FusedArgs& a, int g, int i, Piece& p) {
+__host__ __device__ __forceinline__ bool piece_of(const FusedArgs& a, int g, int i, Piece& p) {
     if (SPLIT) {
         const int s = g % a.ks;
-        p.tile = g / a.ks; p.sc0 = s * a.sc_slice; p.sc1 = min(a.SC, p.sc0 + a.sc_slice);
+        p.tile = g / a.ks; p.sc0 = s * a.sc_slice; p.sc1 = a.SC < p.sc0 + a.sc_slice ? a.SC : p.sc0 + a.sc_slice;
         return i == 0;
     }
     if (i < a.whole) { p.tile = g + i * kPairs; p.sc0 = 0; p.sc1 = a.SC; return true; }
@@ -191,7 +191,7 @@ __device__ __forceinline__ bool piece_of(const FusedArgs& a, int g, int i, Piece
     const int u0 = g * a.stream / a.dealt, u1 = (g + 1) * a.stream / a.dealt;      // below 74 * 74 * 512
     const int t = u0 / a.SC + i, b = t * a.SC;
     if (u1 <= b) return false;
-    p.tile = a.whole * kPairs + t; p.sc0 = u0 > b ? u0 - b : 0; p.sc1 = min(a.SC, u1 - b);
+    p.tile = a.whole * kPairs + t; p.sc0 = u0 > b ? u0 - b : 0; p.sc1 = a.SC < u1 - b ? a.SC : u1 - b;
     return true;
 }
 // rows of x of the p-th product of a stage, which begins at row p0: those that exist, rounded up to 32
@@ -886,6 +886,18 @@ FusedPlan plan_fused(const Layout& l, int M) {
     return best;
 }
 
+// what the kernel is told of a plan
+FusedArgs args_of(const Layout& l, int M, const FusedPlan& p) {
+    FusedArgs a = {};
+    a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L;
+    a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
+    a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
+    a.ks = p.ks; a.sc_slice = p.sc_slice; a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
+    a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
+    return a;
+}
+int pairs_of(const FusedPlan& p) { return p.ks > 1 ? p.pairs * p.tok_tiles * p.ks : p.whole ? kPairs : p.dealt; }
+
 template <int N, int MODE>
 cudaError_t launch_n(const Layout& l, const GemmCall& c, bool converted, cudaStream_t s) {
     const FusedPlan p = plan_fused(l, c.M);
@@ -910,17 +922,12 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, bool converted, cudaStr
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
-    FusedArgs a = {};
+    FusedArgs a = args_of(l, c.M, p);
     a.b = blob_at(c.packed, offsets_of(l));
     a.y = c.y; a.ctrl = (int*)c.workspace; a.part = (float*)((char*)c.workspace + prefill_ctrl_bytes(l));
-    a.rows = l.rows; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots; a.GH = l.GH; a.L = l.L; a.y_kind = c.y_kind;
-    a.pairs = p.pairs; a.tok_tiles = p.tok_tiles; a.T = p.T; a.Tp = p.Tp; a.parts = p.parts;
-    a.slots = p.slots; a.x_bytes = p.parts * p.Tp * 64; a.tab_bytes = (int)p.tab;
-    a.ks = p.ks; a.sc_slice = p.sc_slice; a.whole = p.whole; a.stream = p.stream; a.dealt = p.dealt;
-    a.converted = converted; a.short_cta = c.short_cta;
-    a.tmem_cols = p.T <= 32 ? 32 : p.T <= 64 ? 64 : p.T <= 128 ? 128 : p.T <= 256 ? 256 : 512;
+    a.y_kind = c.y_kind; a.converted = converted; a.short_cta = c.short_cta;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * (p.ks > 1 ? p.pairs * p.tok_tiles * p.ks : p.whole ? kPairs : p.dealt)), 1, 1);
+    cfg.gridDim = dim3((unsigned)(2 * pairs_of(p)), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
@@ -973,6 +980,22 @@ size_t prefill_workspace_for_up_to(const Layout& l, int M) {
         if (w > most) most = w;
     }
     return most;
+}
+
+void fused_plan_report(const Layout& l, int M, int64_t* out) {
+    const FusedPlan p = plan_fused(l, M);
+    const int64_t v[] = {p.T, p.Tp, p.parts, p.tok_tiles, p.pairs, p.slots, p.whole, p.stream, p.dealt, p.ks, p.sc_slice, (int64_t)p.smem,
+                         (int64_t)kSmemMax, kMinSlots, kPairs, pairs_of(p), (int64_t)prefill_ctrl_bytes(l),
+                         (int64_t)fused_workspace_bytes(l, M), l.SC};
+    for (size_t i = 0; i < sizeof v / sizeof v[0]; ++i) out[i] = v[i];
+}
+int fused_piece_report(const Layout& l, int M, int g, int i, int32_t* out) {
+    const FusedPlan p = plan_fused(l, M);
+    const FusedArgs a = args_of(l, M, p);
+    Piece pc = {};
+    const bool is = p.ks > 1 ? piece_of<true>(a, g, i, pc) : piece_of<false>(a, g, i, pc);
+    out[0] = pc.tile; out[1] = pc.sc0; out[2] = pc.sc1;
+    return is;
 }
 
 // c.x: the activations as fp16; or bf16, converted first into x_f16

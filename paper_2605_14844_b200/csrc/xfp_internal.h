@@ -133,6 +133,8 @@ cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaS
 bool fused_preferred(const Layout& l, int M);          // which of the two kernels xfp_gemm takes
 size_t fused_workspace_bytes(const Layout& l, int M);
 cudaError_t launch_gemm_fused(const Layout& l, const GemmCall& c, void* x_f16, cudaStream_t s);
+void fused_plan_report(const Layout& l, int M, int64_t* out);                       // for tests
+int fused_piece_report(const Layout& l, int M, int g, int i, int32_t* out);         // for tests
 // what a call of M rows uses
 inline size_t prefill_workspace_bytes(const Layout& l, int M) {
     return fused_preferred(l, M) ? fused_workspace_bytes(l, M) : gemm_workspace_bytes(l, M);

@@ -14,6 +14,7 @@ import pytest
 import torch
 
 from conftest import to_oracle
+from plans import features
 from oracle import xfp_oracle as xo
 import paper_2605_14844_b200 as xfp
 from paper_2605_14844_b200 import synth
@@ -161,15 +162,16 @@ def test_gemm_more_tiles_than_sms(mode, bits, m):
 
 @pytest.mark.parametrize("mode,bits,rows,cols,m,placement", [
     (0, 4, 255, 128, 65, "uniform"),        # one super-chunk, a pair whose second CTA lacks a channel
-    (0, 3, 257, 384, 96, "one_row"),        # a second pair of one channel; K too short to cut evenly
-    (1, 2, 129, 896, 288, "clustered"),     # two products of 160 and 128 rows
-    (0, 5, 512, 1664, 481, "uniform"),      # two products of 256 rows, the last rows of x missing
-    (1, 5, 300, 256, 513, "uniform"),       # two tiles along x, the second nearly empty
+    (0, 3, 257, 384, 96, "one_row"),        # a second pair of one channel; three super-chunks
+    (1, 2, 129, 896, 288, "clustered"),     # K in unequal parts over a cluster of four pairs, five tiles of 64 rows
+    (0, 5, 512, 1664, 481, "uniform"),      # clusters, the last rows of x missing
+    (1, 5, 300, 256, 513, "uniform"),       # nine tiles along x, the last nearly empty
     (0, 6, 20000, 256, 65, "clustered"),    # more tiles than pairs, two super-chunks each
-    (0, 2, 9500, 1152, 600, "uniform")])    # rounds of whole tiles and a dealt rest along x as well
+    (0, 2, 9500, 1152, 600, "uniform")])    # whole tiles on 40 pairs, three along x
 def test_gemm_on_pairs_of_sms(mode, bits, rows, cols, m, placement):
-    """The pair kernel (more than 64 rows of x) at the edges of its tiles, of its products and of its schedule; a second call
-    over the same workspace gives the same bits.  Tolerances as for every other shape (see _check)."""
+    """The pair kernel (more than 64 rows of x) at the edges of its tiles: ragged ends of channels, rows of x and K, placements of
+    outliers; a second call over the same workspace gives the same bits.  Tolerances as for every other shape (see _check).
+    (Products, rings and schedules: test_gemm_plans_of_the_pair_kernel.)"""
     q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=1400 + rows + m, placement=placement)
     pm = xfp.pack_tensors(q, col_bits=16)
     x16 = synth.activations(m, cols, seed=1410 + m)
@@ -185,11 +187,44 @@ def test_gemm_on_pairs_of_sms(mode, bits, rows, cols, m, placement):
 @pytest.mark.parametrize("mode,bits,rows,cols,m", [(1, 2, 2048, 1920, 512), (0, 3, 700, 1024, 512), (0, 6, 513, 640, 300),
                                                    (1, 5, 520, 896, 257), (1, 2, 20000, 384, 500)])
 def test_gemm_on_pairs_without_outliers_and_with_large_tables(mode, bits, rows, cols, m):
-    """The ring of stages at its shortest (tables and x of 512 rows beside it), the decode warps signalling the products directly.
-    Tolerances as for every other shape (see _check)."""
+    """No outliers: the decode warps signal the products directly; tables of every size beside the ring of stages.  Tolerances as
+    for every other shape (see _check)."""
     q = synth.random_quantized(mode, rows, cols, bits, 0.0, seed=1500 + rows + m)
     pm = xfp.pack_tensors(q, col_bits=16)
     _check(q, pm, synth.activations(m, cols, seed=1510 + m))
+
+
+@pytest.mark.parametrize("mode,bits,L,rows,cols,m,rate,want", [
+    (0, 4, 0, 28672, 8192, 512, 0.003, {"cut", "shortest ring", "two pieces", "two products", "whole tiles"}),
+    (0, 4, 0, 28672, 8192, 512, 0.0, {"cut", "shortest ring", "two pieces", "two products", "whole tiles"}),
+    (0, 6, 0, 6194, 9344, 401, 0.002, {"cut", "shortest ring", "two pieces", "two products"}),
+    (0, 2, 0, 9742, 8320, 257, 0.0, {"cut", "two pieces", "two products"}),
+    (0, 5, 0, 9910, 4352, 68, 0.01, {"cut", "two pieces"}),
+    (0, 5, 0, 1182, 13696, 69, 0.02, {"cut"}),
+    (1, 6, 16, 5018, 2432, 282, 0.005, {"cut", "shortest ring", "two pieces", "whole tiles"}),
+    (1, 5, 32, 4693, 4736, 303, 0.003, {"cut", "two pieces"}),
+    (1, 4, 32, 10007, 4992, 512, 0.003, {"cut", "whole tiles"}),
+    (0, 3, 0, 11056, 128, 325, 0.01, {"shortest ring", "two products", "whole tiles"}),
+    (0, 4, 0, 3130, 1920, 279, 0.01, {"cluster", "two products"}),
+    (1, 5, 32, 3180, 1408, 269, 0.0, {"cluster", "shortest ring", "two products"}),
+    (1, 6, 16, 125, 1152, 90, 0.01, {"cluster", "shortest ring"})])
+def test_gemm_plans_of_the_pair_kernel(mode, bits, L, rows, cols, m, rate, want):
+    """Every form of the pair kernel's plan, on shapes whose plan is checked to have it: one or two products per stage, rings
+    down to the shortest, K cut over a cluster, tiles cut through the workspace, pairs that end one tile and begin the next.
+    Held to x W^T in fp64 (torch) with W the matrix xfp_dequant writes (bit-exact by its own tests); a second call over the same
+    workspace gives the same bits."""
+    q = synth.random_quantized_torch(mode, rows, cols, bits, rate, 1800 + rows + m, lib_size=L or 32, group_size=128)
+    pm = xfp.pack_tensors(q)
+    assert features(pm.desc, m) == want
+    x16 = synth.activations(m, cols, seed=1810 + m)
+    y, ws, xd = _run(q, pm, x16)
+    W, x = pm.dequant().double(), xd.double()
+    err, bound = (y.double() - x @ W.T).abs(), TIGHT * (x.abs() @ W.abs().T) + 1e-30
+    assert bool((err <= bound).all()), float((err / bound).max())
+    y2 = torch.full_like(y, float("nan"))
+    xfp.xfp_gemm(pm.desc, pm.packed, xd, y2, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(y, y2) and int(ws[:4].view(torch.int32).item()) == 0
 
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])

@@ -4,6 +4,7 @@ xfp_dequant must match the oracle bit for bit.  The fused GEMV must satisfy
     max_i |y_i - y_ref_i| <= 1e-3 * sum_k |W_ik x_k|
 (the tolerance the benchmark spec states; fp32 accumulation of exact products sits far inside it).
 """
+import ctypes as C
 import os
 
 import numpy as np
@@ -11,6 +12,7 @@ import pytest
 import torch
 
 from conftest import from_oracle, to_oracle
+from plans import gemv_kernel
 from oracle import xfp_oracle as xo
 import paper_2605_14844_b200 as xfp
 from paper_2605_14844_b200 import synth
@@ -160,9 +162,9 @@ def test_batched_shapes_and_split_k(mode, rows, cols, bits):
                                              (1, 4, 64), (1, 2, 256), (1, 6, 64)])
 def test_several_rows_of_x_on_matrices_of_one_round(mode, bits, group):
     """2..16 rows of x on a matrix of 79 row-blocks (more than half the SMs, fewer than all: one resident CTA per
-    row-block, the last one ragged), the shape class on which the one-channel-per-lane kernel with 2, 4 or 8 B
-    fragments per decoded fragment takes most batches (all of them at N = 6, up to 4 rows otherwise; the kernels with
-    two channels per lane take the rest): tiles of 2, 4 and 8 rows, partial tiles (3, 7), two launches (11, 16)."""
+    row-block, the last one ragged): the kernel in the operand layout with partial tiles of eight rows, the pair kernel at two
+    rows of V2, and the one-channel-per-lane kernel with 2, 4 or 8 B fragments for groups of 64 (partial tiles 3 and 7, two
+    launches at 11 and 16)."""
     rows, cols = 2500, 768
     q = synth.random_quantized(mode, rows, cols, bits, 0.015, seed=9100 + 10 * bits + mode + group, group_size=group)
     pm = xfp.pack_tensors(q, col_bits=16)
@@ -186,6 +188,7 @@ def test_several_rows_of_x_on_matrices_of_one_round(mode, bits, group):
 def test_batches_in_the_operand_layout(mode, bits, rows, cols, batch, placement):
     """The kernel of several rows of x at the edges of its tiles and slices; a second call over the same workspace gives the same
     bits and leaves the counters at zero."""
+    assert gemv_kernel(xfp.XfpDesc(mode, rows, cols, bits, 128, 32 if mode else 0, 32, int(0.01 * rows * cols)), batch) == "frag"
     q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=1700 + rows + batch, placement=placement)
     pm = xfp.pack_tensors(q)
     x16 = synth.activations(batch, cols, seed=1710 + batch)
@@ -198,9 +201,10 @@ def test_batches_in_the_operand_layout(mode, bits, rows, cols, batch, placement)
 @pytest.mark.parametrize("mode,bits,rows,cols", [(0, 6, 9600, 2048), (0, 5, 9700, 1024), (1, 4, 19200, 512), (1, 2, 9600, 2048),
                                                  (1, 6, 4800, 1024), (1, 3, 19000, 512)])
 def test_several_rows_of_x_with_resident_ctas_and_a_cut_tail(mode, bits, rows, cols):
-    """More row-blocks than CTA slots: resident CTAs walk several row-blocks with one staged copy of x, and the blocks
-    of the last partial round are cut along K and meet in the workspace (300 or 600 row-blocks on 148 or 296 slots).
-    Repeating the call gives the same bits; the counters are left zero."""
+    """More row-blocks than CTA slots: resident CTAs walk several row-blocks with one staged copy of x (from five rows the
+    kernel in the operand layout), and at two to four rows of the larger matrices the lane kernels cut the blocks of the last
+    partial round along K (300 or 600 row-blocks on 148 or 296 slots).  Repeating the call gives the same bits; the counters are
+    left zero."""
     q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=9300 + bits + rows, placement="clustered")
     pm = xfp.pack_tensors(q, col_bits=16)
     sample = _sample_rows(rows, 96, seed=9301)
@@ -544,6 +548,45 @@ def test_fused_expert_block(bits, n, rows_gu, hidden, y_fp16):
     torch.cuda.synchronize()
     plain = (yu.cpu().numpy().astype(np.float64) * wts[:, None].astype(np.float64)).sum(0)
     assert np.all(np.abs(got - plain) <= 0.05 * TOL * bound + (2.0 ** -10 * np.abs(want) if y_fp16 else 0.0) + 1e-30)
+
+
+@pytest.mark.parametrize("mode,bits", [(0, 4), (1, 3), (1, 6)])
+@pytest.mark.parametrize("half", [0, 1])
+def test_grouped_c_functions_of_the_abi(mode, bits, half):
+    """xfp_gemv_grouped and xfp_gemv_grouped_epilogue of the C ABI (the Python functions of these names go to
+    xfp_gemv_grouped_typed): the same kernels, so the bits of the typed call, which the other tests hold to the oracle."""
+    n, rows, cols = 5, 192, 1024
+    qs = [synth.random_quantized(mode, rows, cols, bits, 0.003, seed=2600 + j) for j in range(n)]
+    if mode:
+        for q in qs[1:]:
+            q.codebook = qs[0].codebook
+    pms = [xfp.pack_tensors(q, col_bits=16) for q in qs]
+    desc = _group_desc(pms)
+    ptr = lambda ts: torch.tensor([t.data_ptr() for t in ts], dtype=torch.int64, device="cuda")
+    xs = [_x_dev(synth.activations(1, cols, seed=2650 + j)) for j in range(n)]
+    blobs, xp = ptr([p.packed for p in pms]), ptr(xs)
+    ws = torch.zeros(n * xfp.xfp_packed_size(desc)[1], dtype=torch.uint8, device="cuda")
+    w = torch.softmax(torch.randn(n, generator=torch.Generator().manual_seed(2690)), 0).cuda()
+    dt = torch.float16 if half else torch.float32
+    lib, p, s = xfp.load_library(), lambda t: C.c_void_p(t.data_ptr()), C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    for epi in (xfp.XFP_EPI_NONE, xfp.XFP_EPI_SWIGLU, xfp.XFP_EPI_COMBINE):
+        if epi != xfp.XFP_EPI_NONE and (mode == 0 or bits > 5):
+            continue
+        got, want = (torch.full((n, rows), float("nan"), dtype=dt, device="cuda") for _ in range(2))
+        yp = ptr([got[j] for j in range(n)])
+        common = (C.byref(desc), n, p(blobs), p(xp), p(yp), half)
+        if epi == xfp.XFP_EPI_NONE:
+            assert lib.xfp_gemv_grouped(*common, p(ws), ws.numel(), s) == 0
+            torch.cuda.synchronize()
+            assert not torch.isnan(got).any()
+            plain = got.clone()
+            got.fill_(float("nan"))
+        assert lib.xfp_gemv_grouped_epilogue(*common, epi, p(w), p(ws), ws.numel(), s) == 0
+        xfp.xfp_gemv_grouped_typed(desc, n, blobs, xp, torch.float16, ptr([want[j] for j in range(n)]), dt, epi, w, ws)
+        torch.cuda.synchronize()
+        assert torch.equal(got.nan_to_num(nan=7e4), want.nan_to_num(nan=7e4)) and not torch.isnan(got[0, :rows // 2]).any()
+        if epi == xfp.XFP_EPI_NONE:
+            assert torch.equal(plain, want)
 
 
 def test_fused_epilogues_are_refused_where_not_built():

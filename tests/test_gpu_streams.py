@@ -8,6 +8,7 @@ import pytest
 import torch
 
 from conftest import to_oracle
+from plans import gemv_kernel
 from oracle import xfp_oracle as xo
 import paper_2605_14844_b200 as xfp
 from paper_2605_14844_b200 import synth
@@ -27,16 +28,22 @@ def _within_bound(q, x16, y):
     assert np.all(np.isfinite(got)) and np.all(np.abs(got - ref) <= TOL * absum + 1e-30)
 
 
-# shapes that reach every GEMV kernel family: batch-1 lane kernel, the kernels with two channels per lane (batch 2 on a
-# small matrix), the batched lane kernel (79 row-blocks), the batched kernel with two channels per lane (8 rows), the
-# general kernel (bf16 is not used here: N = 6 grouped is covered elsewhere), K slices through the workspace (96 x 12288)
+# the kernel in the operand layout at 1 to 16 rows of x, and (KERNELS_OF, checked below) every other kernel of the dispatch;
+# K slices through the workspace (96 x 12288)
 CASES = [(0, 4, 200, 1024, 1), (1, 3, 200, 1024, 1), (0, 4, 200, 1024, 2), (1, 4, 200, 1024, 2), (0, 6, 2500, 768, 4),
          (1, 5, 2500, 768, 3), (0, 3, 640, 2048, 8), (1, 4, 640, 2048, 16), (0, 5, 96, 12288, 1), (1, 6, 2500, 768, 8)]
+KERNELS_OF = {(0, 4, 200, 1024, 4): "frag", (1, 4, 512, 4096, 1): "lane", (0, 5, 9600, 128, 2): "lane_batch",
+              (1, 4, 19200, 512, 12): "gemm", (0, 3, 200, 1024, 2): "pair", (1, 2, 33, 16384, 3): "batch",
+              (1, 3, 19000, 512, 2): "v2a", (1, 2, 32, 40960, 3): "generic"}
+CASES += list(KERNELS_OF)
 
 
 @pytest.mark.parametrize("mode,bits,rows,cols,batch", CASES)
 def test_calls_are_capturable_in_a_cuda_graph(mode, bits, rows, cols, batch):
     """Three dependent-free calls captured on a side stream and replayed twice give the bits of the eager calls."""
+    desc = xfp.XfpDesc(mode, rows, cols, bits, 128, 32 if mode else 0, 32, int(0.01 * rows * cols))
+    want = KERNELS_OF.get((mode, bits, rows, cols, batch))
+    assert want is None or gemv_kernel(desc, batch) == want
     q = synth.random_quantized(mode, rows, cols, bits, 0.01, seed=9500 + 10 * bits + mode + batch)
     pm = xfp.pack_tensors(q, col_bits=16)
     xs = [synth.activations(batch, cols, seed=9600 + i) for i in range(3)]
