@@ -503,12 +503,14 @@ bool plan_frag(const Layout& l, int batch, int sms, FragPlan& p) {
     }
     if (!S) return false;
     p.room = S;
-    // few row-blocks: K slices until the SMs are busy, at least one super-chunk per warp
-    while (l.RB * (S + 1) <= sms && l.SC / (S + 1) >= kFW) ++S;
+    // few row-blocks: K slices until the SMs are busy, at least one super-chunk per warp, and no more than the workspace that
+    // every GEMV kernel shares holds partial sums of, behind the counters
+    const size_t ws = workspace_bytes_for(l), ctrl = align256((size_t)l.RB * 4), per_slice = (size_t)l.RB * NB * 32 * 4;
+    const long long held = ws > ctrl ? (long long)((ws - ctrl) / per_slice) : 0;
+    while (l.RB * (S + 1) <= sms && l.SC / (S + 1) >= kFW && S < held) ++S;
     p.sc_slice = (l.SC + S - 1) / S;
     p.S = (l.SC + p.sc_slice - 1) / p.sc_slice;
-    // partial sums behind the counters, inside the workspace that every GEMV kernel shares
-    if (p.S > 1 && align256((size_t)l.RB * 4) + (size_t)l.RB * p.S * NB * 32 * 4 > workspace_bytes_for(l)) return false;
+    if (p.S > 1 && p.S > held) return false;
     const int ctas = sms / p.S * p.S;
     if (ctas < 1) return false;
     p.grid = l.RB * p.S < ctas ? l.RB * p.S : ctas;

@@ -184,7 +184,9 @@ def test_several_rows_of_x_on_matrices_of_one_round(mode, bits, group):
     (1, 2, 31, 256, 2, "uniform"),          # two rows of a tile of eight
     (0, 2, 40, 640, 3, "one_row"),
     (0, 6, 70, 4224, 1, "clustered"),       # one row of x
-    (1, 3, 65, 2048, 1, "uniform")])
+    (1, 3, 65, 2048, 1, "uniform"),
+    (0, 4, 33, 65536, 16, "uniform"),       # the longest K: as many slices as the workspace holds sums of
+    (1, 5, 24, 48128, 10, "clustered")])
 def test_batches_in_the_operand_layout(mode, bits, rows, cols, batch, placement):
     """The kernel of several rows of x at the edges of its tiles and slices; a second call over the same workspace gives the same
     bits and leaves the counters at zero."""

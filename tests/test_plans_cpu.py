@@ -75,7 +75,7 @@ def test_counters_do_not_depend_on_the_rows_of_x():
 @pytest.mark.parametrize("kernel,mode,rows,cols,bits,kw,batches", [
     ("frag", 0, 4096, 4096, 4, {}, (3, 4, 5, 8, 9, 16)), ("frag", 1, 4096, 4096, 4, {}, (3, 5, 16)),
     ("frag", 0, 256, 1024, 4, {}, (1,)), ("frag", 0, 28672, 8192, 4, {}, (5, 8)), ("frag", 1, 28672, 8192, 4, {}, (5, 8)),
-    ("frag", 0, 33, 65536, 5, {}, (5, 8)),
+    ("frag", 0, 33, 65536, 5, {}, (5, 8, 9, 16)), ("frag", 1, 24, 48128, 5, {}, (10,)),
     ("lane", 0, 4096, 4096, 4, {}, (1,)), ("lane", 1, 28672, 8192, 4, {}, (1,)),
     ("lane_batch", 0, 9600, 2048, 6, {}, (2, 4)), ("lane_batch", 1, 2500, 768, 4, {"group": 64}, (2, 4, 8, 16)),
     ("gemm", 0, 28672, 8192, 4, {}, (9, 16)), ("gemm", 1, 28672, 8192, 4, {}, (9, 16)),
