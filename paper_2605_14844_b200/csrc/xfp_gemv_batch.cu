@@ -1,4 +1,5 @@
-// Batched fused decode, 3..16 rows of x, for V2 and V2a blobs:  y[b] = (D + S) x[b].
+// Batched fused decode of 3 or 4 rows of x, for V2 and V2a blobs:  y[b] = (D + S) x[b].  (xfp_gemv_frag.cu takes five and more, and
+// the smaller matrices at these.)
 //
 // Same decode as xfp_gemv_pair.cu (tables in per-lane shared-memory banks, looked-up half2 used directly as the A
 // fragment of mma.sync.m16n8k16, x on the diagonal lanes of the B fragment), but every decoded fragment is
@@ -17,7 +18,7 @@
 // x is staged in shared memory as 16-byte chunks ordered [k / 8][batch row], so the two diagonal lane groups of a
 // batch pair read adjacent chunks (one wavefront) and outlier columns are gathered from the same copy.  One CTA
 // per SM (16 warps): tables + x take up to ~200 KB.  After the K loop the x area is reused for the cross-warp
-// reduction.  Batches above 8 run as two tiles.
+// reduction.
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
 
@@ -442,6 +443,8 @@ __global__ void __launch_bounds__(kBThreads, 1) gemv_batch_kernel(const BatchArg
 
 static int batch_rpl(const Layout& l) { return (l.mode == 0 && l.bits == 5) ? 1 : 2; }
 
+constexpr int kTile = 4;   // rows of x of a launch
+
 static size_t batch_smem_bytes(const Layout& l, int nbt) {
     const int rpl = batch_rpl(l);
     const size_t x = (size_t)nbt * l.cols * 2, red = (size_t)kBWarps * nbt * 32 * rpl * 4;
@@ -450,17 +453,11 @@ static size_t batch_smem_bytes(const Layout& l, int nbt) {
     return tab + (x > red ? x : red);
 }
 
-// batch tile (4 or 8 rows of x per launch) that fits one CTA per SM, 0 if none does
-static int batch_tile(const Layout& l, int batch) {
-    if (l.bits < 2 || l.bits > 5) return 0;
-    if (batch > 4 && batch_smem_bytes(l, 8) <= 220u * 1024u) return 8;
-    if (batch_smem_bytes(l, 4) <= 220u * 1024u) return 4;
-    return 0;
-}
-
-// V2 blobs, and V2a blobs whose groups are whole super-chunks (groups of 64 weights go to the generic kernel)
+// V2 blobs, and V2a blobs whose groups are whole super-chunks (groups of 64 weights go to the generic kernel), that fit one CTA
+// per SM
 bool batch_supported(const Layout& l, int batch) {
-    return batch > 2 && (l.mode == 0 || l.GH == 1) && batch_tile(l, batch) != 0;
+    return batch > 2 && batch <= kTile && l.bits >= 2 && l.bits <= 5 && (l.mode == 0 || l.GH == 1) &&
+           batch_smem_bytes(l, kTile) <= 220u * 1024u;
 }
 
 template <int N, int NB, int RPL, bool TIO, int MODE>
@@ -499,57 +496,42 @@ static cudaError_t launch_batch_mode(int mode, const BatchArgs& a, dim3 grid, si
 }
 
 cudaError_t launch_gemv_batch(const Layout& l, const GemvCall& c, cudaStream_t s) {
+    if (!batch_supported(l, c.batch)) return cudaErrorInvalidValue;
     const int rpl = batch_rpl(l);
     const int blocks = (l.RB + rpl - 1) / rpl;
     const int slots = sched_sms();   // one CTA per SM
-    for (int b0 = 0; b0 < c.batch; b0 += 8) {
-        const int nb = c.batch - b0 < 8 ? c.batch - b0 : 8;
-        const int nbt = batch_tile(l, nb);
-        if (nbt == 0) return cudaErrorInvalidValue;
-        // a tile of 4 serves up to 4 rows: split an 8-row step in two when only the small tile fits
-        for (int b1 = 0; b1 < nb; b1 += nbt) {
-            const int n1 = nb - b1 < nbt ? nb - b1 : nbt;
-            BatchArgs a{};
-            a.off = offsets_of(l);
-            a.packed = c.packed;
-            a.x = c.x + (size_t)(b0 + b1) * l.cols;
-            a.y = (void*)((char*)c.y + (size_t)(b0 + b1) * l.rows * (c.y_is_fp16 ? 2 : 4));
-            a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.ell_slots = l.ell_slots; a.L = l.L;
-            a.rows_ws = blocks * 32 * rpl;
-            a.nb = n1; a.y_is_fp16 = c.y_is_fp16; a.x_bf16 = c.x_bf16;
-            // schedule: whole-K blocks in whole rounds of slots; the last partial round cut along K (<= 16 slices)
-            int rem = blocks % slots, kst = 1;
-            if (rem > 0) {
-                kst = slots / rem;
-                const int kmax = l.SC / 4 > 1 ? l.SC / 4 : 1;
-                if (kst > kmax) kst = kmax;
-                if (kst > 16) kst = 16;
-                if (kst > l.SC) kst = l.SC;
-            }
-            if (kst <= 1) { kst = 1; rem = 0; }
-            a.n_full = blocks - rem;
-            a.sc_per_split = (l.SC + kst - 1) / kst;
-            a.kst = (l.SC + a.sc_per_split - 1) / a.sc_per_split;
-            if (a.kst <= 1) { a.kst = 1; a.n_full = blocks; rem = 0; }
-            a.tickets = (int*)c.workspace;
-            a.partial = (float*)((char*)c.workspace + align256((size_t)l.RB * 4));   // behind the common counter region
-            const size_t smem = batch_smem_bytes(l, nbt);
-            dim3 grid((unsigned)(a.n_full + rem * a.kst), 1, 1);
-            cudaError_t e = cudaErrorInvalidValue;
-            switch (l.bits * 10 + nbt) {
-                case 24: e = launch_batch_mode<2, 4>(l.mode, a, grid, smem, s); break;
-                case 28: e = launch_batch_mode<2, 8>(l.mode, a, grid, smem, s); break;
-                case 34: e = launch_batch_mode<3, 4>(l.mode, a, grid, smem, s); break;
-                case 38: e = launch_batch_mode<3, 8>(l.mode, a, grid, smem, s); break;
-                case 44: e = launch_batch_mode<4, 4>(l.mode, a, grid, smem, s); break;
-                case 48: e = launch_batch_mode<4, 8>(l.mode, a, grid, smem, s); break;
-                case 54: e = launch_batch_mode<5, 4>(l.mode, a, grid, smem, s); break;
-                case 58: e = launch_batch_mode<5, 8>(l.mode, a, grid, smem, s); break;
-            }
-            if (e != cudaSuccess) return e;
-        }
+    BatchArgs a{};
+    a.off = offsets_of(l);
+    a.packed = c.packed;
+    a.x = c.x;
+    a.y = c.y;
+    a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.ell_slots = l.ell_slots; a.L = l.L;
+    a.rows_ws = blocks * 32 * rpl;
+    a.nb = c.batch; a.y_is_fp16 = c.y_is_fp16; a.x_bf16 = c.x_bf16;
+    // schedule: whole-K blocks in whole rounds of slots; the last partial round cut along K (<= 16 slices)
+    int rem = blocks % slots, kst = 1;
+    if (rem > 0) {
+        kst = slots / rem;
+        const int kmax = l.SC / 4 > 1 ? l.SC / 4 : 1;
+        if (kst > kmax) kst = kmax;
+        if (kst > 16) kst = 16;
+        if (kst > l.SC) kst = l.SC;
     }
-    return cudaSuccess;
+    if (kst <= 1) { kst = 1; rem = 0; }
+    a.n_full = blocks - rem;
+    a.sc_per_split = (l.SC + kst - 1) / kst;
+    a.kst = (l.SC + a.sc_per_split - 1) / a.sc_per_split;
+    if (a.kst <= 1) { a.kst = 1; a.n_full = blocks; rem = 0; }
+    a.tickets = (int*)c.workspace;
+    a.partial = (float*)((char*)c.workspace + align256((size_t)l.RB * 4));   // behind the common counter region
+    const size_t smem = batch_smem_bytes(l, kTile);
+    const dim3 grid((unsigned)(a.n_full + rem * a.kst), 1, 1);
+    switch (l.bits) {
+        case 2: return launch_batch_mode<2, kTile>(l.mode, a, grid, smem, s);
+        case 3: return launch_batch_mode<3, kTile>(l.mode, a, grid, smem, s);
+        case 4: return launch_batch_mode<4, kTile>(l.mode, a, grid, smem, s);
+        default: return launch_batch_mode<5, kTile>(l.mode, a, grid, smem, s);
+    }
 }
 
 }  // namespace xfp

@@ -1,4 +1,5 @@
-// The one-channel-per-lane decode kernel (xfp_gemv_lane.cu) for 2..8 rows of x, V2 and V2a:  Y = X (D + S)^T.
+// The one-channel-per-lane decode kernel (xfp_gemv_lane.cu) for several rows of x:  Y = X (D + S)^T.  2..4 rows of large matrices,
+// and V2a in groups of 64 weights or with a large library at every batch; xfp_gemv_frag.cu takes the rest.
 //
 // Every decoded A fragment is multiplied with one B fragment per row of x (x on the diagonal lanes, as at batch 1),
 // so the look-ups -- the cost that bounds the decode -- are paid once per weight whatever the batch; a row of x adds
@@ -67,23 +68,24 @@ cudaError_t launch_tile(const BatchPlan& p, const LaneArgs& a, int grid, cudaStr
     switch (p.NB) {
         case 2: return launch_nb<N, SGL, MODE, 2>(p.cfg, a, grid, p.smem, s);
         case 4: return launch_nb<N, SGL, MODE, 4>(p.cfg, a, grid, p.smem, s);
-        default: return launch_nb<N, SGL, MODE, 8>(p.cfg, a, grid, p.smem, s);
+        default: break;
     }
+    if constexpr (MODE == 1) return launch_nb<N, SGL, MODE, 8>(p.cfg, a, grid, p.smem, s);
+    return cudaErrorInvalidValue;      // (V2: up to four rows, see lane_batch_preferred)
 }
 
 }  // namespace
 
-// Where this kernel measured faster than the kernels with two channels per lane (xfp_gemv_pair.cu at 2 rows,
-// xfp_gemv_batch.cu, xfp_gemv_v2a.cu), the general kernel and, from 9 rows (5 for V2a and N >= 5 on large blobs), the tcgen05 kernel; sweep over
-// 4096 x 4096 .. 28672 x 8192, every bit width, 2 / 4 / 8 rows, 1 % outliers on a B200 (us per call, this kernel
-// against the other):
+// Of the calls that xfp_gemv_frag.cu leaves: where this kernel measured faster than the kernels with two channels per lane
+// (xfp_gemv_pair.cu at 2 rows, xfp_gemv_batch.cu, xfp_gemv_v2a.cu), the general kernel and, on large blobs from 9 rows (5 for V2a in
+// groups of 64), the tcgen05 kernel; sweep over 4096 x 4096 .. 28672 x 8192, every bit width, 2 / 4 / 8 rows, 1 % outliers on a B200
+// (us per call, this kernel against the other):
 //   * V2 N = 6 (the other kernel is the general one): everywhere (28672 x 8192, 4 rows: 78 against 240) except 2 rows
 //     on matrices of one round (pair kernel 7.2 against 7.6)
-//   * V2 N = 5 (the others keep one channel per lane there too): beyond one round (28672 x 8192, 8 rows: 114 against
-//     160), and on one round where the batched kernel does not fit its shared memory (4096 x 12288, 4 rows: 19 against 54)
-//   * V2 N <= 4: matrices of one round at 3 or 4 rows (4096 x 4096, 4 rows: 7.1 against 8.2); everywhere else two
-//     channels per lane halve the mma count per weight and stay ahead (8192 x 8192, 4 rows: 16.4 against 19.9;
-//     28672 x 8192, 8 rows: 80 against 105)
+//   * V2 N = 5 (the others keep one channel per lane there too): beyond one round, and on one round where the batched kernel does
+//     not fit its shared memory (4096 x 12288, 4 rows: 19 against 54)
+//   * V2 N <= 4: matrices of one round at 3 or 4 rows (4096 x 4096, 4 rows: 7.1 against 8.2); everywhere else two channels per lane
+//     halve the mma count per weight and stay ahead (8192 x 8192, 4 rows: 16.4 against 19.9)
 //   * V2a: up to 4 rows on matrices of one round (4096 x 4096, 2 rows: 7.9 against 11.2), N = 2 up to 4 rows
 //     everywhere, N = 4 at 2 rows and on large matrices up to 4 rows (28672 x 8192: 86 against 92), N = 5 on large
 //     matrices (8 rows: 158 against 198), N = 3 only at 3..4 rows on large matrices (its pair tables of the whole
@@ -96,9 +98,10 @@ static bool lane_batch_preferred(const Layout& l, int batch) {
     if (batch_prefers_gemm(l, batch) && big) return false;
     const bool many = batch > 4;   // tiles of 8 rows
     if (l.mode == 0) {
+        if (many) return false;
         if (l.bits == 6) return !(small && batch == 2);
         if (l.bits == 5) return small ? (batch >= 3 && !batch_supported(l, batch)) : true;
-        return small && batch >= 3 && !many;
+        return small && batch >= 3;
     }
     if ((size_t)l.L * l.E * 128 > 128 * 1024) return true;   // N = 6 at L = 32: the other kernel is the general one
     if (small) return !many || !batch_supported(l, batch);
