@@ -29,12 +29,6 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
     return v;
 }
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory"); }
-// lo | hi << 16 for words whose upper halves are zero, on the FMA pipe (the decode leans on the ALU pipe)
-__device__ __forceinline__ uint32_t join_halves(uint32_t lo, uint32_t hi) {
-    uint32_t d;
-    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
-    return d;
-}
 
 // The decode tables: PAIR: entry t = (first index | second index << N) holds both fp16 values; else entry q holds one.
 // N = 4 entries lie 256 bytes apart (two tables interleaved), so that an index isolated in its own byte becomes the second
@@ -127,7 +121,7 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
                     d[0] = decoded((uint16_t)l4.x); d[1] = decoded((uint16_t)(l4.x >> 16));
                     d[2] = decoded((uint16_t)l4.y); d[3] = decoded((uint16_t)(l4.y >> 16));
 #pragma unroll
-                    for (int t = 0; t < 16; ++t) sts_u32(tab + t * 128, join_halves(d[t & 3], d[t >> 2]));
+                    for (int t = 0; t < 16; ++t) sts_u32(tab + t * 128, join16(d[t & 3], d[t >> 2]));
                 } else {
 #pragma unroll
                     for (int e = 0; e < E; e += 8) {
@@ -154,9 +148,9 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
                     } else if (N == 4) {
                         const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
                         const uint32_t sel = 0x7604u | ((uint32_t)(p & 3) << 4);   // [tab.b3, tab.b2, index byte, tab.b0]
-                        d[i] = join_halves(lds_u32(__byte_perm(wlo, tab, sel)), lds_u32(__byte_perm(whi, tab, sel)));
+                        d[i] = join16(lds_u32(__byte_perm(wlo, tab, sel)), lds_u32(__byte_perm(whi, tab, sel)));
                     } else {
-                        d[i] = join_halves(lds_u32(single_addr<N, 1>(w, 2 * p, tab)), lds_u32(single_addr<N, 1>(w, 2 * p + 1, tab)));
+                        d[i] = join16(lds_u32(single_addr<N, 1>(w, 2 * p, tab)), lds_u32(single_addr<N, 1>(w, 2 * p + 1, tab)));
                     }
                 }
                 const uint4 v = make_uint4(d[0], d[1], d[2], d[3]);

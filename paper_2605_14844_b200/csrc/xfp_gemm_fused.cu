@@ -7,7 +7,7 @@
 //            N / 16 of an fp16 operand there, and sharing x in a pair halves the rest.  (Decoding into global tiles first
 //            and multiplying from there ran at those 9 TB/s: 4096 x 4096, 100 rows 26 us, 28672 x 8192, 1024 rows 640 us.)
 //   stage    64 k: A = W^ [128 channels][64 k] fp16 in core-matrix order (k / 8, channel, 8), 16 KB; B = the CTA's half of
-//            the rows of x in the 128-byte swizzle, by tensor copies.  2 .. 12 stages in a ring: a stage is in decode for
+//            the rows of x in the 128-byte swizzle, by tensor copies.  4 .. 12 stages in a ring: a stage is in decode for
 //            about 1900 clocks (four of them at once), then 300 for its outliers, then in the products.
 //   warps    1 products, 2 copies, 4 outliers, 16 decode.  A stage is decoded by four warps, one per row-block: 64 look-ups per
 //            lane, stored as eight 16-byte vectors.  Outliers: a lane per channel with the next entries of its list in
@@ -53,7 +53,6 @@ constexpr int kMmaWarp = 0, kCopyWarp = 1, kCopyWarps = 2, kOutWarp = 4, kOutWar
 constexpr int kThreads = (kDecodeWarp + kDecodeWarps) * 32;
 constexpr uint32_t kSpins = 1u << 20, kPollHint = 1000;
 constexpr size_t kSmemMax = 226 * 1024;
-constexpr int kLibEntries = 8192;              // V2a library entries staged in shared memory
 constexpr int kMaxCut = 4;                     // pairs of a cluster
 constexpr int kClusters[kMaxCut + 1] = {0, 74, 33, 22, 15};   // clusters of k pairs that a B200 runs at once (cudaOccupancyMaxActiveClusters:
                                                               // a cluster stays inside a GPC); more of them run in turn
@@ -344,14 +343,14 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
                 const float scale = h2f((uint16_t)(sm & 0xffffu)), mid = h2f((uint16_t)(sm >> 16));
                 auto decoded = [&](uint32_t l) { return (uint32_t)f2h(__fmaf_rn(scale, h2f((uint16_t)l), mid)); };
                 if (N == 2) {
-                    const uint2 l4 = slib ? *(const uint2*)(slib + id * (E + 8)) : __ldg((const uint2*)(a.b.cb + (size_t)id * E));
+                    const uint2 l4 = *(const uint2*)(slib + id * (E + 8));
                     const uint32_t d[4] = {decoded(l4.x & 0xffffu), decoded(l4.x >> 16), decoded(l4.y & 0xffffu), decoded(l4.y >> 16)};
 #pragma unroll
                     for (int t = 0; t < 16; ++t) sts32(tab + t * 128, join16(d[t & 3], d[t >> 2]));
                 } else {
 #pragma unroll
                     for (int e = 0; e < E; e += 8) {
-                        const uint4 l8 = slib ? *(const uint4*)(slib + id * (E + 8) + e) : __ldg((const uint4*)(a.b.cb + (size_t)id * E + e));
+                        const uint4 l8 = *(const uint4*)(slib + id * (E + 8) + e);
                         const uint32_t lw[4] = {l8.x, l8.y, l8.z, l8.w};
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -561,8 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
     // previous call's tail, as before, read weights that an early-releasing producer had not written yet; behind itself a call of
     // 4096 x 4096, 100 rows bf16 was 1.4 us faster for it, 19.8 us.)
     if (!a.converted) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const bool staged = MODE == 1 && a.L * T::E <= kLibEntries;
-    if (staged)
+    if (MODE == 1)               // at most 1024 entries (gemm_tc_supported)
         for (int i = tid; i < a.L * T::E; i += kThreads) lib[(i / T::E) * (T::E + 8) + i % T::E] = __ldg(a.b.cb + i);
     __syncthreads();
     if (warp == kMmaWarp) {
@@ -592,9 +590,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
                 decode_sync();
                 have = tx;
             }
-            const uint16_t* slib = staged ? lib : nullptr;
-            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met)
-                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, slib, sa(pA), bars, ring, met));
+            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, lib, sa(pA), bars, ring, met)
+                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, lib, sa(pA), bars, ring, met));
             ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
             ok = ok && wait_bar(sa(&acc_full), acc_ph, bars.spins);
             acc_ph ^= 1u;
@@ -840,7 +837,7 @@ size_t table_bytes(const Layout& l) {
 FusedPlan plan_fused(const Layout& l, int M) {
     FusedPlan best = {};
     const size_t tab = (table_bytes(l) + 1023) & ~size_t(1023);
-    const size_t lib = l.mode && (size_t)l.L * l.E <= kLibEntries ? ((size_t)l.L * (l.E + 8) * 2 + 15) & ~size_t(15) : 0;
+    const size_t lib = l.mode ? ((size_t)l.L * (l.E + 8) * 2 + 15) & ~size_t(15) : 0;
     const int pairs = (l.RB + 7) / 8;
     int last_T = 0;
     for (int n = (M + 511) / 512; n <= (M + 15) / 16; ++n) {          // tiles along the rows of x
@@ -946,9 +943,6 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, bool converted, cudaStr
 
 bool fused_preferred(const Layout& l, int M) {
     static_assert(2 * kPairs <= kSizingSMs, "two counters for each of fewer than kPairs dealt tiles (prefill_ctrl_bytes)");
-#ifdef LANE_TUNE
-    if (const char* e = getenv("XFP_FUSED")) return M >= atoi(e) && gemm_tc_supported(l, M);
-#endif
     return M > 64 && gemm_tc_supported(l, M);
 }
 size_t fused_workspace_bytes(const Layout& l, int M) {

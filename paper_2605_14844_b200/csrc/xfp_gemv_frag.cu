@@ -107,8 +107,8 @@ __device__ __forceinline__ uint32_t ld_early16(const uint16_t* p) {
     return v;
 }
 
-// Staged x: [tile of eight rows][k][8 rows], 16 bytes per k, which ldmatrix.trans turns into B fragments and which gives an outlier its eight values in one load.  The byte offset of k in a tile: the place of k among the eight of its
-// chunk is exclusive-or'ed so that the eight k of a fragment (32 t + 0, 1) and eight staging threads (consecutive chunks) each
+// Staged x: [tile of eight rows][k][8 rows], 16 bytes per k, which ldmatrix.trans turns into B fragments and which gives an outlier
+// its eight values in one load.  The byte offset of k in a tile: the place of k among the eight of its chunk is exclusive-or'ed so that the eight k of a fragment (32 t + 0, 1) and eight staging threads (consecutive chunks) each
 // meet eight bank groups.
 __device__ __forceinline__ uint32_t x_at(int k) {
     const int c = k >> 3;
@@ -562,9 +562,6 @@ cudaError_t launch_rows(int NB, const FragArgs& a, const FragPlan& p, cudaStream
 //   * 1 row: up to 2^19 weights, where a call is launch and latency (256 x 1024 V2 N = 4 4.0 -> 3.1 us)
 bool frag_preferred(const Layout& l, const GemvCall& c, const FragPlan& p) {
     const long long w = (long long)l.rows * l.cols;
-#ifdef LANE_TUNE
-    if (const char* e = getenv("XFP_FRAG")) return c.batch >= atoi(e);
-#endif
     if (c.batch > 8) return c.x_bf16 || !batch_prefers_gemm(l, c.batch);
     if (c.batch > 4) return true;
     if (c.batch > 2) {
