@@ -312,8 +312,9 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     // half, 2m + 1 in the high half): every lane still reads its own bank, whatever ids and indices the lanes hold,
     // and the tables are half as large (64 KB at N = 5, 128 KB at N = 6 with L = 32)
     constexpr bool kHalf = MODE == 1 && SGL;
-    // N = 4: interleaved tables except in the 8-warp CTAs of one row of x, which gained 2 % on their own and lost 2.4 us behind
-    // another launch (4096 x 4096 and 12288 x 4096 in turn: 23.2 us with plain tables, 25.6; the 16-warp CTAs 20.5 -> 19.5)
+    // N = 4: interleaved tables except in the 8-warp CTAs of one row of x (matrices of more than one round), which gained 2 % on
+    // their own and lost 2.4 us behind another launch (4096 x 4096 and 12288 x 4096 in turn: 23.2 us with plain tables, 25.6; the
+    // 16-warp CTAs 20.5 -> 19.5).  That is one pair of shapes, and which part of the launch it is was not found.
     constexpr bool kInter = kHalf && N == 4 && !(W == 8 && NB == 1);
     constexpr int kIdBytes = (kLibPair ? E * E : E) * 128;   // V2a: bytes between the tables of two ids (kHalf: id pairs)
     constexpr int T = C::T;
