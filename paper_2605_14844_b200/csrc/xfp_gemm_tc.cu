@@ -45,9 +45,8 @@ namespace xfp {
 namespace {
 
 constexpr int kTileRows = 128;   // output channels per CTA (the M of the instruction)
-constexpr int kMaxRows = 64;     // rows of x (the N of the instruction); more go to xfp_gemm_fused.cu
-constexpr int kAccCols = 128;    // first column of the A stages behind the accumulator in a CTA that shares its SM,
-constexpr int kAccColsLone = 256;   // and in one that has it to itself
+constexpr int kSmallT = 128;     // accumulator columns of a CTA that shares its SM,
+constexpr int kBigT = 256;       // and of one that has it to itself
 constexpr int kWarps = 8;        // decode warps of one group (row-block x half); the warp behind the last group issues
                                  // the tensor copies and the products.  The CTA that has its SM to itself runs two groups:
                                  // group g decodes the iterations with it % 2 == g, i.e. owns A stage g
@@ -72,15 +71,16 @@ struct GemmArgs {
     // schedule: CTAs [tier_cta[i], tier_cta[i+1]) are the K slices of tiles tier_tile[i].., tier_ks[i] slices of
     // tier_spp[i] super-chunks per tile, their partial sums from slot tier_slot[i] on (unused tiers start at INT_MAX)
     int tier_cta[3], tier_tile[3], tier_n[3], tier_ks[3], tier_spp[3], tier_slot[3];   // tier_n: tiles of the tier
-    int T;            // rows of x, rounded up to 16: of an x tile and of a slot of partial sums
+    int row_tiles;    // tiles along the output channels; tile = token tile * row_tiles + row tile
+    int tstride;      // rows of x per slot of partial sums (the rows of the launch's largest tile)
     int tab_bytes;    // shared-memory bytes of the look-up tables (the x stages follow)
     int L;            // V2a: library size
     int GH;           // V2a: groups per super-chunk (2 when the format's groups hold 64 weights)
-    int acc_cols;     // first column of the A stages (kAccCols, kAccColsLone)
-    int tmem_cols;    // tensor-memory columns of the CTA: the accumulator's and the A stages
+    int maxT;         // rows of x per tile: kSmallT or kBigT; the accumulator's columns and the first column of the A stages
+    int tmem_cols;    // tensor-memory columns of the CTA: the accumulator (maxT) and the A stages
     int ns_log;       // log2 of the A stages: 1 (two; two CTAs per SM) or 2 (four; the CTA that has the SM to itself)
-    int x_stages;     // x tiles in shared memory: kXStages, or 2 where that keeps two CTAs on an SM
-    int b_half;       // bytes of one 64-k half of an x tile: T * 128 (a multiple of 1024)
+    int x_stages;     // x tiles in shared memory: kXStages, or 2 when three large ones do not fit
+    int b_half;       // bytes of one 64-k half of an x tile: rows of x per tile * 128 (a multiple of 1024)
     // the sparse product of the outliers in the epilogue: x transposed, [K][Mp] fp16 with Mp a multiple of 32
     // and zeros behind row M; null: no outliers
     const uint16_t* xT;
@@ -151,6 +151,14 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[32
         : "memory");
 }
 
+// lo | hi << 16 for two table words whose upper halves are zero, as a multiply-add: the decode is bound by the ALU
+// pipe (PRMT, LOP3, SHF), and this moves one of its operations per two weights to the FMA pipe
+__device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
+    return d;
+}
+
 template <int N>
 struct Tab {
     static constexpr int E = 1 << N;
@@ -215,8 +223,10 @@ __device__ __forceinline__ void sparse_rows(const GemmArgs& a, const Outliers& o
 // of iteration i stored by all eight decode warps" (i & 1).  No CTA-wide barrier inside the loop: a decode warp runs
 // up to NS iterations ahead of the products.
 template <int N, int MODE, int PART>
-__device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok, int q, int lane, int sc0, int sc1,
-                                          const unsigned char* tab, uint64_t* bars, uint32_t tmem, int grp, int G) {
+__device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok, int q, int lane, int tid, int Tn,
+                                          int t0, int sc0, int sc1, const unsigned char* tab, unsigned char* sB,
+                                          uint64_t* bars, uint32_t tmem, const CUtensorMap* tmap,
+                                          int grp, int G) {
     using H = Half<N, PART>;
     const int NS = 1 << a.ns_log;
     // byte offset of the lane inside a table entry; N = 4 (V2): the row-block's half of a 256-byte entry as well
@@ -317,7 +327,7 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
 #pragma unroll
             for (int i = 0; i < 32; ++i) d[i] = 0u;
         }
-        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a.acc_cols + s * kAStageCols + PART * 32);
+        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a.maxT + s * kAStageCols + PART * 32);
         tmem_st16<0>(ta, d);
         tmem_st16<16>(ta + 16, d);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -334,9 +344,9 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
 }
 
 // The ninth warp (one thread): x tiles by tensor copy one iteration ahead, the eight products of every stage.
-__device__ __forceinline__ bool mma_loop(const GemmArgs& a, int sc0, int sc1, unsigned char* sB,
+__device__ __forceinline__ bool mma_loop(const GemmArgs& a, int Tn, int t0, int sc0, int sc1, unsigned char* sB,
                                          uint64_t* bars, uint32_t tmem, const CUtensorMap* tmap) {
-    const uint32_t idesc = (1u << 4) | ((uint32_t)(a.T >> 3) << 17) | ((uint32_t)(kTileRows >> 4) << 24);
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(Tn >> 3) << 17) | ((uint32_t)(kTileRows >> 4) << 24);
     const int NS = 1 << a.ns_log;
     const int b_stage = 2 * a.b_half;
     const uint32_t x_bytes = (uint32_t)b_stage;
@@ -349,7 +359,7 @@ __device__ __forceinline__ bool mma_loop(const GemmArgs& a, int sc0, int sc1, un
         for (int h = 0; h < 2; ++h)
             asm volatile(
                 "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                :: "r"(smem_u32(sB + xs * b_stage + h * a.b_half)), "l"(tmap), "r"(sc * kSuper + h * 64), "r"(0), "r"(bar)
+                :: "r"(smem_u32(sB + xs * b_stage + h * a.b_half)), "l"(tmap), "r"(sc * kSuper + h * 64), "r"(t0), "r"(bar)
                 : "memory");
     };
     stage_x(sc0, 0);
@@ -369,7 +379,7 @@ __device__ __forceinline__ bool mma_loop(const GemmArgs& a, int sc0, int sc1, un
 #pragma unroll
         for (int ks = 0; ks < kSuper / 16; ++ks) {
             const uint64_t db = smem_desc_sw128(b0 + (uint32_t)(ks >> 2) * (uint32_t)a.b_half + (uint32_t)(ks & 3) * 32u);
-            umma_f16_ts(tmem, tmem + (uint32_t)(a.acc_cols + s * kAStageCols + ks * 8), db, idesc, (it > 0 || ks > 0) ? 1u : 0u);
+            umma_f16_ts(tmem, tmem + (uint32_t)(a.maxT + s * kAStageCols + ks * 8), db, idesc, (it > 0 || ks > 0) ? 1u : 0u);
         }
         umma_commit(smem_u32(&bars[s]));
         xs = xn;
@@ -410,9 +420,12 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     const int q = warp & 3, part = (warp >> 2) & 1, grp = warp >> 3;   // row-block of the tile, half of the super-chunk, group
     const Work wk = work_of(a, (int)blockIdx.x);
     const int tile = wk.tile, slice = wk.slice;
-    const int rb = tile * 4 + q;
+    const int tile_x = tile % a.row_tiles, tile_y = tile / a.row_tiles;
+    const int rb = tile_x * 4 + q;
     const bool rb_ok = rb < a.RB && warp < DW;
     const int row = rb * kRowsPerBlock + lane;
+    const int t0 = tile_y * a.maxT;
+    const int Tn = min(a.maxT, (a.M - t0 + 15) & ~15);          // rows of x of this tile, rounded up to 16
     const int sc0 = slice * wk.spp;
     const int sc1 = min(a.SC, sc0 + wk.spp);
 
@@ -436,9 +449,9 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
         // codebooks -> one word per (entry, lane); pair tables are built from a copy staged in the x stages
         uint32_t* one = Tab<N>::kPair ? (uint32_t*)sB : (uint32_t*)sTab;
         for (int i = warp; i < 4 * E; i += DW + 1) {
-            const int qq = i / E, e = i % E, r = (tile * 4 + qq) * kRowsPerBlock + lane;
+            const int qq = i / E, e = i % E, r = (tile_x * 4 + qq) * kRowsPerBlock + lane;
             const int slot = N == 4 ? ((qq >> 1) * E + e) * 64 + (qq & 1) * 32 : (qq * E + e) * 32;   // N = 4: see the look-ups
-            one[slot + lane] = (tile * 4 + qq) < a.RB ? (uint32_t)__ldg(a.b.cb + (size_t)r * E + e) : 0u;
+            one[slot + lane] = (tile_x * 4 + qq) < a.RB ? (uint32_t)__ldg(a.b.cb + (size_t)r * E + e) : 0u;
         }
         if (Tab<N>::kPair) {
             __syncthreads();
@@ -488,12 +501,12 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     const unsigned char* tab = MODE == 1 ? sTab : N == 4 ? sTab + (size_t)(q >> 1) * TW * 256 : sTab + (size_t)q * TW * 128;
     bool done;
     if (warp == DW) {
-        done = lane != 0 || mma_loop(a, sc0, sc1, sB, bars, tmem, &tmap);
+        done = lane != 0 || mma_loop(a, Tn, t0, sc0, sc1, sB, bars, tmem, &tmap);
         __syncwarp();
     } else {
         done = part == 0
-            ? main_loop<N, MODE, 0>(a, rb, rb_ok, q, lane, sc0, sc1, tab, bars, tmem, grp, G)
-            : main_loop<N, MODE, 1>(a, rb, rb_ok, q, lane, sc0, sc1, tab, bars, tmem, grp, G);
+            ? main_loop<N, MODE, 0>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, &tmap, grp, G)
+            : main_loop<N, MODE, 1>(a, rb, rb_ok, q, lane, tid, Tn, t0, sc0, sc1, tab, sB, bars, tmem, &tmap, grp, G);
     }
     // what the finish needs of the schedule is worked out again from a fresh read of the CTA index, so that it does
     // not occupy registers through the main loop
@@ -508,16 +521,16 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     } else {
         // lane = channel (tensor-memory lane 32*(warp%4) + lane), registers = 16 consecutive rows of x
         const int r = q * 32 + lane;
-        float* part_out = a.partial + (size_t)(slot0 + slice) * a.T * kTileRows;
-        for (int cc = part + 2 * grp; warp < DW && cc * 16 < a.T; cc += 2 * G) {
+        float* part_out = a.partial + (size_t)(slot0 + slice) * a.tstride * kTileRows;
+        for (int cc = part + 2 * grp; warp < DW && cc * 16 < Tn; cc += 2 * G) {
             uint32_t v[16];
             tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cc * 16), v);
-            if (a.xT && rb_ok) sparse_rows(a, o, cc * 16, (uint32_t)sc1 * kSuper, v);
+            if (a.xT && rb_ok) sparse_rows(a, o, t0 + cc * 16, (uint32_t)sc1 * kSuper, v);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int t = cc * 16 + j;
                 if (ks > 1) part_out[t * kTileRows + r] = __uint_as_float(v[j]);
-                else if (t < a.M && row < a.rows) put_y(a.y, (size_t)t * a.rows + row, __uint_as_float(v[j]), a.y_kind);
+                else if (t0 + t < a.M && row < a.rows) put_y(a.y, (size_t)(t0 + t) * a.rows + row, __uint_as_float(v[j]), a.y_kind);
             }
         }
     }
@@ -539,19 +552,19 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     if (!s_last) return;
     __threadfence();
     // four consecutive channels of one row of x per thread and step: 16-byte loads, all slices of a step in flight
-    const float4* p0 = (const float4*)(a.partial + (size_t)slot0 * a.T * kTileRows);
+    const float4* p0 = (const float4*)(a.partial + (size_t)slot0 * a.tstride * kTileRows);
     constexpr int kQuads = kTileRows / 4;
-    for (int i = tid; i < a.T * kQuads; i += (DW + 1) * 32) {
+    for (int i = tid; i < Tn * kQuads; i += (DW + 1) * 32) {
         const int t = i / kQuads, r = (i % kQuads) * 4;
-        const int orow = tile * kTileRows + r;
-        if (t >= a.M || orow >= a.rows) continue;
+        const int orow = tile_x * kTileRows + r;
+        if (t0 + t >= a.M || orow >= a.rows) continue;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
         for (int z = 0; z < ks; ++z) {
-            const float4 v = __ldcg(p0 + (size_t)z * (a.T * kQuads) + i);
+            const float4 v = __ldcg(p0 + (size_t)z * (a.tstride * kQuads) + i);
             sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
         }
-        const size_t o0 = (size_t)t * a.rows + orow;
+        const size_t o0 = (size_t)(t0 + t) * a.rows + orow;
         put_y(a.y, o0, sum.x, a.y_kind);
         if (orow + 1 < a.rows) put_y(a.y, o0 + 1, sum.y, a.y_kind);
         if (orow + 2 < a.rows) put_y(a.y, o0 + 2, sum.z, a.y_kind);
@@ -590,11 +603,11 @@ __global__ void __launch_bounds__(256) x_transpose_kernel(const uint16_t* __rest
 }
 
 struct Plan {
-    int tiles, T;                // tiles of 128 channels; rows of x, rounded up to 16
+    int row_tiles, tok_tiles;
     // K slices in up to three tiers of tiles (see schedule_tiles); slots: (tile, slice) pairs that store partial sums
     int tier_cta[3], tier_tile[3], tier_n[3], tier_ks[3], tier_spp[3], tier_slot[3];
     int grid, slots;
-    int acc_cols, x_stages;
+    int maxT, x_stages;
     bool lone;        // the CTA with 16 decode warps, alone on its SM (else 8 decode warps, two CTAs per SM)
     size_t tab_bytes, smem;
 };
@@ -609,12 +622,12 @@ constexpr size_t kSmemLimit = 227 * 1024 - 1024;   // dynamic shared memory a CT
 //     CTAs per SM only); what remains of that round is cut to fill the remaining slots, in tiers of finer slices
 //     (74 tiles in halves fill 148 slots, the last 2 tiles go in 32 slices each), CTAs in launch order.
 // A slice holds at least two super-chunks, and a tile at most 32 slices (fewer for many rows of x).  Slices store fp32 partial sums; the last CTA of a tile adds them.
-void schedule_tiles(Plan& p, int tiles, int SC, int sms, int T) {
+void schedule_tiles(Plan& p, int tiles, int SC, int sms, int tmax) {
     const int S = p.lone ? sms : 2 * sms;
     const int kfine = SC / 2 > 1 ? SC / 2 : 1;     // a slice holds at least two super-chunks
     // the tail of a large matrix: the CTA that adds a tile's slices reads slices x rows of x x 512 bytes at the very
-    // end of the launch, at most 256 KB of them (32 slices at 16 rows of x, 8 at 64)
-    const int kcap = 512 / T;
+    // end of the launch, at most 256 KB of them (32 slices at 16 rows of x, 4 at 128)
+    const int kcap = 512 / tmax > 2 ? 512 / tmax : 2;
     const int kmax = kfine < kcap ? kfine : kcap;
     int nb[3] = {0, 0, 0}, kk[3] = {1, 1, 1}, nt = 0;
     if (tiles * 2 <= S) {
@@ -660,37 +673,50 @@ Plan plan_of(const Layout& l, int M, int sms) {
     p.tab_bytes = l.mode == 1 ? (size_t)l.L * l.E * 128 : (size_t)4 * (l.bits <= 3 ? l.E * l.E : l.E) * 128;
     if (l.mode == 0) p.tab_bytes += 8192;                    // room to align the tables to 8 KB in the shared window
     p.tab_bytes = (p.tab_bytes + 1023) & ~size_t(1023);      // the x stages behind the tables are 1024-byte aligned
-    p.T = (M + 15) & ~15;
-    p.acc_cols = kAccCols; p.x_stages = kXStages;
+    p.maxT = kSmallT; p.x_stages = kXStages; p.lone = false;
     // a CTA of 16 decode warps, alone on its SM, when the tables leave no room for two CTAs on an SM (V2a from N = 4: a 64 KB
-    // library); two x stages instead of three where that keeps two CTAs there
-    p.lone = p.tab_bytes + (size_t)2 * p.T * 256 > 113 * 1024;
-    if (p.lone) p.acc_cols = kAccColsLone;
-    else if (p.tab_bytes + (size_t)kXStages * p.T * 256 > 113 * 1024) p.x_stages = 2;
-    p.smem = p.tab_bytes + (size_t)p.x_stages * p.T * 256;
+    // library)
+    const int tsmall = M >= kSmallT ? kSmallT : (M + 15) & ~15;
+    const bool lone = p.tab_bytes + (size_t)2 * tsmall * 256 > 113 * 1024;
+    if (lone) {
+        for (int xs = kXStages; xs >= 2; --xs) {
+            const int tbig = M >= kBigT ? kBigT : (M + 15) & ~15;    // rows of x its largest tile would hold
+            if (p.tab_bytes + (size_t)xs * tbig * 256 <= kSmemLimit) { p.maxT = kBigT; p.x_stages = xs; p.lone = true; break; }
+        }
+    }
+    const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;    // rows of x in the largest tile of this launch
+    // 128-row tiles: two x stages instead of three where that keeps two CTAs on an SM (N = 3 pair tables and N = 6
+    // tables are 32 KB: 28672 x 8192, M = 128, N = 3: 216 us with one CTA per SM)
+    if (!p.lone && p.tab_bytes + (size_t)kXStages * tmax * 256 > 113 * 1024 &&
+        p.tab_bytes + (size_t)2 * tmax * 256 <= 113 * 1024)
+        p.x_stages = 2;
+    p.smem = p.tab_bytes + (size_t)p.x_stages * 16 * tmax * 16;
     if (p.smem < kMinSmem) p.smem = kMinSmem;
     if (p.lone && p.smem < 120 * 1024) p.smem = 120 * 1024;   // alone on its SM: it may hold all 512 columns
-    p.tiles = (l.RB + 3) / 4;
-    schedule_tiles(p, p.tiles, l.SC, sms, p.T);
+    p.row_tiles = (l.RB + 3) / 4;
+    p.tok_tiles = (M + p.maxT - 1) / p.maxT;
+    schedule_tiles(p, p.row_tiles * p.tok_tiles, l.SC, sms, tmax);
     return p;
 }
 
-size_t partial_bytes(const Plan& p) { return (size_t)p.slots * p.T * kTileRows * 4; }
+size_t partial_bytes(const Plan& p, int M);
 
 template <int N, int MODE>
 cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     Plan p = plan_of(l, c.M, sched_sms());
     // workspaces are sized for kSizingSMs: a device with fewer SMs whose own schedule wants more slots takes that one
-    if (partial_bytes(p) > partial_bytes(plan_of(l, c.M, kSizingSMs))) p = plan_of(l, c.M, kSizingSMs);
+    if (partial_bytes(p, c.M) > partial_bytes(plan_of(l, c.M, kSizingSMs), c.M)) p = plan_of(l, c.M, kSizingSMs);
+    const int tmax = c.M >= p.maxT ? p.maxT : (c.M + 15) & ~15;  // rows of x in the largest tile of this launch
+    const int b_half = tmax * 128;
     const size_t tab_bytes = p.tab_bytes, smem = p.smem;
-    // x [M][K] fp16: a box of 64 k x T rows lands as 128-byte rows in the 128-byte swizzle, the B operand's layout
+    // x [M][K] fp16: a box of 64 k x tmax rows lands as 128-byte rows in the 128-byte swizzle, the B operand's layout
     static const EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return cudaErrorNotSupported;
     CUtensorMap tmap;
     {
         const cuuint64_t dims[2] = {(cuuint64_t)l.cols, (cuuint64_t)c.M};
         const cuuint64_t strides[1] = {(cuuint64_t)l.cols * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)p.T};
+        const cuuint32_t box[2] = {64, (cuuint32_t)tmax};
         const cuuint32_t estr[2] = {1, 1};
         if (encode(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<uint16_t*>(c.x), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -715,17 +741,18 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     a.partial = (float*)((char*)c.workspace + prefill_ctrl_bytes(l));
     a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.M = c.M; a.ell_slots = l.ell_slots;
     a.GH = l.GH;
-    a.y_kind = c.y_kind; a.T = p.T; a.b_half = p.T * 128;
+    a.y_kind = c.y_kind; a.b_half = b_half;
     for (int i = 0; i < 3; ++i) {
         a.tier_cta[i] = p.tier_cta[i]; a.tier_tile[i] = p.tier_tile[i]; a.tier_n[i] = p.tier_n[i]; a.tier_ks[i] = p.tier_ks[i];
         a.tier_spp[i] = p.tier_spp[i]; a.tier_slot[i] = p.tier_slot[i];
     }
+    a.row_tiles = p.row_tiles; a.tstride = tmax;
     a.tab_bytes = (int)tab_bytes; a.L = l.L;
     // two A stages beside the accumulator; the CTA that has its SM to itself takes all 512 columns and four stages, so
     // that a group of decode warps does not wait for the products of its previous iteration before it stores the next
-    a.acc_cols = p.acc_cols; a.x_stages = p.x_stages;
+    a.maxT = p.maxT; a.x_stages = p.x_stages;
     a.ns_log = p.lone ? 2 : 1;
-    a.tmem_cols = p.lone ? 512 : 256;
+    a.tmem_cols = p.lone ? 512 : 2 * p.maxT;
     a.xT = nullptr; a.Mp = (c.M + 31) & ~31;
     const size_t xt_off = gemm_xt_offset(l, c.M), xt_bytes = gemm_xt_bytes(l, c.M);
     if (xt_bytes && c.workspace_bytes >= xt_off + xt_bytes) {
@@ -744,11 +771,18 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
 }  // namespace
 
 bool gemm_tc_supported(const Layout& l, int M) {
-    if (M < 1 || M > 65535 * 128) return false;
+    if (M < 1 || (long long)((M + kSmallT - 1) / kSmallT) > 65535) return false;
     return l.mode == 0 || (size_t)l.L * l.E * 128 <= kV2aTabMax;
 }
 
-size_t gemm_core_bytes(const Layout& l, int M) { return prefill_ctrl_bytes(l) + partial_bytes(plan_of(l, M, kSizingSMs)); }
+namespace {
+size_t partial_bytes(const Plan& p, int M) {
+    const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;      // rows of x in the largest tile: the rows of a slot
+    return (size_t)p.slots * tmax * kTileRows * 4;
+}
+}  // namespace
+
+size_t gemm_core_bytes(const Layout& l, int M) { return prefill_ctrl_bytes(l) + partial_bytes(plan_of(l, M, kSizingSMs), M); }
 
 // the transposed copy of x for the sparse outlier product, on a matrix with outliers
 size_t gemm_xt_bytes(const Layout& l, int M) {
@@ -794,7 +828,6 @@ cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaS
 }
 
 cudaError_t launch_gemm_tc(const Layout& l, const GemmCall& c, cudaStream_t s) {
-    if (c.M > kMaxRows) return cudaErrorInvalidValue;
     if (l.mode == 1) {
         switch (l.bits) {
             case 2: return launch_n<2, 1>(l, c, s);
