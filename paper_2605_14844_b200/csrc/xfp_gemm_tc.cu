@@ -45,6 +45,7 @@ namespace xfp {
 namespace {
 
 constexpr int kTileRows = 128;   // output channels per CTA (the M of the instruction)
+constexpr int kMaxRows = 64;     // rows of x of a call; more go to xfp_gemm_fused.cu
 constexpr int kSmallT = 128;     // accumulator columns of a CTA that shares its SM,
 constexpr int kBigT = 256;       // and of one that has it to itself
 constexpr int kWarps = 8;        // decode warps of one group (row-block x half); the warp behind the last group issues
@@ -149,14 +150,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[32
            "r"(r[O + 6]), "r"(r[O + 7]), "r"(r[O + 8]), "r"(r[O + 9]), "r"(r[O + 10]), "r"(r[O + 11]),
            "r"(r[O + 12]), "r"(r[O + 13]), "r"(r[O + 14]), "r"(r[O + 15])
         : "memory");
-}
-
-// lo | hi << 16 for two table words whose upper halves are zero, as a multiply-add: the decode is bound by the ALU
-// pipe (PRMT, LOP3, SHF), and this moves one of its operations per two weights to the FMA pipe
-__device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) {
-    uint32_t d;
-    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(d) : "r"(hi), "r"(lo));
-    return d;
 }
 
 template <int N>
@@ -424,6 +417,8 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
     const int rb = tile_x * 4 + q;
     const bool rb_ok = rb < a.RB && warp < DW;
     const int row = rb * kRowsPerBlock + lane;
+    // one tile along x (a call has at most 64 rows), but in the general form: with tile_y and t0 folded to 0 the compiler's
+    // schedule of the main loop was 2.5 % slower (28672 x 8192 V2a N = 4, 16 rows 102.6 -> 105.2 us)
     const int t0 = tile_y * a.maxT;
     const int Tn = min(a.maxT, (a.M - t0 + 15) & ~15);          // rows of x of this tile, rounded up to 16
     const int sc0 = slice * wk.spp;
@@ -603,7 +598,7 @@ __global__ void __launch_bounds__(256) x_transpose_kernel(const uint16_t* __rest
 }
 
 struct Plan {
-    int row_tiles, tok_tiles;
+    int row_tiles;
     // K slices in up to three tiers of tiles (see schedule_tiles); slots: (tile, slice) pairs that store partial sums
     int tier_cta[3], tier_tile[3], tier_n[3], tier_ks[3], tier_spp[3], tier_slot[3];
     int grid, slots;
@@ -626,7 +621,7 @@ void schedule_tiles(Plan& p, int tiles, int SC, int sms, int tmax) {
     const int S = p.lone ? sms : 2 * sms;
     const int kfine = SC / 2 > 1 ? SC / 2 : 1;     // a slice holds at least two super-chunks
     // the tail of a large matrix: the CTA that adds a tile's slices reads slices x rows of x x 512 bytes at the very
-    // end of the launch, at most 256 KB of them (32 slices at 16 rows of x, 4 at 128)
+    // end of the launch, at most 256 KB of them (32 slices at 16 rows of x, 8 at 64)
     const int kcap = 512 / tmax > 2 ? 512 / tmax : 2;
     const int kmax = kfine < kcap ? kfine : kcap;
     int nb[3] = {0, 0, 0}, kk[3] = {1, 1, 1}, nt = 0;
@@ -674,28 +669,17 @@ Plan plan_of(const Layout& l, int M, int sms) {
     if (l.mode == 0) p.tab_bytes += 8192;                    // room to align the tables to 8 KB in the shared window
     p.tab_bytes = (p.tab_bytes + 1023) & ~size_t(1023);      // the x stages behind the tables are 1024-byte aligned
     p.maxT = kSmallT; p.x_stages = kXStages; p.lone = false;
+    const int T = (M + 15) & ~15;                            // rows of x of the one tile along x
     // a CTA of 16 decode warps, alone on its SM, when the tables leave no room for two CTAs on an SM (V2a from N = 4: a 64 KB
-    // library)
-    const int tsmall = M >= kSmallT ? kSmallT : (M + 15) & ~15;
-    const bool lone = p.tab_bytes + (size_t)2 * tsmall * 256 > 113 * 1024;
-    if (lone) {
-        for (int xs = kXStages; xs >= 2; --xs) {
-            const int tbig = M >= kBigT ? kBigT : (M + 15) & ~15;    // rows of x its largest tile would hold
-            if (p.tab_bytes + (size_t)xs * tbig * 256 <= kSmemLimit) { p.maxT = kBigT; p.x_stages = xs; p.lone = true; break; }
-        }
-    }
-    const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;    // rows of x in the largest tile of this launch
-    // 128-row tiles: two x stages instead of three where that keeps two CTAs on an SM (N = 3 pair tables and N = 6
-    // tables are 32 KB: 28672 x 8192, M = 128, N = 3: 216 us with one CTA per SM)
-    if (!p.lone && p.tab_bytes + (size_t)kXStages * tmax * 256 > 113 * 1024 &&
-        p.tab_bytes + (size_t)2 * tmax * 256 <= 113 * 1024)
-        p.x_stages = 2;
-    p.smem = p.tab_bytes + (size_t)p.x_stages * 16 * tmax * 16;
+    // library); two x stages instead of three where that keeps two CTAs there
+    p.lone = p.tab_bytes + (size_t)2 * T * 256 > 113 * 1024;
+    if (p.lone) p.maxT = kBigT;
+    else if (p.tab_bytes + (size_t)kXStages * T * 256 > 113 * 1024) p.x_stages = 2;
+    p.smem = p.tab_bytes + (size_t)p.x_stages * 16 * T * 16;
     if (p.smem < kMinSmem) p.smem = kMinSmem;
     if (p.lone && p.smem < 120 * 1024) p.smem = 120 * 1024;   // alone on its SM: it may hold all 512 columns
     p.row_tiles = (l.RB + 3) / 4;
-    p.tok_tiles = (M + p.maxT - 1) / p.maxT;
-    schedule_tiles(p, p.row_tiles * p.tok_tiles, l.SC, sms, tmax);
+    schedule_tiles(p, p.row_tiles, l.SC, sms, T);
     return p;
 }
 
@@ -706,7 +690,7 @@ cudaError_t launch_n(const Layout& l, const GemmCall& c, cudaStream_t s) {
     Plan p = plan_of(l, c.M, sched_sms());
     // workspaces are sized for kSizingSMs: a device with fewer SMs whose own schedule wants more slots takes that one
     if (partial_bytes(p, c.M) > partial_bytes(plan_of(l, c.M, kSizingSMs), c.M)) p = plan_of(l, c.M, kSizingSMs);
-    const int tmax = c.M >= p.maxT ? p.maxT : (c.M + 15) & ~15;  // rows of x in the largest tile of this launch
+    const int tmax = (c.M + 15) & ~15;                           // rows of x of the one tile along x
     const int b_half = tmax * 128;
     const size_t tab_bytes = p.tab_bytes, smem = p.smem;
     // x [M][K] fp16: a box of 64 k x tmax rows lands as 128-byte rows in the 128-byte swizzle, the B operand's layout
@@ -777,8 +761,7 @@ bool gemm_tc_supported(const Layout& l, int M) {
 
 namespace {
 size_t partial_bytes(const Plan& p, int M) {
-    const int tmax = M >= p.maxT ? p.maxT : (M + 15) & ~15;      // rows of x in the largest tile: the rows of a slot
-    return (size_t)p.slots * tmax * kTileRows * 4;
+    return (size_t)p.slots * ((M + 15) & ~15) * kTileRows * 4;   // a slot holds the rows of x, rounded up to 16
 }
 }  // namespace
 
@@ -828,6 +811,7 @@ cudaError_t launch_x_to_f16(const void* x_bf16, void* x_f16, size_t elems, cudaS
 }
 
 cudaError_t launch_gemm_tc(const Layout& l, const GemmCall& c, cudaStream_t s) {
+    if (c.M > kMaxRows) return cudaErrorInvalidValue;
     if (l.mode == 1) {
         switch (l.bits) {
             case 2: return launch_n<2, 1>(l, c, s);
