@@ -186,7 +186,8 @@ int xfp_gemv_grouped_typed(const xfp_desc* desc, int32_t n, const void* const* p
  *   workspace  xfp_gemm_workspace_size(desc, m) bytes, zero-filled once before first use; its counter part is left
  *              zero-filled by every call.  The size grows with m, and one workspace serves calls of any number of rows up
  *              to m in any order (not calls that overlap in time).  Its first 32-bit word is an error flag: the kernel sets it to 1 if one of
- *              its bounded waits ran out (y is then not written); the caller may read it after synchronising.
+ *              its bounded waits ran out (y is then incomplete: sums that lack a part are not stored, the rest
+ *              of y is); the caller may read it after synchronising.
  *              The library never clears the flag, and a call that set it may leave tile counters behind: a
  *              workspace whose flag reads 1 must be zero-filled again before it is reused.
  * Results are deterministic (K slices, when the matrix has few rows, are added in slice order). */

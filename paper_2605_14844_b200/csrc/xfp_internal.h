@@ -160,9 +160,8 @@ inline size_t workspace_bytes_for(const Layout& l) {
 }
 
 inline bool batch_prefers_gemm(const Layout& l, int batch) {
-    // 28672 x 8192, us per call, tensor-core kernel against the batched kernels (0.3 % outliers unless noted):
-    //   9..16 rows: V2 N = 4 74 against 124..148 (2 %: 107 against 146..174), V2a 102 against 210..246, N = 2 73
-    //               against 110..133, N = 6 99 against 494..792
+    // 28672 x 8192, us per call, tensor-core kernel against xfp_gemv_frag.cu (0.3 % outliers):
+    //   9..16 rows: V2 N = 4 78 against 107
     //   5..8 rows:  where xfp_gemv_frag.cu (68..77) does not take the blob (V2a in groups of 64 weights): V2a 102 against 123,
     //               V2 N = 6 98 against 115
     int least = ((l.mode || l.bits >= 5) && l.nnz * 100 <= (long long)l.rows * l.cols) ? 5 : 9;

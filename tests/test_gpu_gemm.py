@@ -1,10 +1,9 @@
 """Parity of the prefill form (xfp_gemm, tcgen05 tensor cores) against the CPU oracle, through the C ABI.
 
 Every row of x is one GEMV of the oracle: |y_ti - y_ref_ti| <= 1e-3 * sum_k |W_ik x_tk|.  The kernel's products are
-exact and its sums fp32, so it is also held far more tightly to the matrix it multiplies: up to 128 rows of x that is
-D16 + S itself where the outliers are a sparse product added to the accumulator (few rows of x and few outliers),
-else the dequantised matrix W^ = fp16(D16 + S) (the outliers are added to the decoded tile); both are built from the
-oracle's dequantised matrices.
+exact and its sums fp32, so it is also held far more tightly to the matrix it multiplies: up to 64 rows of x that is
+D16 + S itself, the outliers being a sparse product added to the accumulator, above the dequantised matrix
+W^ = fp16(D16 + S) (the outliers are added to the decoded tile); both are built from the oracle's dequantised matrices.
 """
 import ctypes as C
 import os
@@ -40,8 +39,8 @@ def _run(q, pm, x16, dtype=torch.float32):
 
 
 def _sparse_product(pm, m):
-    """Whether xfp_gemm adds the outliers as a sparse product (few rows of x, few outliers), read off the workspace it
-    asks for: the transposed copy of x is the only part of it that depends on the outlier count."""
+    """Whether xfp_gemm adds the outliers as a sparse product (up to 64 rows of x), read off the workspace it asks for: up
+    to there the transposed copy of x is the part of it that depends on the outlier count."""
     d = pm.desc
     bare = xfp.XfpDesc(d.mode, d.rows, d.cols, d.bits, d.group_size, d.lib_size, d.col_bits, 0)
     return xfp.xfp_gemm_workspace_size(d, m) > xfp.xfp_gemm_workspace_size(bare, m)
