@@ -24,8 +24,13 @@
 //            Where clusters of 2 or 3 pairs on one tile each fit the GPU at once (few tiles), they cut K instead and the sums
 //            meet through distributed shared memory: writing and reading them through L2 takes 9 us at 4096 x 4096, 100 rows
 //            in four parts, the exchange in a cluster of three pairs 3 us.
-//   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights into a column of its warp's
-//            table (D16 = fp16(fp32(scale * lib + mid))); the look-ups are then those of V2.
+//   look-ups up to N = 4: the codebook in registers, PRMT look-ups (xfp_reg_decode.cuh); a stage's operands,
+//            their copies and 64 look-ups per lane share the data pipe of shared memory, and the PRMTs stay off it (look-ups in
+//            tables -> registers: 10007 x 4992 V2a, 301 rows 57.5 -> 49.1 us; 28672 x 8192 V2a, 512 rows 282 -> 268, V2, 1024 rows
+//            421 -> 406; 4096 x 4096 V2, 100 rows 21.3 -> 20.9).  V2 at N <= 3
+//            in a cluster: pair tables; above N = 4 one entry per index.
+//   V2a      a lane decodes the 2^N entries its channel's group can take once per 64 weights (D16 = fp16(fp32(scale * lib + mid)));
+//            the look-ups are then those of V2.
 // Waits on barriers have an iteration limit; when one runs out the CTA records it in the first word of the workspace and stops
 // issuing; its cluster then stores no sums that lack a part, waits for what is in flight and leaves through the exit that frees
 // its tensor memory.
@@ -33,6 +38,7 @@
 
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
+#include "xfp_reg_decode.cuh"
 
 namespace xfp {
 
@@ -305,13 +311,14 @@ struct Bars {
 };
 
 // The decode warps' share of one tile: half PART of super-chunks grp, grp + 2, ... of [sc0, sc1): every fourth stage.
-template <int N, int MODE, int PART>
+// REG: from a codebook in registers.
+template <int N, int MODE, int PART, bool REG>
 __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_ok, int q, int grp, int lane, int sc0, int sc1,
-                                            uint32_t tab, const uint16_t* slib, uint32_t sA, const Bars& bars, Ring ring, bool& met) {
+                                            uint32_t tab, RegBook<REG ? N : 2>& book, const uint16_t* slib, uint32_t sA,
+                                            const Bars& bars, Ring ring, bool& met) {
     using T = Tab<N, MODE>;
     using H = Half<N, PART>;
     constexpr int E = T::E;
-    const uint32_t nib = ((tab >> 12) & 0xfu) * 0x10101010u;
     const uint4* idx = a.b.idx + ((size_t)rb * a.SC + sc0 + grp) * N * 32 + lane;
     const size_t meta0 = (((size_t)rb * a.SC + sc0 + grp) * a.GH + (a.GH - 1) * PART) * 32 + lane;
     uint4 nx[H::NV];
@@ -340,14 +347,14 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
             const uint32_t id = id_n, sm = sm_n;
             if (sc + 2 < sc1) fetch(it + 1);
             if (MODE == 1) {
-                const float scale = h2f((uint16_t)(sm & 0xffffu)), mid = h2f((uint16_t)(sm >> 16));
-                auto decoded = [&](uint32_t l) { return (uint32_t)f2h(__fmaf_rn(scale, h2f((uint16_t)l), mid)); };
-                if (N == 2) {
-                    const uint2 l4 = *(const uint2*)(slib + id * (E + 8));
-                    const uint32_t d[4] = {decoded(l4.x & 0xffffu), decoded(l4.x >> 16), decoded(l4.y & 0xffffu), decoded(l4.y >> 16)};
-#pragma unroll
-                    for (int t = 0; t < 16; ++t) sts32(tab + t * 128, join16(d[t & 3], d[t >> 2]));
+                if constexpr (REG) {
+                    uint32_t d[E / 2];
+                    load_entries<N>(d, slib + id * (E + 8), [](auto* p) { return *p; });
+                    affine_entries<N>(d, sm);
+                    book = book_of<N>(d);
                 } else {
+                    const float scale = h2f((uint16_t)(sm & 0xffffu)), mid = h2f((uint16_t)(sm >> 16));
+                    auto decoded = [&](uint32_t l) { return (uint32_t)f2h(__fmaf_rn(scale, h2f((uint16_t)l), mid)); };
 #pragma unroll
                     for (int e = 0; e < E; e += 8) {
                         const uint4 l8 = *(const uint4*)(slib + id * (E + 8) + e);
@@ -367,21 +374,20 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
             const uint32_t dst = sA + (uint32_t)ring.slot * kABytes + (uint32_t)(q * 32 + lane) * 16u;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                uint32_t d[4];
+                uint4 v;
+                if constexpr (REG) {
+                    v = reg_decode8_ordered<N>(w, PART * 8 + c, book);
+                } else {
+                    uint32_t d[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int p = PART * 32 + c * 4 + i;
-                    if (T::kPair) {
-                        d[i] = lds32(pair_addr<N, 1>(w, p, tab));
-                    } else if (N == 4) {
-                        const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
-                        const uint32_t sel = 0x7604u | ((uint32_t)(p & 3) << 4);   // [tab.b3, tab.b2, index byte, tab.b0]
-                        d[i] = join16(lds32(__byte_perm(wlo, tab, sel)), lds32(__byte_perm(whi, tab, sel)));
-                    } else {
-                        d[i] = join16(lds32(single_addr<N, 1>(w, 2 * p, tab)), lds32(single_addr<N, 1>(w, 2 * p + 1, tab)));
+                    for (int i = 0; i < 4; ++i) {
+                        const int p = PART * 32 + c * 4 + i;
+                        if (T::kPair) d[i] = lds32(pair_addr<N, 1>(w, p, tab));
+                        else d[i] = join16(lds32(single_addr<N, 1>(w, 2 * p, tab)), lds32(single_addr<N, 1>(w, 2 * p + 1, tab)));
                     }
+                    v = make_uint4(d[0], d[1], d[2], d[3]);
                 }
-                sts128(dst + (uint32_t)c * 2048u, d[0], d[1], d[2], d[3]);
+                sts128(dst + (uint32_t)c * 2048u, v.x, v.y, v.z, v.w);
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the products read through the async proxy
@@ -525,6 +531,10 @@ __device__ __noinline__ void drain_copies(int slot, int slots, int x_bytes, cons
 template <int N, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
     using T = Tab<N, MODE>;
+    // Codebooks in registers: V2a up to N = 4 and V2 at N = 4, which would take a look-up per weight; V2 at N = 2, 3 instead of pair
+    // tables where a pair walks its tiles (10007 x 4992 N = 3, 301 rows 42.5 -> 40.3 us, 28672 x 8192, 512 rows 237 -> 233), not where
+    // a cluster cuts one tile (4096 x 4096, 100 rows 21.3 against 21.5)
+    constexpr bool kReg = MODE == 0 ? N == 4 || (N <= 3 && !SPLIT) : N <= 4;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // tables aligned to 8 KB of the shared window, so that an entry's offset is merged with the address, not added
     unsigned char* smem = smem_raw + ((8192u - (sa(smem_raw) & 8191u)) & 8191u);      // the same offset in every CTA
@@ -580,18 +590,23 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs
         const int dw = warp - kDecodeWarp, q = dw & 3, part = (dw >> 2) & 1, grp = dw >> 3;
         const uint32_t tab = T::at(sa(smem), MODE == 0 ? q : dw, lane);
         bool met = false;                                     // has waited for the other CTA's barriers
-        int have = -1;                                        // tile of channels whose tables are in place
+        int have = -1;                                        // tile of channels whose codebooks are in place
+        RegBook<kReg ? N : 2> book;
         for (int i = 0; piece_of<SPLIT>(a, g, i, pc); ++i) {         // a warp whose wait ran out still meets the others at their barrier
             const int tx = pc.tile / a.tok_tiles, ty = pc.tile % a.tok_tiles, t0 = ty * a.T;
             const int rb = (2 * tx + (int)h) * 4 + q;
             if (MODE == 0 && tx != have) {
-                decode_sync();                                // every warp is done with the previous tables
-                fill_tables<N>(a, sa(smem), rb - q, dw, lane);
-                decode_sync();
+                if constexpr (kReg) {
+                    if (rb < a.RB) book = make_book<N>(a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * T::E);
+                } else {
+                    decode_sync();                            // every warp is done with the previous tables
+                    fill_tables<N>(a, sa(smem), rb - q, dw, lane);
+                    decode_sync();
+                }
                 have = tx;
             }
-            ok = ok && (part == 0 ? decode_tile<N, MODE, 0>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, lib, sa(pA), bars, ring, met)
-                                  : decode_tile<N, MODE, 1>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, lib, sa(pA), bars, ring, met));
+            ok = ok && (part == 0 ? decode_tile<N, MODE, 0, kReg>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, book, lib, sa(pA), bars, ring, met)
+                                  : decode_tile<N, MODE, 1, kReg>(a, rb, rb < a.RB, q, grp, lane, pc.sc0, pc.sc1, tab, book, lib, sa(pA), bars, ring, met));
             ring.jump(2 * (pc.sc1 - pc.sc0), a.slots);
             ok = ok && wait_bar(sa(&acc_full), acc_ph, bars.spins);
             acc_ph ^= 1u;
@@ -827,6 +842,7 @@ double slot_clocks(const Layout& l, int T) {
     return m > feed ? m : feed;
 }
 
+// (the plans keep the room of the tables where codebooks sit in registers)
 size_t table_bytes(const Layout& l) {
     const size_t one = l.mode == 0 ? (l.bits <= 3 ? l.E * l.E : l.E) : (l.bits == 2 ? 16 : l.E);
     const size_t units = l.mode == 0 ? 4 : kDecodeWarps;
