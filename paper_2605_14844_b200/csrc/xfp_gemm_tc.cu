@@ -15,8 +15,10 @@
 //            {64 k, T rows} (128 contiguous bytes per row of x; rows beyond M arrive as zeros).
 //   decode   warp (row-block, half of the super-chunk): index vectors prefetched two super-chunks ahead, 64
 //            look-ups in one straight block into 32 registers.  V2: per-lane shared-memory tables (pair tables up
-//            to N = 3, one entry per index above).  V2a: the library replicated once per bank, then
-//            D16 = fp16(fp32(scale * lib[id][q] + mid)) with the group's scale and mid-point.  The outliers stay out of the
+//            to N = 3, one entry per index above).  V2a: D16 = fp16(fp32(scale * lib[id][q] + mid)) with the group's scale and
+//            mid-point -- up to N = 4 the 2^N values of the group once per 64 weights in registers and PRMT look-ups
+//            (xfp_reg_decode.cuh), above the library replicated once per bank (28672 x 8192 N = 4, 16 rows: replicated library, one CTA per
+//            SM 101.9 us, registers, two CTAs 94.5; 64 rows 131.2 -> 123.2; 4096 x 4096 N = 2, 32 rows 18.0 -> 15.9).  The outliers stay out of the
 //            tile (a walk through a lane's list cost 37 - 50 us of 141 at 28672 x 8192 with 0.3 % outliers): the epilogue
 //            adds S x^T to the accumulator instead, see below.
 //   mma      one thread waits for "A stage stored" (eight arrivals) and "x tile landed" (transaction bytes), issues
@@ -39,6 +41,7 @@
 
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
+#include "xfp_reg_decode.cuh"
 
 namespace xfp {
 
@@ -221,6 +224,7 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
                                           uint64_t* bars, uint32_t tmem, const CUtensorMap* tmap,
                                           int grp, int G) {
     using H = Half<N, PART>;
+    constexpr bool kReg = MODE == 1 && N <= 4;
     const int NS = 1 << a.ns_log;
     // byte offset of the lane inside a table entry; N = 4 (V2): the row-block's half of a 256-byte entry as well
     const uint32_t tbase = (uint32_t)lane * 4u + ((MODE == 0 && N == 4) ? (uint32_t)(q & 1) * 128u : 0u);
@@ -279,17 +283,33 @@ __device__ __forceinline__ bool main_loop(const GemmArgs& a, int rb, bool rb_ok,
             // 64 look-ups in one straight block (every load can be in flight at once)
             float g_scale = 0.f, g_mid = 0.f;
             uint32_t vbase = tbase;
+            RegBook<kReg ? N : 2> book;
             if (MODE == 1) {
                 // D16 = fp16(fp32(scale * lib[id][q] + mid)): the product of two fp16 values is exact in fp32, so the
                 // fused multiply-add rounds once, as the format defines it
-                const __half2 sm = *(const __half2*)&gsm_n;
-                g_scale = __low2float(sm); g_mid = __high2float(sm);
-                vbase = tbase | (gid_n << (7 + N));
+                if constexpr (kReg) {
+                    // up to N = 4 the 2^N values that the group can take, in registers
+                    uint32_t e[(1 << N) / 2];
+                    load_entries<N>(e, (const uint16_t*)tab + gid_n * ((1 << N) + 8), [](auto* p) { return *p; });
+                    affine_entries<N>(e, gsm_n);
+                    book = book_of<N>(e);
+                } else {
+                    const __half2 sm = *(const __half2*)&gsm_n;
+                    g_scale = __low2float(sm); g_mid = __high2float(sm);
+                    vbase = tbase | (gid_n << (7 + N));
+                }
                 if (sc + G < sc1) {
                     const size_t mi = meta0 + (size_t)(it + G) * a.GH * 32;
                     gid_n = __ldg(a.b.gid + mi); gsm_n = __ldg(a.b.gsm + mi);
                 }
             }
+            if constexpr (kReg) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 v = reg_decode8_ordered<N>(w, PART * 8 + c, book);
+                    d[4 * c] = v.x; d[4 * c + 1] = v.y; d[4 * c + 2] = v.z; d[4 * c + 3] = v.w;
+                }
+            } else
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 const int p = PART * 32 + i;
@@ -437,9 +457,14 @@ __global__ void __launch_bounds__(threads_of(BIG), BIG ? 1 : 2) gemm_tc_kernel(c
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (MODE == 1) {
-        // the library, every entry replicated once per bank: word (id * E + q) * 32 + lane
         const int n = a.L * E;
-        for (int i = warp; i < n; i += DW + 1) ((uint32_t*)sTab)[i * 32 + lane] = (uint32_t)__ldg(a.b.cb + i);
+        if (N <= 4) {
+            // the library, 16 bytes of padding behind every codebook spread the ids over the banks
+            for (int i = tid; i < n; i += (DW + 1) * 32) ((uint16_t*)sTab)[(i / E) * (E + 8) + i % E] = __ldg(a.b.cb + i);
+        } else {
+            // every entry replicated once per bank: word (id * E + q) * 32 + lane
+            for (int i = warp; i < n; i += DW + 1) ((uint32_t*)sTab)[i * 32 + lane] = (uint32_t)__ldg(a.b.cb + i);
+        }
     } else {
         // codebooks -> one word per (entry, lane); pair tables are built from a copy staged in the x stages
         uint32_t* one = Tab<N>::kPair ? (uint32_t*)sB : (uint32_t*)sTab;
@@ -665,12 +690,12 @@ void schedule_tiles(Plan& p, int tiles, int SC, int sms, int tmax) {
 // `sms`: SMs to plan for (kSizingSMs when sizing the workspace, the device's own count, capped by it, at launch)
 Plan plan_of(const Layout& l, int M, int sms) {
     Plan p;
-    p.tab_bytes = l.mode == 1 ? (size_t)l.L * l.E * 128 : (size_t)4 * (l.bits <= 3 ? l.E * l.E : l.E) * 128;
+    p.tab_bytes = l.mode == 1 ? (l.bits <= 4 ? (size_t)l.L * (l.E + 8) * 2 : (size_t)l.L * l.E * 128) : (size_t)4 * (l.bits <= 3 ? l.E * l.E : l.E) * 128;
     if (l.mode == 0) p.tab_bytes += 8192;                    // room to align the tables to 8 KB in the shared window
     p.tab_bytes = (p.tab_bytes + 1023) & ~size_t(1023);      // the x stages behind the tables are 1024-byte aligned
     p.maxT = kSmallT; p.x_stages = kXStages; p.lone = false;
     const int T = (M + 15) & ~15;                            // rows of x of the one tile along x
-    // a CTA of 16 decode warps, alone on its SM, when the tables leave no room for two CTAs on an SM (V2a from N = 4: a 64 KB
+    // a CTA of 16 decode warps, alone on its SM, when the tables leave no room for two CTAs on an SM (V2a from N = 5: a 128 KB
     // library); two x stages instead of three where that keeps two CTAs there
     p.lone = p.tab_bytes + (size_t)2 * T * 256 > 113 * 1024;
     if (p.lone) p.maxT = kBigT;
