@@ -203,7 +203,7 @@ __global__ void median_finish(const SelState* st, int64_t n, double scale, doubl
 // Median of a short array (the per-channel cosines), one block, one launch: the keys' range is cut into 2048 equal steps
 // and counted, and the members of the one or two steps that hold the middle values are ranked against each other.  Where
 // those steps hold more than a block's worth of keys (many equal values) their range is cut again.
-__global__ void __launch_bounds__(1024) median_small_kernel(const double* __restrict__ v, int n, double* out) {
+__device__ __forceinline__ void median_small(const double* __restrict__ v, int n, double* out) {
     constexpr int kBins = 2048, kCand = 1024;
     __shared__ unsigned int hist[kBins];
     __shared__ unsigned long long cand[kCand], s_lo, s_hi, s_val[2];
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(256) row_count_kernel(const uint8_t* __restric
 }
 
 // One block; every thread owns a run of consecutive rows.
-__global__ void __launch_bounds__(1024) rowptr_scan(const int* __restrict__ cnt, int rows, int32_t* rowptr) {
+__device__ __forceinline__ void rowptr_block(const int* __restrict__ cnt, int rows, int32_t* rowptr) {
     __shared__ int sh[32];
     __shared__ int total;
     const int per = (rows + 1023) / 1024, b0 = threadIdx.x * per, b1 = b0 + per < rows ? b0 + per : rows;
@@ -501,6 +501,15 @@ __global__ void __launch_bounds__(1024) rowptr_scan(const int* __restrict__ cnt,
 #pragma unroll 8
     for (int b = b0; b < b1; ++b) { const int x = cnt[b]; rowptr[b] = run; run += x; }
     if (threadIdx.x == 0) rowptr[rows] = total;
+}
+__global__ void __launch_bounds__(1024) rowptr_scan(const int* __restrict__ cnt, int rows, int32_t* rowptr) { rowptr_block(cnt, rows, rowptr); }
+
+// The median of the cosines, and in a second block the row pointers (`cnt` not null): two serial blocks of about 10 us each at
+// 12288 channels, side by side.
+__global__ void __launch_bounds__(1024) median_small_kernel(const double* __restrict__ v, int n, double* out, const int* __restrict__ cnt,
+                                                            int32_t* rowptr) {
+    if (blockIdx.x == 0) median_small(v, n, out);
+    else rowptr_block(cnt, n, rowptr);
 }
 
 // A warp per channel.  The mask is read 512 weights at a time (four words per lane in flight); the places of the set bytes
@@ -844,7 +853,7 @@ int xfp_quant_median(const double* v, int64_t n, double* median, void* workspace
     if (n < 1) return XFP_ERR_SHAPE;
     if (workspace_bytes < carve(nullptr, 1, 128).bytes) return XFP_ERR_BUFFER_TOO_SMALL;
     if (n <= (1 << 16)) {
-        median_small_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(v, (int)n, median);
+        median_small_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(v, (int)n, median, nullptr, nullptr);
         return cudaGetLastError() == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
     }
     Workspace w = carve(workspace, 1, 128);
@@ -926,7 +935,8 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
         if (launch_lloyd(W, mask, ms, rows, cols, d.bits, p->lloyd_iters, codebook, mode ? nullptr : idx,
                          mode == 0 && fused ? cos : nullptr, c == 0 && fused ? rowcnt : nullptr, workspace, s) != cudaSuccess)
             return XFP_ERR_CUDA;
-        if (c == 0 && fused) rowptr_scan<<<1, 1024, 0, s>>>(rowcnt, rows, out_rowptr);
+        const bool beside = mode == 0 && c == 0 && fused && rows <= (1 << 16);   // the row pointers beside the median (the library's scratch overlaps the counts)
+        if (c == 0 && fused && !beside) rowptr_scan<<<1, 1024, 0, s>>>(rowcnt, rows, out_rowptr);
         if (mode == 1) {
             st = xfp_quant_libfit_library(codebook, rows, d.bits, lib_size, p->lloyd_iters, lib, workspace, need, stream);
             if (st) return st;
@@ -937,8 +947,8 @@ int xfp_quantize(int32_t mode, const float* W, int32_t rows, int32_t cols, const
             st = xfp_quant_cosine(&d, W, mask, idx, codebook, nullptr, nullptr, nullptr, cos, stream);
             if (st) return st;
         }
-        st = xfp_quant_median(cos, rows, med_dev, workspace, need, stream);
-        if (st) return st;
+        if (beside) median_small_kernel<<<2, 1024, 0, s>>>(cos, rows, med_dev, rowcnt, out_rowptr);
+        else if ((st = xfp_quant_median(cos, rows, med_dev, workspace, need, stream))) return st;
         double med = 0.0;
         if (cudaMemcpyAsync(&med, med_dev, sizeof(med), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
