@@ -2,16 +2,23 @@
 //
 // A block of eight warps takes one row-block (32 channels, a lane each) and a range of super-chunks; a warp decodes one
 // super-chunk at a time from index vectors fetched one super-chunk ahead.
-//   V2   the channels' codebooks in shared memory, one word per lane and entry (no bank conflicts); up to N = 3 indexed by
-//        a PAIR of indices.
-//   V2a  a lane decodes the 2^N entries its channel's group can take once -- D16 = fp16(fp32(scale * lib[id] + mid)) --
-//        into a column of a table of its warp, and the weights of the group are look-ups as in V2: 2^N conversions per
-//        group instead of one per weight (N = 2: pairs; at N = 6 64 entries serve 128 weights).
+//   V2   N <= 4: the channel's codebook in registers (xfp_reg_decode.cuh); above, codebooks in shared memory, one word per lane
+//        and entry (no bank conflicts).
+//   V2a  a lane decodes the 2^N entries its channel's group can take once -- D16 = fp16(fp32(scale * lib[id] + mid)) -- into
+//        registers (N <= 4) or a column of a table of its warp, and the weights of the group are look-ups as in V2: 2^N
+//        conversions per group instead of one per weight.
+//   S    up to N = 4 the block notes where every super-chunk's outliers begin in its channels' slabs and a lane adds those of its
+//        channel to the staged row, one correctly rounded fp16 addition each.  What a slab cannot say (channels longer than their
+//        slab, columns that do not ascend), and all of them above N = 4, is added in place behind the block's stores (above, where
+//        tables leave one or two blocks to an SM, the list in front of the decode cost more: 12288 x 4096 V2a N = 6 38.2 -> 46.1 us
+//        with pack, half of both).
 //   out  a tile of shared memory turns a lane's 64 weights into whole 128-byte lines of the channels' rows.
-//   S    when the block has stored its range, its outliers are added in place, one correctly rounded fp16 addition each:
-//        the slots of the transposed slab are dealt to the warps eight at a time, so that the loads of a batch overlap.
+// Tables in shared memory and outliers in place behind the stores -> this, cold: 12289 x 4096 V2a N = 4, 1 % outliers 35.2 -> 32.0 us,
+// 3072 x 4096 V2a N = 2 14.2 -> 10.8, 12288 x 4096 V2 N = 4 33.3 -> 29.1.  100 MB of stores and 29 MB of loads are 20 us at the copy
+// rate; what is left is the chain of a block's first loads and a single round of blocks.
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
+#include "xfp_reg_decode.cuh"
 
 namespace xfp {
 
@@ -21,6 +28,8 @@ constexpr int kDqWarps = 8;
 constexpr int kDqRange = 32;        // super-chunks of a block at most: the tail of outliers stays short
 constexpr int kTileRow = 144;       // bytes of a row of 64 weights in the staging tile: eight lanes' rows in distinct banks
 constexpr int kLibEntries = 8192;   // library entries (L * 2^N) that are staged in shared memory
+constexpr int kDqSlots = 64;        // outlier slots of a row-block that are staged in shared memory; later ones are read from the blob
+constexpr int kDqStarts = (kDqRange + 1) * 32 * 2, kDqEntries = kDqSlots * 32 * 4;   // bytes of the starts and of the staged slots
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
@@ -30,17 +39,14 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
 }
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory"); }
 
-// The decode tables: PAIR: entry t = (first index | second index << N) holds both fp16 values; else entry q holds one.
-// N = 4 entries lie 256 bytes apart (two tables interleaved), so that an index isolated in its own byte becomes the second
-// byte of the address with one PRMT.
+// The decode tables of N = 5, 6: entry q holds one value per lane.
 template <int N, int MODE>
 struct DqTab {
     static constexpr int E = 1 << N;
-    static constexpr bool kPair = MODE == 0 ? N <= 3 : N == 2;
-    static constexpr int kEntries = kPair ? E * E : E;
-    static constexpr int kBytes = N == 4 ? 4096 : kEntries * 128;            // of one table (N = 4: of an interleaved pair)
-    static constexpr int kTables = MODE == 0 ? 1 : (N == 4 ? kDqWarps / 2 : kDqWarps);
-    static constexpr int kStride = N == 4 ? 256 : 128;                      // bytes between entries
+    static constexpr bool kReg = N <= 4;
+    static constexpr int kBytes = kReg ? 0 : E * 128;                        // of one table
+    static constexpr int kTables = kReg ? 0 : MODE == 0 ? 1 : kDqWarps;
+    static constexpr size_t kAlign = kReg ? 16 : kBytes;                     // aligned to its size: an entry's offset is merged, not added
 };
 
 struct DqArgs {
@@ -51,7 +57,7 @@ struct DqArgs {
 };
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) {
+__global__ void __launch_bounds__(kDqWarps * 32, N <= 4 ? 3 : 0) dequant_kernel(const DqArgs a) {
     using T = DqTab<N, MODE>;
     constexpr int E = T::E;
     extern __shared__ unsigned char dq_smem[];
@@ -59,32 +65,26 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
     const int parts = (a.SC + a.range - 1) / a.range;
     const int rb = (int)blockIdx.x / parts, part = (int)blockIdx.x % parts;
     const int s0 = part * a.range, s1 = min(a.SC, s0 + a.range);
-    // tables aligned to their size in the shared window (at least 1 KB), so that an entry's offset is merged, not added
-    constexpr uint32_t kAlign = T::kBytes < 1024 ? 1024 : T::kBytes;
+    constexpr uint32_t kAlign = (uint32_t)T::kAlign;
     const uint32_t raw = smem_addr(dq_smem), tab0 = (raw + kAlign - 1) & ~(kAlign - 1);
     unsigned char* base = dq_smem + (tab0 - raw);
     unsigned char* tiles = base + T::kTables * kAlign;                        // [warps][32 * kTileRow]
-    uint16_t* slib = (uint16_t*)(tiles + kDqWarps * 32 * kTileRow);   // [L][lib_stride]
+    uint32_t* ents = (uint32_t*)(tiles + kDqWarps * 32 * kTileRow);          // [kDqSlots][32]
+    uint16_t* starts = (uint16_t*)((unsigned char*)ents + kDqEntries);       // [range + 1][32]
+    uint16_t* slib = (uint16_t*)(T::kReg ? (unsigned char*)starts + kDqStarts : (unsigned char*)ents);     // [L][lib_stride]
     constexpr int kLibStride = E + 8;                                        // 16 bytes of padding spread the ids over the banks
     const bool staged = MODE == 1 && a.L * E <= kLibEntries;
-    if (MODE == 0) {
-        const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * E;    // padding rows exist in the blob
-        for (int t = warp; t < T::kEntries; t += kDqWarps) {
-            uint32_t v;
-            if (T::kPair) v = (uint32_t)__ldg(cb + (t & (E - 1))) | ((uint32_t)__ldg(cb + (t >> N)) << 16);
-            else v = (uint32_t)__ldg(cb + t);
-            sts_u32(tab0 + (uint32_t)(t * T::kStride + lane * 4), v);
-        }
-        __syncthreads();
+    RegBook<T::kReg ? N : 2> book;
+    const uint16_t* cb = a.b.cb + (size_t)(rb * kRowsPerBlock + lane) * E;   // V2: padding rows exist in the blob
+    if constexpr (MODE == 0 && T::kReg) {
+        book = make_book<N>(cb);
+    } else if constexpr (MODE == 0) {
+        for (int t = warp; t < E; t += kDqWarps) sts_u32(tab0 + (uint32_t)(t * 128 + lane * 4), (uint32_t)__ldg(cb + t));
     } else if (staged) {
         for (int i = tid; i < a.L * E; i += kDqWarps * 32) slib[(i / E) * kLibStride + i % E] = __ldg(a.b.cb + i);
-        __syncthreads();
     }
     // this lane's column of its table
-    const uint32_t tab = MODE == 0 ? tab0 + (uint32_t)lane * 4u
-                       : N == 4    ? tab0 + (uint32_t)(warp >> 1) * kAlign + (uint32_t)(warp & 1) * 128u + (uint32_t)lane * 4u
-                                   : tab0 + (uint32_t)warp * kAlign + (uint32_t)lane * 4u;
-    const uint32_t nib = ((tab >> 12) & 0xfu) * 0x10101010u;
+    const uint32_t tab = tab0 + (MODE == 0 ? 0u : (uint32_t)warp * kAlign) + (uint32_t)lane * 4u;
     const int row = rb * kRowsPerBlock + lane;
     unsigned char* tile = tiles + warp * 32 * kTileRow;
 
@@ -101,7 +101,41 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
         }
     };
     if (s0 + warp < s1) fetch(s0 + warp);
+    // where the outliers of every super-chunk begin: slot j is the first of the super-chunks behind that of slot j - 1
+    const int nsc = s1 - s0;
+    const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
+    const int len = a.ell_slots && row < a.rows ? (int)__ldg(slab) : 0, in_slab = min(len, a.ell_slots);
+    bool in_place = !T::kReg && a.ell_slots != 0;
+    if (T::kReg && a.ell_slots) {
+        bool descends = false;
+        auto rel = [&](uint32_t e) { return max(-1, min(nsc, (int)((e & 0xffffu) >> 7) - s0)); };
+        // a run of slots to every warp, slot `in_slab` closes a channel's list; the loads do not wait for the channels' lengths
+        const int chunk = (a.ell_slots + kDqWarps) / kDqWarps, j1 = min((warp + 1) * chunk, a.ell_slots + 1);
+        for (int jb = warp * chunk; jb < j1; jb += 8) {
+            uint32_t v[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = jb + i > 0 && jb + i <= a.ell_slots ? __ldg(slab + (size_t)(jb + i) * 32) : 0u;   // slot jb + i - 1
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                const int j = jb + i - 1;
+                if (j >= j1 || j > in_slab) continue;
+                const bool have = j < in_slab;
+                if (j < kDqSlots && have) ents[j * 32 + lane] = v[i];
+                descends |= j > 0 && have && (v[i] & 0xffffu) <= (v[i - 1] & 0xffffu);
+                const int b0 = j > 0 ? rel(v[i - 1]) : -1, b1 = have ? rel(v[i]) : nsc;
+                for (int t = b0 + 1; t <= b1; ++t) starts[t * 32 + lane] = (uint16_t)j;
+            }
+        }
+        in_place = __syncthreads_or(descends) != 0;
+    } else {
+        __syncthreads();
+    }
+    const bool in_tile = T::kReg && a.ell_slots != 0 && !in_place;
     for (int sc = s0 + warp; sc < s1; sc += kDqWarps) {
+        int j = 0, jend = 0;
+        if (in_tile) { j = starts[(sc - s0) * 32 + lane]; jend = starts[(sc - s0 + 1) * 32 + lane]; }
+        auto entry = [&](int i) { return i < kDqSlots ? ents[i * 32 + lane] : __ldg(slab + (size_t)(1 + i) * 32); };
+        uint32_t e = j < jend ? entry(j) : 0u;
         uint32_t w[4 * N + 1];
 #pragma unroll
         for (int v = 0; v < N; ++v) { w[4 * v] = nx[v].x; w[4 * v + 1] = nx[v].y; w[4 * v + 2] = nx[v].z; w[4 * v + 3] = nx[v].w; }
@@ -111,50 +145,50 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (MODE == 1 && (h == 0 || a.GH == 2)) {
-                const float scale = h2f((uint16_t)(sm[h] & 0xffffu)), mid = h2f((uint16_t)(sm[h] >> 16));
-                auto decoded = [&](uint16_t l) { return (uint32_t)f2h(__fmaf_rn(scale, h2f(l), mid)); };
-                if (N == 2) {
-                    uint32_t d[4];
-                    uint2 l4;
-                    if (staged) l4 = *(const uint2*)(slib + id[h] * kLibStride);
-                    else l4 = __ldg((const uint2*)(a.b.cb + (size_t)id[h] * E));
-                    d[0] = decoded((uint16_t)l4.x); d[1] = decoded((uint16_t)(l4.x >> 16));
-                    d[2] = decoded((uint16_t)l4.y); d[3] = decoded((uint16_t)(l4.y >> 16));
-#pragma unroll
-                    for (int t = 0; t < 16; ++t) sts_u32(tab + t * 128, join16(d[t & 3], d[t >> 2]));
+                if constexpr (T::kReg) {
+                    uint32_t d[E / 2];
+                    if (staged) load_entries<N>(d, slib + id[h] * kLibStride, [](auto* p) { return *p; });
+                    else load_entries<N>(d, a.b.cb + (size_t)id[h] * E, [](auto* p) { return __ldg(p); });
+                    affine_entries<N>(d, sm[h]);
+                    book = book_of<N>(d);
                 } else {
+                    const float scale = h2f((uint16_t)(sm[h] & 0xffffu)), mid = h2f((uint16_t)(sm[h] >> 16));
+                    auto decoded = [&](uint32_t v) { return (uint32_t)f2h(__fmaf_rn(scale, h2f((uint16_t)v), mid)); };
 #pragma unroll
-                    for (int e = 0; e < E; e += 8) {
+                    for (int q = 0; q < E; q += 8) {
                         uint4 l8;
-                        if (staged) l8 = *(const uint4*)(slib + id[h] * kLibStride + e);
-                        else l8 = __ldg((const uint4*)(a.b.cb + (size_t)id[h] * E + e));
+                        if (staged) l8 = *(const uint4*)(slib + id[h] * kLibStride + q);
+                        else l8 = __ldg((const uint4*)(a.b.cb + (size_t)id[h] * E + q));
                         const uint32_t lw[4] = {l8.x, l8.y, l8.z, l8.w};
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            sts_u32(tab + (e + 2 * i) * T::kStride, decoded((uint16_t)lw[i]));
-                            sts_u32(tab + (e + 2 * i + 1) * T::kStride, decoded((uint16_t)(lw[i] >> 16)));
+                            sts_u32(tab + (q + 2 * i) * 128, decoded(lw[i] & 0xffffu));
+                            sts_u32(tab + (q + 2 * i + 1) * 128, decoded(lw[i] >> 16));
                         }
                     }
                 }
             }
 #pragma unroll
             for (int c = 0; c < 8; ++c) {                 // 8 weights = 16 bytes
-                uint32_t d[4];
+                uint4 v;
+                if constexpr (T::kReg) {
+                    v = reg_decode8_ordered<N>(w, h * 8 + c, book);
+                } else {
+                    uint32_t d[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int p = h * 32 + c * 4 + i;
-                    if (T::kPair) {
-                        d[i] = lds_u32(pair_addr<N, 1>(w, p, tab));
-                    } else if (N == 4) {
-                        const uint32_t wlo = (w[p >> 2] & 0x0f0f0f0fu) | nib, whi = ((w[p >> 2] >> 4) & 0x0f0f0f0fu) | nib;
-                        const uint32_t sel = 0x7604u | ((uint32_t)(p & 3) << 4);   // [tab.b3, tab.b2, index byte, tab.b0]
-                        d[i] = join16(lds_u32(__byte_perm(wlo, tab, sel)), lds_u32(__byte_perm(whi, tab, sel)));
-                    } else {
+                    for (int i = 0; i < 4; ++i) {
+                        const int p = h * 32 + c * 4 + i;
                         d[i] = join16(lds_u32(single_addr<N, 1>(w, 2 * p, tab)), lds_u32(single_addr<N, 1>(w, 2 * p + 1, tab)));
                     }
+                    v = make_uint4(d[0], d[1], d[2], d[3]);
                 }
-                const uint4 v = make_uint4(d[0], d[1], d[2], d[3]);
                 *(uint4*)(tile + lane * kTileRow + c * 16) = v;
+            }
+            const uint32_t k0 = (uint32_t)sc * kSuper + h * 64;
+            while (T::kReg && j < jend && (e & 0xffffu) < k0 + 64) {
+                __half* t = (__half*)(tile + lane * kTileRow) + ((e & 0xffffu) - k0);
+                *t = __hadd(*t, __ushort_as_half((uint16_t)(e >> 16)));
+                if (++j < jend) e = entry(j);
             }
             __syncwarp();
 #pragma unroll
@@ -167,11 +201,9 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
             __syncwarp();
         }
     }
-    // ---- W^ += S on the values this block has just stored ----
-    if (a.ell_slots) {
-        __syncthreads();
-        const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
-        const int len = row < a.rows ? (int)__ldg(slab) : 0, in_slab = min(len, a.ell_slots);
+    // ---- what is left of S, on the values this block has just stored ----
+    const bool spills = a.ell_slots && len >= a.ell_slots && row < a.rows;
+    if (__syncthreads_or(in_place || spills)) {
         const uint32_t k0 = (uint32_t)s0 * kSuper, k1 = (uint32_t)s1 * kSuper;
         uint16_t* out = a.out + (size_t)row * a.cols;
         constexpr int kBatch = 8;
@@ -191,9 +223,11 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
             for (int i = 0; i < kBatch; ++i)
                 if (ok[i]) out[e[i] & 0xffffu] = __half_as_ushort(__hadd(__ushort_as_half(old[i]), __ushort_as_half((uint16_t)(e[i] >> 16))));
         };
-        const int most = __reduce_max_sync(0xffffffffu, in_slab);
-        for (int j = warp; j < most; j += kBatch * kDqWarps) batch(slab + 32, 32, j, in_slab);
-        if (len >= a.ell_slots && row < a.rows) {        // the channel overflows its slab: the rest is in the CSR arrays
+        if (in_place) {
+            const int most = __reduce_max_sync(0xffffffffu, in_slab);
+            for (int j = warp; j < most; j += kBatch * kDqWarps) batch(slab + 32, 32, j, in_slab);
+        }
+        if (spills) {                                   // the rest of the channel is in the CSR arrays
             const int p0 = __ldg(a.b.rowptr + row), n = __ldg(a.b.rowptr + row + 1) - p0;
             for (int j = a.ell_slots + warp; j < n; j += kBatch * kDqWarps) batch(a.b.oent + p0, 1, j, n);
         }
@@ -203,13 +237,12 @@ __global__ void __launch_bounds__(kDqWarps * 32) dequant_kernel(const DqArgs a) 
 template <int N, int MODE>
 cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s) {
     using T = DqTab<N, MODE>;
-    constexpr size_t kAlign = T::kBytes < 1024 ? 1024 : T::kBytes;
     DqArgs a = {};
     a.b = blob_at(packed, offsets_of(l));
     a.out = W;
     a.rows = l.rows; a.cols = l.cols; a.RB = l.RB; a.SC = l.SC; a.GH = l.GH; a.L = l.L; a.ell_slots = l.ell_slots;
     const size_t lib = MODE == 1 && a.L * T::E <= kLibEntries ? (size_t)a.L * (T::E + 8) * 2 : 0;
-    const size_t smem = kAlign + T::kTables * kAlign + kDqWarps * 32 * kTileRow + lib;
+    const size_t smem = (1 + T::kTables) * T::kAlign + kDqWarps * 32 * kTileRow + (T::kReg ? kDqEntries + kDqStarts : 0) + lib;
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {

@@ -254,6 +254,29 @@ def test_outlier_structures(placement, rate):
         _check_dequant(q, pm)
 
 
+@pytest.mark.parametrize("mode,bits,rows,cols,rate,placement", [
+    (0, 4, 33, 16384, 0.02, "uniform"), (1, 4, 33, 16384, 0.02, "uniform"), (1, 3, 40, 8192, 0.02, "clustered"),
+    (1, 2, 64, 640, 0.05, "one_row"), (0, 2, 70, 4224, 0.01, "uniform"), (0, 3, 1, 128, 0.3, "uniform"), (0, 6, 50, 4224, 0.02, "uniform"),
+    (1, 5, 50, 4224, 0.02, "uniform")])
+def test_dequant_adds_the_outliers_of_every_super_chunk(mode, bits, rows, cols, rate, placement):
+    """Channels of one range of super-chunks and of several, more slots than are staged, slabs that overflow, one super-chunk."""
+    q = synth.random_quantized(mode, rows, cols, bits, rate, seed=8100 + 10 * mode + bits, placement=placement)
+    _check_dequant(q, xfp.pack_tensors(q))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_dequant_of_entries_out_of_order(mode):
+    """Columns that do not ascend are reported and still added, each once."""
+    q = synth.random_quantized(mode, 70, 1024, 4, 0.02, seed=8200 + mode)
+    for r in range(0, 70, 3):
+        a, b = q.rowptr[r], q.rowptr[r + 1]
+        q.ocol[a:b] = q.ocol[a:b][::-1].copy()
+        q.oval[a:b] = q.oval[a:b][::-1].copy()
+    pm = xfp.pack_tensors(q)
+    got = pm.dequant().view(torch.int16).cpu().numpy().view(np.uint16)
+    assert np.array_equal(got, xo.dequant(to_oracle(q))) and int(pm.err_word.item()) == 16
+
+
 def test_adversarial_activations():
     q = synth.random_quantized(0, 64, 1024, 4, 0.01, seed=91)
     qa = synth.random_quantized(1, 64, 1024, 3, 0.01, seed=92)
