@@ -70,20 +70,40 @@ __device__ __forceinline__ void pack_idx_block(const PackArgs& a, unsigned vblk,
 #pragma unroll
     for (int i = 0; i < 4 * N + 1; ++i) w[i] = 0u;
     bool bad = false;
+    if constexpr (N == 5) {         // index by index: 28672 x 8192 78 us against 87
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint4 t = *(const uint4*)(tile + lane * kRowB + i * 16);
-        const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
+        for (int i = 0; i < 8; ++i) {
+            const uint4 t = *(const uint4*)(tile + lane * kRowB + i * 16);
+            const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-        for (int b = 0; b < 16; ++b) {
-            uint32_t q = (tw[b >> 2] >> ((b & 3) * 8)) & 0xffu;
-            bad |= (q >= E);
-            q &= E - 1u;
-            const int j = i * 16 + b;
-            const int bit = j * N, wi = bit >> 5, off = bit & 31;
-            w[wi] |= q << off;
-            if (off + N > 32) w[wi + 1] |= q >> (32 - off);
+            for (int b = 0; b < 16; ++b) {
+                uint32_t q = (tw[b >> 2] >> ((b & 3) * 8)) & 0xffu;
+                bad |= (q >= E);
+                q &= E - 1u;
+                const int j = i * 16 + b;
+                const int bit = j * N, wi = bit >> 5, off = bit & 31;
+                w[wi] |= q << off;
+                if (off + N > 32) w[wi + 1] |= q >> (32 - off);
+            }
         }
+    } else {                        // four indices of a byte each to 4 N adjacent bits: 28672 x 8192 V2 N = 4 80 -> 70 us, N = 6 97 both ways
+        uint32_t over = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint4 t = *(const uint4*)(tile + lane * kRowB + i * 16);
+            const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                over |= tw[b];
+                uint32_t q = tw[b] & ((E - 1u) * 0x01010101u);
+                q = (q & 0x00ff00ffu) | ((q & 0xff00ff00u) >> (8 - N));
+                q = (q & 0x0000ffffu) | ((q & 0xffff0000u) >> (16 - 2 * N));
+                const int bit = (i * 4 + b) * 4 * N, wi = bit >> 5, off = bit & 31;
+                w[wi] |= q << off;
+                if (off + 4 * N > 32) w[wi + 1] |= q >> (32 - off);
+            }
+        }
+        bad = (over & ~((E - 1u) * 0x01010101u)) != 0;
     }
     if (bad && a.err_word) atomicOr(a.err_word, 1);
     uint4* dst = (uint4*)(a.base + a.l.off_idx) + ((size_t)unit * N) * 32 + lane;
