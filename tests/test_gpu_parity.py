@@ -15,7 +15,7 @@ from conftest import from_oracle, to_oracle
 from plans import gemv_kernel
 from oracle import xfp_oracle as xo
 import paper_2605_14844_b200 as xfp
-from paper_2605_14844_b200 import synth
+from paper_2605_14844_b200 import binding, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -275,6 +275,22 @@ def test_dequant_of_entries_out_of_order(mode):
     pm = xfp.pack_tensors(q)
     got = pm.dequant().view(torch.int16).cpu().numpy().view(np.uint16)
     assert np.array_equal(got, xo.dequant(to_oracle(q))) and int(pm.err_word.item()) == 16
+
+
+@pytest.mark.parametrize("least", [0, 1 << 40])
+@pytest.mark.parametrize("spare", [0, 1, 40])
+def test_pack_tensors_takes_the_count_from_the_row_pointers(spare, least, monkeypatch):
+    """Tensors on the device whose entry arrays hold `spare` entries behind the last row pointer, packed before and after the count
+    has been read back."""
+    monkeypatch.setattr(binding, "_SPECULATE", least)
+    q = synth.random_quantized(0, 70, 640, 4, 0.02, seed=8300)
+    want = xfp.pack_tensors(q)
+    dev = {k: torch.from_numpy(v.view(np.int16) if v.dtype == np.uint16 else v).cuda() for k, v in q.__dict__.items() if isinstance(v, np.ndarray)}
+    dev["ocol"] = torch.cat([dev["ocol"], torch.full((spare,), 3, dtype=dev["ocol"].dtype, device="cuda")])
+    dev["oval"] = torch.cat([dev["oval"], torch.ones(spare, dtype=dev["oval"].dtype, device="cuda")])
+    pm = xfp.pack_tensors(synth.QuantTensors(**{**q.__dict__, **dev}))
+    assert pm.desc.nnz == want.desc.nnz == q.nnz and torch.equal(pm.dequant(), want.dequant())
+    assert int(pm.err_word.item()) == 0 and int(pm.workspace.abs().sum().item()) == 0
 
 
 def test_adversarial_activations():
