@@ -3,6 +3,8 @@
 // evaluation, bit for bit.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "xfp_quant_common.cuh"
 #include "xfp_quant_internal.h"
 #include "xfp_internal.h"
@@ -20,6 +22,211 @@ constexpr int kLibThreads = 512;
 constexpr int kLibTile = 4096;      // channels whose members are compacted at a time
 constexpr int kLibVals = 2048;      // member values staged at a time
 constexpr size_t kLibSmemU = 160 * 1024;   // normalised codebooks of this size stay in every block's shared memory
+
+// u_j = (c_j - m) / s, m and s the middle and half-width of the codebook's range; returns |u|^2
+__device__ __forceinline__ double normalise_channel(const uint16_t* __restrict__ cb, int E, double* u) {
+    double lo = INFINITY, hi = -INFINITY;
+    for (int j = 0; j < E; ++j) {
+        const double c = h2d(cb[j]);
+        if (c < lo) lo = c;
+        if (c > hi) hi = c;
+    }
+    const double m = __dmul_rn(0.5, __dadd_rn(hi, lo));
+    double s = __dmul_rn(0.5, __dsub_rn(hi, lo));
+    if (s == 0.0) s = 1.0;
+    double acc = 0.0;
+    for (int j = 0; j < E; ++j) {
+        const double v = __ddiv_rn(__dsub_rn(h2d(cb[j]), m), s);
+        u[j] = v;
+        acc = __dadd_rn(acc, __dmul_rn(v, v));
+    }
+    return acc == acc ? acc : INFINITY;      // a codebook with an infinity has no norm: last, so that `order` is a permutation
+}
+
+__global__ void __launch_bounds__(128) libfit_normalise_kernel(const uint16_t* __restrict__ cb, int rows, int E, double* u, double* nn) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i < rows) nn[i] = normalise_channel(cb + (int64_t)i * E, E, u + (int64_t)i * E);
+}
+
+// order[r] = the channel of rank r by (nn, channel): rank by counting, a warp per channel
+__global__ void __launch_bounds__(256) libfit_rank_kernel(const double* __restrict__ nn, int rows, int* order) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= rows) return;
+    const double mine = __ldg(nn + i);
+    int r = 0;
+#pragma unroll 8
+    for (int j = lane; j < rows; j += 32) {
+        const double o = __ldg(nn + j);
+        r += (o < mine) || (o == mine && j < i);
+    }
+    r = __reduce_add_sync(0xffffffffu, r);
+    if (lane == 0) order[r] = i;
+}
+
+// seed l of the library: L evenly spaced channels of that order
+__device__ __forceinline__ int seed_rank(int l, int rows, int L) {
+    long long t = rows >= L ? (long long)floor(__ddiv_rn(__dmul_rn(__dadd_rn((double)l, 0.5), (double)rows), (double)L))
+                            : (long long)(l % rows);
+    return (int)(t >= rows ? rows - 1 : t);
+}
+
+// the centroid's entries c[0..E) in ascending order, fp16 (thread `tid` < E; entries that are no numbers behind the others, so
+// that every place of the library is written)
+__device__ __forceinline__ void store_ascending(const double* c, int E, int tid, uint16_t* lib) {
+    const double x = c[tid];
+    int r = 0;
+    for (int j = 0; j < E; ++j) {
+        const double v = c[j];
+        const bool before = v < x || (x != x && v == v), after = x < v || (v != v && x == x);
+        r += before || (!before && !after && j < tid);
+    }
+    lib[r] = d2h(x);
+}
+
+// The rounds of the k-means where they fit one cluster of 16 SMs: the channels are dealt to the blocks in runs.
+//   assignment  two threads per channel, its E values in registers, centroids in order with a strict "less than"
+//   update      half a block per centroid: every block has all assignments (a byte per channel, written to each of them),
+//               compacts the members in channel order, fetches their values from the blocks that hold them, and thread j adds
+//               entries j one by one: the order of the serial evaluation
+// A round costs two cluster barriers instead of two grid barriers with their trips through L2.  Bound by the serial sums (about
+// rows / L dependent fp64 additions) and the barriers.  3072 channels, N = 2, L = 32, 20 rounds:
+// 186 -> 155 us with the two kernels in front.
+constexpr int kClBlocks = 16;
+constexpr int kClVals = 2048;                       // member values staged at a time by half a block
+constexpr size_t kClSmem = 200 * 1024;
+constexpr long long kClTerms = 2000000;
+__host__ __device__ inline int cl_per(int rows) { return ((rows + kClBlocks - 1) / kClBlocks + 3) & ~3; }
+inline size_t cl_smem(int rows, int E, int L) {
+    const size_t asg = ((size_t)cl_per(rows) * kClBlocks + 15) & ~size_t(15);
+    return (size_t)cl_per(rows) * E * 8 + (size_t)L * E * 8 + 2 * kClVals * 8 + asg + 2 * 2 * asg;
+}
+
+template <int E>
+__global__ void __launch_bounds__(kLibThreads) libfit_cluster_kernel(const double* __restrict__ u, const int* __restrict__ order, int rows,
+                                                                     int L, int iters, uint16_t* lib) {
+    extern __shared__ __align__(16) double cl[];
+    __shared__ int changed;             // the last round, counted from one, in which a centroid of the cluster moved
+    __shared__ int wsum[2][8];
+    constexpr int HT = kLibThreads / 2;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), per = cl_per(rows);
+    const int tid = threadIdx.x, lane = tid & 31, half = tid / HT, ht = tid % HT, hw = ht >> 5;
+    double* su = cl;                                    // [E][per] values of this block's channels
+    double* cen = su + (size_t)per * E;                 // [L][E]
+    double* vals = cen + (size_t)L * E + half * kClVals;
+    uint8_t* asg = (uint8_t*)(cen + (size_t)L * E + 2 * kClVals);
+    const int asg_bytes = (per * kClBlocks + 15) & ~15;
+    uint16_t* member = (uint16_t*)(asg + asg_bytes) + (size_t)half * asg_bytes;
+    const int c0 = rank * per, mine = max(0, min(rows - c0, per));
+    for (int i = tid; i < mine * E; i += kLibThreads) su[(i % E) * per + i / E] = __ldg(u + (size_t)c0 * E + i);
+    for (int i = tid; i < L * E; i += kLibThreads) cen[i] = __ldg(u + (size_t)__ldg(order + seed_rank(i / E, rows, L)) * E + i % E);
+    if (tid == 0) changed = 0;
+    cluster.sync();
+    auto half_sync = [&]() { asm volatile("bar.sync %0, %1;" :: "r"(1 + half), "r"(HT) : "memory"); };
+    for (int it = 1; it <= iters; ++it) {
+        for (int i0 = 0; i0 < per; i0 += HT) {       // two neighbouring threads to a channel, half of the centroids each
+            const int i = i0 + (tid >> 1), sub = tid & 1, h0 = (L + 1) >> 1, l1 = sub ? L : h0;
+            double x[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) x[j] = i < mine ? su[j * per + i] : 0.0;
+            int best = sub ? h0 : 0;
+            double bd = INFINITY;
+#pragma unroll 4
+            for (int l = best; l < l1; ++l) {
+                double d = 0.0;
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const double t = __dsub_rn(x[j], cen[l * E + j]);
+                    d = __dadd_rn(d, __dmul_rn(t, t));
+                }
+                if (d < bd) { bd = d; best = l; }
+            }
+            const double od = __shfl_xor_sync(0xffffffffu, bd, 1);
+            const int ob = __shfl_xor_sync(0xffffffffu, best, 1);
+            // the upper half's centroid only when strictly nearer
+            if (sub ? !(bd < od) : od < bd) best = ob;
+            // four channels to a word, a copy to every block
+            uint32_t w = (uint32_t)best << (8 * ((lane >> 1) & 3));
+            w |= __shfl_xor_sync(0xffffffffu, w, 2);
+            w |= __shfl_xor_sync(0xffffffffu, w, 4);
+            if (i < per)
+#pragma unroll
+                for (int r = 0; r < kClBlocks / 8; ++r)
+                    *(uint32_t*)(cluster.map_shared_rank(asg, (lane & 7) + 8 * r) + c0 + (i & ~3)) = w;
+        }
+        cluster.sync();
+        for (int l0 = rank; l0 < L; l0 += 2 * kClBlocks) {
+            const int l = l0 + half * kClBlocks;
+            // members of centroid l, in channel order: a run of words to every thread
+            const int words = (rows + 3) / 4, wpt = (words + HT - 1) / HT;
+            const uint32_t want = (uint32_t)(l & 0xff) * 0x01010101u;
+            auto hits = [&](int q) -> uint32_t {
+                if (l >= L || q >= words) return 0u;
+                uint32_t h = __vcmpeq4(*(const uint32_t*)(asg + 4 * q), want) & 0x01010101u;
+                const int over = 4 * q + 4 - rows;                      // channels of this word beyond the last
+                return over > 0 ? h & (0xffffffffu >> (8 * over)) : h;
+            };
+            int c = 0;
+            for (int k = 0; k < wpt; ++k) c += __popc(hits(ht * wpt + k));
+            int inc = c;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += t;
+            }
+            if (lane == 31) wsum[half][hw] = inc;
+            half_sync();
+            int at = inc - c, n = 0;
+#pragma unroll
+            for (int k = 0; k < HT / 32; ++k) { if (k < hw) at += wsum[half][k]; n += wsum[half][k]; }
+            for (int k = 0; k < wpt; ++k) {
+                const int q = ht * wpt + k;
+                for (uint32_t h = hits(q); h; h &= h - 1) member[at++] = (uint16_t)(4 * q + (__ffs(h) >> 3));
+            }
+            half_sync();
+            double acc = 0.0;
+            for (int m0 = 0; m0 < n; m0 += kClVals / E) {
+                const int cnt = min(n - m0, kClVals / E);
+                for (int t = ht; t < cnt * E; t += HT) {
+                    const int i = member[m0 + t / E], owner = i / per;
+                    vals[t] = cluster.map_shared_rank(su, owner)[(t % E) * per + (i - owner * per)];
+                }
+                half_sync();
+                if (ht < E) {
+                    // the next eight values travel under the chain of eight additions
+                    double v[8], w[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] = k < cnt ? vals[k * E + ht] : 0.0;
+                    int m = 0;
+                    for (; m + 8 <= cnt; m += 8) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) w[k] = m + 8 + k < cnt ? vals[(m + 8 + k) * E + ht] : 0.0;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) { acc = __dadd_rn(acc, v[k]); v[k] = w[k]; }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (m + k < cnt) acc = __dadd_rn(acc, v[k]);
+                }
+                half_sync();
+            }
+            if (ht < E && n > 0) {
+                const double m = __ddiv_rn(acc, (double)n);
+                if (m != cen[l * E + ht]) {
+                    for (int r = 0; r < kClBlocks; ++r) {
+                        cluster.map_shared_rank(cen, r)[l * E + ht] = m;
+                        *cluster.map_shared_rank(&changed, r) = it;
+                    }
+                }
+            }
+            half_sync();            // (the counts of the next centroid overwrite this one's)
+        }
+        cluster.sync();
+        if (changed != it) break;
+    }
+    for (int l = rank; l < L; l += kClBlocks)
+        if (tid < E) store_ascending(cen + l * E, E, tid, lib + l * E);
+}
 
 // The whole k-means in one cooperative launch: normalise, order by norm, seed, `iters` rounds of assignment and update,
 // store.  As separate launches (three per round) the rounds were bound by launches and by the update's chain of dependent
@@ -488,8 +695,54 @@ cudaError_t launch_libfit_assign(const float* W, const uint8_t* mask, const doub
     return launch_groups<256>(W, mask, ms, rows, cols, bits, L, lib, idx, gid, gscale, gmid, cosv, s);
 }
 
+namespace {
+
+template <int E>
+cudaError_t launch_cluster(const uint16_t* codebook, int rows, int L, int iters, double* u, double* nn, int* order, uint16_t* lib,
+                           cudaStream_t s, bool* taken) {
+    static std::atomic<int> fits[256] = {};       // per device: 1 a cluster of this size can be resident, 2 it can not
+    const int dev = xfp::DeviceOnce::current();
+    const size_t smem = cl_smem(rows, E, L);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClBlocks);
+    cfg.blockDim = dim3(kLibThreads);
+    cfg.dynamicSmemBytes = kClSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClBlocks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int f = fits[dev].load(std::memory_order_acquire);
+    if (f == 0) {
+        cudaError_t e = cudaFuncSetAttribute(libfit_cluster_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(libfit_cluster_kernel<E>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        int n = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, libfit_cluster_kernel<E>, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();
+        f = e == cudaSuccess && n > 0 ? 1 : 2;
+        fits[dev].store(f, std::memory_order_release);
+    }
+    *taken = f == 1;
+    if (f != 1) return cudaSuccess;
+    libfit_normalise_kernel<<<(rows + 127) / 128, 128, 0, s>>>(codebook, rows, E, u, nn);
+    libfit_rank_kernel<<<(rows + 7) / 8, 256, 0, s>>>(nn, rows, order);
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, libfit_cluster_kernel<E>, (const double*)u, (const int*)order, rows, L, iters, lib);
+}
+
+}  // namespace
+
 cudaError_t launch_libfit_library(const uint16_t* codebook, int rows, int E, int L, int iters, double* u, double* nn,
                                   int* order, int* asg, double* cen, int* flags, uint16_t* lib, cudaStream_t s) {
+    // one cluster at N = 2 while its assignment step (rows L E terms on 16 SMs) costs less than the grid barriers it saves; library
+    // of 32 after 20 rounds, one cluster against all SMs: 3072 channels N = 2 155 against 186 us, 12288 N = 2 493 against 536, 1472
+    // N = 2 122 against 140; 3072 N = 3 230 against 237, N = 4 369 against 290, 6144 N = 3 443 against 396
+    bool taken = false;
+    if (E == 4 && (long long)rows * L * E <= kClTerms && rows <= 65535 && cl_smem(rows, E, L) <= kClSmem) {
+        const cudaError_t e = launch_cluster<4>(codebook, rows, L, iters, u, nn, order, lib, s, &taken);
+        if (taken || e != cudaSuccess) return e;
+    }
     // a warp per channel, within one block per SM (the blocks wait for one another)
     const int want = (rows + kLibThreads / 32 - 1) / (kLibThreads / 32), sms = xfp::sm_count();
     int blocks = want > L ? want : L;

@@ -223,6 +223,23 @@ def test_libfit_library_in_shared_memory_and_beyond(bits, rows):
     assert np.array_equal(_u16(lib), want)
 
 
+@pytest.mark.parametrize("bits,L,rows", [(2, 32, 15625), (2, 32, 15626), (4, 32, 3906), (4, 32, 3907), (3, 32, 3072), (3, 5, 17),
+                                         (2, 40, 5), (4, 1, 16), (2, 256, 1000), (4, 17, 515)])
+def test_libfit_library_on_one_cluster_and_on_all_sms(bits, L, rows):
+    """Either side of the line between the two forms of the rounds (2 000 000 terms per assignment), fewer channels than blocks or
+    than centroids, centroids that no multiple of the blocks deals evenly, members beyond one staging buffer (a single centroid)."""
+    rng = np.random.default_rng(rows + L)
+    cb = np.sort(rng.standard_normal((rows, 1 << bits)), axis=1).astype(np.float16)
+    cb[rows // 2:rows // 2 + 3] = cb[0]
+    cb = np.ascontiguousarray(cb).view(np.uint16)
+    want = np.empty((L, 1 << bits), dtype=np.uint16)
+    xo._lib.xo_libfit_library(cb.reshape(-1), rows, bits, L, 8, want.reshape(-1))
+    lib = torch.zeros((L, 1 << bits), dtype=torch.int16, device="cuda")
+    qb.xfp_quant_libfit_library(_dev(cb), rows, bits, L, 8, lib, _ws(rows, 512))
+    torch.cuda.synchronize()
+    assert np.array_equal(_u16(lib), want)
+
+
 @pytest.mark.parametrize("bits,group", [(2, 128), (3, 128), (4, 128), (5, 128), (3, 64), (4, 256), (6, 64), (2, 256)])
 def test_libfit_assign_is_bit_exact(bits, group):
     """Group assignment at the paper's group size and at the other two the format carries (64, 256)."""
