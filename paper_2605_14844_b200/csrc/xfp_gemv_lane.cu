@@ -20,8 +20,8 @@
 //           address (one PRMT per look-up)
 //   N = 5   pair table, 1024 entries (128 KB, one CTA per SM) or, beyond one round of CTAs, one entry per index
 //   N = 6   one entry per index (a pair table would need 16 KB per channel), two look-ups joined by a PRMT
-// V2a: the library replicated once per bank -- pair tables of every entry where L * 4^N words fit (N = 2 at L = 32),
-// otherwise one entry per index with the entries of two library ids sharing a word -- see the kernel's comment.
+// V2a, N >= 4: the library replicated once per bank, one entry per index with the entries of two library ids sharing a word -- see
+// the kernel's comment.  V2a at N = 2, 3 runs on xfp_gemv_reg.cu, launched from here.
 //
 // x is staged once per CTA in shared memory in an order that lets a diagonal lane fetch the B registers of TWO
 // mma steps with one 16-byte load: inside every group of 16 k the two middle blocks of four are swapped
@@ -115,8 +115,8 @@ LaneConfig lane_config(const Layout& l, int n = 1) {
         int w = 16, p = 1, g = 0, t = -1;
         sscanf(e, "%d,%d,%d,%d", &w, &p, &g, &t);
         if (w == 0) return LaneConfig{16, 1, false, true};
-        const bool pairs = l.mode == 1 && (size_t)l.L * l.E * l.E * 128 <= 64 * 1024 && l.bits <= 3;
-        return LaneConfig{w, p > 2 ? 2 : p, l.mode == 1 ? !pairs : (l.bits == 6 || (l.bits == 5 && g)), false, t < 0 ? p <= 2 : t != 0};
+        if (lane_reg_book(l)) return LaneConfig{w, p, false, false, t < 0 ? RB > 4 * sched_sms() : t != 0};
+        return LaneConfig{w, p > 2 ? 2 : p, l.mode == 1 || (l.bits == 6 || (l.bits == 5 && g)), false, t < 0 ? p <= 2 : t != 0};
     }
 #endif
     // Measured on B200 over 4096 x 4096 .. 28672 x 8192 at every bit width (microseconds per call, graph replay):
@@ -127,18 +127,23 @@ LaneConfig lane_config(const Layout& l, int n = 1) {
     //  * N = 5 beyond one round: one entry per index instead of the 128 KB pair table, whose fill per 32 channels
     //    costs as much as 2048 weights of look-ups and cannot overlap anything with one CTA per SM
     const int sms = sched_sms();
+    if (lane_reg_book(l)) {
+        // No tables, 70 - 96 registers: one CTA of 16 warps per SM up to one CTA each (4096 x 4096, N = 3: 5.1 us, 8 warps 8.0: CTAs are
+        // packed on SMs that have room for two), two of 8 where those hold all row-blocks (8192 x 8192, N = 3: 15.3 against 21.6 with
+        // three, which leave a third of the SMs empty), three beyond (28672 x 8192, N = 3: 42.4, two 43.2; 12288 x 4096 11.9, two 13.0)
+        LaneConfig c{RB <= sms ? 16 : 8, RB <= sms ? 1 : RB <= 2 * sms ? 2 : 3, false};
+        if (c.per_sm == 3 && lane_smem_bytes(l, c) > 73u * 1024u) c.per_sm = 2;        // rows of x beyond 34000 weights
+        if (c.per_sm == 2 && lane_smem_bytes(l, c) > 110u * 1024u) c = LaneConfig{16, 1, false};
+        c.tiers = RB > 4 * sms;
+        return c;
+    }
     if (l.mode) {
-        // V2a: one look-up per weight in the per-bank library.  Up to 64 KB of tables (L * 2^N <= 512) two CTAs fit.
-        // Pair tables of the whole library where they fit the same 64 KB (L * 4^N <= 512: N = 2 with the paper's L = 32).
-        const bool pairs = (size_t)l.L * l.E * l.E * 128 <= 64 * 1024 && l.bits <= 3;
-        const bool two = lane_tab_bytes(l, !pairs) <= 64 * 1024 && RB > sms;
-        // (pair tables between two and four rounds: 16 warps, 12288 x 4096 at N = 2 13.8 against 14.4 us)
-        LaneConfig c{two && !(pairs && RB > 2 * sms && RB <= 4 * sms) ? 8 : 16, two ? 2 : 1, !pairs};
+        // V2a, N >= 4: one look-up per weight in the per-bank library.  Up to 64 KB of tables (L * 2^N <= 512) two CTAs fit.
+        const bool two = lane_tab_bytes(l, true) <= 64 * 1024 && RB > sms;
+        LaneConfig c{two ? 8 : 16, two ? 2 : 1, true};
         c.tiers = RB > 4 * sms;   // up to four rounds unsplit, as in V2 (N = 6, one CTA per SM: 12288 x 4096 33.6 -> 26.6 us)
-        c.off = false;
-        // the blobs of a routed layer in one launch: the resident CTAs of xfp_gemv_v2a.cu (pair tables built once per
-        // SM at N <= 3) measured faster (gate_up 30.7 vs 33.4 us, down 18.7 vs 22.9 us per launch of 8 experts)
-        if (n > 1) c.off = true;
+        // the blobs of a routed layer in one launch: the resident CTAs of xfp_gemv_v2a.cu
+        c.off = n > 1;
         return c;
     }
     if (RB <= sms) return LaneConfig{16, 1, l.bits == 6};
@@ -173,10 +178,10 @@ bool lane_supported(const Layout& l, const GemvCall& c) {
     if (c.batch != 1 || c.n < 1 || c.epilogue != 0) return false;
     if ((c.n > 1) != (c.packed_list != nullptr)) return false;
     if (l.bits < 2 || l.bits > 6) return false;
-    if (l.mode && (size_t)((l.L + 1) / 2) * l.E * 128 > 128 * 1024) return false;   // V2a: the per-bank library must fit 128 KB
+    if (l.mode && lane_tab_bytes(l, true) > 128 * 1024) return false;   // V2a tables: the per-bank library must fit 128 KB
     const LaneConfig cfg = lane_config(l, c.n);
     if (cfg.off) return false;
-    return lane_smem_bytes(l, cfg) <= (cfg.per_sm == 1 ? 220u : 110u) * 1024u;
+    return lane_smem_bytes(l, cfg) <= (cfg.per_sm == 1 ? 220u : cfg.per_sm == 2 ? 110u : 73u) * 1024u;
 }
 
 cudaError_t launch_gemv_lane(const Layout& l, const GemvCall& c, cudaStream_t s) {
@@ -190,12 +195,9 @@ cudaError_t launch_gemv_lane(const Layout& l, const GemvCall& c, cudaStream_t s)
     if (g_lane_trace && g_lane_trace_idx < g_lane_trace_calls) a.trace = g_lane_trace + (g_lane_trace_idx++) * 1024 * 8;
 #endif
     const size_t smem = lane_smem_bytes(l, cfg);
+    if (lane_reg_book(l)) return launch_reg(a, l.bits, cfg.per_sm, 1, sch.grid, smem, s);
     if (l.mode) {
         switch (l.bits) {
-            case 2: return cfg.sgl ? launch_lane_cfg<2, true, 1>(cfg, a, sch.grid, smem, s)
-                                   : launch_lane_cfg<2, false, 1>(cfg, a, sch.grid, smem, s);
-            case 3: return cfg.sgl ? launch_lane_cfg<3, true, 1>(cfg, a, sch.grid, smem, s)
-                                   : launch_lane_cfg<3, false, 1>(cfg, a, sch.grid, smem, s);
             case 4: return launch_lane_cfg<4, true, 1>(cfg, a, sch.grid, smem, s);
             case 5: return launch_lane_cfg<5, true, 1>(cfg, a, sch.grid, smem, s);
             default: return launch_lane_cfg<6, true, 1>(cfg, a, sch.grid, smem, s);

@@ -6,13 +6,6 @@
 #include "xfp_pair_common.cuh"
 
 namespace xfp {
-namespace {
-
-
-constexpr int kLaneSlots = 4;   // outlier slots a warp keeps in flight
-// smallest N whose codebooks travel through shared memory before the table fill (measured: N = 5 gains 4-8 %,
-// N <= 4 loses the extra barrier)
-constexpr int kLaneStageCodebooksFrom = 5;
 
 struct LaneArgs {
     Offsets off;
@@ -43,6 +36,16 @@ struct LaneArgs {
 #endif
 };
 
+// the launches of xfp_gemv_reg.cu: V2a at N = 2, 3, `per_sm` CTAs per SM (1: 16 warps, else 8), tiles of `nb` rows of x
+cudaError_t launch_reg(const LaneArgs& a, int bits, int per_sm, int nb, int grid, size_t smem, cudaStream_t s);
+
+namespace {
+
+constexpr int kLaneSlots = 4;   // outlier slots a warp keeps in flight
+// smallest N whose codebooks travel through shared memory before the table fill (measured: N = 5 gains 4-8 %,
+// N <= 4 loses the extra barrier)
+constexpr int kLaneStageCodebooksFrom = 5;
+
 // Phase stamps of a timing build (-DXFP_TRACE=1); a normal build has neither the stamps nor their plumbing.
 __device__ __forceinline__ void lstamp(const LaneArgs& a, int slot) {
 #ifdef XFP_TRACE
@@ -71,7 +74,7 @@ __device__ __forceinline__ uint32_t xpos(uint32_t k) { return (k & ~12u) | ((k &
 template <int N, bool SGL, int MODE>
 struct LaneCfg {
     static constexpr int E = 1 << N;
-    static constexpr bool kQuad = N == 2 && !SGL && MODE == 0;
+    static constexpr bool kQuad = N == 2 && MODE == 0;
     static constexpr bool kSingle = SGL;   // one entry per index: N = 6 always, N = 5 on short rows (no 128 KB fill)
     static constexpr int T = kQuad ? 256 : (kSingle ? E : E * E);          // table entries per channel
     static constexpr int kStride = (kQuad || N == 4) ? 256 : 128;            // bytes between entries
@@ -181,13 +184,6 @@ __device__ __forceinline__ void fill_tables_v2(unsigned char* tab, uint32_t* cbs
             const int t = warp * TW + i;
             *(uint32_t*)(tab + (size_t)t * kStride + lane * 4) = (i & 1) ? (cw[i >> 1] >> 16) : (cw[i >> 1] & 0xffffu);
         }
-    } else if (C::kSingle) {   // (instantiated for V2a widths only, where this branch is never taken)
-        constexpr int TW = T / W > 0 ? T / W : 1;
-#pragma unroll
-        for (int i = 0; i < TW; ++i) {
-            const int t = warp * TW + i;
-            if (t < T) *(uint32_t*)(tab + (size_t)t * kStride + lane * 4) = (uint32_t)__ldg(cb + t);
-        }
     } else if (T / W >= E) {
         // a warp fills whole rows of the pair matrix: entries (hi, 0..E-1) for its values of hi.  Every warp needs
         // every entry of its lanes' channels: the block's codebooks (32 E fp16, contiguous) are fetched once with
@@ -247,18 +243,17 @@ __device__ __forceinline__ uint32_t half_row(uint32_t e) {
     return (e >> 5) * 4096u + ((e >> 4) & 1u) * 128u + (e & 15u) * 256u;
 }
 
-// V2a tables: every row is one word repeated in the 32 banks -- HALF: row (id / 2) * 2^N + q holds lib[id][q] of ids
-// 2m (low half) and 2m + 1 (high half); else the pair table, row id * 4^N + (q1 << N | q0) holds (lib[id][q0],
-// lib[id][q1]).  A lane fetches the word of row e0 + lane, then the warp stores the 32 rows one after the other, each word
+// V2a tables (N >= 4): every row is one word repeated in the 32 banks, row (id / 2) * 2^N + q holds lib[id][q] of ids 2m (low half)
+// and 2m + 1 (high half).  A lane fetches the word of row e0 + lane, then the warp stores the 32 rows one after the other, each word
 // handed round by a shuffle (a warp that fetched two halves per row with uniform loads paid their latency once per
 // row: 3.9 us for the 1024 rows of N = 6).  Not inlined: inside the kernel the unrolled stores changed the register
-// allocation of the K loop (N = 3, 4: 62.2 against 58.3 us at 28672 x 8192).
-template <int N, int W, bool HALF, bool INTER>
+// allocation of the K loop (N = 4: 62.2 against 58.3 us at 28672 x 8192).
+template <int N, int W, bool INTER>
 __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __restrict__ lib, int L, int warp, int lane) {
     constexpr int E = 1 << N;
-    const int trows = HALF ? ((L + 1) >> 1) * E : L * E * E;
-    if (HALF && trows < 32 * W) {
-        // a small table (N = 3, 4 at L = 32): one row per warp and step, so that every warp takes part
+    const int trows = ((L + 1) >> 1) * E;
+    if (trows < 32 * W) {
+        // a small table (N = 4 at L = 32): one row per warp and step, so that every warp takes part
         for (int e = warp; e < trows; e += W) {
             const int m = e >> N, q = e & (E - 1);
             const uint32_t lo = __ldg(lib + (size_t)(2 * m) * E + q);
@@ -271,26 +266,21 @@ __device__ __noinline__ void fill_library(unsigned char* tab, const uint16_t* __
         const int e = e0 + lane;
         uint32_t word = 0u;
         if (e < trows) {
-            if (HALF) {
-                const int m = e >> N, q = e & (E - 1);
-                word = __ldg(lib + (size_t)(2 * m) * E + q);
-                if (2 * m + 1 < L) word |= (uint32_t)__ldg(lib + (size_t)(2 * m + 1) * E + q) << 16;
-            } else {
-                const uint16_t* cb = lib + (size_t)(e >> (2 * N)) * E;
-                word = (uint32_t)__ldg(cb + (e & (E - 1))) | ((uint32_t)__ldg(cb + ((e >> N) & (E - 1))) << 16);
-            }
+            const int m = e >> N, q = e & (E - 1);
+            word = __ldg(lib + (size_t)(2 * m) * E + q);
+            if (2 * m + 1 < L) word |= (uint32_t)__ldg(lib + (size_t)(2 * m + 1) * E + q) << 16;
         }
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const uint32_t v = __shfl_sync(0xffffffffu, word, r);
-            if (e0 + r < trows) *(uint32_t*)(tab + (HALF ? half_row<INTER>(e0 + r) : (e0 + r) * 128u) + lane * 4) = v;
+            if (e0 + r < trows) *(uint32_t*)(tab + half_row<INTER>(e0 + r) + lane * 4) = v;
         }
     }
 }
 
 // MODE 0: V2 (the channel's own codebook, tables private to the lane).  MODE 1: V2a -- the whole library replicated
-// once per bank (word ((id / 2) * 2^N + q) * 32 + lane holds lib[id][q] in its half id % 2; pair tables of every
-// entry where those fit), the table base of a lane follows the library id
+// once per bank (word ((id / 2) * 2^N + q) * 32 + lane holds lib[id][q] in its half id % 2; N >= 4, xfp_gemv_reg.cu takes the
+// others), the table base of a lane follows the library id
 // of its channel's current group, the fragment accumulates sum lib * x of ONE group, and after the group's steps the
 // sum moves to the lane that owns the channel and is folded into its accumulator with the group's scale and
 // mid-point:  acc += scale * G + mid * X_g,  X_g = sum of x over the group ("V2a: Shared Codebook Library").
@@ -305,18 +295,14 @@ template <int N, int W, int MINB, bool SGL, int MODE, bool TIO, int NB>
 __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs a) {
     using C = LaneCfg<N, SGL, MODE>;
     constexpr int E = C::E;
-    // V2a with a small library (L * 4^N words per bank fit): PAIR tables of every library entry, one look-up per two
-    // weights as in V2
-    constexpr bool kLibPair = MODE == 1 && !SGL;
-    // V2a otherwise: one entry per index, and the word of a bank holds that entry of TWO library ids (2m in the low
+    // V2a: one entry per index, and the word of a bank holds that entry of TWO library ids (2m in the low
     // half, 2m + 1 in the high half): every lane still reads its own bank, whatever ids and indices the lanes hold,
     // and the tables are half as large (64 KB at N = 5, 128 KB at N = 6 with L = 32)
-    constexpr bool kHalf = MODE == 1 && SGL;
+    constexpr bool kHalf = MODE == 1;
     // N = 4: interleaved tables except in the 8-warp CTAs of one row of x (matrices of more than one round), which gained 2 % on
     // their own and lost 2.4 us behind another launch (4096 x 4096 and 12288 x 4096 in turn: 23.2 us with plain tables, 25.6; the
     // 16-warp CTAs 20.5 -> 19.5).  That is one pair of shapes, and which part of the launch it is was not found.
     constexpr bool kInter = kHalf && N == 4 && !(W == 8 && NB == 1);
-    constexpr int kIdBytes = (kLibPair ? E * E : E) * 128;   // V2a: bytes between the tables of two ids (kHalf: id pairs)
     constexpr int T = C::T;
     constexpr int kStride = C::kStride;
     constexpr int kThreads = W * 32;
@@ -344,7 +330,7 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     const int src_a = (lane & ~3) | (t4 >> 1);
     // V2a: table offset of library id `id`
     auto id_offset = [](uint32_t id) -> uint32_t {
-        return kHalf ? half_row<kInter>((id >> 1) * (uint32_t)E) + (id & 1u) * 2u : id * (uint32_t)kIdBytes;
+        return half_row<kInter>((id >> 1) * (uint32_t)E) + (id & 1u) * 2u;
     };
 
 #pragma unroll 1
@@ -428,8 +414,8 @@ __global__ void __launch_bounds__(W * 32, MINB) gemv_lane_kernel(const LaneArgs 
     // ---- tables: warp w fills entries [w T / W, (w+1) T / W) of every lane's channel
     if (MODE != 0) {
         if (!kMulti || it == 0) {   // one library per blob: a resident CTA fills it once
-        if constexpr (N >= 5 || kLibPair || W == 8) {
-            fill_library<N, W, kHalf, kInter>(tab, b.cb, a.L, warp, lane);
+        if constexpr (N >= 5 || W == 8) {
+            fill_library<N, W, kInter>(tab, b.cb, a.L, warp, lane);
         } else {
             // small tables in a CTA that has its SM to itself: inline, so that the index loads issued above stay in
             // flight (registers that are the target of a load are written back around a call, which waits for them:
@@ -713,13 +699,16 @@ cudaError_t launch_lane_io(const LaneArgs& a, int grid, size_t smem, cudaStream_
 // ---- launch configurations: warps per CTA, CTAs per SM (64 registers per thread at 16 x 2), single-entry tables
 struct LaneConfig { int W, per_sm; bool sgl; bool off = false; bool tiers = true; };
 
+// V2a at N = 2, 3: codebooks in registers (xfp_gemv_reg.cu)
+inline bool lane_reg_book(const Layout& l) { return l.mode && l.bits <= 3; }
+
 inline size_t lane_tab_bytes(const Layout& l, bool sgl) {
     const int bits = l.bits;
     const size_t E = (size_t)1 << bits;
-    if (l.mode) {   // the library, one copy per bank: a word per entry (per pair of entries), or half a word when that does not fit
-        if (!sgl) return (size_t)l.L * E * E * 128;
+    if (lane_reg_book(l)) return ((size_t)l.L * E * 2 + 15) & ~size_t(15);   // the library's byte planes
+    if (l.mode) {   // the library, one copy per bank, a word holds one entry of two library ids (two tables interleaved at N = 4)
         const size_t tables = (size_t)(l.L + 1) / 2;
-        return (bits == 4 ? (tables + 1) & ~size_t(1) : tables) * E * 128;   // (two interleaved at N = 4) a word holds one entry of two library ids
+        return (bits == 4 ? (tables + 1) & ~size_t(1) : tables) * E * 128;
     }
     if (bits == 2) return 256 * 256;
     if (sgl) return E * 128;

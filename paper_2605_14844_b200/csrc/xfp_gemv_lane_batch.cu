@@ -37,8 +37,8 @@ bool batch_plan(const Layout& l, int rows_x, BatchPlan& p) {
     if (l.RB * 2 <= sms) return false;   // tiny matrices cut every block along K: the kernels with clusters do that
     bool sgl;
     if (l.mode) {
-        if ((size_t)((l.L + 1) / 2) * l.E * 128 > 128 * 1024) return false;
-        sgl = !((size_t)l.L * l.E * l.E * 128 <= 64 * 1024 && l.bits <= 3);
+        if (lane_tab_bytes(l, true) > 128 * 1024) return false;
+        sgl = l.bits >= 4;
     } else {
         sgl = l.bits >= 5;   // the 128 KB pair table of N = 5 leaves no room for several rows of x
     }
@@ -164,10 +164,10 @@ cudaError_t launch_gemv_lane_batch(const Layout& l, const GemvCall& c, cudaStrea
         a.tier_spp[0] = spp;
         a.tier_cta[1] = tail * a.tier_kst[0];
         cudaError_t e;
-        if (l.mode) {
+        if (lane_reg_book(l)) {
+            e = launch_reg(a, l.bits, p.cfg.per_sm, p.NB, G, p.smem, s);
+        } else if (l.mode) {
             switch (l.bits) {
-                case 2: e = p.cfg.sgl ? launch_tile<2, true, 1>(p, a, G, s) : launch_tile<2, false, 1>(p, a, G, s); break;
-                case 3: e = p.cfg.sgl ? launch_tile<3, true, 1>(p, a, G, s) : launch_tile<3, false, 1>(p, a, G, s); break;
                 case 4: e = launch_tile<4, true, 1>(p, a, G, s); break;
                 case 5: e = launch_tile<5, true, 1>(p, a, G, s); break;
                 default: e = launch_tile<6, true, 1>(p, a, G, s); break;

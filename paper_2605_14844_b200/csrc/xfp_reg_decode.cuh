@@ -7,7 +7,7 @@
 //   N = 2  10.5   (2 selector words of eight indices each per 32 stream bits, 4 shifts and masks, 16 PRMT per 16 weights)
 //   N = 3  13.5   (24 bits spread to eight nibbles: three masks here and three multiply-adds on the FMA pipe, 8 PRMT)
 //   N = 4  21     (indices are nibbles as they stand: 5 shifts and masks, 16 PRMT)
-// against 8 shared-memory wavefronts of single look-ups (V2a: 4 lanes' worth of banks hold the library) or 4 of pair look-ups.
+// against 8 look-ups of one weight or 4 of two on the data pipe of shared memory, a wavefront each where no banks conflict.
 #pragma once
 #include "xfp_common.cuh"
 

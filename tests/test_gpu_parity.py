@@ -235,6 +235,17 @@ def test_v2a_library_sizes(bits, lib_size):
     _check_dequant(q, pm)
 
 
+@pytest.mark.parametrize("bits,rows,cols,group", [(2, 6016, 384, 128), (3, 6016, 384, 64), (3, 4769, 768, 256), (2, 9500, 128, 64),
+                                                  (3, 33, 16384, 128)])
+def test_v2a_register_codebooks(bits, rows, cols, group):
+    """N = 2, 3 where one, two and three CTAs share an SM, K slices of few channels, both orders of the staged x with outliers in it."""
+    q = synth.random_quantized(1, rows, cols, bits, 0.01, seed=9950 + rows + bits, group_size=group)
+    pm = xfp.pack_tensors(q, col_bits=16)
+    sample = _sample_rows(rows, 64, seed=9951)
+    for batch in (1, 2, 4):
+        _check_gemv(q, pm, synth.activations(batch, cols, seed=9960 + batch), rows=sample)
+
+
 @pytest.mark.parametrize("mode,bits", [(0, 4), (0, 5), (1, 3), (1, 4)])
 def test_longest_rows(mode, bits):
     """K = 65536, the largest the descriptor admits (u16 outlier columns): x alone is 128 KB per batch row."""
