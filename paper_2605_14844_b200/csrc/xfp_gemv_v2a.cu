@@ -8,18 +8,11 @@
 // format's 128-weight groups, so a lane meets one (id, scale, mid) triple per channel and
 // super-chunk.
 //
-// Look-up.  Every lane may need a different library codebook, so the tables cannot be private to a
-// channel as in the V2 kernel.  Two layouts, chosen by the bit width:
-//   * N <= 3 (the routed-MoE mode): PAIR tables of the whole library, replicated 16 times: word
-//     (id * 4^N + pair) * 16 + (lane & 15) holds the half2 (lib[id][pair & (E-1)], lib[id][pair >> N]).
-//     One look-up decodes two weights.  Lanes l and l+16 share a copy; their words fall into the
-//     same bank only when their pair indices have the same parity (the bank is
-//     16 * (pair & 1) + (lane & 15)), so a look-up costs 1.5 shared-memory wavefronts on average,
-//     0.75 per weight.  128 KB at N = 3, L = 32: one CTA of 12 or 16 warps per SM.
-//   * N >= 4: the pair tables would not fit, so the library itself is replicated once per bank: word
-//     (id * 2^N + q) * 32 + lane holds lib[id][q] (fp16 in the low half).  Lane l only touches bank l;
-//     one look-up decodes one weight and a PRMT joins two of them into the half2 the tensor pipe
-//     wants.  Two CTAs of 8 warps per SM.
+// Look-up.  Every lane may need a different library codebook, so tables cannot be private to a channel as in the V2 kernel.
+//   * N <= 4: the library sits in shared memory once, as byte planes (a few KB); a lane loads the codebook of its channel's
+//     group into registers and decodes with PRMTs (xfp_reg_decode.cuh).  There is no table to fill.
+//   * N = 5: the library replicated once per bank: word (id * 2^N + q) * 32 + lane holds lib[id][q] (fp16 in the low half).
+//     Lane l only touches bank l; one look-up decodes one weight and a multiply-add joins two of them.
 //
 // Multiply-accumulate.  The half2 of a lane's two channels form the A fragment of
 // mma.sync.m16n8k16 and x sits on the diagonal lanes of the B fragment (see xfp_gemv_pair.cu).  The
@@ -36,6 +29,7 @@
 
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
+#include "xfp_reg_decode.cuh"
 
 namespace xfp {
 
@@ -60,7 +54,7 @@ struct V2aArgs {
     int epi;                 // 0 plain store; 1 SiLU(gate) * up inside every 64-channel block; 2 weighted sum over the blobs
     const float* epi_w;      // epi 2: [n] weights
     int comb_G, comb_ng;     // epi 2: runs per block of channels, blobs per run
-    int persist;             // per-bank library: resident CTAs walk the items
+    int persist;             // resident CTAs walk the items
 };
 
 __device__ __forceinline__ void mma16816a(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -87,27 +81,12 @@ __device__ __forceinline__ uint32_t entry_addr(const uint32_t* w, int j, uint32_
     return (v & mask) | base;
 }
 
-// Byte offset (pair << 6) of pair p (compile time) of a 128-weight stream, merged with `base`
-// (= id * 4^N * 64 + (lane & 15) * 4; the pair field occupies bits 6 .. 6+2N, which base leaves clear).
-template <int N>
-__device__ __forceinline__ uint32_t pair_entry_addr(const uint32_t* w, int p, uint32_t base) {
-    constexpr uint32_t mask = ((1u << (2 * N)) - 1u) << 6;
-    const int bit = p * 2 * N, wi = bit >> 5, off = bit & 31;
-    uint32_t v;
-    if (off + 2 * N > 32)
-        v = __funnelshift_r(w[wi], w[wi + 1], off - 6);   // field straight to bit 6
-    else if (off >= 6)
-        v = w[wi] >> (off - 6);
-    else
-        v = w[wi] << (6 - off);
-    return (v & mask) | base;
-}
-
 // FEAT instantiations carry typed IO (bf16 x, bf16 y) and the fused stores; the plain ones compile them out.
-template <int N, int NB, int W, bool PAIR, bool FEAT>
-__global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_kernel(const V2aArgs a) {
+template <int N, int NB, int W, bool FEAT>
+__global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const V2aArgs a) {
     const int epi = FEAT ? a.epi : 0;
     constexpr int E = 1 << N;
+    constexpr bool kReg = N <= 4;
     constexpr int kAWarps = W;
     constexpr int kAThreads = W * 32;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -115,12 +94,14 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     asm volatile("griddepcontrol.launch_dependents;");
     const int K = a.SC * kSuper;
-    const int tab_bytes = PAIR ? a.L * E * E * 64 : a.L * E * 128;
+    const int tab_bytes = kReg ? (a.L * E * 2 + 15) & ~15 : a.L * E * 128;
     unsigned char* tab = smem;
     uint16_t* xs = (uint16_t*)(smem + tab_bytes);             // [NB][K]
     float* xg = (float*)(xs + (size_t)NB * K);                // [NB][SC]
     float* red = xg + NB * a.SC;                              // [W][NB][64]
     __shared__ int s_last;
+    // where activation k sits in the staged copy
+    auto xat = [](uint32_t k) { return N == 2 ? (k & ~7u) | ((k & 1u) << 2) | ((k & 7u) >> 1) : k; };
 
     // the library the tables were built from, on the next 16-byte boundary (NB * SC floats of xg precede red)
     uint4* libcopy = (uint4*)(((uintptr_t)(red + (size_t)kAWarps * NB * kARows) + 15) & ~(uintptr_t)15);
@@ -223,7 +204,7 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
     // two groups per warp on the routed experts' shapes, and the chain pointer - header - slab cost as much as one of them)
     const bool same_run = epi == 2 && jj + 1 < per && prob + 1 < a.n;
     const int run_n = same_run ? run : run + (int)gridDim.x, jj_n = same_run ? jj + 1 : 0;
-    const bool more = (PAIR || a.persist) && run_n < nrun;
+    const bool more = a.persist && run_n < nrun;
     Item item_n = item;
     const void* packed_n = packed; const uint32_t* ell_n = ell; int slots_n = ell_slots;
     if (more) {
@@ -263,7 +244,7 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
 #pragma unroll
             for (int q = 0; q < kASlots; ++q) {
                 const float v = h2f((uint16_t)(oe[h][q] >> 16));
-                const uint32_t col = oe[h][q] & 0xffffu;
+                const uint32_t col = xat(oe[h][q] & 0xffffu);
 #pragma unroll
                 for (int bb = 0; bb < NB; ++bb) acc[bb][h] = fmaf(v, h2f(xs[(size_t)bb * K + col]), acc[bb][h]);
             }
@@ -285,16 +266,8 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
         if (__syncthreads_or(differs)) {
             fresh = true;
             for (int i = threadIdx.x; i < nvec; i += kAThreads) libcopy[i] = __ldg(cb4 + i);
-            if (PAIR) {
-                // pair tables, 16 copies: words (id * E*E + pair) * 16 .. + 15 hold the same half2.  Four threads per
-                // entry, 16 bytes each: a warp's store covers 512 contiguous bytes (one thread writing the entry's 64
-                // bytes put a quarter-warp into two bank groups: 4300 wavefronts per fill instead of 1024)
-                for (int t = threadIdx.x; t < a.L * E * E * 4; t += kAThreads) {
-                    const int e = t >> 2, id = e / (E * E), pr = e % (E * E);
-                    const uint32_t v = (uint32_t)__ldg(b.cb + id * E + (pr & (E - 1))) |
-                                       ((uint32_t)__ldg(b.cb + id * E + (pr >> N)) << 16);
-                    ((uint4*)(tab + (size_t)e * 64))[t & 3] = make_uint4(v, v, v, v);
-                }
+            if constexpr (kReg) {
+                for (int id = threadIdx.x; id < a.L; id += kAThreads) store_book<N>(tab, a.L, id, make_book<N>(b.cb + (size_t)id * E));
             } else {
                 // one copy per bank: word (e * 32 + lane) = lib[e] for every lane.  A lane fetches entry e0 + lane, the warp
                 // stores 32 rows, the entries handed round by shuffle (one uniform load per row paid its latency per row)
@@ -325,6 +298,8 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
                 if (bb < a.nb) v = __ldg((const uint4*)(x + (size_t)bb * a.cols + kk));
                 if (FEAT) v = x8_as_f16(v, a.x_bf16);
+                if (N == 2)   // the even k of every eight, then the odd ones: the order in which two steps decode them
+                    v = make_uint4(prmt(v.x, v.y, 0x5410u), prmt(v.z, v.w, 0x5410u), prmt(v.x, v.y, 0x7632u), prmt(v.z, v.w, 0x7632u));
                 *(uint4*)(xs + (size_t)t * 8) = v;
             }
         }
@@ -362,14 +337,8 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
     const int src0 = (lane & ~3) | (t4 >> 1);
     const bool odd = t4 & 1;
 
+    RegBook<kReg ? N : 2> book0, book1;
     auto lookup = [&](uint32_t (&f)[4], int m, uint32_t base0, uint32_t base1) {
-        if (PAIR) {
-            f[0] = *(const uint32_t*)(tab + pair_entry_addr<N>(w0, 2 * m, base0));       // (k, k+1) of channel 0
-            f[1] = *(const uint32_t*)(tab + pair_entry_addr<N>(w1, 2 * m, base1));       // (k, k+1) of channel 1
-            f[2] = *(const uint32_t*)(tab + pair_entry_addr<N>(w0, 2 * m + 1, base0));   // (k+2, k+3) of channel 0
-            f[3] = *(const uint32_t*)(tab + pair_entry_addr<N>(w1, 2 * m + 1, base1));   // (k+2, k+3) of channel 1
-            return;
-        }
         const uint32_t l00 = *(const uint32_t*)(tab + entry_addr<N>(w0, 4 * m + 0, base0));
         const uint32_t l01 = *(const uint32_t*)(tab + entry_addr<N>(w0, 4 * m + 1, base0));
         const uint32_t l02 = *(const uint32_t*)(tab + entry_addr<N>(w0, 4 * m + 2, base0));
@@ -396,16 +365,12 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
             consume_slots();
             if (++oround < nrounds) fetch_slots(oround);
         }
-        const uint32_t base0 = PAIR ? id0 * (uint32_t)(E * E * 64) + (uint32_t)(lane & 15) * 4u
-                                    : id0 * (uint32_t)(E * 128) + (uint32_t)lane * 4u;
-        const uint32_t base1 = PAIR ? id1 * (uint32_t)(E * E * 64) + (uint32_t)(lane & 15) * 4u
-                                    : id1 * (uint32_t)(E * 128) + (uint32_t)lane * 4u;
+        const uint32_t base0 = id0 * (uint32_t)(E * 128) + (uint32_t)lane * 4u, base1 = id1 * (uint32_t)(E * 128) + (uint32_t)lane * 4u;
+        if constexpr (kReg) { book0 = load_book<N>(tab, a.L, id0); book1 = load_book<N>(tab, a.L, id1); }
         const unsigned char* xp = xrow + (size_t)s * (kSuper * 2);
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-        uint32_t fa[4], fb[4];
         uint4 xa = make_uint4(0u, 0u, 0u, 0u), xb = make_uint4(0u, 0u, 0u, 0u);
         if (diag) xa = *(const uint4*)xp;
-        lookup(fa, 0, base0, base1);
         auto reload = [&](int gi) {   // index vectors are reloaded for the next group once fully consumed
 #pragma unroll
             for (int v = 0; v < N; ++v) {
@@ -418,6 +383,31 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
                 }
             }
         };
+        if constexpr (kReg) {
+            // eight weights of both channels at a time, one batch ahead of the tensor pipe
+            uint32_t p0[4], p1[4], q0[4], q1[4];
+            reg_decode8<N>(p0, w0, 0, book0);
+            reg_decode8<N>(p1, w1, 0, book1);
+#pragma unroll
+            for (int m = 0; m < kSuper / 4; m += 4) {
+                if (diag) xb = *(const uint4*)(xp + (m + 2) * 8);
+                reg_decode8<N>(q0, w0, m / 2 + 1, book0);
+                reg_decode8<N>(q1, w1, m / 2 + 1, book1);
+                mma16816a(c0, p0[0], p1[0], p0[2], p1[2], xa.x, xa.y);
+                mma16816a(c1, p0[1], p1[1], p0[3], p1[3], xa.z, xa.w);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) reload(m + i);
+                if (m + 4 < kSuper / 4) {
+                    if (diag) xa = *(const uint4*)(xp + (m + 4) * 8);
+                    reg_decode8<N>(p0, w0, m / 2 + 2, book0);
+                    reg_decode8<N>(p1, w1, m / 2 + 2, book1);
+                }
+                mma16816a(c0, q0[0], q1[0], q0[2], q1[2], xb.x, xb.y);
+                mma16816a(c1, q0[1], q1[1], q0[3], q1[3], xb.z, xb.w);
+            }
+        } else {
+        uint32_t fa[4], fb[4];
+        lookup(fa, 0, base0, base1);
 #pragma unroll
         for (int m = 0; m < kSuper / 4; m += 4) {   // one mma per 4 consecutive k, look-ups one mma ahead
             if (diag) xb = *(const uint4*)(xp + (m + 2) * 8);
@@ -436,6 +426,7 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
                 reload(m + 4);
             }
             mma16816a(c1, fb[0], fb[1], fb[2], fb[3], xb.z, xb.w);
+        }
         }
         // group sums to their owners, then  acc += scale * G + mid * X_g
         const float d0 = c0[0] + c1[0], d1 = c0[1] + c1[1], d2 = c0[2] + c1[2], d3 = c0[3] + c1[3];
@@ -465,7 +456,7 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
                     const uint32_t e = __ldg(b.oent + p);
 #pragma unroll
                     for (int bb = 0; bb < NB; ++bb)
-                        acc[bb][h] = fmaf(h2f((uint16_t)(e >> 16)), h2f(xs[(size_t)bb * K + (e & 0xffffu)]), acc[bb][h]);
+                        acc[bb][h] = fmaf(h2f((uint16_t)(e >> 16)), h2f(xs[(size_t)bb * K + xat(e & 0xffffu)]), acc[bb][h]);
                 }
             }
         }
@@ -565,46 +556,28 @@ __global__ void __launch_bounds__(W * 32, W == 4 ? 4 : W == 8 ? 2 : 1) gemv_v2a_
 
 // ------------------------------------------------------------------------------------ host side
 
-// Launch configuration of a layout: pair tables (one CTA per SM, 12 or 16 warps) when they fit, else the
-// per-bank library (two CTAs of 8 warps per SM, or one of 16 warps when the library is too large for two).
-struct V2aConfig { bool pair; int warps, slots; size_t smem; };
+// Launch configuration of a layout: two CTAs of 8 warps per SM, or one of 16 where x (or the tables of N = 5) leave no room for two.
+struct V2aConfig { int warps, slots; size_t smem; };
 
-static size_t v2a_smem_bytes(const Layout& l, int nb, bool pair, int warps) {
-    const size_t tab = pair ? (size_t)l.L * l.E * l.E * 64 : (size_t)l.L * l.E * 128;
+static size_t v2a_smem_bytes(const Layout& l, int nb, int warps, bool tables) {
+    const size_t tab = tables ? (size_t)l.L * l.E * 128 : ((size_t)l.L * l.E * 2 + 15) & ~size_t(15);
     return tab + (size_t)nb * l.cols * 2 + (size_t)nb * l.SC * 4 + (size_t)warps * nb * kARows * 4 +
            (size_t)l.L * l.E * 2 + 16;   // + the copy of the library the tables were built from, 16-byte aligned
 }
 
-static V2aConfig v2a_config(const Layout& l, int nb, int n = 1, int epilogue = 0) {
-    // Pair tables cost 128 KB of fills per resident CTA and run one CTA of 12 or 16 warps per SM: they pay off
-    // when every SM has a few hundred thousand weights to decode and K is long enough to keep those warps busy
-    // (measured: 28672 x 8192 53 vs 61 us, 8192 x 8192 18.6 vs 22.9, 12288 x 4096 18.7 vs 20.0 in their favour;
-    // 4096 x 4096 10.4 vs 9.1 and the routed experts' 4096 x 1536 down projections 20.6 vs 18.7 against them).
-    const bool big = (long long)l.rows * l.cols * n >= 40ll * 1000 * 1000 && l.SC >= 32;
+static V2aConfig v2a_config(const Layout& l, int nb) {
     const int sms = sched_sms();
-    if (l.bits <= 3 && big) {
-        // K is shared by the warps in super-chunks: 12 warps when that divides the count and 16 does not
-        const int warps = (l.SC % 16 != 0 && l.SC % 12 == 0) ? 12 : 16;
-        const size_t sm = v2a_smem_bytes(l, nb, true, warps);
-        if (sm <= 224u * 1024u) return V2aConfig{true, warps, sms, sm};
-    }
-    // The weighted sum over the blobs (K is the routed experts' short hidden size) with more items than two CTAs per SM: four
-    // CTAs of four warps leave fewer warps without a group (12 groups are 3 each, against 2 or 1 of 8 warps) and wait for one
-    // another at four barriers instead of two.  Routed block of 8 experts, N = 3: 4096 x 1536 49.9 -> 47.1 us, 7168 x 2048
-    // 101.9 -> 95.8; with fewer items the SMs run out of warps (6144 x 2560, 2 experts: 39.5 -> 50.6).
-    const size_t sm4 = v2a_smem_bytes(l, nb, false, 4);
-    if (epilogue == 2 && l.bits <= 3 && (long long)((l.RB + 1) / 2) * n > 2 * sms && sm4 <= 55u * 1024u)
-        return V2aConfig{false, 4, 4 * sms, sm4};
-    const size_t sm8 = v2a_smem_bytes(l, nb, false, 8);
-    if (sm8 <= 110u * 1024u) return V2aConfig{false, 8, 2 * sms, sm8};
-    return V2aConfig{false, 16, sms, v2a_smem_bytes(l, nb, false, 16)};   // large library (N = 5): one CTA per SM
+    const bool tables = l.bits > 4;
+    const size_t sm8 = v2a_smem_bytes(l, nb, 8, tables);
+    if (sm8 <= 110u * 1024u) return V2aConfig{8, 2 * sms, sm8};
+    return V2aConfig{16, sms, v2a_smem_bytes(l, nb, 16, tables)};
 }
 
 bool v2a_supported(const Layout& l, int batch) {
     if (l.mode != 1 || l.bits < 2 || l.bits > 5 || batch > 2) return false;
     if (l.GH != 1) return false;   // groups of 64 weights: two table bases per super-chunk, served by the generic kernel
-    const V2aConfig cfg = v2a_config(l, batch);
-    return cfg.smem <= (cfg.warps == 8 ? 110u : 224u) * 1024u;
+    // libraries whose copy per bank fits beside x (what the fused stores take; the general kernel serves the others)
+    return v2a_smem_bytes(l, batch, 16, true) <= 224u * 1024u;
 }
 
 size_t v2a_workspace_bytes(const Layout& l) {
@@ -613,13 +586,13 @@ size_t v2a_workspace_bytes(const Layout& l) {
     return align256((size_t)l.RB * 4) + align256((size_t)64 * 2 * (size_t)blocks * kARows * 4);
 }
 
-template <int N, int NB, int W, bool PAIR, bool FEAT>
+template <int N, int NB, int W, bool FEAT>
 static cudaError_t launch_v2a_feat(const V2aArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(gemv_v2a_kernel<N, NB, W, PAIR, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             W == 4 ? 56 * 1024 : W == 8 ? 112 * 1024 : 226 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(gemv_v2a_kernel<N, NB, W, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             W == 8 ? 112 * 1024 : 226 * 1024);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
@@ -633,27 +606,24 @@ static cudaError_t launch_v2a_feat(const V2aArgs& a, dim3 grid, size_t smem, cud
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_v2a_kernel<N, NB, W, PAIR, FEAT>, a);
+    return cudaLaunchKernelEx(&cfg, gemv_v2a_kernel<N, NB, W, FEAT>, a);
 }
 
-template <int N, int NB, int W, bool PAIR>
+template <int N, int NB, int W>
 static cudaError_t launch_v2a(const V2aArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-    if (a.epi != 0 || a.x_bf16 || a.y_is_fp16 == 2) return launch_v2a_feat<N, NB, W, PAIR, true>(a, grid, smem, s);
-    return launch_v2a_feat<N, NB, W, PAIR, false>(a, grid, smem, s);
+    if (a.epi != 0 || a.x_bf16 || a.y_is_fp16 == 2) return launch_v2a_feat<N, NB, W, true>(a, grid, smem, s);
+    return launch_v2a_feat<N, NB, W, false>(a, grid, smem, s);
 }
 
 template <int N, int NB>
 static cudaError_t launch_v2a_cfg(const V2aConfig& cfg, const V2aArgs& a, dim3 grid, cudaStream_t s) {
-    if (N <= 3 && cfg.pair)
-        return cfg.warps == 12 ? launch_v2a<(N <= 3 ? N : 3), NB, 12, true>(a, grid, cfg.smem, s)
-                               : launch_v2a<(N <= 3 ? N : 3), NB, 16, true>(a, grid, cfg.smem, s);
-    if (N <= 3 && NB == 1 && cfg.warps == 4) return launch_v2a<(N <= 3 ? N : 3), 1, 4, false>(a, grid, cfg.smem, s);
-    if (cfg.warps == 16) return launch_v2a<N, NB, 16, false>(a, grid, cfg.smem, s);
-    return launch_v2a<N, NB, 8, false>(a, grid, cfg.smem, s);
+    if (cfg.warps == 16) return launch_v2a<N, NB, 16>(a, grid, cfg.smem, s);
+    return launch_v2a<N, NB, 8>(a, grid, cfg.smem, s);
 }
 
 cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s) {
-    const V2aConfig cfg = v2a_config(l, c.batch, c.n, c.epilogue);
+    if (expert_supported(l, c)) return launch_gemv_expert(l, c, s);
+    const V2aConfig cfg = v2a_config(l, c.batch);
     V2aArgs a{};
     a.off = offsets_of(l);
     a.packed = c.packed; a.x = c.x; a.y = c.y;
@@ -706,17 +676,15 @@ cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s) 
     long long items = (long long)a.items_x * c.n;
     a.comb_G = 1; a.comb_ng = 1;
     if (c.epilogue == 2) {
-        // pair tables: as few runs per block as still fill the resident CTAs; per-bank library: one blob per CTA
-        int G = cfg.pair ? std::max(1, std::min(c.n, cfg.slots / std::max(1, a.blocks))) : c.n;
+        const int G = c.n;     // one blob per run: a CTA walks them where there are more than slots
         a.comb_ng = (c.n + G - 1) / G;
         a.comb_G = (c.n + a.comb_ng - 1) / a.comb_ng;
         items = (long long)a.blocks * a.comb_G;
     }
-    // pair tables are expensive to build: resident CTAs walk the items; the per-bank library launches one CTA per item
-    // several blobs on the per-bank library with more items than CTA slots: resident CTAs walk the items, so the
-    // tables are not rebuilt for the later rounds (routed experts' down projections: 1 % per token-layer)
-    a.persist = (!cfg.pair && c.n > 1 && items > cfg.slots) ? 1 : 0;
-    dim3 grid((unsigned)((cfg.pair || a.persist) ? (items < cfg.slots ? items : cfg.slots) : items), 1, 1);
+    // several blobs with more items than CTA slots: resident CTAs walk the items, so that x is staged once per CTA and an item's
+    // first loads travel under the previous one
+    a.persist = c.n > 1 && (items > cfg.slots || a.comb_ng > 1);
+    dim3 grid((unsigned)(a.persist && items > cfg.slots ? cfg.slots : items), 1, 1);
     switch (l.bits * 10 + c.batch) {
         case 21: return launch_v2a_cfg<2, 1>(cfg, a, grid, s);
         case 22: return launch_v2a_cfg<2, 2>(cfg, a, grid, s);

@@ -94,6 +94,9 @@ cudaError_t launch_gemv_frag(const Layout& l, const GemvCall& c, cudaStream_t s)
 bool v2a_supported(const Layout& l, int batch);
 size_t v2a_workspace_bytes(const Layout& l);
 cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s);
+// Of these the fused stores of a routed expert block at N <= 4; see xfp_gemv_expert.cu.
+bool expert_supported(const Layout& l, const GemvCall& c);
+cudaError_t launch_gemv_expert(const Layout& l, const GemvCall& c, cudaStream_t s);
 
 // Batched path (3..16 rows of x), V2 and V2a; see xfp_gemv_batch.cu.
 bool batch_supported(const Layout& l, int batch);

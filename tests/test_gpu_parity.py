@@ -602,6 +602,41 @@ def test_fused_expert_block(bits, n, rows_gu, hidden, y_fp16):
     assert np.all(np.abs(got - plain) <= 0.05 * TOL * bound + (2.0 ** -10 * np.abs(want) if y_fp16 else 0.0) + 1e-30)
 
 
+@pytest.mark.parametrize("bits,n,rows,cols,lib_size,rate,placement", [
+    (3, 40, 96, 128, 32, 0.01, "uniform"), (2, 5, 4104, 1664, 7, 0.002, "uniform"), (4, 3, 70, 2048, 40, 0.05, "one_row"),
+    (3, 9, 160, 384, 1, 0.0, "uniform"), (4, 10, 64, 768, 33, 0.02, "clustered"), (2, 2, 64, 40960, 32, 0.001, "uniform"),
+    (3, 70, 32, 2048, 32, 0.005, "uniform")])
+def test_fused_stores_over_blobs_with_libraries_of_their_own(bits, n, rows, cols, lib_size, rate, placement):
+    """Weighted sums of one run and of several runs per row-block, one super-chunk, more blobs than a CTA takes, rows that fill no
+    row-block, slabs that overflow, x beyond what the fused kernel stages; gated stores of the same blobs where rows allow."""
+    qs = [synth.random_quantized(1, rows, cols, bits, rate, seed=2600 + j, lib_size=lib_size, placement=placement) for j in range(n)]
+    pms = [xfp.pack_tensors(q, col_bits=16) for q in qs]
+    d = _group_desc(pms)
+    ws = torch.zeros(n * xfp.xfp_packed_size(d)[1], dtype=torch.uint8, device="cuda")
+    ptr = lambda ts: torch.tensor([t.data_ptr() for t in ts], dtype=torch.int64, device="cuda")
+    x16 = synth.activations(n, cols, seed=2610)
+    xd = _x_dev(x16)
+    wts = np.random.default_rng(2611).standard_normal(n).astype(np.float32)
+    refs = [xo.gemv(to_oracle(q), x16[j:j + 1]) for j, q in enumerate(qs)]
+    y = torch.full((rows,), float("nan"), dtype=torch.float32, device="cuda")
+    xs, blobs = ptr([xd[j] for j in range(n)]), ptr([p.packed for p in pms])
+    for _ in range(2):
+        xfp.xfp_gemv_grouped_epilogue(d, n, blobs, xs, ptr([y] * n), False, xfp.XFP_EPI_COMBINE, torch.from_numpy(wts).cuda(), ws)
+    want = sum(float(w) * r[0][0] for w, r in zip(wts, refs))
+    bound = sum(abs(float(w)) * r[1][0] for w, r in zip(wts, refs))
+    assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - want) <= TOL * bound + 1e-30)
+    if rows % 64 == 0:
+        h = torch.full((n, rows // 2), float("nan"), dtype=torch.float32, device="cuda")
+        xfp.xfp_gemv_grouped_epilogue(d, n, blobs, xs, ptr([h[j] for j in range(n)]), False, xfp.XFP_EPI_SWIGLU, None, ws)
+        got = h.cpu().numpy().astype(np.float64)
+        gate = (np.arange(rows // 64)[:, None] * 64 + np.arange(32)[None, :]).reshape(-1)
+        for j, (ref, absum) in enumerate(refs):
+            g, u, eg, eu = ref[0][gate], ref[0][gate + 32], TOL * absum[0][gate], TOL * absum[0][gate + 32]
+            lim = 1.1 * np.abs(u) * eg + np.abs(g / (1.0 + np.exp(-g))) * eu + 1.1 * eg * eu + 2.0 ** -20 * np.abs(g * u) + 1e-30
+            assert np.all(np.abs(got[j] - xo.silu_mul(g, u)) <= lim)
+    assert int(ws[:4 * ((rows + 31) // 32) * n].view(torch.int32).abs().sum().item()) == 0
+
+
 @pytest.mark.parametrize("mode,bits", [(0, 4), (1, 3), (1, 6)])
 @pytest.mark.parametrize("half", [0, 1])
 def test_grouped_c_functions_of_the_abi(mode, bits, half):
