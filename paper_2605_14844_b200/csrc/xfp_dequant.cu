@@ -28,7 +28,8 @@ constexpr int kDqWarps = 8;
 constexpr int kDqRange = 32;        // super-chunks of a block at most: the tail of outliers stays short
 constexpr int kTileRow = 144;       // bytes of a row of 64 weights in the staging tile: eight lanes' rows in distinct banks
 constexpr int kLibEntries = 8192;   // library entries (L * 2^N) that are staged in shared memory
-constexpr int kDqSlots = 64;        // outlier slots of a row-block that are staged in shared memory; later ones are read from the blob
+constexpr int kDqSlots = 64;        // outliers of a channel in the block's range that are staged in shared memory; where there are more,
+                                    // the channel's are read from the blob
 constexpr int kDqStarts = (kDqRange + 1) * 32 * 2, kDqEntries = kDqSlots * 32 * 4;   // bytes of the starts and of the staged slots
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -120,9 +121,9 @@ __global__ void __launch_bounds__(kDqWarps * 32, N <= 4 ? 3 : 0) dequant_kernel(
                 const int j = jb + i - 1;
                 if (j >= j1 || j > in_slab) continue;
                 const bool have = j < in_slab;
-                if (j < kDqSlots && have) ents[j * 32 + lane] = v[i];
                 descends |= j > 0 && have && (v[i] & 0xffffu) <= (v[i - 1] & 0xffffu);
                 const int b0 = j > 0 ? rel(v[i - 1]) : -1, b1 = have ? rel(v[i]) : nsc;
+                if (have && b1 >= 0 && b1 < nsc) ents[(j % kDqSlots) * 32 + lane] = v[i];
                 for (int t = b0 + 1; t <= b1; ++t) starts[t * 32 + lane] = (uint16_t)j;
             }
         }
@@ -131,10 +132,11 @@ __global__ void __launch_bounds__(kDqWarps * 32, N <= 4 ? 3 : 0) dequant_kernel(
         __syncthreads();
     }
     const bool in_tile = T::kReg && a.ell_slots != 0 && !in_place;
+    const bool ents_whole = in_tile && starts[nsc * 32 + lane] - starts[lane] <= kDqSlots;
     for (int sc = s0 + warp; sc < s1; sc += kDqWarps) {
         int j = 0, jend = 0;
         if (in_tile) { j = starts[(sc - s0) * 32 + lane]; jend = starts[(sc - s0 + 1) * 32 + lane]; }
-        auto entry = [&](int i) { return i < kDqSlots ? ents[i * 32 + lane] : __ldg(slab + (size_t)(1 + i) * 32); };
+        auto entry = [&](int i) { return ents_whole ? ents[(i % kDqSlots) * 32 + lane] : __ldg(slab + (size_t)(1 + i) * 32); };
         uint32_t e = j < jend ? entry(j) : 0u;
         uint32_t w[4 * N + 1];
 #pragma unroll
@@ -250,9 +252,21 @@ cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cuda
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
-    // few row-blocks: shorter ranges, at least one super-chunk per warp, until the blocks fill the GPU twice
     int range = a.SC < kDqRange ? a.SC : kDqRange;
-    while (range > kDqWarps && (long long)l.RB * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
+    if (T::kReg) {
+        // rounds of three blocks per SM times (turns of a warp and one for the block's first loads), in the fewest parts that reach
+        // the least: 4096 x 4096 V2 N = 4 13.0 us with ranges of 16, 15.8 with 8, 14.5 with 32; 12288 x 4096 30.9 with 32, 32.8 with
+        // 16; 8192 x 8192 N = 3 35.6 with 22, 37.0 with 16, 43.1 with 32
+        const long long slots = 3ll * sm_count();
+        long long best = -1;
+        for (int parts = (a.SC + kDqRange - 1) / kDqRange; parts <= (a.SC + kDqWarps - 1) / kDqWarps; ++parts) {
+            const int r = (a.SC + parts - 1) / parts;
+            const long long cost = (l.RB * (long long)((a.SC + r - 1) / r) + slots - 1) / slots * ((r + kDqWarps - 1) / kDqWarps + 1);
+            if (best < 0 || cost < best) { best = cost; range = r; }
+        }
+    } else {        // few row-blocks: shorter ranges, at least one super-chunk per warp, until the blocks fill the GPU twice
+        while (range > kDqWarps && (long long)l.RB * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
+    }
     a.range = range;
     dequant_kernel<N, MODE><<<(unsigned)(l.RB * ((a.SC + range - 1) / range)), kDqWarps * 32, smem, s>>>(a);
     return cudaGetLastError();
