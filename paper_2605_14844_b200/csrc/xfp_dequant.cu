@@ -7,11 +7,11 @@
 //   V2a  a lane decodes the 2^N entries its channel's group can take once -- D16 = fp16(fp32(scale * lib[id] + mid)) -- into
 //        registers (N <= 4) or a column of a table of its warp, and the weights of the group are look-ups as in V2: 2^N
 //        conversions per group instead of one per weight.
-//   S    up to N = 4 the block notes where every super-chunk's outliers begin in its channels' slabs and a lane adds those of its
-//        channel to the staged row, one correctly rounded fp16 addition each.  What a slab cannot say (channels longer than their
-//        slab, columns that do not ascend), and all of them above N = 4, is added in place behind the block's stores (above, where
-//        tables leave one or two blocks to an SM, the list in front of the decode cost more: 12288 x 4096 V2a N = 6 38.2 -> 46.1 us
-//        with pack, half of both).
+//   S    up to N = 4, and four blocks to a row-block, the block notes where every super-chunk's outliers begin in its channels'
+//        slabs and a lane adds those of its channel to the staged row, one correctly rounded fp16 addition each.  What a slab
+//        cannot say (channels longer than their slab, columns that do not ascend), and all of them elsewhere, is added in place
+//        behind the block's stores (above N = 4, where tables leave one or two blocks to an SM, the list in front of the decode
+//        cost more: 12288 x 4096 V2a N = 6 38.2 -> 46.1 us with pack, half of both).
 //   out  a tile of shared memory turns a lane's 64 weights into whole 128-byte lines of the channels' rows.
 // Tables in shared memory and outliers in place behind the stores -> this, cold: 12289 x 4096 V2a N = 4, 1 % outliers 35.2 -> 32.0 us,
 // 3072 x 4096 V2a N = 2 14.2 -> 10.8, 12288 x 4096 V2 N = 4 33.3 -> 29.1.  100 MB of stores and 29 MB of loads are 20 us at the copy
@@ -55,6 +55,7 @@ struct DqArgs {
     uint16_t* out;
     int rows, cols, RB, SC, GH, L, ell_slots;
     int range;                // super-chunks of a block
+    bool lists;               // outliers are added to the staged rows
 };
 
 template <int N, int MODE>
@@ -106,8 +107,8 @@ __global__ void __launch_bounds__(kDqWarps * 32, N <= 4 ? 3 : 0) dequant_kernel(
     const int nsc = s1 - s0;
     const uint32_t* slab = a.b.ell + (size_t)rb * (a.ell_slots + 1) * 32 + lane;
     const int len = a.ell_slots && row < a.rows ? (int)__ldg(slab) : 0, in_slab = min(len, a.ell_slots);
-    bool in_place = !T::kReg && a.ell_slots != 0;
-    if (T::kReg && a.ell_slots) {
+    bool in_place = a.ell_slots != 0 && !(T::kReg && a.lists);
+    if (T::kReg && a.lists) {
         bool descends = false;
         auto rel = [&](uint32_t e) { return max(-1, min(nsc, (int)((e & 0xffffu) >> 7) - s0)); };
         // a run of slots to every warp, slot `in_slab` closes a channel's list; the loads do not wait for the channels' lengths
@@ -268,6 +269,9 @@ cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cuda
         while (range > kDqWarps && (long long)l.RB * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
     }
     a.range = range;
+    // every block of a row-block walks all of its slots for the lists: beyond four parts that costs more than adding in place
+    // (1024 x 8192 V2 N = 4, eight parts, 1 % outliers: 12.5 us with lists, 8.3 without; 3072 x 4096 V2a N = 4, four: 12.5, 12.9)
+    a.lists = T::kReg && a.ell_slots != 0 && (a.SC + range - 1) / range <= 4;
     dequant_kernel<N, MODE><<<(unsigned)(l.RB * ((a.SC + range - 1) / range)), kDqWarps * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
