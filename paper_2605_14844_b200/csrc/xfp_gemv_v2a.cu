@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     auto xat = [](uint32_t k) { return N == 2 ? (k & ~7u) | ((k & 1u) << 2) | ((k & 7u) >> 1) : k; };
 
     // the library the tables were built from, on the next 16-byte boundary (NB * SC floats of xg precede red)
-    uint4* libcopy = (uint4*)(((uintptr_t)(red + (size_t)kAWarps * NB * kARows) + 15) & ~(uintptr_t)15);
+    uint2* libcopy = (uint2*)(((uintptr_t)(red + (size_t)kAWarps * NB * kARows) + 15) & ~(uintptr_t)15);
     bool have_tables = false;
     bool waited = false;
     const uint16_t* x_staged = nullptr;
@@ -254,13 +254,13 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     //      built once per CTA; a blob whose library differs from the one they were built from rebuilds them.
     bool fresh = false;
     {
-        const uint4* cb4 = (const uint4*)b.cb;
-        const int nvec = a.L * E / 8;   // the library in 16-byte vectors (L * E is a multiple of 8)
+        const uint2* cb4 = (const uint2*)b.cb;
+        const int nvec = a.L * E / 4;   // the library in vectors of four entries: all of an odd number of codebooks at N = 2 too
         int differs = !have_tables;
         if (have_tables)
             for (int i = threadIdx.x; i < nvec; i += kAThreads) {
-                const uint4 u = __ldg(cb4 + i), v = libcopy[i];
-                differs |= (u.x != v.x) | (u.y != v.y) | (u.z != v.z) | (u.w != v.w);
+                const uint2 u = __ldg(cb4 + i), v = libcopy[i];
+                differs |= (u.x != v.x) | (u.y != v.y);
             }
         // (also the barrier behind which the previous item's sums and flag may be overwritten)
         if (__syncthreads_or(differs)) {

@@ -637,6 +637,43 @@ def test_fused_stores_over_blobs_with_libraries_of_their_own(bits, n, rows, cols
     assert int(ws[:4 * ((rows + 31) // 32) * n].view(torch.int32).abs().sum().item()) == 0
 
 
+@pytest.mark.parametrize("epilogue", [xfp.XFP_EPI_SWIGLU, xfp.XFP_EPI_COMBINE])
+def test_fused_stores_of_blobs_whose_libraries_differ_in_the_last_codebook(epilogue):
+    """N = 2 with seven codebooks (56 bytes, no multiple of 16) and rows of x too long for the expert kernel: more blobs than the launch
+    has CTAs, so that some meet a second blob, whose library is that of the first but for its last codebook."""
+    rows, cols, n = 64, 65536, 420
+    qa = synth.random_quantized(1, rows, cols, 2, 0.0, seed=2700, lib_size=7)
+    book = qa.codebook.copy()
+    book[6] = book[6][::-1]
+    qb = synth.QuantTensors(**{**qa.__dict__, "codebook": book})
+    pms = [xfp.pack_tensors(q, col_bits=16) for q in (qa, qb)]
+    which = [0] * 300 + [1] * (n - 300)
+    d = pms[0].desc
+    x16 = synth.activations(1, cols, seed=2701)
+    xd = _x_dev(x16)
+    ptr = lambda ts: torch.tensor([t.data_ptr() for t in ts], dtype=torch.int64, device="cuda")
+    ws = torch.zeros(n * xfp.xfp_packed_size(d)[1], dtype=torch.uint8, device="cuda")
+    refs = [xo.gemv(to_oracle(q), x16) for q in (qa, qb)]
+    if epilogue == xfp.XFP_EPI_SWIGLU:
+        h = torch.empty((n, rows // 2), dtype=torch.float32, device="cuda")
+        xfp.xfp_gemv_grouped_epilogue(d, n, ptr([pms[w].packed for w in which]), ptr([xd] * n), ptr([h[j] for j in range(n)]), False,
+                                      epilogue, None, ws)
+        got = h.cpu().numpy().astype(np.float64)
+        for j, w in enumerate(which):
+            ref, absum = refs[w]
+            g, u, eg, eu = ref[0][:32], ref[0][32:], TOL * absum[0][:32], TOL * absum[0][32:]
+            lim = 1.1 * np.abs(u) * eg + np.abs(g / (1.0 + np.exp(-g))) * eu + 1.1 * eg * eu + 2.0 ** -20 * np.abs(g * u) + 1e-30
+            assert np.all(np.abs(got[j] - xo.silu_mul(g, u)) <= lim), j
+    else:
+        wts = torch.from_numpy(np.random.default_rng(2702).uniform(0.5, 1.5, n).astype(np.float32)).cuda()
+        wts[:300] = 0.0                    # the blobs of the second library carry the sum
+        y = torch.empty(rows, dtype=torch.float32, device="cuda")
+        xfp.xfp_gemv_grouped_epilogue(d, n, ptr([pms[w].packed for w in which]), ptr([xd] * n), ptr([y] * n), False, epilogue, wts, ws)
+        total = wts[300:].double().cpu().numpy()
+        want, bound = total.sum() * refs[1][0][0], total.sum() * refs[1][1][0]
+        assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - want) <= TOL * bound + 1e-30)
+
+
 @pytest.mark.parametrize("mode,bits", [(0, 4), (1, 3), (1, 6)])
 @pytest.mark.parametrize("half", [0, 1])
 def test_grouped_c_functions_of_the_abi(mode, bits, half):
