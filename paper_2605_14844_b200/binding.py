@@ -339,8 +339,10 @@ def pack_tensors(q, device="cuda", col_bits: int = 32, stream=None) -> PackedMat
         last, arrived = _read_back(device.index)
         last.copy_(q.rowptr[-1:], non_blocking=True)
         arrived.record()
-        pm = pack(n)
-        arrived.synchronize()
+        try:
+            pm = pack(n)
+        finally:
+            arrived.synchronize()       # whatever ends this call: the next one uses the same word, perhaps on another stream
         nnz = last.item()
         return pm if nnz == n else pack(nnz)
     return pack(int(q.rowptr[-1]))

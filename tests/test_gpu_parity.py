@@ -304,6 +304,21 @@ def test_pack_tensors_takes_the_count_from_the_row_pointers(spare, least, monkey
     assert int(pm.err_word.item()) == 0 and int(pm.workspace.abs().sum().item()) == 0
 
 
+def test_pack_tensors_waits_for_the_count_when_a_pack_fails(monkeypatch):
+    """The count on its way to the host has arrived before pack_tensors ends, whatever ends it: the next call, on another stream,
+    uses the same word."""
+    monkeypatch.setattr(binding, "_SPECULATE", 0)
+    q = synth.random_quantized_torch(0, 70, 640, 4, 0.02, seed=8310)
+
+    def fails(*args, **kwargs):
+        raise xfp.XfpError("refused")
+    monkeypatch.setattr(binding, "xfp_pack", fails)
+    torch.cuda._sleep(40_000_000)                      # about 20 ms before the copy of the count
+    with pytest.raises(xfp.XfpError):
+        xfp.pack_tensors(q)
+    assert binding._read_back(torch.cuda.current_device())[1].query()
+
+
 def test_adversarial_activations():
     q = synth.random_quantized(0, 64, 1024, 4, 0.01, seed=91)
     qa = synth.random_quantized(1, 64, 1024, 3, 0.01, seed=92)
