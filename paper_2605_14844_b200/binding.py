@@ -314,6 +314,8 @@ def pack_tensors(q, device="cuda", col_bits: int = 32, stream=None) -> PackedMat
         ocol = q.ocol.astype(np.uint16) if col_bits == 16 else q.ocol.astype(np.int32)
         ocol = _dev(ocol, torch.int16 if col_bits == 16 else torch.int32, device)
     oval = _dev(q.oval, torch.int16, device)
+    # filled on the current stream before the wait for the count: a pack on another stream may set bits in it at once
+    err = torch.zeros(1, dtype=torch.int32, device=device) if stream is not None else None
 
     def pack(nnz):
         desc = XfpDesc(q.mode, q.rows, q.cols, q.bits, q.group_size, q.lib_size if q.mode else 0, col_bits, nnz)
@@ -321,9 +323,9 @@ def pack_tensors(q, device="cuda", col_bits: int = 32, stream=None) -> PackedMat
         wb = -(-max(wb, 16) // 16) * 16
         packed = torch.empty(pb, dtype=torch.uint8, device=device)
         zeros = torch.zeros(wb + 16, dtype=torch.uint8, device=device)      # the workspace and the error word, in one fill
-        err = zeros[wb:wb + 4].view(torch.int32)
-        xfp_pack(desc, idx, cb, gid, gs, gm, rowptr, ocol, oval, packed, err, stream)
-        return PackedMatrix(desc, packed, zeros[:wb], err)
+        word = zeros[wb:wb + 4].view(torch.int32) if err is None else err
+        xfp_pack(desc, idx, cb, gid, gs, gm, rowptr, ocol, oval, packed, word, stream)
+        return PackedMatrix(desc, packed, zeros[:wb], word)
 
     # The count of outliers is the last row pointer.  Where that lives on the device, the matrix is packed for the count that the
     # entry arrays hold while the pointer travels to the host, and once more in the rare case that they hold others behind it: the

@@ -319,6 +319,24 @@ def test_pack_tensors_waits_for_the_count_when_a_pack_fails(monkeypatch):
     assert binding._read_back(torch.cuda.current_device())[1].query()
 
 
+def test_pack_tensors_on_another_stream_reports_bad_indices(monkeypatch):
+    """The error word is zero before the pack on the caller's stream writes to it."""
+    q = synth.random_quantized_torch(0, 70, 640, 4, 0.02, seed=8320)
+    side = torch.cuda.Stream()
+    xfp.pack_tensors(q, stream=side)                   # a kernel's first launch may wait for the device
+    q.idx[3, 5] = 200
+    torch.cuda.synchronize()
+    zeros = torch.zeros
+
+    def late(*args, **kwargs):
+        torch.cuda._sleep(40_000_000)                  # about 20 ms in front of the fill
+        return zeros(*args, **kwargs)
+    monkeypatch.setattr(torch, "zeros", late)
+    pm = xfp.pack_tensors(q, stream=side)
+    torch.cuda.synchronize()
+    assert int(pm.err_word.item()) == 1
+
+
 def test_adversarial_activations():
     q = synth.random_quantized(0, 64, 1024, 4, 0.01, seed=91)
     qa = synth.random_quantized(1, 64, 1024, 3, 0.01, seed=92)
