@@ -92,7 +92,7 @@ def _native():
             raise XfpError(f"_xfp_native.so: {e}: run `python -m paper_2605_14844_b200.build`") from e
         native.bind(*[C.cast(getattr(lib, n), C.c_void_p).value for n in
                       ("xfp_pack", "xfp_gemv_v2", "xfp_gemv_v2a", "xfp_gemv_typed", "xfp_gemv_grouped_typed",
-                       "xfp_gemv_host", "xfp_gemv_v2_noalloc", "xfp_gemm_typed", "xfp_dequant")])
+                       "xfp_gemv_host", "xfp_gemv_v2_noalloc", "xfp_gemm_typed", "xfp_dequant", "xfp_pack_counted")])
         _NATIVE = native
     return _NATIVE
 
@@ -127,6 +127,13 @@ def xfp_pack(desc: XfpDesc, idx, codebook, group_id, group_scale, group_mid, out
              packed: torch.Tensor, err_word: Optional[torch.Tensor] = None, stream=None) -> None:
     status = (_NATIVE or _native()).pack(desc, idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, out_val,
                                          packed, err_word, stream)
+    if status:
+        _check(status, "xfp_pack")
+
+
+def _pack_counted(*args) -> None:
+    """xfp_pack for a count not read back yet: the GPU leaves the blob alone where the last row pointer is another."""
+    status = (_NATIVE or _native()).pack_counted(*args)
     if status:
         _check(status, "xfp_pack")
 
@@ -317,34 +324,49 @@ def pack_tensors(q, device="cuda", col_bits: int = 32, stream=None) -> PackedMat
     # filled on the current stream before the wait for the count: a pack on another stream may set bits in it at once
     err = torch.zeros(1, dtype=torch.int32, device=device) if stream is not None else None
 
-    def pack(nnz):
+    def blob(nnz, zeros=None):
         desc = XfpDesc(q.mode, q.rows, q.cols, q.bits, q.group_size, q.lib_size if q.mode else 0, col_bits, nnz)
         pb, wb = xfp_packed_size(desc)
-        wb = -(-max(wb, 16) // 16) * 16
-        packed = torch.empty(pb, dtype=torch.uint8, device=device)
-        zeros = torch.zeros(wb + 16, dtype=torch.uint8, device=device)      # the workspace and the error word, in one fill
-        word = zeros[wb:wb + 4].view(torch.int32) if err is None else err
-        xfp_pack(desc, idx, cb, gid, gs, gm, rowptr, ocol, oval, packed, word, stream)
-        return PackedMatrix(desc, packed, zeros[:wb], word)
+        wb = -(-max(wb, 16) // 16) * 16 + 16
+        if zeros is None or zeros.numel() != wb:
+            zeros = torch.zeros(wb, dtype=torch.uint8, device=device)       # the workspace and the error word, in one fill
+        return desc, torch.empty(pb, dtype=torch.uint8, device=device), zeros
+
+    def pack(entry, desc, packed, zeros):
+        word = zeros[-16:-12].view(torch.int32) if err is None else err
+        entry(desc, idx, cb, gid, gs, gm, rowptr, ocol, oval, packed, word, stream)
+        return PackedMatrix(desc, packed, zeros[:-16], word)
 
     # The count of outliers is the last row pointer.  Where that lives on the device, the matrix is packed for the count that the
-    # entry arrays hold while the pointer travels to the host, and once more in the rare case that they hold others behind it: the
-    # GPU does not idle for the host's wait (12289 x 4096 V2a, pack and dequant: 94 -> 73 us with the kernels as they are).  On the
-    # current stream only: work for another one is complete when the wait for the pointer is over, not before.  Below _SPECULATE
-    # weights the host, not the GPU, sets the time, and the plain wait is the shorter way (1419 x 3072: 62 us; 83 with the first
-    # form of this).
+    # entry arrays hold while the pointer travels to the host: the GPU does not idle for the host's wait.  Entries behind the last row
+    # pointer cost a launch that ends at once; arrays that hold more than one weight of 32 are taken for capacities, and nothing is
+    # allocated for them.  On the current stream only: work for another one is complete when the wait for the pointer is over, not
+    # before.  us for pack and dequant, plain wait -> this, calls behind one another / a call alone (the saving is an overlap, which
+    # a lone call does not have): 12289 x 4096 V2a N = 4 88 -> 73 / 104 -> 105, 8200 x 4096 73 -> 56 / 87 -> 89, 28672 x 8192 V2
+    # 225 -> 213 / 240 -> 243; with 1000 spare entries 12289 x 4096 88 -> 86 / 104 -> 125, 28672 x 8192 225 -> 225 / 239 -> 264.
+    # Below _SPECULATE weights, twice as many without outliers, the host sets the time and not the GPU: 4096 x 4096 49 -> 51 /
+    # 64 -> 69, 1419 x 3072 48 -> 59 / 62 -> 82, 8200 x 4096 V2 N = 2 without outliers 62 -> 67 / 84 -> 87 (6016 x 4096 61 -> 53 /
+    # 76 -> 78).
     n = q.ocol.numel() if isinstance(q.ocol, torch.Tensor) and isinstance(q.oval, torch.Tensor) else -1
-    if (stream is None and q.rows * q.cols >= _SPECULATE and isinstance(q.rowptr, torch.Tensor) and q.rowptr.is_cuda
+    if (stream is None and q.rows * q.cols >= _SPECULATE * (1 if n else 2) and isinstance(q.rowptr, torch.Tensor) and q.rowptr.is_cuda
             and q.rowptr.dim() == 1 and q.rowptr.dtype == torch.int32 and rowptr.numel() == q.rows + 1
             and device.index == torch.cuda.current_device() and q.rowptr.device == device
-            and 0 <= n <= min(q.rows * q.cols, 2 ** 31 - 1) and q.oval.numel() == n):
+            and 0 <= n <= min(q.rows * q.cols // 32, 2 ** 31 - 1) and q.oval.numel() == n):
         last, arrived = _read_back(device.index)
         last.copy_(q.rowptr[-1:], non_blocking=True)
         arrived.record()
+        made = done = None
         try:
-            pm = pack(n)
+            made = blob(n)
+            done = pack(_pack_counted, *made)
+        except RuntimeError:            # no memory for spare entries, or what is refused below as well
+            pass
         finally:
             arrived.synchronize()       # whatever ends this call: the next one uses the same word, perhaps on another stream
         nnz = last.item()
-        return pm if nnz == n else pack(nnz)
-    return pack(int(q.rowptr[-1]))
+        if nnz == n and done:
+            return done
+        zeros = made[2] if made else None
+        made = done = None
+        return pack(xfp_pack, *blob(nnz, zeros))
+    return pack(xfp_pack, *blob(int(q.rowptr[-1])))

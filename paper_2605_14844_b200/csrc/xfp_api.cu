@@ -156,20 +156,37 @@ int xfp_packed_size(const xfp_desc* desc, size_t* packed_bytes, size_t* workspac
     return XFP_OK;
 }
 
-int xfp_pack(const xfp_desc* desc, const uint8_t* idx, const uint16_t* codebook, const uint8_t* group_id,
-             const uint16_t* group_scale, const uint16_t* group_mid, const int32_t* out_rowptr, const void* out_col,
-             const uint16_t* out_val, void* packed, size_t packed_bytes, int32_t* err_word, void* stream) {
+static int pack_common(const xfp_desc* desc, const uint8_t* idx, const uint16_t* codebook, const uint8_t* group_id,
+                       const uint16_t* group_scale, const uint16_t* group_mid, const int32_t* out_rowptr, const void* out_col,
+                       const uint16_t* out_val, void* packed, size_t packed_bytes, int32_t* err_word, void* stream, bool counted) {
     int st = check_desc(desc);
     if (st) return st;
     if (!idx || !codebook || !packed) return XFP_ERR_NULL;
     if (desc->mode == 1 && (!group_id || !group_scale || !group_mid)) return XFP_ERR_NULL;
     if (desc->nnz > 0 && (!out_rowptr || !out_col || !out_val)) return XFP_ERR_NULL;
+    if (counted && !out_rowptr) return XFP_ERR_NULL;
     if (!aligned16(idx) || !aligned16(codebook) || !aligned16(packed)) return XFP_ERR_ALIGN;
     if (err_word && (reinterpret_cast<uintptr_t>(err_word) & 3u)) return XFP_ERR_ALIGN;
     const Layout l = layout_of(desc);
     if (packed_bytes < l.total) return XFP_ERR_BUFFER_TOO_SMALL;
     PackInputs in{idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, desc->col_bits, out_val};
-    return launch_pack(l, in, packed, err_word, (cudaStream_t)stream) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+    return launch_pack(l, in, packed, err_word, (cudaStream_t)stream, counted) == cudaSuccess ? XFP_OK : XFP_ERR_CUDA;
+}
+
+int xfp_pack(const xfp_desc* desc, const uint8_t* idx, const uint16_t* codebook, const uint8_t* group_id,
+             const uint16_t* group_scale, const uint16_t* group_mid, const int32_t* out_rowptr, const void* out_col,
+             const uint16_t* out_val, void* packed, size_t packed_bytes, int32_t* err_word, void* stream) {
+    return pack_common(desc, idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, out_val, packed, packed_bytes,
+                       err_word, stream, false);
+}
+
+// For the Python binding, not part of the API: xfp_pack for a count that the caller has not read yet.  Where the last row pointer
+// turns out to be another than desc->nnz, the kernel ends at once and leaves blob and error word as they are.
+int xfp_pack_counted(const xfp_desc* desc, const uint8_t* idx, const uint16_t* codebook, const uint8_t* group_id,
+                     const uint16_t* group_scale, const uint16_t* group_mid, const int32_t* out_rowptr, const void* out_col,
+                     const uint16_t* out_val, void* packed, size_t packed_bytes, int32_t* err_word, void* stream) {
+    return pack_common(desc, idx, codebook, group_id, group_scale, group_mid, out_rowptr, out_col, out_val, packed, packed_bytes,
+                       err_word, stream, true);
 }
 
 int xfp_gemv_v2(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t batch, void* y,

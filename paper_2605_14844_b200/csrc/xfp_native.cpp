@@ -23,6 +23,7 @@ struct Entry {
     decltype(&xfp_gemv_v2_noalloc) noalloc;
     decltype(&xfp_gemm_typed) gemm_typed;
     decltype(&xfp_dequant) dequant;
+    decltype(&xfp_pack) pack_counted;
 } g;
 
 // One call's arguments; the first problem sets a Python exception and `bad`.
@@ -250,7 +251,7 @@ PyObject* dequant(PyObject*, PyObject* const* args, Py_ssize_t n) {
 }
 
 // (desc, idx, codebook, gid, gscale, gmid, rowptr, ocol, oval, packed, err_word, stream)
-PyObject* pack(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* pack_by(decltype(&xfp_pack) f, PyObject* const* args, Py_ssize_t n) {
     Args a(args, n, 12);
     const xfp_desc d = a.desc(0);
     void* p[8];
@@ -260,13 +261,15 @@ PyObject* pack(PyObject*, PyObject* const* args, Py_ssize_t n) {
     int32_t* err = (int32_t*)a.ptr(10);
     void* s = a.stream(11);
     return call(a, [&] {
-        return g.pack(&d, (const uint8_t*)p[0], (const uint16_t*)p[1], (const uint8_t*)p[2], (const uint16_t*)p[3],
-                      (const uint16_t*)p[4], (const int32_t*)p[5], p[6], (const uint16_t*)p[7], packed, bytes, err, s);
+        return f(&d, (const uint8_t*)p[0], (const uint16_t*)p[1], (const uint8_t*)p[2], (const uint16_t*)p[3],
+                 (const uint16_t*)p[4], (const int32_t*)p[5], p[6], (const uint16_t*)p[7], packed, bytes, err, s);
     });
 }
+PyObject* pack(PyObject*, PyObject* const* args, Py_ssize_t n) { return pack_by(g.pack, args, n); }
+PyObject* pack_counted(PyObject*, PyObject* const* args, Py_ssize_t n) { return pack_by(g.pack_counted, args, n); }
 
 // bind(addresses of xfp_pack, xfp_gemv_v2, xfp_gemv_v2a, xfp_gemv_typed, xfp_gemv_grouped_typed, xfp_gemv_host,
-//      xfp_gemv_v2_noalloc, xfp_gemm_typed, xfp_dequant)
+//      xfp_gemv_v2_noalloc, xfp_gemm_typed, xfp_dequant, xfp_pack_counted)
 PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void** slot = (void**)&g;
     constexpr Py_ssize_t kSlots = sizeof g / sizeof(void*);
@@ -281,6 +284,7 @@ PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
 #define XFP_METHOD(f) {#f, (PyCFunction)(void*)f, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {XFP_METHOD(bind), XFP_METHOD(gemv), XFP_METHOD(gemv_typed), XFP_METHOD(grouped), XFP_METHOD(gemm),
                          XFP_METHOD(gemv_host), XFP_METHOD(noalloc), XFP_METHOD(dequant), XFP_METHOD(pack),
+                         XFP_METHOD(pack_counted),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_xfp_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

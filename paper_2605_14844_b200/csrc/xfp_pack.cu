@@ -22,6 +22,7 @@ struct PackArgs {
     char* base;             // the blob
     Layout l;
     int* err_word;
+    bool counted;           // nothing is written when the last row pointer is not l.nnz
     // first block of every part, in this order: slabs, entries, rowptr, group, codebook, idx; [6] = grid.  (Spreading
     // the blocks of the small parts evenly among those of the index part measured the same: 110.6 against 106.5 us at
     // 28672 x 8192 with 2 % outliers.)
@@ -239,6 +240,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackArgs a) {
     __shared__ __align__(16) unsigned char tiles[kPackWarps * 32 * 144];   // 36864 bytes; the slab part uses 33792 + 132
     static_assert(kPackWarps * 32 * 144 >= kEllWindow * 33 * 4 + 33 * 4, "slab window and row pointers fit the tile area");
     const unsigned b = blockIdx.x;
+    if (a.counted && __ldg(a.in.rowptr + a.l.rows) != a.l.nnz) return;
     if (b < a.first[1]) ell_fill_block(a, b, tiles);
     else if (b < a.first[2]) pack_entries_block(a, b - a.first[1]);
     else if (b < a.first[3]) pack_rowptr_block(a, b - a.first[2]);
@@ -247,9 +249,9 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const PackArgs a) {
     else pack_idx_block<N>(a, b - a.first[5], tiles);
 }
 
-cudaError_t launch_pack(const Layout& l, const PackInputs& in, void* packed, int* err_word, cudaStream_t s) {
+cudaError_t launch_pack(const Layout& l, const PackInputs& in, void* packed, int* err_word, cudaStream_t s, bool counted) {
     PackArgs a;
-    a.in = in; a.base = (char*)packed; a.l = l; a.err_word = err_word;
+    a.in = in; a.base = (char*)packed; a.l = l; a.err_word = err_word; a.counted = counted;
     auto blocks = [](long long n, int per) { return (unsigned)((n + per - 1) / per); };
     const long long n_cb = (long long)(l.mode ? l.L : l.rows_pad) * l.E;
     unsigned n[6];

@@ -313,10 +313,39 @@ def test_pack_tensors_waits_for_the_count_when_a_pack_fails(monkeypatch):
     def fails(*args, **kwargs):
         raise xfp.XfpError("refused")
     monkeypatch.setattr(binding, "xfp_pack", fails)
+    monkeypatch.setattr(binding, "_pack_counted", fails)
     torch.cuda._sleep(40_000_000)                      # about 20 ms before the copy of the count
     with pytest.raises(xfp.XfpError):
         xfp.pack_tensors(q)
     assert binding._read_back(torch.cuda.current_device())[1].query()
+
+
+def test_pack_tensors_packs_once(monkeypatch):
+    """Entries behind the last row pointer: the pack for the count that the arrays hold writes nothing, and one that has no memory
+    is left out.  Arrays of another order of size are not packed for at all."""
+    monkeypatch.setattr(binding, "_SPECULATE", 0)
+    q = synth.random_quantized_torch(0, 70, 640, 4, 0.02, seed=8330)
+    want = xfp.pack_tensors(q)
+    more = lambda k: synth.QuantTensors(**{**q.__dict__, "ocol": torch.cat([q.ocol, q.ocol.new_full((k,), 3)]),
+                                           "oval": torch.cat([q.oval, q.oval.new_ones(k)])})
+    seen, counted = [], binding._pack_counted
+
+    def watched(desc, *args):
+        packed, err = args[8], args[9]
+        packed.fill_(0x5a)
+        counted(desc, *args)
+        seen.append((int(desc.nnz), bool((packed == 0x5a).all()), int(err.item())))
+    monkeypatch.setattr(binding, "_pack_counted", watched)
+    for spare in (0, 1, 100):
+        pm = xfp.pack_tensors(more(spare))
+        assert seen.pop() == (want.desc.nnz + spare, spare > 0, 0) and pm.desc.nnz == want.desc.nnz
+        assert torch.equal(pm.dequant(), want.dequant()) and int(pm.err_word.item()) == 0 and int(pm.workspace.max().item()) == 0
+    assert xfp.pack_tensors(more(70 * 640 // 32)).desc.nnz == want.desc.nnz and not seen
+
+    def no_memory(*args):
+        raise torch.OutOfMemoryError("no memory")
+    monkeypatch.setattr(binding, "_pack_counted", no_memory)
+    assert torch.equal(xfp.pack_tensors(more(1)).dequant(), want.dequant())
 
 
 def test_pack_tensors_on_another_stream_reports_bad_indices(monkeypatch):
