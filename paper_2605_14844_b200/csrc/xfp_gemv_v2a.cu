@@ -11,7 +11,7 @@
 // Look-up.  Every lane may need a different library codebook, so tables cannot be private to a channel as in the V2 kernel.
 //   * N <= 4: the library sits in shared memory once, as byte planes (a few KB); a lane loads the codebook of its channel's
 //     group into registers and decodes with PRMTs (xfp_reg_decode.cuh).  There is no table to fill.
-//   * N = 5: the library replicated once per bank: word (id * 2^N + q) * 32 + lane holds lib[id][q] (fp16 in the low half).
+//   * N = 5, and N = 4 at two rows of x (see v2a_config): the library replicated once per bank: word (id * 2^N + q) * 32 + lane holds lib[id][q] (fp16 in the low half).
 //     Lane l only touches bank l; one look-up decodes one weight and a multiply-add joins two of them.
 //
 // Multiply-accumulate.  The half2 of a lane's two channels form the A fragment of
@@ -53,7 +53,6 @@ struct V2aArgs {
     int items_x, n;   // work items per blob (whole blocks + K slices), blobs
     int epi;                 // 0 plain store; 1 SiLU(gate) * up inside every 64-channel block; 2 weighted sum over the blobs
     const float* epi_w;      // epi 2: [n] weights
-    int comb_G, comb_ng;     // epi 2: runs per block of channels, blobs per run
     int persist;             // resident CTAs walk the items
 };
 
@@ -81,12 +80,11 @@ __device__ __forceinline__ uint32_t entry_addr(const uint32_t* w, int j, uint32_
     return (v & mask) | base;
 }
 
-// FEAT instantiations carry typed IO (bf16 x, bf16 y) and the fused stores; the plain ones compile them out.
-template <int N, int NB, int W, bool FEAT>
+// FEAT: 1 typed IO (bf16 x, bf16 y), 2 typed IO and the fused stores (one row of x), 0 neither.  REG: codebooks in registers, no tables.
+template <int N, int NB, int W, int FEAT, bool REG>
 __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const V2aArgs a) {
-    const int epi = FEAT ? a.epi : 0;
+    const int epi = FEAT == 2 ? a.epi : 0;
     constexpr int E = 1 << N;
-    constexpr bool kReg = N <= 4;
     constexpr int kAWarps = W;
     constexpr int kAThreads = W * 32;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -94,14 +92,14 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     asm volatile("griddepcontrol.launch_dependents;");
     const int K = a.SC * kSuper;
-    const int tab_bytes = kReg ? (a.L * E * 2 + 15) & ~15 : a.L * E * 128;
+    const int tab_bytes = REG ? (a.L * E * 2 + 15) & ~15 : a.L * E * 128;
     unsigned char* tab = smem;
     uint16_t* xs = (uint16_t*)(smem + tab_bytes);             // [NB][K]
     float* xg = (float*)(xs + (size_t)NB * K);                // [NB][SC]
     float* red = xg + NB * a.SC;                              // [W][NB][64]
     __shared__ int s_last;
     // where activation k sits in the staged copy
-    auto xat = [](uint32_t k) { return N == 2 ? (k & ~7u) | ((k & 1u) << 2) | ((k & 7u) >> 1) : k; };
+    auto xat = [](uint32_t k) { return REG && N == 2 ? (k & ~7u) | ((k & 1u) << 2) | ((k & 7u) >> 1) : k; };
 
     // the library the tables were built from, on the next 16-byte boundary (NB * SC floats of xg precede red)
     uint2* libcopy = (uint2*)(((uintptr_t)(red + (size_t)kAWarps * NB * kARows) + 15) & ~(uintptr_t)15);
@@ -109,25 +107,21 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     bool waited = false;
     const uint16_t* x_staged = nullptr;
 
-    // ---- work items: (blob, whole block or K slice of a block), dealt round-robin to the CTAs of the launch
-    // The weighted sum over the blobs (epi 2) deals RUNS instead: a CTA takes comb_ng consecutive blobs of
-    // one block of channels and adds their weighted results in registers; only the comb_G runs of a block
-    // meet in the scratch (none when one run covers all blobs).
-    const int per = epi == 2 ? a.comb_ng : 1;
-    const int nrun = epi == 2 ? a.blocks * a.comb_G : a.items_x * a.n;
-    float csum = 0.f;   // epi 2: this thread's channel, weighted sum over the blobs of the run
-    int run = blockIdx.x, jj = 0;
-    if (run >= nrun) return;
+    // ---- work items: (blob, whole block or K slice of a block), dealt round-robin to the CTAs of the launch.  Where the blobs'
+    // weighted sum is asked for (epi 2) the blobs of a block follow one another: they meet in the scratch.
+    const int items = a.items_x * a.n;
+    int at = blockIdx.x;
+    if (at >= items) return;
     // where an item lies: blob, block, K slice
     struct Item { int prob, bx, blk, ks, KS, sc0, nsc; };
-    auto locate = [&](int run_, int jj_) {
+    auto locate = [&](int i) {
         Item t;
         if (epi == 2) {
-            t.bx = run_ / a.comb_G;
-            t.prob = (run_ - t.bx * a.comb_G) * a.comb_ng + jj_;
+            t.bx = i / a.n;
+            t.prob = i - t.bx * a.n;
         } else {
-            t.prob = run_ / a.items_x;
-            t.bx = run_ - t.prob * a.items_x;
+            t.prob = i / a.items_x;
+            t.bx = i - t.prob * a.items_x;
         }
         int spp;
         if (t.bx < a.n_full) {
@@ -189,26 +183,24 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
             }
         }
     };
-    Item item = locate(run, 0);
+    Item item = locate(at);
     open(item.prob, packed, ell, ell_slots);
     issue(item, packed, ell, ell_slots);
 #pragma unroll 1
     for (;;) {
-    const int prob = item.prob, bx = item.bx, blk = item.blk, ks = item.ks, KS = item.KS, sc0 = item.sc0, nsc = item.nsc;
-    if (jj == 0) csum = 0.f;
+    const int prob = item.prob, blk = item.blk, ks = item.ks, KS = item.KS, sc0 = item.sc0, nsc = item.nsc;
     const float epi_wj = epi == 2 ? __ldg(a.epi_w + prob) : 0.f;   // fetched now, used in the store
     const uint16_t* x = a.x_list ? a.x_list[prob] : a.x;
     void* y = a.y_list ? a.y_list[prob] : a.y;
     const Blob b = blob_at(packed, a.off);
     // the CTA's next item: its pointers travel under this one's K loop, its first loads under this one's reduction (an item is
     // two groups per warp on the routed experts' shapes, and the chain pointer - header - slab cost as much as one of them)
-    const bool same_run = epi == 2 && jj + 1 < per && prob + 1 < a.n;
-    const int run_n = same_run ? run : run + (int)gridDim.x, jj_n = same_run ? jj + 1 : 0;
-    const bool more = a.persist && run_n < nrun;
+    const int at_n = at + (int)gridDim.x;
+    const bool more = a.persist && at_n < items;
     Item item_n = item;
     const void* packed_n = packed; const uint32_t* ell_n = ell; int slots_n = ell_slots;
     if (more) {
-        item_n = locate(run_n, jj_n);
+        item_n = locate(at_n);
         open(item_n.prob, packed_n, ell_n, slots_n);
     }
     const int blk0 = 2 * blk;
@@ -266,7 +258,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
         if (__syncthreads_or(differs)) {
             fresh = true;
             for (int i = threadIdx.x; i < nvec; i += kAThreads) libcopy[i] = __ldg(cb4 + i);
-            if constexpr (kReg) {
+            if constexpr (REG) {
                 for (int id = threadIdx.x; id < a.L; id += kAThreads) store_book<N>(tab, a.L, id, make_book<N>(b.cb + (size_t)id * E));
             } else {
                 // one copy per bank: word (e * 32 + lane) = lib[e] for every lane.  A lane fetches entry e0 + lane, the warp
@@ -298,7 +290,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
                 if (bb < a.nb) v = __ldg((const uint4*)(x + (size_t)bb * a.cols + kk));
                 if (FEAT) v = x8_as_f16(v, a.x_bf16);
-                if (N == 2)   // the even k of every eight, then the odd ones: the order in which two steps decode them
+                if (REG && N == 2)   // the even k of every eight, then the odd ones: the order in which two steps decode them
                     v = make_uint4(prmt(v.x, v.y, 0x5410u), prmt(v.z, v.w, 0x5410u), prmt(v.x, v.y, 0x7632u), prmt(v.z, v.w, 0x7632u));
                 *(uint4*)(xs + (size_t)t * 8) = v;
             }
@@ -337,7 +329,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     const int src0 = (lane & ~3) | (t4 >> 1);
     const bool odd = t4 & 1;
 
-    RegBook<kReg ? N : 2> book0, book1;
+    RegBook<REG ? N : 2> book0, book1;
     auto lookup = [&](uint32_t (&f)[4], int m, uint32_t base0, uint32_t base1) {
         const uint32_t l00 = *(const uint32_t*)(tab + entry_addr<N>(w0, 4 * m + 0, base0));
         const uint32_t l01 = *(const uint32_t*)(tab + entry_addr<N>(w0, 4 * m + 1, base0));
@@ -366,7 +358,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
             if (++oround < nrounds) fetch_slots(oround);
         }
         const uint32_t base0 = id0 * (uint32_t)(E * 128) + (uint32_t)lane * 4u, base1 = id1 * (uint32_t)(E * 128) + (uint32_t)lane * 4u;
-        if constexpr (kReg) { book0 = load_book<N>(tab, a.L, id0); book1 = load_book<N>(tab, a.L, id1); }
+        if constexpr (REG) { book0 = load_book<N>(tab, a.L, id0); book1 = load_book<N>(tab, a.L, id1); }
         const unsigned char* xp = xrow + (size_t)s * (kSuper * 2);
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
         uint4 xa = make_uint4(0u, 0u, 0u, 0u), xb = make_uint4(0u, 0u, 0u, 0u);
@@ -383,7 +375,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
                 }
             }
         };
-        if constexpr (kReg) {
+        if constexpr (REG) {
             // eight weights of both channels at a time, one batch ahead of the tensor pipe
             uint32_t p0[4], p1[4], q0[4], q1[4];
             reg_decode8<N>(p0, w0, 0, book0);
@@ -502,7 +494,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
     }
     if (epi == 0) {
         if (writer && active && !dup && bb < a.nb && row < a.rows) {
-            store_y<FEAT>(y, (size_t)bb * a.rows + row, total, a.y_is_fp16);
+            store_y<FEAT != 0>(y, (size_t)bb * a.rows + row, total, a.y_is_fp16);
         }
     } else if (epi == 1) {
         // gated activation of a routed expert: channels 0..31 of the block are gates, 32..63 the matching
@@ -519,45 +511,33 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
             }
         }
     } else {
-        // weighted sum over the blobs of the launch (the routed experts' down projections)
-        if (t < kARows) csum = fmaf(epi_wj, total, csum);
-        const bool run_done = jj == per - 1 || prob == a.n - 1;
-        if (run_done && a.comb_G == 1) {
-            if (t < kARows && !dup && row < a.rows) {
-                void* y0 = a.y_list ? a.y_list[0] : a.y;
-                put_y(y0, row, csum, a.y_is_fp16);
-            }
-        } else if (run_done) {
-            // the runs of this block leave their sums in the scratch, the last one to arrive adds them in run order
-            float* comb = a.partial;            // [run of the block][rows_ws]; the K-split scratch is idle in these launches
-            int* ticket = a.tickets + blk;      // one counter per block of channels
-            const int g = run - bx * a.comb_G;
-            if (t < kARows) comb[(size_t)g * a.rows_ws + row] = csum;
+        // weighted sum over the blobs of the launch (the routed experts' down projections): they leave their terms in the scratch
+        // (the K-split scratch is idle in these launches), the last one of the block to arrive adds them in blob order
+        int* ticket = a.tickets + blk;      // one counter per block of channels
+        if (t < kARows) a.partial[(size_t)prob * a.rows_ws + row] = epi_wj * total;
+        __threadfence();
+        __syncthreads();
+        if (t == 0) s_last = (atomicAdd(ticket, 1) == a.n - 1);
+        __syncthreads();
+        if (s_last) {
             __threadfence();
-            __syncthreads();
-            if (t == 0) s_last = (atomicAdd(ticket, 1) == a.comb_G - 1);
-            __syncthreads();
-            if (s_last) {
-                __threadfence();
-                if (t < kARows && !dup && row < a.rows) {
-                    float sum = 0.f;
-                    for (int g2 = 0; g2 < a.comb_G; ++g2) sum += __ldcg(comb + (size_t)g2 * a.rows_ws + row);
-                    void* y0 = a.y_list ? a.y_list[0] : a.y;
-                    put_y(y0, row, sum, a.y_is_fp16);
-                }
-                if (t == 0) *ticket = 0;
+            if (t < kARows && !dup && row < a.rows) {
+                float sum = 0.f;
+                for (int j = 0; j < a.n; ++j) sum += __ldcg(a.partial + (size_t)j * a.rows_ws + row);
+                put_y(a.y_list ? a.y_list[0] : a.y, row, sum, a.y_is_fp16);
             }
+            if (t == 0) *ticket = 0;
         }
     }
-    if (!more) break;   // (the per-bank library may be launched with one CTA per item)
-    item = item_n; packed = packed_n; ell = ell_n; ell_slots = slots_n; run = run_n; jj = jj_n;
+    if (!more) break;
+    item = item_n; packed = packed_n; ell = ell_n; ell_slots = slots_n; at = at_n;
     }
 }
 
 // ------------------------------------------------------------------------------------ host side
 
 // Launch configuration of a layout: two CTAs of 8 warps per SM, or one of 16 where x (or the tables of N = 5) leave no room for two.
-struct V2aConfig { int warps, slots; size_t smem; };
+struct V2aConfig { int warps, slots; size_t smem; bool tables; };
 
 static size_t v2a_smem_bytes(const Layout& l, int nb, int warps, bool tables) {
     const size_t tab = tables ? (size_t)l.L * l.E * 128 : ((size_t)l.L * l.E * 2 + 15) & ~size_t(15);
@@ -567,10 +547,16 @@ static size_t v2a_smem_bytes(const Layout& l, int nb, int warps, bool tables) {
 
 static V2aConfig v2a_config(const Layout& l, int nb) {
     const int sms = sched_sms();
-    const bool tables = l.bits > 4;
-    const size_t sm8 = v2a_smem_bytes(l, nb, 8, tables);
-    if (sm8 <= 110u * 1024u) return V2aConfig{8, 2 * sms, sm8};
-    return V2aConfig{16, sms, v2a_smem_bytes(l, nb, 16, tables)};
+    // N = 4: two rows of x halve the look-ups of a product, and the tables, where they leave room for two CTAs or no SM gets a second one, are the faster form
+    // (bf16, 12288 x 4096 22.0 us against 25.7 with codebooks in registers, 4096 x 12288 21.5 and 25.3, 28672 x 8192 75.7 and 77.8); at
+    // one row of several blobs the registers (8 x 3072 x 4096, fp16 34.2 against 40.3, 3 x 14336 x 4096 47.9 and 54.9), and where
+    // the tables would take the SM for one CTA (64 codebooks, two rows, 28672 x 4096 45.1 against 51.8)
+    const size_t tab8 = v2a_smem_bytes(l, nb, 8, true);
+    const bool room = tab8 <= 110u * 1024u || (l.RB <= 2 * sms && v2a_smem_bytes(l, nb, 16, true) <= 224u * 1024u);
+    const bool tables = l.bits == 5 || (l.bits == 4 && nb == 2 && room);
+    const size_t sm8 = tables ? tab8 : v2a_smem_bytes(l, nb, 8, false);
+    if (sm8 <= 110u * 1024u) return V2aConfig{8, 2 * sms, sm8, tables};
+    return V2aConfig{16, sms, v2a_smem_bytes(l, nb, 16, tables), tables};
 }
 
 bool v2a_supported(const Layout& l, int batch) {
@@ -586,12 +572,12 @@ size_t v2a_workspace_bytes(const Layout& l) {
     return align256((size_t)l.RB * 4) + align256((size_t)64 * 2 * (size_t)blocks * kARows * 4);
 }
 
-template <int N, int NB, int W, bool FEAT>
+template <int N, int NB, int W, int FEAT, bool REG>
 static cudaError_t launch_v2a_feat(const V2aArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
     static DeviceOnce attr_done;
     const int dev = DeviceOnce::current();
     if (!attr_done.is_set(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(gemv_v2a_kernel<N, NB, W, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(gemv_v2a_kernel<N, NB, W, FEAT, REG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              W == 8 ? 112 * 1024 : 226 * 1024);
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
@@ -606,19 +592,23 @@ static cudaError_t launch_v2a_feat(const V2aArgs& a, dim3 grid, size_t smem, cud
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_v2a_kernel<N, NB, W, FEAT>, a);
+    return cudaLaunchKernelEx(&cfg, gemv_v2a_kernel<N, NB, W, FEAT, REG>, a);
 }
 
-template <int N, int NB, int W>
+template <int N, int NB, int W, bool REG>
 static cudaError_t launch_v2a(const V2aArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-    if (a.epi != 0 || a.x_bf16 || a.y_is_fp16 == 2) return launch_v2a_feat<N, NB, W, true>(a, grid, smem, s);
-    return launch_v2a_feat<N, NB, W, false>(a, grid, smem, s);
+    if constexpr (NB == 1)
+        if (a.epi != 0) return launch_v2a_feat<N, NB, W, 2, REG>(a, grid, smem, s);
+    if (a.x_bf16 || a.y_is_fp16 == 2) return launch_v2a_feat<N, NB, W, 1, REG>(a, grid, smem, s);
+    return launch_v2a_feat<N, NB, W, 0, REG>(a, grid, smem, s);
 }
 
 template <int N, int NB>
 static cudaError_t launch_v2a_cfg(const V2aConfig& cfg, const V2aArgs& a, dim3 grid, cudaStream_t s) {
-    if (cfg.warps == 16) return launch_v2a<N, NB, 16>(a, grid, cfg.smem, s);
-    return launch_v2a<N, NB, 8>(a, grid, cfg.smem, s);
+    if constexpr (N == 4 && NB == 2)
+        if (cfg.tables) return cfg.warps == 16 ? launch_v2a<N, NB, 16, false>(a, grid, cfg.smem, s) : launch_v2a<N, NB, 8, false>(a, grid, cfg.smem, s);
+    if (cfg.warps == 16) return launch_v2a<N, NB, 16, N <= 4>(a, grid, cfg.smem, s);
+    return launch_v2a<N, NB, 8, N <= 4>(a, grid, cfg.smem, s);
 }
 
 cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s) {
@@ -673,18 +663,11 @@ cudaError_t launch_gemv_v2a(const Layout& l, const GemvCall& c, cudaStream_t s) 
     a.items_x = a.n_full + a.n_a * a.kst + n_b * a.kst_b;
     a.n = c.n;
     a.epi = c.epilogue; a.epi_w = c.epi_weights;
-    long long items = (long long)a.items_x * c.n;
-    a.comb_G = 1; a.comb_ng = 1;
-    if (c.epilogue == 2) {
-        const int G = c.n;     // one blob per run: a CTA walks them where there are more than slots
-        a.comb_ng = (c.n + G - 1) / G;
-        a.comb_G = (c.n + a.comb_ng - 1) / a.comb_ng;
-        items = (long long)a.blocks * a.comb_G;
-    }
+    const long long items = (long long)a.items_x * c.n;
     // several blobs with more items than CTA slots: resident CTAs walk the items, so that x is staged once per CTA and an item's
     // first loads travel under the previous one
-    a.persist = c.n > 1 && (items > cfg.slots || a.comb_ng > 1);
-    dim3 grid((unsigned)(a.persist && items > cfg.slots ? cfg.slots : items), 1, 1);
+    a.persist = c.n > 1 && items > cfg.slots;
+    dim3 grid((unsigned)(a.persist ? cfg.slots : items), 1, 1);
     switch (l.bits * 10 + c.batch) {
         case 21: return launch_v2a_cfg<2, 1>(cfg, a, grid, s);
         case 22: return launch_v2a_cfg<2, 2>(cfg, a, grid, s);
