@@ -142,8 +142,11 @@ LaneConfig lane_config(const Layout& l, int n = 1) {
         const bool two = lane_tab_bytes(l, true) <= 64 * 1024 && RB > sms;
         LaneConfig c{two ? 8 : 16, two ? 2 : 1, true};
         c.tiers = RB > 4 * sms;   // up to four rounds unsplit, as in V2 (N = 6, one CTA per SM: 12288 x 4096 33.6 -> 26.6 us)
-        // the blobs of a routed layer in one launch: the resident CTAs of xfp_gemv_v2a.cu
-        c.off = n > 1;
+        // Several blobs in one launch: the resident CTAs of xfp_gemv_v2a.cu, but at N = 4 up to one row-block per SM, or three of
+        // rows of 1536 weights and more, which leave SMs without one of their blocks of 64 channels (2 x 3072 x 4096 10.1 us
+        // against 16.3, 4 x 1024 x 4096 6.5 and 11.7, 8 x 1536 x 2048 10.8 and 11.1; 4 x 3500 x 1024 8.0 and 6.9,
+        // 8 x 4096 x 1536 24.3 and 18.5)
+        c.off = n > 1 && !(l.bits == 4 && RB <= (l.SC >= 12 ? 3 : 1) * sms);
         return c;
     }
     if (RB <= sms) return LaneConfig{16, 1, l.bits == 6};
