@@ -86,12 +86,31 @@ cudaError_t launch_tile(const BatchPlan& p, const LaneArgs& a, int grid, cudaStr
 //     not fit its shared memory (4096 x 12288, 4 rows: 19 against 54)
 //   * V2 N <= 4: matrices of one round at 3 or 4 rows (4096 x 4096, 4 rows: 7.1 against 8.2); everywhere else two channels per lane
 //     halve the mma count per weight and stay ahead (8192 x 8192, 4 rows: 16.4 against 19.9)
-//   * V2a: up to 4 rows on matrices of one round (4096 x 4096, 2 rows: 7.9 against 11.2), N = 2 up to 4 rows
-//     everywhere, N = 4 at 2 rows and on large matrices up to 4 rows (28672 x 8192: 86 against 92), N = 5 on large
-//     matrices (8 rows: 158 against 198), N = 3 only at 3..4 rows on large matrices (its pair tables of the whole
-//     library serve the other kernel), N = 6 everywhere (28672 x 8192, 8 rows: 193 against 766)
+//   * V2a: up to 4 rows on matrices of one round (4096 x 4096, 2 rows: 7.9 against 11.2), N = 2, 3 at 2 rows by reg_two_rows,
+//     N = 2 at 3..4 rows everywhere, N = 3 at 3..4 rows on large matrices, N = 4 at 2 rows and on large matrices up to 4 rows
+//     (28672 x 8192: 86 against 92), N = 5 on large matrices (8 rows: 158 against 198), N = 6 everywhere (28672 x 8192, 8 rows:
+//     193 against 766)
 //   * many rows on a large matrix with few outliers stay on the tcgen05 kernel (28672 x 8192, 16 rows, 0.3 %: V2a 159
 //     against 246)
+// V2a at N = 2, 3, two rows of x: both kernels decode from registers, this one a row-block per CTA, two CTAs per SM, the row-blocks
+// of the last partial round cut along K; xfp_gemv_v2a.cu blocks of 64 channels, two per SM too (N = 3, fp16, us, this | the other):
+//   up to two row-blocks per SM   4768 x 4096 9.6 | 11.1, 8192 x 8192 17.7 | 20.1, 9472 x 1024 4.0 | 7.5; not where the other cuts its
+//                                 blocks in three along a long K (5600 x 8192 17.7 | 17.0)
+//   up to four                    where the cut leaves slices times super-chunks enough: 10007 x 8192 22.5 | 29.5, x 4096 14.4 | 15.9,
+//                                 12288 x 8192 28.1 | 29.6, x 4096 16.8 | 15.9, x 2048 10.8 | 9.5, 16000 x 8192 32.1 | 29.8,
+//                                 10007 x 1024 7.4 | 5.7
+//   beyond                        28672 x 8192 47.2 | 54.5, 20000 x 1024 10.6 | 12.9, N = 2 x 512 6.2 | 7.1 (N = 3 not measured there)
+static bool reg_two_rows(const Layout& l) {
+    const int sms = sched_sms(), slots = 2 * sms;
+    if (!v2a_supported(l, 2)) return true;
+    if (l.RB > 4 * sms) return l.SC >= 8 || l.bits == 2;
+    if (l.RB <= slots) return l.SC < 64 || 3 * ((l.RB + 1) / 2) > slots;
+    const int tail = l.RB % slots;
+    if (!tail || l.SC < 4) return false;
+    const int cut = pow2_floor_b(slots / tail), most = pow2_floor_b(l.SC / 4);       // as launch_gemv_lane_batch cuts
+    return (cut < most ? cut : most) * l.SC >= 128;
+}
+
 static bool lane_batch_preferred(const Layout& l, int batch) {
     const int sms = sched_sms();
     const bool small = l.RB <= sms, big = l.RB > 4 * sms;
@@ -104,6 +123,7 @@ static bool lane_batch_preferred(const Layout& l, int batch) {
         return small && batch >= 3;
     }
     if ((size_t)l.L * l.E * 128 > 128 * 1024) return true;   // N = 6 at L = 32: the other kernel is the general one
+    if (batch == 2 && lane_reg_book(l) && !small) return reg_two_rows(l);
     if (small) return !many || !batch_supported(l, batch);
     switch (l.bits) {
         case 2: return !many;
@@ -113,10 +133,10 @@ static bool lane_batch_preferred(const Layout& l, int batch) {
     }
 }
 
-// 2..16 rows of fp16 x, one blob, fp32 or fp16 y, no fused store
+// 2..16 rows of x, one blob, no fused store; bf16 x or y at two rows where codebooks sit in registers, else fp16 x, fp32 or fp16 y
 bool lane_batch_supported(const Layout& l, const GemvCall& c) {
     if (c.batch < 2 || c.n != 1 || c.packed_list || c.epilogue != 0) return false;
-    if (c.x_bf16 || c.y_is_fp16 == 2) return false;
+    if ((c.x_bf16 || c.y_is_fp16 == 2) && !(c.batch == 2 && lane_reg_book(l))) return false;
 #ifdef LANE_TUNE
     if (const char* e = getenv("XFP_LANE_BATCH")) {   // tuning build: largest batch this kernel takes, whatever the rule
         if (c.batch > atoi(e)) return false;

@@ -19,7 +19,7 @@ namespace xfp {
 
 namespace {
 
-// NB rows of x (1, 2, 4 or 8); TIO: bf16 x, bf16 y, several blobs through pointer lists (see xfp_gemv_lane.cuh)
+// NB rows of x (1, 2, 4 or 8); TIO (one row or two): bf16 x, bf16 y, several blobs through pointer lists (see xfp_gemv_lane.cuh)
 template <int N, int W, int MINB, bool TIO, int NB>
 __global__ void __launch_bounds__(W * 32, MINB) gemv_reg_kernel(const LaneArgs a) {
     constexpr int E = 1 << N;
@@ -358,6 +358,7 @@ cudaError_t launch_rows(const LaneArgs& a, int nb, int grid, size_t smem, cudaSt
         return launch_io<N, W, MINB, false, 1>(a, grid, smem, s);
     }
     if constexpr (MINB < 3) {
+        if (nb == 2 && (a.x_bf16 || a.y_is_fp16 == 2)) return launch_io<N, W, MINB, true, 2>(a, grid, smem, s);
         if (nb == 2) return launch_io<N, W, MINB, false, 2>(a, grid, smem, s);
         if (nb == 4) return launch_io<N, W, MINB, false, 4>(a, grid, smem, s);
         return launch_io<N, W, MINB, false, 8>(a, grid, smem, s);
