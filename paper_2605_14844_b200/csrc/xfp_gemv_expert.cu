@@ -9,7 +9,7 @@
 //             number take the gates' row-block, the others the up channels'.  Three CTAs per SM (80 registers): the 384 blocks of 8
 //             experts of 3072 x 4096 are resident at once, where 296 resident CTAs with two channels per lane left most SMs waiting
 //             for those with a second block.
-//   COMBINE   a CTA of 16 warps owns one row-block of 32 channels of ALL experts (or of a run of them): (expert, super-chunk) units
+//   COMBINE   a CTA of 16 or 8 warps (combine_plan) owns one row-block of 32 channels of ALL experts (or of a run of them): (expert, super-chunk) units
 //             are dealt to the warps in one sequence, so that short rows (12 super-chunks) leave no warp idle and the experts cost
 //             one staging of x, one reduction and no barrier between them.  A lane's sum of one expert is scaled by its weight when
 //             the expert ends.  Runs of a row-block meet through the workspace in run order; one run per row-block needs none.
@@ -308,19 +308,34 @@ cudaError_t launch(const ExpertArgs& a, int grid, size_t smem, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, gemv_expert_kernel<N, W, R, MINB>, a);
 }
 
-// Runs per row-block of the weighted sum: rounds of CTAs (one per SM) times an item's time -- 150 clocks per unit of 32 channels and
-// 128 weights, 5000 around them, 2500 more where runs meet through the workspace -- over the runs that fit shared memory and the
-// scratch of one GEMV call.
-int combine_runs(const Layout& l, int n, int* per_run) {
-    int best = 0;
+// The weighted sum: CTAs of 16 warps, one per SM, or of 8 warps, three per SM, and runs per row-block (G; ng blobs each).
+struct CombinePlan { int warps, G, ng; };
+
+// Up to one row-block per SM: 16 warps.  Rounds of CTAs times an item's time -- 150 clocks per unit of 32 channels and 128 weights,
+// 5000 around them, 2500 more where runs meet through the workspace -- over the runs that fit shared memory and the scratch of one
+// GEMV call.  Beyond, a second round of 16-warp CTAs leaves most SMs idle: 8 warps, three CTAs per SM, and more runs (us for 16 warps
+// -> this, N = 3: 6 experts 5120 x 1536 23.9 -> 17.5, 2 of 7168 x 3072 16.7 -> 16.1, 8 of 6144 x 2048 36.4 -> 26.4; 8 of 4096 x 1536 take
+// 15.3 in 16 warps, 17.5 in 8).  A CTA's time is its units, three to an SM in full rounds; of a last round of one CTA per SM a unit
+// takes 1.8 of the time it would take alone at full occupancy, and a further round costs 18 units of x and first loads.
+CombinePlan combine_plan(const Layout& l, int n) {
+    const int sms = sched_sms(), slots = 3 * sms;
+    CombinePlan best{16, 0, 0};
     double least = 0.0;
-    for (int G = 1; G <= n && G <= 64; ++G) {
-        const int ng = (n + G - 1) / G, runs = (n + ng - 1) / ng;
-        if (runs != G || ng > kExpertBlobs || expert_smem(l, ng, 16) > kExpertSmemOne) continue;
-        const double rounds = (double)(((long long)l.RB * G + sched_sms() - 1) / sched_sms());
-        const double t = rounds * (ng * (double)l.SC * 150.0 + 5000.0) + (G > 1 ? 2500.0 : 0.0);
-        if (!best || t < least) { best = G; least = t; *per_run = ng; }
-    }
+    for (int warps = l.RB > sms ? 8 : 16; warps <= 16 && !best.G; warps += 8)
+        for (int G = 1; G <= n && G <= 64; ++G) {
+            const int ng = (n + G - 1) / G, runs = (n + ng - 1) / ng;
+            if (runs != G || ng > kExpertBlobs || expert_smem(l, ng, warps) > (warps == 8 ? kExpertSmemThree : kExpertSmemOne)) continue;
+            const long long ctas = (long long)l.RB * G;
+            const double run = (double)ng * l.SC;
+            double t;
+            if (warps == 16) {
+                t = (double)((ctas + sms - 1) / sms) * (run * 150.0 + 5000.0) + (G > 1 ? 2500.0 : 0.0);
+            } else {
+                const long long full = ctas / slots, rest = ctas % slots;
+                t = (double)full * 3.0 * run + (double)(full + (rest > 0) - 1) * 18.0 + (rest == 0 ? 0.0 : rest <= sms ? 1.8 : 3.0) * run;
+            }
+            if (!best.G || t < least) { best = CombinePlan{warps, G, ng}; least = t; }
+        }
     return best;
 }
 
@@ -329,9 +344,8 @@ int combine_runs(const Layout& l, int n, int* per_run) {
 // fused stores of V2a blobs at N <= 4, groups of 128 or 256 weights, where x and the libraries fit shared memory
 bool expert_supported(const Layout& l, const GemvCall& c) {
     if (l.mode != 1 || l.bits > 4 || l.GH != 1 || c.batch != 1 || !c.packed_list) return false;
-    int ng;
     if (c.epilogue == 1) return expert_smem(l, 1, 8) <= kExpertSmemThree;
-    return c.epilogue == 2 && combine_runs(l, c.n, &ng) > 0;
+    return c.epilogue == 2 && combine_plan(l, c.n).G > 0;
 }
 
 cudaError_t launch_gemv_expert(const Layout& l, const GemvCall& c, cudaStream_t s) {
@@ -364,13 +378,14 @@ cudaError_t launch_gemv_expert(const Layout& l, const GemvCall& c, cudaStream_t 
             default: return launch<4, 8, 2, 3>(a, grid, smem, s);
         }
     }
-    a.G = combine_runs(l, c.n, &a.ng);
-    const int grid = l.RB * a.G;
-    const size_t smem = expert_smem(l, a.ng, 16);
+    const CombinePlan p = combine_plan(l, c.n);
+    a.G = p.G; a.ng = p.ng;
+    const int grid = l.RB * p.G;
+    const size_t smem = expert_smem(l, p.ng, p.warps);
     switch (l.bits) {
-        case 2: return launch<2, 16, 1, 1>(a, grid, smem, s);
-        case 3: return launch<3, 16, 1, 1>(a, grid, smem, s);
-        default: return launch<4, 16, 1, 1>(a, grid, smem, s);
+        case 2: return p.warps == 8 ? launch<2, 8, 1, 3>(a, grid, smem, s) : launch<2, 16, 1, 1>(a, grid, smem, s);
+        case 3: return p.warps == 8 ? launch<3, 8, 1, 3>(a, grid, smem, s) : launch<3, 16, 1, 1>(a, grid, smem, s);
+        default: return p.warps == 8 ? launch<4, 8, 1, 3>(a, grid, smem, s) : launch<4, 16, 1, 1>(a, grid, smem, s);
     }
 }
 
