@@ -329,6 +329,14 @@ int xfp_debug_prefill_piece(const xfp_desc* desc, int32_t m, int32_t g, int32_t 
     return fused_piece_report(layout_of(desc), m, g, i, out);
 }
 
+// ... the plan of xfp_dequant (super-chunks of a block, blocks of a row-block, outliers added to the staged rows) ...
+int xfp_debug_dequant_plan(const xfp_desc* desc, int32_t* out) {
+    const int st = check_desc(desc);
+    if (st) return st;
+    dequant_plan_report(layout_of(desc), out);
+    return XFP_OK;
+}
+
 // ... and xfp_gemm of more than 64 rows in which the bounded waits of one CTA give up at once.
 int xfp_debug_gemm_short_waits(const xfp_desc* desc, const void* packed, const uint16_t* x, int32_t m, void* y, int32_t y_type,
                                void* workspace, size_t workspace_bytes, int32_t cta, void* stream) {

@@ -7,7 +7,7 @@
 //   V2a  a lane decodes the 2^N entries its channel's group can take once -- D16 = fp16(fp32(scale * lib[id] + mid)) -- into
 //        registers (N <= 4) or a column of a table of its warp, and the weights of the group are look-ups as in V2: 2^N
 //        conversions per group instead of one per weight.
-//   S    up to N = 4, and four blocks to a row-block, the block notes where every super-chunk's outliers begin in its channels'
+//   S    up to N = 4, where outliers are many (plan_of), the block notes where every super-chunk's outliers begin in its channels'
 //        slabs and a lane adds those of its channel to the staged row, one correctly rounded fp16 addition each.  What a slab
 //        cannot say (channels longer than their slab, columns that do not ascend), and all of them elsewhere, is added in place
 //        behind the block's stores (above N = 4, where tables leave one or two blocks to an SM, the list in front of the decode
@@ -237,6 +237,44 @@ __global__ void __launch_bounds__(kDqWarps * 32, N <= 4 ? 3 : 0) dequant_kernel(
     }
 }
 
+// Super-chunks of a block, blocks of a row-block, whether outliers are added to the staged rows.
+struct DqPlan { int range, parts; bool lists; };
+
+DqPlan plan_of(const Layout& l) {
+    const int sms = sm_count();
+    const long long slots = 3ll * sms;
+    int range = l.SC < kDqRange ? l.SC : kDqRange;
+    auto parts = [&](int r) { return (l.SC + r - 1) / r; };
+    if (l.bits > 4) {       // few row-blocks: shorter ranges, at least one super-chunk per warp, until the blocks fill the GPU twice
+        while (range > kDqWarps && (long long)l.RB * parts(range) < 4ll * sms) range = (range + 1) / 2;
+        return DqPlan{range, parts(range), false};
+    }
+    // Rounds of three blocks per SM times (turns of a warp and one for the block's first loads), in the fewest parts that reach
+    // the least: 3072 x 4096 V2 N = 4 6.5 us with ranges of 8, 4096 x 4096 8.2 with 16, 10.9 with 24.
+    long long best = -1;
+    for (int n = parts(kDqRange); n <= parts(kDqWarps); ++n) {
+        const int r = (l.SC + n - 1) / n;
+        const long long cost = (l.RB * (long long)parts(r) + slots - 1) / slots * ((r + kDqWarps - 1) / kDqWarps + 1);
+        if (best < 0 || cost < best) { best = cost; range = r; }
+    }
+    // Lists of the outliers in front of the decode, or in place behind the stores.  Every block walks all slots of its row-block
+    // for either; the lists' walk stands in front of everything else.  They win where outliers are many and the matrix is not
+    // cut into many parts: from 3 % on, and at N <= 3, whose decode is the shorter, from 1/128 on beyond four row-blocks per SM
+    // and from 1/64 on for one part of up to 16 super-chunks (us, lists | in place: 28672 x 2048 N = 2, 2 % 36.8 | 41.5, 28672 x 8192
+    // N = 2, 2 % 136 | 148, 1 % 115 | 121, 8192 x 2048 N = 3, 2 % 11.1 | 11.9; 12288 x 4096 N = 4, 5 % 49.9 | 74.9, 2 % 35.9 | 34.3,
+    // 0.3 % 27.8 | 24.5; 512 x 2048 N = 4, 2 % 6.8 | 4.8).
+    const long long weights = (long long)l.rows * l.cols;
+    const bool many = l.nnz * 100 >= 3 * weights || (l.bits <= 3 && ((l.RB > 4 * sms && l.nnz * 128 >= weights) ||
+                                                                     (l.SC <= 16 && l.nnz * 64 >= weights)));
+    const bool lists = l.ell_slots != 0 && many && l.RB > sms && parts(range) <= 4;
+    // More than a round of blocks without lists: short ranges, whose blocks the SMs take as they become free -- 16 super-chunks,
+    // so that the slots are not walked too often, or 8 where there are none (28672 x 8192 V2 N = 4, 2 % 144 us with 16, 162
+    // with 8, 196 with 32; without outliers 96.8, 92.7, 107; N = 2 without outliers 91.0, 85.2, 100).
+    const int s = l.SC < 16 ? l.SC : l.ell_slots ? 16 : 8;
+    if (!lists && (long long)l.RB * parts(16) > slots) range = (l.SC + parts(s) - 1) / parts(s);
+    return DqPlan{range, parts(range), lists};
+}
+
 template <int N, int MODE>
 cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s) {
     using T = DqTab<N, MODE>;
@@ -253,30 +291,19 @@ cudaError_t launch_decode(const Layout& l, const void* packed, uint16_t* W, cuda
         if (e != cudaSuccess) return e;
         attr_done.set(dev);
     }
-    int range = a.SC < kDqRange ? a.SC : kDqRange;
-    if (T::kReg) {
-        // rounds of three blocks per SM times (turns of a warp and one for the block's first loads), in the fewest parts that reach
-        // the least: 4096 x 4096 V2 N = 4 13.0 us with ranges of 16, 15.8 with 8, 14.5 with 32; 12288 x 4096 30.9 with 32, 32.8 with
-        // 16; 8192 x 8192 N = 3 35.6 with 22, 37.0 with 16, 43.1 with 32
-        const long long slots = 3ll * sm_count();
-        long long best = -1;
-        for (int parts = (a.SC + kDqRange - 1) / kDqRange; parts <= (a.SC + kDqWarps - 1) / kDqWarps; ++parts) {
-            const int r = (a.SC + parts - 1) / parts;
-            const long long cost = (l.RB * (long long)((a.SC + r - 1) / r) + slots - 1) / slots * ((r + kDqWarps - 1) / kDqWarps + 1);
-            if (best < 0 || cost < best) { best = cost; range = r; }
-        }
-    } else {        // few row-blocks: shorter ranges, at least one super-chunk per warp, until the blocks fill the GPU twice
-        while (range > kDqWarps && (long long)l.RB * ((a.SC + range - 1) / range) < 4ll * sm_count()) range = (range + 1) / 2;
-    }
-    a.range = range;
-    // every block of a row-block walks all of its slots for the lists: beyond four parts that costs more than adding in place
-    // (1024 x 8192 V2 N = 4, eight parts, 1 % outliers: 12.5 us with lists, 8.3 without; 3072 x 4096 V2a N = 4, four: 12.5, 12.9)
-    a.lists = T::kReg && a.ell_slots != 0 && (a.SC + range - 1) / range <= 4;
-    dequant_kernel<N, MODE><<<(unsigned)(l.RB * ((a.SC + range - 1) / range)), kDqWarps * 32, smem, s>>>(a);
+    const DqPlan p = plan_of(l);
+    a.range = p.range;
+    a.lists = p.lists;
+    dequant_kernel<N, MODE><<<(unsigned)(l.RB * p.parts), kDqWarps * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 }  // namespace
+
+void dequant_plan_report(const Layout& l, int32_t* out) {
+    const DqPlan p = plan_of(l);
+    out[0] = p.range; out[1] = p.parts; out[2] = p.lists;
+}
 
 cudaError_t launch_dequant(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s) {
     if (l.mode == 0) {

@@ -51,6 +51,7 @@ struct PackInputs {
 // counted: the kernel leaves the blob as it is when the last row pointer is not l.nnz
 cudaError_t launch_pack(const Layout& l, const PackInputs& in, void* packed, int* err_word, cudaStream_t s, bool counted = false);
 cudaError_t launch_dequant(const Layout& l, const void* packed, uint16_t* W, cudaStream_t s);
+void dequant_plan_report(const Layout& l, int32_t* out);                            // for tests
 
 // One GEMV problem set: either a single blob (packed/x/y) or n blobs through device pointer lists.
 struct GemvCall {

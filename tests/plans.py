@@ -15,6 +15,13 @@ def gemv_kernel(desc, batch, n=1, x_type=xfp.XFP_T_F16, y_type=xfp.XFP_T_F32, ep
     return KERNELS[k.value]
 
 
+def dequant_plan(desc):
+    """(super-chunks of a block, blocks of a row-block, outliers added to the staged rows)"""
+    out = (C.c_int32 * 3)()
+    assert xfp.load_library().xfp_debug_dequant_plan(C.byref(desc), out) == 0
+    return out[0], out[1], bool(out[2])
+
+
 def plan(desc, m):
     """A dict of FIELDS; None where the pair kernel does not take the call."""
     out = (C.c_int64 * len(FIELDS))()

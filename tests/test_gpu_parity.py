@@ -12,7 +12,7 @@ import pytest
 import torch
 
 from conftest import from_oracle, to_oracle
-from plans import gemv_kernel
+from plans import dequant_plan, gemv_kernel
 from oracle import xfp_oracle as xo
 import paper_2605_14844_b200 as xfp
 from paper_2605_14844_b200 import binding, synth
@@ -270,9 +270,39 @@ def test_outlier_structures(placement, rate):
     (1, 2, 64, 640, 0.05, "one_row"), (0, 2, 70, 4224, 0.01, "uniform"), (0, 3, 1, 128, 0.3, "uniform"), (0, 6, 50, 4224, 0.02, "uniform"),
     (1, 5, 50, 4224, 0.02, "uniform")])
 def test_dequant_adds_the_outliers_of_every_super_chunk(mode, bits, rows, cols, rate, placement):
-    """Channels of one range of super-chunks and of several, more slots than are staged, slabs that overflow, one super-chunk."""
+    """Outliers in place: channels of one range of super-chunks and of several, slabs that overflow, one super-chunk."""
     q = synth.random_quantized(mode, rows, cols, bits, rate, seed=8100 + 10 * mode + bits, placement=placement)
-    _check_dequant(q, xfp.pack_tensors(q))
+    pm = xfp.pack_tensors(q)
+    assert not dequant_plan(pm.desc)[2]
+    _check_dequant(q, pm)
+
+
+@pytest.mark.parametrize("mode,bits,rows,cols,rate,parts", [
+    (0, 2, 4741, 128, 0.04, 1), (1, 4, 14240, 1024, 0.08, 1), (0, 3, 18960, 1280, 0.012, 1), (0, 4, 4740, 1152, 0.035, 2),
+    (1, 3, 4740, 4224, 0.05, 2), (1, 2, 6080, 8320, 0.035, 3)])
+def test_dequant_adds_listed_outliers_to_the_staged_rows(mode, bits, rows, cols, rate, parts):
+    """One to three ranges of super-chunks, fewer outliers of a channel in a range than are staged and more, a channel that overflows
+    its slab, one whose columns descend in the last range only, one without outliers."""
+    q = synth.random_quantized(mode, rows, cols, bits, rate, seed=8150 + 10 * mode + bits + parts)
+    cut = lambda r: (q.ocol[q.rowptr[r]:q.rowptr[r + 1]], q.oval[q.rowptr[r]:q.rowptr[r + 1]])
+    rowsets = [cut(r) for r in range(rows)]
+    rng = np.random.default_rng(8160)
+    rowsets[37] = (np.arange(cols, dtype=np.int32), synth._f16bits(rng.standard_normal(cols)))      # longer than any slab
+    rowsets[38] = (rowsets[38][0][:0], rowsets[38][1][:0])
+    rowsets[rows - 1] = (np.arange(cols, dtype=np.int32), synth._f16bits(rng.standard_normal(cols)))
+    flat = synth.QuantTensors(**{**q.__dict__, "rowptr": np.concatenate([[0], np.cumsum([len(c) for c, _ in rowsets])]).astype(np.int32),
+                                 "ocol": np.concatenate([c for c, _ in rowsets]), "oval": np.concatenate([v for _, v in rowsets])})
+    pm = xfp.pack_tensors(flat)
+    assert dequant_plan(pm.desc)[1:] == (parts, True)
+    _check_dequant(flat, pm)
+    r = 70                                             # a row-block of its own: its columns descend behind the first range
+    a, b = flat.rowptr[r], flat.rowptr[r + 1]
+    if b - a >= 2:
+        flat.ocol[b - 2:b] = flat.ocol[b - 2:b][::-1].copy()
+        flat.oval[b - 2:b] = flat.oval[b - 2:b][::-1].copy()
+        pm = xfp.pack_tensors(flat)
+        got = pm.dequant().view(torch.int16).cpu().numpy().view(np.uint16)
+        assert np.array_equal(got, xo.dequant(to_oracle(flat))) and int(pm.err_word.item()) == 16
 
 
 @pytest.mark.parametrize("mode", [0, 1])
