@@ -83,7 +83,7 @@ __device__ __forceinline__ void store_ascending(const double* c, int E, int tid,
     lib[r] = d2h(x);
 }
 
-// The rounds of the k-means where they fit one cluster of 16 SMs: the channels are dealt to the blocks in runs.
+// The rounds of the k-means where they fit one cluster of 16 SMs (N = 2: see launch_libfit_library): the channels are dealt to the blocks in runs.
 //   assignment  two threads per channel, its E values in registers, centroids in order with a strict "less than"
 //   update      half a block per centroid: every block has all assignments (a byte per channel, written to each of them),
 //               compacts the members in channel order, fetches their values from the blocks that hold them, and thread j adds
@@ -95,6 +95,7 @@ constexpr int kClBlocks = 16;
 constexpr int kClVals = 2048;                       // member values staged at a time by half a block
 constexpr size_t kClSmem = 200 * 1024;
 constexpr long long kClTerms = 2000000;
+constexpr int kClLib = 40;                          // centroids at most
 __host__ __device__ inline int cl_per(int rows) { return ((rows + kClBlocks - 1) / kClBlocks + 3) & ~3; }
 inline size_t cl_smem(int rows, int E, int L) {
     const size_t asg = ((size_t)cl_per(rows) * kClBlocks + 15) & ~size_t(15);
@@ -735,11 +736,14 @@ cudaError_t launch_cluster(const uint16_t* codebook, int rows, int L, int iters,
 
 cudaError_t launch_libfit_library(const uint16_t* codebook, int rows, int E, int L, int iters, double* u, double* nn,
                                   int* order, int* asg, double* cen, int* flags, uint16_t* lib, cudaStream_t s) {
-    // one cluster at N = 2 while its assignment step (rows L E terms on 16 SMs) costs less than the grid barriers it saves; library
-    // of 32 after 20 rounds, one cluster against all SMs: 3072 channels N = 2 155 against 186 us, 12288 N = 2 493 against 536, 1472
-    // N = 2 122 against 140; 3072 N = 3 230 against 237, N = 4 369 against 290, 6144 N = 3 443 against 396
+    // One cluster at N = 2 while its assignment step (rows L E terms on 16 SMs) costs less than the grid barriers it saves: at few
+    // centroids whatever the rows, at many only where rows are many too.  us, 20 rounds at most, one cluster | all SMs:
+    //   3072 channels  L = 8 203 | 248, 32 146 | 173, 40 192 | 197, 64 196 | 183, 128 270 | 204, 256 315 | 219
+    //   1024 channels  L = 8 91 | 136, 32 99 | 128, 40 93 | 101, 64 103 | 96, 128 134 | 93, 256 177 | 102
+    //   12288 channels L = 8 641 | 791, 32 472 | 522, 40 561 | 606, 64 552 | 576, 128 790 | 744
+    // N = 3 and 4 lose from 32 centroids on: 3072 channels N = 3 230 | 237, N = 4 369 | 290, 6144 N = 3 443 | 396
     bool taken = false;
-    if (E == 4 && (long long)rows * L * E <= kClTerms && rows <= 65535 && cl_smem(rows, E, L) <= kClSmem) {
+    if (E == 4 && L <= kClLib && (long long)rows * L * E <= kClTerms && rows <= 65535 && cl_smem(rows, E, L) <= kClSmem) {
         const cudaError_t e = launch_cluster<4>(codebook, rows, L, iters, u, nn, order, lib, s, &taken);
         if (taken || e != cudaSuccess) return e;
     }

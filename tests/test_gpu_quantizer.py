@@ -224,10 +224,12 @@ def test_libfit_library_in_shared_memory_and_beyond(bits, rows):
 
 
 @pytest.mark.parametrize("bits,L,rows", [(2, 32, 15625), (2, 32, 15626), (4, 32, 3906), (4, 32, 3907), (3, 32, 3072), (3, 5, 17),
-                                         (2, 40, 5), (4, 1, 16), (2, 256, 1000), (4, 17, 515)])
+                                         (2, 40, 5), (4, 1, 16), (2, 256, 1000), (4, 17, 515), (2, 1, 1500), (2, 5, 17), (2, 33, 515),
+                                         (2, 1, 3), (2, 40, 700), (2, 41, 700)])
 def test_libfit_library_on_one_cluster_and_on_all_sms(bits, L, rows):
-    """Either side of the line between the two forms of the rounds (2 000 000 terms per assignment), fewer channels than blocks or
-    than centroids, centroids that no multiple of the blocks deals evenly, members beyond one staging buffer (a single centroid)."""
+    """N = 2 on either side of the lines between the two forms of the rounds (2 000 000 terms per assignment, 40 centroids), other
+    widths, which always run on all SMs; fewer channels than blocks or than centroids, an odd number of centroids and one that no
+    multiple of the blocks deals evenly, members beyond one staging buffer of the cluster's blocks (1500 of a single centroid)."""
     rng = np.random.default_rng(rows + L)
     cb = np.sort(rng.standard_normal((rows, 1 << bits)), axis=1).astype(np.float16)
     cb[rows // 2:rows // 2 + 3] = cb[0]
@@ -238,6 +240,45 @@ def test_libfit_library_on_one_cluster_and_on_all_sms(bits, L, rows):
     qb.xfp_quant_libfit_library(_dev(cb), rows, bits, L, 8, lib, _ws(rows, 512))
     torch.cuda.synchronize()
     assert np.array_equal(_u16(lib), want)
+
+
+@pytest.mark.parametrize("L,rows", [(1, 40), (7, 300), (32, 130)])
+def test_libfit_library_of_codebooks_that_are_not_finite(L, rows):
+    """N = 2, on one cluster: channels whose codebook has no norm come last in the order of the seeds,
+    are nearest to no centroid and count for the first one, as the same steps in numpy's fp64 give it."""
+    rng = np.random.default_rng(8400 + rows + L)
+    cb = np.sort(rng.standard_normal((rows, 4)), axis=1).astype(np.float16)
+    cb[rows // 3, 3], cb[rows // 2, 0], cb[rows - 1, 3] = np.inf, -np.inf, np.nan
+    with np.errstate(all="ignore"):
+        c = cb.astype(np.float64)
+        lo, hi = np.fmin.reduce(c, axis=1), np.fmax.reduce(c, axis=1)
+        m, s = 0.5 * (hi + lo), 0.5 * (hi - lo)
+        s[s == 0.0] = 1.0
+        u = (c - m[:, None]) / s[:, None]
+        nn = np.zeros(rows)
+        for j in range(4):
+            nn += u[:, j] * u[:, j]
+        order = np.argsort(np.where(np.isnan(nn), np.inf, nn), kind="stable")
+        cen = u[order[[min(rows - 1, int((l + 0.5) * rows / L)) for l in range(L)]]].copy()
+        for _ in range(6):
+            d = np.zeros((rows, L))
+            for j in range(4):
+                t = u[:, j:j + 1] - cen[None, :, j]
+                d += t * t
+            best = np.argmin(np.where(np.isnan(d), np.inf, d), axis=1)
+            for l in range(L):
+                rows_l = np.flatnonzero(best == l)
+                if len(rows_l):
+                    acc = np.zeros(4)
+                    for i in rows_l:
+                        acc = acc + u[i]
+                    cen[l] = acc / len(rows_l)
+        want = np.sort(cen, axis=1).astype(np.float16)
+    lib = torch.zeros((L, 4), dtype=torch.int16, device="cuda")
+    qb.xfp_quant_libfit_library(_dev(np.ascontiguousarray(cb).view(np.uint16)), rows, 2, L, 6, lib, _ws(rows, 512))
+    torch.cuda.synchronize()
+    got = _u16(lib).view(np.float16).reshape(L, 4)
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(got[~np.isnan(want)], want[~np.isnan(want)])
 
 
 @pytest.mark.parametrize("bits,group", [(2, 128), (3, 128), (4, 128), (5, 128), (3, 64), (4, 256), (6, 64), (2, 256)])
