@@ -319,6 +319,7 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
                         const double t = __dsub_rn(x, staged ? vals[j * L + l] : __ldcg(cen + l * E + j));
                         d = __dadd_rn(d, __dmul_rn(t, t));
                     }
+                    if (d != d) d = INFINITY;    // nearest to nothing, as in a scan; no lane may drop what it compares it with
                 }
                 int bl = l;
 #pragma unroll

@@ -242,9 +242,9 @@ def test_libfit_library_on_one_cluster_and_on_all_sms(bits, L, rows):
     assert np.array_equal(_u16(lib), want)
 
 
-@pytest.mark.parametrize("L,rows", [(1, 40), (7, 300), (32, 130)])
+@pytest.mark.parametrize("L,rows", [(1, 40), (7, 300), (32, 130), (48, 300)])
 def test_libfit_library_of_codebooks_that_are_not_finite(L, rows):
-    """N = 2, on one cluster: channels whose codebook has no norm come last in the order of the seeds,
+    """N = 2, on one cluster and (48 centroids) on all SMs: channels whose codebook has no norm come last in the order of the seeds,
     are nearest to no centroid and count for the first one, as the same steps in numpy's fp64 give it."""
     rng = np.random.default_rng(8400 + rows + L)
     cb = np.sort(rng.standard_normal((rows, 4)), axis=1).astype(np.float16)
