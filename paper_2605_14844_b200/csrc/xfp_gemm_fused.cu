@@ -206,23 +206,16 @@ __device__ __forceinline__ int product_rows(const FusedArgs& a, int p0, int p) {
 // the pair that has dealt super-chunk u: the largest g with g S / D <= u
 __device__ __forceinline__ int dealt_to(const FusedArgs& a, int u) { return ((u + 1) * a.dealt - 1) / a.stream; }
 
-// Decode tables.  kPair: entry t = first index | second index << N holds two fp16 values; else entry q one.  N = 4 entries lie
-// 256 bytes apart (two tables interleaved): an index isolated in its own byte becomes the second byte of the address.
-// V2: a table per row-block.  V2a: a table per warp.
+// Decode tables, where codebooks do not sit in registers (kReg).  kPair (V2, N <= 3): entry t = first index | second index << N holds
+// two fp16 values; else entry q one.  V2: a table per row-block.  V2a: a table per warp.
 template <int N, int MODE>
 struct Tab {
     static constexpr int E = 1 << N;
-    static constexpr bool kPair = MODE == 0 ? N <= 3 : N == 2;
+    static constexpr bool kPair = MODE == 0 && N <= 3;
     static constexpr int kEntries = kPair ? E * E : E;
-    static constexpr int kStride = N == 4 ? 256 : 128;
-    static constexpr int kOne = N == 4 ? 4096 : (kEntries * 128 < 1024 ? 1024 : kEntries * 128);   // of one (N = 4: two) tables
-    static constexpr int kUnits = MODE == 0 ? 4 : kDecodeWarps;
-    static constexpr int kBytes = N == 4 ? kOne * kUnits / 2 : kOne * kUnits;
+    static constexpr int kOne = kEntries * 128;      // of one table
     // address of table u's entry 0 for this lane
-    __device__ static __forceinline__ uint32_t at(uint32_t base, int u, int lane) {
-        return N == 4 ? base + (uint32_t)(u >> 1) * kOne + (uint32_t)(u & 1) * 128u + (uint32_t)lane * 4u
-                      : base + (uint32_t)u * kOne + (uint32_t)lane * 4u;
-    }
+    __device__ static __forceinline__ uint32_t at(uint32_t base, int u, int lane) { return base + (uint32_t)u * kOne + (uint32_t)lane * 4u; }
 };
 
 // W^ = fp16(D16 + S) in place
@@ -266,8 +259,8 @@ __device__ __forceinline__ void fill_tables(const FusedArgs& a, uint32_t tab0, i
         for (int e = 0; e < E / 4; e += 4) {
             const int e0 = sub * (E / 4) + e;
             const uint2 p = __ldg((const uint2*)(cb + e0));
-            sts32(t + (uint32_t)(e0 * T::kStride), p.x & 0xffffu); sts32(t + (uint32_t)((e0 + 1) * T::kStride), p.x >> 16);
-            sts32(t + (uint32_t)((e0 + 2) * T::kStride), p.y & 0xffffu); sts32(t + (uint32_t)((e0 + 3) * T::kStride), p.y >> 16);
+            sts32(t + (uint32_t)(e0 * 128), p.x & 0xffffu); sts32(t + (uint32_t)((e0 + 1) * 128), p.x >> 16);
+            sts32(t + (uint32_t)((e0 + 2) * 128), p.y & 0xffffu); sts32(t + (uint32_t)((e0 + 3) * 128), p.y >> 16);
         }
     }
 }
@@ -361,8 +354,8 @@ __device__ __forceinline__ bool decode_tile(const FusedArgs& a, int rb, bool rb_
                         const uint32_t lw[4] = {l8.x, l8.y, l8.z, l8.w};
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            sts32(tab + (e + 2 * i) * T::kStride, decoded(lw[i] & 0xffffu));
-                            sts32(tab + (e + 2 * i + 1) * T::kStride, decoded(lw[i] >> 16));
+                            sts32(tab + (e + 2 * i) * 128, decoded(lw[i] & 0xffffu));
+                            sts32(tab + (e + 2 * i + 1) * 128, decoded(lw[i] >> 16));
                         }
                     }
                 }
@@ -832,7 +825,8 @@ struct FusedPlan {
 
 // Clocks of a tile's super-chunk: the products (4 T), or shared memory, which every byte crosses at 128 per clock -- per 64 k
 // the look-ups of 4 warps (one wavefront each, half with pair tables), V2a's tables, 128 for storing A, 128 for the products'
-// reading it, T / 2 for x coming in and T / 2 for its being read --, or the operands' way from L2.
+// reading it, T / 2 for x coming in and T / 2 for its being read --, or the operands' way from L2.  Fitted to look-ups in tables at
+// every width: where codebooks sit in registers now (kReg) a stage leaves shared memory more time than this.
 double slot_clocks(const Layout& l, int T) {
     const bool pair = l.mode ? l.bits == 2 : l.bits <= 3;
     const double smem = 2.0 * ((pair ? 128 : 256) + (l.mode ? (l.bits == 2 ? 64 : 4 * l.E) : 0) + 256 + T) * 1.08;
@@ -842,7 +836,8 @@ double slot_clocks(const Layout& l, int T) {
     return m > feed ? m : feed;
 }
 
-// (the plans keep the room of the tables where codebooks sit in registers)
+// The room of the tables in the plans, that of widths whose codebooks sit in registers included: the costs above were fitted with it,
+// and without it (a stage more at 10007 x 4992 V2a N = 4, 301 rows, and at 4096 x 4096 V2 N = 4, 100 rows) they have not been yet.
 size_t table_bytes(const Layout& l) {
     const size_t one = l.mode == 0 ? (l.bits <= 3 ? l.E * l.E : l.E) : (l.bits == 2 ? 16 : l.E);
     const size_t units = l.mode == 0 ? 4 : kDecodeWarps;
