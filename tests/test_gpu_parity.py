@@ -246,6 +246,59 @@ def test_v2a_register_codebooks(bits, rows, cols, group):
         _check_gemv(q, pm, synth.activations(batch, cols, seed=9960 + batch), rows=sample)
 
 
+@pytest.mark.parametrize("bits,n,rows,cols,group,kernel", [
+    (2, 5, 4000, 1024, 128, "lane"), (3, 5, 4000, 1024, 64, "lane"), (3, 3, 300, 4096, 64, "lane"), (2, 2, 90, 8192, 256, "lane"),
+    (2, 7, 2144, 384, 64, "lane"), (4, 3, 300, 4096, 64, "lane"), (4, 4, 3300, 1536, 128, "lane"), (4, 2, 70, 256, 128, "lane"),
+    (4, 4, 3300, 1408, 128, "v2a"), (4, 5, 4000, 1024, 256, "v2a")])
+@pytest.mark.parametrize("dt", [torch.float16, torch.bfloat16])
+def test_v2a_over_several_blobs(bits, n, rows, cols, group, kernel, dt):
+    """Launches over several blobs with libraries of their own: cut along K (few row-blocks, and the last round of many), whole rounds,
+    groups of 64 weights, either side of the lines between the two kernels of N = 4."""
+    qs = [synth.random_quantized(1, rows, cols, bits, 0.005 * (j + 1), seed=2800 + j, group_size=group) for j in range(n)]
+    pms = [xfp.pack_tensors(q, col_bits=16) for q in qs]
+    d = _group_desc(pms)
+    t = xfp.XFP_T_BF16 if dt == torch.bfloat16 else xfp.XFP_T_F16
+    assert gemv_kernel(d, 1, n, t, t) == kernel
+    ws = torch.zeros(n * xfp.xfp_packed_size(d)[1], dtype=torch.uint8, device="cuda")
+    x = _x_dev(synth.activations(n, cols, seed=2810)).to(dt)
+    x16 = x.to(torch.float16).view(torch.int16).cpu().numpy().view(np.uint16)
+    y = torch.empty((n, rows), dtype=torch.float32, device="cuda")
+    ptr = lambda ts: torch.tensor([v.data_ptr() for v in ts], dtype=torch.int64, device="cuda")
+    blobs, xs, ys = ptr([p.packed for p in pms]), ptr([x[j] for j in range(n)]), ptr([y[j] for j in range(n)])
+    for _ in range(2):                                 # the second launch finds the counters as the first one left them
+        y.fill_(float("nan"))
+        xfp.xfp_gemv_grouped_typed(d, n, blobs, xs, dt, ys, torch.float32, xfp.XFP_EPI_NONE, None, ws)
+        got = y.cpu().numpy().astype(np.float64)
+        for j, q in enumerate(qs):
+            ref, absum = xo.gemv(to_oracle(q), x16[j:j + 1])
+            assert np.all(np.abs(got[j] - ref[0]) <= TOL * absum[0] + 1e-30)
+
+
+@pytest.mark.parametrize("bits,rows,cols,group,lib_size,kernel", [
+    (2, 4769, 1024, 64, 32, "lane_batch"), (3, 4769, 3584, 128, 7, "lane_batch"), (3, 19000, 1024, 128, 32, "lane_batch"),
+    (2, 19000, 1024, 256, 33, "lane_batch"), (2, 12288, 2048, 128, 32, "v2a"), (3, 10007, 2048, 128, 32, "v2a"),
+    (3, 10007, 4096, 128, 32, "lane_batch"), (4, 9700, 2048, 128, 32, "v2a"), (4, 9700, 2048, 128, 64, "v2a"),
+    (4, 1100, 16384, 128, 32, "v2a"), (4, 1200, 14336, 128, 64, "v2a")])
+def test_v2a_two_rows_of_bf16(bits, rows, cols, group, lib_size, kernel):
+    """N = 2, 3 on either side of the lines between the two kernels with codebooks in registers; N = 4 with tables (two CTAs per SM
+    and one) and, where those leave no room, registers."""
+    q = synth.random_quantized(1, rows, cols, bits, 0.003, seed=2850 + rows + cols, group_size=group, lib_size=lib_size)
+    pm = xfp.pack_tensors(q, col_bits=16)
+    assert gemv_kernel(pm.desc, 2, 1, xfp.XFP_T_BF16, xfp.XFP_T_F32) == kernel
+    x = _x_dev(synth.activations(2, cols, seed=2860)).to(torch.bfloat16)
+    x16 = x.to(torch.float16).view(torch.int16).cpu().numpy().view(np.uint16)
+    y = torch.full((2, rows), float("nan"), dtype=torch.float32, device="cuda")
+    m, sample = to_oracle(q), _sample_rows(rows, 96, seed=2861)
+    for _ in range(2):
+        y.fill_(float("nan"))
+        xfp.xfp_gemv_typed(pm.desc, pm.packed, x, 2, y, pm.workspace)
+        got = y.cpu().numpy().astype(np.float64)
+        assert np.all(np.isfinite(got))
+        for r in sample:
+            ref, absum = xo.gemv(m, x16, int(r), int(r) + 1)
+            assert np.all(np.abs(got[:, r] - ref[:, r]) <= TOL * absum[:, r] + 1e-30)
+
+
 @pytest.mark.parametrize("mode,bits", [(0, 4), (0, 5), (1, 3), (1, 4)])
 def test_longest_rows(mode, bits):
     """K = 65536, the largest the descriptor admits (u16 outlier columns): x alone is 128 KB per batch row."""
