@@ -14,8 +14,9 @@
 //        cost more: 12288 x 4096 V2a N = 6 38.2 -> 46.1 us with pack, half of both).
 //   out  a tile of shared memory turns a lane's 64 weights into whole 128-byte lines of the channels' rows.
 // Tables in shared memory and outliers in place behind the stores -> this, cold: 12289 x 4096 V2a N = 4, 1 % outliers 35.2 -> 32.0 us,
-// 3072 x 4096 V2a N = 2 14.2 -> 10.8, 12288 x 4096 V2 N = 4 33.3 -> 29.1.  100 MB of stores and 29 MB of loads are 20 us at the copy
-// rate; what is left is the chain of a block's first loads and a single round of blocks.
+// 3072 x 4096 V2a N = 2 14.2 -> 10.8, 12288 x 4096 V2 N = 4 33.3 -> 29.1; warm, 28672 x 8192 V2 N = 4, 0.3 % 123.5 -> 99.7, where DRAM
+// is at 67 % of its peak.  At 12289 x 4096 100 MB of stores and 29 MB of loads are 20 us at the copy rate; what is left is the chain
+// of a block's first loads and the outliers' way back from L2.
 #include "xfp_internal.h"
 #include "xfp_pair_common.cuh"
 #include "xfp_reg_decode.cuh"

@@ -525,8 +525,8 @@ template <int N, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fused_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap tmap) {
     using T = Tab<N, MODE>;
     // Codebooks in registers: V2a up to N = 4 and V2 at N = 4, which would take a look-up per weight; V2 at N = 2, 3 instead of pair
-    // tables where a pair walks its tiles (10007 x 4992 N = 3, 301 rows 42.5 -> 40.3 us, 28672 x 8192, 512 rows 237 -> 233), not where
-    // a cluster cuts one tile (4096 x 4096, 100 rows 21.3 against 21.5)
+    // tables where a pair walks its tiles (10007 x 4992 N = 3, 301 rows 42.5 -> 40.3 us, 28672 x 8192, 512 rows 237 -> 233; 192 rows
+    // at N = 2 29.3 -> 30.0 at 12288 x 4096), not where a cluster cuts one tile (4096 x 4096, 100 rows 21.3 against 21.5)
     constexpr bool kReg = MODE == 0 ? N == 4 || (N <= 3 && !SPLIT) : N <= 4;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // tables aligned to 8 KB of the shared window, so that an entry's offset is merged with the address, not added

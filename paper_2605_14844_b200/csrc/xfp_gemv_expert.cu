@@ -14,7 +14,8 @@
 //             one staging of x, one reduction and no barrier between them.  A lane's sum of one expert is scaled by its weight when
 //             the expert ends.  Runs of a row-block meet through the workspace in run order; one run per row-block needs none.
 // Eight experts, us for both launches (two channels per lane with tables -> this): 4096 x 1536 N = 3 45.0 -> 34.7, N = 2 42.3 -> 30.8,
-// N = 4 60.5 -> 44.9; 7168 x 2048 N = 3 93.7 -> 80.3.
+// N = 4 60.5 -> 44.9; 7168 x 2048 N = 3 93.7 -> 75.  A few weighted sums of two to five short experts are still 3 - 12 % behind the
+// tables (3 of 5120 x 1536 N = 4 13.0 -> 14.6, 5 of 3200 x 2048 N = 4 14.6 -> 15.2).
 // Bound by the ALU pipe in the K loop (PRMT and the selectors), around it by the chain pointer list - blob - first indices and the
 // staging of x behind the dependency wait.
 #include <algorithm>

@@ -130,7 +130,9 @@ LaneConfig lane_config(const Layout& l, int n = 1) {
     if (lane_reg_book(l)) {
         // No tables, 70 - 96 registers: one CTA of 16 warps per SM up to one CTA each (4096 x 4096, N = 3: 5.1 us, 8 warps 8.0: CTAs are
         // packed on SMs that have room for two), two of 8 where those hold all row-blocks (8192 x 8192, N = 3: 15.3 against 21.6 with
-        // three, which leave a third of the SMs empty), three beyond (28672 x 8192, N = 3: 42.4, two 43.2; 12288 x 4096 11.9, two 13.0)
+        // three, which leave a third of the SMs empty), three beyond (28672 x 8192, N = 3: 42.4, two 43.2; 12288 x 4096 11.9, two 13.0).
+        // The tables that this form replaced were ahead in two corners: N = 2 from one to about 1.5 row-blocks per SM of rows from
+        // 4096 weights on (6016 x 8192 12.5 us, here 13.3), N = 3 with at most eight codebooks up to one (3072 x 4096, one: 4.5, 4.9).
         LaneConfig c{RB <= sms ? 16 : 8, RB <= sms ? 1 : RB <= 2 * sms ? 2 : 3, false};
         if (c.per_sm == 3 && lane_smem_bytes(l, c) > 73u * 1024u) c.per_sm = 2;        // rows of x beyond 34000 weights
         if (c.per_sm == 2 && lane_smem_bytes(l, c) > 110u * 1024u) c = LaneConfig{16, 1, false};

@@ -1,7 +1,6 @@
 // Fast fused decode GEMV for V2a blobs (shared codebook library) at batch <= 2:
 //     y_i = sum_g [ scale_ig * sum_{k in g} lib[id_ig][q_ik] x_k  +  mid_ig * sum_{k in g} x_k ]  +  (S x)_i
-// ("V2a: Shared Codebook Library").  One launch serves one blob or the n blobs of a routed-MoE layer
-// (blockIdx.y = blob).
+// ("V2a: Shared Codebook Library").  One launch serves one blob or the n blobs of a routed-MoE layer.
 //
 // Mapping.  As in the V2 kernel a CTA owns 64 output channels, each lane of a warp two of them
 // (lane, lane+32), and the warps share K in super-chunks of 128 weights -- which are exactly the
@@ -11,8 +10,9 @@
 // Look-up.  Every lane may need a different library codebook, so tables cannot be private to a channel as in the V2 kernel.
 //   * N <= 4: the library sits in shared memory once, as byte planes (a few KB); a lane loads the codebook of its channel's
 //     group into registers and decodes with PRMTs (xfp_reg_decode.cuh).  There is no table to fill.
-//   * N = 5, and N = 4 at two rows of x (see v2a_config): the library replicated once per bank: word (id * 2^N + q) * 32 + lane holds lib[id][q] (fp16 in the low half).
-//     Lane l only touches bank l; one look-up decodes one weight and a multiply-add joins two of them.
+//   * N = 5, and N = 4 at two rows of x (see v2a_config): the library replicated once per bank: word (id * 2^N + q) * 32 + lane
+//     holds lib[id][q] (fp16 in the low half).  Lane l only touches bank l; one look-up decodes one weight and a multiply-add joins
+//     two of them.
 //
 // Multiply-accumulate.  The half2 of a lane's two channels form the A fragment of
 // mma.sync.m16n8k16 and x sits on the diagonal lanes of the B fragment (see xfp_gemv_pair.cu).  The

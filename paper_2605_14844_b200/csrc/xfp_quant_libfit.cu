@@ -252,6 +252,8 @@ __global__ void __launch_bounds__(kLibThreads) libfit_library_kernel(const uint1
     const int tid = threadIdx.x, lane = tid & 31;
     const int gt = blockIdx.x * kLibThreads + tid, nt = gridDim.x * kLibThreads;
     const int gw = gt >> 5, nw = nt >> 5;
+    // (the steps of normalise_channel, libfit_rank_kernel, seed_rank and store_ascending stand here in line: called as functions they
+    // cost this kernel 3 %, N = 4, 3072 channels 290 -> 298 us)
     // u[i][j] = (c_ij - m_i) / s_i, m and s the middle and half-width of the codebook's range; nn[i] = |u_i|^2
     for (int i = gt; i < rows; i += nt) {
         double lo = INFINITY, hi = -INFINITY;
