@@ -510,6 +510,8 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1) gemv_v2a_kernel(const 
                 put_y(y, o, h, a.y_is_fp16);
             }
         }
+    } else if (a.n == 1) {
+        if (t < kARows && !dup && row < a.rows) put_y(y, row, epi_wj * total, a.y_is_fp16);
     } else {
         // weighted sum over the blobs of the launch (the routed experts' down projections): they leave their terms in the scratch
         // (the K-split scratch is idle in these launches), the last one of the block to arrive adds them in blob order

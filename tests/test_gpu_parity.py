@@ -751,7 +751,8 @@ def test_fused_expert_block(bits, n, rows_gu, hidden, y_fp16):
     (3, 40, 96, 128, 32, 0.01, "uniform"), (2, 5, 4104, 1664, 7, 0.002, "uniform"), (4, 3, 70, 2048, 40, 0.05, "one_row"),
     (3, 9, 160, 384, 1, 0.0, "uniform"), (4, 10, 64, 768, 33, 0.02, "clustered"), (2, 2, 64, 40960, 32, 0.001, "uniform"),
     (3, 70, 32, 2048, 32, 0.005, "uniform"), (3, 6, 4800, 384, 32, 0.01, "uniform"), (2, 1, 4750, 128, 5, 0.02, "one_row"),
-    (4, 11, 4768, 256, 33, 0.003, "uniform"), (4, 2, 4768, 12288, 32, 0.0005, "uniform")])
+    (4, 11, 4768, 256, 33, 0.003, "uniform"), (4, 2, 4768, 12288, 32, 0.0005, "uniform"), (5, 1, 96, 256, 32, 0.01, "uniform"),
+    (5, 3, 4104, 128, 31, 0.01, "uniform")])
 def test_fused_stores_over_blobs_with_libraries_of_their_own(bits, n, rows, cols, lib_size, rate, placement):
     """Weighted sums of one run and of several runs per row-block, one super-chunk, more blobs than a CTA takes, rows that fill no
     row-block, slabs that overflow, x beyond what the fused kernel stages, more row-blocks than SMs (CTAs of 8 warps; one blob, runs
